@@ -74,7 +74,7 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     w.status = take(256);
     w.z0 = take((size_t)s.NT * unit_elems * s.esize);
     w.z1 = take((size_t)s.NT * s.NB * unit_elems * s.esize);  // Z1 of a pair, or the four layers' deviations of a block
-    w.z1drop = take(s.dtype == FDKV_BF16 && s.d == 128 ? (size_t)s.NU * s.NB * unit_elems * s.esize : 0);
+    w.z1drop = take(s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule ? (size_t)s.NU * s.NB * unit_elems * s.esize : 0);
     w.energy = take(s.B == 4 ? (size_t)s.NT * unit_elems * 4 : 0);
     w.eval = take(s.B == 4 ? (size_t)s.NT * s.kcap * 4 : 0);
     w.hist = take((size_t)s.NT * kHistBins * 4);
@@ -86,7 +86,7 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     w.val = take((size_t)s.NT * s.NB * s.kcap * s.esize);
     w.packed = take(s.dtype == FDKV_BF16 && s.d == 128 ? (size_t)s.NT * s.NB * s.kcap * 4 : 0);
     w.tok_score = take(s.tok_rule ? (size_t)s.NU * s.Tmax * 4 : 0);
-    w.tok_flag = take(s.tok_rule ? (size_t)s.NU * s.Tmax : 0);
+    w.tok_err = take(s.tok_rule ? (size_t)s.NU * token_err_slots(s.B, s.G, s.dtype == FDKV_BF16 && s.d == 128, kMaxW) * s.Tmax * 4 : 0);
     w.tok_list = take(s.tok_rule ? (size_t)s.NU * s.ktok_cap * 4 : 0);
     w.tok_off = take(s.tok_rule ? (size_t)s.NU * (s.ntiles_max + 1) * 4 : 0);
     w.probe_part = take((size_t)s.NU * s.nptiles_max * 16);
@@ -216,14 +216,13 @@ fdkv_status fdkv_create(const fdkv_config* cfg, void* arena, size_t arena_bytes,
     c->packed_lists = c->has_tmap && s.max_batch * s.Hkv <= kFastMaxUnits;
     if (s.rows_f8 && !(c->packed_lists && make_rows_tensor_map_u8(c->arena, arena_bytes, kRowPad, c->tmap_u8))) { delete c; return FDKV_ERR_UNSUPPORTED; }
     // token rule: the tensor-core score kernel and the packed decode kernel serve bf16 / head_dim 128; everything else
-    // takes the float32 score kernel, the float32 probe kernel (which masks the selected rows itself) and the portable decode kernel
+    // takes the float32 score kernel and the portable decode kernel
     if (s.tok_rule && c->packed_lists)
         c->tok_tc = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NT * s.NB * s.Tmax * s.d * s.esize, 128, c->tmap_z1_128);
     if (s.tok_rule && s.dtype == FDKV_BF16 && s.d == 128 && !c->tok_tc) { delete c; return FDKV_ERR_UNSUPPORTED; }
-    if (s.dtype == FDKV_BF16 && s.d == 128)
+    if (s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule)
         c->has_probe_tmaps = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NT * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_z1) &&
                              make_rows_tensor_map(c->work + c->ws.z1drop, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_drop);
-    if (c->tok_tc && !c->has_probe_tmaps) { delete c; return FDKV_ERR_UNSUPPORTED; }
     *out = c;
     return FDKV_OK;
 }
@@ -295,7 +294,7 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
             a4.unit_stride = (int64_t)s.Tmax * s.d;
             a4.z0 = c->work + c->ws.z0; a4.dev = c->work + c->ws.z1;
             a4.energy = wsp<float>(c, c->ws.energy);
-            a4.drop = (c->has_probe_tmaps && !s.tok_rule) ? c->work + c->ws.z1drop : nullptr;  // (the token rule writes its own copy in fdkv_probe)
+            a4.drop = c->has_probe_tmaps ? c->work + c->ws.z1drop : nullptr;
             a4.hist = wsp<uint32_t>(c, c->ws.hist);
             CU(launch_split4_hist(a4, s.dtype, st));
         }
@@ -400,7 +399,7 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
     a.z1 = c->work + c->ws.z1;
     a.idx = wsp<int32_t>(c, c->ws.idx);
     a.tile_off = wsp<int32_t>(c, c->ws.tile_off);
-    a.tok_flag = (s.tok_rule && !c->tok_tc) ? wsp<uint8_t>(c, c->ws.tok_flag) : nullptr;
+    a.sums_ready = s.tok_rule;
     a.q_layers_dev = qptr_dev;
     a.pos = pos_dev;
     a.part = wsp<double>(c, c->ws.probe_part);
@@ -420,9 +419,11 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
         t.unit_begin = a.unit_begin; t.unit_count = a.unit_count;
         t.T = T; t.Tmax = s.Tmax; t.Hq = s.Hq; t.Hkv = s.Hkv; t.G = s.G; t.W = W; t.ntiles_max = s.ntiles_max;
         t.k_tok = (int64_t)T * s.keep_num / s.keep_den; t.ktok_cap = s.ktok_cap; t.unit_stride = (int64_t)s.Tmax * s.d;
-        t.z1 = c->work + c->ws.z1; t.z1drop = c->work + c->ws.z1drop;
+        t.z1 = c->work + c->ws.z1;
         t.q_layers_dev = qptr_dev; t.pos = pos_dev; t.pos_host = probe_pos;
-        t.score = wsp<uint32_t>(c, c->ws.tok_score); t.flag = wsp<uint8_t>(c, c->ws.tok_flag);
+        t.score = wsp<uint32_t>(c, c->ws.tok_score);
+        t.err = wsp<float>(c, c->ws.tok_err); t.nslots = token_err_slots(s.B, s.G, c->tok_tc, W);
+        t.part = a.part; t.nptiles_max = s.nptiles_max; t.pos_last = probe_pos[W - 1];
         t.list = wsp<int32_t>(c, c->ws.tok_list); t.off = wsp<int32_t>(c, c->ws.tok_off);
         t.tmap_z1_128 = c->tmap_z1_128;
         t.status = wsp<int32_t>(c, c->ws.status);

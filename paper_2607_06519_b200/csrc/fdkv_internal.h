@@ -78,7 +78,7 @@ struct Shape {
 };
 
 struct WsLayout {
-    size_t tok_score, tok_flag, tok_list, tok_off;
+    size_t tok_score, tok_err, tok_list, tok_off;
     size_t energy, eval;  // four-layer blocks: per-position high-frequency energy (float32) and the kept energies
     size_t status, z0, z1, z1drop, hist, sel, lb_records, lb_ticket, tile_off, idx, val, packed, probe_part, probe_pos, scores, modes,
         partials, counters, io_q, io_k, io_v, io_out, jobs, total;  // io_*: host-I/O staging, [L] layers each
@@ -203,7 +203,7 @@ struct ProbeArgs {
     const void* z1;  // staged Z1 (unit-tensor ut = unit*2 for K)
     const int32_t* idx;
     const int32_t* tile_off;
-    const uint8_t* tok_flag;          // token rule, float32 probe kernel: [NU][Tmax] flags of the selected tokens (else null)
+    bool sums_ready;                  // token rule: part slot 0 of every unit holds the error sums already
     const void* const* q_layers_dev;  // device array [L] of pointers
     const int32_t* pos;
     double* part;    // [NU][nptiles_max][2]
@@ -299,18 +299,23 @@ struct TokenArgs {
     int T, Tmax, Hq, Hkv, G, W, ntiles_max;
     int64_t k_tok, ktok_cap, unit_stride;
     const void* z1;                    // staged Z1 (K of unit u at unit-tensor 2u)
-    void* z1drop;                      // [unit][Tmax*128] Z1 of K with the selected rows zeroed
     const void* const* q_layers_dev;
     const int32_t* pos;
     const int32_t* pos_host;
     uint32_t* score;                   // [unit][Tmax] float bits (non-negative)
-    uint8_t* flag;                     // [unit][Tmax]
+    float* err;                        // [unit][nslots][Tmax] sum of squared products per token
+    int nslots;                        // items a token's sum is spread over: layers x 256-row blocks, or 1 (float32 kernel)
+    double* part;                      // [NU][nptiles_max][2]: slot 0 gets the unit's error sums (shared, residual)
+    int nptiles_max;
+    int pos_last;                      // the last probe position
     int32_t* list;                     // [unit][ktok_cap]
     int32_t* off;                      // [unit][ntiles_max + 1]
     const void* tmap_z1_128;
     int32_t* status;
 };
-// tensor_core: bf16 / head_dim 128 contexts (tcgen05 score kernel + the dropped-row copy); otherwise the float32 score kernel
+// TokenArgs::nslots of a context for W probe queries
+inline int token_err_slots(int B, int G, bool tensor_core, int W) { return tensor_core ? B * ((G * W + 255) / 256) : 1; }
+// tensor_core: bf16 / head_dim 128 contexts (tcgen05 score kernel); otherwise the float32 score kernel
 cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tensor_core, cudaStream_t st);
 cudaError_t launch_token_gather(const void* z1, const int32_t* list, int64_t k_tok, void* out, int row_bytes, int twice, cudaStream_t st);
 

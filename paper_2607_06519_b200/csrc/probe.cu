@@ -48,20 +48,13 @@ __global__ void __launch_bounds__(256) probe_tile_kernel(ProbeArgs a) {
             drop[t * ld + c] = v;
         }
         __syncthreads();
-        if (a.tok_flag) {
-            // token rule: the residual candidate keeps whole rows -- the selected tokens drop nothing
-            const uint8_t* flag = a.tok_flag + (int64_t)unit * a.Tmax + t0;
-            for (int i = threadIdx.x; i < nt * d; i += blockDim.x)
-                if (flag[i / d]) drop[(i / d) * ld + (i % d)] = 0.f;
-        } else {
-            const int32_t* off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1);
-            const int ntiles = (a.T + kResTile - 1) / kResTile;
-            const int j0 = t0 / kResTile, j1 = min(ntiles, (t0 + kProbeTile) / kResTile);
-            const int32_t* idx = a.idx + (int64_t)ut * a.kcap;
-            for (int e = off[j0] + threadIdx.x; e < off[j1]; e += blockDim.x) {
-                const int f = idx[e] - t0 * d;
-                drop[(f / d) * ld + (f % d)] = 0.f;
-            }
+        const int32_t* off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1);
+        const int ntiles = (a.T + kResTile - 1) / kResTile;
+        const int j0 = t0 / kResTile, j1 = min(ntiles, (t0 + kProbeTile) / kResTile);
+        const int32_t* idx = a.idx + (int64_t)ut * a.kcap;
+        for (int e = off[j0] + threadIdx.x; e < off[j1]; e += blockDim.x) {
+            const int f = idx[e] - t0 * d;
+            drop[(f / d) * ld + (f % d)] = 0.f;
         }
         __syncthreads();
         for (int rb = 0; rb < M; rb += kRowsBlk) {
@@ -160,10 +153,10 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
 
 cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st) {
     if (a.unit_count <= 0) return cudaSuccess;
-    int nparts = (a.T + kProbeTile - 1) / kProbeTile;
-    bool handled = false;
-    cudaError_t e = launch_probe_tc(a, dtype, st, &handled, &nparts);
-    if (e != cudaSuccess) return e;
+    int nparts = a.sums_ready ? 1 : (a.T + kProbeTile - 1) / kProbeTile;
+    bool handled = a.sums_ready;
+    cudaError_t e = cudaSuccess;
+    if (!handled && (e = launch_probe_tc(a, dtype, st, &handled, &nparts)) != cudaSuccess) return e;
     if (!handled) {
         const size_t smem = (size_t)(2 * kProbeTile * (a.d + 1) + kRowsBlk * a.d) * sizeof(float);
         static PerDevice once;

@@ -12,10 +12,13 @@
 //    tokens of Z1K per tile (TMA ring, shared memory), B = the item's 256 Q rows (shared memory, resident),
 //    M = 128, N = 256, K = 16, two accumulator sets of 256 TMEM columns.  Items of the two layers / row blocks of a
 //    unit merge with atomicMax on the (non-negative) float bit patterns, which is order-independent.
+//    The same registers give Eq. 2's errors: the token's sum of D^2 over the rows that see it, one float per item.  Shared
+//    drops every token's high-frequency row, residual every unselected one's, so both errors are sums of these numbers
+//    and the probe needs no second product (it was two more passes over T x rows x 128, and a copy of Z1K with the
+//    selected rows zeroed to run one of them on: 8 191 tokens, 8 blocks of four: the probe 627 -> 250 us).
 // 2. token_select_kernel: per unit an MSB-first radix select (4 x 8 bits) of the k_tok-th largest score and an
-//    index-ordered compaction: ascending token list, per-token flags, per-16-token-slice counts.
-// 3. token_drop_kernel: Z1K with the selected rows zeroed (the residual candidate's B operand in the probe).
-// 4. token_gather_kernel (commit): the selected rows of Z1, densely packed.
+//    index-ordered compaction: ascending token list, per-16-token-slice counts, and the two error sums in float64.
+// 3. token_gather_kernel (commit): the selected rows of Z1, densely packed.
 #include <cuda.h>
 
 #include <algorithm>
@@ -190,8 +193,9 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
             }
         }
     } else {
-        // ---- epilogue: thread = token (TMEM lane); maximum of |D| over the probe rows that can see the token ----
+        // ---- epilogue: thread = token (TMEM lane); maximum of |D| and sum of D^2 over the probe rows that see the token ----
         const int lq = warp & 3;
+        float* const err = a.err + ((int64_t)unit * a.nslots + layer * pl.mblocks + mblock) * a.Tmax;
         const float c32 = a.B == 4 ? 1.f : __uint_as_float(0x3F3504F3u);  // a pair's rows are Z1: K - Khat^shared = +-c Z1
         uint32_t* score = a.score + (int64_t)unit * a.Tmax;
         for (int i = 0; i < ntile; ++i) {
@@ -199,7 +203,7 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
             const int t = (tile0 + i) * kTM + lq * 32 + lane;
             mb_wait(sm0 + tTFull + 8 * as, ((uint32_t)i >> 1) & 1u, abort_flag, a.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float m = 0.f;
+            float m = 0.f, e0 = 0.f, e1 = 0.f;
             if (!*abort_flag) {
                 const bool all_visible = (tile0 + i) * kTM + kTM - 1 <= pl.pos_min;
 #pragma unroll
@@ -211,17 +215,26 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     if (all_visible) {
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) m = fmaxf(m, fmaxf(fabsf(__uint_as_float(r0[j])), fabsf(__uint_as_float(r1[j]))));
+                        for (int j = 0; j < 32; ++j) {
+                            const float u = __uint_as_float(r0[j]), v = __uint_as_float(r1[j]);
+                            m = fmaxf(m, fmaxf(fabsf(u), fabsf(v)));
+                            e0 = fmaf(u, u, e0);
+                            e1 = fmaf(v, v, e1);
+                        }
                     } else {
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
-                            if (pos_col[cp * 64 + j] >= t) m = fmaxf(m, fabsf(__uint_as_float(r0[j])));
-                            if (pos_col[cp * 64 + 32 + j] >= t) m = fmaxf(m, fabsf(__uint_as_float(r1[j])));
+                            const float u = __uint_as_float(r0[j]), v = __uint_as_float(r1[j]);
+                            if (pos_col[cp * 64 + j] >= t) { m = fmaxf(m, fabsf(u)); e0 = fmaf(u, u, e0); }
+                            if (pos_col[cp * 64 + 32 + j] >= t) { m = fmaxf(m, fabsf(v)); e1 = fmaf(v, v, e1); }
                         }
                     }
                 }
             }
-            if (t < a.T && m > 0.f && !*abort_flag) atomicMax(score + t, __float_as_uint(m * c32));
+            if (t < a.T && !*abort_flag) {
+                if (m > 0.f) atomicMax(score + t, __float_as_uint(m * c32));
+                err[t] = e0 + e1;
+            }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mb_arrive(sm0 + tTEmpty + 8 * as);
@@ -265,14 +278,15 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* s_warp
 
 // One CTA per unit: threshold of the k-th largest score (32-bit patterns of non-negative floats order like the
 // floats), then the ascending list of kept tokens (score above the threshold, or equal and among the first `need`
-// such tokens), their flags and the number of kept tokens before every 16-token slice.
+// such tokens), the number of kept tokens before every 16-token slice, and the unit's two error sums: all tokens'
+// (shared) and the unselected ones' (residual), float64 over the score kernel's per-token sums in a fixed order.
 __global__ void __launch_bounds__(1024) token_select_kernel(TokenArgs a) {
     __shared__ uint32_t s_hist[256];
     __shared__ uint32_t s_warp[33];
     __shared__ uint32_t s_prefix, s_krem;
     const int unit = a.unit_begin + blockIdx.x;
     const uint32_t* key = a.score + (int64_t)unit * a.Tmax;
-    uint8_t* flag = a.flag + (int64_t)unit * a.Tmax;
+    const float* err = a.err + (int64_t)unit * a.nslots * a.Tmax;
     int32_t* list = a.list + (int64_t)unit * a.ktok_cap;
     int32_t* off = a.off + (int64_t)unit * (a.ntiles_max + 1);
     const int T = a.T;
@@ -307,6 +321,8 @@ __global__ void __launch_bounds__(1024) token_select_kernel(TokenArgs a) {
     }
     // ordered compaction, 1024 tokens per round
     uint32_t base_keep = 0, base_eq = 0;
+    double sum_all = 0.0, sum_dropped = 0.0;
+    const int seen = min(T, a.pos_last + 1);  // later tokens are seen by no probe query: no error, nothing was written
     for (int t0 = 0; t0 < T; t0 += 1024) {
         const int t = t0 + threadIdx.x;
         const uint32_t k = t < T ? key[t] : 0u;
@@ -315,32 +331,35 @@ __global__ void __launch_bounds__(1024) token_select_kernel(TokenArgs a) {
         const uint32_t rank_eq = base_eq + block_excl_scan(eq, s_warp, &tot_eq);
         const uint32_t keep = gt || (eq && rank_eq < need);
         const uint32_t posk = base_keep + block_excl_scan(keep, s_warp, &tot_keep);
+        if (t < seen) {
+            double e = 0.0;
+            for (int j = 0; j < a.nslots; ++j) e += (double)err[(int64_t)j * a.Tmax + t];
+            sum_all += e;
+            if (!keep) sum_dropped += e;
+        }
         if (t < T) {
-            flag[t] = (uint8_t)keep;
             if (keep) list[posk] = t;
             if ((t & (kResTile - 1)) == 0) off[t / kResTile] = (int32_t)posk;
         }
         base_eq += tot_eq;
         base_keep += tot_keep;
     }
+    __shared__ double s_err[2][32];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        sum_all += __shfl_xor_sync(0xFFFFFFFFu, sum_all, o);
+        sum_dropped += __shfl_xor_sync(0xFFFFFFFFu, sum_dropped, o);
+    }
+    if ((threadIdx.x & 31) == 0) { s_err[0][threadIdx.x >> 5] = sum_all; s_err[1][threadIdx.x >> 5] = sum_dropped; }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double e = 0.0;
+        for (int w = 0; w < 32; ++w) e += s_err[threadIdx.x][w];
+        a.part[(int64_t)unit * a.nptiles_max * 2 + threadIdx.x] = e;
+    }
     if (threadIdx.x == 0) {
         off[nslice] = (int32_t)base_keep;
         if ((int64_t)base_keep != a.k_tok) atomicMax(a.status, (int32_t)kFlagCountMismatch);
-    }
-}
-
-// Z1K with the selected rows zeroed.  grid (row blocks, units), 256 threads, one 16-byte vector per thread and step.
-__global__ void __launch_bounds__(256) token_drop_kernel(TokenArgs a) {
-    const int unit = a.unit_begin + blockIdx.y;
-    const int nb = a.B == 4 ? 4 : 1, l = blockIdx.z;  // staged high-frequency tensors per unit-tensor
-    const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.z1) + ((int64_t)unit * 2 * nb + l) * a.unit_stride);
-    uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.z1drop) + ((int64_t)unit * nb + l) * a.unit_stride);
-    const uint8_t* flag = a.flag + (int64_t)unit * a.Tmax;
-    const int64_t nvec = (int64_t)a.T * 16;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvec; v += (int64_t)gridDim.x * blockDim.x) {
-        uint4 x = src[v];
-        if (flag[v >> 4]) x = make_uint4(0u, 0u, 0u, 0u);
-        dst[v] = x;
     }
 }
 
@@ -370,9 +389,9 @@ __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 x) { return
 
 constexpr int kSTile = 64;   // tokens per thread block
 constexpr int kSRows = 16;   // probe rows staged per round
-// grid (64-token tiles, units), 256 threads: thread (token j, row group rg) takes the maximum of |q_r . z[t]| over the
-// rows r of its group whose probe position sees token t; the groups and the layers merge by atomicMax on the bit
-// patterns of the non-negative floats.
+// grid (64-token tiles, units), 256 threads: thread (token j, row group rg) takes the maximum of |q_r . z[t]| and the sum of
+// its square over the rows r of its group whose probe position sees token t; the groups' maxima merge by atomicMax on
+// the bit patterns of the non-negative floats, their sums through shared memory.
 template <typename T>
 __global__ void __launch_bounds__(256) token_score_tile_kernel(TokenArgs a, int d) {
     extern __shared__ float ssm[];
@@ -387,7 +406,7 @@ __global__ void __launch_bounds__(256) token_score_tile_kernel(TokenArgs a, int 
     const int j = (warp & 1) * 32 + lane, rg = warp >> 1;
     const int n_ops = a.B == 4 ? 4 : 1;
     const int M = (a.B == 4 ? 1 : 2) * a.G * a.W;  // probe rows per operand
-    float best = 0.f;
+    float best = 0.f, esum = 0.f;
     for (int op = 0; op < n_ops; ++op) {
         const T* z1 = reinterpret_cast<const T*>(a.z1) + ((int64_t)unit * 2 * n_ops + op) * a.unit_stride + (int64_t)t0 * d;
         for (int i = threadIdx.x; i < kSTile * d; i += blockDim.x) {
@@ -418,11 +437,18 @@ __global__ void __launch_bounds__(256) token_score_tile_kernel(TokenArgs a, int 
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = rb + rg * 4 + i;
-                if (r < M && j < nt && t0 + j <= a.pos[r % a.W]) best = fmaxf(best, fabsf(acc[i]));
+                if (r < M && j < nt && t0 + j <= a.pos[r % a.W]) {
+                    best = fmaxf(best, fabsf(acc[i]));
+                    esum = fmaf(acc[i], acc[i], esum);
+                }
             }
             __syncthreads();
         }
     }
+    float* const s_e = qs;  // [4][64]: the row groups' sums (every product is done: the loop ends on a barrier)
+    s_e[rg * kSTile + j] = esum;
+    __syncthreads();
+    if (rg == 0 && j < nt) a.err[(int64_t)unit * a.nslots * a.Tmax + t0 + j] = (s_e[j] + s_e[kSTile + j]) + (s_e[2 * kSTile + j] + s_e[3 * kSTile + j]);
     // the score carries the factor of Eq. 1's inverse (c for a pair; a block of four's deviations are in layer space already)
     if (j < nt) atomicMax(a.score + (int64_t)unit * a.Tmax + t0 + j, __float_as_uint(best * (a.B == 4 ? 1.f : __uint_as_float(0x3F3504F3u))));
 }
@@ -453,12 +479,13 @@ cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tenso
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         token_select_kernel<<<a.unit_count, 1024, 0, st>>>(a);
         count_launch(2);
-        return cudaGetLastError();  // (the float32 probe kernel masks the selected rows itself: no dropped copy)
+        count_kernel(FDKV_KERNEL_PROBE_PORTABLE);
+        return cudaGetLastError();
     }
     ScorePlan pl;
     pl.pos_min = a.pos_host[0];
     pl.ntiles = a.pos_host[a.W - 1] / kTM + 1;  // tokens after the last probe position are seen by nobody: score 0
-    pl.mblocks = (a.G * a.W + kTN - 1) / kTN;
+    pl.mblocks = (a.G * a.W + kTN - 1) / kTN;  // (a.nslots = B x mblocks)
     const int base_items = a.unit_count * a.B * pl.mblocks;
     int nsplits = std::max(1, std::min((4 * sm_count + base_items - 1) / base_items, (pl.ntiles + 7) / 8));
     pl.tiles_per_split = (pl.ntiles + nsplits - 1) / nsplits;
@@ -467,11 +494,9 @@ cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tenso
     token_score_kernel<<<a.unit_count * pl.items_per_unit, kTThreads, kTSmem, st>>>(*reinterpret_cast<const CUtensorMap*>(a.tmap_z1_128), a, pl);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     token_select_kernel<<<a.unit_count, 1024, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int blocks = (int)std::min<int64_t>(64, ((int64_t)a.T * 16 + 255) / 256);
-    token_drop_kernel<<<dim3(blocks, a.unit_count, a.B == 4 ? 4 : 1), 256, 0, st>>>(a);
-    count_launch(3);
+    count_launch(2);
     count_kernel(FDKV_KERNEL_TOKEN_SCORE);
+    count_kernel(FDKV_KERNEL_PROBE_TC);  // (it is the probe's product too)
     return cudaGetLastError();
 }
 
