@@ -67,6 +67,9 @@ bool make_shape(const fdkv_config& c, Shape& s) {
     return true;
 }
 
+constexpr size_t quant_table_bytes(const Shape& s) { return s.rows_f8 ? (size_t)s.NU * 2 * s.B * (sizeof(QuantJob) + sizeof(RepackJob)) : 0; }
+constexpr size_t gather_table_bytes(const Shape& s) { return s.tok_rule ? (size_t)s.NU * 2 * sizeof(TokenGatherJob) : 0; }
+
 void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
@@ -75,8 +78,8 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     w.z0 = take((size_t)s.NT * unit_elems * s.esize);
     w.z1 = take((size_t)s.NT * s.NB * unit_elems * s.esize);  // Z1 of a pair, or the four layers' deviations of a block
     w.z1drop = take(s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule ? (size_t)s.NU * s.NB * unit_elems * s.esize : 0);
-    w.energy = take(s.B == 4 ? (size_t)s.NT * unit_elems * 4 : 0);
-    w.eval = take(s.B == 4 ? (size_t)s.NT * s.kcap * 4 : 0);
+    w.energy = take(s.B == 4 && !s.tok_rule ? (size_t)s.NT * unit_elems * 4 : 0);
+    w.eval = take(s.B == 4 && !s.tok_rule ? (size_t)s.NT * s.kcap * 4 : 0);
     w.hist = take((size_t)s.NT * kHistBins * 4);
     w.sel = take((size_t)s.NT * sizeof(SelState));
     w.lb_records = take((size_t)s.NT * s.ntiles_max * 8);
@@ -99,11 +102,10 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     w.io_k = take((size_t)s.L * s.max_batch * s.Hkv * s.d * 4);
     w.io_v = take((size_t)s.L * s.max_batch * s.Hkv * s.d * 4);
     w.io_out = take((size_t)s.L * s.max_batch * s.Hq * s.d * 4);
-    // job tables of the 8-bit commit: one quantise job per stored tensor, one repack job per residual list
-    // job tables of a commit: quantise / repack jobs (8-bit rows), then the copy jobs (at most 2 B row copies, or 2 row
-    // copies, 2 offset tables and 2 NB lists, per unit)
-    w.jobs = take((s.rows_f8 ? (size_t)s.NU * 2 * s.B * (sizeof(QuantJob) + sizeof(RepackJob)) : 0) +
-                  (size_t)s.NU * (2 * s.B + 4 + 2 * s.NB) * sizeof(CopyJob));
+    // job tables of a commit: quantise jobs (one per stored tensor) and repack jobs (one per residual list) of 8-bit rows,
+    // gather jobs of the token rule, then the copy jobs (at most 2 B row copies, or 2 row copies, 2 offset tables and 2 NB
+    // lists, per unit)
+    w.jobs = take(quant_table_bytes(s) + gather_table_bytes(s) + (size_t)s.NU * (2 * s.B + 4 + 2 * s.NB) * sizeof(CopyJob));
     w.total = o;
 
     o = 0;
@@ -276,6 +278,26 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
     }
     cudaStream_t st = S(stream);
     const int ut_begin = pb * s.Hkv * 2, ut_count = (pe - pb) * s.Hkv * 2;
+    if (s.tok_rule) {
+        // the token rule selects inside fdkv_probe: only the split here
+        constexpr int kMost = kSplitLayers;
+        for (int p0 = pb; p0 < pe; p0 += kMost / s.B) {
+            SplitRowsArgs a;
+            a.n_blocks = std::min(pe - p0, kMost / s.B);
+            for (int l = 0; l < a.n_blocks * s.B; ++l) {
+                a.k[l] = c->k_layers[s.B * p0 + l] = k_layers[s.B * p0 + l];
+                a.v[l] = c->v_layers[s.B * p0 + l] = v_layers[s.B * p0 + l];
+            }
+            a.stride_t = stride_t; a.stride_h = stride_h;
+            a.T = T; a.d = s.d; a.Hkv = s.Hkv;
+            a.ut_base = p0 * s.Hkv * 2;
+            a.unit_stride = (int64_t)s.Tmax * s.d;
+            a.z0 = c->work + c->ws.z0; a.hf = c->work + c->ws.z1;
+            CU(launch_split_rows(a, s.B, s.dtype, st));
+        }
+        for (int p = pb; p < pe; ++p) { c->pair_compressed[p] = 1; c->pair_probed[p] = 0; c->pair_scored[p] = 0; }
+        return FDKV_OK;
+    }
     CU(cudaMemsetAsync(wsp<uint32_t>(c, c->ws.hist) + (size_t)ut_begin * kHistBins, 0, (size_t)ut_count * kHistBins * 4, st));
     if (s.B == 4) {
         // blocks of four layers: Z0, the layers' deviations and the positions' energies; one kept set per tensor from
@@ -297,10 +319,6 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
             a4.drop = c->has_probe_tmaps ? c->work + c->ws.z1drop : nullptr;
             a4.hist = wsp<uint32_t>(c, c->ws.hist);
             CU(launch_split4_hist(a4, s.dtype, st));
-        }
-        if (s.tok_rule) {  // the token rule selects inside fdkv_probe
-            for (int p = pb; p < pe; ++p) { c->pair_compressed[p] = 1; c->pair_probed[p] = 0; c->pair_scored[p] = 0; }
-            return FDKV_OK;
         }
         SelectArgs sa;
         sa.ut_begin = ut_begin; sa.ut_count = ut_count;
@@ -365,7 +383,7 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
     sa.packed = c->packed_lists ? wsp<uint32_t>(c, c->ws.packed) : nullptr;
     sa.z1drop = c->has_probe_tmaps ? c->work + c->ws.z1drop : nullptr;
     sa.status = wsp<int32_t>(c, c->ws.status);
-    if (!s.tok_rule) CU(launch_select_and_compact(sa, s.dtype, st));  // the token rule selects inside fdkv_probe
+    CU(launch_select_and_compact(sa, s.dtype, st));
     for (int p = pb; p < pe; ++p) { c->pair_compressed[p] = 1; c->pair_probed[p] = 0; c->pair_scored[p] = 0; }
     return FDKV_OK;
 }
@@ -545,6 +563,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
     const size_t unit_stride_b = (size_t)s.Tmax * s.d * s.esize;
     std::vector<QuantJob> qjobs;   // 8-bit rows: every stored tensor is quantised by one batched pass after this loop
     std::vector<RepackJob> rjobs;  // ... and every residual list repacked relative to its tensor's scales
+    std::vector<TokenGatherJob> gjobs;  // token rule: the selected rows, formed from the caller's K and V
     std::vector<CopyJob> cjobs;    // device-to-device copies into the arena: one launch over this table after the loop
     int64_t copy_max = 0;
     auto copy_job = [&](const void* src, void* dst, size_t bytes, int64_t src_pitch, int row_bytes) {
@@ -614,11 +633,16 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                     // opposite signs), each layer's own deviation rows of a block of four (stored doubled: see the gather kernel)
                     // (the list is read where the probe left it: its copy into the arena runs with the other copies after this loop)
                     char* rows_l[4] = {nullptr, nullptr, nullptr, nullptr};
-                    for (int j = 0; j < s.NB; ++j) {
-                        rows_l[j] = take(trow_b);
-                        CU(launch_token_gather(c->work + c->ws.z1 + (ut * s.NB + j) * unit_stride_b, wsp<int32_t>(c, c->ws.tok_list) + (size_t)u * s.ktok_cap, k_tok,
-                                               rows_l[j], s.d * s.esize, (s.B == 4 && c->packed_lists) ? 1 : 0, st));
-                    }
+                    TokenGatherJob gj;
+                    std::memset(&gj, 0, sizeof(gj));
+                    for (int l = 0; l < s.B; ++l)
+                        gj.x[l] = (const char*)(is_v ? c->v_layers[s.B * p + l] : c->k_layers[s.B * p + l]) + (size_t)h * c->stride_h * s.esize;
+                    for (int j = 0; j < s.NB; ++j) gj.dst[j] = rows_l[j] = take(trow_b);
+                    gj.list = wsp<int32_t>(c, c->ws.tok_list) + (size_t)u * s.ktok_cap;
+                    gj.stride_t = c->stride_t;
+                    gj.k_tok = k_tok;
+                    gj.twice = (s.B == 4 && c->packed_lists) ? 1 : 0;
+                    gjobs.push_back(gj);
                     if (s.rows_f8)  // 8-bit rows: the kept rows become f16(value / scale[channel]) in the fragment order of the 8-bit tiles
                         for (int j = 0; j < s.NB; ++j)
                             rjobs.push_back(RepackJob{reinterpret_cast<uint32_t*>(rows_l[j]), reinterpret_cast<const uint32_t*>(rows_l[j]), k_tok, sc8, is_v, 1});
@@ -665,8 +689,13 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
             }
         }
     }
+    char* const table = c->work + c->ws.jobs + quant_table_bytes(s);
+    if (!gjobs.empty()) {
+        CU(cudaMemcpyAsync(table, gjobs.data(), gjobs.size() * sizeof(TokenGatherJob), cudaMemcpyHostToDevice, st));
+        CU(launch_token_gather_jobs(reinterpret_cast<TokenGatherJob*>(table), (int)gjobs.size(), k_tok, s.d, s.B, s.dtype, st));
+    }
     if (!cjobs.empty()) {
-        CopyJob* cd = reinterpret_cast<CopyJob*>(c->work + c->ws.jobs + (s.rows_f8 ? (size_t)s.NU * 2 * s.B * (sizeof(QuantJob) + sizeof(RepackJob)) : 0));
+        CopyJob* cd = reinterpret_cast<CopyJob*>(table + gather_table_bytes(s));
         CU(cudaMemcpyAsync(cd, cjobs.data(), cjobs.size() * sizeof(CopyJob), cudaMemcpyHostToDevice, st));
         CU(launch_copy_jobs(cd, (int)cjobs.size(), copy_max, st));
     }

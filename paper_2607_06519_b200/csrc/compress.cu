@@ -121,6 +121,107 @@ __global__ void __launch_bounds__(1024) split_hist_kernel(CompressArgs a, int to
     }
 }
 
+// ----- C1 without a selection (token rule: the probe selects) ----------------------------------------
+// Shared coefficients of K and V and the high-frequency rows of K (Z1 of a pair, or the four layers' deviations: what the
+// probe scores), in the arithmetic of split_hist_kernel / split4_hist_kernel.  V's high-frequency rows are only wanted for
+// the few tokens that are kept, so the commit step forms those from the caller's rows instead of staging all of them.
+// Bound by HBM: no histogram, so no shared memory, full occupancy and one launch over all blocks (it shared the histogram
+// kernel before, one launch per block of four: 8 191 tokens, 8 blocks of four: 963 us); two vectors of every
+// layer in flight per thread.
+template <typename T, int B>
+__global__ void __launch_bounds__(256) split_rows_kernel(SplitRowsArgs a) {
+    using S = Store<T>;
+    constexpr int VEC = S::VEC;
+    constexpr int NV = 2;
+    const int h = blockIdx.y >> 1, is_v = blockIdx.y & 1, blk = blockIdx.z;
+    const int64_t ut = a.ut_base + (int64_t)blk * a.Hkv * 2 + blockIdx.y;
+    T* const z0 = reinterpret_cast<T*>(a.z0) + ut * a.unit_stride;
+    T* const hf = reinterpret_cast<T*>(a.hf) + ut * (B == 4 ? 4 : 1) * a.unit_stride;
+    const float c32 = __uint_as_float(0x3F3504F3u);
+    const int vpr = a.d / VEC;
+    const int nvec = a.T * vpr;
+    typename S::vec_t r[NV][B];
+    int64_t off_out[NV];
+    bool live[NV];
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+        const int v = (blockIdx.x * NV + u) * 256 + (int)threadIdx.x;
+        live[u] = v < nvec;
+        const int t = v / vpr, cv = (v - t * vpr) * VEC;
+        const int64_t off_in = (int64_t)t * a.stride_t + (int64_t)h * a.stride_h + cv;
+        off_out[u] = (int64_t)v * VEC;
+        if (live[u])
+#pragma unroll
+            for (int l = 0; l < B; ++l)
+                r[u][l] = *reinterpret_cast<const typename S::vec_t*>(reinterpret_cast<const T*>(is_v ? a.v[B * blk + l] : a.k[B * blk + l]) + off_in);
+    }
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+        if (!live[u]) continue;
+        float f[B][VEC], z[VEC];
+#pragma unroll
+        for (int l = 0; l < B; ++l) S::unpack(r[u][l], f[l]);
+        if constexpr (B == 2) {
+            float f1[VEC];
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) {
+                z[i] = __fmul_rn(__fadd_rn(f[0][i], f[1][i]), c32);
+                f1[i] = __fmul_rn(__fsub_rn(f[0][i], f[1][i]), c32);
+            }
+            if (!is_v) *reinterpret_cast<typename S::vec_t*>(hf + off_out[u]) = S::pack(f1);
+        } else {
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) {
+                z[i] = stored<T>(__fmul_rn(0.5f, __fadd_rn(__fadd_rn(f[0][i], f[1][i]), __fadd_rn(f[2][i], f[3][i]))));
+                const float half = __fmul_rn(0.5f, z[i]);  // exact
+#pragma unroll
+                for (int l = 0; l < B; ++l) f[l][i] = __fsub_rn(f[l][i], half);
+            }
+            if (!is_v)
+#pragma unroll
+                for (int l = 0; l < B; ++l) *reinterpret_cast<typename S::vec_t*>(hf + (int64_t)l * a.unit_stride + off_out[u]) = S::pack(f[l]);
+        }
+        *reinterpret_cast<typename S::vec_t*>(z0 + off_out[u]) = S::pack(z);
+    }
+}
+
+// Token rule, commit: the high-frequency rows of the selected tokens, densely packed, formed from the caller's rows of the
+// block's layers (one job per unit-tensor, one thread per 16-byte vector: reads B rows, writes one row per stored
+// tensor).  `twice` doubles the stored rows (bf16 rows of the tensor-core decode kernel; exact): a block of four scales its
+// rows by 1/2 at decode time and its deviations by 1.
+template <typename T, int B>
+__global__ void __launch_bounds__(256) token_gather_kernel(const TokenGatherJob* jobs, int d) {
+    using S = Store<T>;
+    constexpr int VEC = S::VEC;
+    const TokenGatherJob& jb = jobs[blockIdx.y];
+    const int vpr = d / VEC;
+    const int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int64_t j = v / vpr;
+    if (j >= jb.k_tok) return;
+    const int cv = (int)(v - j * vpr) * VEC;
+    const int64_t off_in = (int64_t)jb.list[j] * jb.stride_t + cv;
+    float f[B][VEC];
+#pragma unroll
+    for (int l = 0; l < B; ++l) S::unpack(*reinterpret_cast<const typename S::vec_t*>(reinterpret_cast<const T*>(jb.x[l]) + off_in), f[l]);
+    if constexpr (B == 2) {
+        const float c32 = __uint_as_float(0x3F3504F3u);
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) f[0][i] = __fmul_rn(__fsub_rn(f[0][i], f[1][i]), c32);
+        *reinterpret_cast<typename S::vec_t*>(reinterpret_cast<T*>(jb.dst[0]) + v * VEC) = S::pack(f[0]);
+    } else {
+        const float k = jb.twice ? 2.f : 1.f;
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            const float z = stored<T>(__fmul_rn(0.5f, __fadd_rn(__fadd_rn(f[0][i], f[1][i]), __fadd_rn(f[2][i], f[3][i]))));
+            const float half = __fmul_rn(0.5f, z);  // exact
+#pragma unroll
+            for (int l = 0; l < B; ++l) f[l][i] = stored<T>(__fsub_rn(f[l][i], half)) * k;
+        }
+#pragma unroll
+        for (int l = 0; l < B; ++l) *reinterpret_cast<typename S::vec_t*>(reinterpret_cast<T*>(jb.dst[l]) + v * VEC) = S::pack(f[l]);
+    }
+}
+
 // ----- C2: threshold from a histogram --------------------------------------------------------------
 // One CTA per unit-tensor.  Scans `nbins` bins from the top: finds the bin where the running count of larger
 // keys first reaches k_rem, appends the bin to the prefix and lowers k_rem.  Clears the bins it read.
@@ -291,6 +392,38 @@ cudaError_t launch_split_hist(const CompressArgs& a, int dtype, cudaStream_t st)
     else
         split_hist_kernel<float><<<grid, 1024, smem, st>>>(a, tokens_per_cta);
     count_launch(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_split_rows(const SplitRowsArgs& a, int B, int dtype, cudaStream_t st) {
+    if (a.T <= 0 || a.n_blocks <= 0) return cudaSuccess;
+    const int per_block = 2 * 256 * (dtype == FDKV_BF16 ? 8 : 4);  // elements one thread block covers
+    dim3 grid((unsigned)(((int64_t)a.T * a.d + per_block - 1) / per_block), a.Hkv * 2, a.n_blocks);
+    if (dtype == FDKV_BF16) {
+        if (B == 4) split_rows_kernel<__nv_bfloat16, 4><<<grid, 256, 0, st>>>(a);
+        else split_rows_kernel<__nv_bfloat16, 2><<<grid, 256, 0, st>>>(a);
+    } else {
+        if (B == 4) split_rows_kernel<float, 4><<<grid, 256, 0, st>>>(a);
+        else split_rows_kernel<float, 2><<<grid, 256, 0, st>>>(a);
+    }
+    count_launch(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_token_gather_jobs(const TokenGatherJob* jobs_dev, int njobs, int64_t k_tok, int d, int B, int dtype, cudaStream_t st) {
+    if (njobs <= 0 || k_tok <= 0) return cudaSuccess;
+    const int64_t nvec = k_tok * (d / (dtype == FDKV_BF16 ? 8 : 4));
+    for (int j0 = 0; j0 < njobs; j0 += 65535) {
+        const dim3 grid((unsigned)((nvec + 255) / 256), std::min(njobs - j0, 65535));
+        if (dtype == FDKV_BF16) {
+            if (B == 4) token_gather_kernel<__nv_bfloat16, 4><<<grid, 256, 0, st>>>(jobs_dev + j0, d);
+            else token_gather_kernel<__nv_bfloat16, 2><<<grid, 256, 0, st>>>(jobs_dev + j0, d);
+        } else {
+            if (B == 4) token_gather_kernel<float, 4><<<grid, 256, 0, st>>>(jobs_dev + j0, d);
+            else token_gather_kernel<float, 2><<<grid, 256, 0, st>>>(jobs_dev + j0, d);
+        }
+        count_launch(1);
+    }
     return cudaGetLastError();
 }
 

@@ -146,6 +146,20 @@ struct CompressArgs {
 };
 cudaError_t launch_split_hist(const CompressArgs& a, int dtype, cudaStream_t st);
 
+// The split alone (token rule), either block size; layer B * j + l is layer l of the launch's block j.
+constexpr int kSplitLayers = 64;  // layers one launch covers
+struct SplitRowsArgs {
+    const void *k[kSplitLayers], *v[kSplitLayers];
+    int n_blocks;
+    int64_t stride_t, stride_h;
+    int T, d, Hkv;
+    int ut_base;          // first unit-tensor of the first block
+    int64_t unit_stride;  // elements between staged tensors (Tmax*d)
+    void* z0;             // [NT][unit_stride]
+    void* hf;             // [NT][1 or 4][unit_stride]: Z1 of a pair, or the layers' deviations of a block of four; K tensors only
+};
+cudaError_t launch_split_rows(const SplitRowsArgs& a, int B, int dtype, cudaStream_t st);
+
 struct SelectArgs {
     int ut_begin, ut_count;
     int T, d;
@@ -282,6 +296,15 @@ struct CopyJob {
     int64_t src_pitch;
     int32_t row_bytes, pad_;
 };
+// Token rule: the selected tokens' high-frequency rows of one unit-tensor, formed from the caller's rows of the block's layers.
+struct TokenGatherJob {
+    const void* x[4];   // layer rows of the head (element (t, c) at t*stride_t + c); two for a pair
+    void* dst[4];       // one stored tensor for a pair, four for a block of four
+    const int32_t* list;
+    int64_t stride_t, k_tok;
+    int32_t twice, pad_;
+};
+cudaError_t launch_token_gather_jobs(const TokenGatherJob* jobs_dev, int njobs, int64_t k_tok, int d, int B, int dtype, cudaStream_t st);
 cudaError_t plan_decode_host(const DecodeArgs& a, int n_ctas, uint32_t* start_out, int32_t* ncta_out, int32_t* parts_out);
 cudaError_t launch_copy_jobs(const CopyJob* jobs_dev, int njobs, int64_t bytes_max, cudaStream_t st);
 cudaError_t launch_quantise_jobs(const QuantJob* jobs_dev, int njobs, int T_max, cudaStream_t st);
@@ -317,7 +340,6 @@ struct TokenArgs {
 inline int token_err_slots(int B, int G, bool tensor_core, int W) { return tensor_core ? B * ((G * W + 255) / 256) : 1; }
 // tensor_core: bf16 / head_dim 128 contexts (tcgen05 score kernel); otherwise the float32 score kernel
 cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tensor_core, cudaStream_t st);
-cudaError_t launch_token_gather(const void* z1, const int32_t* list, int64_t k_tok, void* out, int row_bytes, int twice, cudaStream_t st);
 
 // Function attributes (the opt-in to large dynamic shared memory) and the SM count belong to a device, not to the
 // process: every launcher keeps one of these and runs its set-up the first time it meets the current device.

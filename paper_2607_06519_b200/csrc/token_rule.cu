@@ -18,7 +18,7 @@
 //    selected rows zeroed to run one of them on: 8 191 tokens, 8 blocks of four: the probe 627 -> 250 us).
 // 2. token_select_kernel: per unit an MSB-first radix select (4 x 8 bits) of the k_tok-th largest score and an
 //    index-ordered compaction: ascending token list, per-16-token-slice counts, and the two error sums in float64.
-// 3. token_gather_kernel (commit): the selected rows of Z1, densely packed.
+// (The commit step forms the selected rows from the caller's K and V: token_gather_kernel in compress.cu.)
 #include <cuda.h>
 
 #include <algorithm>
@@ -363,22 +363,6 @@ __global__ void __launch_bounds__(1024) token_select_kernel(TokenArgs a) {
     }
 }
 
-// out[j][:] = z1[list[j]][:] (rows of row_u4 16-byte vectors), optionally doubled (bf16 rows of the tensor-core decode
-// kernel only; exact): a block of four scales its rows by 1/2 at decode time and its deviations by 1, so their stored
-// rows carry the factor 2
-__global__ void __launch_bounds__(256) token_gather_kernel(const uint4* z1, const int32_t* list, int64_t k_tok, uint4* out, int row_u4,
-                                                           int twice) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < k_tok * row_u4; v += (int64_t)gridDim.x * blockDim.x) {
-        uint4 x = z1[(int64_t)list[v / row_u4] * row_u4 + (v % row_u4)];
-        if (twice) {
-            __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&x);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) h[i] = __hadd2(h[i], h[i]);
-        }
-        out[v] = x;
-    }
-}
-
 // ---- storage types and head dimensions without the tensor-core kernel: the same score as a float32 product ----
 template <typename T>
 __device__ __forceinline__ float to_f32(T x);
@@ -497,15 +481,6 @@ cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tenso
     count_launch(2);
     count_kernel(FDKV_KERNEL_TOKEN_SCORE);
     count_kernel(FDKV_KERNEL_PROBE_TC);  // (it is the probe's product too)
-    return cudaGetLastError();
-}
-
-cudaError_t launch_token_gather(const void* z1, const int32_t* list, int64_t k_tok, void* out, int row_bytes, int twice, cudaStream_t st) {
-    if (k_tok <= 0) return cudaSuccess;
-    const int row_u4 = row_bytes / 16;
-    const int blocks = (int)std::min<int64_t>(256, (k_tok * row_u4 + 255) / 256);
-    token_gather_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const uint4*>(z1), list, k_tok, reinterpret_cast<uint4*>(out), row_u4, twice);
-    count_launch(1);
     return cudaGetLastError();
 }
 
