@@ -69,6 +69,7 @@ bool make_shape(const fdkv_config& c, Shape& s) {
 
 constexpr size_t quant_table_bytes(const Shape& s) { return s.rows_f8 ? (size_t)s.NU * 2 * s.B * (sizeof(QuantJob) + sizeof(RepackJob)) : 0; }
 constexpr size_t gather_table_bytes(const Shape& s) { return s.tok_rule ? (size_t)s.NU * 2 * sizeof(TokenGatherJob) : 0; }
+constexpr size_t max_copy_jobs(const Shape& s) { return (size_t)s.NU * (4 * s.B + 8 + 4 * s.NB); }
 
 void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     size_t o = 0;
@@ -103,9 +104,9 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     w.io_v = take((size_t)s.L * s.max_batch * s.Hkv * s.d * 4);
     w.io_out = take((size_t)s.L * s.max_batch * s.Hq * s.d * 4);
     // job tables of a commit: quantise jobs (one per stored tensor) and repack jobs (one per residual list) of 8-bit rows,
-    // gather jobs of the token rule, then the copy jobs (at most 2 B row copies, or 2 row copies, 2 offset tables and 2 NB
-    // lists, per unit)
-    w.jobs = take(quant_table_bytes(s) + gather_table_bytes(s) + (size_t)s.NU * (2 * s.B + 4 + 2 * s.NB) * sizeof(CopyJob));
+    // gather jobs of the token rule, then the copy jobs (at most 2 B row copies with a fill each, or 2 row copies and fills,
+    // 2 offset tables, 2 index and 2 NB value or packed lists, per unit)
+    w.jobs = take(quant_table_bytes(s) + gather_table_bytes(s) + max_copy_jobs(s) * sizeof(CopyJob));
     w.total = o;
 
     o = 0;
@@ -564,12 +565,13 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
     std::vector<QuantJob> qjobs;   // 8-bit rows: every stored tensor is quantised by one batched pass after this loop
     std::vector<RepackJob> rjobs;  // ... and every residual list repacked relative to its tensor's scales
     std::vector<TokenGatherJob> gjobs;  // token rule: the selected rows, formed from the caller's K and V
-    std::vector<CopyJob> cjobs;    // device-to-device copies into the arena: one launch over this table after the loop
-    int64_t copy_max = 0;
-    auto copy_job = [&](const void* src, void* dst, size_t bytes, int64_t src_pitch, int row_bytes) {
-        cjobs.push_back(CopyJob{(const char*)src, (char*)dst, (int64_t)bytes, src_pitch, row_bytes, 0});
-        copy_max = std::max<int64_t>(copy_max, (int64_t)bytes);
+    // device-to-device copies into the arena and zero fills: one launch per class of size after the loop
+    enum { kRowJobs, kListJobs, kSmallJobs, kJobClasses };
+    std::vector<CopyJob> cjobs[kJobClasses];
+    auto copy_job = [&](int cls, const void* src, void* dst, size_t bytes, int64_t src_pitch, int row_bytes) {
+        cjobs[cls].push_back(CopyJob{(const char*)src, (char*)dst, (int64_t)bytes, src_pitch, row_bytes, 0});
     };
+    auto zero_job = [&](void* dst, size_t bytes) { if (bytes) copy_job(kSmallJobs, nullptr, dst, bytes, 16, 16); };
     for (int u = 0; u < s.NU; ++u) {
         const int m = q.modes[u], p = u / s.Hkv, h = u % s.Hkv;
         UnitDesc* dl[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -589,7 +591,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                     if (s.rows_f8) {
                         char* dst = take(rows8_pad);
                         float* sc = reinterpret_cast<float*>(take(scale_slot));
-                        if (rows8_pad > rows8) CU(cudaMemsetAsync(dst + rows8, 0, rows8_pad - rows8, st));
+                        zero_job(dst + rows8, rows8_pad - rows8);
                         qjobs.push_back(QuantJob{sp, c->stride_t, T, 0, reinterpret_cast<uint8_t*>(dst), sc});
                         (is_v ? dl[l]->v_rows : dl[l]->k_rows) = dst;
                         (is_v ? dl[l]->v_scale : dl[l]->k_scale) = sc;
@@ -597,8 +599,8 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                         continue;
                     }
                     char* dst = take(rows_pad);
-                    if (rows_pad > rows) CU(cudaMemsetAsync(dst + rows, 0, rows_pad - rows, st));
-                    copy_job(sp, dst, rows, (int64_t)c->stride_t * s.esize, s.d * s.esize);
+                    zero_job(dst + rows, rows_pad - rows);
+                    copy_job(kRowJobs, sp, dst, rows, (int64_t)c->stride_t * s.esize, s.d * s.esize);
                     (is_v ? dl[l]->v_rows : dl[l]->k_rows) = dst;
                 }
             by_mode[2] += 2 * (size_t)s.B * (s.rows_f8 ? rows8 + 512 : rows);
@@ -607,8 +609,8 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
             if (s.tok_rule && m == FDKV_MODE_RESIDUAL) {  // one token list and one offset table serve K and V
                 tl = take(tlist_b);
                 to = take(off_b);
-                copy_job(c->work + c->ws.tok_list + (size_t)u * s.ktok_cap * 4, tl, (size_t)k_tok * 4, 16, 16);
-                copy_job(c->work + c->ws.tok_off + (size_t)u * (s.ntiles_max + 1) * 4, to, off_copy, 16, 16);
+                copy_job(kSmallJobs, c->work + c->ws.tok_list + (size_t)u * s.ktok_cap * 4, tl, (size_t)k_tok * 4, 16, 16);
+                copy_job(kSmallJobs, c->work + c->ws.tok_off + (size_t)u * (s.ntiles_max + 1) * 4, to, off_copy, 16, 16);
                 by_mode[1] += (size_t)k_tok * 4;
             }
             for (int is_v = 0; is_v < 2; ++is_v) {
@@ -618,13 +620,13 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                 if (s.rows_f8) {
                     z0 = take(rows8_pad);
                     sc8 = reinterpret_cast<float*>(take(scale_slot));
-                    if (rows8_pad > rows8) CU(cudaMemsetAsync(z0 + rows8, 0, rows8_pad - rows8, st));
+                    zero_job(z0 + rows8, rows8_pad - rows8);
                     qjobs.push_back(QuantJob{c->work + c->ws.z0 + ut * unit_stride_b, s.d, T, 0, reinterpret_cast<uint8_t*>(z0), sc8});
                     for (int l = 0; l < s.B; ++l) { (is_v ? dl[l]->v_scale : dl[l]->k_scale) = sc8; dl[l]->rows_f8 = 1; }
                 } else {
                     z0 = take(rows_pad);
-                    if (rows_pad > rows) CU(cudaMemsetAsync(z0 + rows, 0, rows_pad - rows, st));
-                    copy_job(c->work + c->ws.z0 + ut * unit_stride_b, z0, rows, 16, 16);
+                    zero_job(z0 + rows, rows_pad - rows);
+                    copy_job(kRowJobs, c->work + c->ws.z0 + ut * unit_stride_b, z0, rows, 16, 16);
                 }
                 for (int l = 0; l < s.B; ++l) (is_v ? dl[l]->v_rows : dl[l]->k_rows) = z0;
                 by_mode[m] += s.rows_f8 ? rows8 + 512 : rows;
@@ -656,11 +658,11 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                     by_mode[1] += (size_t)s.NB * k_tok * s.d * s.esize;
                 } else if (m == FDKV_MODE_RESIDUAL) {
                     char* po = take(off_b);
-                    copy_job(c->work + c->ws.tile_off + ut * (s.ntiles_max + 1) * 4, po, off_copy, 16, 16);
+                    copy_job(kSmallJobs, c->work + c->ws.tile_off + ut * (s.ntiles_max + 1) * 4, po, off_copy, 16, 16);
                     char* pi_shared = nullptr;
                     if (!c->packed_lists) {
                         pi_shared = take(idx_b);
-                        CU(cudaMemcpyAsync(pi_shared, c->work + c->ws.idx + ut * s.kcap * 4, idx_copy, cudaMemcpyDeviceToDevice, st));
+                        copy_job(kListJobs, c->work + c->ws.idx + ut * s.kcap * 4, pi_shared, idx_copy, 16, 16);
                     }
                     char *pi_l[4] = {nullptr, nullptr, nullptr, nullptr}, *pv_l[4] = {nullptr, nullptr, nullptr, nullptr};
                     for (int j = 0; j < s.NB; ++j) {  // one list per stored high-frequency tensor
@@ -670,11 +672,12 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                             if (s.rows_f8)  // values relative to the channel scales, positions in the converted fragments' order
                                 rjobs.push_back(RepackJob{reinterpret_cast<uint32_t*>(pi_l[j]), wsp<uint32_t>(c, c->ws.packed) + lt * s.kcap, k, sc8, is_v, 0});
                             else
-                                copy_job(c->work + c->ws.packed + lt * s.kcap * 4, pi_l[j], idx_copy, 16, 16);
+                                copy_job(kListJobs, c->work + c->ws.packed + lt * s.kcap * 4, pi_l[j], idx_copy, 16, 16);
                         } else {
                             pi_l[j] = pi_shared;
                             pv_l[j] = take(val_b);
-                            CU(cudaMemcpyAsync(pv_l[j], c->work + c->ws.val + lt * s.kcap * s.esize, val_copy, cudaMemcpyDeviceToDevice, st));
+                            // (whole words: an odd count of 2-byte values takes one value of the list's slack along)
+                            copy_job(kListJobs, c->work + c->ws.val + lt * s.kcap * s.esize, pv_l[j], (val_copy + 3) & ~(size_t)3, 16, 16);
                         }
                     }
                     for (int l = 0; l < s.B; ++l) {
@@ -694,10 +697,15 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
         CU(cudaMemcpyAsync(table, gjobs.data(), gjobs.size() * sizeof(TokenGatherJob), cudaMemcpyHostToDevice, st));
         CU(launch_token_gather_jobs(reinterpret_cast<TokenGatherJob*>(table), (int)gjobs.size(), k_tok, s.d, s.B, s.dtype, st));
     }
-    if (!cjobs.empty()) {
-        CopyJob* cd = reinterpret_cast<CopyJob*>(table + gather_table_bytes(s));
-        CU(cudaMemcpyAsync(cd, cjobs.data(), cjobs.size() * sizeof(CopyJob), cudaMemcpyHostToDevice, st));
-        CU(launch_copy_jobs(cd, (int)cjobs.size(), copy_max, st));
+    CopyJob* cd = reinterpret_cast<CopyJob*>(table + gather_table_bytes(s));
+    std::vector<CopyJob> all;
+    for (const auto& v : cjobs) all.insert(all.end(), v.begin(), v.end());
+    if (!all.empty()) CU(cudaMemcpyAsync(cd, all.data(), all.size() * sizeof(CopyJob), cudaMemcpyHostToDevice, st));
+    for (const auto& v : cjobs) {
+        int64_t most = 0;
+        for (const CopyJob& jb : v) most = std::max(most, jb.bytes);
+        CU(launch_copy_jobs(cd, (int)v.size(), most, st));
+        cd += v.size();
     }
     if (!qjobs.empty()) {
         QuantJob* qd = reinterpret_cast<QuantJob*>(c->work + c->ws.jobs);

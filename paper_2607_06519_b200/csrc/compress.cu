@@ -359,20 +359,6 @@ __global__ void __launch_bounds__(256) refine_candidates_kernel(int ut_begin, co
 
 // (C3-C5, the index-ordered compaction, live in select_fused.cu.)
 
-template <typename T>
-__global__ void strided_copy_kernel(const T* src, int64_t stride_t, T* dst, int T_, int d) {
-    using S = Store<T>;
-    constexpr int VEC = S::VEC;
-    const int vpr = d / VEC;
-    const int64_t n = (int64_t)T_ * vpr;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = v / vpr;
-        const int cv = (int)(v % vpr) * VEC;
-        *reinterpret_cast<typename S::vec_t*>(dst + t * d + cv) =
-            *reinterpret_cast<const typename S::vec_t*>(src + t * stride_t + cv);
-    }
-}
-
 }  // namespace
 
 cudaError_t launch_split_hist(const CompressArgs& a, int dtype, cudaStream_t st) {
@@ -452,14 +438,19 @@ cudaError_t launch_select_and_compact(const SelectArgs& a, int dtype, cudaStream
     return launch_select_fused(a, dtype, st);
 }
 
-// grid (chunks of 32 KiB, jobs): the device-to-device copies of a commit (row streams, strided source rows of exact
-// units, residual lists, offset tables) as one launch instead of several hundred copy calls
+// grid (chunks of 32 KiB of the largest job, jobs): the device-to-device copies of a commit (row streams, strided source
+// rows of exact units, residual lists, offset tables) and its zero fills as one launch per class of job size, so that
+// few blocks find nothing to do, instead of several hundred copy and fill calls of about 1.2 us each on the host and on the device
 constexpr int kCopyChunk = 32 * 1024;
 __global__ void __launch_bounds__(256) copy_jobs_kernel(const CopyJob* jobs) {
     const CopyJob jb = jobs[blockIdx.y];
     const int64_t c0 = (int64_t)blockIdx.x * kCopyChunk;
     if (c0 >= jb.bytes) return;
     const int64_t c1 = min(jb.bytes, c0 + kCopyChunk);
+    if (!jb.src) {
+        for (int64_t o = c0 + threadIdx.x * 4; o < c1; o += 256 * 4) *reinterpret_cast<uint32_t*>(jb.dst + o) = 0u;
+        return;
+    }
     const bool plain = jb.src_pitch == jb.row_bytes;
     auto src_of = [&](int64_t o) {
         if (plain) return o;
@@ -476,9 +467,10 @@ __global__ void __launch_bounds__(256) copy_jobs_kernel(const CopyJob* jobs) {
         *reinterpret_cast<uint32_t*>(jb.dst + o) = *reinterpret_cast<const uint32_t*>(jb.src + src_of(o));
 }
 cudaError_t launch_copy_jobs(const CopyJob* jobs_dev, int njobs, int64_t bytes_max, cudaStream_t st) {
-    if (njobs <= 0 || bytes_max <= 0) return cudaSuccess;
-    copy_jobs_kernel<<<dim3((unsigned)((bytes_max + kCopyChunk - 1) / kCopyChunk), njobs), 256, 0, st>>>(jobs_dev);
-    count_launch(1);
+    for (int j0 = 0; j0 < njobs && bytes_max > 0; j0 += 65535) {
+        copy_jobs_kernel<<<dim3((unsigned)((bytes_max + kCopyChunk - 1) / kCopyChunk), std::min(njobs - j0, 65535)), 256, 0, st>>>(jobs_dev + j0);
+        count_launch(1);
+    }
     return cudaGetLastError();
 }
 
@@ -489,21 +481,6 @@ __global__ void offset_copy_kernel(int32_t* dst, const int32_t* src, int n, int 
 cudaError_t launch_offset_copy(int32_t* dst, const int32_t* src, int n, int add, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     offset_copy_kernel<<<(n + 255) / 256, 256, 0, st>>>(dst, src, n, add);
-    count_launch(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_strided_copy(const void* src, int64_t stride_t, void* dst, int T, int d, int esize, cudaStream_t st) {
-    if (T <= 0) return cudaSuccess;
-    const int vec = esize == 2 ? 8 : 4;
-    const int64_t n = (int64_t)T * (d / vec);
-    const int blocks = (int)std::min<int64_t>(148 * 8, (n + 255) / 256);
-    if (esize == 2)
-        strided_copy_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(src), stride_t,
-                                                                  reinterpret_cast<__nv_bfloat16*>(dst), T, d);
-    else
-        strided_copy_kernel<float><<<blocks, 256, 0, st>>>(reinterpret_cast<const float*>(src), stride_t,
-                                                           reinterpret_cast<float*>(dst), T, d);
     count_launch(1);
     return cudaGetLastError();
 }

@@ -287,8 +287,8 @@ struct RepackJob {
     int32_t is_v, rows;
 };
 // One copy of the commit step: dst[0, bytes) = consecutive rows of row_bytes taken every src_pitch bytes from src
-// (row_bytes == src_pitch: a plain copy).  Pointers 16-byte aligned, row_bytes and src_pitch multiples of 16, bytes a
-// multiple of 4.  All copies of a commit run as one launch over a job table.
+// (row_bytes == src_pitch: a plain copy; src null: zeros).  Pointers 16-byte aligned, row_bytes and src_pitch multiples of
+// 16, bytes a multiple of 4.  All copies of a commit run as one launch per size class over a job table.
 struct CopyJob {
     const char* src;
     char* dst;
@@ -313,7 +313,6 @@ bool make_rows_tensor_map_u8(void* base, size_t bytes, int box_rows, void* tmap_
 
 // dst[i] = src[i] + add, i < n (list offsets and indices of a folded chunk)
 cudaError_t launch_offset_copy(int32_t* dst, const int32_t* src, int n, int add, cudaStream_t st);
-cudaError_t launch_strided_copy(const void* src, int64_t stride_t, void* dst, int T, int d, int esize, cudaStream_t st);
 
 // ---- token-granular residual (token_rule.cu) ----
 struct TokenArgs {
