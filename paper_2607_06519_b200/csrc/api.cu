@@ -69,7 +69,7 @@ bool make_shape(const fdkv_config& c, Shape& s) {
 
 constexpr size_t quant_table_bytes(const Shape& s) { return s.rows_f8 ? (size_t)s.NU * 2 * s.B * (sizeof(QuantJob) + sizeof(RepackJob)) : 0; }
 constexpr size_t gather_table_bytes(const Shape& s) { return s.tok_rule ? (size_t)s.NU * 2 * sizeof(TokenGatherJob) : 0; }
-constexpr size_t max_copy_jobs(const Shape& s) { return (size_t)s.NU * (4 * s.B + 8 + 4 * s.NB); }
+constexpr size_t max_copy_jobs(const Shape& s) { return (size_t)s.NU * (4 * s.B + 10 + 4 * s.NB); }
 
 void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     size_t o = 0;
@@ -132,6 +132,11 @@ template <typename T>
 inline T* wsp(fdkv_ctx* c, size_t off) { return reinterpret_cast<T*>(c->work + off); }
 template <typename T>
 inline T* arp(fdkv_ctx* c, size_t off) { return reinterpret_cast<T*>(c->arena + off); }
+
+// One committed row stream of T tokens: whole boxes, with room for the tokens fdkv_fold_tail may append later.
+size_t row_stream_bytes(const Shape& s, int T) {
+    return (size_t)((T + s.max_fold + kRowPad - 1) / kRowPad * kRowPad) * s.d * s.esize;
+}
 
 bool seq_ok(fdkv_ctx* c, int seq) { return c && seq >= 0 && seq < c->s.max_batch; }
 
@@ -274,6 +279,15 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
         c->seqs[seq].modes.assign(s.NU, -1);
         c->stride_t = stride_t;
         c->stride_h = stride_h;
+        // Every unit's committed form holds at least two row streams, so the shared coefficients go where commit would
+        // put them (shared / residual units keep them there; an exact unit's two slots take two of its own streams): commit
+        // then copies nothing for most units.  A full arena, or rows that commit quantises, stage them in the workspace.
+        const size_t stream = align_up(row_stream_bytes(s, T));
+        c->z0_in_arena = !s.rows_f8 && c->bump + (size_t)s.NT * stream <= c->arena_bytes;
+        c->z0_base = c->z0_in_arena ? c->arena + c->bump : c->work + c->ws.z0;
+        c->z0_stride = c->z0_in_arena ? stream : (size_t)s.Tmax * s.d * s.esize;
+        c->z0_loc.resize(s.NT);
+        for (int ut = 0; ut < s.NT; ++ut) c->z0_loc[ut] = c->z0_base + ut * c->z0_stride;
     } else if (c->stride_t != stride_t || c->stride_h != stride_h) {
         return FDKV_ERR_INVALID_ARG;
     }
@@ -292,8 +306,8 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
             a.stride_t = stride_t; a.stride_h = stride_h;
             a.T = T; a.d = s.d; a.Hkv = s.Hkv;
             a.ut_base = p0 * s.Hkv * 2;
-            a.unit_stride = (int64_t)s.Tmax * s.d;
-            a.z0 = c->work + c->ws.z0; a.hf = c->work + c->ws.z1;
+            a.unit_stride = (int64_t)s.Tmax * s.d; a.z0_stride = (int64_t)(c->z0_stride / s.esize);
+            a.z0 = c->z0_base; a.hf = c->work + c->ws.z1;
             CU(launch_split_rows(a, s.B, s.dtype, st));
         }
         for (int p = pb; p < pe; ++p) { c->pair_compressed[p] = 1; c->pair_probed[p] = 0; c->pair_scored[p] = 0; }
@@ -314,8 +328,8 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
             a4.stride_t = stride_t; a4.stride_h = stride_h;
             a4.T = T; a4.d = s.d; a4.Hkv = s.Hkv;
             a4.ut_base = p * s.Hkv * 2;
-            a4.unit_stride = (int64_t)s.Tmax * s.d;
-            a4.z0 = c->work + c->ws.z0; a4.dev = c->work + c->ws.z1;
+            a4.unit_stride = (int64_t)s.Tmax * s.d; a4.z0_stride = (int64_t)(c->z0_stride / s.esize);
+            a4.z0 = c->z0_base; a4.dev = c->work + c->ws.z1;
             a4.energy = wsp<float>(c, c->ws.energy);
             a4.drop = c->has_probe_tmaps ? c->work + c->ws.z1drop : nullptr;
             a4.hist = wsp<uint32_t>(c, c->ws.hist);
@@ -363,8 +377,8 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
         a.stride_t = stride_t; a.stride_h = stride_h;
         a.T = T; a.d = s.d; a.Hkv = s.Hkv; a.tensors = 2;
         a.ut_base = p0 * s.Hkv * 2;
-        a.unit_stride = (int64_t)s.Tmax * s.d;
-        a.z0 = c->work + c->ws.z0; a.z1 = c->work + c->ws.z1;
+        a.unit_stride = (int64_t)s.Tmax * s.d; a.z0_stride = (int64_t)(c->z0_stride / s.esize);
+        a.z0 = c->z0_base; a.z1 = c->work + c->ws.z1;
         a.hist = wsp<uint32_t>(c, c->ws.hist);
         CU(launch_split_hist(a, s.dtype, st));
     }
@@ -531,8 +545,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
         CU(cudaMemcpy(q.modes.data(), c->work + c->ws.modes, (size_t)s.NU * 4, cudaMemcpyDeviceToHost));
     const int T = c->staged_T;
     const size_t rows = (size_t)T * s.d * s.esize;
-    // zero rows up to a whole box, with room for the tokens fdkv_fold_tail may append later
-    const size_t rows_pad = (size_t)((T + s.max_fold + kRowPad - 1) / kRowPad * kRowPad) * s.d * s.esize;
+    const size_t rows_pad = row_stream_bytes(s, T);  // (zero rows up to its end)
     const int64_t k = (int64_t)T * s.d * s.keep_num / s.keep_den;
     const int ntiles = (T + kResTile - 1) / kResTile;
     // list copies include the slack so that aligned over-reads of the last tile stay inside the allocation
@@ -558,7 +571,8 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
         else need += 2 * stream_b + (m == FDKV_MODE_RESIDUAL ? 2 * (lists_b + align_up(off_b)) : 0);
     }
     if (c->bump + need > c->arena_bytes) return FDKV_ERR_ARENA_FULL;
-    size_t o = c->bump;
+    const bool in_place = c->z0_in_arena;
+    size_t o = c->bump + (in_place ? (size_t)s.NT * c->z0_stride : 0);
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return c->arena + r; };
     size_t by_mode[3] = {0, 0, 0};
     const size_t unit_stride_b = (size_t)s.Tmax * s.d * s.esize;
@@ -566,7 +580,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
     std::vector<RepackJob> rjobs;  // ... and every residual list repacked relative to its tensor's scales
     std::vector<TokenGatherJob> gjobs;  // token rule: the selected rows, formed from the caller's K and V
     // device-to-device copies into the arena and zero fills: one launch per class of size after the loop
-    enum { kRowJobs, kListJobs, kSmallJobs, kJobClasses };
+    enum { kSaveJobs, kRowJobs, kListJobs, kSmallJobs, kJobClasses };  // (in launch order)
     std::vector<CopyJob> cjobs[kJobClasses];
     auto copy_job = [&](int cls, const void* src, void* dst, size_t bytes, int64_t src_pitch, int row_bytes) {
         cjobs[cls].push_back(CopyJob{(const char*)src, (char*)dst, (int64_t)bytes, src_pitch, row_bytes, 0});
@@ -598,7 +612,15 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                         dl[l]->rows_f8 = 1;
                         continue;
                     }
-                    char* dst = take(rows_pad);
+                    char* dst;
+                    if (in_place && l == 0) {  // the unit's own Z0 slot; its Z0 stays readable in the workspace
+                        const size_t ut = (size_t)u * 2 + is_v;
+                        dst = c->z0_base + ut * c->z0_stride;
+                        c->z0_loc[ut] = c->work + c->ws.z0 + ut * unit_stride_b;
+                        copy_job(kSaveJobs, dst, c->z0_loc[ut], rows, 16, 16);
+                    } else {
+                        dst = take(rows_pad);
+                    }
                     zero_job(dst + rows, rows_pad - rows);
                     copy_job(kRowJobs, sp, dst, rows, (int64_t)c->stride_t * s.esize, s.d * s.esize);
                     (is_v ? dl[l]->v_rows : dl[l]->k_rows) = dst;
@@ -624,9 +646,9 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                     qjobs.push_back(QuantJob{c->work + c->ws.z0 + ut * unit_stride_b, s.d, T, 0, reinterpret_cast<uint8_t*>(z0), sc8});
                     for (int l = 0; l < s.B; ++l) { (is_v ? dl[l]->v_scale : dl[l]->k_scale) = sc8; dl[l]->rows_f8 = 1; }
                 } else {
-                    z0 = take(rows_pad);
+                    z0 = in_place ? c->z0_base + ut * c->z0_stride : take(rows_pad);
                     zero_job(z0 + rows, rows_pad - rows);
-                    copy_job(kRowJobs, c->work + c->ws.z0 + ut * unit_stride_b, z0, rows, 16, 16);
+                    if (!in_place) copy_job(kRowJobs, c->z0_loc[ut], z0, rows, 16, 16);
                 }
                 for (int l = 0; l < s.B; ++l) (is_v ? dl[l]->v_rows : dl[l]->k_rows) = z0;
                 by_mode[m] += s.rows_f8 ? rows8 + 512 : rows;
@@ -888,7 +910,7 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
             a4.stride_t = s.d; a4.stride_h = (int64_t)s.tail_rows * s.d;
             a4.T = n; a4.d = s.d; a4.Hkv = s.Hkv;
             a4.ut_base = p * s.Hkv * 2;
-            a4.unit_stride = (int64_t)s.Tmax * s.d;
+            a4.unit_stride = a4.z0_stride = (int64_t)s.Tmax * s.d;
             a4.z0 = c->work + c->ws.z0; a4.dev = c->work + c->ws.z1;
             a4.energy = wsp<float>(c, c->ws.energy);
             a4.drop = nullptr;
@@ -920,7 +942,7 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
             a.stride_t = s.d; a.stride_h = (int64_t)s.tail_rows * s.d;
             a.T = n; a.d = s.d; a.Hkv = s.Hkv; a.tensors = 2;
             a.ut_base = p0 * s.Hkv * 2;
-            a.unit_stride = (int64_t)s.Tmax * s.d;
+            a.unit_stride = a.z0_stride = (int64_t)s.Tmax * s.d;
             a.z0 = c->work + c->ws.z0; a.z1 = c->work + c->ws.z1;
             a.hist = wsp<uint32_t>(c, c->ws.hist);
             CU(launch_split_hist(a, s.dtype, st));
@@ -1014,7 +1036,7 @@ fdkv_status fdkv_get_shared(fdkv_ctx* c, int32_t seq, int32_t pair, int32_t h, i
     if (c->staged_seq != seq || !c->pair_compressed[pair]) return FDKV_ERR_STATE;
     const Shape& s = c->s;
     const size_t ut = ((size_t)pair * s.Hkv + h) * 2 + (is_v ? 1 : 0);
-    CU(cudaMemcpyAsync(z0_out, c->work + c->ws.z0 + ut * s.Tmax * s.d * s.esize, (size_t)c->staged_T * s.d * s.esize,
+    CU(cudaMemcpyAsync(z0_out, c->z0_loc[ut], (size_t)c->staged_T * s.d * s.esize,
                        cudaMemcpyDeviceToDevice, S(stream)));
     CU(cudaStreamSynchronize(S(stream)));
     return FDKV_OK;

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(512) split4_hist_kernel(Split4Args a, int toke
     const T* x[4];
 #pragma unroll
     for (int l = 0; l < 4; ++l) x[l] = reinterpret_cast<const T*>(is_v ? a.v[l] : a.k[l]) + (int64_t)h * a.stride_h;
-    T* z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.unit_stride;
+    T* z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride;
     T* dev = reinterpret_cast<T*>(a.dev) + (int64_t)ut * 4 * a.unit_stride;
     float* en = a.energy + (int64_t)ut * a.unit_stride;
     T* drop = (a.drop && !is_v) ? reinterpret_cast<T*>(a.drop) + (int64_t)(ut >> 1) * 4 * a.unit_stride : nullptr;

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(1024) split_hist_kernel(CompressArgs a, int to
     const int ut = a.ut_base + pj * a.Hkv * a.tensors + blockIdx.y;
     const T* x0 = reinterpret_cast<const T*>(is_v ? a.v0[pj] : a.k0[pj]) + (int64_t)h * a.stride_h;
     const T* x1 = reinterpret_cast<const T*>(is_v ? a.v1[pj] : a.k1[pj]) + (int64_t)h * a.stride_h;
-    T* z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.unit_stride;
+    T* z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride;
     T* z1 = reinterpret_cast<T*>(a.z1) + (int64_t)ut * a.unit_stride;
     const float c32 = __uint_as_float(0x3F3504F3u);
 
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(SplitRowsArgs a) {
     constexpr int NV = 2;
     const int h = blockIdx.y >> 1, is_v = blockIdx.y & 1, blk = blockIdx.z;
     const int64_t ut = a.ut_base + (int64_t)blk * a.Hkv * 2 + blockIdx.y;
-    T* const z0 = reinterpret_cast<T*>(a.z0) + ut * a.unit_stride;
+    T* const z0 = reinterpret_cast<T*>(a.z0) + ut * a.z0_stride;
     T* const hf = reinterpret_cast<T*>(a.hf) + ut * (B == 4 ? 4 : 1) * a.unit_stride;
     const float c32 = __uint_as_float(0x3F3504F3u);
     const int vpr = a.d / VEC;
@@ -564,7 +564,7 @@ extern "C" fdkv_status fdkv_compress_unit_noalloc(const void* x0, const void* x1
     a.n_pairs = 1;
     a.stride_t = stride_t; a.stride_h = 0;
     a.T = T; a.d = head_dim; a.Hkv = 1; a.tensors = 1;
-    a.ut_base = 0; a.unit_stride = 0;
+    a.ut_base = 0; a.unit_stride = 0; a.z0_stride = 0;
     a.z0 = z0_out; a.z1 = sc + kNaZ1;
     a.hist = reinterpret_cast<uint32_t*>(sc + kNaHist);
     if ((e = launch_split_hist(a, dtype, st)) != cudaSuccess) return record_cuda_error(e);

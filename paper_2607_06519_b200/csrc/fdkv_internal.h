@@ -112,6 +112,12 @@ struct fdkv_ctx {
     int staged_seq = -1;
     int staged_T = 0;
     std::vector<uint8_t> pair_compressed, pair_probed;
+    // Shared coefficients of the staged sequence: [NT] at z0_base, z0_stride bytes apart -- in the arena where commit leaves
+    // them when it has room for them (z0_in_arena), else in the workspace; z0_loc is where each can be read now.
+    char* z0_base = nullptr;
+    size_t z0_stride = 0;
+    bool z0_in_arena = false;
+    std::vector<char*> z0_loc;
     std::vector<const void*> k_layers, v_layers;
     int64_t stride_t = 0, stride_h = 0;
     bool modes_overridden = false;
@@ -141,6 +147,7 @@ struct CompressArgs {
     int tensors;  // 2: K and V of every head (unit-tensor = head*2 + is_v); 1: K only (unit-tensor = head)
     int ut_base;  // first unit-tensor of the first pair in the stage; pair j adds j*Hkv*tensors
     int64_t unit_stride;  // elements between staged unit-tensors (Tmax*d)
+    int64_t z0_stride;    // elements between the unit-tensors' shared coefficients
     void *z0, *z1;
     uint32_t* hist;
 };
@@ -155,7 +162,8 @@ struct SplitRowsArgs {
     int T, d, Hkv;
     int ut_base;          // first unit-tensor of the first block
     int64_t unit_stride;  // elements between staged tensors (Tmax*d)
-    void* z0;             // [NT][unit_stride]
+    int64_t z0_stride;    // elements between the unit-tensors' shared coefficients
+    void* z0;             // [NT][z0_stride]
     void* hf;             // [NT][1 or 4][unit_stride]: Z1 of a pair, or the layers' deviations of a block of four; K tensors only
 };
 cudaError_t launch_split_rows(const SplitRowsArgs& a, int B, int dtype, cudaStream_t st);
@@ -190,7 +198,8 @@ struct Split4Args {
     int T, d, Hkv;
     int ut_base;          // first unit-tensor of the block (unit-tensor = head*2 + is_v)
     int64_t unit_stride;  // elements between staged tensors (Tmax*d)
-    void* z0;             // [NT][unit_stride]
+    int64_t z0_stride;    // elements between the unit-tensors' shared coefficients
+    void* z0;             // [NT][z0_stride]
     void* dev;            // [NT][4][unit_stride]: deviation of each layer from the block mean
     float* energy;        // [NT][unit_stride]
     void* drop;           // optional [NU][4][unit_stride]: second copy of the K deviations (the gather zeroes its kept positions)
