@@ -138,6 +138,32 @@ size_t row_stream_bytes(const Shape& s, int T) {
     return (size_t)((T + s.max_fold + kRowPad - 1) / kRowPad * kRowPad) * s.d * s.esize;
 }
 
+// Copies of a commit or a fold, collected in classes that are launched one after the other.
+template <int CLASSES>
+struct CopyTable {
+    std::vector<CopyJob> jobs[CLASSES];
+    void rows(int cls, const void* src, void* dst, size_t bytes, int64_t src_pitch, int row_bytes) {
+        jobs[cls].push_back(CopyJob{(const char*)src, (char*)dst, (int64_t)bytes, src_pitch, row_bytes, 0});
+    }
+    void plain(int cls, const void* src, void* dst, size_t bytes, int add = 0) {
+        if (bytes) jobs[cls].push_back(CopyJob{(const char*)src, (char*)dst, (int64_t)bytes, 16, 16, add});
+    }
+    void zero(int cls, void* dst, size_t bytes) { plain(cls, nullptr, dst, bytes); }
+    cudaError_t launch(CopyJob* table_dev, cudaStream_t st) const {
+        std::vector<CopyJob> all;
+        for (const auto& v : jobs) all.insert(all.end(), v.begin(), v.end());
+        if (all.empty()) return cudaSuccess;
+        cudaError_t e = cudaMemcpyAsync(table_dev, all.data(), all.size() * sizeof(CopyJob), cudaMemcpyHostToDevice, st);
+        for (const auto& v : jobs) {
+            int64_t most = 0;
+            for (const CopyJob& jb : v) most = std::max(most, jb.bytes);
+            if (e == cudaSuccess) e = launch_copy_jobs(table_dev, (int)v.size(), most, st);
+            table_dev += v.size();
+        }
+        return e;
+    }
+};
+
 bool seq_ok(fdkv_ctx* c, int seq) { return c && seq >= 0 && seq < c->s.max_batch; }
 
 // Omega(m) of Eq. 2 for one unit (K and V together): bytes of the mode / bytes of the exact mode.  Returns the latter.
@@ -581,11 +607,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
     std::vector<TokenGatherJob> gjobs;  // token rule: the selected rows, formed from the caller's K and V
     // device-to-device copies into the arena and zero fills: one launch per class of size after the loop
     enum { kSaveJobs, kRowJobs, kListJobs, kSmallJobs, kJobClasses };  // (in launch order)
-    std::vector<CopyJob> cjobs[kJobClasses];
-    auto copy_job = [&](int cls, const void* src, void* dst, size_t bytes, int64_t src_pitch, int row_bytes) {
-        cjobs[cls].push_back(CopyJob{(const char*)src, (char*)dst, (int64_t)bytes, src_pitch, row_bytes, 0});
-    };
-    auto zero_job = [&](void* dst, size_t bytes) { if (bytes) copy_job(kSmallJobs, nullptr, dst, bytes, 16, 16); };
+    CopyTable<kJobClasses> copies;
     for (int u = 0; u < s.NU; ++u) {
         const int m = q.modes[u], p = u / s.Hkv, h = u % s.Hkv;
         UnitDesc* dl[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -605,7 +627,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                     if (s.rows_f8) {
                         char* dst = take(rows8_pad);
                         float* sc = reinterpret_cast<float*>(take(scale_slot));
-                        zero_job(dst + rows8, rows8_pad - rows8);
+                        copies.zero(kSmallJobs, dst + rows8, rows8_pad - rows8);
                         qjobs.push_back(QuantJob{sp, c->stride_t, T, 0, reinterpret_cast<uint8_t*>(dst), sc});
                         (is_v ? dl[l]->v_rows : dl[l]->k_rows) = dst;
                         (is_v ? dl[l]->v_scale : dl[l]->k_scale) = sc;
@@ -617,12 +639,12 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                         const size_t ut = (size_t)u * 2 + is_v;
                         dst = c->z0_base + ut * c->z0_stride;
                         c->z0_loc[ut] = c->work + c->ws.z0 + ut * unit_stride_b;
-                        copy_job(kSaveJobs, dst, c->z0_loc[ut], rows, 16, 16);
+                        copies.plain(kSaveJobs, dst, c->z0_loc[ut], rows);
                     } else {
                         dst = take(rows_pad);
                     }
-                    zero_job(dst + rows, rows_pad - rows);
-                    copy_job(kRowJobs, sp, dst, rows, (int64_t)c->stride_t * s.esize, s.d * s.esize);
+                    copies.zero(kSmallJobs, dst + rows, rows_pad - rows);
+                    copies.rows(kRowJobs, sp, dst, rows, (int64_t)c->stride_t * s.esize, s.d * s.esize);
                     (is_v ? dl[l]->v_rows : dl[l]->k_rows) = dst;
                 }
             by_mode[2] += 2 * (size_t)s.B * (s.rows_f8 ? rows8 + 512 : rows);
@@ -631,8 +653,8 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
             if (s.tok_rule && m == FDKV_MODE_RESIDUAL) {  // one token list and one offset table serve K and V
                 tl = take(tlist_b);
                 to = take(off_b);
-                copy_job(kSmallJobs, c->work + c->ws.tok_list + (size_t)u * s.ktok_cap * 4, tl, (size_t)k_tok * 4, 16, 16);
-                copy_job(kSmallJobs, c->work + c->ws.tok_off + (size_t)u * (s.ntiles_max + 1) * 4, to, off_copy, 16, 16);
+                copies.plain(kSmallJobs, c->work + c->ws.tok_list + (size_t)u * s.ktok_cap * 4, tl, (size_t)k_tok * 4);
+                copies.plain(kSmallJobs, c->work + c->ws.tok_off + (size_t)u * (s.ntiles_max + 1) * 4, to, off_copy);
                 by_mode[1] += (size_t)k_tok * 4;
             }
             for (int is_v = 0; is_v < 2; ++is_v) {
@@ -642,13 +664,13 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                 if (s.rows_f8) {
                     z0 = take(rows8_pad);
                     sc8 = reinterpret_cast<float*>(take(scale_slot));
-                    zero_job(z0 + rows8, rows8_pad - rows8);
+                    copies.zero(kSmallJobs, z0 + rows8, rows8_pad - rows8);
                     qjobs.push_back(QuantJob{c->work + c->ws.z0 + ut * unit_stride_b, s.d, T, 0, reinterpret_cast<uint8_t*>(z0), sc8});
                     for (int l = 0; l < s.B; ++l) { (is_v ? dl[l]->v_scale : dl[l]->k_scale) = sc8; dl[l]->rows_f8 = 1; }
                 } else {
                     z0 = in_place ? c->z0_base + ut * c->z0_stride : take(rows_pad);
-                    zero_job(z0 + rows, rows_pad - rows);
-                    if (!in_place) copy_job(kRowJobs, c->z0_loc[ut], z0, rows, 16, 16);
+                    copies.zero(kSmallJobs, z0 + rows, rows_pad - rows);
+                    if (!in_place) copies.plain(kRowJobs, c->z0_loc[ut], z0, rows);
                 }
                 for (int l = 0; l < s.B; ++l) (is_v ? dl[l]->v_rows : dl[l]->k_rows) = z0;
                 by_mode[m] += s.rows_f8 ? rows8 + 512 : rows;
@@ -680,11 +702,11 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                     by_mode[1] += (size_t)s.NB * k_tok * s.d * s.esize;
                 } else if (m == FDKV_MODE_RESIDUAL) {
                     char* po = take(off_b);
-                    copy_job(kSmallJobs, c->work + c->ws.tile_off + ut * (s.ntiles_max + 1) * 4, po, off_copy, 16, 16);
+                    copies.plain(kSmallJobs, c->work + c->ws.tile_off + ut * (s.ntiles_max + 1) * 4, po, off_copy);
                     char* pi_shared = nullptr;
                     if (!c->packed_lists) {
                         pi_shared = take(idx_b);
-                        copy_job(kListJobs, c->work + c->ws.idx + ut * s.kcap * 4, pi_shared, idx_copy, 16, 16);
+                        copies.plain(kListJobs, c->work + c->ws.idx + ut * s.kcap * 4, pi_shared, idx_copy);
                     }
                     char *pi_l[4] = {nullptr, nullptr, nullptr, nullptr}, *pv_l[4] = {nullptr, nullptr, nullptr, nullptr};
                     for (int j = 0; j < s.NB; ++j) {  // one list per stored high-frequency tensor
@@ -694,12 +716,12 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                             if (s.rows_f8)  // values relative to the channel scales, positions in the converted fragments' order
                                 rjobs.push_back(RepackJob{reinterpret_cast<uint32_t*>(pi_l[j]), wsp<uint32_t>(c, c->ws.packed) + lt * s.kcap, k, sc8, is_v, 0});
                             else
-                                copy_job(kListJobs, c->work + c->ws.packed + lt * s.kcap * 4, pi_l[j], idx_copy, 16, 16);
+                                copies.plain(kListJobs, c->work + c->ws.packed + lt * s.kcap * 4, pi_l[j], idx_copy);
                         } else {
                             pi_l[j] = pi_shared;
                             pv_l[j] = take(val_b);
                             // (whole words: an odd count of 2-byte values takes one value of the list's slack along)
-                            copy_job(kListJobs, c->work + c->ws.val + lt * s.kcap * s.esize, pv_l[j], (val_copy + 3) & ~(size_t)3, 16, 16);
+                            copies.plain(kListJobs, c->work + c->ws.val + lt * s.kcap * s.esize, pv_l[j], (val_copy + 3) & ~(size_t)3);
                         }
                     }
                     for (int l = 0; l < s.B; ++l) {
@@ -719,16 +741,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
         CU(cudaMemcpyAsync(table, gjobs.data(), gjobs.size() * sizeof(TokenGatherJob), cudaMemcpyHostToDevice, st));
         CU(launch_token_gather_jobs(reinterpret_cast<TokenGatherJob*>(table), (int)gjobs.size(), k_tok, s.d, s.B, s.dtype, st));
     }
-    CopyJob* cd = reinterpret_cast<CopyJob*>(table + gather_table_bytes(s));
-    std::vector<CopyJob> all;
-    for (const auto& v : cjobs) all.insert(all.end(), v.begin(), v.end());
-    if (!all.empty()) CU(cudaMemcpyAsync(cd, all.data(), all.size() * sizeof(CopyJob), cudaMemcpyHostToDevice, st));
-    for (const auto& v : cjobs) {
-        int64_t most = 0;
-        for (const CopyJob& jb : v) most = std::max(most, jb.bytes);
-        CU(launch_copy_jobs(cd, (int)v.size(), most, st));
-        cd += v.size();
-    }
+    CU(copies.launch(reinterpret_cast<CopyJob*>(table + gather_table_bytes(s)), st));
     if (!qjobs.empty()) {
         QuantJob* qd = reinterpret_cast<QuantJob*>(c->work + c->ws.jobs);
         RepackJob* rd = reinterpret_cast<RepackJob*>(qd + (size_t)s.NU * 2 * s.B);
@@ -956,14 +969,16 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
     const size_t unit_stride_b = (size_t)s.Tmax * s.d * s.esize, chunk_b = (size_t)n * row_b, at = (size_t)T0 * row_b;
     const int64_t k_old = q.k_entries;
     const int nslices = n / kResTile;
+    enum { kRowJobs, kSmallJobs, kJobClasses };
+    CopyTable<kJobClasses> copies;
     for (int u = 0; u < s.NU; ++u) {
         const int m = q.modes[u], p = u / s.Hkv, h = u % s.Hkv;
         UnitDesc* dl[4] = {nullptr, nullptr, nullptr, nullptr};
         for (int l = 0; l < s.B; ++l) dl[l] = &c->desc_host[((size_t)seq * s.L + (size_t)s.B * p + l) * s.Hkv + h];
         if (m == FDKV_MODE_EXACT) {
             for (int l = 0; l < s.B; ++l) {
-                CU(cudaMemcpyAsync((char*)dl[l]->k_rows + at, tail_base(tk, s.B * p + l) + h * tail_head_b, chunk_b, cudaMemcpyDeviceToDevice, st));
-                CU(cudaMemcpyAsync((char*)dl[l]->v_rows + at, tail_base(tv, s.B * p + l) + h * tail_head_b, chunk_b, cudaMemcpyDeviceToDevice, st));
+                copies.plain(kRowJobs, tail_base(tk, s.B * p + l) + h * tail_head_b, (char*)dl[l]->k_rows + at, chunk_b);
+                copies.plain(kRowJobs, tail_base(tv, s.B * p + l) + h * tail_head_b, (char*)dl[l]->v_rows + at, chunk_b);
             }
             q.bytes_by_mode[2] += 2 * (size_t)s.B * chunk_b;
             continue;
@@ -971,7 +986,7 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
         for (int is_v = 0; is_v < 2; ++is_v) {
             const size_t ut = (size_t)u * 2 + is_v;
             char* rows = (char*)(is_v ? dl[0]->v_rows : dl[0]->k_rows);  // every layer of the block shares the coefficient rows
-            CU(cudaMemcpyAsync(rows + at, c->work + c->ws.z0 + ut * unit_stride_b, chunk_b, cudaMemcpyDeviceToDevice, st));
+            copies.plain(kRowJobs, c->work + c->ws.z0 + ut * unit_stride_b, rows + at, chunk_b);
             q.bytes_by_mode[m] += chunk_b;
             if (m != FDKV_MODE_RESIDUAL) continue;
             int32_t* off = const_cast<int32_t*>(is_v ? dl[0]->v_off : dl[0]->k_off);
@@ -980,30 +995,38 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
                 // stored high-frequency tensor (a pair's two layers share theirs)
                 for (int j = 0; j < s.NB; ++j) {
                     int32_t* list = const_cast<int32_t*>(is_v ? dl[j]->v_idx : dl[j]->k_idx);
-                    CU(cudaMemcpyAsync(list + k_old, c->work + c->ws.packed + (ut * s.NB + j) * s.kcap * 4, (size_t)kc * 4, cudaMemcpyDeviceToDevice, st));
+                    copies.plain(kSmallJobs, c->work + c->ws.packed + (ut * s.NB + j) * s.kcap * 4, list + k_old, (size_t)kc * 4);
                 }
             } else {
                 int32_t* list = const_cast<int32_t*>(is_v ? dl[0]->v_idx : dl[0]->k_idx);  // one index list for the unit
-                CU(launch_offset_copy(list + k_old, wsp<int32_t>(c, c->ws.idx) + ut * s.kcap, (int)kc, T0 * s.d, st));
+                copies.plain(kSmallJobs, wsp<int32_t>(c, c->ws.idx) + ut * s.kcap, list + k_old, (size_t)kc * 4, T0 * s.d);
                 for (int j = 0; j < s.NB; ++j) {
                     char* val = (char*)const_cast<void*>(is_v ? dl[j]->v_val : dl[j]->k_val);
-                    CU(cudaMemcpyAsync(val + (size_t)k_old * s.esize, c->work + c->ws.val + (ut * s.NB + j) * s.kcap * s.esize, (size_t)kc * s.esize,
-                                       cudaMemcpyDeviceToDevice, st));
+                    copies.plain(kSmallJobs, c->work + c->ws.val + (ut * s.NB + j) * s.kcap * s.esize, val + (size_t)k_old * s.esize, (size_t)kc * s.esize);
                 }
             }
-            CU(launch_offset_copy(off + T0 / kResTile, wsp<int32_t>(c, c->ws.tile_off) + ut * (s.ntiles_max + 1), nslices + 1, (int)k_old, st));
+            copies.plain(kSmallJobs, wsp<int32_t>(c, c->ws.tile_off) + ut * (s.ntiles_max + 1), off + T0 / kResTile, (size_t)(nslices + 1) * 4, (int)k_old);
             q.bytes_by_mode[1] += (size_t)kc * (c->packed_lists ? (size_t)4 * s.NB : 4 + (size_t)s.NB * s.esize);
         }
     }
-    // ---- the remaining tail rows move down (through the staging area: the ranges may overlap) ----
+    CopyJob* const table = reinterpret_cast<CopyJob*>(c->work + c->ws.jobs + quant_table_bytes(s) + gather_table_bytes(s));
+    CU(copies.launch(table, st));
+    // ---- the remaining tail rows move down: through the staging area, as many layers at a time as it holds, where the ranges
+    // overlap ----
     if (rest > 0) {
-        char* tmp = c->work + c->ws.z1;
-        const size_t w = (size_t)rest * row_b;
-        for (int l = 0; l < s.L; ++l)
-            for (char* base : {tail_base(tk, l), tail_base(tv, l)}) {
-                CU(cudaMemcpy2DAsync(tmp, w, base + (size_t)n * row_b, tail_head_b, w, s.Hkv, cudaMemcpyDeviceToDevice, st));
-                CU(cudaMemcpy2DAsync(base, tail_head_b, tmp, w, w, s.Hkv, cudaMemcpyDeviceToDevice, st));
-            }
+        const size_t w = (size_t)rest * row_b, layer_b = 2 * (size_t)s.Hkv * w, room = (size_t)s.NT * s.NB * unit_stride_b;
+        const int group = rest <= n ? s.L : (int)std::max<size_t>(1, std::min<size_t>(s.L, room / layer_b));
+        for (int l0 = 0; l0 < s.L; l0 += group) {
+            CopyTable<2> moves;
+            char* tmp = c->work + c->ws.z1;
+            for (int l = l0; l < std::min(s.L, l0 + group); ++l)
+                for (char* base : {tail_base(tk, l), tail_base(tv, l)})
+                    for (int h = 0; h < s.Hkv; ++h, base += tail_head_b, tmp += w) {
+                        moves.plain(0, base + (size_t)n * row_b, rest <= n ? base : tmp, w);
+                        if (rest > n) moves.plain(1, tmp, base, w);
+                    }
+            CU(moves.launch(table, st));
+        }
     }
     CU(launch_set_tail_len(arp<int32_t>(c, c->ar.tail_len), s.L, s.max_batch, seq, rest, st));
     q.tail_len.assign(s.L, rest);

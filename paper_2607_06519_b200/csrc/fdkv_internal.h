@@ -295,15 +295,16 @@ struct RepackJob {
     const float* scale;
     int32_t is_v, rows;
 };
-// One copy of the commit step: dst[0, bytes) = consecutive rows of row_bytes taken every src_pitch bytes from src
-// (row_bytes == src_pitch: a plain copy; src null: zeros).  Pointers 16-byte aligned, row_bytes and src_pitch multiples of
-// 16, bytes a multiple of 4.  All copies of a commit run as one launch per size class over a job table.
+// One copy of a commit or a fold: dst[0, bytes) = consecutive rows of row_bytes taken every src_pitch bytes from src
+// (row_bytes == src_pitch: a plain copy; src null: zeros; add != 0: a plain copy of 32-bit words with `add` added).
+// row_bytes and src_pitch multiples of 16, strided sources and destinations 16-byte aligned, bytes a multiple of 4 (of 2
+// for plain copies).  All copies of a step run as one launch per size class over a job table.
 struct CopyJob {
     const char* src;
     char* dst;
     int64_t bytes;
     int64_t src_pitch;
-    int32_t row_bytes, pad_;
+    int32_t row_bytes, add;
 };
 // Token rule: the selected tokens' high-frequency rows of one unit-tensor, formed from the caller's rows of the block's layers.
 struct TokenGatherJob {
@@ -320,8 +321,6 @@ cudaError_t launch_quantise_jobs(const QuantJob* jobs_dev, int njobs, int T_max,
 cudaError_t launch_repack_jobs(const RepackJob* jobs_dev, int njobs, int64_t n_max, cudaStream_t st);
 bool make_rows_tensor_map_u8(void* base, size_t bytes, int box_rows, void* tmap_out);
 
-// dst[i] = src[i] + add, i < n (list offsets and indices of a folded chunk)
-cudaError_t launch_offset_copy(int32_t* dst, const int32_t* src, int n, int add, cudaStream_t st);
 
 // ---- token-granular residual (token_rule.cu) ----
 struct TokenArgs {

@@ -157,3 +157,27 @@ def test_fold_tail_block_of_four():
         step(j, check=True)
     assert pf.ctx.device_status() == 0
     pf.ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d,keep", [("bf16", 64, (1, 7)), ("bf16", 128, (1, 16))])
+def test_fold_of_a_short_chunk_moves_a_long_rest_down(dtype, d, keep):
+    """16 of 150 tokens: the tail rows that stay overlap their new place; bf16 lists with an odd number of entries leave later
+    ones on 2-byte boundaries."""
+    from paper_2607_06519_b200 import runner
+
+    w = synth.Workload(name="fold", n_layers=4, n_q_heads=8, n_kv_heads=2, head_dim=d, batch=1, T=48, dtype=dtype, keep_num=keep[0],
+                       keep_den=keep[1], n_needles=4, W=8, seed=32, n_steps=200)
+    pf = runner.Prefilled(w, max_tail=160, max_fold=32)
+    pf.compress(0)
+    units = {(p, h): oracle_unit(w, 0, p, h) for p in range(2) for h in range(2)}
+    modes = np.array([[0, 1], [2, 1]], dtype=np.int32)
+    pf.ctx.set_modes(0, modes)
+    pf.commit(0)
+    for step in range(150):
+        _check_step(pf, w, modes, units, step, check=False)
+    for step in (150, 151):
+        pf.ctx.fold_tail(0, 16)
+        for u in units.values():
+            u.fold(16, *keep)
+        assert _check_step(pf, w, modes, units, step, check=True) <= TOL[dtype]
+    assert pf.ctx.device_status() == 0
