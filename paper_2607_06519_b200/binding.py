@@ -84,6 +84,7 @@ def _load():
 
 
 _lib = _load()
+_decode_attn = _lib.fdkv_decode_attn
 
 
 def launch_count() -> int:
@@ -137,8 +138,8 @@ def _check(st: int, where: str):
 
 
 def _stream(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    # (the raw handle: building a torch.cuda.Stream object per call costs a microsecond)
+    return stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
@@ -263,12 +264,14 @@ class Context:
 
     def decode_attn(self, layer, q, k_new=None, v_new=None, out=None, out_dtype=None, stream=None):
         """q: [batch, n_q_heads, d]; returns out [batch, n_q_heads, d]."""
-        batch = q.shape[0]
         od = self.cfg.dtype if out_dtype is None else out_dtype
         if out is None:
             out = torch.empty(q.shape, dtype=torch.bfloat16 if od == BF16 else torch.float32, device=self.device)
-        _check(_lib.fdkv_decode_attn(self.h, layer, batch, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out), od,
-                                     _stream(stream)), "fdkv_decode_attn")
+        # one call per layer and token: plain integers, no wrapper objects
+        st = _decode_attn(self.h, layer, len(q), q.data_ptr(), None if k_new is None else k_new.data_ptr(),
+                          None if v_new is None else v_new.data_ptr(), out.data_ptr(), od, _stream(stream))
+        if st:
+            raise FdkvError(st, "fdkv_decode_attn")
         return out
 
     def decode_attn_host(self, layer, q, k_new, v_new, out, out_dtype, stream=None):

@@ -98,7 +98,6 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     w.scores = take((size_t)s.NU * 16);
     w.modes = take((size_t)s.NU * 4);
     w.partials = take((size_t)s.max_batch * s.Hq * kMaxSplits * (s.d + 4) * 4);
-    w.counters = take((size_t)s.max_batch * s.Hkv * 4);
     w.io_q = take((size_t)s.L * s.max_batch * s.Hq * s.d * 4);  // host-I/O staging: room for every layer of a step
     w.io_k = take((size_t)s.L * s.max_batch * s.Hkv * s.d * 4);
     w.io_v = take((size_t)s.L * s.max_batch * s.Hkv * s.d * 4);
@@ -239,9 +238,9 @@ fdkv_status fdkv_create(const fdkv_config* cfg, void* arena, size_t arena_bytes,
     c->seqs.resize(s.max_batch);
     for (auto& q : c->seqs) { q.modes.assign(s.NU, -1); q.tail_len.assign(s.L, 0); }
     c->desc_host.resize((size_t)s.max_batch * s.L * s.Hkv);
+    c->plans.resize(s.L);
     cudaError_t e = cudaMemset(c->arena + c->ar.tail_len, 0, (size_t)s.L * s.max_batch * 4);
     if (e == cudaSuccess) e = cudaMemset(c->work + c->ws.status, 0, 256);
-    if (e == cudaSuccess) e = cudaMemset(c->work + c->ws.counters, 0, (size_t)s.max_batch * s.Hkv * 4);
     if (e == cudaSuccess) e = cudaMemset(c->arena + c->ar.desc, 0, c->desc_host.size() * sizeof(UnitDesc));
     // tails start as zero rows: the fast decode kernel loads whole 64-row boxes and relies on finite padding
     if (e == cudaSuccess) e = cudaMemset(c->arena + c->ar.tail_k, 0, c->ar.bump - c->ar.tail_k);
@@ -270,6 +269,7 @@ fdkv_status fdkv_reset(fdkv_ctx* c) {
     CU(cudaMemset(c->work + c->ws.status, 0, 256));
     CU(cudaMemset(c->arena + c->ar.tail_k, 0, c->ar.bump - c->ar.tail_k));
     c->bump = c->ar.bump;
+    ++c->plan_epoch;
     c->staged_seq = -1;
     for (auto& q : c->seqs) {
         q.committed = false;
@@ -757,6 +757,7 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
                        seq_desc * sizeof(UnitDesc), cudaMemcpyHostToDevice, st));
     CU(cudaStreamSynchronize(st));
     c->bump = o;
+    ++c->plan_epoch;
     q.committed = true;
     q.T = T;
     q.fold_used = 0;
@@ -778,7 +779,8 @@ static fdkv_status decode_impl(fdkv_ctx* c, int32_t layer, int32_t batch, const 
             if (c->seqs[b].tail_len[layer] >= s.max_tail) return FDKV_ERR_STATE;
         for (int b = 0; b < batch; ++b) c->seqs[b].tail_len[layer]++;
     }
-    std::vector<int32_t> host_T(batch), host_modes((size_t)batch * s.Hkv);
+    std::vector<int32_t>&host_T = c->host_T, &host_modes = c->host_modes, &host_tail = c->host_tail;
+    host_T.resize(batch); host_modes.resize((size_t)batch * s.Hkv); host_tail.resize(batch);
     for (int b = 0; b < batch; ++b) {
         host_T[b] = c->seqs[b].T;
         for (int h = 0; h < s.Hkv; ++h) host_modes[(size_t)b * s.Hkv + h] = c->seqs[b].modes[(layer / s.B) * s.Hkv + h];
@@ -786,9 +788,10 @@ static fdkv_status decode_impl(fdkv_ctx* c, int32_t layer, int32_t batch, const 
     DecodeArgs a;
     a.tail_rows = s.tail_rows;
     a.host_T = host_T.data(); a.host_modes = host_modes.data();
-    std::vector<int32_t> host_tail(batch);  // (already counts this call's append)
+    a.plan = &c->plans[layer];
+    a.plan_epoch = c->plan_epoch;
     a.any_tail = 0;
-    for (int b = 0; b < batch; ++b) {
+    for (int b = 0; b < batch; ++b) {  // (already counts this call's append)
         host_tail[b] = c->seqs[b].tail_len[layer];
         a.any_tail |= host_tail[b] > 0;
     }
@@ -807,7 +810,6 @@ static fdkv_status decode_impl(fdkv_ctx* c, int32_t layer, int32_t batch, const 
     a.tail_k = c->arena + c->ar.tail_k; a.tail_v = c->arena + c->ar.tail_v;
     a.tail_len = arp<int32_t>(c, c->ar.tail_len);
     a.partials = wsp<float>(c, c->ws.partials);
-    a.counters = wsp<int32_t>(c, c->ws.counters);
     a.status = wsp<int32_t>(c, c->ws.status);
     CU(launch_decode(a, s.dtype, st));
     return FDKV_OK;
@@ -1036,6 +1038,7 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
     CU(cudaMemcpyAsync(c->arena + c->ar.desc + (size_t)seq * seq_desc * sizeof(UnitDesc), &c->desc_host[(size_t)seq * seq_desc],
                        seq_desc * sizeof(UnitDesc), cudaMemcpyHostToDevice, st));
     CU(cudaStreamSynchronize(st));
+    ++c->plan_epoch;
     q.T = T0 + n;
     q.k_entries = k_old + kc;
     q.fold_used += n;

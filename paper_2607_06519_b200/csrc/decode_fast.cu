@@ -18,8 +18,8 @@
 // The list ranges are loaded one tile per lane 32-64 tiles ahead and handed out by shuffle; the lists themselves
 // are pulled into L2 three tiles ahead and into registers one tile ahead.
 // Work is a flat list of (unit, tile) pairs cut into one contiguous range per CTA (cost-weighted), so a CTA may
-// finish one unit and start the next; each (CTA, unit) segment writes one split-K partial and the CTA that takes
-// the unit's last ticket combines them.
+// finish one unit and start the next; each (CTA, unit) segment writes one split-K partial and a second small kernel
+// (decode_combine_kernel) joins a head's parts.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -42,28 +42,20 @@ constexpr int kScratchBytes = 4096;          // per consumer warp: 16 tokens x 1
 constexpr int kHeaderBytes = 2048;
 constexpr int kMaxSeg = 24;  // (unit, range) segments one CTA can walk: at most units / CTAs + 2
 constexpr int kSmemBytes = kHeaderBytes + kStages * kStageBytes + kCW * kScratchBytes;
-constexpr int kMaxCtas = 296;
+constexpr int kMaxCtas = kMaxSplits;
 constexpr int kMaxUnits = kFastMaxUnits;
 constexpr int kPF = 8;  // residual entries prefetched per lane and list
 constexpr int kPartStride = 128 + 4;  // floats per split-K part: max, sum, 2 pad, 128 accumulators (16-byte aligned)
 static_assert(kTT == kRowPad, "row blocks are padded to whole stages");
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 
-struct FastSched {
-    uint32_t start[kMaxCtas + 1];  // unit << 20 | first 16-token slice of CTA c; start[ncta] = units << 20
-    int ncta, units;
-    int any_tail;  // some sequence of the batch holds generated tokens in this layer's tail (host mirror)
-};
-struct PartCount {
-    uint8_t n[kMaxUnits];  // split-K parts per unit (at most kMaxSplits)
-};
 struct TailLens {
     int32_t n[kMaxUnits];  // generated tokens in this layer's tail per sequence, this call's append included (host mirror)
 };
 static_assert(kMaxSplits < 256 && kMaxSplits % 32 == 0, "part counts are bytes; the combine holds one part per lane and round");
 
 // header offsets
-constexpr int kOffFull = 0, kOffAbort = 128, kOffTicket = 132, kOffM = 256, kOffL = 512, kOffSeg = 1024, kOffSegInfo = 1920,
+constexpr int kOffFull = 0, kOffAbort = 128, kOffM = 256, kOffL = 512, kOffSeg = 1024, kOffSegInfo = 1920,
               kOffCnt = 1936;
 // one (unit, tile range) segment of a CTA: arena rows of its K / V boxes and tail, first tile, prefill tiles, first
 // index in the CTA's tile sequence, and the sequence / head whose tail it also streams (or -1)
@@ -161,8 +153,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // fragments' channel order (the commit step writes the lists that way).  The generated-token tails stay bf16: when a
 // segment reaches them the warp stashes the softmax state of its 8-bit tiles, runs the tails with the plain bf16 code
 // on a fresh state and joins the two at the merge.
+// (at most 232 registers: two warps of this kernel on a quarter of an SM leave 1 536 of its 16 384, one warp of
+// decode_combine_kernel with at most 48)
 template <bool F8>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __maxnreg__(232)
 decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap8, DecodeArgs a, FastSched sch,
                    PartCount pc, TailLens tl) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -232,7 +226,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
     };
     int prologue_issued = 0;
     if (is_producer) {
-        // static part (packed cache, fixed since commit): may run before the dependency wait
+        // static part (packed cache, fixed since commit; tail lengths are the host's): may run before the dependency wait
         int n = 0, it0 = 0;
         for (int u = u_first; u <= u_last && u < sch.units; ++u) {
             const int b = u / a.Hkv, h = u % a.Hkv;
@@ -250,13 +244,20 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             g.rows16 = (min(se, nsl) - sb) * kResTile;
             g.npre = (g.rows16 + kTT - 1) / kTT;
             g.it0 = it0;
-            g.tail_u = se == nsl ? u : -1;  // this CTA also streams the unit's tail (length known after the wait)
-            segs[n++] = g;
+            g.tail_u = se == nsl ? u : -1;  // this CTA also streams the unit's tail
             it0 += g.npre;
+            if (sch.any_tail && g.tail_u >= 0) {
+                const int64_t o = (((int64_t)a.layer * a.max_batch + b) * a.Hkv + h) * a.tail_rows;
+                g.tkrow = (int)(((reinterpret_cast<uint64_t>(a.tail_k) - arena) >> 8) + o);
+                g.tvrow = (int)(((reinterpret_cast<uint64_t>(a.tail_v) - arena) >> 8) + o);
+                it0 += (min(tl.n[b], a.max_tail) + kTT - 1) / kTT;
+            }
+            segs[n++] = g;
         }
         seg_info[0] = n;
         seg_info[1] = it0;
         for (int s = 0; s < kStages; ++s) stage_cnt[s] = 0;
+        // fill the stages up to the first tile of a tail, whose rows may still be written by the kernels ahead
         if (n > 0)
             for (; prologue_issued < kStages && prologue_issued < segs[0].npre; ++prologue_issued)
                 issue_tile(prologue_issued);
@@ -264,55 +265,36 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
     // per-warp scratch starts zeroed
     for (int i = threadIdx.x; i < kCW * kScratchBytes / 16; i += kThreads)
         st_shared_zero16(smem0 + kHeaderBytes + kStages * kStageBytes + i * 16);
-    __syncthreads();  // barriers initialised, static table built (still inside the previous kernel's shadow)
-    // everything below may depend on the kernels launched before this one (q, appended tail rows, partial slots)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (!sch.any_tail) {
-        // no tails anywhere: the static table is final; a short first segment may have left stages to fill
+    __syncthreads();  // barriers initialised, table built (still inside the previous kernel's shadow)
+    // Everything that may depend on the kernels launched before this one (q, appended tail rows, partial slots) comes
+    // behind this: called by every thread of the block in its first segment, after that segment's static reads.
+    bool waited = false;
+    auto dependency_wait = [&]() {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        waited = true;
+        if (sch.any_tail && warp == 0 && a.k_new) {
+            // Generated tokens of this call: the thread block that streams a unit's tail appends the unit's new K and V
+            // rows itself (16 lanes x 16 bytes each) and makes them visible to the tensor copies it issues next; k_new /
+            // v_new are read behind the dependency wait.
+            for (int i = 0; i < seg_info[0]; ++i) {
+                const int tu = segs[i].tail_u;
+                if (tu < 0) continue;
+                const int tb = tu / a.Hkv, th = tu % a.Hkv;
+                const int n = min(tl.n[tb], a.max_tail);
+                if (n <= 0) continue;
+                const int64_t row = (((int64_t)a.layer * a.max_batch + tb) * a.Hkv + th) * a.tail_rows + (n - 1);
+                const uint4* src = reinterpret_cast<const uint4*>(lane < 16 ? a.k_new : a.v_new) + ((int64_t)tb * a.Hkv + th) * 16 + (lane & 15);
+                uint4* dst = reinterpret_cast<uint4*>(lane < 16 ? a.tail_k : a.tail_v) + row * 16 + (lane & 15);
+                *dst = *src;
+                if (lane == 0 && th == 0) a.tail_len[a.layer * a.max_batch + tb] = n;  // the device copy of the length (other kernels read it)
+            }
+            asm volatile("fence.proxy.async;" ::: "memory");
+            __syncwarp();
+        }
         if (is_producer)
             for (int it = prologue_issued; it < kStages && it < seg_info[1]; ++it) issue_tile(it);
-    } else {
-    if (warp == 0 && a.k_new) {
-        // Generated tokens of this call: the thread block that streams a unit's tail appends the unit's new K and V
-        // rows itself (16 lanes x 16 bytes each) and makes them visible to the tensor copies it issues next; a layer
-        // call stays one kernel, and k_new / v_new are read behind the dependency wait.
-        for (int i = 0; i < seg_info[0]; ++i) {
-            const int tu = segs[i].tail_u;
-            if (tu < 0) continue;
-            const int tb = tu / a.Hkv, th = tu % a.Hkv;
-            const int n = min(tl.n[tb], a.max_tail);
-            if (n <= 0) continue;
-            const int64_t row = (((int64_t)a.layer * a.max_batch + tb) * a.Hkv + th) * a.tail_rows + (n - 1);
-            const uint4* src = reinterpret_cast<const uint4*>(lane < 16 ? a.k_new : a.v_new) + ((int64_t)tb * a.Hkv + th) * 16 + (lane & 15);
-            uint4* dst = reinterpret_cast<uint4*>(lane < 16 ? a.tail_k : a.tail_v) + row * 16 + (lane & 15);
-            *dst = *src;
-            if (lane == 0 && th == 0) a.tail_len[a.layer * a.max_batch + tb] = n;  // the device copy of the length (other kernels read it)
-        }
-        asm volatile("fence.proxy.async;" ::: "memory");
-        __syncwarp();
-    }
-    if (is_producer) {
-        // tails: rows may have been written by the kernel right before this one (or just above); lengths are the host's
-        int it0 = 0;
-        for (int i = 0; i < seg_info[0]; ++i) {
-            Seg g = segs[i];
-            g.it0 = it0;
-            if (g.tail_u >= 0) {
-                const int tail_b = g.tail_u / a.Hkv, tail_h = g.tail_u % a.Hkv;
-                const int n = min(tl.n[tail_b], a.max_tail);
-                const int64_t o = (((int64_t)a.layer * a.max_batch + tail_b) * a.Hkv + tail_h) * a.tail_rows;
-                g.tkrow = (int)(((reinterpret_cast<uint64_t>(a.tail_k) - arena) >> 8) + o);
-                g.tvrow = (int)(((reinterpret_cast<uint64_t>(a.tail_v) - arena) >> 8) + o);
-                it0 += (n + kTT - 1) / kTT;
-            }
-            it0 += g.npre;
-            segs[i] = g;
-        }
-        seg_info[1] = it0;
-        for (int it = prologue_issued; it < kStages && it < it0; ++it) issue_tile(it);  // nobody computes yet: fill every stage
-    }
-    __syncthreads();
-    }
+        if (sch.any_tail) __syncthreads();  // (any warp may refill a stage with a tail tile)
+    };
 
     // ================= compute: every warp takes 16 tokens of every stage =================
     {
@@ -346,40 +328,6 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             const bool coef = ud.mode != FDKV_MODE_EXACT, resid = ud.mode == FDKV_MODE_RESIDUAL;
             const uint32_t sgn = ud.sign < 0.f ? 0x80008000u : 0u;
 
-            // q fragments: B operand columns = the G query heads of this KV head.  With G <= 4 columns 4-7 repeat
-            // them: in the second product those columns carry the bf16 rounding remainder of P, so P acts in ~16 bits.
-            const bool split = a.G <= 4;
-            const int qcol = split ? (gid & 3) : gid;
-            uint32_t qb[8][2];
-            auto load_q = [&](bool f8) {
-                const __nv_bfloat16* qh = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((int64_t)b * a.Hq + h * a.G + qcol) * 128;
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                    if (F8 && f8) {
-                        // a converted register holds channels 4 tig .. 4 tig + 3 of the 16-channel step: its low pair is the
-                        // first k-slot pair, its high pair the second; q carries the K scales, as f16
-                        const int c0 = 16 * kk + 4 * tig;
-                        float qv[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) qv[i] = qcol < a.G ? __bfloat162float(qh[c0 + i]) * ud.k_scale[c0 + i] : 0.f;
-                        qb[kk][0] = pack_f16(qv[0], qv[1]);
-                        qb[kk][1] = pack_f16(qv[2], qv[3]);
-                    } else {
-                        qb[kk][0] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 2 * tig) : 0u;
-                        qb[kk][1] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 8 + 2 * tig) : 0u;
-                    }
-                }
-            };
-            if constexpr (F8) {
-                load_q(true);
-            } else {  // (kept inline for the bf16 kernel: routing it through the lambda cost 0.5 %)
-                const __nv_bfloat16* qh = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((int64_t)b * a.Hq + h * a.G + qcol) * 128;
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                    qb[kk][0] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 2 * tig) : 0u;
-                    qb[kk][1] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 8 + 2 * tig) : 0u;
-                }
-            }
             // O^T[channel][column]: eight 16-channel m-tiles; this thread holds columns 2 tig, 2 tig + 1
             float oacc[8][4];
 #pragma unroll
@@ -387,14 +335,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};  // per held column; l is this thread's share
             float m_st[2] = {-INFINITY, -INFINITY}, l_st[2] = {0.f, 0.f};     // 8-bit rows: the state stashed before the bf16 tails
             bool stashed = false;
-            // split-K part slot of this segment = number of CTAs with tiles of this unit before this one
-            int slot = 0;
-            for (int c2 = cta - 1; c2 >= 0; --c2) {
-                const uint32_t ustart = (uint32_t)u << 20, e2 = sch.start[c2 + 1], s2 = sch.start[c2];
-                if (e2 <= ustart) break;                 // ends before this unit's first tile
-                if (max(s2, ustart) < e2) ++slot;        // a non-empty range inside this unit
-                if (s2 <= ustart) break;
-            }
+            const int slot = u == u_first ? sch.slot[cta] : 0;
 
             // ---- residual lists (packed entries): ranges two tiles ahead, entries one tile ahead ----
             const uint32_t* k_ent = reinterpret_cast<const uint32_t*>(ud.k_idx);
@@ -511,6 +452,42 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                 } else {
                     prefetch(k_ent, cr[0], cr[1], pke);
                     prefetch(v_ent, cr[2], cr[3], pve);
+                }
+            }
+
+            if (!waited) dependency_wait();
+            // q fragments: B operand columns = the G query heads of this KV head.  With G <= 4 columns 4-7 repeat
+            // them: in the second product those columns carry the bf16 rounding remainder of P, so P acts in ~16 bits.
+            const bool split = a.G <= 4;
+            const int qcol = split ? (gid & 3) : gid;
+            uint32_t qb[8][2];
+            auto load_q = [&](bool f8) {
+                const __nv_bfloat16* qh = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((int64_t)b * a.Hq + h * a.G + qcol) * 128;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    if (F8 && f8) {
+                        // a converted register holds channels 4 tig .. 4 tig + 3 of the 16-channel step: its low pair is the
+                        // first k-slot pair, its high pair the second; q carries the K scales, as f16
+                        const int c0 = 16 * kk + 4 * tig;
+                        float qv[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) qv[i] = qcol < a.G ? __bfloat162float(qh[c0 + i]) * ud.k_scale[c0 + i] : 0.f;
+                        qb[kk][0] = pack_f16(qv[0], qv[1]);
+                        qb[kk][1] = pack_f16(qv[2], qv[3]);
+                    } else {
+                        qb[kk][0] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 2 * tig) : 0u;
+                        qb[kk][1] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 8 + 2 * tig) : 0u;
+                    }
+                }
+            };
+            if constexpr (F8) {
+                load_q(true);
+            } else {  // (kept inline for the bf16 kernel: routing it through the lambda cost 0.5 %)
+                const __nv_bfloat16* qh = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((int64_t)b * a.Hq + h * a.G + qcol) * 128;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    qb[kk][0] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 2 * tig) : 0u;
+                    qb[kk][1] = qcol < a.G ? *reinterpret_cast<const uint32_t*>(qh + 16 * kk + 8 + 2 * tig) : 0u;
                 }
             }
 
@@ -648,96 +625,89 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                     if (ch == 0) { part[0] = M * 0.6931471805599453f; part[1] = L; }  // the combine step works in natural-log units
                     part[4 + ch] = A;
                 }
-                // ---- split-K combine by whichever CTA finishes this unit last (atomic ticket, nobody waits) ----
-                // The block barrier orders every thread's part stores before thread 0's fence, which is cumulative: the
-                // ticket increment publishes the whole part at device scope; the last CTA's reads go to L2 (ld.cg).
-                __syncthreads();
-                int* const s_ticket = reinterpret_cast<int*>(smem_raw + kOffTicket);
-                if (threadIdx.x == 0) {
-                    int t;  // one release+acquire read-modify-write instead of fence, atomic, fence
-                    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(t) : "l"(a.counters + u) : "memory");
-                    *s_ticket = t;
-                }
-                __syncthreads();
-                const int nparts = pc.n[u];
-                if (*s_ticket == nparts - 1) {
-                    // Warp w takes head w % G and every (8/G)-th part of it, 4 channels per lane; the scratch area
-                    // holds the per-warp sums, the header the per-warp denominators.
-                    float* const red = reinterpret_cast<float*>(smem_raw + kHeaderBytes + kStages * kStageBytes);  // [8][128]
-                    {
-                        const int g = warp % a.G, pgi = warp / a.G, npg = kCW / a.G;
-                        const float* pp = a.partials + ((int64_t)b * a.Hq + h * a.G + g) * kMaxSplits * kPartStride;
-                        float mreg[kMaxSplits / 32], lreg[kMaxSplits / 32];
-                        float mx = -INFINITY;
-#pragma unroll
-                        for (int i = 0; i < kMaxSplits / 32; ++i) {
-                            const int sp = lane + 32 * i;
-                            mreg[i] = sp < nparts ? __ldcg(pp + sp * kPartStride) : -INFINITY;
-                            lreg[i] = sp < nparts ? __ldcg(pp + sp * kPartStride + 1) : 0.f;
-                        }
-#pragma unroll
-                        for (int i = 0; i < kMaxSplits / 32; ++i) mx = fmaxf(mx, mreg[i]);
-#pragma unroll
-                        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-                        float ls = 0.f;
-#pragma unroll
-                        for (int i = 0; i < kMaxSplits / 32; ++i) {
-                            mreg[i] = mreg[i] == -INFINITY ? 0.f : __expf(mreg[i] - mx);  // now the part's weight
-                            ls = fmaf(lreg[i], mreg[i], ls);
-                        }
-#pragma unroll
-                        for (int o = 16; o; o >>= 1) ls += __shfl_xor_sync(0xFFFFFFFFu, ls, o);
-                        // part weights to shared memory (one row per warp, after the eight 128-float sums), then the
-                        // accumulator rows in batches of eight independent loads
-                        float* const wts = red + kCW * 128 + warp * kMaxSplits;
-#pragma unroll
-                        for (int i = 0; i < kMaxSplits / 32; ++i) wts[lane + 32 * i] = mreg[i];
-                        __syncwarp();
-                        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-                        for (int base = pgi; base < nparts; base += 8 * npg) {
-                            float4 v[8];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const int sp = base + j * npg;
-                                if (sp < nparts) v[j] = __ldcg(reinterpret_cast<const float4*>(pp + sp * kPartStride + 4) + lane);
-                            }
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const int sp = base + j * npg;
-                                if (sp < nparts) {
-                                    const float f = wts[sp];
-                                    acc.x = fmaf(v[j].x, f, acc.x); acc.y = fmaf(v[j].y, f, acc.y);
-                                    acc.z = fmaf(v[j].z, f, acc.z); acc.w = fmaf(v[j].w, f, acc.w);
-                                }
-                            }
-                        }
-                        reinterpret_cast<float4*>(red + warp * 128)[lane] = acc;
-                        if (lane == 0) sm_l[warp] = ls;
-                    }
+                if (u < u_last && u + 1 < sch.units) {  // (another segment may follow: the scratch tiles and sums are read by now)
                     __syncthreads();
-                    for (int i = threadIdx.x; i < a.G * 128; i += kThreads) {
-                        const int g = i >> 7, ch = i & 127;
-                        float A = 0.f;
-                        for (int w = g; w < kCW; w += a.G) A += red[w * 128 + ch];
-                        const float L = sm_l[g];
-                        const float r = L > 0.f ? A / L : 0.f;
-                        const int64_t o = ((int64_t)b * a.Hq + h * a.G + g) * 128 + ch;
-                        if (a.out_dtype == FDKV_BF16)
-                            reinterpret_cast<__nv_bfloat16*>(a.out)[o] = __float2bfloat16_rn(r);
-                        else
-                            reinterpret_cast<float*>(a.out)[o] = r;
-                    }
-                    if (threadIdx.x == 0) a.counters[u] = 0;  // ready for the next launch
+                    zero_scratch();
                     __syncthreads();
                 }
-                zero_scratch();
-                __syncthreads();
             }
         }
     }
     // after a timed-out wait: give copies that may still be in flight time to land before the CTA retires
     if (*abort_flag)
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
+}
+
+// out = sum_s e^{m_s - M} acc_s / sum_s e^{m_s - M} l_s over a query head's split-K parts.  One warp per 32 VEC channels of a
+// head; it rides on programmatic dependent launch between two decode launches.  A block has 32 threads and few registers
+// so that it becomes resident beside a decode block (which leaves 2 048 registers and 1 KiB of shared memory of an SM) and
+// its start costs nothing.  Latency-bound: the maxima, sums and accumulators of 32 parts are requested in one round.
+// (Before, the last block of a unit combined behind an atomic ticket: a release, an atomic round trip and two rounds of
+// loads on the critical path of every layer call, and the SM it ran on started the next call late.)
+template <int VEC>
+__global__ void __maxnreg__(48) decode_combine_kernel(const float* partials, int Hq, int Hkv, int G, PartCount pc, void* out, int out_dtype) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int lane = threadIdx.x, i = blockIdx.y, b = blockIdx.z, ch = (blockIdx.x * 32 + lane) * VEC;
+    const int n = pc.n[b * Hkv + i / G];
+    const float* const pp = partials + ((int64_t)b * Hq + i) * kMaxSplits * kPartStride;
+    constexpr int BATCH = VEC == 1 ? 16 : 4;  // accumulator loads in flight
+    float M = -INFINITY, L = 0.f, A[VEC];
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) A[k] = 0.f;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int base = 0; base < n; base += 32) {
+        float m = -INFINITY, l = 0.f;
+        if (base + lane < n) {
+            m = __ldcg(pp + (base + lane) * kPartStride);
+            l = __ldcg(pp + (base + lane) * kPartStride + 1);
+        }
+        float w = 0.f;
+        for (int j0 = 0; j0 < 32 && base + j0 < n; j0 += BATCH) {
+            float v[BATCH][VEC];
+#pragma unroll
+            for (int j = 0; j < BATCH; ++j) {
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) v[j][k] = 0.f;
+                if (base + j0 + j < n) {
+                    const float* p = pp + (base + j0 + j) * kPartStride + 4 + ch;
+                    if constexpr (VEC == 4) {
+                        const float4 x = __ldcg(reinterpret_cast<const float4*>(p));
+                        v[j][0] = x.x; v[j][1] = x.y; v[j][2] = x.z; v[j][3] = x.w;
+                    } else {
+                        v[j][0] = __ldcg(p);
+                    }
+                }
+            }
+            if (j0 == 0) {
+                float mx = m;
+#pragma unroll
+                for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+                mx = fmaxf(mx, M);
+                w = m == -INFINITY ? 0.f : __expf(m - mx);
+                const float f = M == -INFINITY ? 0.f : __expf(M - mx);
+                float ls = l * w;
+#pragma unroll
+                for (int o = 16; o; o >>= 1) ls += __shfl_xor_sync(0xFFFFFFFFu, ls, o);
+                L = fmaf(L, f, ls);
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) A[k] *= f;
+                M = mx;
+            }
+#pragma unroll
+            for (int j = 0; j < BATCH; ++j) {
+                const float wj = __shfl_sync(0xFFFFFFFFu, w, (j0 + j) & 31);  // (zero beyond the last part)
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) A[k] = fmaf(v[j][k], wj, A[k]);
+            }
+        }
+    }
+    const int64_t o = ((int64_t)b * Hq + i) * 128 + ch;
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) {
+        const float r = L > 0.f ? A[k] / L : 0.f;
+        if (out_dtype == FDKV_BF16) reinterpret_cast<__nv_bfloat16*>(out)[o + k] = __float2bfloat16_rn(r);
+        else reinterpret_cast<float*>(out)[o + k] = r;
+    }
 }
 
 }  // namespace
@@ -816,6 +786,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     // tensor (keep 1/16), 1.65 at 512 (keep 1/32); with 8-bit rows (a dearer plain tile) about 1.7 at either density.
     const double res_a = a.rows_f8 ? 1.55 : 1.25;
     const double res_b = a.rows_f8 ? 0.15 : 0.87;
+    const int ctas = (int)std::min<int64_t>(std::min(std::min(sm_count, kMaxCtas), kMaxSplits), total_tiles);
     auto weigh = [&](double rc) {
         for (int u = 0; u < units; ++u) {
             const int T = a.host_T[u / a.Hkv];
@@ -830,17 +801,17 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
             // the CTA that ends a unit also streams its tail of generated tokens (whole plain tiles): counted as slices
             // of the unit's kind behind the unit's own, so that this CTA gets correspondingly fewer of those
             const int tail = a.host_tail ? std::min(a.host_tail[u / a.Hkv], a.max_tail) : 0;
-            // Measured: the CTA that ends a unit runs behind its siblings at equal shares (with tails it also reads their
-            // lengths behind the dependency wait); charging it eight plain tiles' worth of slices (in eighths of a tile
-            // below) is the optimum of a sweep at 32k, with and without tails (+1.6 % / +6 %), and neutral at 128k.
-            constexpr int kEndExtra = 64;  // (eighths of a plain tile)
-            es[u] = ns[u] + ((tail + kTT - 1) / kTT * (kTT / kResTile) + kEndExtra) * (2 * kTT * 256 / 512) / std::max(1, wt[u]);
+            // Measured: it runs behind its siblings at equal shares (cause not found); charging it five eighths of a block's share, at
+            // most eight plain tiles, on top is within 0.3 % of the best of a sweep at 2k to 128k and on a batch (against no
+            // charge: 32k 26.5 -> 26.2 us a layer, 128k 84.7 -> 83.1, batch of eight 132.8 -> 130.7).
+            const int64_t end_extra = std::min<int64_t>(64, 5 * total_tiles / std::max(1, ctas));  // (eighths of a plain tile)
+            es[u] = ns[u] + ((tail + kTT - 1) / kTT * (kTT / kResTile) + (int)end_extra) * (2 * kTT * 256 / 512) / std::max(1, wt[u]);
             wp[u + 1] = wp[u] + (int64_t)es[u] * wt[u];  // (in eighths of the tile cost)
         }
     };
     // (measured best: 1.7 when every unit gets whole CTAs, 1.5 in the flat cut of a batch)
     weigh(a.tok_rule ? 1.7 : 0.0);
-    const int ncta = (int)std::min<int64_t>(std::min(std::min(sm_count, kMaxCtas), kMaxSplits), total_tiles);
+    const int ncta = ctas;
     sch.ncta = ncta;
     sch.any_tail = a.any_tail;
     sch.units = units;
@@ -867,10 +838,13 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
             ++given;
         }
         if (given != ncta) whole = false;
-        // with few CTAs per unit the integer shares are too uneven (2 vs 3 CTAs is +50 %): cut the flat list instead
+        // with few CTAs per unit the integer shares are too uneven (2 vs 3 CTAs is +50 %): cut the flat list instead, unless
+        // the unevenness is less than what a CTA that straddles two units pays for its second merge
+        // (short contexts: a layer call of 2k tokens 9.7 us with the flat cut, 7.0 us without)
+        constexpr double kFlatExtra = 4.0;  // (plain tiles)
         double worst = 0.0;
         for (int u = 0; u < units; ++u) worst = std::max(worst, (double)(wp[u + 1] - wp[u]) / nc[u]);
-        if (worst > 1.06 * (double)wp[units] / ncta) whole = false;
+        if (worst > (double)wp[units] / ncta + kFlatExtra * (kTT / kResTile) * (2 * kTT * 256 / 512)) whole = false;
     }
     if (whole) {
         int c = 0;
@@ -906,6 +880,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     // parts per unit = CTAs whose range contains at least one of its tiles
     for (int u = 0; u < kMaxUnits; ++u) cs.n[u] = 0;
     for (int c = 0; c < ncta; ++c) {
+        sch.slot[c] = (sch.start[c] >> 20) < (uint32_t)units ? cs.n[sch.start[c] >> 20] : 0;
         const int ua = (int)(sch.start[c] >> 20), ta = (int)(sch.start[c] & 0xFFFFFu);
         const int ub = (int)(sch.start[c + 1] >> 20), tb = (int)(sch.start[c + 1] & 0xFFFFFu);
         int nseg_cta = 0;
@@ -944,16 +919,26 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     int sm_count = 0;
     cudaError_t e0 = once.ensure([&]() {
         cudaError_t e = cudaFuncSetAttribute(decode_fast_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(decode_fast_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_fast_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        // the same division of the SM's memory as the decode kernel's, or the two could not share an SM
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        return e;
     }, &sm_count);
     if (e0 != cudaSuccess) return e0;
-    FastSched sch;
-    PartCount cs;
-    {
-        const cudaError_t pe = plan_decode_schedule(a, units, sm_count, sch, cs);
+    FastPlan& plan = *a.plan;
+    bool current = plan.epoch == a.plan_epoch && plan.batch == a.batch && plan.sm_count == sm_count;
+    for (int b = 0; current && b < a.batch; ++b) current = plan.tail_tiles[b] == (a.host_tail[b] + kTT - 1) / kTT;
+    if (!current) {
+        plan.epoch = 0;
+        const cudaError_t pe = plan_decode_schedule(a, units, sm_count, plan.sch, plan.pc);
         if (pe != cudaSuccess) return pe;
+        plan.epoch = a.plan_epoch; plan.batch = a.batch; plan.sm_count = sm_count;
+        plan.tail_tiles.resize(a.batch);
+        for (int b = 0; b < a.batch; ++b) plan.tail_tiles[b] = (a.host_tail[b] + kTT - 1) / kTT;
     }
+    const FastSched& sch = plan.sch;
+    const PartCount& cs = plan.pc;
     const int ncta = sch.ncta;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ncta);
@@ -968,11 +953,20 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     const CUtensorMap& m16 = *reinterpret_cast<const CUtensorMap*>(a.tmap);
     const CUtensorMap& m8 = *reinterpret_cast<const CUtensorMap*>(a.rows_f8 ? a.tmap_u8 : a.tmap);
     TailLens tl;
-    for (int b = 0; b < a.batch; ++b) tl.n[b] = a.host_tail ? a.host_tail[b] : 0;
+    for (int b = 0; b < a.batch; ++b) tl.n[b] = a.host_tail[b];
     cudaError_t e = a.rows_f8 ? cudaLaunchKernelEx(&cfg, decode_fast_kernel<true>, m16, m8, a, sch, cs, tl)
                               : cudaLaunchKernelEx(&cfg, decode_fast_kernel<false>, m16, m8, a, sch, cs, tl);
     if (e != cudaSuccess) return e;
-    count_launch(1);
+    // one channel per lane where a head has many parts (few heads: latency), four where the heads fill the machine
+    const bool wide = units * a.G > sm_count;
+    cfg.gridDim = dim3(wide ? 1 : 4, a.Hq, a.batch);
+    cfg.blockDim = dim3(32);
+    cfg.dynamicSmemBytes = 0;
+    const float* parts = a.partials;
+    e = wide ? cudaLaunchKernelEx(&cfg, decode_combine_kernel<4>, parts, a.Hq, a.Hkv, a.G, cs, a.out, a.out_dtype)
+             : cudaLaunchKernelEx(&cfg, decode_combine_kernel<1>, parts, a.Hq, a.Hkv, a.G, cs, a.out, a.out_dtype);
+    if (e != cudaSuccess) return e;
+    count_launch(2);
     count_kernel(FDKV_KERNEL_DECODE_FAST);
     *handled = true;
     return cudaGetLastError();

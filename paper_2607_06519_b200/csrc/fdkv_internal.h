@@ -50,6 +50,27 @@ struct UnitDesc {
     const float* v_scale;
 };
 
+// Schedule of one launch of the bf16 / head_dim 128 decode kernel (decode_fast.cu): travels in the launch parameters.
+struct FastSched {
+    uint32_t start[kMaxSplits + 1];  // unit << 20 | first 16-token slice of CTA c; start[ncta] = units << 20
+    uint8_t slot[kMaxSplits];        // split-K part of CTA c's first unit that CTA c writes (its later units start with it: part 0)
+    int ncta, units;
+    int any_tail;  // some sequence of the batch holds generated tokens in this layer's tail (host mirror)
+};
+struct PartCount {
+    uint8_t n[kFastMaxUnits];  // split-K parts per unit (at most kMaxSplits)
+};
+// The schedule depends on the committed lengths and modes, the batch and the tails in whole tiles, and costs more host time
+// than the rest of a call: every layer keeps its last one (in the context) until one of these changes.
+struct FastPlan {
+    uint64_t epoch = 0;             // fdkv_ctx::plan_epoch it was made in (0: none yet)
+    int batch = 0;
+    int sm_count = 0;
+    std::vector<int32_t> tail_tiles;  // [batch]
+    FastSched sch;
+    PartCount pc;
+};
+
 struct SelState {
     uint32_t prefix;  // magnitude-key prefix fixed so far (left-aligned in 31 bits once complete)
     uint32_t k_rem;   // entries still to take at or below the prefix
@@ -81,7 +102,7 @@ struct WsLayout {
     size_t tok_score, tok_err, tok_list, tok_off;
     size_t energy, eval;  // four-layer blocks: per-position high-frequency energy (float32) and the kept energies
     size_t status, z0, z1, z1drop, hist, sel, lb_records, lb_ticket, tile_off, idx, val, packed, probe_part, probe_pos, scores, modes,
-        partials, counters, io_q, io_k, io_v, io_out, jobs, total;  // io_*: host-I/O staging, [L] layers each
+        partials, io_q, io_k, io_v, io_out, jobs, total;  // io_*: host-I/O staging, [L] layers each
 };
 struct ArenaLayout {
     size_t tail_len, desc, tail_k, tail_v, bump, worst_total;
@@ -123,6 +144,9 @@ struct fdkv_ctx {
     bool modes_overridden = false;
     std::vector<fdkv::SeqState> seqs;
     std::vector<fdkv::UnitDesc> desc_host;  // [max_batch][L][Hkv]
+    uint64_t plan_epoch = 1;                // advanced whenever a committed length or mode changes
+    std::vector<fdkv::FastPlan> plans;      // [L]
+    std::vector<int32_t> host_T, host_modes, host_tail;  // what a decode call's launch is planned from (kept: no allocation per call)
     alignas(64) unsigned char tmap[128];    // CUtensorMap of the arena (bf16, head_dim 128 only)
     bool has_tmap = false;
     alignas(64) unsigned char tmap_z1[128], tmap_drop[128];  // probe operands (bf16, head_dim 128 only)
@@ -257,6 +281,8 @@ struct DecodeArgs {
     const int32_t* host_T;      // [batch]
     const int32_t* host_modes;  // [batch][Hkv] modes of this layer's pair
     const int32_t* host_tail;   // [batch] generated tokens in this layer's tail per sequence (after this call's append), or null
+    FastPlan* plan;             // the layer's kept schedule, or null (planning without a context)
+    uint64_t plan_epoch;
     int any_tail;               // some sequence of the batch has generated tokens in this layer's tail (after this call's append)
     const void* tmap;           // CUtensorMap over the arena as rows of 256 bytes, or null
     const void* tmap_u8;        // the same arena as rows of 128 bytes (8-bit row streams), or null
@@ -267,7 +293,6 @@ struct DecodeArgs {
     int tok_rule;
     int32_t* tail_len;      // [L][max_batch]
     float* partials;        // [batch][Hq][kMaxSplits][d+4]: max, sum, 2 pad, d accumulators
-    int32_t* counters;      // [max_batch][Hkv] split-K arrival tickets, zero between launches
     int32_t* status;
 };
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, cudaStream_t st);
