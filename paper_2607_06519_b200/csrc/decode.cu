@@ -1,36 +1,16 @@
 // Decode attention over the compressed cache (the fused reconstruct-and-attend step after Eq. 3):
-// tail append, split-K partial attention with per-mode reconstruction, split-K combine.
+// split-K partial attention with per-mode reconstruction (which also appends the generated token), split-K combine.
 // This file holds the portable kernel (float32 or bf16 storage, head_dim 64/128, any group size up to 8);
 // the bulk-copy / tensor-core kernel for bf16, head_dim 128 lives in decode_fast.cu.
+#include <algorithm>
+#include <type_traits>
+
 #include "fdkv_internal.h"
 
 namespace fdkv {
 
 namespace {
 
-template <typename T, int EPL>
-__device__ __forceinline__ void load_row(const T* row, int lane, float* f);
-template <>
-__device__ __forceinline__ void load_row<float, 4>(const float* row, int lane, float* f) {
-    const float4 v = *reinterpret_cast<const float4*>(row + lane * 4);
-    f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
-}
-template <>
-__device__ __forceinline__ void load_row<float, 2>(const float* row, int lane, float* f) {
-    const float2 v = *reinterpret_cast<const float2*>(row + lane * 2);
-    f[0] = v.x; f[1] = v.y;
-}
-template <>
-__device__ __forceinline__ void load_row<__nv_bfloat16, 4>(const __nv_bfloat16* row, int lane, float* f) {
-    const uint2 v = *reinterpret_cast<const uint2*>(row + lane * 4);
-    f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xFFFF0000u);
-    f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xFFFF0000u);
-}
-template <>
-__device__ __forceinline__ void load_row<__nv_bfloat16, 2>(const __nv_bfloat16* row, int lane, float* f) {
-    const uint32_t v = *reinterpret_cast<const uint32_t*>(row + lane * 2);
-    f[0] = __uint_as_float(v << 16); f[1] = __uint_as_float(v & 0xFFFF0000u);
-}
 template <typename T>
 __device__ __forceinline__ float ldf(const T* p);
 template <>
@@ -38,287 +18,344 @@ __device__ __forceinline__ float ldf<float>(const float* p) { return *p; }
 template <>
 __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
-// Appends k_new / v_new rows of every sequence to the layer's tail and bumps the tail length.
-template <typename T>
-__global__ void append_tail_kernel(DecodeArgs a) {
-    // Programmatic dependent launch: the kernel may become resident, and let the decode kernel behind it start its
-    // own prologue, while the kernel ahead of it in the stream still runs.  Everything it reads was possibly written by
-    // that kernel -- k_new / v_new come from the caller's projection, the tail length from the previous step's append,
-    // and the previous step's decode kernel of this layer may still be reading the length -- so the dependency wait
-    // comes before the first read.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int b = blockIdx.x;
-    int32_t* len = a.tail_len + a.layer * a.max_batch + b;
-    const int n = *len;
-    if (n >= a.max_tail) {
-        if (threadIdx.x == 0) atomicMax(a.status, (int32_t)kFlagTailFull);
-        return;
+// eight consecutive channels of a row
+__device__ __forceinline__ void load8(const float* p, float (&f)[8]) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+}
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&f)[8]) {
+    const uint4 v = *reinterpret_cast<const uint4*>(p);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        f[2 * i] = __uint_as_float(w[i] << 16);
+        f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
-    const int row = a.Hkv * a.d;
-    const T* kn = reinterpret_cast<const T*>(a.k_new) + (int64_t)b * row;
-    const T* vn = reinterpret_cast<const T*>(a.v_new) + (int64_t)b * row;
-    T* tk = reinterpret_cast<T*>(a.tail_k);
-    T* tv = reinterpret_cast<T*>(a.tail_v);
-    for (int i = threadIdx.x; i < row; i += blockDim.x) {
-        const int h = i / a.d, c = i % a.d;
-        const int64_t o = ((((int64_t)a.layer * a.max_batch + b) * a.Hkv + h) * a.tail_rows + n) * a.d + c;
-        tk[o] = kn[i];
-        tv[o] = vn[i];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) *len = n + 1;
 }
 
-constexpr int kWarps = 4;
-constexpr int kGTile = 32;                  // tokens per warp tile of the portable kernel
-constexpr int kSub = kGTile / kResTile;     // residual-offset tiles per warp tile
+template <typename ACC>
+__device__ __forceinline__ ACC dot8(const float (&x)[8], const float (&y)[8]) {
+    ACC a = (ACC)x[0] * (ACC)y[0], b = (ACC)x[4] * (ACC)y[4];
+#pragma unroll
+    for (int i = 1; i < 4; ++i) {
+        a = fma((ACC)x[i], (ACC)y[i], a);
+        b = fma((ACC)x[i + 4], (ACC)y[i + 4], b);
+    }
+    return a + b;
+}
 
-// grid (splits, Hkv, batch); 4 warps; each warp owns whole 32-token tiles and a private online-softmax state.
+constexpr int kWarps = 8;
+constexpr int kParts = 4;  // floats before a part's accumulators: max, sum, 2 pad
+
+// grid (splits, Hkv, batch); eight warps, each on whole 16-token tiles (the granularity of the residual lists).  D / 8 lanes
+// share a token, eight channels each, so a warp works on 256 / D tokens at a time; every such lane group keeps a softmax
+// state of its own (maximum, sum, D accumulators) over the tokens it meets, and the groups are joined once at the end:
+// a score costs log2(D / 8) shuffles per head and the weighted sum of V none.  A residual tile is scattered into a zeroed
+// float32 tile in shared memory and read beside the rows.  Bound by latency at the sizes this path serves:
+// a tile's K and V rows are requested together, and the split gives every warp few tiles.
+// A layer of 4 099 tokens, two KV heads of two query heads, float32 / 64 channels: 36.9 -> 9.5 us against one lane group per
+// warp with a five-step reduction per token and head, 32-token tiles and shared-memory atomics for the residual, in a few
+// blocks, and an append kernel of its own; bf16 with 8 query heads per KV head at 6 000 tokens 70.7 -> 11.1.
 template <typename T, int D, int G>
-__global__ void __launch_bounds__(kWarps * 32) decode_generic_kernel(DecodeArgs a, int splits) {
-    constexpr int EPL = D / 32;
-    __shared__ float qs[G][D];
-    __shared__ float s_corr[kWarps][G][32];
-    __shared__ float s_p[kWarps][G][32];
-    __shared__ float s_vacc[kWarps][G][D];
+__global__ void __launch_bounds__(kWarps * 32, G <= 2 && sizeof(T) == 2 ? 2 : 1) decode_generic_kernel(DecodeArgs a, int splits) {
+    // float32 storage: logits of a few tens, whose rounding the exponential magnifies to more than the outputs' own; float64
+    // products cost nothing here (less than 1 % of the time)
+    using ACC = typename std::conditional<sizeof(T) == 4, double, float>::type;
+    constexpr int LPT = D / 8;         // lanes per token
+    constexpr int TPI = 32 / LPT;      // tokens per step
+    constexpr int STEPS = kResTile / TPI;
+    constexpr int PF = D == 128 ? (G == 8 ? 2 : 4) : STEPS;  // steps whose rows are requested together
+    extern __shared__ __align__(16) float smem[];  // [kWarps][16][D] residual tiles; at the end the warps' accumulators [kWarps][G][D]
     __shared__ float s_m[kWarps][G], s_l[kWarps][G];
-
     const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const UnitDesc u = a.desc[((int64_t)b * a.L + a.layer) * a.Hkv + h];
-    const T* qg = reinterpret_cast<const T*>(a.q) + ((int64_t)b * a.Hq + h * G) * D;
-    for (int i = threadIdx.x; i < G * D; i += blockDim.x) qs[i / D][i % D] = ldf<T>(qg + i);
-    for (int i = threadIdx.x; i < kWarps * G * D; i += blockDim.x) (&s_vacc[0][0][0])[i] = 0.f;
-    __syncthreads();
-
-    float q[G][EPL], acc[G][EPL], m[G], l[G];
+    const int grp = lane / LPT, c0 = (lane % LPT) * 8;
+    float* const tilez = smem + warp * (kResTile * D);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const UnitDesc u = a.desc[((int64_t)b * a.L + a.layer) * a.Hkv + h];  // (static since commit)
+    const bool coef = u.mode != FDKV_MODE_EXACT;
+    const bool resid = u.mode == FDKV_MODE_RESIDUAL;
+    const int ntiles = (u.T + kResTile - 1) / kResTile;
+    const int per = (ntiles + splits - 1) / splits;
+    const int j0 = min(ntiles, split * per), j1 = min(ntiles, j0 + per);
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // q, the tails and the parts belong to the kernels ahead
+    const T* const qg = reinterpret_cast<const T*>(a.q) + ((int64_t)b * a.Hq + h * G) * D + c0;
+    float q[G][8], acc[G][8], m[G], l[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
+        load8(qg + g * D, q[g]);
         m[g] = -INFINITY;
         l[g] = 0.f;
 #pragma unroll
-        for (int i = 0; i < EPL; ++i) { q[g][i] = qs[g][lane * EPL + i]; acc[g][i] = 0.f; }
+        for (int i = 0; i < 8; ++i) acc[g][i] = 0.f;
     }
-
     const float inv_sqrt_d = rsqrtf((float)D);
-    const float c = u.scale;  // what the stored rows are multiplied by (1/sqrt 2 for a pair, 1/2 for a block of four)
-    const bool coef = u.mode != FDKV_MODE_EXACT;
-    const bool resid = u.mode == FDKV_MODE_RESIDUAL;
 
-    const int nres = (u.T + kResTile - 1) / kResTile;
-    // ---- one 32-token tile: rows [row0, row0 + nrows) of kbase / vbase ----
-    auto tile = [&](const T* kbase, const T* vbase, int nrows, float kscale, float vscale, bool with_res, int jt) {
-        float s[G];
+    // adds the residual of this tile (K or V side) to the zeroed shared-memory tile
+    auto scatter = [&](int jt, const int32_t* idx, const void* vals, const int32_t* off) {
+        const int e0 = off[jt], e1 = off[jt + 1];
 #pragma unroll
-        for (int g = 0; g < G; ++g) s[g] = 0.f;
-        for (int tt = 0; tt < nrows; ++tt) {
-            float kf[EPL];
-            load_row<T, EPL>(kbase + (int64_t)tt * D, lane, kf);
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                float p = 0.f;
-#pragma unroll
-                for (int i = 0; i < EPL; ++i) p = fmaf(q[g][i], kf[i], p);
-#pragma unroll
-                for (int o = 16; o; o >>= 1) p += __shfl_xor_sync(0xFFFFFFFFu, p, o);
-                if (lane == tt) s[g] = p;
+        for (int i = 0; i < kResTile * D / 4; i += 32) *reinterpret_cast<float4*>(tilez + (i + lane) * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncwarp();
+        const T* const val = reinterpret_cast<const T*>(vals);
+        if (u.res_kind == 1) {  // whole rows of selected tokens
+            for (int e = e0; e < e1; ++e) {
+                const int tt = idx[e] - jt * kResTile;
+                for (int c = lane; c < D; c += 32) tilez[tt * D + c] = ldf<T>(val + (int64_t)e * D + c);
             }
+        } else {
+            const int base = jt * kResTile * D;
+            for (int e = e0 + lane; e < e1; e += 32) tilez[idx[e] - base] = ldf<T>(val + e);
         }
-        if (with_res && u.res_kind == 1) {
-            // token rule: the tile's selected tokens carry whole high-frequency rows (k_idx = ascending token list, k_off =
-            // tokens kept before every 16-token slice, k_val / v_val = their rows, densely packed)
-            const T* rows = reinterpret_cast<const T*>(u.k_val);
-            const int j1 = u.k_off[min(nres, (jt + 1) * kSub)];
-            for (int j = u.k_off[jt * kSub]; j < j1; ++j) {
-                const int tt = u.k_idx[j] - jt * kGTile;
-                float kf[EPL];
-                load_row<T, EPL>(rows + (int64_t)j * D, lane, kf);
+        __syncwarp();
+    };
+    // one tile: rows [0, nrows) of kb / vb (rows behind the last are read as the last and masked)
+    auto tile = [&](const T* kb, const T* vb, int nrows, float kscale, float vscale, bool with_res, int jt) {
+        float p[G][STEPS], kf[PF][8], vf[PF][8];
+#pragma unroll
+        for (int s0 = 0; s0 < STEPS; s0 += PF) {
+#pragma unroll
+            for (int s = 0; s < PF; ++s) {
+                const int t = min((s0 + s) * TPI + grp, nrows - 1);
+                load8(kb + (int64_t)t * D + c0, kf[s]);
+                if (s0 == 0) load8(vb + (int64_t)t * D + c0, vf[s]);
+            }
+            if (with_res && s0 == 0) scatter(jt, u.k_idx, u.k_val, u.k_off);
+#pragma unroll
+            for (int s = 0; s < PF; ++s) {
+                const int t = (s0 + s) * TPI + grp;
+                // the residual's product is its own sum: adding it to the row first would round every coefficient once more
+                float z[8];
+                if (with_res) load8(tilez + t * D + c0, z);
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    float p = 0.f;
+                    ACC d = dot8<ACC>(q[g], kf[s]);
+                    if (with_res) d = fma((ACC)u.sign, dot8<ACC>(q[g], z), d);
 #pragma unroll
-                    for (int i = 0; i < EPL; ++i) p = fmaf(q[g][i], kf[i], p);
-#pragma unroll
-                    for (int o = 16; o; o >>= 1) p += __shfl_xor_sync(0xFFFFFFFFu, p, o);
-                    if (lane == tt) s[g] = fmaf(u.sign, p, s[g]);
+                    for (int o = LPT / 2; o; o >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, o);
+                    p[g][s0 + s] = t < nrows ? (float)d * kscale : -INFINITY;
                 }
             }
-        } else if (with_res) {
-            // sparse correction in the logit domain: q . z1 over this tile's kept K entries
-#pragma unroll
-            for (int g = 0; g < G; ++g) s_corr[warp][g][lane] = 0.f;
-            __syncwarp();
-            const int64_t base = (int64_t)jt * kGTile * D;
-            const T* val = reinterpret_cast<const T*>(u.k_val);
-            const int ke1 = u.k_off[min(nres, (jt + 1) * kSub)];
-            for (int e = u.k_off[jt * kSub] + lane; e < ke1; e += 32) {
-                const int f = (int)(u.k_idx[e] - base);
-                const float v = ldf<T>(val + e);
-#pragma unroll
-                for (int g = 0; g < G; ++g) atomicAdd(&s_corr[warp][g][f / D], qs[g][f % D] * v);
-            }
-            __syncwarp();
-#pragma unroll
-            for (int g = 0; g < G; ++g) s[g] = fmaf(u.sign, s_corr[warp][g][lane], s[g]);
         }
-        float p[G];
+        if (with_res) {
+            __syncwarp();
+            scatter(jt, u.v_idx ? u.v_idx : u.k_idx, u.v_val, u.v_off ? u.v_off : u.k_off);
+        }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const float sg = lane < nrows ? s[g] * kscale : -INFINITY;
-            float mx = sg;
+            float mx = m[g];
 #pragma unroll
-            for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-            const float m_new = fmaxf(m[g], mx);
-            const float alpha = __expf(m[g] - m_new);  // m_new is finite here (nrows >= 1)
-            p[g] = lane < nrows ? __expf(sg - m_new) : 0.f;
-            float ps = p[g];
+            for (int s = 0; s < STEPS; ++s) mx = fmaxf(mx, p[g][s]);
+            if (mx > m[g]) {
+                const float alpha = __expf(m[g] - mx);
+                l[g] *= alpha;
 #pragma unroll
-            for (int o = 16; o; o >>= 1) ps += __shfl_xor_sync(0xFFFFFFFFu, ps, o);
-            l[g] = l[g] * alpha + ps;
-            m[g] = m_new;
+                for (int i = 0; i < 8; ++i) acc[g][i] *= alpha;
+                m[g] = mx;
+            }
 #pragma unroll
-            for (int i = 0; i < EPL; ++i) acc[g][i] *= alpha;
-            p[g] *= vscale;
-        }
-        for (int tt = 0; tt < nrows; ++tt) {
-            float vf[EPL];
-            load_row<T, EPL>(vbase + (int64_t)tt * D, lane, vf);
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                const float pg = __shfl_sync(0xFFFFFFFFu, p[g], tt);
-#pragma unroll
-                for (int i = 0; i < EPL; ++i) acc[g][i] = fmaf(pg, vf[i], acc[g][i]);
+            for (int s = 0; s < STEPS; ++s) {
+                p[g][s] = p[g][s] == -INFINITY ? 0.f : __expf(p[g][s] - mx);
+                l[g] += p[g][s];
+                p[g][s] *= vscale;
             }
         }
-        if (with_res && u.res_kind == 1) {
-            const T* rows = reinterpret_cast<const T*>(u.v_val);
-            const int j1 = u.k_off[min(nres, (jt + 1) * kSub)];
-            for (int j = u.k_off[jt * kSub]; j < j1; ++j) {
-                const int tt = u.k_idx[j] - jt * kGTile;
-                float vf[EPL];
-                load_row<T, EPL>(rows + (int64_t)j * D, lane, vf);
 #pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    const float pg = u.sign * __shfl_sync(0xFFFFFFFFu, p[g], tt);
+        for (int s0 = 0; s0 < STEPS; s0 += PF) {
+            if (s0 > 0)
 #pragma unroll
-                    for (int i = 0; i < EPL; ++i) acc[g][i] = fmaf(pg, vf[i], acc[g][i]);
+                for (int s = 0; s < PF; ++s) load8(vb + (int64_t)min((s0 + s) * TPI + grp, nrows - 1) * D + c0, vf[s]);
+#pragma unroll
+            for (int s = 0; s < PF; ++s) {
+                if (with_res) {
+                    float z[8];
+                    load8(tilez + ((s0 + s) * TPI + grp) * D + c0, z);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) vf[s][i] = fmaf(u.sign, z[i], vf[s][i]);
                 }
-            }
-        } else if (with_res) {
-#pragma unroll
-            for (int g = 0; g < G; ++g) s_p[warp][g][lane] = p[g];
-            __syncwarp();
-            const int64_t base = (int64_t)jt * kGTile * D;
-            const T* val = reinterpret_cast<const T*>(u.v_val);
-            const int e0 = u.v_off[jt * kSub], e1 = u.v_off[min(nres, (jt + 1) * kSub)];
-            for (int e = e0 + lane; e < e1; e += 32) {
-                const int f = (int)(u.v_idx[e] - base);
-                const float v = ldf<T>(val + e);
-#pragma unroll
-                for (int g = 0; g < G; ++g) atomicAdd(&s_vacc[warp][g][f % D], s_p[warp][g][f / D] * v);
-            }
-            __syncwarp();
-            if (e1 > e0) {
 #pragma unroll
                 for (int g = 0; g < G; ++g)
 #pragma unroll
-                    for (int i = 0; i < EPL; ++i) {
-                        acc[g][i] = fmaf(u.sign, s_vacc[warp][g][lane * EPL + i], acc[g][i]);
-                        s_vacc[warp][g][lane * EPL + i] = 0.f;
-                    }
+                    for (int i = 0; i < 8; ++i) acc[g][i] = fmaf(p[g][s0 + s], vf[s][i], acc[g][i]);
             }
-            __syncwarp();
         }
+        if (with_res) __syncwarp();
     };
 
     // ---- prefill rows of this split ----
     {
-        const int ntiles = (u.T + kGTile - 1) / kGTile;
-        const int tiles_per_split = (ntiles + splits - 1) / splits;
-        const int j0 = split * tiles_per_split, j1 = min(ntiles, j0 + tiles_per_split);
         const T* kr = reinterpret_cast<const T*>(u.k_rows);
         const T* vr = reinterpret_cast<const T*>(u.v_rows);
-        const float kscale = coef ? c * inv_sqrt_d : inv_sqrt_d;
-        const float vscale = coef ? c : 1.f;
+        const float kscale = coef ? u.scale * inv_sqrt_d : inv_sqrt_d, vscale = coef ? u.scale : 1.f;
         for (int jt = j0 + warp; jt < j1; jt += kWarps) {
-            const int t0 = jt * kGTile;
-            tile(kr + (int64_t)t0 * D, vr + (int64_t)t0 * D, min(kGTile, u.T - t0), kscale, vscale, resid, jt);
+            const int t0 = jt * kResTile;
+            tile(kr + (int64_t)t0 * D, vr + (int64_t)t0 * D, min(kResTile, u.T - t0), kscale, vscale, resid, jt);
         }
     }
     // ---- uncompressed tail rows (last split only) ----
     if (split == splits - 1) {
-        const int n = min(a.tail_len[a.layer * a.max_batch + b], a.max_tail);
+        int n = min(a.tail_len[a.layer * a.max_batch + b], a.max_tail);
         const int64_t o = (((int64_t)a.layer * a.max_batch + b) * a.Hkv + h) * a.tail_rows * D;
-        const T* tk = reinterpret_cast<const T*>(a.tail_k) + o;
-        const T* tv = reinterpret_cast<const T*>(a.tail_v) + o;
-        for (int t0 = warp * 32; t0 < n; t0 += kWarps * 32)
-            tile(tk + (int64_t)t0 * D, tv + (int64_t)t0 * D, min(32, n - t0), inv_sqrt_d, 1.f, false, 0);
+        T* tk = reinterpret_cast<T*>(a.tail_k) + o;
+        T* tv = reinterpret_cast<T*>(a.tail_v) + o;
+        if (a.k_new) {  // this call's row joins the tail here (the length is advanced by the combine kernel)
+            if (n < a.max_tail) {
+                for (int c = threadIdx.x; c < D; c += kWarps * 32) {
+                    const int64_t src = ((int64_t)b * a.Hkv + h) * D + c;
+                    tk[(int64_t)n * D + c] = reinterpret_cast<const T*>(a.k_new)[src];
+                    tv[(int64_t)n * D + c] = reinterpret_cast<const T*>(a.v_new)[src];
+                }
+                ++n;
+            } else if (threadIdx.x == 0) {
+                atomicMax(a.status, (int32_t)kFlagTailFull);
+            }
+            __syncthreads();
+        }
+        for (int t0 = warp * kResTile; t0 < n; t0 += kWarps * kResTile)
+            tile(tk + (int64_t)t0 * D, tv + (int64_t)t0 * D, min(kResTile, n - t0), inv_sqrt_d, 1.f, false, 0);
     }
 
-    // ---- merge the warps' states and write the split's partial ----
-    if (lane == 0)
-#pragma unroll
-        for (int g = 0; g < G; ++g) { s_m[warp][g] = m[g]; s_l[warp][g] = l[g]; }
-    __syncthreads();
+    // ---- join the lane groups, then the warps, and write the split's part ----
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-        float M = -INFINITY;
-        for (int w = 0; w < kWarps; ++w) M = fmaxf(M, s_m[w][g]);
-        const float f = M == -INFINITY ? 0.f : __expf(m[g] - M);
+        float M = m[g];
 #pragma unroll
-        for (int i = 0; i < EPL; ++i) s_vacc[warp][g][lane * EPL + i] = acc[g][i] * f;
+        for (int o = LPT; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+        const float f = m[g] == -INFINITY ? 0.f : __expf(m[g] - M);
+        l[g] *= f;
+#pragma unroll
+        for (int o = LPT; o < 32; o <<= 1) l[g] += __shfl_xor_sync(0xFFFFFFFFu, l[g], o);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            acc[g][i] *= f;
+#pragma unroll
+            for (int o = LPT; o < 32; o <<= 1) acc[g][i] += __shfl_xor_sync(0xFFFFFFFFu, acc[g][i], o);
+        }
+        m[g] = M;
     }
+    __syncthreads();  // (the residual tiles are read)
+    float* const s_acc = smem + warp * G * D;
+    if (grp == 0)
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            *reinterpret_cast<float4*>(s_acc + g * D + c0) = make_float4(acc[g][0], acc[g][1], acc[g][2], acc[g][3]);
+            *reinterpret_cast<float4*>(s_acc + g * D + c0 + 4) = make_float4(acc[g][4], acc[g][5], acc[g][6], acc[g][7]);
+            if (lane == 0) { s_m[warp][g] = m[g]; s_l[warp][g] = l[g]; }
+        }
     __syncthreads();
-    for (int i = threadIdx.x; i < G * D; i += blockDim.x) {
+    for (int i = threadIdx.x; i < G * D; i += kWarps * 32) {
         const int g = i / D, ch = i % D;
         float M = -INFINITY;
+#pragma unroll
         for (int w = 0; w < kWarps; ++w) M = fmaxf(M, s_m[w][g]);
         float L = 0.f, A = 0.f;
-        for (int w = 0; w < kWarps; ++w) {
-            L += M == -INFINITY ? 0.f : s_l[w][g] * __expf(s_m[w][g] - M);
-            A += s_vacc[w][g][ch];
-        }
-        float* part = a.partials + (((int64_t)b * a.Hq + h * G + g) * kMaxSplits + split) * (D + 4);
+        if (M != -INFINITY)
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const float f = s_m[w][g] == -INFINITY ? 0.f : __expf(s_m[w][g] - M);
+                L = fmaf(s_l[w][g], f, L);
+                A = fmaf(smem[(w * G + g) * D + ch], f, A);
+            }
+        float* part = a.partials + (((int64_t)b * a.Hq + h * G + g) * kMaxSplits + split) * (D + kParts);
         if (ch == 0) { part[0] = M; part[1] = L; }
-        part[4 + ch] = A;
+        part[kParts + ch] = A;
     }
 }
 
-// out = sum_s e^{m_s - M} acc_s / sum_s e^{m_s - M} l_s.  grid (Hq, batch), D threads.
+// out = sum_s e^{m_s - M} acc_s / sum_s e^{m_s - M} l_s.  grid (D / 32, Hq, batch), eight warps: lane = channel, the warps take
+// every eighth part, so that a head's parts are read in a few rounds of loads.  Also advances the tail lengths of a call
+// that appended.
 template <int D>
-__global__ void combine_kernel(const float* partials, int Hq, int splits, void* out, int out_dtype) {
-    const int i = blockIdx.x, b = blockIdx.y, ch = threadIdx.x;
-    const float* p = partials + ((int64_t)b * Hq + i) * kMaxSplits * (D + 4);
-    float M = -INFINITY;
-    for (int s = 0; s < splits; ++s) M = fmaxf(M, p[s * (D + 4)]);
-    float L = 0.f, A = 0.f;
-    for (int s = 0; s < splits; ++s) {
-        const float ms = p[s * (D + 4)];
-        if (ms == -INFINITY) continue;
-        const float f = __expf(ms - M);
-        L = fmaf(p[s * (D + 4) + 1], f, L);
-        A = fmaf(p[s * (D + 4) + 4 + ch], f, A);
+__global__ void __launch_bounds__(256) combine_kernel(DecodeArgs a, int splits) {
+    __shared__ float s_m[8], s_l[8], s_a[8][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.y, b = blockIdx.z, ch = blockIdx.x * 32 + lane;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const float* p = a.partials + ((int64_t)b * a.Hq + i) * kMaxSplits * (D + kParts);
+    float M = -INFINITY, L = 0.f, A = 0.f;
+    for (int s0 = warp; s0 < splits; s0 += 32) {
+        float ms[4], ls[4], as[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool on = s0 + 8 * k < splits;
+            const float* ps = p + (int64_t)(on ? s0 + 8 * k : s0) * (D + kParts);
+            ms[k] = on ? __ldcg(ps) : -INFINITY;
+            ls[k] = on ? __ldcg(ps + 1) : 0.f;
+            as[k] = on ? __ldcg(ps + kParts + ch) : 0.f;
+        }
+        const float Mn = fmaxf(fmaxf(M, fmaxf(ms[0], ms[1])), fmaxf(ms[2], ms[3]));
+        if (Mn == -INFINITY) continue;
+        const float f = M == -INFINITY ? 0.f : __expf(M - Mn);
+        L *= f;
+        A *= f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float w = ms[k] == -INFINITY ? 0.f : __expf(ms[k] - Mn);
+            L = fmaf(ls[k], w, L);
+            A = fmaf(as[k], w, A);
+        }
+        M = Mn;
     }
-    const float r = L > 0.f ? A / L : 0.f;
-    const int64_t o = ((int64_t)b * Hq + i) * D + ch;
-    if (out_dtype == FDKV_BF16)
-        reinterpret_cast<__nv_bfloat16*>(out)[o] = __float2bfloat16_rn(r);
-    else
-        reinterpret_cast<float*>(out)[o] = r;
+    if (lane == 0) { s_m[warp] = M; s_l[warp] = L; }
+    s_a[warp][lane] = A;
+    __syncthreads();
+    if (warp == 0) {
+        M = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) M = fmaxf(M, s_m[w]);
+        L = A = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const float f = s_m[w] == -INFINITY ? 0.f : __expf(s_m[w] - M);
+            L = fmaf(s_l[w], f, L);
+            A = fmaf(s_a[w][lane], f, A);
+        }
+        const float r = L > 0.f ? A / L : 0.f;
+        const int64_t o = ((int64_t)b * a.Hq + i) * D + ch;
+        if (a.out_dtype == FDKV_BF16)
+            reinterpret_cast<__nv_bfloat16*>(a.out)[o] = __float2bfloat16_rn(r);
+        else
+            reinterpret_cast<float*>(a.out)[o] = r;
+        if (a.k_new && i == 0 && blockIdx.x == 0 && lane == 0) {
+            int32_t* len = a.tail_len + a.layer * a.max_batch + b;
+            if (*len < a.max_tail) ++*len;
+        }
+    }
+}
+
+template <typename T, int D, int G>
+cudaError_t launch_generic_g(const DecodeArgs& a, int splits, cudaLaunchConfig_t& cfg) {
+    static PerDevice once;
+    cfg.dynamicSmemBytes = (size_t)kWarps * std::max(kResTile, G) * D * sizeof(float);
+    cudaError_t e = once.ensure([&]() { return cudaFuncSetAttribute(decode_generic_kernel<T, D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes); });
+    return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, decode_generic_kernel<T, D, G>, a, splits);
 }
 
 template <typename T, int D>
 cudaError_t launch_generic(const DecodeArgs& a, int splits, cudaStream_t st) {
-    dim3 grid(splits, a.Hkv, a.batch);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(splits, a.Hkv, a.batch);
+    cfg.blockDim = dim3(kWarps * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e;
     switch (a.G) {
-        case 1: decode_generic_kernel<T, D, 1><<<grid, kWarps * 32, 0, st>>>(a, splits); break;
-        case 2: decode_generic_kernel<T, D, 2><<<grid, kWarps * 32, 0, st>>>(a, splits); break;
-        case 4: decode_generic_kernel<T, D, 4><<<grid, kWarps * 32, 0, st>>>(a, splits); break;
-        case 8: decode_generic_kernel<T, D, 8><<<grid, kWarps * 32, 0, st>>>(a, splits); break;
+        case 1: e = launch_generic_g<T, D, 1>(a, splits, cfg); break;
+        case 2: e = launch_generic_g<T, D, 2>(a, splits, cfg); break;
+        case 4: e = launch_generic_g<T, D, 4>(a, splits, cfg); break;
+        case 8: e = launch_generic_g<T, D, 8>(a, splits, cfg); break;
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3(D / 32, a.Hq, a.batch);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = 0;
+    return cudaLaunchKernelEx(&cfg, combine_kernel<D>, a, splits);
 }
 
 }  // namespace
@@ -339,38 +376,16 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, cudaStream_t st) {
     bool handled = false;
     if ((e = launch_decode_fast(a, st, &handled)) != cudaSuccess) return e;  // (appends k_new / v_new itself)
     if (handled) return cudaSuccess;
-    if (a.k_new) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(a.batch);
-        cfg.blockDim = dim3(128);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (dtype == FDKV_BF16)
-            e = cudaLaunchKernelEx(&cfg, append_tail_kernel<__nv_bfloat16>, a);
-        else
-            e = cudaLaunchKernelEx(&cfg, append_tail_kernel<float>, a);
-        if (e != cudaSuccess) return e;
-        count_launch(1);
-    }
     if (a.packed_lists) return cudaErrorNotSupported;  // packed residual lists are only read by the kernel above
 
-    const int ntiles = (a.Tmax_batch + kGTile - 1) / kGTile;
-    int splits = (2 * 148 + a.Hkv * a.batch - 1) / (a.Hkv * a.batch);
-    splits = max(1, min(min(splits, kMaxSplits), (ntiles + 7) / 8));
+    // one tile per warp while the blocks are resident at one time (two on an SM for bf16 up to two heads per group), then longer ranges
+    const int ntiles = (a.Tmax_batch + kResTile - 1) / kResTile, units = a.Hkv * a.batch;
+    const int splits = std::max(1, std::min(std::min(((a.G <= 2 && dtype == FDKV_BF16 ? 2 : 1) * 148 + units - 1) / units, kMaxSplits), (ntiles + kWarps - 1) / kWarps));
     if (dtype == FDKV_BF16)
         e = a.d == 128 ? launch_generic<__nv_bfloat16, 128>(a, splits, st) : launch_generic<__nv_bfloat16, 64>(a, splits, st);
     else
         e = a.d == 128 ? launch_generic<float, 128>(a, splits, st) : launch_generic<float, 64>(a, splits, st);
     if (e != cudaSuccess) return e;
-    dim3 cgrid(a.Hq, a.batch);
-    if (a.d == 128)
-        combine_kernel<128><<<cgrid, 128, 0, st>>>(a.partials, a.Hq, splits, a.out, a.out_dtype);
-    else
-        combine_kernel<64><<<cgrid, 64, 0, st>>>(a.partials, a.Hq, splits, a.out, a.out_dtype);
     count_launch(2);
     count_kernel(FDKV_KERNEL_DECODE_PORTABLE);
     return cudaGetLastError();
