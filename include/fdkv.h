@@ -287,8 +287,8 @@ fdkv_status fdkv_decode_bytes(fdkv_ctx* ctx, int32_t layer, int32_t batch, size_
  * Who needs it: code that runs where cudaMalloc is off limits -- inside a serving engine whose memory pool owns
  * every byte of the device, in a plugin that is only handed tensors, or in a latency-critical path where an
  * allocation (an implicit device synchronisation) is not acceptable -- and that has no fdkv context, whose
- * workspace would otherwise provide the scratch.  The scratch this needs (the Z1 temporary, the magnitude
- * histogram, per-tile counts and offsets; about 4.3 MB) is a static array inside the library's device image:
+ * workspace would otherwise provide the scratch.  The scratch this needs (candidate lists, per-chunk counts and tile
+ * offsets; about 6.3 MB) is a static array inside the library's device image:
  * every GPU that loads libfdkv holds it until the process exits, whether or not this function is ever called.
  *
  * Computes exactly what fdkv_compress_prefill computes for one unit-tensor: z0_out[T][head_dim] (storage
@@ -298,11 +298,11 @@ fdkv_status fdkv_decode_bytes(fdkv_ctx* ctx, int32_t layer, int32_t batch, size_
  *
  * Limits and rules
  *  - T * head_dim <= FDKV_NOALLOC_MAX_ELEMS, else FDKV_ERR_TOO_LARGE and nothing is enqueued.
- *  - Calls cudaMalloc / cudaFree or any allocating routine never; it enqueues a memset and kernels on `stream`.
+ *  - Calls cudaMalloc / cudaFree or any allocating routine never; it enqueues kernels on `stream`.
  *  - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with that device
  *    current).  Make that first call outside any stream capture.
- *  - Every call on a device uses the same array, which still holds the previous call's data; the function
- *    clears what has to start at zero itself.  Two calls whose work overlaps on the GPU (different streams
+ *  - Every call on a device uses the same array, which still holds the previous call's data (nothing has to
+ *    start at zero).  Two calls whose work overlaps on the GPU (different streams
  *    without an ordering between them) race on it: serialise them.
  *  - A device-side count mismatch is not reported here (there is no context to hold a status word the caller
  *    could read); compare *count_host with what you expect to find in idx_out if in doubt.

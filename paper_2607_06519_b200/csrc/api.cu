@@ -62,6 +62,8 @@ bool make_shape(const fdkv_config& c, Shape& s) {
     s.tok_rule = c.residual_rule == FDKV_RESIDUAL_TOKENS;
     s.ktok_max = (int64_t)s.Tmax * s.keep_num / s.keep_den;
     s.ktok_cap = (int64_t)align_up((size_t)(s.ktok_max + 32), 64);
+    s.cand_stride = ((int64_t)s.Tmax * s.d + kMaxCompressChunk - 1) / kMaxCompressChunk * kMaxCompressChunk;
+    s.chunks_max = (int)(s.cand_stride / compress_chunk(B, s.esize));
     s.NU = s.P * s.Hkv;
     s.NT = 2 * s.NU;
     return true;
@@ -77,14 +79,15 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     const size_t unit_elems = (size_t)s.Tmax * s.d;
     w.status = take(256);
     w.z0 = take((size_t)s.NT * unit_elems * s.esize);
-    w.z1 = take((size_t)s.NT * s.NB * unit_elems * s.esize);  // Z1 of a pair, or the four layers' deviations of a block
+    w.z1 = take((size_t)s.NU * s.NB * unit_elems * s.esize);  // high-frequency rows of K: Z1 of a pair, or the four layers' deviations
     w.z1drop = take(s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule ? (size_t)s.NU * s.NB * unit_elems * s.esize : 0);
-    w.energy = take(s.B == 4 && !s.tok_rule ? (size_t)s.NT * unit_elems * 4 : 0);
-    w.eval = take(s.B == 4 && !s.tok_rule ? (size_t)s.NT * s.kcap * 4 : 0);
-    w.hist = take((size_t)s.NT * kHistBins * 4);
+    const size_t entry_rule = s.tok_rule ? 0 : 1;
+    w.cand_pos = take(entry_rule * s.NT * s.cand_stride * 2);
+    w.cand_val = take(entry_rule * s.NT * s.NB * s.cand_stride * s.esize);
+    w.cand_n = take(entry_rule * s.NT * s.chunks_max * 4);
+    w.chunk_base = take(entry_rule * s.NT * s.chunks_max * 8);
+    w.keep = take(entry_rule * s.NU * (s.cand_stride / 8));
     w.sel = take((size_t)s.NT * sizeof(SelState));
-    w.lb_records = take((size_t)s.NT * s.ntiles_max * 8);
-    w.lb_ticket = take(256);
     w.tile_off = take((size_t)s.NT * (s.ntiles_max + 1) * 4);
     w.idx = take((size_t)s.NT * s.kcap * 4);
     w.val = take((size_t)s.NT * s.NB * s.kcap * s.esize);
@@ -180,6 +183,30 @@ double omega_of(const Shape& s, int T, double (&om)[3]) {
     return b_ex;
 }
 
+// What a prompt of T tokens and a folded chunk of T tokens have in common.
+CompressArgs entry_args(fdkv_ctx* c, int T) {
+    const Shape& s = c->s;
+    CompressArgs a;
+    a.T = T; a.d = s.d; a.Hkv = s.Hkv; a.tensors = 2;
+    a.unit_stride = (int64_t)s.Tmax * s.d;
+    a.z1 = nullptr;
+    a.sel = wsp<SelState>(c, c->ws.sel);
+    a.cand_pos = wsp<uint16_t>(c, c->ws.cand_pos);
+    a.cand_val = c->work + c->ws.cand_val;
+    a.cand_n = wsp<int32_t>(c, c->ws.cand_n);
+    a.chunk_base = wsp<int2>(c, c->ws.chunk_base);
+    a.cand_stride = s.cand_stride; a.chunks_max = s.chunks_max;
+    a.n_keep = (int64_t)T * s.d * s.keep_num / s.keep_den; a.kcap = s.kcap;
+    a.ntiles_max = s.ntiles_max;
+    a.tile_off = wsp<int32_t>(c, c->ws.tile_off);
+    a.idx = wsp<int32_t>(c, c->ws.idx);
+    a.val = c->work + c->ws.val;
+    a.packed = c->packed_lists ? wsp<uint32_t>(c, c->ws.packed) : nullptr;
+    a.keep = nullptr; a.keep_stride = s.cand_stride / 32;
+    a.status = wsp<int32_t>(c, c->ws.status);
+    return a;
+}
+
 }  // namespace
 
 namespace fdkv {
@@ -251,10 +278,10 @@ fdkv_status fdkv_create(const fdkv_config* cfg, void* arena, size_t arena_bytes,
     // token rule: the tensor-core score kernel and the packed decode kernel serve bf16 / head_dim 128; everything else
     // takes the float32 score kernel and the portable decode kernel
     if (s.tok_rule && c->packed_lists)
-        c->tok_tc = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NT * s.NB * s.Tmax * s.d * s.esize, 128, c->tmap_z1_128);
+        c->tok_tc = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, 128, c->tmap_z1_128);
     if (s.tok_rule && s.dtype == FDKV_BF16 && s.d == 128 && !c->tok_tc) { delete c; return FDKV_ERR_UNSUPPORTED; }
     if (s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule)
-        c->has_probe_tmaps = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NT * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_z1) &&
+        c->has_probe_tmaps = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_z1) &&
                              make_rows_tensor_map(c->work + c->ws.z1drop, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_drop);
     *out = c;
     return FDKV_OK;
@@ -318,7 +345,7 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
         return FDKV_ERR_INVALID_ARG;
     }
     cudaStream_t st = S(stream);
-    const int ut_begin = pb * s.Hkv * 2, ut_count = (pe - pb) * s.Hkv * 2;
+    for (int l = s.B * pb; l < s.B * pe; ++l) { c->k_layers[l] = k_layers[l]; c->v_layers[l] = v_layers[l]; }
     if (s.tok_rule) {
         // the token rule selects inside fdkv_probe: only the split here
         constexpr int kMost = kSplitLayers;
@@ -326,8 +353,8 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
             SplitRowsArgs a;
             a.n_blocks = std::min(pe - p0, kMost / s.B);
             for (int l = 0; l < a.n_blocks * s.B; ++l) {
-                a.k[l] = c->k_layers[s.B * p0 + l] = k_layers[s.B * p0 + l];
-                a.v[l] = c->v_layers[s.B * p0 + l] = v_layers[s.B * p0 + l];
+                a.k[l] = k_layers[s.B * p0 + l];
+                a.v[l] = v_layers[s.B * p0 + l];
             }
             a.stride_t = stride_t; a.stride_h = stride_h;
             a.T = T; a.d = s.d; a.Hkv = s.Hkv;
@@ -339,92 +366,12 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t 
         for (int p = pb; p < pe; ++p) { c->pair_compressed[p] = 1; c->pair_probed[p] = 0; c->pair_scored[p] = 0; }
         return FDKV_OK;
     }
-    CU(cudaMemsetAsync(wsp<uint32_t>(c, c->ws.hist) + (size_t)ut_begin * kHistBins, 0, (size_t)ut_count * kHistBins * 4, st));
-    if (s.B == 4) {
-        // blocks of four layers: Z0, the layers' deviations and the positions' energies; one kept set per tensor from
-        // the float32 radix select on the energies; then the four layers' values at the kept positions
-        for (int p = pb; p < pe; ++p) {
-            Split4Args a4;
-            for (int l = 0; l < 4; ++l) {
-                a4.k[l] = k_layers[4 * p + l];
-                a4.v[l] = v_layers[4 * p + l];
-                c->k_layers[4 * p + l] = a4.k[l];
-                c->v_layers[4 * p + l] = a4.v[l];
-            }
-            a4.stride_t = stride_t; a4.stride_h = stride_h;
-            a4.T = T; a4.d = s.d; a4.Hkv = s.Hkv;
-            a4.ut_base = p * s.Hkv * 2;
-            a4.unit_stride = (int64_t)s.Tmax * s.d; a4.z0_stride = (int64_t)(c->z0_stride / s.esize);
-            a4.z0 = c->z0_base; a4.dev = c->work + c->ws.z1;
-            a4.energy = wsp<float>(c, c->ws.energy);
-            a4.drop = c->has_probe_tmaps ? c->work + c->ws.z1drop : nullptr;
-            a4.hist = wsp<uint32_t>(c, c->ws.hist);
-            CU(launch_split4_hist(a4, s.dtype, st));
-        }
-        SelectArgs sa;
-        sa.ut_begin = ut_begin; sa.ut_count = ut_count;
-        sa.T = T; sa.d = s.d;
-        sa.k = (int64_t)T * s.d * s.keep_num / s.keep_den;
-        sa.unit_stride = (int64_t)s.Tmax * s.d; sa.kcap = s.kcap; sa.ntiles_max = s.ntiles_max;
-        sa.z1 = c->work + c->ws.energy;
-        sa.hist = wsp<uint32_t>(c, c->ws.hist);
-        sa.sel = wsp<SelState>(c, c->ws.sel);
-        sa.lb_records = wsp<unsigned long long>(c, c->ws.lb_records);
-        sa.lb_ticket = wsp<uint32_t>(c, c->ws.lb_ticket);
-        sa.tile_off = wsp<int32_t>(c, c->ws.tile_off);
-        sa.idx = wsp<int32_t>(c, c->ws.idx);
-        sa.val = c->work + c->ws.eval;
-        sa.packed = nullptr;
-        sa.z1drop = nullptr;
-        sa.status = wsp<int32_t>(c, c->ws.status);
-        CU(launch_select_and_compact(sa, FDKV_F32, st));
-        Gather4Args g;
-        g.ut_begin = ut_begin; g.ut_count = ut_count;
-        g.k = sa.k; g.kcap = s.kcap; g.unit_stride = (int64_t)s.Tmax * s.d;
-        g.dev = c->work + c->ws.z1;
-        g.idx = wsp<int32_t>(c, c->ws.idx);
-        g.val = c->work + c->ws.val;
-        g.packed = c->packed_lists ? wsp<uint32_t>(c, c->ws.packed) : nullptr;
-        g.drop = c->has_probe_tmaps ? c->work + c->ws.z1drop : nullptr;  // tensor-core probe: the K deviations without the kept positions
-        CU(launch_gather4(g, s.dtype, st));
-        for (int p = pb; p < pe; ++p) { c->pair_compressed[p] = 1; c->pair_probed[p] = 0; c->pair_scored[p] = 0; }
-        return FDKV_OK;
-    }
-    for (int p0 = pb; p0 < pe; p0 += kSplitPairs) {
-        CompressArgs a;
-        a.n_pairs = pe - p0 < kSplitPairs ? pe - p0 : kSplitPairs;
-        for (int j = 0; j < a.n_pairs; ++j) {
-            const int p = p0 + j;
-            a.k0[j] = k_layers[2 * p]; a.k1[j] = k_layers[2 * p + 1];
-            a.v0[j] = v_layers[2 * p]; a.v1[j] = v_layers[2 * p + 1];
-            c->k_layers[2 * p] = a.k0[j]; c->k_layers[2 * p + 1] = a.k1[j];
-            c->v_layers[2 * p] = a.v0[j]; c->v_layers[2 * p + 1] = a.v1[j];
-        }
-        a.stride_t = stride_t; a.stride_h = stride_h;
-        a.T = T; a.d = s.d; a.Hkv = s.Hkv; a.tensors = 2;
-        a.ut_base = p0 * s.Hkv * 2;
-        a.unit_stride = (int64_t)s.Tmax * s.d; a.z0_stride = (int64_t)(c->z0_stride / s.esize);
-        a.z0 = c->z0_base; a.z1 = c->work + c->ws.z1;
-        a.hist = wsp<uint32_t>(c, c->ws.hist);
-        CU(launch_split_hist(a, s.dtype, st));
-    }
-    SelectArgs sa;
-    sa.ut_begin = ut_begin; sa.ut_count = ut_count;
-    sa.T = T; sa.d = s.d;
-    sa.k = (int64_t)T * s.d * s.keep_num / s.keep_den;
-    sa.unit_stride = (int64_t)s.Tmax * s.d; sa.kcap = s.kcap; sa.ntiles_max = s.ntiles_max;
-    sa.z1 = c->work + c->ws.z1;
-    sa.hist = wsp<uint32_t>(c, c->ws.hist);
-    sa.sel = wsp<SelState>(c, c->ws.sel);
-    sa.lb_records = wsp<unsigned long long>(c, c->ws.lb_records);
-    sa.lb_ticket = wsp<uint32_t>(c, c->ws.lb_ticket);
-    sa.tile_off = wsp<int32_t>(c, c->ws.tile_off);
-    sa.idx = wsp<int32_t>(c, c->ws.idx);
-    sa.val = c->work + c->ws.val;
-    sa.packed = c->packed_lists ? wsp<uint32_t>(c, c->ws.packed) : nullptr;
-    sa.z1drop = c->has_probe_tmaps ? c->work + c->ws.z1drop : nullptr;
-    sa.status = wsp<int32_t>(c, c->ws.status);
-    CU(launch_select_and_compact(sa, s.dtype, st));
+    CompressArgs a = entry_args(c, T);
+    a.stride_t = stride_t; a.stride_h = stride_h;
+    a.z0 = c->z0_base; a.z0_stride = (int64_t)(c->z0_stride / s.esize);
+    a.z1 = c->work + c->ws.z1;
+    a.keep = c->has_probe_tmaps ? wsp<uint32_t>(c, c->ws.keep) : nullptr;
+    CU(launch_compress(a, s.B, s.dtype, k_layers, v_layers, pb, pe, st));
     for (int p = pb; p < pe; ++p) { c->pair_compressed[p] = 1; c->pair_probed[p] = 0; c->pair_scored[p] = 0; }
     return FDKV_OK;
 }
@@ -455,7 +402,8 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
     a.T = T; a.d = s.d; a.Hq = s.Hq; a.Hkv = s.Hkv; a.G = s.G; a.W = W;
     a.unit_stride = (int64_t)s.Tmax * s.d; a.kcap = s.kcap;
     a.ntiles_max = s.ntiles_max; a.nptiles_max = s.nptiles_max;
-    a.z1 = c->work + c->ws.z1;
+    a.z1 = c->work + c->ws.z1; a.z1drop = c->work + c->ws.z1drop;
+    a.keep = s.tok_rule ? nullptr : wsp<uint32_t>(c, c->ws.keep); a.keep_stride = s.cand_stride / 32;
     a.idx = wsp<int32_t>(c, c->ws.idx);
     a.tile_off = wsp<int32_t>(c, c->ws.tile_off);
     a.sums_ready = s.tok_rule;
@@ -904,68 +852,14 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
     // ---- Eq. 1 and the chunk's own selection, through the staging area ----
     c->staged_seq = -1;
     std::fill(c->pair_compressed.begin(), c->pair_compressed.end(), 0);
-    CU(cudaMemsetAsync(wsp<uint32_t>(c, c->ws.hist), 0, (size_t)s.NT * kHistBins * 4, st));
     const int64_t kc = (int64_t)n * s.d * s.keep_num / s.keep_den;
-    SelectArgs sa;
-    sa.ut_begin = 0; sa.ut_count = s.NT;
-    sa.T = n; sa.d = s.d; sa.k = kc;
-    sa.unit_stride = (int64_t)s.Tmax * s.d; sa.kcap = s.kcap; sa.ntiles_max = s.ntiles_max;
-    sa.hist = wsp<uint32_t>(c, c->ws.hist);
-    sa.sel = wsp<SelState>(c, c->ws.sel);
-    sa.lb_records = wsp<unsigned long long>(c, c->ws.lb_records);
-    sa.lb_ticket = wsp<uint32_t>(c, c->ws.lb_ticket);
-    sa.tile_off = wsp<int32_t>(c, c->ws.tile_off);
-    sa.idx = wsp<int32_t>(c, c->ws.idx);
-    sa.z1drop = nullptr;
-    sa.status = wsp<int32_t>(c, c->ws.status);
-    if (s.B == 4) {
-        for (int p = 0; p < s.P; ++p) {
-            Split4Args a4;
-            for (int l = 0; l < 4; ++l) { a4.k[l] = tail_base(tk, 4 * p + l); a4.v[l] = tail_base(tv, 4 * p + l); }
-            a4.stride_t = s.d; a4.stride_h = (int64_t)s.tail_rows * s.d;
-            a4.T = n; a4.d = s.d; a4.Hkv = s.Hkv;
-            a4.ut_base = p * s.Hkv * 2;
-            a4.unit_stride = a4.z0_stride = (int64_t)s.Tmax * s.d;
-            a4.z0 = c->work + c->ws.z0; a4.dev = c->work + c->ws.z1;
-            a4.energy = wsp<float>(c, c->ws.energy);
-            a4.drop = nullptr;
-            a4.hist = wsp<uint32_t>(c, c->ws.hist);
-            CU(launch_split4_hist(a4, s.dtype, st));
-        }
-        sa.z1 = c->work + c->ws.energy;
-        sa.val = c->work + c->ws.eval;
-        sa.packed = nullptr;
-        CU(launch_select_and_compact(sa, FDKV_F32, st));
-        Gather4Args g;
-        g.ut_begin = 0; g.ut_count = s.NT;
-        g.k = kc; g.kcap = s.kcap; g.unit_stride = (int64_t)s.Tmax * s.d;
-        g.dev = c->work + c->ws.z1;
-        g.idx = wsp<int32_t>(c, c->ws.idx);
-        g.val = c->work + c->ws.val;
-        g.packed = c->packed_lists ? wsp<uint32_t>(c, c->ws.packed) : nullptr;
-        g.drop = nullptr;
-        CU(launch_gather4(g, s.dtype, st));
-    } else {
-        for (int p0 = 0; p0 < s.P; p0 += kSplitPairs) {
-            CompressArgs a;
-            a.n_pairs = s.P - p0 < kSplitPairs ? s.P - p0 : kSplitPairs;
-            for (int j = 0; j < a.n_pairs; ++j) {
-                const int p = p0 + j;
-                a.k0[j] = tail_base(tk, 2 * p); a.k1[j] = tail_base(tk, 2 * p + 1);
-                a.v0[j] = tail_base(tv, 2 * p); a.v1[j] = tail_base(tv, 2 * p + 1);
-            }
-            a.stride_t = s.d; a.stride_h = (int64_t)s.tail_rows * s.d;
-            a.T = n; a.d = s.d; a.Hkv = s.Hkv; a.tensors = 2;
-            a.ut_base = p0 * s.Hkv * 2;
-            a.unit_stride = a.z0_stride = (int64_t)s.Tmax * s.d;
-            a.z0 = c->work + c->ws.z0; a.z1 = c->work + c->ws.z1;
-            a.hist = wsp<uint32_t>(c, c->ws.hist);
-            CU(launch_split_hist(a, s.dtype, st));
-        }
-        sa.z1 = c->work + c->ws.z1;
-        sa.val = c->work + c->ws.val;
-        sa.packed = c->packed_lists ? wsp<uint32_t>(c, c->ws.packed) : nullptr;
-        CU(launch_select_and_compact(sa, s.dtype, st));
+    {
+        std::vector<const void*> kp(s.L), vp(s.L);
+        for (int l = 0; l < s.L; ++l) { kp[l] = tail_base(tk, l); vp[l] = tail_base(tv, l); }
+        CompressArgs a = entry_args(c, n);
+        a.stride_t = s.d; a.stride_h = (int64_t)s.tail_rows * s.d;
+        a.z0 = c->work + c->ws.z0; a.z0_stride = (int64_t)s.Tmax * s.d;
+        CU(launch_compress(a, s.B, s.dtype, kp.data(), vp.data(), 0, s.P, st));
     }
     // ---- append behind every unit's rows and lists, under the unit's mode ----
     const size_t unit_stride_b = (size_t)s.Tmax * s.d * s.esize, chunk_b = (size_t)n * row_b, at = (size_t)T0 * row_b;
@@ -1016,7 +910,7 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
     // ---- the remaining tail rows move down: through the staging area, as many layers at a time as it holds, where the ranges
     // overlap ----
     if (rest > 0) {
-        const size_t w = (size_t)rest * row_b, layer_b = 2 * (size_t)s.Hkv * w, room = (size_t)s.NT * s.NB * unit_stride_b;
+        const size_t w = (size_t)rest * row_b, layer_b = 2 * (size_t)s.Hkv * w, room = (size_t)s.NU * s.NB * unit_stride_b;
         const int group = rest <= n ? s.L : (int)std::max<size_t>(1, std::min<size_t>(s.L, room / layer_b));
         for (int l0 = 0; l0 < s.L; l0 += group) {
             CopyTable<2> moves;

@@ -1,6 +1,5 @@
-// Prefill compression kernels: depth split (Eq. 1, B = 2) fused with the magnitude histogram and the
-// radix-select threshold of the sparse residual (Eq. 3, entry form); the index-ordered compaction that follows
-// is select_fused.cu.
+// Prefill kernels beside the selection (select.cu): the depth split of the token rule (Eq. 1), the rows it keeps, the copies
+// of the commit step, and the entry point that compresses one tensor pair without a context.
 #include <algorithm>
 #include <mutex>
 
@@ -9,8 +8,6 @@
 namespace fdkv {
 
 namespace {
-
-__device__ __forceinline__ uint32_t key_of(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
 
 // ----- storage traits -------------------------------------------------------------------------------
 template <typename T>
@@ -55,75 +52,9 @@ __device__ __forceinline__ float stored<float>(float x) { return x; }
 template <>
 __device__ __forceinline__ float stored<__nv_bfloat16>(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-// ----- C1: depth split + histogram of the top 15 magnitude bits of z1 ---------------------------------
-// grid (chunks, Hkv*tensors, pairs); each CTA owns a token range of one unit-tensor and a private 128 KiB histogram.
-template <typename T>
-__global__ void __launch_bounds__(1024) split_hist_kernel(CompressArgs a, int tokens_per_cta) {
-    extern __shared__ uint32_t s_hist[];
-    using S = Store<T>;
-    constexpr int VEC = S::VEC;
-    for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) s_hist[b] = 0;
-    __syncthreads();
-
-    const int h = blockIdx.y / a.tensors, is_v = blockIdx.y % a.tensors, pj = blockIdx.z;
-    const int ut = a.ut_base + pj * a.Hkv * a.tensors + blockIdx.y;
-    const T* x0 = reinterpret_cast<const T*>(is_v ? a.v0[pj] : a.k0[pj]) + (int64_t)h * a.stride_h;
-    const T* x1 = reinterpret_cast<const T*>(is_v ? a.v1[pj] : a.k1[pj]) + (int64_t)h * a.stride_h;
-    T* z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride;
-    T* z1 = reinterpret_cast<T*>(a.z1) + (int64_t)ut * a.unit_stride;
-    const float c32 = __uint_as_float(0x3F3504F3u);
-
-    const int t_begin = blockIdx.x * tokens_per_cta;
-    const int t_end = min(a.T, t_begin + tokens_per_cta);
-    const int vpr = a.d / VEC;
-    const int64_t nvec = (int64_t)max(0, t_end - t_begin) * vpr;
-    // two vector pairs in flight per thread: all four loads are issued before the first is used
-    for (int64_t v0 = threadIdx.x; v0 < nvec; v0 += 2 * (int64_t)blockDim.x) {
-        typename S::vec_t va[2], vb[2];
-        int64_t off_in[2], off_out[2];
-        bool live[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int64_t v = v0 + (int64_t)u * blockDim.x;
-            live[u] = v < nvec;
-            const int t = t_begin + (int)(v / vpr);
-            const int cv = (int)(v % vpr) * VEC;
-            off_in[u] = (int64_t)t * a.stride_t + cv;
-            off_out[u] = (int64_t)t * a.d + cv;
-            if (live[u]) {
-                va[u] = *reinterpret_cast<const typename S::vec_t*>(x0 + off_in[u]);
-                vb[u] = *reinterpret_cast<const typename S::vec_t*>(x1 + off_in[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (!live[u]) continue;
-            float fa[VEC], fb[VEC], f0[VEC], f1[VEC];
-            S::unpack(va[u], fa);
-            S::unpack(vb[u], fb);
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) {
-                // one float32 add (subtract), one float32 multiply: never contracted into an FMA
-                f0[i] = __fmul_rn(__fadd_rn(fa[i], fb[i]), c32);
-                f1[i] = __fmul_rn(__fsub_rn(fa[i], fb[i]), c32);
-            }
-            *reinterpret_cast<typename S::vec_t*>(z0 + off_out[u]) = S::pack(f0);
-            *reinterpret_cast<typename S::vec_t*>(z1 + off_out[u]) = S::pack(f1);
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) atomicAdd(&s_hist[key_of(stored<T>(f1[i])) >> 16], 1u);
-        }
-    }
-    __syncthreads();
-    uint32_t* gh = a.hist + (int64_t)ut * kHistBins;
-    for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) {
-        const uint32_t c = s_hist[b];
-        if (c) atomicAdd(&gh[b], c);
-    }
-}
-
-// ----- C1 without a selection (token rule: the probe selects) ----------------------------------------
+// ----- the split without a selection (token rule: the probe selects) ---------------------------------
 // Shared coefficients of K and V and the high-frequency rows of K (Z1 of a pair, or the four layers' deviations: what the
-// probe scores), in the arithmetic of split_hist_kernel / split4_hist_kernel.  V's high-frequency rows are only wanted for
+// probe scores), in the arithmetic of select.cu.  V's high-frequency rows are only wanted for
 // the few tokens that are kept, so the commit step forms those from the caller's rows instead of staging all of them.
 // Bound by HBM: no histogram, so no shared memory, full occupancy and one launch over all blocks (it shared the histogram
 // kernel before, one launch per block of four: 8 191 tokens, 8 blocks of four: 963 us); two vectors of every
@@ -136,7 +67,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(SplitRowsArgs a) {
     const int h = blockIdx.y >> 1, is_v = blockIdx.y & 1, blk = blockIdx.z;
     const int64_t ut = a.ut_base + (int64_t)blk * a.Hkv * 2 + blockIdx.y;
     T* const z0 = reinterpret_cast<T*>(a.z0) + ut * a.z0_stride;
-    T* const hf = reinterpret_cast<T*>(a.hf) + ut * (B == 4 ? 4 : 1) * a.unit_stride;
+    T* const hf = reinterpret_cast<T*>(a.hf) + (ut >> 1) * (B == 4 ? 4 : 1) * a.unit_stride;
     const float c32 = __uint_as_float(0x3F3504F3u);
     const int vpr = a.d / VEC;
     const int nvec = a.T * vpr;
@@ -222,164 +153,7 @@ __global__ void __launch_bounds__(256) token_gather_kernel(const TokenGatherJob*
     }
 }
 
-// ----- C2: threshold from a histogram --------------------------------------------------------------
-// One CTA per unit-tensor.  Scans `nbins` bins from the top: finds the bin where the running count of larger
-// keys first reaches k_rem, appends the bin to the prefix and lowers k_rem.  Clears the bins it read.
-// On the last pass writes tau (prefix left-aligned to 31 bits) and need.
-__global__ void __launch_bounds__(1024) threshold_kernel(uint32_t* hist, SelState* sel, int ut_begin, int nbins,
-                                                         int bits, int first, int last, int shift_final,
-                                                         uint32_t k_init) {
-    __shared__ uint32_t s_tot[32];
-    __shared__ uint32_t s_found_bin, s_found_above;
-    const int ut = ut_begin + blockIdx.x;
-    uint32_t* h = hist + (int64_t)ut * kHistBins;
-    SelState st = sel[ut];
-    if (first) { st.prefix = 0; st.k_rem = k_init; }
-    // Warp w owns the segment of nbins / nwarps bins below nbins - w * seg (warp 0 the largest keys) and reads it in
-    // rows of 32 consecutive bins, largest first: lane l of row i holds bin hi - 1 - 32 i - l.
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int seg = nbins / nwarps, rows = seg / 32;  // nbins is a multiple of 32 * nwarps (32768 / 1024 threads, 256 / 256)
-    const int hi = nbins - warp * seg;
-    uint32_t mine = 0;
-    for (int i = 0; i < rows; ++i) mine += h[hi - 1 - 32 * i - lane];
-#pragma unroll
-    for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
-    if (lane == 0) s_tot[warp] = mine;
-    if (threadIdx.x == 0) { s_found_bin = 0xFFFFFFFFu; s_found_above = 0; }
-    __syncthreads();
-    uint32_t above = 0;  // keys in the segments of larger keys
-    for (int w = 0; w < warp; ++w) above += s_tot[w];
-    if (st.k_rem > 0 && above < st.k_rem && st.k_rem <= above + mine) {
-        // the k-th key lies in this warp's segment: walk its rows with a warp scan (the condition is warp-uniform)
-        for (int i = 0; i < rows; ++i) {
-            const int b = hi - 1 - 32 * i - lane;
-            const uint32_t c = h[b];
-            uint32_t incl = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const uint32_t before = above + incl - c;  // keys larger than bin b
-            const uint32_t hit = __ballot_sync(0xFFFFFFFFu, before < st.k_rem && st.k_rem <= before + c);
-            if (hit) {
-                if (lane == __ffs((int)hit) - 1) { s_found_bin = (uint32_t)b; s_found_above = before; }
-                break;
-            }
-            above += __shfl_sync(0xFFFFFFFFu, incl, 31);
-        }
-    }
-    __syncthreads();
-    for (int i = 0; i < rows; ++i) h[hi - 1 - 32 * i - lane] = 0;
-    if (threadIdx.x == 0) {
-        if (st.k_rem == 0 || s_found_bin == 0xFFFFFFFFu) {
-            // nothing (left) to take: a threshold above every key
-            st.prefix = 0xFFFFFFFFu;
-            st.k_rem = 0;
-            if (last) { st.tau = 0xFFFFFFFFu; st.need = 0; }
-        } else {
-            st.prefix = (st.prefix << bits) | s_found_bin;
-            st.k_rem -= s_found_above;
-            if (last) { st.tau = st.prefix << shift_final; st.need = st.k_rem; }
-        }
-        sel[ut] = st;
-    }
-}
-
-// ----- C2b (float32 only): histogram of the next 8 key bits among entries that match the prefix ------
-// The first refinement (prefix = the 15 bits of the split's histogram) also collects the low 16 bits of every matching
-// key in the unit-tensor's index list, which nothing has written yet (`cap` entries); the histogram holds the bins in
-// words [0, 256), the candidate count in word 256 and an overflow flag in word 257.  The second refinement then reads
-// those candidates instead of the whole tensor; only if they did not fit does the full pass run again.
-constexpr int kCandCount = 256, kCandOverflow = 257;
-constexpr int kCandBlock = 2048;  // candidates a thread block of the first refinement gathers before its one reservation in the list
-__global__ void __launch_bounds__(256) refine_hist_kernel(const float* z1, int64_t unit_stride, int64_t n,
-                                                          int ut_begin, const SelState* sel, uint32_t* hist,
-                                                          int shift_prefix, int shift_digit, int32_t* cand_all, int64_t cap,
-                                                          int only_on_overflow) {
-    __shared__ uint32_t s_h[256];
-    __shared__ uint16_t s_c[kCandBlock];
-    __shared__ uint32_t s_n, s_base;
-    const int ut = ut_begin + blockIdx.y;
-    uint32_t* const h = hist + (int64_t)ut * kHistBins;
-    if (only_on_overflow && !h[kCandOverflow]) return;  // (block-uniform: the candidates served this pass)
-    s_h[threadIdx.x] = 0;
-    if (threadIdx.x == 0) s_n = 0;
-    __syncthreads();
-    const uint32_t prefix = sel[ut].prefix;
-    if (prefix != 0xFFFFFFFFu) {
-        const float* z = z1 + (int64_t)ut * unit_stride;
-        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-            const uint32_t key = key_of(z[i]);
-            if ((key >> shift_prefix) == prefix) {
-                atomicAdd(&s_h[(key >> shift_digit) & 0xFFu], 1u);
-                if (cand_all) {
-                    const uint32_t pos = atomicAdd(&s_n, 1u);
-                    if (pos < (uint32_t)kCandBlock) s_c[pos] = (uint16_t)(key & 0xFFFFu);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    if (s_h[threadIdx.x]) atomicAdd(&h[threadIdx.x], s_h[threadIdx.x]);
-    if (cand_all) {
-        const uint32_t mine = s_n;
-        if (threadIdx.x == 0) {
-            s_base = atomicAdd(&h[kCandCount], mine);
-            if (mine > (uint32_t)kCandBlock) h[kCandOverflow] = 1u;  // more than the block could hold: the full pass runs again
-        }
-        __syncthreads();
-        const uint32_t base = s_base;
-        for (uint32_t i = threadIdx.x; i < min(mine, (uint32_t)kCandBlock); i += blockDim.x)
-            if ((int64_t)(base + i) < cap) cand_all[(int64_t)ut * cap + base + i] = (int32_t)s_c[i];
-    }
-}
-// second refinement from the collected candidates: one thread block per unit-tensor
-__global__ void __launch_bounds__(256) refine_candidates_kernel(int ut_begin, const SelState* sel, uint32_t* hist, const int32_t* cand_all,
-                                                                int64_t cap) {
-    __shared__ uint32_t s_h[256];
-    const int ut = ut_begin + blockIdx.x;
-    uint32_t* const h = hist + (int64_t)ut * kHistBins;
-    const uint32_t count = h[kCandCount];
-    if ((int64_t)count > cap || h[kCandOverflow]) {  // they did not fit: the full pass that follows does the work
-        if (threadIdx.x == 0) h[kCandOverflow] = 1u;
-        return;
-    }
-    s_h[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t prefix = sel[ut].prefix;  // 23 bits by now: the candidates share its upper 15
-    if (prefix != 0xFFFFFFFFu)
-        for (uint32_t i = threadIdx.x; i < count; i += blockDim.x) {
-            const uint32_t c = (uint32_t)cand_all[(int64_t)ut * cap + i];
-            if ((c >> 8) == (prefix & 0xFFu)) atomicAdd(&s_h[c & 0xFFu], 1u);
-        }
-    __syncthreads();
-    if (s_h[threadIdx.x]) h[threadIdx.x] = s_h[threadIdx.x];
-}
-
-// (C3-C5, the index-ordered compaction, live in select_fused.cu.)
-
 }  // namespace
-
-cudaError_t launch_split_hist(const CompressArgs& a, int dtype, cudaStream_t st) {
-    static PerDevice once;
-    const size_t smem = (size_t)kHistBins * sizeof(uint32_t);
-    cudaError_t e0 = once.ensure([&]() {
-        cudaError_t e = cudaFuncSetAttribute(split_hist_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(split_hist_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    });
-    if (e0 != cudaSuccess) return e0;
-    if (a.T <= 0 || a.n_pairs <= 0) return cudaSuccess;
-    const int tokens_per_cta = 4096 * 128 / a.d / (dtype == FDKV_BF16 ? 1 : 2);
-    dim3 grid((a.T + tokens_per_cta - 1) / tokens_per_cta, a.Hkv * a.tensors, a.n_pairs);
-    if (dtype == FDKV_BF16)
-        split_hist_kernel<__nv_bfloat16><<<grid, 1024, smem, st>>>(a, tokens_per_cta);
-    else
-        split_hist_kernel<float><<<grid, 1024, smem, st>>>(a, tokens_per_cta);
-    count_launch(1);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_split_rows(const SplitRowsArgs& a, int B, int dtype, cudaStream_t st) {
     if (a.T <= 0 || a.n_blocks <= 0) return cudaSuccess;
@@ -411,31 +185,6 @@ cudaError_t launch_token_gather_jobs(const TokenGatherJob* jobs_dev, int njobs, 
         count_launch(1);
     }
     return cudaGetLastError();
-}
-
-cudaError_t launch_select_and_compact(const SelectArgs& a, int dtype, cudaStream_t st) {
-    if (a.ut_count <= 0) return cudaSuccess;
-    const uint32_t k = (uint32_t)a.k;
-    const int64_t n = (int64_t)a.T * a.d;
-    if (dtype == FDKV_BF16) {
-        threshold_kernel<<<a.ut_count, 1024, 0, st>>>(a.hist, a.sel, a.ut_begin, kHistBins, 15, 1, 1, 16, k);
-        count_launch(1);
-    } else {
-        threshold_kernel<<<a.ut_count, 1024, 0, st>>>(a.hist, a.sel, a.ut_begin, kHistBins, 15, 1, 0, 0, k);
-        const int chunks = (int)std::min<int64_t>(64, (n + 256 * 16 - 1) / (256 * 16));
-        refine_hist_kernel<<<dim3(chunks, a.ut_count), 256, 0, st>>>(reinterpret_cast<const float*>(a.z1), a.unit_stride,
-                                                                     n, a.ut_begin, a.sel, a.hist, 16, 8, a.idx, a.kcap, 0);
-        threshold_kernel<<<a.ut_count, 256, 0, st>>>(a.hist, a.sel, a.ut_begin, 256, 8, 0, 0, 0, k);
-        refine_candidates_kernel<<<a.ut_count, 256, 0, st>>>(a.ut_begin, a.sel, a.hist, a.idx, a.kcap);
-        refine_hist_kernel<<<dim3(chunks, a.ut_count), 256, 0, st>>>(reinterpret_cast<const float*>(a.z1), a.unit_stride,
-                                                                     n, a.ut_begin, a.sel, a.hist, 8, 0, nullptr, 0, 1);
-        threshold_kernel<<<a.ut_count, 256, 0, st>>>(a.hist, a.sel, a.ut_begin, 256, 8, 0, 1, 0, k);
-        count_launch(6);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (a.T <= 0) return cudaSuccess;
-    return launch_select_fused(a, dtype, st);
 }
 
 // grid (chunks of 32 KiB of the largest job, jobs): the device-to-device copies of a commit or a fold (row streams, strided
@@ -489,23 +238,24 @@ cudaError_t launch_copy_jobs(const CopyJob* jobs_dev, int njobs, int64_t bytes_m
 
 // ---------------------------------------------------------------------------------------------------------------
 // Allocation-free compression of one [T][d] tensor pair (declared in fdkv.h as fdkv_compress_unit_noalloc).
-// Same kernels as fdkv_compress_prefill; the scratch they need (the Z1 temporary, the magnitude histogram, the
-// select state, the look-back records and the tile offsets) lives in the file-scope device array below instead of a
-// caller-provided workspace.  Every GPU that loads this library holds the array until the process exits.
+// Same kernels as fdkv_compress_prefill; the scratch they need (the candidate lists, the select state and the tile
+// offsets) lives in the file-scope device array below instead of a caller-provided workspace.  Every GPU that loads this library holds the array until the process exits.
 // ---------------------------------------------------------------------------------------------------------------
 namespace fdkv {
 namespace {
 
 constexpr int64_t kNoAllocMaxElems = FDKV_NOALLOC_MAX_ELEMS;                    // T * head_dim
 constexpr int64_t kNoAllocMaxTiles = kNoAllocMaxElems / 64 / fdkv::kResTile;    // head_dim >= 64
-constexpr size_t kNaZ1 = 0;                                                     // Z1 temporary, float32 worst case
-constexpr size_t kNaHist = kNaZ1 + (size_t)kNoAllocMaxElems * 4;
-constexpr size_t kNaSel = kNaHist + (size_t)fdkv::kHistBins * 4;
+constexpr int64_t kNoAllocChunks = kNoAllocMaxElems / fdkv::compress_chunk(2, 4);  // (the smallest chunk a pair has)
+constexpr size_t kNaPos = 0;
+constexpr size_t kNaVal = kNaPos + (size_t)kNoAllocMaxElems * 2;                // float32 worst case
+constexpr size_t kNaCount = kNaVal + (size_t)kNoAllocMaxElems * 4;
+constexpr size_t kNaBase = kNaCount + (size_t)kNoAllocChunks * 4;
+constexpr size_t kNaSel = kNaBase + (size_t)kNoAllocChunks * 8;
 constexpr size_t kNaStatus = kNaSel + 256;
-constexpr size_t kNaRecords = kNaStatus + 256;
-constexpr size_t kNaTicket = kNaRecords + (size_t)kNoAllocMaxTiles * 8;
-constexpr size_t kNaOff = kNaTicket + 256;
+constexpr size_t kNaOff = kNaStatus + 256;
 constexpr size_t kNaBytes = (kNaOff + (size_t)(kNoAllocMaxTiles + 1) * 4 + 255) / 256 * 256;
+static_assert(kNoAllocMaxElems % fdkv::kMaxCompressChunk == 0 && kNaSel % 256 == 0, "whole chunks, aligned parts");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaBytes];
 
@@ -555,32 +305,24 @@ extern "C" fdkv_status fdkv_compress_unit_noalloc(const void* x0, const void* x1
     cudaError_t e = noalloc_scratch(&sc);
     if (e != cudaSuccess) return record_cuda_error(e);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    // the array keeps the previous call's contents: the histogram and the status word must start at zero
-    e = cudaMemsetAsync(sc + kNaHist, 0, (size_t)kHistBins * 4 + 512, st);
-    if (e != cudaSuccess) return record_cuda_error(e);
-
+    // (the array keeps the previous call's contents: the kernels write what they read; the status word is nobody's here)
     CompressArgs a;
-    a.k0[0] = x0; a.k1[0] = x1; a.v0[0] = x0; a.v1[0] = x1;
-    a.n_pairs = 1;
     a.stride_t = stride_t; a.stride_h = 0;
     a.T = T; a.d = head_dim; a.Hkv = 1; a.tensors = 1;
-    a.ut_base = 0; a.unit_stride = 0; a.z0_stride = 0;
-    a.z0 = z0_out; a.z1 = sc + kNaZ1;
-    a.hist = reinterpret_cast<uint32_t*>(sc + kNaHist);
-    if ((e = launch_split_hist(a, dtype, st)) != cudaSuccess) return record_cuda_error(e);
-
-    SelectArgs sa;
-    sa.ut_begin = 0; sa.ut_count = 1;
-    sa.T = T; sa.d = head_dim; sa.k = k;
-    sa.unit_stride = 0; sa.kcap = 0; sa.ntiles_max = (int)kNoAllocMaxTiles;
-    sa.z1 = sc + kNaZ1;
-    sa.hist = reinterpret_cast<uint32_t*>(sc + kNaHist);
-    sa.sel = reinterpret_cast<SelState*>(sc + kNaSel);
-    sa.lb_records = reinterpret_cast<unsigned long long*>(sc + kNaRecords);
-    sa.lb_ticket = reinterpret_cast<uint32_t*>(sc + kNaTicket);
-    sa.tile_off = reinterpret_cast<int32_t*>(sc + kNaOff);
-    sa.idx = idx_out; sa.val = val_out; sa.packed = nullptr; sa.z1drop = nullptr;
-    sa.status = reinterpret_cast<int32_t*>(sc + kNaStatus);
-    if ((e = launch_select_and_compact(sa, dtype, st)) != cudaSuccess) return record_cuda_error(e);
+    a.unit_stride = 0; a.z0_stride = 0;
+    a.z0 = z0_out; a.z1 = nullptr;
+    a.sel = reinterpret_cast<SelState*>(sc + kNaSel);
+    a.cand_pos = reinterpret_cast<uint16_t*>(sc + kNaPos);
+    a.cand_val = sc + kNaVal;
+    a.cand_n = reinterpret_cast<int32_t*>(sc + kNaCount);
+    a.chunk_base = reinterpret_cast<int2*>(sc + kNaBase);
+    a.cand_stride = kNoAllocMaxElems; a.chunks_max = (int)kNoAllocChunks;
+    a.n_keep = k; a.kcap = 0; a.ntiles_max = (int)kNoAllocMaxTiles;
+    a.tile_off = reinterpret_cast<int32_t*>(sc + kNaOff);
+    a.idx = idx_out; a.val = val_out; a.packed = nullptr;
+    a.keep = nullptr; a.keep_stride = 0;
+    a.status = reinterpret_cast<int32_t*>(sc + kNaStatus);
+    const void* const layers[2] = {x0, x1};
+    if ((e = launch_compress(a, 2, dtype, layers, layers, 0, 1, st)) != cudaSuccess) return record_cuda_error(e);
     return FDKV_OK;
 }

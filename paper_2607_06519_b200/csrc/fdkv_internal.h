@@ -14,7 +14,6 @@
 namespace fdkv {
 
 constexpr int kResTile = 16;         // tokens per residual-offset tile: off[j] = first list entry of tokens >= 16 j
-constexpr int kHistBins = 32768;     // one bin per 15-bit magnitude prefix (a whole bf16 key)
 constexpr int kMaxSplits = 160;      // split-K partial slots per (sequence, query head)
 constexpr int kMaxW = 128;           // probe queries
 constexpr int kListPad = 32;         // slack entries after each residual list (aligned over-reads stay in bounds)
@@ -72,10 +71,10 @@ struct FastPlan {
 };
 
 struct SelState {
-    uint32_t prefix;  // magnitude-key prefix fixed so far (left-aligned in 31 bits once complete)
-    uint32_t k_rem;   // entries still to take at or below the prefix
-    uint32_t tau;     // final threshold key (31-bit magnitude pattern; bf16 keys are shifted left by 16)
+    uint32_t lo;      // bound the candidates reach (31-bit key pattern; bf16 magnitudes are shifted left by 16)
+    uint32_t tau;     // threshold key: that of the k-th largest
     uint32_t need;    // entries with key == tau to keep (lowest flat indices first)
+    uint32_t redo;    // fewer than k positions reached the bound: split and threshold run again with bound 0
 };
 
 struct Shape {
@@ -94,14 +93,15 @@ struct Shape {
     int max_fold;      // generated tokens that may be folded into the compressed form per sequence
     int rows_f8;       // committed row streams are e4m3 codes with per-channel scales
     int64_t kfold_max; // floor(max_fold*d*num/den): list room reserved for them
-    int NB;            // staged high-frequency tensors per unit-tensor: 1 (Z1 of a pair) or 4 (the layers' deviations)
+    int NB;            // high-frequency tensors per unit-tensor: 1 (Z1 of a pair) or 4 (the layers' deviations)
+    int64_t cand_stride;  // Tmax*d rounded up to whole candidate chunks
+    int chunks_max;
     int64_t ktok_max, ktok_cap;  // floor(Tmax*num/den) and the list capacity incl. slack
 };
 
 struct WsLayout {
     size_t tok_score, tok_err, tok_list, tok_off;
-    size_t energy, eval;  // four-layer blocks: per-position high-frequency energy (float32) and the kept energies
-    size_t status, z0, z1, z1drop, hist, sel, lb_records, lb_ticket, tile_off, idx, val, packed, probe_part, probe_pos, scores, modes,
+    size_t status, z0, z1, z1drop, cand_pos, cand_val, cand_n, chunk_base, keep, sel, tile_off, idx, val, packed, probe_part, probe_pos, scores, modes,
         partials, io_q, io_k, io_v, io_out, jobs, total;  // io_*: host-I/O staging, [L] layers each
 };
 struct ArenaLayout {
@@ -161,22 +161,6 @@ struct fdkv_ctx {
 namespace fdkv {
 
 // ---- launchers implemented in compress.cu / probe.cu / decode.cu; each returns cudaGetLastError() ----
-constexpr int kSplitPairs = 32;  // layer pairs one launch of the split kernel covers
-struct CompressArgs {
-    // the four [T][Hkv][d] strided tensors (K and V of layers 2p, 2p+1) of each pair of the launch
-    const void *k0[kSplitPairs], *k1[kSplitPairs], *v0[kSplitPairs], *v1[kSplitPairs];
-    int n_pairs;
-    int64_t stride_t, stride_h;
-    int T, d, Hkv;
-    int tensors;  // 2: K and V of every head (unit-tensor = head*2 + is_v); 1: K only (unit-tensor = head)
-    int ut_base;  // first unit-tensor of the first pair in the stage; pair j adds j*Hkv*tensors
-    int64_t unit_stride;  // elements between staged unit-tensors (Tmax*d)
-    int64_t z0_stride;    // elements between the unit-tensors' shared coefficients
-    void *z0, *z1;
-    uint32_t* hist;
-};
-cudaError_t launch_split_hist(const CompressArgs& a, int dtype, cudaStream_t st);
-
 // The split alone (token rule), either block size; layer B * j + l is layer l of the launch's block j.
 constexpr int kSplitLayers = 64;  // layers one launch covers
 struct SplitRowsArgs {
@@ -188,58 +172,44 @@ struct SplitRowsArgs {
     int64_t unit_stride;  // elements between staged tensors (Tmax*d)
     int64_t z0_stride;    // elements between the unit-tensors' shared coefficients
     void* z0;             // [NT][z0_stride]
-    void* hf;             // [NT][1 or 4][unit_stride]: Z1 of a pair, or the layers' deviations of a block of four; K tensors only
+    void* hf;             // [unit][1 or 4][unit_stride]: Z1 of K of a pair, or the layers' deviations of a block of four
 };
 cudaError_t launch_split_rows(const SplitRowsArgs& a, int B, int dtype, cudaStream_t st);
 
-struct SelectArgs {
-    int ut_begin, ut_count;
-    int T, d;
-    int64_t k;
-    int64_t unit_stride, kcap;
-    int ntiles_max;
-    const void* z1;
-    uint32_t* hist;
-    SelState* sel;
-    unsigned long long* lb_records;  // look-back records of the ordered select: one 64-bit word per (unit-tensor, chunk), ntiles_max per unit-tensor
-    uint32_t* lb_ticket;             // its ticket counter (one word)
-    int32_t* tile_off;
-    int32_t* idx;
-    void* val;
-    void* z1drop;      // optional [unit][Tmax*d]: Z1 of K with the kept entries zeroed (tensor-core probe), or null
-    uint32_t* packed;  // optional packed entries for the bf16 / head_dim 128 decode kernel (null otherwise)
-    int32_t* status;
-};
-cudaError_t launch_select_and_compact(const SelectArgs& a, int dtype, cudaStream_t st);
-// count, offsets and ordered write as one pass over the keys (select_fused.cu); a.sel holds the thresholds
-cudaError_t launch_select_fused(const SelectArgs& a, int dtype, cudaStream_t st);
-
-// ---- four-layer blocks (block4.cu) ----
-struct Split4Args {
-    const void* k[4];  // the block's four [T][Hkv][d] strided K tensors, layer order
-    const void* v[4];
+// ---- entry rule: split, threshold, lists (select.cu) ----
+// positions of a candidate chunk: 256 threads take 8 positions of B layers as 128 bytes of each thread's loads
+__host__ __device__ constexpr int compress_chunk(int B, int esize) { return 8 / (B * esize / 2) * 256 * 8; }
+constexpr int kMaxCompressChunk = 8192;
+struct CompressArgs {
+    const void *k[kSplitLayers], *v[kSplitLayers];  // set by launch_compress: layer B * j + l is layer l of the launch's block j
     int64_t stride_t, stride_h;
     int T, d, Hkv;
-    int ut_base;          // first unit-tensor of the block (unit-tensor = head*2 + is_v)
-    int64_t unit_stride;  // elements between staged tensors (Tmax*d)
+    int tensors;          // 2: K and V of every head (unit-tensor = head*2 + is_v); 1: K only (unit-tensor = head)
+    int ut_base;          // set by launch_compress
+    int64_t unit_stride;  // elements between staged high-frequency tensors (Tmax*d)
     int64_t z0_stride;    // elements between the unit-tensors' shared coefficients
     void* z0;             // [NT][z0_stride]
-    void* dev;            // [NT][4][unit_stride]: deviation of each layer from the block mean
-    float* energy;        // [NT][unit_stride]
-    void* drop;           // optional [NU][4][unit_stride]: second copy of the K deviations (the gather zeroes its kept positions)
-    uint32_t* hist;
+    void* z1;             // optional [unit][1 or 4][unit_stride]: high-frequency rows of K (Z1 of a pair, the deviations of a block of four)
+    SelState* sel;        // [NT]
+    uint16_t* cand_pos;   // [NT][cand_stride] positions inside the chunk, ascending; chunk c's at c * compress_chunk
+    void* cand_val;       // [NT][1 or 4][cand_stride] their high-frequency values
+    int32_t* cand_n;      // [NT][chunks_max] candidates per chunk
+    int2* chunk_base;     // [NT][chunks_max] keys above / equal to the threshold in the chunks before
+    int64_t cand_stride;  // Tmax*d rounded up to whole chunks
+    int chunks_max;
+    int chunks;           // set by launch_compress: chunks of T tokens
+    int64_t n_keep, kcap; // entries per list and list capacity
+    int ntiles_max;
+    int32_t* tile_off;    // [NT][ntiles_max + 1]
+    int32_t* idx;         // [NT][kcap]
+    void* val;            // [NT][1 or 4][kcap]
+    uint32_t* packed;     // optional [NT][1 or 4][kcap] packed entries of the bf16 / head_dim 128 decode kernel
+    uint32_t* keep;       // optional [unit][keep_stride] bit map of the kept positions of K
+    int64_t keep_stride;  // 32-bit words
+    int32_t* status;
 };
-cudaError_t launch_split4_hist(const Split4Args& a, int dtype, cudaStream_t st);
-struct Gather4Args {
-    int ut_begin, ut_count;
-    int64_t k, kcap, unit_stride;
-    const void* dev;     // [NT][4][unit_stride]
-    const int32_t* idx;  // [NT][kcap] ascending kept positions
-    void* val;           // [NT][4][kcap] the four layers' values at the kept positions
-    uint32_t* packed;    // optional [NT][4][kcap] packed entries (value doubled: the rows are scaled by 1/2), or null
-    void* drop;          // optional [NU][4][unit_stride]: the K deviations (copied there beforehand); kept positions get zeroed
-};
-cudaError_t launch_gather4(const Gather4Args& a, int dtype, cudaStream_t st);
+cudaError_t launch_compress(CompressArgs& a, int B, int dtype, const void* const* k_layers, const void* const* v_layers, int block_begin, int block_end,
+                            cudaStream_t st);
 
 struct ProbeArgs {
     int B;  // layers per block: 2 (one Z1 operand, both layers' queries) or 4 (one deviation operand per layer)
@@ -247,7 +217,10 @@ struct ProbeArgs {
     int T, d, Hq, Hkv, G, W;
     int64_t unit_stride, kcap;
     int ntiles_max, nptiles_max;
-    const void* z1;  // staged Z1 (unit-tensor ut = unit*2 for K)
+    const void* z1;        // [unit][1 or 4][unit_stride] high-frequency rows of K
+    void* z1drop;          // [unit][1 or 4][unit_stride] room for a copy without the kept entries (tensor-core probe), or null
+    const uint32_t* keep;  // [unit][keep_stride] bit map of the kept positions of K
+    int64_t keep_stride;
     const int32_t* idx;
     const int32_t* tile_off;
     bool sums_ready;                  // token rule: part slot 0 of every unit holds the error sums already
@@ -353,7 +326,7 @@ struct TokenArgs {
     int unit_begin, unit_count;
     int T, Tmax, Hq, Hkv, G, W, ntiles_max;
     int64_t k_tok, ktok_cap, unit_stride;
-    const void* z1;                    // staged Z1 (K of unit u at unit-tensor 2u)
+    const void* z1;                    // [unit][1 or 4][unit_stride] high-frequency rows of K
     const void* const* q_layers_dev;
     const int32_t* pos;
     const int32_t* pos_host;

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(256) probe_tile_kernel(ProbeArgs a) {
     const int M = (a.B == 4 ? 1 : 2) * a.G * a.W;  // probe rows per operand
     float sum_f = 0.f, sum_d = 0.f;
     for (int op = 0; op < n_ops; ++op) {
-        const T* z1 = reinterpret_cast<const T*>(a.z1) + ((int64_t)ut * n_ops + op) * a.unit_stride + (int64_t)t0 * d;
+        const T* z1 = reinterpret_cast<const T*>(a.z1) + ((int64_t)unit * n_ops + op) * a.unit_stride + (int64_t)t0 * d;
         for (int i = threadIdx.x; i < kProbeTile * d; i += blockDim.x) {
             const int t = i / d, c = i % d;
             const float v = t < nt ? ldf<T>(z1 + i) : 0.f;

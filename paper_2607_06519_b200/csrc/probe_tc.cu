@@ -170,10 +170,8 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
         // ================= TMA producer =================
         if (lane == 0) {
             const CUtensorMap* map = cand ? &tmap_drop : &tmap_z1;
-            // rows of this unit's K coefficients: staged Z1 holds K and V per unit (unit-tensor 2*unit), the dropped copy K only
-            // (a block of four layers stages one operand per layer: [unit-tensor][4] and [unit][4])
-            const int64_t row0 = a.B == 4 ? ((cand ? (int64_t)unit : (int64_t)unit * 2) * 4 + layer) * a.Tmax
-                                          : (cand ? (int64_t)unit : (int64_t)unit * 2) * a.Tmax;
+            // rows of this unit's K coefficients (a block of four stages one operand per layer)
+            const int64_t row0 = a.B == 4 ? ((int64_t)unit * 4 + layer) * a.Tmax : (int64_t)unit * a.Tmax;
             for (int i = 0; i < ntile; ++i) {
                 const int s = i % kBStages;
                 const uint32_t ph = (uint32_t)(i / kBStages) & 1u;
@@ -290,6 +288,25 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
     }
 }
 
+// Rows [t0, t1) of every operand with the kept entries zeroed: the residual candidate's operand.  grid (blocks, units, operands
+// per unit), one 16-byte vector per thread and step.
+__global__ void __launch_bounds__(256) drop_rows_kernel(ProbeArgs a, int n_ops, int t0, int t1) {
+    const int unit = a.unit_begin + blockIdx.y;
+    const int64_t op = ((int64_t)unit * n_ops + blockIdx.z) * a.unit_stride;
+    const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.z1) + op);
+    uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.z1drop) + op);
+    const uint8_t* bits = reinterpret_cast<const uint8_t*>(a.keep + (int64_t)unit * a.keep_stride);
+    for (int64_t v = (int64_t)t0 * 16 + (int64_t)blockIdx.x * 256 + threadIdx.x; v < (int64_t)t1 * 16; v += (int64_t)gridDim.x * 256) {
+        uint4 x = src[v];
+        const uint32_t b = bits[v], m = b | (b << 15);  // bit j: element j is kept; word w's are bits 2w and 16 + 2w of m
+        x.x &= ~((m & 0x00010001u) * 0xFFFFu);
+        x.y &= ~(((m >> 2) & 0x00010001u) * 0xFFFFu);
+        x.z &= ~(((m >> 4) & 0x00010001u) * 0xFFFFu);
+        x.w &= ~(((m >> 6) & 0x00010001u) * 0xFFFFu);
+        dst[v] = x;
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool* handled, int* nparts) {
@@ -313,6 +330,11 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     pl.items_per_unit = a.B * pl.mblocks * 2 * nsplits;
     const int slots = a.B * pl.mblocks * nsplits;
     if (slots > a.nptiles_max) return cudaErrorInvalidValue;  // cannot happen: the part array is sized for max_probe_parts()
+    {
+        const int t1 = std::min(a.T, pl.ntiles * kBN), n_ops = a.B == 4 ? 4 : 1;
+        drop_rows_kernel<<<dim3((unsigned)std::min<int64_t>(64, ((int64_t)t1 * 16 + 255) / 256), a.unit_count, n_ops), 256, 0, st>>>(a, n_ops, 0, t1);
+        count_launch(1);
+    }
     probe_tc_kernel<<<a.unit_count * pl.items_per_unit, kPThreads, kProbeSmem, st>>>(
         *reinterpret_cast<const CUtensorMap*>(a.tmap_z1), *reinterpret_cast<const CUtensorMap*>(a.tmap_drop), a, pl);
     cudaError_t e = cudaGetLastError();

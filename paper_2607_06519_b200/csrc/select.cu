@@ -1,0 +1,701 @@
+// Prefill compression with the entry rule (Eq. 1 and Eq. 3): depth split, threshold and index-ordered compaction of the
+// sparse residual, for pairs and for blocks of four layers, in one read of K and V.
+//
+// What is stored per position (float32, never contracted; rs = rounding to the storage type):
+//   pair:           z0 = rs((x0 + x1) c), z1 = rs((x0 - x1) c); key = magnitude of z1
+//   block of four:  s = (x0 + x1) + (x2 + x3), z0 = rs(s / 2), dev_l = rs(x_l - z0 / 2) (F_4's first row is 1/2 four
+//                   times, so z0 / 2 is the block mean and the other three coefficients contribute x_l - mean);
+//                   key = e = (dev_0^2 + dev_1^2) + (dev_2^2 + dev_3^2), the squared error dropping the position costs
+// and the k positions of largest key (31-bit patterns of non-negative floats; ties to the lowest flat index) are listed in
+// ascending order with their values.
+//
+//   1. sample_kernel     one block per unit-tensor reads up to 64 Ki positions (whole rows, spread over the tokens with a
+//                        fixed jitter; all of them where there are no more) and sets a bound that about 1.2 k positions reach;
+//   2. split_kernel      reads every row once, writes Z0 (and, of K, the high-frequency rows the probe reads) and appends the
+//                        positions that reach the bound, in order, to the chunk's candidate list;
+//   3. threshold_kernel  one block per unit-tensor: the k-th largest key among the candidates (a radix select in shared
+//                        memory), then the keys above and equal to it before every chunk;
+//   4. compact_kernel    one block per chunk: candidates -> the lists, the offsets of the 16-token tiles and, of K, a bit
+//                        map of the kept positions.
+// The bound is only a guess: where fewer than k positions reach it, step 3 says so and steps 2 and 3 run again for that
+// unit-tensor with bound 0 (a chunk's list holds all of its positions), so the result never depends on the sample.
+// Bound by HBM: K and V are read once and about k / N x 1.2 of them written again; a pass that writes all high-frequency
+// values and reads them back to select (what this replaces) moved 5 instead of 3.6 times a tensor's bytes, and its
+// histogram of every key took 128 KiB of shared memory, one block per SM.
+#include <algorithm>
+#include <cmath>
+
+#include "fdkv_internal.h"
+
+namespace fdkv {
+
+namespace {
+
+constexpr int kSplitThreads = 256;
+constexpr int kSampleThreads = 512, kSampleBins = 4096;
+constexpr int64_t kSampleElems = 65536;
+constexpr int kThrThreads = 1024, kThrBins = 4096;
+constexpr uint32_t kNoKey = 0xFFFFFFFFu;  // a bound or threshold above every key
+
+// two float32 operations at a time, each rounded to nearest
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(uint32_t lo, uint32_t hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ f32x2 bf2(uint32_t w) { return pack2(w << 16, w & 0xFFFF0000u); }  // two bf16 values, widened
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return add2(a, b ^ 0x8000000080000000ull); }
+__device__ __forceinline__ uint32_t to_bf2(f32x2 a) {  // both halves to nearest-even bf16
+    uint32_t lo, hi, r;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(a));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
+    return r;
+}
+
+__device__ __forceinline__ float to_f32(float x) { return x; }
+__device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
+
+// the key of a position from its stored high-frequency value(s)
+template <int B>
+__device__ __forceinline__ uint32_t key_of(const float* v) {
+    if constexpr (B == 2) return __float_as_uint(v[0]) & 0x7FFFFFFFu;
+    else
+        return __float_as_uint(__fadd_rn(__fadd_rn(__fmul_rn(v[0], v[0]), __fmul_rn(v[1], v[1])),
+                                         __fadd_rn(__fmul_rn(v[2], v[2]), __fmul_rn(v[3], v[3])))) & 0x7FFFFFFFu;
+}
+
+// Eight consecutive positions as 16-byte vectors, Q of them per row: x[layer] -> shared coefficients z0 and high-frequency
+// values hf[1 or 4], and for_key(position, key) for each.
+template <typename T, int B>
+struct Eight;
+template <int B>
+struct Eight<__nv_bfloat16, B> {
+    static constexpr int Q = 1;
+    template <typename F>
+    __device__ static void split(const uint4 (&x)[B][1], uint4 (&z0)[1], uint4 (&hf)[B == 4 ? 4 : 1][1], F&& for_key) {
+        const f32x2 c = pack2(0x3F3504F3u, 0x3F3504F3u), half1 = pack2(0x3F000000u, 0x3F000000u);  // the float32 nearest 1/sqrt 2; 1/2
+        const uint32_t* const xw[B == 4 ? 4 : 2] = {reinterpret_cast<const uint32_t*>(&x[0][0]), reinterpret_cast<const uint32_t*>(&x[1][0])};
+        uint32_t* const zw = reinterpret_cast<uint32_t*>(&z0[0]);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if constexpr (B == 2) {
+                const f32x2 a = bf2(xw[0][w]), b = bf2(xw[1][w]);
+                zw[w] = to_bf2(mul2(add2(a, b), c));
+                const uint32_t h = to_bf2(mul2(sub2(a, b), c));
+                reinterpret_cast<uint32_t*>(&hf[0][0])[w] = h;
+                for_key(2 * w, (h << 16) & 0x7FFF0000u);
+                for_key(2 * w + 1, h & 0x7FFF0000u);
+            } else {
+                f32x2 v[4];
+#pragma unroll
+                for (int l = 0; l < 4; ++l) v[l] = bf2(reinterpret_cast<const uint32_t*>(&x[l][0])[w]);
+                zw[w] = to_bf2(mul2(half1, add2(add2(v[0], v[1]), add2(v[2], v[3]))));
+                const f32x2 half = mul2(half1, bf2(zw[w]));  // exact
+#pragma unroll
+                for (int l = 0; l < 4; ++l) {
+                    const uint32_t h = to_bf2(sub2(v[l], half));
+                    reinterpret_cast<uint32_t*>(&hf[l][0])[w] = h;
+                    v[l] = bf2(h);
+                    v[l] = mul2(v[l], v[l]);
+                }
+                const f32x2 e = add2(add2(v[0], v[1]), add2(v[2], v[3]));
+                for_key(2 * w, (uint32_t)e & 0x7FFFFFFFu);
+                for_key(2 * w + 1, (uint32_t)(e >> 32) & 0x7FFFFFFFu);
+            }
+        }
+    }
+};
+template <int B>
+struct Eight<float, B> {
+    static constexpr int Q = 2;
+    template <typename F>
+    __device__ static void split(const uint4 (&x)[B][2], uint4 (&z0)[2], uint4 (&hf)[B == 4 ? 4 : 1][2], F&& for_key) {
+        const float c32 = __uint_as_float(0x3F3504F3u);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float f[B], h[B == 4 ? 4 : 1];
+#pragma unroll
+            for (int l = 0; l < B; ++l) f[l] = reinterpret_cast<const float*>(&x[l][0])[i];
+            float z;
+            if constexpr (B == 2) {
+                z = __fmul_rn(__fadd_rn(f[0], f[1]), c32);
+                h[0] = __fmul_rn(__fsub_rn(f[0], f[1]), c32);
+            } else {
+                z = __fmul_rn(0.5f, __fadd_rn(__fadd_rn(f[0], f[1]), __fadd_rn(f[2], f[3])));
+                const float half = __fmul_rn(0.5f, z);  // exact
+#pragma unroll
+                for (int l = 0; l < 4; ++l) h[l] = __fsub_rn(f[l], half);
+            }
+            reinterpret_cast<float*>(&z0[0])[i] = z;
+#pragma unroll
+            for (int l = 0; l < (B == 4 ? 4 : 1); ++l) reinterpret_cast<float*>(&hf[l][0])[i] = h[l];
+            for_key(i, key_of<B>(h));
+        }
+    }
+};
+
+// programmatic dependent launch: the next kernel of the chain may start its prologue now; nothing is read before the kernels
+// ahead are complete
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// The bin, from the top, at which the running count of BINS shared-memory bins first reaches `target`: every thread of the
+// block gets (bin, count in larger bins); false if the total is smaller.  A thread owns BINS / THREADS consecutive bins.
+template <int THREADS, int BINS>
+__device__ __forceinline__ bool find_bin(const uint32_t* bins, uint32_t target, uint32_t& bin, uint32_t& above) {
+    __shared__ uint32_t s_tot[THREADS / 32], s_bin, s_above;
+    constexpr int PER = BINS / THREADS;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int hi = BINS - PER * tid;
+    uint32_t c[PER], mine = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) { c[i] = bins[hi - 1 - i]; mine += c[i]; }
+    uint32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_tot[warp] = incl;
+    __syncthreads();
+    uint32_t before = incl - mine, total = 0;
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) {
+        if (w < warp) before += s_tot[w];
+        total += s_tot[w];
+    }
+    if (before < target && target <= before + mine) {
+        bool found = false;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            if (!found && before + c[i] >= target) { s_bin = (uint32_t)(hi - 1 - i); s_above = before; found = true; }
+            before += c[i];
+        }
+    }
+    __syncthreads();
+    bin = s_bin;
+    above = s_above;
+    __syncthreads();  // (the scratch words may be reused)
+    return target <= total;
+}
+
+// ---- 1: the bound -------------------------------------------------------------------------------------
+// grid (heads x tensors, blocks of the launch)
+template <typename T, int B>
+__global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, int n_rows, uint32_t target) {
+    __shared__ uint32_t s_hist[kSampleBins];
+    constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
+    const int tid = threadIdx.x;
+    const int ut = a.ut_base + blockIdx.y * gridDim.x + blockIdx.x;
+    const int h = blockIdx.x / a.tensors, is_v = blockIdx.x % a.tensors;
+    for (int i = tid; i < kSampleBins; i += kSampleThreads) s_hist[i] = 0;
+    chain_wait();
+    __syncthreads();
+    const T* x[B];
+#pragma unroll
+    for (int l = 0; l < B; ++l) x[l] = reinterpret_cast<const T*>(is_v ? a.v[B * blockIdx.y + l] : a.k[B * blockIdx.y + l]) + (int64_t)h * a.stride_h;
+    const int vshift = a.d == 128 ? 4 : 3, nvec = n_rows << vshift;
+    constexpr int U = 4;  // groups of eight whose rows are requested together
+    for (int v0 = tid; v0 < nvec; v0 += U * kSampleThreads) {
+        uint4 f[U][B][Q];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int v = v0 + q * kSampleThreads;
+            if (v >= nvec) break;
+            const int r = v >> vshift, cv = (v & ((1 << vshift) - 1)) * 8;
+            int t = r;
+            if (n_rows < a.T) {  // row r of the sample: somewhere in the r-th of n_rows equal parts of the tokens
+                const uint32_t jitter = (uint32_t)r * 2654435761u >> 16;  // (a multiplicative hash, 16 bits)
+                t = (int)((((uint64_t)(uint32_t)r << 16 | jitter) * (uint64_t)a.T) / ((uint64_t)n_rows << 16));
+            }
+#pragma unroll
+            for (int l = 0; l < B; ++l)
+#pragma unroll
+                for (int k = 0; k < Q; ++k) f[q][l][k] = reinterpret_cast<const uint4*>(x[l] + (int64_t)t * a.stride_t + cv)[k];
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            if (v0 + q * kSampleThreads >= nvec) break;
+            uint4 z0[Q], hf[NB][Q];
+            Eight<T, B>::split(f[q], z0, hf, [&](int, uint32_t key) { atomicAdd(&s_hist[key >> 19], 1u); });
+        }
+    }
+    __syncthreads();
+    uint32_t bin, above;
+    const bool enough = find_bin<kSampleThreads, kSampleBins>(s_hist, target, bin, above);
+    if (tid == 0) {
+        a.sel[ut].redo = 0;
+        a.sel[ut].lo = a.n_keep == 0 ? kNoKey : enough ? bin << 19 : 0u;
+    }
+}
+
+// position of the k-th (from zero) set bit of x; x has more than k set bits
+__device__ __forceinline__ int kth_set_bit(uint32_t x, uint32_t k) {
+    int pos = 0;
+#pragma unroll
+    for (int width = 16; width >= 1; width >>= 1) {
+        const uint32_t c = __popc(x & ((1u << width) - 1u));
+        if (k >= c) {
+            k -= c;
+            pos += width;
+            x >>= width;
+        }
+    }
+    return pos;
+}
+
+// ---- 2: one read of K and V ---------------------------------------------------------------------------
+// Persistent blocks over (chunk, head x tensor) items; heads and tensors vary fastest, so the blocks that run at one time read
+// neighbouring rows.  A warp owns NV * 256 consecutive positions of a chunk, a lane eight of them per step.  The rows of the
+// next item are copied to shared memory (cp.async, 16 bytes per lane and layer, every lane its own) while one is worked on; the
+// high-frequency values take the place of the rows they came from.  A byte per eight positions goes to a bit map; with its
+// prefix, lane r finds entry r of the warp's part of the list by binary search and a population-count descent, so that the
+// list is written by consecutive lanes whatever the distribution of the candidates.  One block barrier per item (the warps'
+// counts).
+template <typename T, int B>
+__global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a, int items, int redo) {
+    constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
+    constexpr int CE = compress_chunk(B, (int)sizeof(T)), NV = CE / kSplitThreads / 8;
+    constexpr int WW = NV * 8;           // words of a warp's part of the bit map
+    constexpr int ROW = CE * (int)sizeof(T);  // bytes of a layer's part of a stage
+    constexpr int STAGE = B * ROW;       // 32 KiB
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint32_t s_map[8][WW], s_pre[8][WW], s_cnt[2][8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int uts = a.Hkv * a.tensors;
+    chain_wait();
+    if (redo) {  // (almost always there is nothing to do again)
+        const int per_block = items / uts;  // chunks x blocks of the launch
+        const int nb = per_block / a.chunks;
+        int any = 0;
+        for (int i = tid; i < nb * uts; i += kSplitThreads) any |= (int)a.sel[a.ut_base + i].redo;
+        if (!__syncthreads_or(any)) return;
+    }
+    const int64_t n_e = (int64_t)a.T * a.d;
+    const int dshift = a.d == 128 ? 7 : 6;
+    // item -> unit-tensor of the launch, chunk
+    auto locate = [&](int item, int& ut, int& u, int& blk, int64_t& e0) {
+        u = item % uts;
+        const int r = item / uts;
+        blk = r / a.chunks;
+        e0 = (int64_t)(r - blk * a.chunks) * CE;
+        ut = a.ut_base + blk * uts + u;
+    };
+    const int p0 = warp * (NV * 256) + lane * 8;  // position of the lane's first eight; step q adds 256 q
+    auto request = [&](int item, int stage) {
+        if (item < items) {
+            int ut, u, blk;
+            int64_t e0;
+            locate(item, ut, u, blk, e0);
+            const int h = u / a.tensors, is_v = u % a.tensors;
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const int64_t e = e0 + p0 + 256 * q;
+                if (e >= n_e) continue;
+                const int64_t off = (e >> dshift) * a.stride_t + (int64_t)h * a.stride_h + ((int)e & (a.d - 1));
+#pragma unroll
+                for (int l = 0; l < B; ++l) {
+                    const T* src = reinterpret_cast<const T*>(is_v ? a.v[B * blk + l] : a.k[B * blk + l]) + off;
+                    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem + stage * STAGE + l * ROW + (p0 + 256 * q) * sizeof(T));
+#pragma unroll
+                    for (int k = 0; k < Q; ++k)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * k), "l"(reinterpret_cast<const uint4*>(src) + k) : "memory");
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    request(blockIdx.x, 0);
+    request(blockIdx.x + gridDim.x, 1);
+    for (int item = blockIdx.x, it = 0; item < items; item += gridDim.x, ++it) {
+        int ut, u, blk;
+        int64_t e0;
+        locate(item, ut, u, blk, e0);
+        const bool work = !redo || a.sel[ut].redo;  // (block-uniform)
+        const uint32_t lo = a.sel[ut].lo;
+        const bool is_k = u % a.tensors == 0;
+        uint8_t* const st = smem + (it & 1) * STAGE;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        if (work) {
+            T* const z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride + e0;
+            T* const z1 = a.z1 && is_k ? reinterpret_cast<T*>(a.z1) + (int64_t)(ut / a.tensors) * NB * a.unit_stride + e0 : nullptr;
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const int p = p0 + 256 * q;
+                uint32_t m8 = 0;
+                if (e0 + p < n_e) {
+                    uint4 x[B][Q], z[Q], hf[NB][Q];
+#pragma unroll
+                    for (int l = 0; l < B; ++l)
+#pragma unroll
+                        for (int k = 0; k < Q; ++k) x[l][k] = reinterpret_cast<const uint4*>(st + l * ROW + p * sizeof(T))[k];
+                    Eight<T, B>::split(x, z, hf, [&](int i, uint32_t key) { m8 |= (uint32_t)(key >= lo) << i; });
+                    if (lo == kNoKey) m8 = 0;
+#pragma unroll
+                    for (int k = 0; k < Q; ++k) {
+                        if (!redo) reinterpret_cast<uint4*>(z0 + p)[k] = z[k];
+#pragma unroll
+                        for (int l = 0; l < NB; ++l) {
+                            if (z1 && !redo) reinterpret_cast<uint4*>(z1 + (int64_t)l * a.unit_stride + p)[k] = hf[l][k];
+                            reinterpret_cast<uint4*>(st + l * ROW + p * sizeof(T))[k] = hf[l][k];
+                        }
+                    }
+                }
+                reinterpret_cast<uint8_t*>(s_map[warp])[32 * q + lane] = (uint8_t)m8;
+            }
+            __syncwarp();
+            uint32_t mine = lane < WW ? (uint32_t)__popc(s_map[warp][lane]) : 0u;
+            uint32_t incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane < WW) s_pre[warp][lane] = incl - mine;
+            const uint32_t n_w = __shfl_sync(0xFFFFFFFFu, incl, 31);
+            if (lane == 0) s_cnt[it & 1][warp] = n_w;
+            __syncthreads();
+            uint32_t base = 0, n = 0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                const uint32_t y = s_cnt[it & 1][w];
+                if (w < warp) base += y;
+                n += y;
+            }
+            if (tid == 0) a.cand_n[(int64_t)ut * a.chunks_max + (int)(e0 / CE)] = (int32_t)n;
+            uint16_t* const pos = a.cand_pos + (int64_t)ut * a.cand_stride + e0 + base;
+            T* const val = reinterpret_cast<T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0 + base;
+            for (uint32_t r = lane; r < n_w; r += 32) {
+                // the last word whose prefix does not exceed r holds entry r (empty words share their successor's prefix)
+                int w = 0;
+#pragma unroll
+                for (int s = WW / 2; s; s >>= 1)
+                    if (s_pre[warp][w + s] <= r) w += s;
+                const int p = warp * (NV * 256) + w * 32 + kth_set_bit(s_map[warp][w], r - s_pre[warp][w]);
+                pos[r] = (uint16_t)p;
+#pragma unroll
+                for (int l = 0; l < NB; ++l) val[(int64_t)l * a.cand_stride + r] = reinterpret_cast<const T*>(st + l * ROW)[p];
+            }
+            __syncwarp();  // (the warp's part of the stage is read)
+        }
+        request(item + 2 * gridDim.x, it & 1);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// ---- 3: the threshold ---------------------------------------------------------------------------------
+// f(key) for every candidate of chunk c; eight candidates per lane and load, STEPS of them requested together
+template <typename T, int B, typename F>
+__device__ __forceinline__ void each_candidate(const CompressArgs& a, int ut, int c, int n, F&& f) {
+    constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
+    constexpr int CE = compress_chunk(B, (int)sizeof(T));
+    constexpr int STEPS = NB * Q == 1 ? 3 : NB * Q == 2 ? 2 : 1;
+    const int lane = threadIdx.x & 31;
+    const T* const val = reinterpret_cast<const T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + (int64_t)c * CE;
+    for (int i0 = lane * 8; i0 < n; i0 += 256 * STEPS) {
+        uint4 v[STEPS][NB][Q];
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s)
+            if (i0 + 256 * s < n)
+#pragma unroll
+                for (int l = 0; l < NB; ++l)
+#pragma unroll
+                    for (int k = 0; k < Q; ++k) v[s][l][k] = reinterpret_cast<const uint4*>(val + (int64_t)l * a.cand_stride + i0 + 256 * s)[k];
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (i0 + 256 * s + j >= n) break;
+                float w[NB];
+#pragma unroll
+                for (int l = 0; l < NB; ++l) w[l] = to_f32(reinterpret_cast<const T*>(&v[s][l][0])[j]);
+                f(key_of<B>(w));
+            }
+    }
+}
+
+// One block per unit-tensor (grid ut_count).  First digit: the key's top 15 bits, in a window of 4 095 bins from the bound up
+// (32 octaves; the last bin counts what is larger, and in the unheard-of case that the k-th key is there the window moves
+// up): with 128 bins per octave the atomics hardly collide, and 16 KiB leave room for two blocks on an SM.  32-bit keys:
+// two more digits of 12 and 4 bits among the few keys that share the first.
+template <typename T, int B>
+__global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, int ut_begin, int redo) {
+    __shared__ uint32_t s_hist[kThrBins], s_sum[2][32];
+    constexpr bool F32KEY = !(sizeof(T) == 2 && B == 2);  // a bf16 magnitude is 15 bits
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int ut = ut_begin + blockIdx.x, chunks = a.chunks;
+    SelState* const sel = a.sel + ut;
+    chain_wait();
+    if (redo && !sel->redo) return;
+    const int32_t* const cn = a.cand_n + (int64_t)ut * a.chunks_max;
+    auto all_candidates = [&](auto&& f) {
+        int n = warp < chunks ? cn[warp] : 0;
+        for (int c = warp; c < chunks; c += 32) {
+            const int n_next = c + 32 < chunks ? cn[c + 32] : 0;
+            each_candidate<T, B>(a, ut, c, n, f);
+            n = n_next;
+        }
+    };
+    uint32_t tau = kNoKey, need = 0;
+    if (a.n_keep > 0) {
+        // are there k candidates?
+        uint32_t mine = 0;
+        for (int c = tid; c < chunks; c += kThrThreads) mine += (uint32_t)cn[c];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
+        if (lane == 0) s_sum[0][warp] = mine;
+        __syncthreads();
+        uint32_t total = 0;
+#pragma unroll
+        for (int w = 0; w < 32; ++w) total += s_sum[0][w];
+        if ((int64_t)total < a.n_keep) {
+            if (tid == 0) { sel->redo = 1; sel->lo = 0; }
+            return;
+        }
+        uint32_t k_rem = (uint32_t)a.n_keep, prefix, above;
+        for (uint32_t from = sel->lo >> 16;; from += kThrBins - 1) {
+            for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
+            __syncthreads();
+            all_candidates([&](uint32_t key) {
+                const uint32_t k16 = key >> 16;
+                if (k16 >= from) atomicAdd(&s_hist[min(k16 - from, (uint32_t)kThrBins - 1)], 1u);
+            });
+            __syncthreads();
+            uint32_t bin;
+            find_bin<kThrThreads, kThrBins>(s_hist, k_rem, bin, above);
+            prefix = from + bin;
+            if (bin < kThrBins - 1 || from + kThrBins - 1 >= 32767) break;
+        }
+        k_rem -= above;
+        if constexpr (F32KEY) {
+            const uint32_t top = prefix;
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                const int shift = pass == 0 ? 4 : 0, bits = pass == 0 ? 12 : 4;
+                for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
+                __syncthreads();
+                const uint32_t want = pass == 0 ? top : prefix;
+                all_candidates([&](uint32_t key) {
+                    if ((key >> (shift + bits)) == want) atomicAdd(&s_hist[(key >> shift) & ((1u << bits) - 1u)], 1u);
+                });
+                __syncthreads();
+                uint32_t bin;
+                find_bin<kThrThreads, kThrBins>(s_hist, k_rem, bin, above);
+                prefix = (want << bits) | bin;
+                k_rem -= above;
+            }
+        }
+        tau = F32KEY ? prefix : prefix << 16;
+        need = k_rem;
+    }
+    if (tid == 0) { sel->tau = tau; sel->need = need; }
+    // ---- keys above and equal to the threshold before every chunk ----
+    int2* const base = a.chunk_base + (int64_t)ut * a.chunks_max;
+    {
+        int n = warp < chunks ? cn[warp] : 0;
+        for (int c = warp; c < chunks; c += 32) {
+            const int n_next = c + 32 < chunks ? cn[c + 32] : 0;
+            uint32_t both = 0;  // above in the low half, equal in the high half (a lane meets at most 2^13 candidates of a chunk)
+            if (a.n_keep > 0) each_candidate<T, B>(a, ut, c, n, [&](uint32_t key) { both += key > tau ? 1u : key == tau ? 0x10000u : 0u; });
+            // (sums of 32 lanes stay below 2^16: a chunk has at most 2^13 positions)
+#pragma unroll
+            for (int o = 16; o; o >>= 1) both += __shfl_xor_sync(0xFFFFFFFFu, both, o);
+            if (lane == 0) base[c] = make_int2((int)(both & 0xFFFFu), (int)(both >> 16));
+            n = n_next;
+        }
+    }
+    __syncthreads();
+    uint32_t run_gt = 0, run_eq = 0;
+    for (int c0 = 0; c0 < chunks; c0 += kThrThreads) {
+        const int c = c0 + tid;
+        const int2 m = c < chunks ? base[c] : make_int2(0, 0);
+        uint32_t ig = (uint32_t)m.x, ie = (uint32_t)m.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t yg = __shfl_up_sync(0xFFFFFFFFu, ig, o), ye = __shfl_up_sync(0xFFFFFFFFu, ie, o);
+            if (lane >= o) { ig += yg; ie += ye; }
+        }
+        __syncthreads();
+        if (lane == 31) { s_sum[0][warp] = ig; s_sum[1][warp] = ie; }
+        __syncthreads();
+        uint32_t tg = 0, te = 0, bg = run_gt, be = run_eq;
+#pragma unroll
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) { bg += s_sum[0][w]; be += s_sum[1][w]; }
+            tg += s_sum[0][w];
+            te += s_sum[1][w];
+        }
+        if (c < chunks) base[c] = make_int2((int)(bg + ig) - m.x, (int)(be + ie) - m.y);
+        run_gt += tg;
+        run_eq += te;
+    }
+}
+
+// ---- 4: the lists -------------------------------------------------------------------------------------
+// Packed entry of the bf16 / head_dim 128 decode kernel: low half = value bits, high half = (byte offset / 2) of the position
+// inside a 16-token x 128-channel tile of two 64-channel halves with 128-byte rows whose 16-byte chunks are XOR-swizzled
+// with the row.
+__device__ __forceinline__ uint32_t packed_entry(float v, int flat) {
+    const int row = (flat >> 7) & 15, ch = flat & 127;
+    const uint32_t off = (uint32_t)((ch >> 6) * 2048 + row * 128 + ((((ch >> 3) & 7) ^ (row & 7)) << 4) + (ch & 7) * 2);
+    return (__float_as_uint(v) >> 16) | ((off >> 1) << 16);
+}
+
+// grid (groups of eight chunks, unit-tensors), a chunk per warp: no block barriers, U rounds of candidates requested together
+// (one chunk per block with a block scan per round took 767 us for 32 layers of 32k tokens)
+template <typename T, int B>
+__global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_begin) {
+    constexpr int NB = B == 4 ? 4 : 1, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
+    constexpr int U = 4;
+    __shared__ uint32_t s_map[8][WORDS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ut = ut_begin + blockIdx.y, c = blockIdx.x * 8 + warp;
+    chain_wait();
+    if (c >= a.chunks) return;
+    uint32_t* const map = s_map[warp];
+    for (int w = lane; w < WORDS; w += 32) map[w] = 0;
+    const uint32_t tau = a.sel[ut].tau, need = a.sel[ut].need;
+    const int n = a.cand_n[(int64_t)ut * a.chunks_max + c];
+    const int2 b0 = a.chunk_base[(int64_t)ut * a.chunks_max + c];
+    const int64_t e0 = (int64_t)c * CE, n_e = (int64_t)a.T * a.d;
+    const uint16_t* const pos = a.cand_pos + (int64_t)ut * a.cand_stride + e0;
+    const T* const val = reinterpret_cast<const T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0;
+    uint32_t run_gt = (uint32_t)b0.x, run_eq = (uint32_t)b0.y;
+    const uint32_t first = run_gt + min(run_eq, need);  // list position of the chunk's first entry
+    const uint32_t below = (1u << lane) - 1u;
+    __syncwarp();
+    for (int i0 = lane; i0 < n + lane; i0 += 32 * U) {
+        uint32_t p[U];
+        T raw[U][NB];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int i = i0 + 32 * q;
+            p[q] = 0;
+            if (i < n) {
+                p[q] = pos[i];
+#pragma unroll
+                for (int l = 0; l < NB; ++l) raw[q][l] = val[(int64_t)l * a.cand_stride + i];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const bool on = i0 + 32 * q < n;
+            float v[NB];
+#pragma unroll
+            for (int l = 0; l < NB; ++l) v[l] = on ? to_f32(raw[q][l]) : 0.f;
+            const uint32_t key = key_of<B>(v);
+            const bool gt = on && key > tau, eq = on && key == tau;
+            const uint32_t mg = __ballot_sync(0xFFFFFFFFu, gt), me = __ballot_sync(0xFFFFFFFFu, eq);
+            const uint32_t be = run_eq + __popc(me & below);
+            if (gt || (eq && be < need)) {  // ties in index order while fewer than `need` precede them
+                const int64_t at = run_gt + __popc(mg & below) + min(be, need);
+                const int flat = (int)e0 + (int)p[q];
+                a.idx[(int64_t)ut * a.kcap + at] = flat;
+#pragma unroll
+                for (int l = 0; l < NB; ++l) {
+                    const int64_t o = ((int64_t)ut * NB + l) * a.kcap + at;
+                    reinterpret_cast<T*>(a.val)[o] = raw[q][l];
+                    // (a block of four scales its rows by 1/2 at decode time and its deviations by 1: twice the deviation is stored)
+                    if constexpr (sizeof(T) == 2)
+                        if (a.packed) a.packed[o] = packed_entry(B == 4 ? 2.f * v[l] : v[l], flat);
+                }
+                atomicOr(&map[p[q] >> 5], 1u << (p[q] & 31));
+            }
+            run_gt += __popc(mg);
+            run_eq += __popc(me);
+        }
+    }
+    __syncwarp();
+    // K: the bit map of the kept positions (whole chunks: the map is padded like the candidate lists)
+    if (a.keep && !(ut % a.tensors)) {
+        uint32_t* const keep = a.keep + (int64_t)(ut / a.tensors) * a.keep_stride + e0 / 32;
+        for (int w = lane; w < WORDS; w += 32) keep[w] = map[w];
+    }
+    // tile offsets
+    const int tile_e = kResTile * a.d, tile_words = tile_e / 32;
+    const int tiles = (int)((min((int64_t)CE, n_e - e0) + tile_e - 1) / tile_e);
+    int32_t* const off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1) + (int)(e0 / tile_e);
+    uint32_t at = first;
+    for (int j = 0; j < tiles; ++j) {
+        uint32_t s = 0;
+        for (int w = lane; w < tile_words; w += 32) s += __popc(map[j * tile_words + w]);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+        if (lane == 0) off[j] = (int32_t)at;
+        at += s;
+    }
+    if (lane == 0 && c == a.chunks - 1) {
+        off[tiles] = (int32_t)at;
+        if ((int64_t)at != a.n_keep) atomicMax(a.status, (int32_t)kFlagCountMismatch);
+    }
+}
+
+template <typename... A>
+cudaError_t launch_chain(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    count_launch(1);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename T, int B>
+cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* const* v_layers, int block_begin, int block_end, cudaStream_t st) {
+    static PerDevice once;
+    int sms = 0;
+    constexpr int CE = compress_chunk(B, (int)sizeof(T));
+    const size_t smem = 2 * (size_t)B * CE * sizeof(T);
+    cudaError_t e = once.ensure([&]() { return cudaFuncSetAttribute(split_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); }, &sms);
+    if (e != cudaSuccess) return e;
+    const int64_t n = (int64_t)a.T * a.d;
+    a.chunks = (int)((n + CE - 1) / CE);
+    const int uts = a.Hkv * a.tensors, ut_begin = block_begin * uts, ut_count = (block_end - block_begin) * uts;
+    // about 1.2 k candidates (and four standard deviations of a small sample on top); a sample of everything is exact
+    const int n_rows = (int)std::min<int64_t>(a.T, std::max<int64_t>(1, kSampleElems / a.d));
+    const bool exact = n_rows == a.T;
+    const double expect = (double)a.n_keep * n_rows / a.T;
+    const uint32_t target = exact ? (uint32_t)a.n_keep : (uint32_t)std::ceil(1.2 * expect + 4.0 * std::sqrt(expect) + 16.0);
+    // (items are counted in 32 bits)
+    const int per_launch = (int)std::max<int64_t>(1, std::min<int64_t>(kSplitLayers / B, 0x7FFFFFFF / ((int64_t)a.chunks * uts) / 4));
+    for (int redo = 0; redo < (exact || a.n_keep == 0 ? 1 : 2); ++redo) {
+        for (int b0 = block_begin; b0 < block_end; b0 += per_launch) {
+            const int nb = std::min(block_end - b0, per_launch);
+            for (int l = 0; l < nb * B; ++l) {
+                a.k[l] = k_layers[B * b0 + l];
+                a.v[l] = v_layers[B * b0 + l];
+            }
+            a.ut_base = b0 * uts;
+            if (!redo && (e = launch_chain(sample_kernel<T, B>, dim3(uts, nb), kSampleThreads, 0, st, a, n_rows, target)) != cudaSuccess) return e;
+            const int items = a.chunks * uts * nb;
+            if ((e = launch_chain(split_kernel<T, B>, dim3(std::min(items, 3 * sms)), kSplitThreads, smem, st, a, items, redo)) != cudaSuccess) return e;
+        }
+        if ((e = launch_chain(threshold_kernel<T, B>, dim3(ut_count), kThrThreads, 0, st, a, ut_begin, redo)) != cudaSuccess) return e;
+    }
+    return launch_chain(compact_kernel<T, B>, dim3((a.chunks + 7) / 8, ut_count), 256, 0, st, a, ut_begin);
+}
+
+}  // namespace
+
+cudaError_t launch_compress(CompressArgs& a, int B, int dtype, const void* const* k_layers, const void* const* v_layers, int block_begin, int block_end,
+                            cudaStream_t st) {
+    if (a.T <= 0 || block_end <= block_begin) return cudaSuccess;
+    if (dtype == FDKV_BF16)
+        return B == 4 ? compress<__nv_bfloat16, 4>(a, k_layers, v_layers, block_begin, block_end, st)
+                      : compress<__nv_bfloat16, 2>(a, k_layers, v_layers, block_begin, block_end, st);
+    return B == 4 ? compress<float, 4>(a, k_layers, v_layers, block_begin, block_end, st)
+                  : compress<float, 2>(a, k_layers, v_layers, block_begin, block_end, st);
+}
+
+}  // namespace fdkv

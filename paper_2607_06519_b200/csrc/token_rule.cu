@@ -157,8 +157,8 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
 
     if (warp == 0) {
         if (lane == 0) {
-            // K high-frequency rows of the unit: unit-tensor 2*unit (a block of four stages one operand per layer)
-            const int64_t row0 = a.B == 4 ? ((int64_t)unit * 2 * 4 + layer) * a.Tmax : (int64_t)unit * 2 * a.Tmax;
+            // K high-frequency rows of the unit (a block of four stages one operand per layer)
+            const int64_t row0 = a.B == 4 ? ((int64_t)unit * 4 + layer) * a.Tmax : (int64_t)unit * a.Tmax;
             for (int i = 0; i < ntile; ++i) {
                 const int s = i % kTStages;
                 mb_wait(sm0 + tEmpty + 8 * s, ((uint32_t)(i / kTStages) & 1u) ^ 1u, abort_flag, a.status);
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(256) token_score_tile_kernel(TokenArgs a, int 
     const int M = (a.B == 4 ? 1 : 2) * a.G * a.W;  // probe rows per operand
     float best = 0.f, esum = 0.f;
     for (int op = 0; op < n_ops; ++op) {
-        const T* z1 = reinterpret_cast<const T*>(a.z1) + ((int64_t)unit * 2 * n_ops + op) * a.unit_stride + (int64_t)t0 * d;
+        const T* z1 = reinterpret_cast<const T*>(a.z1) + ((int64_t)unit * n_ops + op) * a.unit_stride + (int64_t)t0 * d;
         for (int i = threadIdx.x; i < kSTile * d; i += blockDim.x) {
             const int t = i / d, c = i % d;
             zs[t * ld + c] = t < nt ? to_f32<T>(z1[i]) : 0.f;
