@@ -54,9 +54,10 @@ bool make_shape(const fdkv_config& c, Shape& s) {
     s.kcap = (int64_t)align_up((size_t)(s.kmax + kListPad), 64);
     s.ntiles_max = (s.Tmax + kResTile - 1) / kResTile;
     // per-unit partial-sum slots of the probe: one per 64-token tile (portable kernel) or one per work item of the
-    // tensor-core kernel (layers x 128-row blocks x key splits of at least 8 tiles), whichever is more
+    // tensor-core kernel (layers x 128-row blocks x key splits of at least 8 tiles) and the blocks of the second-moment
+    // kernel that share a unit, whichever is more
     s.nptiles_max = std::max((s.Tmax + kProbeTile - 1) / kProbeTile,
-                             B * ((G * kMaxW + 127) / 128) * (((s.Tmax - 1) / kProbeBoxRows + 1 + 7) / 8));
+                             B * ((G * kMaxW + 127) / 128) * (((s.Tmax - 1) / kProbeBoxRows + 1 + 7) / 8) + kMaxGramCtas + 2 * 4);
     s.tail_rows = (s.max_tail + kRowPad - 1) / kRowPad * kRowPad;
     if (c.residual_rule != FDKV_RESIDUAL_ENTRIES && c.residual_rule != FDKV_RESIDUAL_TOKENS) return false;
     s.tok_rule = c.residual_rule == FDKV_RESIDUAL_TOKENS;
@@ -281,7 +282,8 @@ fdkv_status fdkv_create(const fdkv_config* cfg, void* arena, size_t arena_bytes,
         c->tok_tc = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, 128, c->tmap_z1_128);
     if (s.tok_rule && s.dtype == FDKV_BF16 && s.d == 128 && !c->tok_tc) { delete c; return FDKV_ERR_UNSUPPORTED; }
     if (s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule)
-        c->has_probe_tmaps = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_z1) &&
+        c->has_probe_tmaps = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, 128, c->tmap_z1_128) &&
+                             make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_z1) &&
                              make_rows_tensor_map(c->work + c->ws.z1drop, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_drop);
     *out = c;
     return FDKV_OK;
@@ -417,6 +419,7 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
     a.modes_out = modes; a.scores_out = scores;
     a.tmap_z1 = c->has_probe_tmaps ? c->tmap_z1 : nullptr;
     a.tmap_drop = c->has_probe_tmaps ? c->tmap_drop : nullptr;
+    a.tmap_z1_128 = c->tmap_z1_128;
     a.Tmax = s.Tmax;
     a.pos_host = probe_pos;
     a.status = wsp<int32_t>(c, c->ws.status);

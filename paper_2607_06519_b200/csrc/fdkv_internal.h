@@ -151,7 +151,7 @@ struct fdkv_ctx {
     bool has_tmap = false;
     alignas(64) unsigned char tmap_z1[128], tmap_drop[128];  // probe operands (bf16, head_dim 128 only)
     bool has_probe_tmaps = false;
-    alignas(64) unsigned char tmap_z1_128[128];  // staged Z1 with 128-token boxes (token-score kernel)
+    alignas(64) unsigned char tmap_z1_128[128];  // staged Z1 with 128-token boxes (token-score and second-moment kernels)
     bool tok_tc = false;                         // token rule served by the tensor-core kernels (bf16, head_dim 128)
     std::vector<uint8_t> pair_scored;            // token rule: the probe has chosen this pair's token sets
     bool packed_lists = false;              // decode runs the bf16 / head_dim 128 kernel on packed residual entries
@@ -235,11 +235,14 @@ struct ProbeArgs {
     // tensor-core path (bf16, head_dim 128): tensor maps over the staged Z1 and the dropped copy, viewed as
     // [rows][128] bf16 with 128-token x 64-channel boxes; null when unavailable
     const void *tmap_z1, *tmap_drop;
+    const void* tmap_z1_128;  // the staged Z1 with 128-token boxes
     int Tmax;
     const int32_t* pos_host;
     int32_t* status;
 };
 cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st);
+constexpr int kMaxGramCtas = 160;  // blocks of the second-moment kernel, and so part slots a unit may need
+cudaError_t launch_probe_gram(const ProbeArgs& a, int t_full, cudaStream_t st, int* nparts);
 
 struct DecodeArgs {
     const UnitDesc* desc;  // [batch][.. layer ..] : desc + (b*L + layer)*Hkv + h

@@ -20,12 +20,10 @@
 //     item, summed across items in a fixed order by the finalize kernel.
 // Every mbarrier wait is bounded; on expiry the CTA flags the device status word, stops waiting and still frees
 // its tensor memory before it retires.
-#include <cuda.h>
-
 #include <algorithm>
 
 #include "fdkv_internal.h"
-#include "mbar_wait.cuh"
+#include "umma.cuh"
 
 namespace fdkv {
 
@@ -47,66 +45,16 @@ constexpr int kTmemCols = 512;
 constexpr int kAccSet = kMT * kBN;
 static_assert(kAccSets * kAccSet <= kTmemCols && (kBN == 128 || kBN == 256), "tensor memory budget");
 // header: full[8] @0, empty[8] @64, tfull[2] @128, tempty[2] @144, tmem slot @160, abort @164, reduce @192 (4 doubles)
+constexpr uint32_t kIdesc = umma_idesc(128, kBN, false);
 constexpr int oFull = 0, oEmpty = 64, oTFull = 128, oTEmpty = 144, oSlot = 160, oAbort = 164, oRed = 192;
 
-__device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mb_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mb_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mb_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mb_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, int32_t* status) {
-    mbar_wait_bounded(bar, parity, abort_flag, status);
-}
-__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(map), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-// shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);          // start address
-    d |= (uint64_t)1 << 16;                            // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;                  // stride byte offset
-    d |= (uint64_t)1 << 46;                            // descriptor version
-    d |= (uint64_t)2 << 61;                            // 128-byte swizzle
-    return d;
-}
-// instruction descriptor: D = f32, A = B = bf16, both K-major, M = 128, N = kBN
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-
-// D[tmem] (+)= A[smem] * B[smem]^T; ACC = 0 overwrites D
-template <int ACC>
-__device__ __forceinline__ void umma_ss(uint32_t tmem_d, uint64_t da, uint64_t db) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(kIdesc), "n"(ACC)
-        : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-          "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
 
 struct TcPlan {
     int items_per_unit;  // B layers x mblocks x 2 candidates x nsplits
     int mblocks, nsplits, ntiles, tiles_per_split;
     int pos_min, pos_max;
+    int tile_first;   // first 256-key tile (the keys before it are probe_gram_kernel's)
+    int slot0;        // first part slot
 };
 
 __global__ void __launch_bounds__(kPThreads, 1)
@@ -128,7 +76,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
     const int mblock = it % pl.mblocks; it /= pl.mblocks;
     const int layer = it;  // layer inside the depth block: 0 .. B-1
     const int h = unit % a.Hkv, pair = unit / a.Hkv;
-    const int tile0 = split * pl.tiles_per_split;
+    const int tile0 = pl.tile_first + split * pl.tiles_per_split;
     const int tile1 = min(pl.ntiles, tile0 + pl.tiles_per_split);
     const int ntile = max(0, tile1 - tile0);
     const int rows_layer = a.G * a.W;
@@ -203,8 +151,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
                     for (int mt = 0; mt < kMT; ++mt) {  // the M tiles alternate: consecutive MMAs never wait for each other's accumulator
                         const uint64_t db = db_stage + (uint64_t)(((k >> 2) * kBHalf + (k & 3) * 32) >> 4);
                         const uint64_t da = da_all + (uint64_t)((mt * 2 * kAHalf + (k >> 2) * kAHalf + (k & 3) * 32) >> 4);
-                        if (k == 0) umma_ss<0>(d0 + mt * kBN, da, db);
-                        else umma_ss<1>(d0 + mt * kBN, da, db);
+                        umma_ss<kIdesc>(d0 + mt * kBN, da, db, k > 0);
                     }
                 }
                 umma_commit(sm0 + oEmpty + 8 * s);    // the B stage is free once these MMAs have read it
@@ -283,7 +230,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
     if (threadIdx.x == 0) {
         const double* red = reinterpret_cast<const double*>(smem + oRed);
         // part slot of this item inside its unit: (layer, mblock, split); candidate selects the column
-        const int slot = (layer * pl.mblocks + mblock) * pl.nsplits + split;
+        const int slot = pl.slot0 + (layer * pl.mblocks + mblock) * pl.nsplits + split;
         a.part[((int64_t)unit * a.nptiles_max + slot) * 2 + cand] = red[0] + red[1] + red[2] + red[3];
     }
 }
@@ -297,13 +244,7 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(ProbeArgs a, int n_ops, 
     uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.z1drop) + op);
     const uint8_t* bits = reinterpret_cast<const uint8_t*>(a.keep + (int64_t)unit * a.keep_stride);
     for (int64_t v = (int64_t)t0 * 16 + (int64_t)blockIdx.x * 256 + threadIdx.x; v < (int64_t)t1 * 16; v += (int64_t)gridDim.x * 256) {
-        uint4 x = src[v];
-        const uint32_t b = bits[v], m = b | (b << 15);  // bit j: element j is kept; word w's are bits 2w and 16 + 2w of m
-        x.x &= ~((m & 0x00010001u) * 0xFFFFu);
-        x.y &= ~(((m >> 2) & 0x00010001u) * 0xFFFFu);
-        x.z &= ~(((m >> 4) & 0x00010001u) * 0xFFFFu);
-        x.w &= ~(((m >> 6) & 0x00010001u) * 0xFFFFu);
-        dst[v] = x;
+        dst[v] = drop_kept(src[v], bits[v]);
     }
 }
 
@@ -320,26 +261,36 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     pl.pos_min = a.pos_host[0];
     pl.pos_max = a.pos_host[a.W - 1];
     pl.ntiles = pl.pos_max / kBN + 1;  // keys after the last probe position never count
+    // keys that every probe query sees: second moments (one read of Z1 and 2 x 2 x 128 x 128 flops per key, against a second
+    // copy of Z1 and 2 x 2 x rows x 128 flops here; 32 layers of 32k tokens, 512 rows per pair: 1 190 -> 320 us with this
+    // kernel's share of the last keys)
+    pl.tile_first = (pl.pos_min + 1) / kBN;
+    pl.slot0 = 0;
+    if (pl.tile_first > 0) {
+        cudaError_t e = launch_probe_gram(a, pl.tile_first * kBN, st, &pl.slot0);
+        if (e != cudaSuccess) return e;
+    }
+    const int ntiles = pl.ntiles - pl.tile_first;
     pl.mblocks = (a.G * a.W + 128 * kMT - 1) / (128 * kMT);
     const int base_items = a.unit_count * a.B * pl.mblocks * 2;
     // split the key range so that the grid fills the machine several times over, but keep >= 8 tiles per item
-    int nsplits = std::max(1, std::min((4 * sm_count + base_items - 1) / base_items, (pl.ntiles + 7) / 8));
-    pl.tiles_per_split = (pl.ntiles + nsplits - 1) / nsplits;
-    nsplits = (pl.ntiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
+    int nsplits = std::max(1, std::min((4 * sm_count + base_items - 1) / base_items, (ntiles + 7) / 8));
+    pl.tiles_per_split = (ntiles + nsplits - 1) / std::max(1, nsplits);
+    nsplits = ntiles > 0 ? (ntiles + pl.tiles_per_split - 1) / pl.tiles_per_split : 0;
     pl.nsplits = nsplits;
     pl.items_per_unit = a.B * pl.mblocks * 2 * nsplits;
-    const int slots = a.B * pl.mblocks * nsplits;
+    const int slots = pl.slot0 + a.B * pl.mblocks * nsplits;
     if (slots > a.nptiles_max) return cudaErrorInvalidValue;  // cannot happen: the part array is sized for max_probe_parts()
-    {
-        const int t1 = std::min(a.T, pl.ntiles * kBN), n_ops = a.B == 4 ? 4 : 1;
-        drop_rows_kernel<<<dim3((unsigned)std::min<int64_t>(64, ((int64_t)t1 * 16 + 255) / 256), a.unit_count, n_ops), 256, 0, st>>>(a, n_ops, 0, t1);
-        count_launch(1);
+    if (nsplits > 0) {
+        const int t0 = pl.tile_first * kBN, t1 = std::min(a.T, pl.ntiles * kBN), n_ops = a.B == 4 ? 4 : 1;
+        const int blocks = (int)std::min<int64_t>(64, ((int64_t)(t1 - t0) * 16 + 255) / 256);
+        drop_rows_kernel<<<dim3(blocks, a.unit_count, n_ops), 256, 0, st>>>(a, n_ops, t0, t1);
+        probe_tc_kernel<<<a.unit_count * pl.items_per_unit, kPThreads, kProbeSmem, st>>>(
+            *reinterpret_cast<const CUtensorMap*>(a.tmap_z1), *reinterpret_cast<const CUtensorMap*>(a.tmap_drop), a, pl);
+        count_launch(2);
     }
-    probe_tc_kernel<<<a.unit_count * pl.items_per_unit, kPThreads, kProbeSmem, st>>>(
-        *reinterpret_cast<const CUtensorMap*>(a.tmap_z1), *reinterpret_cast<const CUtensorMap*>(a.tmap_drop), a, pl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    count_launch(1);
     count_kernel(FDKV_KERNEL_PROBE_TC);
     *nparts = slots;
     *handled = true;

@@ -19,13 +19,11 @@
 // 2. token_select_kernel: per unit an MSB-first radix select (4 x 8 bits) of the k_tok-th largest score and an
 //    index-ordered compaction: ascending token list, per-16-token-slice counts, and the two error sums in float64.
 // (The commit step forms the selected rows from the caller's K and V: token_gather_kernel in compress.cu.)
-#include <cuda.h>
-
 #include <algorithm>
 #include <cstdlib>
 
 #include "fdkv_internal.h"
-#include "mbar_wait.cuh"
+#include "umma.cuh"
 
 namespace fdkv {
 
@@ -41,60 +39,9 @@ constexpr int kTBBytes = 2 * kTBHalf;       // 64 KiB
 constexpr int kTHdr = 2048;                 // barriers, TMEM slot, abort flag, probe position of every column
 constexpr int kTSmem = kTHdr + kTBBytes + kTStages * kTAStage;  // 194 KiB
 constexpr int kTThreads = 6 * 32;
+constexpr uint32_t kTIdesc = umma_idesc(kTM, kTN, false);
 constexpr int tFull = 0, tEmpty = 32, tTFull = 64, tTEmpty = 80, tSlot = 96, tAbort = 100, tPosCol = 1024;  // pos_col: 256 ints
 
-__device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mb_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mb_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mb_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mb_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, int32_t* status) {
-    mbar_wait_bounded(bar, parity, abort_flag, status);
-}
-__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(map), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-// shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-// instruction descriptor: D = f32, A = B = bf16, both K-major, M = 128, N = 256
-constexpr uint32_t kTIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTN >> 3) << 17) | ((uint32_t)(kTM >> 4) << 24);
-
-template <int ACC>
-__device__ __forceinline__ void umma_ss(uint32_t tmem_d, uint64_t da, uint64_t db) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(kTIdesc), "n"(ACC)
-        : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-          "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
 
 struct ScorePlan {
     int items_per_unit, mblocks, nsplits, ntiles, tiles_per_split, pos_min;
@@ -185,8 +132,7 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
                 for (int k = 0; k < 8; ++k) {
                     const uint64_t da = da0 + (uint64_t)(((k >> 2) * kTAHalf + (k & 3) * 32) >> 4);
                     const uint64_t db = db0 + (uint64_t)(((k >> 2) * kTBHalf + (k & 3) * 32) >> 4);
-                    if (k == 0) umma_ss<0>(d_tmem, da, db);
-                    else umma_ss<1>(d_tmem, da, db);
+                    umma_ss<kTIdesc>(d_tmem, da, db, k > 0);
                 }
                 umma_commit(sm0 + tEmpty + 8 * s);
                 umma_commit(sm0 + tTFull + 8 * as);

@@ -1,0 +1,38 @@
+"""Probe errors by second moments (keys every probe query sees) and by products (the keys after): both block sizes, lengths
+and probe positions around the 128- and 256-key tiles, more and fewer probe rows than a 128-row tile, units shared by
+several thread blocks and thread blocks that share units."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import fdkv_ref as R
+from oracle import fdkv_ref_b4 as R4
+from paper_2607_06519_b200 import runner, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("block", [2, 4])
+@pytest.mark.parametrize("hkv,group,T,pos", [
+    (1, 1, 257, [254]), (1, 1, 257, [255]), (1, 2, 300, [256, 299]), (2, 4, 1000, range(990, 1000)), (1, 1, 20000, [19999]),
+    (3, 4, 700, range(600, 700)), (8, 4, 2049, range(1985, 2049)), (2, 8, 5000, [10, 3000, 4999]), (2, 1, 1100, [511, 512, 1023, 1024]),
+])
+def test_probe_errors(block, hkv, group, T, pos):
+    pos = np.array(list(pos), dtype=np.int32)
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2 * block, n_kv_heads=hkv, n_q_heads=hkv * group, T=T, W=len(pos), n_needles=4, keep_den=7,
+                                            block_size=block, name="moments")
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    _, scores = pf.ctx.probe(0, 0, w.n_blocks, pf.upload_probe_q(0), pos, 0.0)
+    scores = scores.cpu().numpy()
+    for p in range(w.n_blocks):
+        pq = [synth.probe_q(w, 0, block * p + l) for l in range(block)]
+        for h in sorted({0, hkv - 1}):
+            if block == 4:
+                u = R4.Unit4(synth.block_tensor(w, 0, p, h, False), synth.block_tensor(w, 0, p, h, True), True, w.keep_num, w.keep_den)
+                want = R4.probe_error4(u.dev["k"], u.kept["k"], pq, group, h, pos)
+            else:
+                u = R.Unit(*synth.unit_tensor(w, 0, p, h, False), *synth.unit_tensor(w, 0, p, h, True), True, w.keep_num, w.keep_den)
+                want = R.probe_error(u.z1["k"], u.kept["k"], pq[0], pq[1], group, h, pos)
+            np.testing.assert_allclose(scores[p, h], want, rtol=2e-5)
+    assert pf.ctx.device_status() == 0
