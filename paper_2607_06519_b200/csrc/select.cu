@@ -47,7 +47,11 @@ __device__ __forceinline__ f32x2 pack2(uint32_t lo, uint32_t hi) {
 __device__ __forceinline__ f32x2 bf2(uint32_t w) { return pack2(w << 16, w & 0xFFFF0000u); }  // two bf16 values, widened
 __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return add2(a, b ^ 0x8000000080000000ull); }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {  // a + (-1) b, rounded once: the difference
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(pack2(0xBF800000u, 0xBF800000u)), "l"(a));
+    return r;
+}
 __device__ __forceinline__ uint32_t to_bf2(f32x2 a) {  // both halves to nearest-even bf16
     uint32_t lo, hi, r;
     asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(a));
@@ -67,74 +71,106 @@ __device__ __forceinline__ uint32_t key_of(const float* v) {
                                          __fadd_rn(__fmul_rn(v[2], v[2]), __fmul_rn(v[3], v[3])))) & 0x7FFFFFFFu;
 }
 
-// Eight consecutive positions as 16-byte vectors, Q of them per row: x[layer] -> shared coefficients z0 and high-frequency
-// values hf[1 or 4], and for_key(position, key) for each.
+// bits of four words' eight 16-bit halves whose sums g carry into bit 15 / 31, in order
+__device__ __forceinline__ uint32_t pair_mask8(uint32_t g0, uint32_t g1, uint32_t g2, uint32_t g3) {
+    uint32_t t = (g0 >> 15) & 0x00010001u;  // word j -> bits 2j and 16 + 2j
+    t |= (g1 >> 13) & 0x00040004u;
+    t |= (g2 >> 11) & 0x00100010u;
+    t |= (g3 >> 9) & 0x00400040u;
+    return (t | (t >> 15)) & 0xFFu;
+}
+
+// Eight consecutive positions as 16-byte vectors, Q of them per row.  split: x[layer] -> shared coefficients z0 and
+// high-frequency values hf[1 or 4]; keys: f(position, key) for each; reach: bit i = position i's key is at least lo.
 template <typename T, int B>
-struct Eight;
-template <int B>
-struct Eight<__nv_bfloat16, B> {
-    static constexpr int Q = 1;
-    template <typename F>
-    __device__ static void split(const uint4 (&x)[B][1], uint4 (&z0)[1], uint4 (&hf)[B == 4 ? 4 : 1][1], F&& for_key) {
-        const f32x2 c = pack2(0x3F3504F3u, 0x3F3504F3u), half1 = pack2(0x3F000000u, 0x3F000000u);  // the float32 nearest 1/sqrt 2; 1/2
-        const uint32_t* const xw[B == 4 ? 4 : 2] = {reinterpret_cast<const uint32_t*>(&x[0][0]), reinterpret_cast<const uint32_t*>(&x[1][0])};
-        uint32_t* const zw = reinterpret_cast<uint32_t*>(&z0[0]);
+struct Eight {
+    static constexpr int Q = (int)sizeof(T) / 2, NB = B == 4 ? 4 : 1;
+    __device__ static void split(const uint4 (&x)[B][Q], uint4 (&z0)[Q], uint4 (&hf)[NB][Q]) {
+        if constexpr (sizeof(T) == 2) {
+            const f32x2 c = pack2(0x3F3504F3u, 0x3F3504F3u), half1 = pack2(0x3F000000u, 0x3F000000u);  // the float32 nearest 1/sqrt 2; 1/2
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            if constexpr (B == 2) {
-                const f32x2 a = bf2(xw[0][w]), b = bf2(xw[1][w]);
-                zw[w] = to_bf2(mul2(add2(a, b), c));
-                const uint32_t h = to_bf2(mul2(sub2(a, b), c));
-                reinterpret_cast<uint32_t*>(&hf[0][0])[w] = h;
-                for_key(2 * w, (h << 16) & 0x7FFF0000u);
-                for_key(2 * w + 1, h & 0x7FFF0000u);
-            } else {
-                f32x2 v[4];
+            for (int w = 0; w < 4; ++w) {
+                f32x2 v[B];
 #pragma unroll
-                for (int l = 0; l < 4; ++l) v[l] = bf2(reinterpret_cast<const uint32_t*>(&x[l][0])[w]);
-                zw[w] = to_bf2(mul2(half1, add2(add2(v[0], v[1]), add2(v[2], v[3]))));
-                const f32x2 half = mul2(half1, bf2(zw[w]));  // exact
+                for (int l = 0; l < B; ++l) v[l] = bf2(word(x[l][0], w));
+                if constexpr (B == 2) {
+                    word(z0[0], w) = to_bf2(mul2(add2(v[0], v[1]), c));
+                    word(hf[0][0], w) = to_bf2(mul2(sub2(v[0], v[1]), c));
+                } else {
+                    const uint32_t z = to_bf2(mul2(half1, add2(add2(v[0], v[1]), add2(v[2], v[3]))));
+                    word(z0[0], w) = z;
+                    const f32x2 half = mul2(half1, bf2(z));  // exact
 #pragma unroll
-                for (int l = 0; l < 4; ++l) {
-                    const uint32_t h = to_bf2(sub2(v[l], half));
-                    reinterpret_cast<uint32_t*>(&hf[l][0])[w] = h;
-                    v[l] = bf2(h);
-                    v[l] = mul2(v[l], v[l]);
+                    for (int l = 0; l < 4; ++l) word(hf[l][0], w) = to_bf2(sub2(v[l], half));
                 }
-                const f32x2 e = add2(add2(v[0], v[1]), add2(v[2], v[3]));
-                for_key(2 * w, (uint32_t)e & 0x7FFFFFFFu);
-                for_key(2 * w + 1, (uint32_t)(e >> 32) & 0x7FFFFFFFu);
+            }
+        } else {
+            const float c32 = __uint_as_float(0x3F3504F3u);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float f[B];
+#pragma unroll
+                for (int l = 0; l < B; ++l) f[l] = __uint_as_float(word(x[l][i >> 2], i & 3));
+                if constexpr (B == 2) {
+                    word(z0[i >> 2], i & 3) = __float_as_uint(__fmul_rn(__fadd_rn(f[0], f[1]), c32));
+                    word(hf[0][i >> 2], i & 3) = __float_as_uint(__fmul_rn(__fsub_rn(f[0], f[1]), c32));
+                } else {
+                    const float z = __fmul_rn(0.5f, __fadd_rn(__fadd_rn(f[0], f[1]), __fadd_rn(f[2], f[3])));
+                    const float half = __fmul_rn(0.5f, z);  // exact
+                    word(z0[i >> 2], i & 3) = __float_as_uint(z);
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) word(hf[l][i >> 2], i & 3) = __float_as_uint(__fsub_rn(f[l], half));
+                }
             }
         }
     }
-};
-template <int B>
-struct Eight<float, B> {
-    static constexpr int Q = 2;
     template <typename F>
-    __device__ static void split(const uint4 (&x)[B][2], uint4 (&z0)[2], uint4 (&hf)[B == 4 ? 4 : 1][2], F&& for_key) {
-        const float c32 = __uint_as_float(0x3F3504F3u);
+    __device__ static void keys(const uint4 (&hf)[NB][Q], F&& f) {
+        if constexpr (sizeof(T) == 2) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float f[B], h[B == 4 ? 4 : 1];
+            for (int w = 0; w < 4; ++w) {
+                if constexpr (B == 2) {
+                    const uint32_t h = word(hf[0][0], w);
+                    f(2 * w, (h << 16) & 0x7FFF0000u);
+                    f(2 * w + 1, h & 0x7FFF0000u);
+                } else {
+                    f32x2 v[4];
 #pragma unroll
-            for (int l = 0; l < B; ++l) f[l] = reinterpret_cast<const float*>(&x[l][0])[i];
-            float z;
-            if constexpr (B == 2) {
-                z = __fmul_rn(__fadd_rn(f[0], f[1]), c32);
-                h[0] = __fmul_rn(__fsub_rn(f[0], f[1]), c32);
-            } else {
-                z = __fmul_rn(0.5f, __fadd_rn(__fadd_rn(f[0], f[1]), __fadd_rn(f[2], f[3])));
-                const float half = __fmul_rn(0.5f, z);  // exact
-#pragma unroll
-                for (int l = 0; l < 4; ++l) h[l] = __fsub_rn(f[l], half);
+                    for (int l = 0; l < 4; ++l) { v[l] = bf2(word(hf[l][0], w)); v[l] = mul2(v[l], v[l]); }
+                    const f32x2 e = add2(add2(v[0], v[1]), add2(v[2], v[3]));
+                    f(2 * w, (uint32_t)e & 0x7FFFFFFFu);
+                    f(2 * w + 1, (uint32_t)(e >> 32) & 0x7FFFFFFFu);
+                }
             }
-            reinterpret_cast<float*>(&z0[0])[i] = z;
+        } else {
 #pragma unroll
-            for (int l = 0; l < (B == 4 ? 4 : 1); ++l) reinterpret_cast<float*>(&hf[l][0])[i] = h[l];
-            for_key(i, key_of<B>(h));
+            for (int i = 0; i < 8; ++i) {
+                float h[NB];
+#pragma unroll
+                for (int l = 0; l < NB; ++l) h[l] = __uint_as_float(word(hf[l][i >> 2], i & 3));
+                f(i, key_of<B>(h));
+            }
         }
     }
+    __device__ static uint32_t reach(const uint4 (&hf)[NB][Q], uint32_t lo) {
+        if (lo == kNoKey) return 0u;
+        if constexpr (sizeof(T) == 2 && B == 2) {
+            // bit 15 (31) of a + (0x8000 - lo16) * 0x10001 says that the low (high) half reaches lo16: no carry crosses
+            const uint32_t add = (0x8000u - (lo >> 16)) * 0x00010001u;
+            const uint4& h = hf[0][0];
+            return pair_mask8((h.x & 0x7FFF7FFFu) + add, (h.y & 0x7FFF7FFFu) + add, (h.z & 0x7FFF7FFFu) + add, (h.w & 0x7FFF7FFFu) + add);
+        } else {
+            uint32_t k8[8], m = 0;
+            keys(hf, [&](int i, uint32_t key) { k8[i] = key - lo; });  // (both below 2^31: bit 31 says that the key is smaller)
+#pragma unroll
+            for (int i = 7; i >= 0; --i) m = __funnelshift_l(k8[i], m, 1);
+            return ~m & 0xFFu;
+        }
+    }
+
+private:
+    __device__ static uint32_t& word(uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+    __device__ static uint32_t word(const uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
 };
 
 // programmatic dependent launch: the next kernel of the chain may start its prologue now; nothing is read before the kernels
@@ -222,7 +258,8 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, 
         for (int q = 0; q < U; ++q) {
             if (v0 + q * kSampleThreads >= nvec) break;
             uint4 z0[Q], hf[NB][Q];
-            Eight<T, B>::split(f[q], z0, hf, [&](int, uint32_t key) { atomicAdd(&s_hist[key >> 19], 1u); });
+            Eight<T, B>::split(f[q], z0, hf);
+            Eight<T, B>::keys(hf, [&](int, uint32_t key) { atomicAdd(&s_hist[key >> 19], 1u); });
         }
     }
     __syncthreads();
@@ -234,156 +271,149 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, 
     }
 }
 
-// position of the k-th (from zero) set bit of x; x has more than k set bits
-__device__ __forceinline__ int kth_set_bit(uint32_t x, uint32_t k) {
-    int pos = 0;
-#pragma unroll
-    for (int width = 16; width >= 1; width >>= 1) {
-        const uint32_t c = __popc(x & ((1u << width) - 1u));
-        if (k >= c) {
-            k -= c;
-            pos += width;
-            x >>= width;
-        }
-    }
-    return pos;
-}
-
 // ---- 2: one read of K and V ---------------------------------------------------------------------------
 // Persistent blocks over (chunk, head x tensor) items; heads and tensors vary fastest, so the blocks that run at one time read
 // neighbouring rows.  A warp owns NV * 256 consecutive positions of a chunk, a lane eight of them per step.  The rows of the
 // next item are copied to shared memory (cp.async, 16 bytes per lane and layer, every lane its own) while one is worked on; the
-// high-frequency values take the place of the rows they came from.  A byte per eight positions goes to a bit map; with its
-// prefix, lane r finds entry r of the warp's part of the list by binary search and a population-count descent, so that the
-// list is written by consecutive lanes whatever the distribution of the candidates.  One block barrier per item (the warps'
-// counts).
+// high-frequency values take the place of the rows they came from.  A byte per eight positions goes to a bit map; then
+// every lane writes the candidates of its NV * 8 consecutive positions behind those of the lanes and warps before it.  One
+// block barrier per item (the warps' counts).  The issue slots are as busy as HBM here, hence the packed arithmetic, the
+// bit tricks and the running item coordinates (with scalar arithmetic, a binary search per list entry and divisions per item:
+// 1 550 us for 32 layers of 32k tokens).
 template <typename T, int B>
 __global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a, int items, int redo) {
     constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
     constexpr int CE = compress_chunk(B, (int)sizeof(T)), NV = CE / kSplitThreads / 8;
-    constexpr int WW = NV * 8;           // words of a warp's part of the bit map
+    constexpr int BITS = NV * 8;         // bits of the map per lane = words per warp
     constexpr int ROW = CE * (int)sizeof(T);  // bytes of a layer's part of a stage
     constexpr int STAGE = B * ROW;       // 32 KiB
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ uint32_t s_map[8][WW], s_pre[8][WW], s_cnt[2][8];
+    __shared__ uint32_t s_map[8][BITS], s_cnt[2][8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int uts = a.Hkv * a.tensors;
     chain_wait();
     if (redo) {  // (almost always there is nothing to do again)
-        const int per_block = items / uts;  // chunks x blocks of the launch
-        const int nb = per_block / a.chunks;
+        const int n_ut = items / a.chunks;
         int any = 0;
-        for (int i = tid; i < nb * uts; i += kSplitThreads) any |= (int)a.sel[a.ut_base + i].redo;
+        for (int i = tid; i < n_ut; i += kSplitThreads) any |= (int)a.sel[a.ut_base + i].redo;
         if (!__syncthreads_or(any)) return;
     }
     const int64_t n_e = (int64_t)a.T * a.d;
     const int dshift = a.d == 128 ? 7 : 6;
-    // item -> unit-tensor of the launch, chunk
-    auto locate = [&](int item, int& ut, int& u, int& blk, int64_t& e0) {
-        u = item % uts;
-        const int r = item / uts;
-        blk = r / a.chunks;
-        e0 = (int64_t)(r - blk * a.chunks) * CE;
-        ut = a.ut_base + blk * uts + u;
+    // an item's coordinates: head x tensor, chunk, block of the launch; a step is gridDim.x items
+    struct Item { int u, chunk, blk; };
+    const int step_u = gridDim.x % uts, step_r = gridDim.x / uts;
+    auto norm = [&](Item& m) {
+        while (m.chunk >= a.chunks) { m.chunk -= a.chunks; ++m.blk; }
+    };
+    auto advance = [&](Item& m) {
+        m.u += step_u;
+        m.chunk += step_r;
+        if (m.u >= uts) { m.u -= uts; ++m.chunk; }
+        norm(m);
     };
     const int p0 = warp * (NV * 256) + lane * 8;  // position of the lane's first eight; step q adds 256 q
-    auto request = [&](int item, int stage) {
-        if (item < items) {
-            int ut, u, blk;
-            int64_t e0;
-            locate(item, ut, u, blk, e0);
-            const int h = u / a.tensors, is_v = u % a.tensors;
+    const int64_t q_step = (int64_t)(256 >> dshift) * a.stride_t;
+    const uint32_t dst0 = (uint32_t)__cvta_generic_to_shared(smem) + p0 * (int)sizeof(T);
+    auto request = [&](const Item& m, int stage) {
+        const int h = m.u / a.tensors, is_v = m.u - h * a.tensors;
+        const int64_t e = (int64_t)m.chunk * CE + p0;
+        const int64_t off = (e >> dshift) * a.stride_t + (int64_t)h * a.stride_h + ((int)e & (a.d - 1));
 #pragma unroll
-            for (int q = 0; q < NV; ++q) {
-                const int64_t e = e0 + p0 + 256 * q;
-                if (e >= n_e) continue;
-                const int64_t off = (e >> dshift) * a.stride_t + (int64_t)h * a.stride_h + ((int)e & (a.d - 1));
+        for (int l = 0; l < B; ++l) {
+            const T* src = reinterpret_cast<const T*>(is_v ? a.v[B * m.blk + l] : a.k[B * m.blk + l]) + off;
 #pragma unroll
-                for (int l = 0; l < B; ++l) {
-                    const T* src = reinterpret_cast<const T*>(is_v ? a.v[B * blk + l] : a.k[B * blk + l]) + off;
-                    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem + stage * STAGE + l * ROW + (p0 + 256 * q) * sizeof(T));
+            for (int q = 0; q < NV; ++q, src += q_step)
+                if (e + 256 * q < n_e)
 #pragma unroll
                     for (int k = 0; k < Q; ++k)
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * k), "l"(reinterpret_cast<const uint4*>(src) + k) : "memory");
-                }
-            }
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst0 + stage * STAGE + l * ROW + 256 * q * (int)sizeof(T) + 16 * k),
+                                     "l"(reinterpret_cast<const uint4*>(src) + k)
+                                     : "memory");
+        }
+    };
+    Item now = {(int)(blockIdx.x % uts), (int)(blockIdx.x / uts), 0}, ahead;
+    norm(now);
+    ahead = now;
+    int left = (items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, to_request = left;  // items of this block
+    auto request_next = [&](int stage) {
+        if (to_request > 0) {
+            request(ahead, stage);
+            advance(ahead);
+            --to_request;
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    request(blockIdx.x, 0);
-    request(blockIdx.x + gridDim.x, 1);
-    for (int item = blockIdx.x, it = 0; item < items; item += gridDim.x, ++it) {
-        int ut, u, blk;
-        int64_t e0;
-        locate(item, ut, u, blk, e0);
-        const bool work = !redo || a.sel[ut].redo;  // (block-uniform)
+    request_next(0);
+    request_next(1);
+    for (int it = 0; left > 0; --left, it ^= 1, advance(now)) {
+        const int ut = a.ut_base + now.blk * uts + now.u;
+        const int64_t e0 = (int64_t)now.chunk * CE;
         const uint32_t lo = a.sel[ut].lo;
-        const bool is_k = u % a.tensors == 0;
-        uint8_t* const st = smem + (it & 1) * STAGE;
+        uint8_t* const st = smem + it * STAGE;
         asm volatile("cp.async.wait_group 1;" ::: "memory");
-        if (work) {
-            T* const z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride + e0;
-            T* const z1 = a.z1 && is_k ? reinterpret_cast<T*>(a.z1) + (int64_t)(ut / a.tensors) * NB * a.unit_stride + e0 : nullptr;
+        if (!redo || a.sel[ut].redo) {  // (block-uniform)
+            const int h = now.u / a.tensors;
+            const bool is_k = now.u == h * a.tensors;
+            T* const z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride + e0 + p0;
+            T* const z1 = a.z1 && is_k ? reinterpret_cast<T*>(a.z1) + (int64_t)(now.blk * a.Hkv + h + a.ut_base / a.tensors) * NB * a.unit_stride + e0 + p0 : nullptr;
 #pragma unroll
             for (int q = 0; q < NV; ++q) {
-                const int p = p0 + 256 * q;
                 uint32_t m8 = 0;
-                if (e0 + p < n_e) {
+                if (e0 + p0 + 256 * q < n_e) {
                     uint4 x[B][Q], z[Q], hf[NB][Q];
 #pragma unroll
                     for (int l = 0; l < B; ++l)
 #pragma unroll
-                        for (int k = 0; k < Q; ++k) x[l][k] = reinterpret_cast<const uint4*>(st + l * ROW + p * sizeof(T))[k];
-                    Eight<T, B>::split(x, z, hf, [&](int i, uint32_t key) { m8 |= (uint32_t)(key >= lo) << i; });
-                    if (lo == kNoKey) m8 = 0;
+                        for (int k = 0; k < Q; ++k) x[l][k] = reinterpret_cast<const uint4*>(st + l * ROW + (p0 + 256 * q) * sizeof(T))[k];
+                    Eight<T, B>::split(x, z, hf);
+                    m8 = Eight<T, B>::reach(hf, lo);
 #pragma unroll
                     for (int k = 0; k < Q; ++k) {
-                        if (!redo) reinterpret_cast<uint4*>(z0 + p)[k] = z[k];
+                        if (!redo) reinterpret_cast<uint4*>(z0 + 256 * q)[k] = z[k];
 #pragma unroll
                         for (int l = 0; l < NB; ++l) {
-                            if (z1 && !redo) reinterpret_cast<uint4*>(z1 + (int64_t)l * a.unit_stride + p)[k] = hf[l][k];
-                            reinterpret_cast<uint4*>(st + l * ROW + p * sizeof(T))[k] = hf[l][k];
+                            if (z1 && !redo) reinterpret_cast<uint4*>(z1 + (int64_t)l * a.unit_stride + 256 * q)[k] = hf[l][k];
+                            reinterpret_cast<uint4*>(st + l * ROW + (p0 + 256 * q) * sizeof(T))[k] = hf[l][k];
                         }
                     }
                 }
                 reinterpret_cast<uint8_t*>(s_map[warp])[32 * q + lane] = (uint8_t)m8;
             }
             __syncwarp();
-            uint32_t mine = lane < WW ? (uint32_t)__popc(s_map[warp][lane]) : 0u;
+            // the lane's BITS consecutive positions of the warp's part
+            uint32_t bits = BITS == 32   ? s_map[warp][lane]
+                            : BITS == 16 ? (uint32_t)reinterpret_cast<const uint16_t*>(s_map[warp])[lane]
+                                         : (uint32_t)reinterpret_cast<const uint8_t*>(s_map[warp])[lane];
+            const uint32_t mine = __popc(bits);
             uint32_t incl = mine;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
                 if (lane >= o) incl += y;
             }
-            if (lane < WW) s_pre[warp][lane] = incl - mine;
-            const uint32_t n_w = __shfl_sync(0xFFFFFFFFu, incl, 31);
-            if (lane == 0) s_cnt[it & 1][warp] = n_w;
+            if (lane == 31) s_cnt[it][warp] = incl;
             __syncthreads();
-            uint32_t base = 0, n = 0;
+            uint32_t at = incl - mine, n = 0;
 #pragma unroll
             for (int w = 0; w < 8; ++w) {
-                const uint32_t y = s_cnt[it & 1][w];
-                if (w < warp) base += y;
+                const uint32_t y = s_cnt[it][w];
+                if (w < warp) at += y;
                 n += y;
             }
-            if (tid == 0) a.cand_n[(int64_t)ut * a.chunks_max + (int)(e0 / CE)] = (int32_t)n;
-            uint16_t* const pos = a.cand_pos + (int64_t)ut * a.cand_stride + e0 + base;
-            T* const val = reinterpret_cast<T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0 + base;
-            for (uint32_t r = lane; r < n_w; r += 32) {
-                // the last word whose prefix does not exceed r holds entry r (empty words share their successor's prefix)
-                int w = 0;
+            if (tid == 0) a.cand_n[(int64_t)ut * a.chunks_max + now.chunk] = (int32_t)n;
+            uint16_t* const pos = a.cand_pos + (int64_t)ut * a.cand_stride + e0;
+            T* const val = reinterpret_cast<T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0;
+            const uint32_t first = warp * (NV * 256) + lane * BITS;
+            for (; bits; bits &= bits - 1, ++at) {
+                const uint32_t p = first + __ffs((int)bits) - 1;
+                pos[at] = (uint16_t)p;
 #pragma unroll
-                for (int s = WW / 2; s; s >>= 1)
-                    if (s_pre[warp][w + s] <= r) w += s;
-                const int p = warp * (NV * 256) + w * 32 + kth_set_bit(s_map[warp][w], r - s_pre[warp][w]);
-                pos[r] = (uint16_t)p;
-#pragma unroll
-                for (int l = 0; l < NB; ++l) val[(int64_t)l * a.cand_stride + r] = reinterpret_cast<const T*>(st + l * ROW)[p];
+                for (int l = 0; l < NB; ++l) val[(int64_t)l * a.cand_stride + at] = reinterpret_cast<const T*>(st + l * ROW)[p];
             }
             __syncwarp();  // (the warp's part of the stage is read)
         }
-        request(item + 2 * gridDim.x, it & 1);
+        request_next(it);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -407,15 +437,11 @@ __device__ __forceinline__ void each_candidate(const CompressArgs& a, int ut, in
 #pragma unroll
                     for (int k = 0; k < Q; ++k) v[s][l][k] = reinterpret_cast<const uint4*>(val + (int64_t)l * a.cand_stride + i0 + 256 * s)[k];
 #pragma unroll
-        for (int s = 0; s < STEPS; ++s)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (i0 + 256 * s + j >= n) break;
-                float w[NB];
-#pragma unroll
-                for (int l = 0; l < NB; ++l) w[l] = to_f32(reinterpret_cast<const T*>(&v[s][l][0])[j]);
-                f(key_of<B>(w));
-            }
+        for (int s = 0; s < STEPS; ++s) {
+            const int m = n - i0 - 256 * s;  // candidates from this vector on
+            if (m >= 8) Eight<T, B>::keys(v[s], [&](int, uint32_t key) { f(key); });
+            else if (m > 0) Eight<T, B>::keys(v[s], [&](int j, uint32_t key) { if (j < m) f(key); });
+        }
     }
 }
 
@@ -539,11 +565,10 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
 // ---- 4: the lists -------------------------------------------------------------------------------------
 // Packed entry of the bf16 / head_dim 128 decode kernel: low half = value bits, high half = (byte offset / 2) of the position
 // inside a 16-token x 128-channel tile of two 64-channel halves with 128-byte rows whose 16-byte chunks are XOR-swizzled
-// with the row.
-__device__ __forceinline__ uint32_t packed_entry(float v, int flat) {
-    const int row = (flat >> 7) & 15, ch = flat & 127;
-    const uint32_t off = (uint32_t)((ch >> 6) * 2048 + row * 128 + ((((ch >> 3) & 7) ^ (row & 7)) << 4) + (ch & 7) * 2);
-    return (__float_as_uint(v) >> 16) | ((off >> 1) << 16);
+// with the row.  p: position in a chunk (a whole number of tiles).
+__device__ __forceinline__ uint32_t packed_place(uint32_t p) {
+    const uint32_t half = (p >> 6) & 1u, row = (p >> 7) & 15u, chunk = ((p >> 3) ^ (p >> 7)) & 7u;
+    return (half << 10 | row << 6 | chunk << 3 | (p & 7u)) << 16;
 }
 
 // grid (groups of eight chunks, unit-tensors), a chunk per warp: no block barriers, U rounds of candidates requested together
@@ -568,6 +593,9 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
     uint32_t run_gt = (uint32_t)b0.x, run_eq = (uint32_t)b0.y;
     const uint32_t first = run_gt + min(run_eq, need);  // list position of the chunk's first entry
     const uint32_t below = (1u << lane) - 1u;
+    int32_t* const idx = a.idx + (int64_t)ut * a.kcap;
+    T* const out = reinterpret_cast<T*>(a.val) + (int64_t)ut * NB * a.kcap;
+    uint32_t* const packed = sizeof(T) == 2 && a.packed ? a.packed + (int64_t)ut * NB * a.kcap : nullptr;
     __syncwarp();
     for (int i0 = lane; i0 < n + lane; i0 += 32 * U) {
         uint32_t p[U];
@@ -575,7 +603,6 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const int i = i0 + 32 * q;
-            p[q] = 0;
             if (i < n) {
                 p[q] = pos[i];
 #pragma unroll
@@ -587,22 +614,21 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
             const bool on = i0 + 32 * q < n;
             float v[NB];
 #pragma unroll
-            for (int l = 0; l < NB; ++l) v[l] = on ? to_f32(raw[q][l]) : 0.f;
+            for (int l = 0; l < NB; ++l) v[l] = to_f32(raw[q][l]);
             const uint32_t key = key_of<B>(v);
             const bool gt = on && key > tau, eq = on && key == tau;
             const uint32_t mg = __ballot_sync(0xFFFFFFFFu, gt), me = __ballot_sync(0xFFFFFFFFu, eq);
             const uint32_t be = run_eq + __popc(me & below);
             if (gt || (eq && be < need)) {  // ties in index order while fewer than `need` precede them
-                const int64_t at = run_gt + __popc(mg & below) + min(be, need);
-                const int flat = (int)e0 + (int)p[q];
-                a.idx[(int64_t)ut * a.kcap + at] = flat;
+                const uint32_t at = run_gt + __popc(mg & below) + min(be, need);
+                idx[at] = (int)e0 + (int)p[q];
+                const uint32_t place = sizeof(T) == 2 ? packed_place(p[q]) : 0u;
 #pragma unroll
                 for (int l = 0; l < NB; ++l) {
-                    const int64_t o = ((int64_t)ut * NB + l) * a.kcap + at;
-                    reinterpret_cast<T*>(a.val)[o] = raw[q][l];
+                    out[(int64_t)l * a.kcap + at] = raw[q][l];
                     // (a block of four scales its rows by 1/2 at decode time and its deviations by 1: twice the deviation is stored)
                     if constexpr (sizeof(T) == 2)
-                        if (a.packed) a.packed[o] = packed_entry(B == 4 ? 2.f * v[l] : v[l], flat);
+                        if (packed) packed[(int64_t)l * a.kcap + at] = (__float_as_uint(B == 4 ? 2.f * v[l] : v[l]) >> 16) | place;
                 }
                 atomicOr(&map[p[q] >> 5], 1u << (p[q] & 31));
             }
