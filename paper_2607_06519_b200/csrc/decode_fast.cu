@@ -33,7 +33,7 @@ namespace fdkv {
 namespace {
 
 constexpr int kTT = 128;         // tokens per stage
-constexpr int kStages = 3;
+constexpr int kMaxStages = 3;  // (two in clusters, whose blocks have few tiles and need room for their peers' parts)
 constexpr int kCW = kTT / 16;    // warps, 16 tokens of a stage each
 constexpr int kThreads = kCW * 32;  // 256 threads: two warps per scheduler, so up to 255 registers per thread
 constexpr int kHalfBytes = kTT * 128;        // one 64-channel box of 128 tokens
@@ -41,9 +41,12 @@ constexpr int kStageBytes = 4 * kHalfBytes;  // K ch 0-63, K ch 64-127, V ch 0-6
 constexpr int kScratchBytes = 4096;          // per consumer warp: 16 tokens x 128 channels bf16 (or its O tile at merge)
 constexpr int kHeaderBytes = 2048;
 constexpr int kMaxSeg = 24;  // (unit, range) segments one CTA can walk: at most units / CTAs + 2
-constexpr int kSmemBytes = kHeaderBytes + kStages * kStageBytes + kCW * kScratchBytes;
+constexpr int kSmemBytes = kHeaderBytes + kMaxStages * kStageBytes + kCW * kScratchBytes;
+constexpr int kJointBytes = 8 * 128 * 4 + 2 * 8 * 8 * 4;  // a cluster's parts of this block's outputs: [blocks][share], then maxima and sums [blocks][8]
+constexpr int kSmemBytesCl = kHeaderBytes + 2 * kStageBytes + kCW * kScratchBytes + kJointBytes;
 constexpr int kMaxCtas = kMaxSplits;
 constexpr int kMaxUnits = kFastMaxUnits;
+constexpr int kMaxCluster = 8;  // thread blocks of a cluster (the largest portable size)
 constexpr int kPF = 8;  // residual entries prefetched per lane and list
 constexpr int kPartStride = 128 + 4;  // floats per split-K part: max, sum, 2 pad, 128 accumulators (16-byte aligned)
 static_assert(kTT == kRowPad, "row blocks are padded to whole stages");
@@ -129,6 +132,15 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_smem(uint32_t addr, int rank) {  // the same shared-memory address in another block of the cluster
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
 __device__ __forceinline__ void st_shared_u16(uint32_t addr, uint16_t v) {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
 }
@@ -155,10 +167,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // on a fresh state and joins the two at the merge.
 // (at most 232 registers: two warps of this kernel on a quarter of an SM leave 1 536 of its 16 384, one warp of
 // decode_combine_kernel with at most 48)
-template <bool F8>
+// CL: every unit's thread blocks form a cluster (its dimension is the unit's number of blocks) and join their states through
+// distributed shared memory, so that a call is one kernel: for short contexts, whose cost is the chain of hand-overs.
+template <bool F8, bool CL>
 __global__ void __maxnreg__(232)
 decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap8, DecodeArgs a, FastSched sch,
                    PartCount pc, TailLens tl) {
+    constexpr int kStages = CL ? 2 : kMaxStages;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t smem0 = smem_u32(smem_raw);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem_raw + kOffAbort);
@@ -170,6 +185,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
     // Let the next kernel in the stream start its own prologue as soon as SMs free up (programmatic dependent
     // launch); everything this kernel reads before its own griddepcontrol.wait is static since commit.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (CL) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // "running": awaited before the first write to a peer
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(smem0 + kOffFull + 8 * s, 1);
@@ -272,28 +288,8 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
     auto dependency_wait = [&]() {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         waited = true;
-        if (sch.any_tail && warp == 0 && a.k_new) {
-            // Generated tokens of this call: the thread block that streams a unit's tail appends the unit's new K and V
-            // rows itself (16 lanes x 16 bytes each) and makes them visible to the tensor copies it issues next; k_new /
-            // v_new are read behind the dependency wait.
-            for (int i = 0; i < seg_info[0]; ++i) {
-                const int tu = segs[i].tail_u;
-                if (tu < 0) continue;
-                const int tb = tu / a.Hkv, th = tu % a.Hkv;
-                const int n = min(tl.n[tb], a.max_tail);
-                if (n <= 0) continue;
-                const int64_t row = (((int64_t)a.layer * a.max_batch + tb) * a.Hkv + th) * a.tail_rows + (n - 1);
-                const uint4* src = reinterpret_cast<const uint4*>(lane < 16 ? a.k_new : a.v_new) + ((int64_t)tb * a.Hkv + th) * 16 + (lane & 15);
-                uint4* dst = reinterpret_cast<uint4*>(lane < 16 ? a.tail_k : a.tail_v) + row * 16 + (lane & 15);
-                *dst = *src;
-                if (lane == 0 && th == 0) a.tail_len[a.layer * a.max_batch + tb] = n;  // the device copy of the length (other kernels read it)
-            }
-            asm volatile("fence.proxy.async;" ::: "memory");
-            __syncwarp();
-        }
         if (is_producer)
             for (int it = prologue_issued; it < kStages && it < seg_info[1]; ++it) issue_tile(it);
-        if (sch.any_tail) __syncthreads();  // (any warp may refill a stage with a tail tile)
     };
 
     // ================= compute: every warp takes 16 tokens of every stage =================
@@ -324,6 +320,10 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                 n_tail_rows = min(tl.n[b], a.max_tail);
                 ntail = (n_tail_rows + kTT - 1) / kTT;
             }
+            // The row that this call appends is the last of the tail.  Its copy from the tail is stale: the warp that owns it takes
+            // it from the caller, puts it into the landed tile and stores it to the tail for later calls, so that the tail's
+            // copy is requested right behind the dependency wait and no store has to become visible to it.
+            const bool append = ntail > 0 && a.k_new && warp == ((n_tail_rows - 1) & (kTT - 1)) >> 4;
             const int npre = (rows16 + kTT - 1) / kTT, nseg = npre + ntail;
             const bool coef = ud.mode != FDKV_MODE_EXACT, resid = ud.mode == FDKV_MODE_RESIDUAL;
             const uint32_t sgn = ud.sign < 0.f ? 0x80008000u : 0u;
@@ -606,24 +606,69 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                     for (int e = 0; e < 2; ++e) { sm_m[warp * 8 + 2 * tig + e] = m_run[e]; sm_l[warp * 8 + 2 * tig + e] = lq[e]; }
                 }
                 __syncthreads();
-                for (int i = threadIdx.x; i < a.G * 128; i += kThreads) {
-                    const int g = i >> 7, ch = i & 127;
+                uint32_t rank = 0, nb = 1, share = 1024;
+                if constexpr (CL) {
+                    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+                    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nb));
+                    share = (uint32_t)a.G * 128 / nb;  // outputs of the unit that a block joins
+                    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+                }
+                for (int i = threadIdx.x; i < a.G * 64; i += kThreads) {  // two channels per thread
+                    const int g = i >> 6, ch = 2 * (i & 63);
                     float M = -INFINITY;
 #pragma unroll
                     for (int w = 0; w < kCW; ++w) M = fmaxf(M, sm_m[w * 8 + g]);
-                    float L = 0.f, A = 0.f;
+                    float L = 0.f;
+                    float2 A = make_float2(0.f, 0.f);
                     if (M != -INFINITY) {
 #pragma unroll
                         for (int w = 0; w < kCW; ++w) {
                             const float f = ex2(sm_m[w * 8 + g] - M);
                             L = fmaf(sm_l[w * 8 + g], f, L);
-                            const float* ow = reinterpret_cast<const float*>(smem_raw + kHeaderBytes + kStages * kStageBytes + w * kScratchBytes);
-                            A = fmaf(ow[g * 128 + ch], f, A);
+                            const float2 o = *reinterpret_cast<const float2*>(smem_raw + kHeaderBytes + kStages * kStageBytes + w * kScratchBytes + (g * 128 + ch) * 4);
+                            A.x = fmaf(o.x, f, A.x);
+                            A.y = fmaf(o.y, f, A.y);
                         }
                     }
-                    float* part = a.partials + (((int64_t)b * a.Hq + h * a.G + g) * kMaxSplits + slot) * kPartStride;
-                    if (ch == 0) { part[0] = M * 0.6931471805599453f; part[1] = L; }  // the combine step works in natural-log units
-                    part[4 + ch] = A;
+                    if constexpr (CL) {
+                        // to the block that joins these channels
+                        const uint32_t o = (uint32_t)(g * 128 + ch), to = o / share;
+                        const uint32_t joint = peer_smem(smem0 + kHeaderBytes + kStages * kStageBytes + kCW * kScratchBytes, (int)to);
+                        st_peer(joint + (rank * share + (o - to * share)) * 4, A.x);
+                        st_peer(joint + (rank * share + (o - to * share) + 1) * 4, A.y);
+                        if (o % share == 0 || ch == 0) {  // (a share starts inside a head or covers whole heads)
+                            st_peer(joint + (1024 + rank * 8 + g) * 4, M);
+                            st_peer(joint + (1024 + 64 + rank * 8 + g) * 4, L);
+                        }
+                    } else {
+                        float* part = a.partials + (((int64_t)b * a.Hq + h * a.G + g) * kMaxSplits + slot) * kPartStride;
+                        if (ch == 0) { part[0] = M * 0.6931471805599453f; part[1] = L; }  // the combine step works in natural-log units
+                        *reinterpret_cast<float2*>(part + 4 + ch) = A;
+                    }
+                }
+                if constexpr (CL) {
+                    cluster_barrier();
+                    const float* const joint = reinterpret_cast<const float*>(smem_raw + kHeaderBytes + kStages * kStageBytes + kCW * kScratchBytes);
+                    for (uint32_t i = threadIdx.x; i < share; i += kThreads) {
+                        const uint32_t o = rank * share + i, g = o >> 7;
+                        float m[kMaxCluster], M = -INFINITY, L = 0.f, A = 0.f;
+#pragma unroll
+                        for (int c = 0; c < kMaxCluster; ++c) {
+                            m[c] = c < (int)nb ? joint[1024 + c * 8 + g] : -INFINITY;
+                            M = fmaxf(M, m[c]);
+                        }
+#pragma unroll
+                        for (int c = 0; c < kMaxCluster; ++c)
+                            if (c < (int)nb) {
+                                const float f = m[c] == -INFINITY ? 0.f : ex2(m[c] - M);
+                                L = fmaf(joint[1024 + 64 + c * 8 + g], f, L);
+                                A = fmaf(joint[c * share + i], f, A);
+                            }
+                        const float r = L > 0.f ? A / L : 0.f;
+                        const int64_t at = ((int64_t)b * a.Hq + h * a.G) * 128 + o;
+                        if (a.out_dtype == FDKV_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[at] = __float2bfloat16_rn(r);
+                        else reinterpret_cast<float*>(a.out)[at] = r;
+                    }
                 }
                 if (u < u_last && u + 1 < sch.units) {  // (another segment may follow: the scratch tiles and sums are read by now)
                     __syncthreads();
@@ -765,7 +810,8 @@ bool make_arena_tensor_map(void* arena, size_t arena_bytes, void* tmap_out) {
 
 // Host side of a launch: the cost-weighted cut of the batch's (unit, 16-token slice) list into one range per CTA and the
 // split-K part count of every unit.  Uses only the host views in `a` (lengths, modes, shape); no device access.
-static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_count, FastSched& sch, PartCount& cs) {
+// max_clusters[i]: clusters of 2^i blocks that fit the device at one time (null: plan without clusters).
+static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_count, const int* max_clusters, FastSched& sch, PartCount& cs) {
     // ---- cost-weighted schedule: whole CTAs per unit when there are enough CTAs, else a flat cut of the (unit, tile) list ----
     std::vector<int64_t> wp(units + 1, 0);
     // ranges are cut on 16-token slices (the granularity of the residual lists), so that the CTAs of a unit differ by
@@ -815,6 +861,41 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     sch.ncta = ncta;
     sch.any_tail = a.any_tail;
     sch.units = units;
+    sch.cluster = 0;
+    // Clusters, as many blocks per unit as fit: one kernel instead of two, where that is worth more than the blocks that are
+    // left out.  The hand-over to the combine kernel and its launch cost as much as kClusterGain plain tiles: a layer call of two
+    // KV heads, 512 tokens, 6.3 -> 5.0 us replayed and 8.2 -> 5.5 issued on a stream, 2k tokens 6.0 -> 6.6 and 8.0 -> 7.3, 8k tokens
+    // (two kernels stay) 8.2 against 14.4.
+    if (max_clusters) {
+        constexpr double kClusterGain = 2.0;
+        int least = ns[0];
+        for (int u = 1; u < units; ++u) least = std::min(least, ns[u]);
+        int lg = 3;
+        while (lg > 0 && (units > max_clusters[lg] || (1 << lg) > least)) --lg;
+        const int C = 1 << lg;
+        if (units <= max_clusters[lg] && units * C <= kMaxCtas) {
+            double worst = 0.0, tile = 2 * kTT * 256 / 512, all = 0.0;  // in plain tiles
+            for (int u = 0; u < units; ++u) {
+                const double mine = (double)es[u] * wt[u] / (kTT / kResTile) / tile;
+                // (whole tiles per block)
+                worst = std::max(worst, std::ceil((double)es[u] / C / (kTT / kResTile)) * wt[u] / tile);
+                all += mine;
+            }
+            if (worst <= std::max(1.0, all / ctas) + kClusterGain) {
+                int c = 0;
+                for (int u = 0; u < units; ++u)
+                    for (int j = 0; j < C; ++j, ++c) {
+                        sch.start[c] = ((uint32_t)u << 20) | (uint32_t)std::min((int64_t)es[u] * j / C, (int64_t)(ns[u] - (C - j)));
+                        sch.slot[c] = (uint8_t)j;
+                    }
+                sch.start[c] = (uint32_t)units << 20;
+                sch.ncta = c;
+                sch.cluster = C;
+                for (int u = 0; u < kMaxUnits; ++u) cs.n[u] = u < units ? C : 0;
+                return cudaSuccess;
+            }
+        }
+    }
     bool whole = units <= ncta;
     std::vector<int> nc(units, 1);
     if (whole) {
@@ -902,7 +983,7 @@ cudaError_t plan_decode_host(const DecodeArgs& a, int n_ctas, uint32_t* start_ou
     if (units < 1 || units > kMaxUnits || n_ctas < 1) return cudaErrorInvalidValue;
     FastSched sch;
     PartCount cs;
-    const cudaError_t e = plan_decode_schedule(a, units, n_ctas, sch, cs);
+    const cudaError_t e = plan_decode_schedule(a, units, n_ctas, nullptr, sch, cs);
     if (e != cudaSuccess) return e;
     for (int c = 0; c <= sch.ncta; ++c) start_out[c] = sch.start[c];
     for (int u = 0; u < units; ++u) parts_out[u] = cs.n[u];
@@ -916,13 +997,33 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     if (!a.tmap || !a.packed_lists || a.d != 128 || units > kMaxUnits || units < 1) return cudaSuccess;
     if (a.rows_f8 && !a.tmap_u8) return cudaSuccess;
     static PerDevice once;
-    int sm_count = 0;
-    cudaError_t e0 = once.ensure([&]() {
-        cudaError_t e = cudaFuncSetAttribute(decode_fast_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_fast_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    static int max_clusters_of[PerDevice::kMaxDevices][4];  // [device][log2 of the blocks]
+    int sm_count = 0, dev = 0;
+    cudaError_t e0 = cudaGetDevice(&dev);
+    if (e0 == cudaSuccess) e0 = once.ensure([&]() {
+        cudaError_t e = cudaSuccess;
+        auto opt_in = [&](auto kernel, int smem) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        };
+        opt_in(decode_fast_kernel<false, false>, kSmemBytes);
+        opt_in(decode_fast_kernel<true, false>, kSmemBytes);
+        opt_in(decode_fast_kernel<false, true>, kSmemBytesCl);
+        opt_in(decode_fast_kernel<true, true>, kSmemBytesCl);
         // the same division of the SM's memory as the decode kernel's, or the two could not share an SM
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        for (int lg = 0; lg < 4 && e == cudaSuccess; ++lg) {
+            cudaLaunchConfig_t q = {};
+            q.gridDim = dim3(8 << lg);
+            q.blockDim = dim3(kThreads);
+            q.dynamicSmemBytes = kSmemBytesCl;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = 1u << lg; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            q.attrs = at;
+            q.numAttrs = 1;
+            e = cudaOccupancyMaxActiveClusters(&max_clusters_of[dev][lg], decode_fast_kernel<false, true>, &q);
+        }
         return e;
     }, &sm_count);
     if (e0 != cudaSuccess) return e0;
@@ -931,7 +1032,7 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     for (int b = 0; current && b < a.batch; ++b) current = plan.tail_tiles[b] == (a.host_tail[b] + kTT - 1) / kTT;
     if (!current) {
         plan.epoch = 0;
-        const cudaError_t pe = plan_decode_schedule(a, units, sm_count, plan.sch, plan.pc);
+        const cudaError_t pe = plan_decode_schedule(a, units, sm_count, max_clusters_of[dev], plan.sch, plan.pc);
         if (pe != cudaSuccess) return pe;
         plan.epoch = a.plan_epoch; plan.batch = a.batch; plan.sm_count = sm_count;
         plan.tail_tiles.resize(a.batch);
@@ -943,32 +1044,38 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ncta);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.dynamicSmemBytes = sch.cluster ? kSmemBytesCl : kSmemBytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = std::max(1, sch.cluster); attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = sch.cluster ? 2 : 1;
     const CUtensorMap& m16 = *reinterpret_cast<const CUtensorMap*>(a.tmap);
     const CUtensorMap& m8 = *reinterpret_cast<const CUtensorMap*>(a.rows_f8 ? a.tmap_u8 : a.tmap);
     TailLens tl;
     for (int b = 0; b < a.batch; ++b) tl.n[b] = a.host_tail[b];
-    cudaError_t e = a.rows_f8 ? cudaLaunchKernelEx(&cfg, decode_fast_kernel<true>, m16, m8, a, sch, cs, tl)
-                              : cudaLaunchKernelEx(&cfg, decode_fast_kernel<false>, m16, m8, a, sch, cs, tl);
+    auto* const kernel = sch.cluster ? (a.rows_f8 ? decode_fast_kernel<true, true> : decode_fast_kernel<false, true>)
+                                     : (a.rows_f8 ? decode_fast_kernel<true, false> : decode_fast_kernel<false, false>);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, cs, tl);
     if (e != cudaSuccess) return e;
+    count_launch(1);
+    count_kernel(FDKV_KERNEL_DECODE_FAST);
+    *handled = true;
+    if (sch.cluster) return cudaSuccess;
     // one channel per lane where a head has many parts (few heads: latency), four where the heads fill the machine
     const bool wide = units * a.G > sm_count;
     cfg.gridDim = dim3(wide ? 1 : 4, a.Hq, a.batch);
     cfg.blockDim = dim3(32);
     cfg.dynamicSmemBytes = 0;
+    cfg.numAttrs = 1;
     const float* parts = a.partials;
     e = wide ? cudaLaunchKernelEx(&cfg, decode_combine_kernel<4>, parts, a.Hq, a.Hkv, a.G, cs, a.out, a.out_dtype)
              : cudaLaunchKernelEx(&cfg, decode_combine_kernel<1>, parts, a.Hq, a.Hkv, a.G, cs, a.out, a.out_dtype);
     if (e != cudaSuccess) return e;
-    count_launch(2);
-    count_kernel(FDKV_KERNEL_DECODE_FAST);
-    *handled = true;
+    count_launch(1);
     return cudaGetLastError();
 }
 

@@ -54,6 +54,7 @@ struct FastSched {
     uint32_t start[kMaxSplits + 1];  // unit << 20 | first 16-token slice of CTA c; start[ncta] = units << 20
     uint8_t slot[kMaxSplits];        // split-K part of CTA c's first unit that CTA c writes (its later units start with it: part 0)
     int ncta, units;
+    int cluster;   // thread blocks per unit, one cluster each, in one kernel; 0: the ranges are free and a second kernel combines
     int any_tail;  // some sequence of the batch holds generated tokens in this layer's tail (host mirror)
 };
 struct PartCount {

@@ -1,0 +1,38 @@
+"""Short contexts: a unit's thread blocks as one cluster, from one block to eight, with and without appended rows (the appended
+row of a call is not read back from the tail), first and last row of a 16-row slice and of a 128-row box, both row formats."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import TOL, f32, oracle_unit, vector_errors
+from oracle import fdkv_ref_fp8 as R8
+from paper_2607_06519_b200 import runner, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("rows", [0, 1])
+@pytest.mark.parametrize("hkv,group,T,n", [(1, 4, 1, 2), (2, 1, 17, 18), (1, 2, 130, 3), (8, 4, 513, 129), (3, 4, 1000, 2), (16, 2, 300, 2)])
+def test_generated_rows(hkv, group, T, n, rows):
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=hkv, n_q_heads=hkv * group, T=T, n_needles=1, W=1, n_steps=n, row_format=rows,
+                                            name="clusters")
+    pf = runner.Prefilled(w, max_tail=n)
+    modes = np.array([[(1 + h) % 3 for h in range(hkv)]])
+    pf.prefill(0, modes)
+    units = {}
+    for h in {0, hkv - 1}:
+        if rows:
+            units[h] = R8.UnitFp8(*synth.unit_tensor(w, 0, 0, h, False), *synth.unit_tensor(w, 0, 0, h, True), True, w.keep_num, w.keep_den)
+        else:
+            units[h] = oracle_unit(w, 0, 0, h)
+    for step in range(n):
+        for layer in range(2):
+            q = pf.decode_q(layer, step)
+            kn, vn = pf.new_rows(layer, step)
+            out = pf.ctx.decode_attn(layer, q, kn, vn)
+            for h, u in units.items():
+                u.append(layer, f32(kn)[0, h], f32(vn)[0, h])
+                if step in (0, 1, 15, 16, 17, 127, 128) or step == n - 1:
+                    ref = u.attend(int(modes[0, h]), layer, f32(q)[0][h * group:(h + 1) * group])
+                    assert vector_errors(f32(out)[0][h * group:(h + 1) * group], ref).max() <= TOL["bf16"], (step, layer, h)
+    assert pf.ctx.device_status() == 0
