@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfdkv.so")
 SOURCES = ["api.cu", "compress.cu", "select.cu", "rows_fp8.cu", "probe.cu", "probe_tc.cu", "probe_gram.cu", "token_rule.cu", "decode.cu", "decode_fast.cu", "test_hooks.cu"]
-HEADERS = ["fdkv_internal.h", "mbar_wait.cuh", "umma.cuh", "decode_fast_tile.inc", os.path.join("..", "..", "include", "fdkv.h"),
+HEADERS = ["fdkv_internal.h", "mbar_wait.cuh", "umma.cuh", "decode_fast_tile.inc", "decode_fast_tile8.inc", os.path.join("..", "..", "include", "fdkv.h"),
            os.path.join("..", "..", "include", "fdkv_testing.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas", "-v"]

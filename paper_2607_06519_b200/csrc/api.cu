@@ -275,7 +275,7 @@ fdkv_status fdkv_create(const fdkv_config* cfg, void* arena, size_t arena_bytes,
     if (e != cudaSuccess) { delete c; return cuda_fail(e); }
     if (s.dtype == FDKV_BF16 && s.d == 128) c->has_tmap = make_arena_tensor_map(c->arena, arena_bytes, c->tmap);
     c->packed_lists = c->has_tmap && s.max_batch * s.Hkv <= kFastMaxUnits;
-    if (s.rows_f8 && !(c->packed_lists && make_rows_tensor_map_u8(c->arena, arena_bytes, kRowPad, c->tmap_u8))) { delete c; return FDKV_ERR_UNSUPPORTED; }
+    if (s.rows_f8 && !(c->packed_lists && make_arena_tensor_map_u8(c->arena, arena_bytes, c->tmap_u8))) { delete c; return FDKV_ERR_UNSUPPORTED; }
     // token rule: the tensor-core score kernel and the packed decode kernel serve bf16 / head_dim 128; everything else
     // takes the float32 score kernel and the portable decode kernel
     if (s.tok_rule && c->packed_lists)

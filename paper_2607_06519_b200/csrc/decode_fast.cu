@@ -2,7 +2,7 @@
 // coefficients broadcast to both layers of the pair, residual coefficients added only where indexed, the full
 // cache never materialised).
 //
-// One persistent CTA of eight warps per SM.  128-token K and V boxes of the packed cache stream through a ring of
+// One persistent CTA of eight warps per SM.  128-token (8-bit rows: 256-token) K and V boxes of the packed cache stream through a ring of
 // shared-memory stages with TMA (128-byte swizzle, mbarrier completion).  The CTA's tile sequence sits in a small
 // segment table in shared memory; whichever warp finishes a tile last re-arms its stage with the tile three ahead,
 // so no warp is a dedicated producer.  Each warp owns 16 tokens of a stage and a private online-softmax state:
@@ -33,24 +33,29 @@ namespace fdkv {
 namespace {
 
 constexpr int kTT = 128;         // tokens per stage
-constexpr int kMaxStages = 3;  // (two in clusters, whose blocks have few tiles and need room for their peers' parts)
+constexpr int kTT8 = 256;        // tokens per stage of 8-bit rows: the same bytes
+// Stages: three; two in clusters, whose blocks have few tiles and need room for their peers' parts, and with 8-bit rows, whose
+// warps hold two residual tiles.
+constexpr int stages_of(bool f8, bool cl) { return f8 || cl ? 2 : 3; }
 constexpr int kCW = kTT / 16;    // warps, 16 tokens of a stage each
 constexpr int kThreads = kCW * 32;  // 256 threads: two warps per scheduler, so up to 255 registers per thread
 constexpr int kHalfBytes = kTT * 128;        // one 64-channel box of 128 tokens
 constexpr int kStageBytes = 4 * kHalfBytes;  // K ch 0-63, K ch 64-127, V ch 0-63, V ch 64-127
-constexpr int kScratchBytes = 4096;          // per consumer warp: 16 tokens x 128 channels bf16 (or its O tile at merge)
+constexpr int kScratchTile = 4096;           // 16 tokens x 128 channels bf16: the residual of one slice
+constexpr int scratch_of(bool f8) { return f8 ? 2 * kScratchTile : kScratchTile; }  // per warp (also its O tile at merge)
 constexpr int kHeaderBytes = 2048;
 constexpr int kMaxSeg = 24;  // (unit, range) segments one CTA can walk: at most units / CTAs + 2
-constexpr int kSmemBytes = kHeaderBytes + kMaxStages * kStageBytes + kCW * kScratchBytes;
 constexpr int kJointBytes = 8 * 128 * 4 + 2 * 8 * 8 * 4;  // a cluster's parts of this block's outputs: [blocks][share], then maxima and sums [blocks][8]
-constexpr int kSmemBytesCl = kHeaderBytes + 2 * kStageBytes + kCW * kScratchBytes + kJointBytes;
+constexpr int smem_of(bool f8, bool cl) {
+    return kHeaderBytes + stages_of(f8, cl) * kStageBytes + kCW * scratch_of(f8) + (cl ? kJointBytes : 0);
+}
 constexpr int kMaxCtas = kMaxSplits;
 constexpr int kMaxUnits = kFastMaxUnits;
 constexpr int kMaxCluster = 8;  // thread blocks of a cluster (the largest portable size)
-constexpr int kPF = 8;  // residual entries prefetched per lane and list
 constexpr int kPartStride = 128 + 4;  // floats per split-K part: max, sum, 2 pad, 128 accumulators (16-byte aligned)
 static_assert(kTT == kRowPad, "row blocks are padded to whole stages");
-static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+static_assert(smem_of(false, false) <= 227 * 1024 && smem_of(true, true) <= 227 * 1024, "shared memory budget");
+static_assert(kTT8 * 128 * 2 == kStageBytes, "a stage holds as many bytes in either row format");
 
 struct TailLens {
     int32_t n[kMaxUnits];  // generated tokens in this layer's tail per sequence, this call's append included (host mirror)
@@ -173,7 +178,12 @@ template <bool F8, bool CL>
 __global__ void __maxnreg__(232)
 decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap8, DecodeArgs a, FastSched sch,
                    PartCount pc, TailLens tl) {
-    constexpr int kStages = CL ? 2 : kMaxStages;
+    constexpr int kStages = CL || F8 ? 2 : 3, kScratchBytes = F8 ? 2 * kScratchTile : kScratchTile;
+    constexpr int TT = F8 ? kTT8 : kTT;   // tokens of a packed tile
+    constexpr int SW = TT / 16 / kCW;     // 16-token slices of it per warp
+    // Residual entries prefetched per lane and list (the rest are loaded when used).  8-bit rows, two slices per warp, us a layer of 32k at
+    // keep 1/32, 1/16 and 1/8: eight 21.2, 21.5 and 27.3, twelve 21.6, 21.8 and 25.0.
+    constexpr int kPF = F8 ? 12 : 8;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t smem0 = smem_u32(smem_raw);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem_raw + kOffAbort);
@@ -216,8 +226,8 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
     auto issue_rows = [&](int s, int kr, int vr, bool f8_box) {  // s = the tile's stage (its index in the CTA's sequence mod kStages)
         const uint32_t full = smem0 + kOffFull + 8 * s;
         const uint32_t dst = stage0 + s * kStageBytes;
-        if (F8 && f8_box) {  // one 128-token x 128-byte box per tensor, in the first half of the K and of the V slot
-            mbar_expect_tx(full, 2 * kHalfBytes);
+        if (F8 && f8_box) {  // one 256-token x 128-byte box per tensor
+            mbar_expect_tx(full, kStageBytes);
             tma_load_2d(dst, &tmap8, 0, kr, full);
             tma_load_2d(dst + 2 * kHalfBytes, &tmap8, 0, vr, full);
         } else {
@@ -235,7 +245,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         const int j = it - g.it0;
         // ranges start on any 16-token slice and their tiles count from there; the box of the partial tile that ends a
         // range is moved back over rows the CTA has read already (masked when used), so that no copy passes the range's end
-        const int tok = max(0, g.tb + min((rev ? g.npre - 1 - j : j) * kTT, g.rows16 - kTT));
+        const int tok = max(0, g.tb + min((rev ? g.npre - 1 - j : j) * TT, g.rows16 - TT));
         const int kr = j < g.npre ? g.krow + tok : g.tkrow + (j - g.npre) * kTT;
         const int vr = j < g.npre ? g.vrow + tok : g.tvrow + (j - g.npre) * kTT;
         issue_rows(it % kStages, kr, vr, j < g.npre);
@@ -258,7 +268,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             g.tkrow = g.tvrow = 0;
             g.tb = sb * kResTile;
             g.rows16 = (min(se, nsl) - sb) * kResTile;
-            g.npre = (g.rows16 + kTT - 1) / kTT;
+            g.npre = (g.rows16 + TT - 1) / TT;
             g.it0 = it0;
             g.tail_u = se == nsl ? u : -1;  // this CTA also streams the unit's tail
             it0 += g.npre;
@@ -313,7 +323,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             const int sb = u == u_first ? t_first : 0;
             const int se = u == u_last ? t_last : nres;
             if (se <= sb) continue;
-            // this CTA's tokens of the unit: [tok_b, tok_e), cut on 16-token slices; 128-token tiles count from tok_b
+            // this CTA's tokens of the unit: [tok_b, tok_e), cut on 16-token slices; tiles count from tok_b
             const int tok_b = sb * kResTile, tok_e = min(se * kResTile, T), rows16 = (se - sb) * kResTile;
             int ntail = 0, n_tail_rows = 0;
             if (sch.any_tail && se == nres) {
@@ -324,7 +334,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             // it from the caller, puts it into the landed tile and stores it to the tail for later calls, so that the tail's
             // copy is requested right behind the dependency wait and no store has to become visible to it.
             const bool append = ntail > 0 && a.k_new && warp == ((n_tail_rows - 1) & (kTT - 1)) >> 4;
-            const int npre = (rows16 + kTT - 1) / kTT, nseg = npre + ntail;
+            const int npre = (rows16 + TT - 1) / TT, nseg = npre + ntail;
             const bool coef = ud.mode != FDKV_MODE_EXACT, resid = ud.mode == FDKV_MODE_RESIDUAL;
             const uint32_t sgn = ud.sign < 0.f ? 0x80008000u : 0u;
 
@@ -340,7 +350,9 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             // ---- residual lists (packed entries): ranges two tiles ahead, entries one tile ahead ----
             const uint32_t* k_ent = reinterpret_cast<const uint32_t*>(ud.k_idx);
             const uint32_t* v_ent = reinterpret_cast<const uint32_t*>(ud.v_idx);
-            int cr[4] = {0, 0, 0, 0}, nr[4] = {0, 0, 0, 0}, fr[4] = {0, 0, 0, 0};  // {k begin, k end, v begin, v end}: this tile, next, the one after
+            constexpr int NR = 2 * (SW + 1);
+            // {bounds of the warp's slices in the K list, the same in the V list}: this tile, next, the one after
+            int cr[NR] = {}, nr[NR] = {}, fr[NR] = {};
             uint32_t pke[kPF], pve[kPF];
             // token-granular residual: one ascending token list (k_idx) with per-slice counts (k_off) for K and V,
             // and the selected tokens' Z1 rows packed densely (k_val / v_val, 256 bytes each)
@@ -348,40 +360,41 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             const uint4* t_krows = reinterpret_cast<const uint4*>(ud.k_val);
             const uint4* t_vrows = reinterpret_cast<const uint4*>(ud.v_val);
             int ptk[2] = {0, 0}, ptv[2] = {0, 0};
-            // List ranges of this warp's slice, one tile per lane: lane l of a batch holds tile rb + l of the segment
-            // ({begin, end} of the K and of the V list), loaded 32 to 64 tiles before use and handed out by shuffle.
-            int rb = 0, rk[2] = {0, 0}, rv[2] = {0, 0}, rk_n[2] = {0, 0}, rv_n[2] = {0, 0};
-            auto load_batch = [&](int jb, int (&k)[2], int (&v)[2]) {
+            // List ranges of this warp's slices, one tile per lane: lane l of a batch holds tile rb + l of the segment, loaded
+            // 32 to 64 tiles before use and handed out by shuffle.
+            int rb = 0, rk[NR] = {}, rk_n[NR] = {};
+            auto load_batch = [&](int jb, int (&k)[NR]) {
                 const int jj = jb + lane;
-                k[0] = k[1] = v[0] = v[1] = 0;
+#pragma unroll
+                for (int i = 0; i < NR; ++i) k[i] = 0;
                 if (resid && jj < npre) {
                     // the tile's slices not yet read: [first, se); the box may start before them (see issue_tile)
-                    const int first = sb + (rev ? npre - 1 - jj : jj) * (kTT / kResTile);
-                    const int o = max(0, min(first, se - kTT / kResTile)) + warp;
-                    const int o0 = min(max(o, first), se), o1 = min(max(o + 1, first), se);
-                    k[0] = ud.k_off[o0]; k[1] = ud.k_off[o1];
-                    if (tokmode) { v[0] = k[0]; v[1] = k[1]; }
-                    else { v[0] = ud.v_off[o0]; v[1] = ud.v_off[o1]; }
+                    const int first = sb + (rev ? npre - 1 - jj : jj) * (TT / kResTile);
+                    const int o = max(0, min(first, se - TT / kResTile)) + SW * warp;
+#pragma unroll
+                    for (int i = 0; i <= SW; ++i) {
+                        const int oi = min(max(o + i, first), se);
+                        k[i] = ud.k_off[oi];
+                        k[SW + 1 + i] = tokmode ? k[i] : ud.v_off[oi];
+                    }
                 }
             };
-            auto get_ranges = [&](int j, int (&r)[4]) {  // rb <= j < rb + 64
+            auto get_ranges = [&](int j, int (&r)[NR]) {  // rb <= j < rb + 64
                 const bool nx = j - rb >= 32;
                 const int src = (j - rb) & 31;
-                r[0] = __shfl_sync(0xFFFFFFFFu, nx ? rk_n[0] : rk[0], src);
-                r[1] = __shfl_sync(0xFFFFFFFFu, nx ? rk_n[1] : rk[1], src);
-                r[2] = __shfl_sync(0xFFFFFFFFu, nx ? rv_n[0] : rv[0], src);
-                r[3] = __shfl_sync(0xFFFFFFFFu, nx ? rv_n[1] : rv[1], src);
+#pragma unroll
+                for (int i = 0; i < NR; ++i) r[i] = __shfl_sync(0xFFFFFFFFu, nx ? rk_n[i] : rk[i], src);
             };
             // pull a tile's list slices (or selected token rows) into L2 a few tiles ahead: lanes 0-15 the K side,
             // lanes 16-31 the V side, one 128-byte line each
-            auto l2_prefetch = [&](const int (&r)[4]) {
+            auto l2_prefetch = [&](const int (&r)[NR]) {
                 const int hl = lane & 15;
                 const void* ptr = nullptr;
                 if (tokmode) {
                     const int j = r[0] + (hl >> 1);
-                    if (j < r[1]) ptr = reinterpret_cast<const char*>(lane < 16 ? t_krows : t_vrows) + (int64_t)j * 256 + (hl & 1) * 128;
+                    if (j < r[SW]) ptr = reinterpret_cast<const char*>(lane < 16 ? t_krows : t_vrows) + (int64_t)j * 256 + (hl & 1) * 128;
                 } else {
-                    const int e0 = lane < 16 ? r[0] : r[2], e1 = lane < 16 ? r[1] : r[3];
+                    const int e0 = lane < 16 ? r[0] : r[SW + 1], e1 = lane < 16 ? r[SW] : r[2 * SW + 1];
                     const int e = (e0 & ~31) + 32 * hl;
                     if (e < e1) ptr = (lane < 16 ? k_ent : v_ent) + e;
                 }
@@ -390,20 +403,29 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             auto prefetch = [&](const uint32_t* ent, int e0, int e1, uint32_t (&pe)[kPF]) {
 #pragma unroll
                 for (int i = 0; i < kPF; ++i) {
+                    if (i == 8 && e0 + 256 >= e1) break;
                     const int e = e0 + lane + 32 * i;
                     if (e < e1) pe[i] = ent[e];
                 }
             };
             // scatter one list slice into the scratch tile: each entry carries its own shared-memory offset
-            auto scatter = [&](const uint32_t* ent, int e0, int e1, const uint32_t (&pe)[kPF]) {
+            // (with two slices per warp, entries from `mid` on belong to the second)
+            auto scatter = [&](const uint32_t* ent, int e0, int mid, int e1, const uint32_t (&pe)[kPF]) {
 #pragma unroll
                 for (int i = 0; i < kPF; ++i) {
+                    if (i == 8 && e0 + 256 >= e1) break;
                     const int e = e0 + lane + 32 * i;
-                    if (e < e1) st_shared_u16(scratch + ((pe[i] >> 16) << 1), (uint16_t)(pe[i] & 0xFFFFu));
+                    if (e < e1) st_shared_u16(scratch + ((pe[i] >> 16) << 1) + (SW == 2 && e >= mid ? kScratchTile : 0), (uint16_t)(pe[i] & 0xFFFFu));
                 }
-                for (int e = e0 + 32 * kPF + lane; e < e1; e += 32) {  // dense slices: direct loads
-                    const uint32_t w = ent[e];
-                    st_shared_u16(scratch + ((w >> 16) << 1), (uint16_t)(w & 0xFFFFu));
+                for (int eb = e0 + 32 * kPF; eb < e1; eb += 128) {  // dense slices: direct loads, four in flight
+                    uint32_t w[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) w[i] = eb + lane + 32 * i < e1 ? ent[eb + lane + 32 * i] : 0u;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int e = eb + lane + 32 * i;
+                        if (e < e1) st_shared_u16(scratch + ((w[i] >> 16) << 1) + (SW == 2 && e >= mid ? kScratchTile : 0), (uint16_t)(w[i] & 0xFFFFu));
+                    }
                 }
             };
             // token rows: two tokens per round (half a warp each, 16 bytes per lane), two rounds in registers
@@ -418,20 +440,20 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                     }
                 }
             };
-            auto scatter_tok = [&](const uint4* rows, int e0, int e1, const uint32_t (&pe)[kPF], const int (&pt)[2]) {
+            auto scatter_tok = [&](const uint4* rows, int e0, int mid, int e1, const uint32_t (&pe)[kPF], const int (&pt)[2]) {
                 const int chunk = lane & 15;
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     const int j = e0 + 2 * r + (lane >> 4);
                     if (j < e1) {
                         const int row = pt[r] & 15;
-                        st_shared_v4(scratch + (chunk >> 3) * 2048 + swz(row, chunk), pe[4 * r], pe[4 * r + 1], pe[4 * r + 2], pe[4 * r + 3]);
+                        st_shared_v4(scratch + (SW == 2 && j >= mid ? kScratchTile : 0) + (chunk >> 3) * 2048 + swz(row, chunk), pe[4 * r], pe[4 * r + 1], pe[4 * r + 2], pe[4 * r + 3]);
                     }
                 }
                 for (int j = e0 + 4 + (lane >> 4); j < e1; j += 2) {  // more than four selected tokens in the slice
                     const int row = (int)k_ent[j] & 15;
                     const uint4 v = rows[(int64_t)j * 16 + chunk];
-                    st_shared_v4(scratch + (chunk >> 3) * 2048 + swz(row, chunk), v.x, v.y, v.z, v.w);
+                    st_shared_v4(scratch + (SW == 2 && j >= mid ? kScratchTile : 0) + (chunk >> 3) * 2048 + swz(row, chunk), v.x, v.y, v.z, v.w);
                 }
             };
             auto zero_scratch = [&]() {
@@ -439,19 +461,19 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                 for (int i = 0; i < kScratchBytes / 16 / 32; ++i) st_shared_zero16(scratch + (lane + 32 * i) * 16);
             };
             if (resid) {
-                load_batch(0, rk, rv);
-                load_batch(32, rk_n, rv_n);
+                load_batch(0, rk);
+                load_batch(32, rk_n);
                 get_ranges(0, cr);
                 get_ranges(1, nr);
                 get_ranges(2, fr);
                 l2_prefetch(nr);
                 l2_prefetch(fr);
                 if (tokmode) {
-                    prefetch_tok(t_krows, cr[0], cr[1], pke, ptk);
-                    prefetch_tok(t_vrows, cr[2], cr[3], pve, ptv);
+                    prefetch_tok(t_krows, cr[0], cr[SW], pke, ptk);
+                    prefetch_tok(t_vrows, cr[SW + 1], cr[2 * SW + 1], pve, ptv);
                 } else {
-                    prefetch(k_ent, cr[0], cr[1], pke);
-                    prefetch(v_ent, cr[2], cr[3], pve);
+                    prefetch(k_ent, cr[0], cr[SW], pke);
+                    prefetch(v_ent, cr[SW + 1], cr[2 * SW + 1], pve);
                 }
             }
 
@@ -504,7 +526,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                     if (old == kCW - 1) {
                         const int jn = j + kStages;
                         if (jn < npre) {
-                            const int tok = max(0, tok_b + min((rev ? npre - 1 - jn : jn) * kTT, rows16 - kTT));
+                            const int tok = max(0, tok_b + min((rev ? npre - 1 - jn : jn) * TT, rows16 - TT));
                             issue_rows(s, unit_kr + tok, unit_vr + tok, true);
                         } else if (it + jn < seg_info[1]) {
                             issue_tile(it + jn);
@@ -537,18 +559,13 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                     }
                 }
             };
-            // (the tile body lives in decode_fast_tile.inc so that it can be instantiated per tile kind without a lambda:
-            // as a generic lambda it cost the bf16 kernel 6 %)
-#define FDKV_TAIL_TILE false
-            for (int j = 0; j < (F8 ? npre : nseg); ++j)
-#include "decode_fast_tile.inc"
-#undef FDKV_TAIL_TILE
+            // (the tile bodies are textual includes: as a generic lambda one cost the bf16 kernel 6 %)
             if constexpr (F8) {
-#define FDKV_TAIL_TILE true
-                for (int j = npre; j < nseg; ++j)
-#include "decode_fast_tile.inc"
-#undef FDKV_TAIL_TILE
+                for (int j = 0; j < npre; ++j)
+#include "decode_fast_tile8.inc"
             }
+            for (int j = F8 ? npre : 0; j < nseg; ++j)
+#include "decode_fast_tile.inc"
             it += nseg;
 
             // ---- merge the eight warps' states into this segment's split-K partial ----
@@ -804,6 +821,9 @@ bool make_rows_tensor_map_u8(void* base, size_t bytes, int box_rows, void* tmap_
     return r == CUDA_SUCCESS;
 }
 
+bool make_arena_tensor_map_u8(void* arena, size_t arena_bytes, void* tmap_out) {
+    return make_rows_tensor_map_u8(arena, arena_bytes, kTT8, tmap_out);
+}
 bool make_arena_tensor_map(void* arena, size_t arena_bytes, void* tmap_out) {
     return make_rows_tensor_map(arena, arena_bytes, kTT, tmap_out);
 }
@@ -829,8 +849,10 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     // tiles scaled by the measured ratio of their compute time to a plain tile's (rc)
     // With whole CTAs per unit (latency-bound regime) a residual tile of the entry form costs a fixed part (the scratch
     // tile and the second products) plus a part per list entry: measured 2.0 plain tiles at 1024 entries per tile and
-    // tensor (keep 1/16), 1.65 at 512 (keep 1/32); with 8-bit rows (a dearer plain tile) about 1.7 at either density.
-    const double res_a = a.rows_f8 ? 1.55 : 1.25;
+    // tensor (keep 1/16), 1.65 at 512 (keep 1/32); with 8-bit rows (a dearer plain tile) about 1.9 at either
+    // density (32k, us a layer with the fixed part at 1.55, 1.65, 1.75, 1.85 and 2.0: keep 1/16 23.2, 22.7, 22.1, 22.0, 22.8, keep 1/32
+    // 21.6, 21.5, 21.3, 21.5, 22.6).
+    const double res_a = a.rows_f8 ? 1.75 : 1.25;
     const double res_b = a.rows_f8 ? 0.15 : 0.87;
     const int ctas = (int)std::min<int64_t>(std::min(std::min(sm_count, kMaxCtas), kMaxSplits), total_tiles);
     auto weigh = [&](double rc) {
@@ -1004,11 +1026,12 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
         cudaError_t e = cudaSuccess;
         auto opt_in = [&](auto kernel, int smem) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         };
-        opt_in(decode_fast_kernel<false, false>, kSmemBytes);
-        opt_in(decode_fast_kernel<true, false>, kSmemBytes);
-        opt_in(decode_fast_kernel<false, true>, kSmemBytesCl);
-        opt_in(decode_fast_kernel<true, true>, kSmemBytesCl);
+        opt_in(decode_fast_kernel<false, false>, smem_of(false, false));
+        opt_in(decode_fast_kernel<true, false>, smem_of(true, false));
+        opt_in(decode_fast_kernel<false, true>, smem_of(false, true));
+        opt_in(decode_fast_kernel<true, true>, smem_of(true, true));
         // the same division of the SM's memory as the decode kernel's, or the two could not share an SM
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -1016,13 +1039,13 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
             cudaLaunchConfig_t q = {};
             q.gridDim = dim3(8 << lg);
             q.blockDim = dim3(kThreads);
-            q.dynamicSmemBytes = kSmemBytesCl;
+            q.dynamicSmemBytes = smem_of(true, true);
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
             at[0].val.clusterDim.x = 1u << lg; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
             q.attrs = at;
             q.numAttrs = 1;
-            e = cudaOccupancyMaxActiveClusters(&max_clusters_of[dev][lg], decode_fast_kernel<false, true>, &q);
+            e = cudaOccupancyMaxActiveClusters(&max_clusters_of[dev][lg], decode_fast_kernel<true, true>, &q);
         }
         return e;
     }, &sm_count);
@@ -1044,7 +1067,7 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ncta);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = sch.cluster ? kSmemBytesCl : kSmemBytes;
+    cfg.dynamicSmemBytes = smem_of(a.rows_f8, sch.cluster > 0);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

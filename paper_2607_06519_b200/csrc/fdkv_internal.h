@@ -321,7 +321,7 @@ cudaError_t plan_decode_host(const DecodeArgs& a, int n_ctas, uint32_t* start_ou
 cudaError_t launch_copy_jobs(const CopyJob* jobs_dev, int njobs, int64_t bytes_max, cudaStream_t st);
 cudaError_t launch_quantise_jobs(const QuantJob* jobs_dev, int njobs, int T_max, cudaStream_t st);
 cudaError_t launch_repack_jobs(const RepackJob* jobs_dev, int njobs, int64_t n_max, cudaStream_t st);
-bool make_rows_tensor_map_u8(void* base, size_t bytes, int box_rows, void* tmap_out);
+bool make_arena_tensor_map_u8(void* arena, size_t arena_bytes, void* tmap_out);
 
 
 // ---- token-granular residual (token_rule.cu) ----
