@@ -24,6 +24,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "fdkv_internal.h"
 #include "mbar_wait.cuh"
@@ -885,11 +886,11 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     sch.units = units;
     sch.cluster = 0;
     // Clusters, as many blocks per unit as fit: one kernel instead of two, where that is worth more than the blocks that are
-    // left out.  The hand-over to the combine kernel and its launch cost as much as kClusterGain plain tiles: a layer call of two
-    // KV heads, 512 tokens, 6.3 -> 5.0 us replayed and 8.2 -> 5.5 issued on a stream, 2k tokens 6.0 -> 6.6 and 8.0 -> 7.3, 8k tokens
-    // (two kernels stay) 8.2 against 14.4.
+    // left out.  The hand-over to the combine kernel and its launch cost as much as kClusterGain plain tiles of one block.  Us a layer
+    // replayed (eight KV heads, clusters of eight), clusters against two kernels: 512 tokens 5.4 and 6.6, 1024 5.7 and 7.0, 1536 6.8
+    // and 7.0, 2047 7.1 and 7.4; with a tail 1024 6.8 and 6.8, 1300 6.8 and 6.9, 2047 8.7 and 8.1, 3000 9.3 and 8.8.
     if (max_clusters) {
-        constexpr double kClusterGain = 2.0;
+        constexpr double kClusterGain = 2.1;
         int least = ns[0];
         for (int u = 1; u < units; ++u) least = std::min(least, ns[u]);
         int lg = 3;
@@ -897,17 +898,33 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
         const int C = 1 << lg;
         if (units <= max_clusters[lg] && units * C <= kMaxCtas) {
             double worst = 0.0, tile = 2 * kTT * 256 / 512, all = 0.0;  // in plain tiles
+            // A block's time is its number of tiles, full or not, and the last block has the tail on top: so the blocks before it
+            // take equal shares, or the next smaller or larger whole number of tiles where that leaves the slowest block with less.
+            // (1024 tokens on eight blocks, eight slices each instead of up to nine: 7.0 -> 5.7 us a layer.)
+            const int tsl = (a.rows_f8 ? kTT8 : kTT) / kResTile;  // slices of a tile
+            std::vector<int> per(units);                          // slices of every block but the last
             for (int u = 0; u < units; ++u) {
-                const double mine = (double)es[u] * wt[u] / (kTT / kResTile) / tile;
-                // (whole tiles per block)
-                worst = std::max(worst, std::ceil((double)es[u] / C / (kTT / kResTile)) * wt[u] / tile);
-                all += mine;
+                const int tail = a.host_tail ? (std::min(a.host_tail[u / a.Hkv], a.max_tail) + kTT - 1) / kTT : 0;
+                const int even = (ns[u] + tail * (kTT / kResTile) + C - 1) / C;
+                // (Latencies of one block: a residual tile is less far above a plain one than in the throughput of a full device, and a
+                // tail tile, whose copy starts after the wait for the kernels ahead, takes half a tile more.)
+                const double rl = std::sqrt(wt[u] / tile), tl = 1.5 * tail;
+                double best = -1.0;
+                for (int p : {even / tsl * tsl, even, (even + tsl - 1) / tsl * tsl}) {
+                    p = std::min(p, C > 1 ? (ns[u] - 1) / (C - 1) : 0);
+                    if (p < (C > 1)) continue;
+                    const int rest = ns[u] - (C - 1) * p;
+                    const double t = std::max((p + tsl - 1) / tsl * rl, (rest + tsl - 1) / tsl * rl + tl);
+                    if (best < 0.0 || t < best) { best = t; per[u] = p; }
+                }
+                worst = std::max(worst, best);
+                all += (double)es[u] * wt[u] / (kTT / kResTile) / tile;
             }
             if (worst <= std::max(1.0, all / ctas) + kClusterGain) {
                 int c = 0;
                 for (int u = 0; u < units; ++u)
                     for (int j = 0; j < C; ++j, ++c) {
-                        sch.start[c] = ((uint32_t)u << 20) | (uint32_t)std::min((int64_t)es[u] * j / C, (int64_t)(ns[u] - (C - j)));
+                        sch.start[c] = ((uint32_t)u << 20) | (uint32_t)(per[u] * j);
                         sch.slot[c] = (uint8_t)j;
                     }
                 sch.start[c] = (uint32_t)units << 20;

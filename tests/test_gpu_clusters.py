@@ -36,3 +36,31 @@ def test_generated_rows(hkv, group, T, n, rows):
                     ref = u.attend(int(modes[0, h]), layer, f32(q)[0][h * group:(h + 1) * group])
                     assert vector_errors(f32(out)[0][h * group:(h + 1) * group], ref).max() <= TOL["bf16"], (step, layer, h)
     assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("rows", [0, 1])
+@pytest.mark.parametrize("hkv,T,tail", [(8, 1024, 0), (8, 1024, 3), (8, 1040, 129), (8, 1025, 1), (8, 1536, 0), (4, 2047, 0), (8, 127, 40), (2, 4096, 0)])
+def test_whole_tiles(hkv, T, tail, rows):
+    """Blocks that take whole tiles, the last one with the remainder and the tail: at and beside whole tiles for eight blocks."""
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=hkv, n_q_heads=hkv * 2, T=T, n_needles=1, W=1, n_steps=max(tail, 1), row_format=rows,
+                                            name="clusters_cut")
+    pf = runner.Prefilled(w, max_tail=max(tail, 1))
+    modes = np.array([[(1 + h) % 3 for h in range(hkv)]])
+    pf.prefill(0, modes)
+    for layer in range(2):
+        for step in range(max(tail, 1)):
+            q = pf.decode_q(layer, step)
+            rows_new = pf.new_rows(layer, step) if tail else (None, None)
+            out = pf.ctx.decode_attn(layer, q, *rows_new)
+        for h in (0, hkv - 1):
+            if rows:
+                u = R8.UnitFp8(*synth.unit_tensor(w, 0, 0, h, False), *synth.unit_tensor(w, 0, 0, h, True), True, w.keep_num, w.keep_den)
+            else:
+                u = oracle_unit(w, 0, 0, h)
+            for step in range(tail):
+                kn, vn = pf.new_rows(layer, step)
+                u.append(layer, f32(kn)[0, h], f32(vn)[0, h])
+            ref = u.attend(int(modes[0, h]), layer, f32(q)[0][h * 2:(h + 1) * 2])
+            assert vector_errors(f32(out)[0][h * 2:(h + 1) * 2], ref).max() <= TOL["bf16"], (layer, h)
+    assert pf.ctx.device_status() == 0
+    pf.ctx.close()
