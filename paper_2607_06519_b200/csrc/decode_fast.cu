@@ -58,8 +58,12 @@ static_assert(kTT == kRowPad, "row blocks are padded to whole stages");
 static_assert(smem_of(false, false) <= 227 * 1024 && smem_of(true, true) <= 227 * 1024, "shared memory budget");
 static_assert(kTT8 * 128 * 2 == kStageBytes, "a stage holds as many bytes in either row format");
 
+// (The host copies a kernel's parameters at every launch: up to kFewSeqs sequences travel in a short list.  6.4 KiB of parameters took
+// 0.7 us longer to issue than 1.5 KiB.)
+constexpr int kFewSeqs = 64;
+template <int NB>
 struct TailLens {
-    int32_t n[kMaxUnits];  // generated tokens in this layer's tail per sequence, this call's append included (host mirror)
+    int32_t n[NB];  // generated tokens in this layer's tail per sequence, this call's append included (host mirror)
 };
 static_assert(kMaxSplits < 256 && kMaxSplits % 32 == 0, "part counts are bytes; the combine holds one part per lane and round");
 
@@ -175,10 +179,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // decode_combine_kernel with at most 48)
 // CL: every unit's thread blocks form a cluster (its dimension is the unit's number of blocks) and join their states through
 // distributed shared memory, so that a call is one kernel: for short contexts, whose cost is the chain of hand-overs.
-template <bool F8, bool CL>
+// NB: room for the tail lengths in the parameters.
+template <bool F8, bool CL, int NB>
 __global__ void __maxnreg__(232)
 decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap8, DecodeArgs a, FastSched sch,
-                   PartCount pc, TailLens tl) {
+                   TailLens<NB> tl) {
     constexpr int kStages = CL || F8 ? 2 : 3, kScratchBytes = F8 ? 2 * kScratchTile : kScratchTile;
     constexpr int TT = F8 ? kTT8 : kTT;   // tokens of a packed tile
     constexpr int SW = TT / 16 / kCW;     // 16-token slices of it per warp
@@ -896,7 +901,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
         int lg = 3;
         while (lg > 0 && (units > max_clusters[lg] || (1 << lg) > least)) --lg;
         const int C = 1 << lg;
-        if (units <= max_clusters[lg] && units * C <= kMaxCtas) {
+        if (units <= max_clusters[lg] && units * C <= kMaxCtas && a.batch <= kFewSeqs) {
             double worst = 0.0, tile = 2 * kTT * 256 / 512, all = 0.0;  // in plain tiles
             // A block's time is its number of tiles, full or not, and the last block has the tail on top: so the blocks before it
             // take equal shares, or the next smaller or larger whole number of tiles where that leaves the slowest block with less.
@@ -1045,10 +1050,12 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         };
-        opt_in(decode_fast_kernel<false, false>, smem_of(false, false));
-        opt_in(decode_fast_kernel<true, false>, smem_of(true, false));
-        opt_in(decode_fast_kernel<false, true>, smem_of(false, true));
-        opt_in(decode_fast_kernel<true, true>, smem_of(true, true));
+        opt_in(decode_fast_kernel<false, false, kFewSeqs>, smem_of(false, false));
+        opt_in(decode_fast_kernel<true, false, kFewSeqs>, smem_of(true, false));
+        opt_in(decode_fast_kernel<false, false, kMaxUnits>, smem_of(false, false));
+        opt_in(decode_fast_kernel<true, false, kMaxUnits>, smem_of(true, false));
+        opt_in(decode_fast_kernel<false, true, kFewSeqs>, smem_of(false, true));
+        opt_in(decode_fast_kernel<true, true, kFewSeqs>, smem_of(true, true));
         // the same division of the SM's memory as the decode kernel's, or the two could not share an SM
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -1062,7 +1069,7 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
             at[0].val.clusterDim.x = 1u << lg; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
             q.attrs = at;
             q.numAttrs = 1;
-            e = cudaOccupancyMaxActiveClusters(&max_clusters_of[dev][lg], decode_fast_kernel<true, true>, &q);
+            e = cudaOccupancyMaxActiveClusters(&max_clusters_of[dev][lg], decode_fast_kernel<true, true, kFewSeqs>, &q);
         }
         return e;
     }, &sm_count);
@@ -1095,11 +1102,14 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     cfg.numAttrs = sch.cluster ? 2 : 1;
     const CUtensorMap& m16 = *reinterpret_cast<const CUtensorMap*>(a.tmap);
     const CUtensorMap& m8 = *reinterpret_cast<const CUtensorMap*>(a.rows_f8 ? a.tmap_u8 : a.tmap);
-    TailLens tl;
-    for (int b = 0; b < a.batch; ++b) tl.n[b] = a.host_tail[b];
-    auto* const kernel = sch.cluster ? (a.rows_f8 ? decode_fast_kernel<true, true> : decode_fast_kernel<false, true>)
-                                     : (a.rows_f8 ? decode_fast_kernel<true, false> : decode_fast_kernel<false, false>);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, cs, tl);
+    auto launch = [&](auto* kernel, auto tl) {
+        for (int b = 0; b < a.batch; ++b) tl.n[b] = a.host_tail[b];
+        return cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, tl);
+    };
+    cudaError_t e;
+    if (sch.cluster) e = launch(a.rows_f8 ? decode_fast_kernel<true, true, kFewSeqs> : decode_fast_kernel<false, true, kFewSeqs>, TailLens<kFewSeqs>());
+    else if (a.batch <= kFewSeqs) e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kFewSeqs> : decode_fast_kernel<false, false, kFewSeqs>, TailLens<kFewSeqs>());
+    else e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kMaxUnits> : decode_fast_kernel<false, false, kMaxUnits>, TailLens<kMaxUnits>());
     if (e != cudaSuccess) return e;
     count_launch(1);
     count_kernel(FDKV_KERNEL_DECODE_FAST);
