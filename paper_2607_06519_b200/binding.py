@@ -48,7 +48,7 @@ def _load():
         "fdkv_compress_prefill": [vp, i32, i32, i32, i32, P(vp), P(vp), i64, i64, vp],
         "fdkv_probe": [vp, i32, i32, i32, P(vp), P(i32), i32, C.c_double, vp, vp, vp],
         "fdkv_set_modes": [vp, i32, P(i32)],
-        "fdkv_route_budget": [vp, i32, sz, P(C.c_double), P(i32), vp],
+        "fdkv_route_budget": [vp, i32, sz, P(C.c_double), vp, vp],
         "fdkv_commit": [vp, i32, vp],
         "fdkv_decode_attn": [vp, i32, i32, vp, vp, vp, vp, i32, vp],
         "fdkv_decode_attn_host": [vp, i32, i32, vp, vp, vp, vp, i32, vp],
@@ -220,13 +220,16 @@ class Context:
     def compress_prefill(self, seq, pair_begin, pair_end, T, k_layers, v_layers, stream=None):
         """k_layers / v_layers: per-layer tensors [T, n_kv_heads, head_dim] (None outside the pair range)."""
         L = self.cfg.n_layers
-        ref = k_layers[2 * pair_begin]
+        layout, dtype = k_layers[2 * pair_begin].stride(), self.tdtype
         kp = (C.c_void_p * L)(*[None if t is None else t.data_ptr() for t in k_layers])
         vp = (C.c_void_p * L)(*[None if t is None else t.data_ptr() for t in v_layers])
-        for t in list(k_layers) + list(v_layers):
-            if t is not None and (t.stride() != ref.stride() or t.dtype != self.tdtype or t.stride(2) != 1):
-                raise ValueError("all K/V layers must share one [T, Hkv, d] strided layout and the context dtype")
-        _check(_lib.fdkv_compress_prefill(self.h, seq, pair_begin, pair_end, T, kp, vp, ref.stride(0), ref.stride(1),
+        for layers in (k_layers, v_layers):
+            for t in layers:
+                if t is not None and (t.stride() != layout or t.dtype is not dtype):
+                    raise ValueError("all K/V layers must share one [T, Hkv, d] strided layout and the context dtype")
+        if layout[2] != 1:
+            raise ValueError("all K/V layers must share one [T, Hkv, d] strided layout and the context dtype")
+        _check(_lib.fdkv_compress_prefill(self.h, seq, pair_begin, pair_end, T, kp, vp, layout[0], layout[1],
                                           _stream(stream)), "fdkv_compress_prefill")
 
     def probe(self, seq, pair_begin, pair_end, q_layers, probe_pos, lam, stream=None):
@@ -253,11 +256,11 @@ class Context:
         """Smallest lambda whose routing fits the byte budget: (fits, lambda, modes int32 [pairs, Hkv]); sets the modes."""
         n = self.n_pairs * self.cfg.n_kv_heads
         lam = C.c_double(0.0)
-        arr = (C.c_int32 * n)()
-        st = _lib.fdkv_route_budget(self.h, seq, int(budget_bytes), C.byref(lam), arr, _stream(stream))
+        modes = torch.zeros(n, dtype=torch.int32)
+        st = _lib.fdkv_route_budget(self.h, seq, int(budget_bytes), C.byref(lam), modes.data_ptr(), _stream(stream))
         if st not in (0, 3):
             raise FdkvError(st, "fdkv_route_budget")
-        return st == 0, float(lam.value), torch.tensor(list(arr), dtype=torch.int32).view(self.n_pairs, -1)
+        return st == 0, float(lam.value), modes.view(self.n_pairs, -1)
 
     def commit(self, seq, stream=None):
         _check(_lib.fdkv_commit(self.h, seq, _stream(stream)), "fdkv_commit")

@@ -3,6 +3,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "fdkv_internal.h"
@@ -152,11 +153,15 @@ struct CopyTable {
         if (bytes) jobs[cls].push_back(CopyJob{(const char*)src, (char*)dst, (int64_t)bytes, 16, 16, add});
     }
     void zero(int cls, void* dst, size_t bytes) { plain(cls, nullptr, dst, bytes); }
-    cudaError_t launch(CopyJob* table_dev, cudaStream_t st) const {
-        std::vector<CopyJob> all;
-        for (const auto& v : jobs) all.insert(all.end(), v.begin(), v.end());
-        if (all.empty()) return cudaSuccess;
-        cudaError_t e = cudaMemcpyAsync(table_dev, all.data(), all.size() * sizeof(CopyJob), cudaMemcpyHostToDevice, st);
+    // `pin`: page-locked room for the whole table, not written again before `st` has been waited for
+    cudaError_t launch(CopyJob* table_dev, CopyJob* pin, cudaStream_t st) const {
+        size_t n = 0;
+        for (const auto& v : jobs) {
+            if (!v.empty()) std::memcpy(pin + n, v.data(), v.size() * sizeof(CopyJob));
+            n += v.size();
+        }
+        if (n == 0) return cudaSuccess;
+        cudaError_t e = cudaMemcpyAsync(table_dev, pin, n * sizeof(CopyJob), cudaMemcpyHostToDevice, st);
         for (const auto& v : jobs) {
             int64_t most = 0;
             for (const CopyJob& jb : v) most = std::max(most, jb.bytes);
@@ -166,6 +171,48 @@ struct CopyTable {
         return e;
     }
 };
+
+// Page-locked blocks of closed contexts, kept for the next ones (page-locking takes 0.14 ms): at most kBlocks of at most kMost
+// bytes each, the rest is freed.  A context gives its block back when no copy from or to it is under way.
+struct PinPool {
+    static constexpr size_t kBlocks = 4, kMost = 1 << 20;
+    std::mutex lock;
+    std::vector<std::pair<size_t, char*>> idle;  // (bytes, block)
+    cudaError_t take(size_t& bytes, char** out) {  // (bytes: in, what is needed; out, what the block has)
+        {
+            std::lock_guard<std::mutex> g(lock);
+            for (size_t i = 0; i < idle.size(); ++i)
+                if (idle[i].first >= bytes) {
+                    bytes = idle[i].first;
+                    *out = idle[i].second;
+                    idle.erase(idle.begin() + i);
+                    return cudaSuccess;
+                }
+        }
+        return cudaHostAlloc(reinterpret_cast<void**>(out), bytes, cudaHostAllocPortable);
+    }
+    void give(size_t bytes, char* block) {
+        {
+            std::lock_guard<std::mutex> g(lock);
+            if (idle.size() < kBlocks && bytes <= kMost) {
+                idle.emplace_back(bytes, block);
+                return;
+            }
+        }
+        cudaFreeHost(block);
+    }
+};
+PinPool& pin_pool() {
+    static PinPool* p = new PinPool;  // (never destroyed: contexts may be closed while the process exits)
+    return *p;
+}
+
+// A sequence's descriptors to the device (the caller waits for `st` before they change again).
+cudaError_t copy_descriptors(fdkv_ctx* c, int seq, cudaStream_t st) {
+    const size_t n = (size_t)c->s.L * c->s.Hkv, bytes = n * sizeof(UnitDesc);
+    std::memcpy(c->pin + c->pin_desc, &c->desc_host[(size_t)seq * n], bytes);
+    return cudaMemcpyAsync(c->arena + c->ar.desc + (size_t)seq * bytes, c->pin + c->pin_desc, bytes, cudaMemcpyHostToDevice, st);
+}
 
 bool seq_ok(fdkv_ctx* c, int seq) { return c && seq >= 0 && seq < c->s.max_batch; }
 
@@ -272,15 +319,21 @@ fdkv_status fdkv_create(const fdkv_config* cfg, void* arena, size_t arena_bytes,
     if (e == cudaSuccess) e = cudaMemset(c->arena + c->ar.desc, 0, c->desc_host.size() * sizeof(UnitDesc));
     // tails start as zero rows: the fast decode kernel loads whole 64-row boxes and relies on finite padding
     if (e == cudaSuccess) e = cudaMemset(c->arena + c->ar.tail_k, 0, c->ar.bump - c->ar.tail_k);
-    if (e != cudaSuccess) { delete c; return cuda_fail(e); }
+    c->pin_jobs = align_up((size_t)s.NU * 16);
+    c->pin_gather = c->pin_jobs + 2 * align_up(max_copy_jobs(s) * sizeof(CopyJob));  // (a fold has two tables on the way)
+    c->pin_desc = c->pin_gather + align_up(gather_table_bytes(s));
+    c->pin_bytes = c->pin_desc + (size_t)s.L * s.Hkv * sizeof(UnitDesc);
+    if (e == cudaSuccess) e = pin_pool().take(c->pin_bytes, &c->pin);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->probe_done, cudaEventDisableTiming);
+    if (e != cudaSuccess) { fdkv_destroy(c); return cuda_fail(e); }
     if (s.dtype == FDKV_BF16 && s.d == 128) c->has_tmap = make_arena_tensor_map(c->arena, arena_bytes, c->tmap);
     c->packed_lists = c->has_tmap && s.max_batch * s.Hkv <= kFastMaxUnits;
-    if (s.rows_f8 && !(c->packed_lists && make_arena_tensor_map_u8(c->arena, arena_bytes, c->tmap_u8))) { delete c; return FDKV_ERR_UNSUPPORTED; }
+    if (s.rows_f8 && !(c->packed_lists && make_arena_tensor_map_u8(c->arena, arena_bytes, c->tmap_u8))) { fdkv_destroy(c); return FDKV_ERR_UNSUPPORTED; }
     // token rule: the tensor-core score kernel and the packed decode kernel serve bf16 / head_dim 128; everything else
     // takes the float32 score kernel and the portable decode kernel
     if (s.tok_rule && c->packed_lists)
         c->tok_tc = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, 128, c->tmap_z1_128);
-    if (s.tok_rule && s.dtype == FDKV_BF16 && s.d == 128 && !c->tok_tc) { delete c; return FDKV_ERR_UNSUPPORTED; }
+    if (s.tok_rule && s.dtype == FDKV_BF16 && s.d == 128 && !c->tok_tc) { fdkv_destroy(c); return FDKV_ERR_UNSUPPORTED; }
     if (s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule)
         c->has_probe_tmaps = make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, 128, c->tmap_z1_128) &&
                              make_rows_tensor_map(c->work + c->ws.z1, (size_t)s.NU * s.NB * s.Tmax * s.d * s.esize, kProbeBoxRows, c->tmap_z1) &&
@@ -289,7 +342,13 @@ fdkv_status fdkv_create(const fdkv_config* cfg, void* arena, size_t arena_bytes,
     return FDKV_OK;
 }
 
-void fdkv_destroy(fdkv_ctx* ctx) { delete ctx; }
+void fdkv_destroy(fdkv_ctx* ctx) {
+    if (!ctx) return;
+    const bool idle = !ctx->probe_recorded || cudaEventSynchronize(ctx->probe_done) == cudaSuccess;  // (scores on their way)
+    if (ctx->probe_done) cudaEventDestroy(ctx->probe_done);
+    if (ctx->pin && idle) pin_pool().give(ctx->pin_bytes, ctx->pin);
+    delete ctx;
+}
 
 fdkv_status fdkv_reset(fdkv_ctx* c) {
     if (!c) return FDKV_ERR_INVALID_ARG;
@@ -441,6 +500,12 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
         for (int p = pb; p < pe; ++p) c->pair_scored[p] = 1;
     }
     CU(launch_probe(a, s.dtype, st));
+    const size_t su = (size_t)a.unit_begin * 16;
+    CU(cudaMemcpyAsync(c->pin + su, c->work + c->ws.scores + su, (size_t)a.unit_count * 16, cudaMemcpyDeviceToHost, st));
+    if (c->probe_recorded && c->probe_stream != st) CU(cudaStreamWaitEvent(st, c->probe_done, 0));
+    CU(cudaEventRecord(c->probe_done, st));
+    c->probe_stream = st;
+    c->probe_recorded = true;
     for (int p = pb; p < pe; ++p) c->pair_probed[p] = 1;
     return FDKV_OK;
 }
@@ -453,8 +518,8 @@ fdkv_status fdkv_route_budget(fdkv_ctx* c, int32_t seq, size_t budget_bytes, dou
     for (int p = 0; p < s.P; ++p)
         if (!c->pair_probed[p]) return FDKV_ERR_STATE;
     CU(cudaStreamSynchronize(S(stream)));
-    std::vector<double> e((size_t)s.NU * 2);
-    CU(cudaMemcpy(e.data(), c->work + c->ws.scores, e.size() * sizeof(double), cudaMemcpyDeviceToHost));
+    CU(cudaEventSynchronize(c->probe_done));  // (probed on another stream)
+    const double* const e = reinterpret_cast<const double*>(c->pin);
     // Omega of the staged sequence, as in fdkv_probe
     const int T = c->staged_T;
     double om[3];
@@ -467,29 +532,37 @@ fdkv_status fdkv_route_budget(fdkv_ctx* c, int32_t seq, size_t budget_bytes, dou
         if (L2 < best) { best = L2; m = 2; }
         return m;
     };
-    // the footprint only changes where two loss lines of a unit cross: try 0 and every crossing, in ascending order
+    // The footprint only changes where two loss lines of a unit cross, and only downwards: the smallest lambda that fits is 0 or
+    // just past a crossing, found by bisection (128 units, 385 crossings: the device waited 0.1 ms for a scan of them).
     std::vector<double> cand;
     cand.reserve((size_t)s.NU * 3 + 1);
     cand.push_back(0.0);
+    auto add = [&](double cv) { if (cv >= 0.0 && !std::isinf(cv)) cand.push_back(cv); };
     for (int u = 0; u < s.NU; ++u) {
-        cand.push_back((e[2 * u] - e[2 * u + 1]) / (om[1] - om[0]));
-        cand.push_back(e[2 * u + 1] / (om[2] - om[1]));
-        cand.push_back(e[2 * u] / (om[2] - om[0]));
+        add((e[2 * u] - e[2 * u + 1]) / (om[1] - om[0]));
+        add(e[2 * u + 1] / (om[2] - om[1]));
+        add(e[2 * u] / (om[2] - om[0]));
     }
     std::sort(cand.begin(), cand.end());
     std::vector<int32_t> modes(s.NU, 0);
-    bool fits = false;
-    double lam_found = INFINITY;
-    for (double cv : cand) {
-        if (!(cv >= 0.0) || std::isinf(cv)) continue;
-        const double lam = cv * (1.0 + std::ldexp(1.0, -40));  // just past the crossing: that unit already took its cheaper mode
+    // (just past a crossing: the unit already took its cheaper mode, 2^-40 being far above the rounding of the losses)
+    auto past = [&](size_t i) { return cand[i] * (1.0 + std::ldexp(1.0, -40)); };
+    auto fits_at = [&](size_t i) {
+        const double lam = past(i);
         double total = 0.0;
         for (int u = 0; u < s.NU; ++u) {
             modes[u] = mode_at(u, lam);
             total += om[modes[u]] * b_ex;
         }
-        if (total <= (double)budget_bytes) { fits = true; lam_found = lam; break; }
+        return total <= (double)budget_bytes;
+    };
+    size_t lo = 0, hi = cand.size();  // [0, lo) do not fit, [hi, end) fit
+    while (lo < hi) {
+        const size_t mid = (lo + hi) / 2;
+        if (fits_at(mid)) hi = mid; else lo = mid + 1;
     }
+    const bool fits = lo < cand.size() && fits_at(lo);  // (leaves the modes of lo)
+    const double lam_found = fits ? past(lo) : INFINITY;
     if (!fits) std::fill(modes.begin(), modes.end(), 0);
     c->seqs[seq].modes = modes;
     c->modes_overridden = true;
@@ -689,10 +762,12 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
     }
     char* const table = c->work + c->ws.jobs + quant_table_bytes(s);
     if (!gjobs.empty()) {
-        CU(cudaMemcpyAsync(table, gjobs.data(), gjobs.size() * sizeof(TokenGatherJob), cudaMemcpyHostToDevice, st));
+        std::memcpy(c->pin + c->pin_gather, gjobs.data(), gjobs.size() * sizeof(TokenGatherJob));
+        CU(cudaMemcpyAsync(table, c->pin + c->pin_gather, gjobs.size() * sizeof(TokenGatherJob), cudaMemcpyHostToDevice, st));
         CU(launch_token_gather_jobs(reinterpret_cast<TokenGatherJob*>(table), (int)gjobs.size(), k_tok, s.d, s.B, s.dtype, st));
     }
-    CU(copies.launch(reinterpret_cast<CopyJob*>(table + gather_table_bytes(s)), st));
+    CU(copy_descriptors(c, seq, st));
+    CU(copies.launch(reinterpret_cast<CopyJob*>(table + gather_table_bytes(s)), reinterpret_cast<CopyJob*>(c->pin + c->pin_jobs), st));
     if (!qjobs.empty()) {
         QuantJob* qd = reinterpret_cast<QuantJob*>(c->work + c->ws.jobs);
         RepackJob* rd = reinterpret_cast<RepackJob*>(qd + (size_t)s.NU * 2 * s.B);
@@ -703,9 +778,6 @@ fdkv_status fdkv_commit(fdkv_ctx* c, int32_t seq, void* stream) {
             CU(launch_repack_jobs(rd, (int)rjobs.size(), s.tok_rule ? k_tok * 32 : k, st));
         }
     }
-    const size_t seq_desc = (size_t)s.L * s.Hkv;
-    CU(cudaMemcpyAsync(c->arena + c->ar.desc + (size_t)seq * seq_desc * sizeof(UnitDesc), &c->desc_host[(size_t)seq * seq_desc],
-                       seq_desc * sizeof(UnitDesc), cudaMemcpyHostToDevice, st));
     CU(cudaStreamSynchronize(st));
     c->bump = o;
     ++c->plan_epoch;
@@ -909,7 +981,7 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
         }
     }
     CopyJob* const table = reinterpret_cast<CopyJob*>(c->work + c->ws.jobs + quant_table_bytes(s) + gather_table_bytes(s));
-    CU(copies.launch(table, st));
+    CU(copies.launch(table, reinterpret_cast<CopyJob*>(c->pin + c->pin_jobs), st));
     // ---- the remaining tail rows move down: through the staging area, as many layers at a time as it holds, where the ranges
     // overlap ----
     if (rest > 0) {
@@ -924,7 +996,8 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
                         moves.plain(0, base + (size_t)n * row_b, rest <= n ? base : tmp, w);
                         if (rest > n) moves.plain(1, tmp, base, w);
                     }
-            CU(moves.launch(table, st));
+            if (l0 > 0) CU(cudaStreamSynchronize(st));  // (the page-locked table is written again)
+            CU(moves.launch(table, reinterpret_cast<CopyJob*>(c->pin + c->pin_jobs + align_up(max_copy_jobs(s) * sizeof(CopyJob))), st));
         }
     }
     CU(launch_set_tail_len(arp<int32_t>(c, c->ar.tail_len), s.L, s.max_batch, seq, rest, st));
@@ -932,8 +1005,7 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
     // ---- descriptors: every layer of the sequence now holds T0 + n prompt-side tokens ----
     const size_t seq_desc = (size_t)s.L * s.Hkv;
     for (size_t i = 0; i < seq_desc; ++i) c->desc_host[(size_t)seq * seq_desc + i].T = T0 + n;
-    CU(cudaMemcpyAsync(c->arena + c->ar.desc + (size_t)seq * seq_desc * sizeof(UnitDesc), &c->desc_host[(size_t)seq * seq_desc],
-                       seq_desc * sizeof(UnitDesc), cudaMemcpyHostToDevice, st));
+    CU(copy_descriptors(c, seq, st));
     CU(cudaStreamSynchronize(st));
     ++c->plan_epoch;
     q.T = T0 + n;

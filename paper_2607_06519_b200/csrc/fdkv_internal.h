@@ -154,6 +154,13 @@ struct fdkv_ctx {
     bool has_probe_tmaps = false;
     alignas(64) unsigned char tmap_z1_128[128];  // staged Z1 with 128-token boxes (token-score and second-moment kernels)
     bool tok_tc = false;                         // token rule served by the tensor-core kernels (bf16, head_dim 128)
+    // Page-locked host memory, so that the tables of a commit or a fold go to the device without being staged by the driver, and
+    // the probe's scores come back behind the probe's kernels instead of in a copy of their own when the budget is solved.
+    char* pin = nullptr;
+    size_t pin_bytes = 0, pin_jobs = 0, pin_gather = 0, pin_desc = 0;  // its size and offsets (the scores come first)
+    cudaEvent_t probe_done = nullptr;                   // the scores of every probe call so far have landed
+    cudaStream_t probe_stream = nullptr;                // where it was recorded last
+    bool probe_recorded = false;
     std::vector<uint8_t> pair_scored;            // token rule: the probe has chosen this pair's token sets
     bool packed_lists = false;              // decode runs the bf16 / head_dim 128 kernel on packed residual entries
     alignas(64) unsigned char tmap_u8[128]; // CUtensorMap of the arena as 128-byte rows (8-bit row streams)
