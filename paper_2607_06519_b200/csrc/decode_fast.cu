@@ -68,7 +68,7 @@ struct TailLens {
 static_assert(kMaxSplits < 256 && kMaxSplits % 32 == 0, "part counts are bytes; the combine holds one part per lane and round");
 
 // header offsets
-constexpr int kOffFull = 0, kOffAbort = 128, kOffM = 256, kOffL = 512, kOffSeg = 1024, kOffSegInfo = 1920,
+constexpr int kOffFull = 0, kOffJoint = 64, kOffAbort = 128, kOffM = 256, kOffL = 512, kOffSeg = 1024, kOffSegInfo = 1920,
               kOffCnt = 1936;
 // one (unit, tile range) segment of a CTA: arena rows of its K / V boxes and tail, first tile, prefill tiles, first
 // index in the CTA's tile sequence, and the sequence / head whose tail it also streams (or -1)
@@ -142,15 +142,15 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t peer_smem(uint32_t addr, int rank) {  // the same shared-memory address in another block of the cluster
     uint32_t r;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_peer(uint32_t addr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
+// two floats into a peer's shared memory; its barrier counts the bytes when they have landed
+__device__ __forceinline__ void st_peer2(uint32_t addr, float x, float y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void st_shared_u16(uint32_t addr, uint16_t v) {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
 }
@@ -201,13 +201,24 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
     // Let the next kernel in the stream start its own prologue as soon as SMs free up (programmatic dependent
     // launch); everything this kernel reads before its own griddepcontrol.wait is static since commit.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if constexpr (CL) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // "running": awaited before the first write to a peer
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(smem0 + kOffFull + 8 * s, 1);
         }
+        if constexpr (CL) {  // counts the bytes of every block's part of this block's share: its channels, a maximum and a sum per head
+            uint32_t rank, nb;
+            asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+            asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nb));
+            const uint32_t share = (uint32_t)a.G * 128 / nb, heads = ((rank + 1) * share - 1) / 128 - rank * share / 128 + 1;
+            mbar_init(smem0 + kOffJoint, 1);
+            mbar_expect_tx(smem0 + kOffJoint, nb * (share * 4 + heads * 8));
+        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if constexpr (CL) {  // awaited before the first write to a peer
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     }
 
     const int cta = blockIdx.x;
@@ -541,28 +552,38 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                 }
             };
             // O[head][channel] into the warp's float scratch: column g plus (G <= 4) its remainder column g + 4, held by the
-            // lane two over.  Rows gid / gid + 8 of an m-tile are channels gid and gid + 8, or (8-bit tiles) 2 gid and
-            // 2 gid + 1, whose code sums are still to be multiplied by the channel's V scale.
+            // lane two over: of two m-tiles such a pair of lanes adds up and stores one each.  Rows gid / gid + 8 of an m-tile are
+            // channels gid and gid + 8, or (8-bit tiles) 2 gid and 2 gid + 1, whose code sums are still to be multiplied by the
+            // channel's V scale.  Channels are stored xor 8 (column / 2 mod 4): the columns of a store lie in different banks.
+            const int ocol = split ? 2 * (tig & 1) : 2 * tig, oswz = (split ? tig & 1 : tig) << 3;
             auto store_o = [&](bool f8_layout, bool accumulate, float f0, float f1) {
-#pragma unroll
-                for (int jm = 0; jm < 8; ++jm) {
-                    float v[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        v[i] = oacc[jm][i];
-                        if (split) v[i] += __shfl_xor_sync(0xFFFFFFFFu, v[i], 2);
+                auto put = [&](int jm, const float (&v)[4]) {
+                    const int ch_a = f8_layout ? 16 * jm + 2 * gid : 16 * jm + gid, ch_b = f8_layout ? ch_a + 1 : ch_a + 8;
+                    const float sa = f8_layout ? ud.v_scale[ch_a] : 1.f, sb = f8_layout ? ud.v_scale[ch_b] : 1.f;
+                    float* p0 = scratch_f + ocol * 128;
+                    float* p1 = p0 + 128;
+                    const int a_ = ch_a ^ oswz, b_ = ch_b ^ oswz;
+                    if (accumulate) {
+                        p0[a_] += v[0] * sa * f0; p1[a_] += v[1] * sa * f1; p0[b_] += v[2] * sb * f0; p1[b_] += v[3] * sb * f1;
+                    } else {
+                        p0[a_] = v[0] * sa; p1[a_] = v[1] * sa; p0[b_] = v[2] * sb; p1[b_] = v[3] * sb;
                     }
-                    if (!split || tig < 2) {
-                        const int ch_a = f8_layout ? 16 * jm + 2 * gid : 16 * jm + gid, ch_b = f8_layout ? ch_a + 1 : ch_a + 8;
-                        const float sa = f8_layout ? ud.v_scale[ch_a] : 1.f, sb = f8_layout ? ud.v_scale[ch_b] : 1.f;
-                        float* p0 = scratch_f + 2 * tig * 128;
-                        float* p1 = p0 + 128;
-                        if (accumulate) {
-                            p0[ch_a] += v[0] * sa * f0; p1[ch_a] += v[1] * sa * f1; p0[ch_b] += v[2] * sb * f0; p1[ch_b] += v[3] * sb * f1;
-                        } else {
-                            p0[ch_a] = v[0] * sa; p1[ch_a] = v[1] * sa; p0[ch_b] = v[2] * sb; p1[ch_b] = v[3] * sb;
+                };
+                if (split) {
+#pragma unroll
+                    for (int jm = 0; jm < 8; jm += 2) {
+                        const bool odd = tig >= 2;
+                        float v[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float other = __shfl_xor_sync(0xFFFFFFFFu, odd ? oacc[jm][i] : oacc[jm + 1][i], 2);
+                            v[i] = (odd ? oacc[jm + 1][i] : oacc[jm][i]) + other;
                         }
+                        put(odd ? jm + 1 : jm, v);
                     }
+                } else {
+#pragma unroll
+                    for (int jm = 0; jm < 8; ++jm) put(jm, oacc[jm]);
                 }
             };
             // (the tile bodies are textual includes: as a generic lambda one cost the bf16 kernel 6 %)
@@ -593,36 +614,17 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                         lq[e] = l_st[e] * f_st[e] + lq[e] * f_tl[e];
                         m_run[e] = M;
                     }
-                    if (!split || tig < 2) {  // the positions this lane wrote at the stash
+                    // (the positions this lane wrote at the stash)
 #pragma unroll
-                        for (int jm = 0; jm < 8; ++jm) {
-                            float* p0 = scratch_f + 2 * tig * 128 + 16 * jm + 2 * gid;
-                            p0[0] *= f_st[0]; p0[1] *= f_st[0]; p0[128] *= f_st[1]; p0[129] *= f_st[1];
-                        }
+                    for (int jm = 0; jm < 8; ++jm) {
+                        if (split && (jm & 1) != (tig >> 1)) continue;
+                        float* p0 = scratch_f + ocol * 128 + ((16 * jm + 2 * gid) ^ oswz);
+                        p0[0] *= f_st[0]; p0[1] *= f_st[0]; p0[128] *= f_st[1]; p0[129] *= f_st[1];
                     }
                     __syncwarp();
                     store_o(false, true, f_tl[0], f_tl[1]);
                 } else {
-                    if constexpr (F8) {
-                        store_o(true, false, 1.f, 1.f);
-                    } else {
-#pragma unroll
-                        for (int jm = 0; jm < 8; ++jm) {
-                            float v[4];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                v[i] = oacc[jm][i];
-                                if (split) v[i] += __shfl_xor_sync(0xFFFFFFFFu, v[i], 2);
-                            }
-                            if (!split || tig < 2) {
-                                const int ch = 16 * jm + gid, col = 2 * tig;
-                                scratch_f[col * 128 + ch] = v[0];
-                                scratch_f[(col + 1) * 128 + ch] = v[1];
-                                scratch_f[col * 128 + ch + 8] = v[2];
-                                scratch_f[(col + 1) * 128 + ch + 8] = v[3];
-                            }
-                        }
-                    }
+                    store_o(F8, false, 1.f, 1.f);
                 }
                 if (gid == 0) {
 #pragma unroll
@@ -630,11 +632,12 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                 }
                 __syncthreads();
                 uint32_t rank = 0, nb = 1, share = 1024;
+                const uint32_t joint0 = smem0 + kHeaderBytes + kStages * kStageBytes + kCW * kScratchBytes;
                 if constexpr (CL) {
                     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
                     asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nb));
                     share = (uint32_t)a.G * 128 / nb;  // outputs of the unit that a block joins
-                    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+                    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // (the peers' barriers are set up)
                 }
                 for (int i = threadIdx.x; i < a.G * 64; i += kThreads) {  // two channels per thread
                     const int g = i >> 6, ch = 2 * (i & 63);
@@ -648,21 +651,17 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                         for (int w = 0; w < kCW; ++w) {
                             const float f = ex2(sm_m[w * 8 + g] - M);
                             L = fmaf(sm_l[w * 8 + g], f, L);
-                            const float2 o = *reinterpret_cast<const float2*>(smem_raw + kHeaderBytes + kStages * kStageBytes + w * kScratchBytes + (g * 128 + ch) * 4);
+                            const float2 o = *reinterpret_cast<const float2*>(smem_raw + kHeaderBytes + kStages * kStageBytes + w * kScratchBytes + (g * 128 + (ch ^ ((g >> 1 & 3) << 3))) * 4);
                             A.x = fmaf(o.x, f, A.x);
                             A.y = fmaf(o.y, f, A.y);
                         }
                     }
                     if constexpr (CL) {
-                        // to the block that joins these channels
-                        const uint32_t o = (uint32_t)(g * 128 + ch), to = o / share;
-                        const uint32_t joint = peer_smem(smem0 + kHeaderBytes + kStages * kStageBytes + kCW * kScratchBytes, (int)to);
-                        st_peer(joint + (rank * share + (o - to * share)) * 4, A.x);
-                        st_peer(joint + (rank * share + (o - to * share) + 1) * 4, A.y);
-                        if (o % share == 0 || ch == 0) {  // (a share starts inside a head or covers whole heads)
-                            st_peer(joint + (1024 + rank * 8 + g) * 4, M);
-                            st_peer(joint + (1024 + 64 + rank * 8 + g) * 4, L);
-                        }
+                        // to the block that joins these channels, counted by its barrier
+                        const uint32_t o = (uint32_t)(g * 128 + ch), to = (uint32_t)(((float)o + 0.5f) * sch.inv_share);
+                        const uint32_t joint = peer_smem(joint0, (int)to), bar = peer_smem(smem0 + kOffJoint, (int)to), at = o - to * share;
+                        st_peer2(joint + (rank * share + at) * 4, A.x, A.y, bar);
+                        if (at == 0 || ch == 0) st_peer2(joint + (1024 + 2 * (rank * 8 + g)) * 4, M, L, bar);  // (a share starts inside a head or covers whole heads)
                     } else {
                         float* part = a.partials + (((int64_t)b * a.Hq + h * a.G + g) * kMaxSplits + slot) * kPartStride;
                         if (ch == 0) { part[0] = M * 0.6931471805599453f; part[1] = L; }  // the combine step works in natural-log units
@@ -670,21 +669,27 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
                     }
                 }
                 if constexpr (CL) {
-                    cluster_barrier();
+                    // All parts of this block's share.  Every block sends its parts whatever happened to its copies, so this wait ends
+                    // when the slowest one is through; no block leaves before, so that nobody writes to one that has left.
+                    if (!mbar_try_wait(smem0 + kOffJoint, 0)) {
+                        uint32_t polls = 0;
+                        while (!mbar_try_wait(smem0 + kOffJoint, 0) && ++polls < 4 * kWaitCap) {}
+                        if (polls >= 4 * kWaitCap) { *abort_flag = 1; atomicMax(a.status, (int32_t)kFlagTimeout); }
+                    }
                     const float* const joint = reinterpret_cast<const float*>(smem_raw + kHeaderBytes + kStages * kStageBytes + kCW * kScratchBytes);
                     for (uint32_t i = threadIdx.x; i < share; i += kThreads) {
                         const uint32_t o = rank * share + i, g = o >> 7;
                         float m[kMaxCluster], M = -INFINITY, L = 0.f, A = 0.f;
 #pragma unroll
                         for (int c = 0; c < kMaxCluster; ++c) {
-                            m[c] = c < (int)nb ? joint[1024 + c * 8 + g] : -INFINITY;
+                            m[c] = c < (int)nb ? joint[1024 + 2 * (c * 8 + g)] : -INFINITY;
                             M = fmaxf(M, m[c]);
                         }
 #pragma unroll
                         for (int c = 0; c < kMaxCluster; ++c)
                             if (c < (int)nb) {
                                 const float f = m[c] == -INFINITY ? 0.f : ex2(m[c] - M);
-                                L = fmaf(joint[1024 + 64 + c * 8 + g], f, L);
+                                L = fmaf(joint[1024 + 2 * (c * 8 + g) + 1], f, L);
                                 A = fmaf(joint[c * share + i], f, A);
                             }
                         const float r = L > 0.f ? A / L : 0.f;
@@ -892,10 +897,12 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     sch.cluster = 0;
     // Clusters, as many blocks per unit as fit: one kernel instead of two, where that is worth more than the blocks that are
     // left out.  The hand-over to the combine kernel and its launch cost as much as kClusterGain plain tiles of one block.  Us a layer
-    // replayed (eight KV heads, clusters of eight), clusters against two kernels: 512 tokens 5.4 and 6.6, 1024 5.7 and 7.0, 1536 6.8
-    // and 7.0, 2047 7.1 and 7.4; with a tail 1024 6.8 and 6.8, 1300 6.8 and 6.9, 2047 8.7 and 8.1, 3000 9.3 and 8.8.
+    // replayed (eight KV heads, clusters of eight), clusters against two kernels: 512 tokens 4.6 and 6.6, 1024 5.0 and 7.0, 2047 6.4
+    // and 7.7, 4096 9.9 and 8.9; with a tail 1024 6.0 and 6.8, 2047 7.7 and 7.9, 3000 9.1 and 8.6.  8-bit rows, whose tails make the
+    // last block later: 1024 6.5 and 8.8, 4096 10.5 and 10.7, 8192 15.2 and 11.5; with a tail 1024 8.5 and 9.1, 3000 9.1 and 9.9,
+    // 4096 13.0 and 11.5.
     if (max_clusters) {
-        constexpr double kClusterGain = 2.1;
+        const double kClusterGain = a.rows_f8 ? 3.0 : 2.1;
         int least = ns[0];
         for (int u = 1; u < units; ++u) least = std::min(least, ns[u]);
         int lg = 3;
@@ -912,8 +919,9 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
                 const int tail = a.host_tail ? (std::min(a.host_tail[u / a.Hkv], a.max_tail) + kTT - 1) / kTT : 0;
                 const int even = (ns[u] + tail * (kTT / kResTile) + C - 1) / C;
                 // (Latencies of one block: a residual tile is less far above a plain one than in the throughput of a full device, and a
-                // tail tile, whose copy starts after the wait for the kernels ahead, takes half a tile more.)
-                const double rl = std::sqrt(wt[u] / tile), tl = 1.5 * tail;
+                // tail tile, whose copy starts after the wait for the kernels ahead, takes half a tile more.  A 256-token tile of
+                // 8-bit rows counts as 1.7 plain ones.)
+                const double rl = std::sqrt(wt[u] / tile) * (a.rows_f8 ? 1.7 : 1.0), tl = 1.5 * tail;
                 double best = -1.0;
                 for (int p : {even / tsl * tsl, even, (even + tsl - 1) / tsl * tsl}) {
                     p = std::min(p, C > 1 ? (ns[u] - 1) / (C - 1) : 0);
@@ -935,6 +943,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
                 sch.start[c] = (uint32_t)units << 20;
                 sch.ncta = c;
                 sch.cluster = C;
+                sch.inv_share = (float)C / (float)(128 * a.G);
                 for (int u = 0; u < kMaxUnits; ++u) cs.n[u] = u < units ? C : 0;
                 return cudaSuccess;
             }
@@ -943,7 +952,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     bool whole = units <= ncta;
     std::vector<int> nc(units, 1);
     if (whole) {
-        // Whole CTAs per unit (no CTA pays a second merge + ticket): shares proportional to the unit's cost, at least
+        // Whole CTAs per unit (no CTA pays a second merge): shares proportional to the unit's cost, at least
         // one each, the remainder to the units with the largest cost per CTA; never more CTAs than tiles.
         int given = units;
         for (int u = 0; u < units; ++u) {

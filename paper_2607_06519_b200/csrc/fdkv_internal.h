@@ -55,6 +55,7 @@ struct FastSched {
     uint8_t slot[kMaxSplits];        // split-K part of CTA c's first unit that CTA c writes (its later units start with it: part 0)
     int ncta, units;
     int cluster;   // thread blocks per unit, one cluster each, in one kernel; 0: the ranges are free and a second kernel combines
+    float inv_share;  // (clusters) 1 / outputs of a unit that one block joins
     int any_tail;  // some sequence of the batch holds generated tokens in this layer's tail (host mirror)
 };
 struct PartCount {
