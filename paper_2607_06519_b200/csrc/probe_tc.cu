@@ -8,9 +8,10 @@
 //     one CTA per item, 6 warps: warp 0 = TMA producer, warp 1 = MMA issuer (and TMEM owner), warps 2-5 = epilogue;
 //   * A (the item's 128 Q rows) is written once into shared memory by the epilogue threads, in the
 //     128-byte-swizzled K-major layout a TMA copy would give it; B tiles (256 tokens x 128 channels, same layout)
-//     stream through a 3-stage TMA ring;
+//     stream through a TMA ring of three stages (one in short items);
 //   * per key tile 8 tcgen05.mma (M = 128, N = 256, K = 16, kind::f16, both operands from shared memory,
 //     bf16 x bf16 -> f32) fill one of two alternating 128 x 256 f32 accumulators: all 512 columns of tensor memory.
+//     (In short items there is one.)
 //     The hand-over of an accumulator (commit -> epilogue -> release -> next MMA) is a round trip of about a
 //     microsecond; with a single set it was paid on every tile and cost as much as the arithmetic, which is why A
 //     lives in shared memory: the columns it took in tensor memory buy the second set.  (Two M tiles against
@@ -31,19 +32,17 @@ namespace {
 
 constexpr int kBN = kProbeBoxRows;             // key tokens per tile (N of the MMA)
 constexpr int kMT = 256 / kBN;                 // M tiles (128 Q rows each) per work item: 2 at N = 128, 1 at N = 256
-constexpr int kBStages = kBN == 128 ? 5 : 3;
-constexpr int kAccSets = 2;
+static_assert(kMT == 1, "one M tile per item");
 constexpr int kBHalf = kBN * 128;              // one 64-channel half of a B tile: 32 KiB
 constexpr int kBStageBytes = 2 * kBHalf;       // 64 KiB
 constexpr int kHdr = 1024;
 constexpr int kAHalf = 128 * 128;              // one 64-channel half of an A tile (128 Q rows): 16 KiB
 constexpr int kABytes = kMT * 2 * kAHalf;      // the item's M tiles
-constexpr int kProbeSmem = kHdr + kABytes + kBStages * kBStageBytes;  // 225 KiB in either form
+constexpr int probe_smem(int stages) { return kHdr + kABytes + stages * kBStageBytes; }  // 225 KiB with three, 97 with one
 constexpr int kPThreads = 6 * 32;
-// Tensor memory (512 columns): two alternating sets of kMT 128 x kBN f32 accumulators (one per M tile).
-constexpr int kTmemCols = 512;
+// Tensor memory (512 columns): alternating sets of kMT 128 x kBN f32 accumulators (one per M tile).
 constexpr int kAccSet = kMT * kBN;
-static_assert(kAccSets * kAccSet <= kTmemCols && (kBN == 128 || kBN == 256), "tensor memory budget");
+static_assert(2 * kAccSet <= 512, "tensor memory budget");
 // header: full[8] @0, empty[8] @64, tfull[2] @128, tempty[2] @144, tmem slot @160, abort @164, reduce @192 (4 doubles)
 constexpr uint32_t kIdesc = umma_idesc(128, kBN, false);
 constexpr int oFull = 0, oEmpty = 64, oTFull = 128, oTEmpty = 144, oSlot = 160, oAbort = 164, oRed = 192;
@@ -57,9 +56,17 @@ struct TcPlan {
     int slot0;        // first part slot
 };
 
-__global__ void __launch_bounds__(kPThreads, 1)
+// kBStages, kAccSets: three and two for items of many tiles; one and one for items of a tile or two, whose time is the chain from
+// the loads to the sum: two such blocks share an SM.  Us a probe of 32 layers, one block against two per SM: 300 tokens (one or
+// two tiles) 87 and 64, 1k (four) 110 and 89, 2k (eight) 143 and 128, 8k by products alone (nine or more) 338 and 363.
+constexpr int kShortItem = 8;
+// 256-key tiles that every query sees up to which the product takes them too (see launch_probe_tc)
+constexpr int kGramTiles = 4;
+template <int kBStages, int kAccSets>
+__global__ void __launch_bounds__(kPThreads, kBStages == 1 ? 2 : 1)
 probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_constant__ CUtensorMap tmap_drop, ProbeArgs a, TcPlan pl) {
     extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr int kTmemCols = kAccSets * kAccSet;
     const uint32_t sm0 = s_u32(smem);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + oAbort);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -87,7 +94,7 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {  // tensor memory: all 512 columns
+    if (warp == 1) {  // tensor memory
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm0 + oSlot), "r"((uint32_t)kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -255,7 +262,10 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     if (dtype != FDKV_BF16 || a.d != 128 || !a.tmap_z1 || !a.tmap_drop) return cudaSuccess;
     static PerDevice once;
     int sm_count = 0;
-    cudaError_t e0 = once.ensure([&]() { return cudaFuncSetAttribute(probe_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kProbeSmem); }, &sm_count);
+    cudaError_t e0 = once.ensure([&]() {
+        const cudaError_t e = cudaFuncSetAttribute(probe_tc_kernel<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, probe_smem(3));
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(probe_tc_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, probe_smem(1));
+    }, &sm_count);
     if (e0 != cudaSuccess) return e0;
     TcPlan pl;
     pl.pos_min = a.pos_host[0];
@@ -265,6 +275,9 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     // copy of Z1 and 2 x 2 x rows x 128 flops here; 32 layers of 32k tokens, 512 rows per pair: 1 190 -> 320 us with this
     // kernel's share of the last keys)
     pl.tile_first = (pl.pos_min + 1) / kBN;
+    // ... from a range on that pays for the fixed part, every unit's queries times its moments (us, 32 layers, product of all
+    // keys against moments: 1k tokens 89 and 100, 2k 128 and 117, 4k 208 and 149; blocks of four 1k 105 and 110, 4k 256 and 175)
+    if (pl.tile_first <= kGramTiles) pl.tile_first = 0;
     pl.slot0 = 0;
     if (pl.tile_first > 0) {
         cudaError_t e = launch_probe_gram(a, pl.tile_first * kBN, st, &pl.slot0);
@@ -285,8 +298,9 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
         const int t0 = pl.tile_first * kBN, t1 = std::min(a.T, pl.ntiles * kBN), n_ops = a.B == 4 ? 4 : 1;
         const int blocks = (int)std::min<int64_t>(64, ((int64_t)(t1 - t0) * 16 + 255) / 256);
         drop_rows_kernel<<<dim3(blocks, a.unit_count, n_ops), 256, 0, st>>>(a, n_ops, t0, t1);
-        probe_tc_kernel<<<a.unit_count * pl.items_per_unit, kPThreads, kProbeSmem, st>>>(
-            *reinterpret_cast<const CUtensorMap*>(a.tmap_z1), *reinterpret_cast<const CUtensorMap*>(a.tmap_drop), a, pl);
+        const CUtensorMap &mz = *reinterpret_cast<const CUtensorMap*>(a.tmap_z1), &md = *reinterpret_cast<const CUtensorMap*>(a.tmap_drop);
+        if (pl.tiles_per_split <= kShortItem) probe_tc_kernel<1, 1><<<a.unit_count * pl.items_per_unit, kPThreads, probe_smem(1), st>>>(mz, md, a, pl);
+        else probe_tc_kernel<3, 2><<<a.unit_count * pl.items_per_unit, kPThreads, probe_smem(3), st>>>(mz, md, a, pl);
         count_launch(2);
     }
     cudaError_t e = cudaGetLastError();

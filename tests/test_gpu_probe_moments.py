@@ -36,3 +36,9 @@ def test_probe_errors(block, hkv, group, T, pos):
                 want = R.probe_error(u.z1["k"], u.kept["k"], pq[0], pq[1], group, h, pos)
             np.testing.assert_allclose(scores[p, h], want, rtol=2e-5)
     assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("hkv,T,pos", [(1, 1300, [1278, 1299]), (1, 1300, [1279, 1299]), (150, 2048, [5, 2047]), (150, 2049, [5, 2048])])
+def test_products_of_short_prompts_and_items(hkv, T, pos):
+    """The most keys that go to the products although every query sees them, and one tile more; items of eight tiles and of nine."""
+    test_probe_errors(2, hkv, 1, T, pos)
