@@ -17,6 +17,7 @@
 //                        memory), then the keys above and equal to it before every chunk;
 //   4. compact_kernel    one block per chunk: candidates -> the lists, the offsets of the 16-token tiles and, of K, a bit
 //                        map of the kept positions.
+// (Few short unit-tensors take small_kernel instead of all of these.)
 // The bound is only a guess: where fewer than k positions reach it, step 3 says so and steps 2 and 3 run again for that
 // unit-tensor with bound 0 (a chunk's list holds all of its positions), so the result never depends on the sample.
 // Bound by HBM: K and V are read once and about k / N x 1.2 of them written again; a pass that writes all high-frequency
@@ -661,18 +662,220 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
     }
 }
 
+// ---- all of it for a short unit-tensor ------------------------------------------------------------------
+// One cluster per unit-tensor, a range of whole 16-token tiles per block, at most kSmallElems positions: the high-frequency
+// values stay in shared memory, the threshold is a radix select over histograms that every block adds up from the cluster's
+// shared memories (11, 10 and 10 bits of the key; a bf16 pair's has no more than 15), and a thread writes the entries of its 32
+// consecutive positions.  Bound by the chain of its steps (loads, five cluster barriers with reads across the cluster between, block
+// scans), not by bytes: one bf16 pair of 509 x 128 24.5 -> 11.7 us against the four kernels, 1000 x 128 32.8 -> 12.9, eight of
+// 900 x 128 47.9 -> 26.6.  Only while every cluster runs at once: 256 pairs of 1024 x 128, seven turns, 195 us against 133.
+constexpr int kSmallThreads = 512, kSmallElems = 32 * kSmallThreads, kSmallSmem = 128 * 1024;
+
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the sum over the cluster of two consecutive 32-bit words at a shared-memory address, all loads in flight together
+__device__ __forceinline__ uint2 cluster_sum2(uint32_t addr, int blocks) {
+    uint2 v[8], sum = make_uint2(0, 0);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        uint32_t at;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(r < blocks ? r : 0));
+        asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v[r].x), "=r"(v[r].y) : "r"(at));
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+        if (r < blocks) { sum.x += v[r].x; sum.y += v[r].y; }
+    return sum;
+}
+
+template <typename T, int B>
+__global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a, int blocks, int range) {
+    constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
+    constexpr bool TWO = sizeof(T) == 2 && B == 2;  // (the key's lower 16 bits are zero)
+    constexpr int CH = 4 * Q;                       // 16-byte chunks of 32 positions
+    extern __shared__ __align__(16) uint8_t smem[];  // [NB][range] values, the chunks of a word of 32 positions swizzled
+    __shared__ __align__(16) uint32_t s_h1[2048], s_h2[TWO ? 1024 : 2048], s_all[2048];
+    __shared__ uint32_t s_count, s_warp[kSmallThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x % blocks, item = blockIdx.x / blocks, uts = a.Hkv * a.tensors;
+    const int ut = a.ut_base + item, blk = item / uts, u = item % uts, h = u / a.tensors, is_v = u % a.tensors;
+    const int n_e = a.T * a.d, e0 = rank * range, n = max(0, min(range, n_e - e0));
+    const int dshift = a.d == 128 ? 7 : 6;
+    const int plane = range * (int)sizeof(T);
+    for (int i = tid; i < 2048; i += kSmallThreads) {
+        s_h1[i] = 0;
+        if (i < (TWO ? 1024 : 2048)) s_h2[i] = 0;
+    }
+    auto chunk_at = [&](int word, int j) { return (word * CH + (j ^ (Q == 1 ? (word >> 1) & 3 : word & 7))) * 16; };
+    chain_wait();
+    __syncthreads();
+    const T* x[B];
+#pragma unroll
+    for (int l = 0; l < B; ++l) x[l] = reinterpret_cast<const T*>(is_v ? a.v[B * blk + l] : a.k[B * blk + l]) + (int64_t)h * a.stride_h;
+    T* const z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride + e0;
+    T* const z1 = a.z1 && !is_v ? reinterpret_cast<T*>(a.z1) + (int64_t)(ut / a.tensors) * NB * a.unit_stride + e0 : nullptr;
+    constexpr int U = B == 4 ? 1 : 2;  // groups of eight whose rows are requested together
+    for (int v0 = tid; v0 < n / 8; v0 += U * kSmallThreads) {
+        uint4 f[U][B][Q];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int p = (v0 + q * kSmallThreads) * 8;
+            if (p >= n) break;
+            const int64_t off = (int64_t)((e0 + p) >> dshift) * a.stride_t + ((e0 + p) & (a.d - 1));
+#pragma unroll
+            for (int l = 0; l < B; ++l)
+#pragma unroll
+                for (int k = 0; k < Q; ++k) f[q][l][k] = reinterpret_cast<const uint4*>(x[l] + off)[k];
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int p = (v0 + q * kSmallThreads) * 8;
+            if (p >= n) break;
+            uint4 z[Q], hf[NB][Q];
+            Eight<T, B>::split(f[q], z, hf);
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                reinterpret_cast<uint4*>(z0 + p)[k] = z[k];
+#pragma unroll
+                for (int l = 0; l < NB; ++l) {
+                    if (z1) reinterpret_cast<uint4*>(z1 + (int64_t)l * a.unit_stride + p)[k] = hf[l][k];
+                    *reinterpret_cast<uint4*>(smem + l * plane + chunk_at(p >> 5, ((p >> 3) & 3) * Q + k)) = hf[l][k];
+                }
+            }
+            Eight<T, B>::keys(hf, [&](int, uint32_t key) { atomicAdd(&s_h1[key >> 20], 1u); });
+        }
+    }
+    // f(i, key) for the thread's 32 positions, which are all there or none of them
+    const bool mine = 32 * tid < n;
+    auto each = [&](auto&& f) {
+        if (!mine) return;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            uint4 hf[NB][Q];
+#pragma unroll
+            for (int l = 0; l < NB; ++l)
+#pragma unroll
+                for (int k = 0; k < Q; ++k) hf[l][k] = *reinterpret_cast<const uint4*>(smem + l * plane + chunk_at(tid, g * Q + k));
+            Eight<T, B>::keys(hf, [&](int i, uint32_t key) { f(8 * g + i, key); });
+        }
+    };
+    // ---- the n_keep-th largest key of the cluster ----
+    uint32_t tau = kNoKey, need = 0;
+    cluster_sync();
+    if (a.n_keep > 0) {  // (the same for every block)
+        uint32_t bin, above, left = (uint32_t)a.n_keep;
+        {
+            const uint32_t at = (uint32_t)__cvta_generic_to_shared(s_h1) + 8 * tid;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) *reinterpret_cast<uint2*>(&s_all[1024 * i + 2 * tid]) = cluster_sum2(at + 4096 * i, blocks);
+        }
+        __syncthreads();
+        find_bin<kSmallThreads, 2048>(s_all, left, bin, above);
+        left -= above;
+        tau = bin;
+        auto level = [&](uint32_t* hist, int shift) {
+            each([&](int, uint32_t key) { if (key >> (shift + 10) == tau) atomicAdd(&hist[key >> shift & 1023u], 1u); });
+            cluster_sync();
+            *reinterpret_cast<uint2*>(&s_all[2 * tid]) = cluster_sum2((uint32_t)__cvta_generic_to_shared(hist) + 8 * tid, blocks);
+            __syncthreads();
+            find_bin<kSmallThreads, 1024>(s_all, left, bin, above);
+            left -= above;
+            tau = tau << 10 | bin;
+        };
+        level(s_h2, 10);
+        if constexpr (TWO) tau <<= 10;
+        else level(s_h2 + 1024, 0);
+        need = left;  // of the positions whose key is tau, the lowest
+    }
+    // ---- entries: those above in the blocks, warps and threads before, then those equal (counts in halves: at most 2^14) ----
+    uint32_t gt = 0, eq = 0;
+    each([&](int i, uint32_t key) {
+        gt |= (uint32_t)(key > tau) << i;
+        eq |= (uint32_t)(key == tau) << i;
+    });
+    const uint32_t cnt = (uint32_t)__popc(gt) << 16 | (uint32_t)__popc(eq);
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t before = incl - cnt, total = 0;
+#pragma unroll
+    for (int w = 0; w < kSmallThreads / 32; ++w) {
+        if (w < warp) before += s_warp[w];
+        total += s_warp[w];
+    }
+    if (tid == 0) s_count = total;
+    cluster_sync();
+    uint32_t run_gt = before >> 16, run_eq = before & 0xFFFFu;
+    {
+        uint32_t at, v;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_count)), "r"(lane < rank ? lane : rank));
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+        if (lane >= rank) v = 0;
+        run_gt += __reduce_add_sync(0xFFFFFFFFu, v >> 16);
+        run_eq += __reduce_add_sync(0xFFFFFFFFu, v & 0xFFFFu);
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // (nothing is read from another block after this)
+    int32_t* const idx = a.idx + (int64_t)ut * a.kcap;
+    T* const out = reinterpret_cast<T*>(a.val) + (int64_t)ut * NB * a.kcap;
+    uint32_t* const packed = sizeof(T) == 2 && a.packed ? a.packed + (int64_t)ut * NB * a.kcap : nullptr;
+    const int tile_words = kResTile * a.d / 32;
+    int32_t* const off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1);
+    if (mine) {
+        if (tid % tile_words == 0) off[(e0 / 32 + tid) / tile_words] = (int32_t)(run_gt + min(run_eq, need));
+        // the ties that are kept: while fewer than `need` precede them
+        const int ties = (int)min((uint32_t)__popc(eq), need - min(run_eq, need));
+        uint32_t kept = gt, rest = eq;
+        for (int i = 0; i < ties; ++i) {
+            kept |= rest & (0u - rest);
+            rest &= rest - 1;
+        }
+        uint32_t at = run_gt + min(run_eq, need);
+        if (a.keep && !is_v) a.keep[(int64_t)(ut / a.tensors) * a.keep_stride + e0 / 32 + tid] = kept;
+        for (uint32_t bits = kept; bits; bits &= bits - 1, ++at) {
+            const int i = __ffs((int)bits) - 1, p = 32 * tid + i;
+            idx[at] = e0 + p;
+            const uint32_t place = sizeof(T) == 2 ? packed_place((uint32_t)p) : 0u;
+            constexpr int PER = 16 / (int)sizeof(T);
+            const int from = chunk_at(tid, i / PER) + (i % PER) * (int)sizeof(T);
+#pragma unroll
+            for (int l = 0; l < NB; ++l) {
+                const T raw = *reinterpret_cast<const T*>(smem + l * plane + from);
+                out[(int64_t)l * a.kcap + at] = raw;
+                // (a block of four scales its rows by 1/2 at decode time and its deviations by 1: twice the deviation is stored)
+                if constexpr (sizeof(T) == 2)
+                    if (packed) packed[(int64_t)l * a.kcap + at] = (__float_as_uint(B == 4 ? 2.f * to_f32(raw) : to_f32(raw)) >> 16) | place;
+            }
+        }
+        if (e0 + 32 * (tid + 1) == n_e) {  // the last positions of all
+            off[(n_e / 32 + tile_words - 1) / tile_words] = (int32_t)at;
+            if ((int64_t)at != a.n_keep) atomicMax(a.status, (int32_t)kFlagCountMismatch);
+        }
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <typename... A>
-cudaError_t launch_chain(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+cudaError_t launch_chain(int cluster, void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster ? 2 : 1;
     count_launch(1);
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
@@ -683,11 +886,34 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     int sms = 0;
     constexpr int CE = compress_chunk(B, (int)sizeof(T));
     const size_t smem = 2 * (size_t)B * CE * sizeof(T);
-    cudaError_t e = once.ensure([&]() { return cudaFuncSetAttribute(split_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); }, &sms);
+    cudaError_t e = once.ensure([&]() {
+        const cudaError_t e1 = cudaFuncSetAttribute(split_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return e1 != cudaSuccess ? e1 : cudaFuncSetAttribute(small_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+    }, &sms);
     if (e != cudaSuccess) return e;
     const int64_t n = (int64_t)a.T * a.d;
     a.chunks = (int)((n + CE - 1) / CE);
-    const int uts = a.Hkv * a.tensors, ut_begin = block_begin * uts, ut_count = (block_end - block_begin) * uts;
+    // few short unit-tensors: a cluster each, of as many blocks as have a tile, two blocks per SM
+    const int tile_e = kResTile * a.d;
+    const int64_t tiles = (n + tile_e - 1) / tile_e;
+    int cluster = 8;
+    while (cluster > tiles) cluster /= 2;
+    const int64_t range = (tiles + cluster - 1) / cluster * tile_e;
+    const size_t small_smem = (size_t)range * (B == 4 ? 4 : 1) * sizeof(T);
+    const int uts = a.Hkv * a.tensors;
+    if (range <= kSmallElems && small_smem <= (size_t)kSmallSmem && (int64_t)cluster * uts * (block_end - block_begin) <= 2 * sms) {
+        for (int b0 = block_begin; b0 < block_end; b0 += kSplitLayers / B) {
+            const int nb = std::min(block_end - b0, kSplitLayers / B);
+            for (int l = 0; l < nb * B; ++l) {
+                a.k[l] = k_layers[B * b0 + l];
+                a.v[l] = v_layers[B * b0 + l];
+            }
+            a.ut_base = b0 * uts;
+            if ((e = launch_chain(cluster, small_kernel<T, B>, dim3(cluster * uts * nb), kSmallThreads, small_smem, st, a, cluster, (int)range)) != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+    const int ut_begin = block_begin * uts, ut_count = (block_end - block_begin) * uts;
     // about 1.2 k candidates (and four standard deviations of a small sample on top); a sample of everything is exact
     const int n_rows = (int)std::min<int64_t>(a.T, std::max<int64_t>(1, kSampleElems / a.d));
     const bool exact = n_rows == a.T;
@@ -703,13 +929,13 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
                 a.v[l] = v_layers[B * b0 + l];
             }
             a.ut_base = b0 * uts;
-            if (!redo && (e = launch_chain(sample_kernel<T, B>, dim3(uts, nb), kSampleThreads, 0, st, a, n_rows, target)) != cudaSuccess) return e;
+            if (!redo && (e = launch_chain(0, sample_kernel<T, B>, dim3(uts, nb), kSampleThreads, 0, st, a, n_rows, target)) != cudaSuccess) return e;
             const int items = a.chunks * uts * nb;
-            if ((e = launch_chain(split_kernel<T, B>, dim3(std::min(items, 3 * sms)), kSplitThreads, smem, st, a, items, redo)) != cudaSuccess) return e;
+            if ((e = launch_chain(0, split_kernel<T, B>, dim3(std::min(items, 3 * sms)), kSplitThreads, smem, st, a, items, redo)) != cudaSuccess) return e;
         }
-        if ((e = launch_chain(threshold_kernel<T, B>, dim3(ut_count), kThrThreads, 0, st, a, ut_begin, redo)) != cudaSuccess) return e;
+        if ((e = launch_chain(0, threshold_kernel<T, B>, dim3(ut_count), kThrThreads, 0, st, a, ut_begin, redo)) != cudaSuccess) return e;
     }
-    return launch_chain(compact_kernel<T, B>, dim3((a.chunks + 7) / 8, ut_count), 256, 0, st, a, ut_begin);
+    return launch_chain(0, compact_kernel<T, B>, dim3((a.chunks + 7) / 8, ut_count), 256, 0, st, a, ut_begin);
 }
 
 }  // namespace

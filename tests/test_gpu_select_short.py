@@ -1,0 +1,65 @@
+"""Few short unit-tensors, one cluster each: the edges of its tiles, blocks and 32-position words, every key equal, everything and
+nothing kept; and as many of the same lengths that the four kernels of longer ones take them."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import check_compression
+from oracle import fdkv_ref as R
+from oracle import fdkv_ref_b4 as R4
+from paper_2607_06519_b200 import binding as B
+from paper_2607_06519_b200 import runner, synth
+
+pytestmark = pytest.mark.gpu
+
+
+LENGTHS = [(1, 2), (15, 3), (16, 16), (17, 5), (113, 8), (128, 8), (129, 8), (1008, 16), (1024, 16), (1025, 16), (2048, 16), (2049, 16)]
+
+
+@pytest.mark.parametrize("hkv,T,den", [(1, *x) for x in LENGTHS] + [(40, *x) for x in LENGTHS if x[0] < 200])
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("bf16", 64), ("f32", 128), ("f32", 64)])
+def test_lengths(dtype, d, hkv, T, den):
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=hkv, n_q_heads=hkv, head_dim=d, T=T, dtype=dtype, n_needles=min(T, 2), W=1,
+                                            keep_num=1, keep_den=den, name="short")
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    for h in {0, hkv - 1}:
+        check_compression(pf.ctx, w, 0, 0, h)
+    assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("keep", [(0, 1), (1, 1), (1, 3), (2, 3)])
+@pytest.mark.parametrize("equal", [True, False])
+def test_ties_and_extremes(dtype, keep, equal):
+    """Keys of one or of three values, so that ties go on over blocks and words."""
+    T, d = 500, 128
+    rng = np.random.default_rng(3)
+    diff = np.ones((T, d), np.float32) if equal else rng.integers(-1, 2, (T, d)).astype(np.float32)
+    base = rng.integers(-4, 5, (T, d)).astype(np.float32)
+    x0, x1 = (torch.from_numpy(a).cuda().to(dtype) for a in (base + diff, base - diff))
+    k = T * d * keep[0] // keep[1]
+    z0, idx, val = torch.empty((T, d), dtype=dtype, device="cuda"), torch.full((max(k, 4),), -1, dtype=torch.int32, device="cuda"), torch.empty(max(k, 4), dtype=dtype, device="cuda")
+    assert B.compress_unit_noalloc(x0, x1, *keep, z0, idx[:k] if k else idx, val[:k] if k else val) == k
+    torch.cuda.synchronize()
+    want_z0, z1 = R.depth_split(x0.float().cpu().numpy(), x1.float().cpu().numpy(), dtype == torch.bfloat16)
+    want = R.select_entries(z1, k)
+    assert np.array_equal(z0.float().cpu().numpy(), want_z0)
+    assert np.array_equal(idx[:k].cpu().numpy(), want)
+    assert np.array_equal(val[:k].float().cpu().numpy(), z1.ravel()[want])
+
+
+@pytest.mark.parametrize("T", [16, 100, 509, 512, 513])
+def test_blocks_of_four(T):
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=4, n_kv_heads=2, n_q_heads=4, T=T, n_needles=2, W=1, keep_num=1, keep_den=9, block_size=4,
+                                            name="short4")
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    for h in range(2):
+        for is_v, name in ((0, "k"), (1, "v")):
+            u = R4.Unit4(synth.block_tensor(w, 0, 0, h, False), synth.block_tensor(w, 0, 0, h, True), True, 1, 9)
+            idx, val = pf.ctx.get_residual(0, 0, h, is_v)
+            assert np.array_equal(idx.cpu().numpy(), u.kept[name])
+            want = np.stack([u.dev[name][l].ravel()[u.kept[name]] for l in range(4)])
+            assert np.array_equal(val.float().cpu().numpy(), want)
+    assert pf.ctx.device_status() == 0
