@@ -7,24 +7,27 @@ namespace fdkv {
 
 namespace {
 
-template <typename T>
-__device__ __forceinline__ float ldf(const T* p);
-template <>
-__device__ __forceinline__ float ldf<float>(const float* p) { return *p; }
-template <>
-__device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
+    const uint2 w = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
+}
 
-constexpr int kRowsBlk = 16;
+constexpr int kRowsBlk = 32, kProbeThreads = 512, kProbePad = 4;
+constexpr size_t probe_tile_smem(int d) { return (size_t)(2 * kProbeTile * (d + kProbePad) + 2 * kRowsBlk * d) * sizeof(float); }
 
-// grid (probe tiles, units).  Each CTA: 64 tokens of one unit, all 2*G*W probe rows, both candidates.
+// grid (probe tiles, units).  Each CTA: 64 tokens of one unit, all 2*G*W probe rows, both candidates; a thread has one token and
+// four of 32 rows, whose values the next turn's loads replace in the other half of the buffer.  Four channels per shared-memory
+// load: 6 loads for 32 multiply-adds (with one channel per load, 16 rows and the loads between two barriers: 4k tokens of four
+// layers, two heads, head_dim 64, 58 -> 19 us).
 template <typename T>
-__global__ void __launch_bounds__(256) probe_tile_kernel(ProbeArgs a) {
-    extern __shared__ float smem[];
-    const int d = a.d, ld = d + 1;
-    float* full = smem;                      // [64][d+1]  Z1 of K: what the shared candidate drops
-    float* drop = full + kProbeTile * ld;    // [64][d+1]  Z1 of K minus the kept entries: what residual drops
-    float* qs = drop + kProbeTile * ld;      // [16][d]
-    __shared__ double s_red[2][8];
+__global__ void __launch_bounds__(kProbeThreads) probe_tile_kernel(ProbeArgs a) {
+    extern __shared__ __align__(16) float smem[];
+    const int d = a.d, ld = d + kProbePad, d4 = d / 4, s4 = d == 128 ? 5 : 4;
+    float* full = smem;                      // [64][d+4]  Z1 of K: what the shared candidate drops
+    float* drop = full + kProbeTile * ld;    // [64][d+4]  Z1 of K minus the kept entries: what residual drops
+    float* qs = drop + kProbeTile * ld;      // [2][32][d]
+    __shared__ double s_red[2][kProbeThreads / 32];
 
     const int unit = a.unit_begin + blockIdx.y;
     const int t0 = blockIdx.x * kProbeTile;
@@ -33,54 +36,68 @@ __global__ void __launch_bounds__(256) probe_tile_kernel(ProbeArgs a) {
     const int ut = unit * 2;  // K
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j = (warp & 1) * 32 + lane;  // token within the tile
-    const int rg = warp >> 1;              // 4 row groups
+    const int rg = warp >> 1;              // 8 groups of 4 rows
     // A pair has one high-frequency operand (Z1) that both layers' queries see; a block of four layers has one
     // operand per layer (its deviation from the block mean), seen by that layer's queries only.
     const int n_ops = a.B == 4 ? 4 : 1;
     const int M = (a.B == 4 ? 1 : 2) * a.G * a.W;  // probe rows per operand
     float sum_f = 0.f, sum_d = 0.f;
     for (int op = 0; op < n_ops; ++op) {
+        // 32 probe rows from rb on: row r = (layer*G + g)*W + qi  ->  Q[layer][qi][h*G + g][:], this thread's 16-byte vectors
+        constexpr int QV = kRowsBlk * 32 / kProbeThreads;  // (head_dim 64 has half of them)
+        float4 qv[QV];
+        auto load_q = [&](int rb) {
+#pragma unroll
+            for (int q = 0; q < QV; ++q) {
+                const int i = threadIdx.x + q * kProbeThreads, r = rb + (i >> s4), c = (i & (d4 - 1)) * 4;
+                qv[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (i < kRowsBlk * d4 && r < M) {
+                    const int layer = a.B == 4 ? op : r / (a.G * a.W), g = (r / a.W) % a.G, qi = r % a.W;
+                    qv[q] = ld4(reinterpret_cast<const T*>(a.q_layers_dev[a.B * pair + layer]) + ((int64_t)qi * a.Hq + h * a.G + g) * d + c);
+                }
+            }
+        };
+        auto store_q = [&](int half) {
+#pragma unroll
+            for (int q = 0; q < QV; ++q) {
+                const int i = threadIdx.x + q * kProbeThreads;
+                if (i < kRowsBlk * d4) *reinterpret_cast<float4*>(qs + half * kRowsBlk * d + 4 * i) = qv[q];
+            }
+        };
+        load_q(0);
         const T* z1 = reinterpret_cast<const T*>(a.z1) + ((int64_t)unit * n_ops + op) * a.unit_stride + (int64_t)t0 * d;
-        for (int i = threadIdx.x; i < kProbeTile * d; i += blockDim.x) {
-            const int t = i / d, c = i % d;
-            const float v = t < nt ? ldf<T>(z1 + i) : 0.f;
-            full[t * ld + c] = v;
-            drop[t * ld + c] = v;
+        for (int i = threadIdx.x; i < kProbeTile * d4; i += kProbeThreads) {
+            const int t = i >> s4, c = (i & (d4 - 1)) * 4;
+            const float4 v = t < nt ? ld4(z1 + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            *reinterpret_cast<float4*>(full + t * ld + c) = v;
+            *reinterpret_cast<float4*>(drop + t * ld + c) = v;
         }
+        store_q(0);
         __syncthreads();
         const int32_t* off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1);
         const int ntiles = (a.T + kResTile - 1) / kResTile;
         const int j0 = t0 / kResTile, j1 = min(ntiles, (t0 + kProbeTile) / kResTile);
         const int32_t* idx = a.idx + (int64_t)ut * a.kcap;
-        for (int e = off[j0] + threadIdx.x; e < off[j1]; e += blockDim.x) {
+        for (int e = off[j0] + threadIdx.x; e < off[j1]; e += kProbeThreads) {
             const int f = idx[e] - t0 * d;
-            drop[(f / d) * ld + (f % d)] = 0.f;
+            drop[(f >> (s4 + 2)) * ld + (f & (d - 1))] = 0.f;
         }
         __syncthreads();
-        for (int rb = 0; rb < M; rb += kRowsBlk) {
-            // stage 16 probe rows: row r = (layer*G + g)*W + qi  ->  Q[layer][qi][h*G + g][:]
-            for (int i = threadIdx.x; i < kRowsBlk * d; i += blockDim.x) {
-                const int r = rb + i / d, c = i % d;
-                float v = 0.f;
-                if (r < M) {
-                    const int layer = a.B == 4 ? op : r / (a.G * a.W), g = (r / a.W) % a.G, qi = r % a.W;
-                    const T* q = reinterpret_cast<const T*>(a.q_layers_dev[a.B * pair + layer]);
-                    v = ldf<T>(q + ((int64_t)qi * a.Hq + h * a.G + g) * d + c);
-                }
-                qs[i] = v;
-            }
-            __syncthreads();
+        for (int rb = 0, half = 0; rb < M; rb += kRowsBlk, half ^= 1) {
+            const bool more = rb + kRowsBlk < M;
+            if (more) load_q(rb + kRowsBlk);
             float af[4] = {0.f, 0.f, 0.f, 0.f}, ad[4] = {0.f, 0.f, 0.f, 0.f};
             const float* zf = full + j * ld;
             const float* zd = drop + j * ld;
-            const float* qr = qs + rg * 4 * d;
-            for (int c = 0; c < d; ++c) {
-                const float vf = zf[c], vd = zd[c];
+            const float* qr = qs + half * kRowsBlk * d + rg * 4 * d;
+#pragma unroll 4
+            for (int c = 0; c < d; c += 4) {
+                const float4 vf = ld4(zf + c), vd = ld4(zd + c);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float qv = qr[i * d + c];
-                    af[i] = fmaf(qv, vf, af[i]);
-                    ad[i] = fmaf(qv, vd, ad[i]);
+                    const float4 w = ld4(qr + i * d + c);
+                    af[i] = fmaf(w.x, vf.x, af[i]); af[i] = fmaf(w.y, vf.y, af[i]); af[i] = fmaf(w.z, vf.z, af[i]); af[i] = fmaf(w.w, vf.w, af[i]);
+                    ad[i] = fmaf(w.x, vd.x, ad[i]); ad[i] = fmaf(w.y, vd.y, ad[i]); ad[i] = fmaf(w.z, vd.z, ad[i]); ad[i] = fmaf(w.w, vd.w, ad[i]);
                 }
             }
 #pragma unroll
@@ -91,6 +108,7 @@ __global__ void __launch_bounds__(256) probe_tile_kernel(ProbeArgs a) {
                     sum_d = fmaf(ad[i], ad[i], sum_d);
                 }
             }
+            if (more) store_q(half ^ 1);  // (read two turns ago, behind the last barrier)
             __syncthreads();
         }
     }
@@ -104,7 +122,7 @@ __global__ void __launch_bounds__(256) probe_tile_kernel(ProbeArgs a) {
     __syncthreads();
     if (threadIdx.x == 0) {
         double tf = 0, td = 0;
-        for (int w = 0; w < 8; ++w) { tf += s_red[0][w]; td += s_red[1][w]; }
+        for (int w = 0; w < kProbeThreads / 32; ++w) { tf += s_red[0][w]; td += s_red[1][w]; }
         double* p = a.part + ((int64_t)unit * a.nptiles_max + blockIdx.x) * 2;
         p[0] = tf;
         p[1] = td;
@@ -158,19 +176,19 @@ cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     if (!handled && (e = launch_probe_tc(a, dtype, st, &handled, &nparts)) != cudaSuccess) return e;
     if (!handled) {
-        const size_t smem = (size_t)(2 * kProbeTile * (a.d + 1) + kRowsBlk * a.d) * sizeof(float);
+        const size_t smem = probe_tile_smem(a.d);
         static PerDevice once;
         e = once.ensure([&]() {
-            cudaError_t e2 = cudaFuncSetAttribute(probe_tile_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+            cudaError_t e2 = cudaFuncSetAttribute(probe_tile_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)probe_tile_smem(128));
             if (e2 != cudaSuccess) return e2;
-            return cudaFuncSetAttribute(probe_tile_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+            return cudaFuncSetAttribute(probe_tile_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)probe_tile_smem(128));
         });
         if (e != cudaSuccess) return e;
         dim3 grid(nparts, a.unit_count);
         if (dtype == FDKV_BF16)
-            probe_tile_kernel<__nv_bfloat16><<<grid, 256, smem, st>>>(a);
+            probe_tile_kernel<__nv_bfloat16><<<grid, kProbeThreads, smem, st>>>(a);
         else
-            probe_tile_kernel<float><<<grid, 256, smem, st>>>(a);
+            probe_tile_kernel<float><<<grid, kProbeThreads, smem, st>>>(a);
         count_launch(1);
         count_kernel(FDKV_KERNEL_PROBE_PORTABLE);
         e = cudaGetLastError();
