@@ -264,22 +264,23 @@ def bench_workload(args, w, dev, dist, rank, local, world, steps, warmup, with_c
     n_ut = 2 * units
     N = w.T * w.head_dim
     if w.residual_rule == 1:
-        # token rule: compression is the depth split alone (the probe selects); the probe runs three products
-        # (token scores, then the two candidates' errors)
+        # token rule: compression is the depth split alone (the probe selects); the probe runs one product, whose scores and
+        # squares give the token sets and the errors
         nbl, nhf = w.block_size, (1 if w.block_size == 2 else 4)  # layers per block; stored high-frequency rows per kept token and tensor
         compress_min_bytes = n_ut * (nbl * N * esize + N * esize) + units * (2 * nhf * w.k_tok * w.head_dim * esize + 4 * w.k_tok)
-        probe_flops = 2.0 * units * 3 * (nbl * w.group * w.W) * w.T * w.head_dim
+        probe_flops = 2.0 * units * (nbl * w.group * w.W) * w.T * w.head_dim
     else:
         # read the block's layers, write the shared coefficient, the index and the kept values
         nbl = w.block_size
         compress_min_bytes = n_ut * (nbl * N * esize + N * esize + w.k_keep * (4 + (1 if nbl == 2 else 4) * esize))
-        probe_flops = 2.0 * units * 2 * (nbl * w.group * w.W) * w.T * w.head_dim
-    # bytes the compression kernels really move (pairs, entry rule, bf16 / head_dim 128): split reads both layers and
-    # writes Z0 and the staged Z1; the one-pass select reads Z1 once more and emits the canonical (index, value) list,
-    # the packed decode entries and, for K, the copy of Z1 without the kept entries for the probe
+        # two candidates: the product with every probe row, or where there are more of those than channels the second moments
+        probe_flops = 2.0 * units * 2 * min(nbl * w.group * w.W, w.head_dim * (1 if nbl == 2 else 4)) * w.T * w.head_dim
+    # bytes the compression kernels move (pairs, entry rule, bf16 / head_dim 128): split reads both layers and writes Z0, for K
+    # the staged Z1, and about 1.2 k candidates (position and value); those are read for the threshold (values) and for the
+    # lists: the canonical (index, value) list and the packed decode entries
     compress_moved_bytes = None
     if w.residual_rule == 0 and w.block_size == 2 and w.dtype == "bf16" and w.head_dim == 128:
-        compress_moved_bytes = n_ut * (5 * N * esize + w.k_keep * (8 + esize)) + units * N * esize
+        compress_moved_bytes = n_ut * (3 * N * esize + 1.2 * w.k_keep * (2 * (2 + esize) + esize) + w.k_keep * (8 + esize)) + units * N * esize
     modes_all = np.stack([ctx.get_modes(b).numpy() for b in range(w.batch)])
     mix = [int((modes_all == m).sum()) for m in range(3)]
     torch.cuda.empty_cache()
@@ -460,10 +461,10 @@ def bench_workload(args, w, dev, dist, rank, local, world, steps, warmup, with_c
                                          "moved_bytes": compress_moved_bytes,
                                          "achieved_moved_bytes": compress_moved_bytes / compress_ms / 1e6 if compress_moved_bytes else None,
                                          "frac_moved_bytes": compress_moved_bytes / compress_ms / 1e6 / hbm_peak if compress_moved_bytes else None,
-                                         "kernels": "depth split + histogram, threshold, one-pass ordered select (one fdkv_compress_prefill call, CUDA events)"},
+                                         "kernels": "sampled bound, split with candidate lists, threshold, ordered lists (one fdkv_compress_prefill call, CUDA events)"},
                         "probe": {"bound": "tensor", "unit": "TFLOP/s", "achieved": probe_flops / probe_ms / 1e9, "peak": tf_peak,
                                   "of": peak_kind + " bf16 burst (a millisecond kernel timed alone)", "frac": probe_flops / probe_ms / 1e9 / tf_peak,
-                                  "flops": probe_flops, "kernels": "one fdkv_probe call (error products of both candidates + mode rule, CUDA events)"}}},
+                                  "flops": probe_flops, "kernels": "one fdkv_probe call (second moments and products of both candidates + mode rule, CUDA events)"}}},
         "step_bytes": step_bytes,
     }
     pf.ctx.close()
