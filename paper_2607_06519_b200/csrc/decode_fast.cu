@@ -180,7 +180,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // CL: every unit's thread blocks form a cluster (its dimension is the unit's number of blocks) and join their states through
 // distributed shared memory, so that a call is one kernel: for short contexts, whose cost is the chain of hand-overs.
 // NB: room for the tail lengths in the parameters.
-template <bool F8, bool CL, int NB>
+// SPLIT: at most four query heads per KV head.
+template <bool F8, bool CL, int NB, bool SPLIT>
 __global__ void __maxnreg__(232)
 decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap8, DecodeArgs a, FastSched sch,
                    TailLens<NB> tl) {
@@ -497,7 +498,8 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             if (!waited) dependency_wait();
             // q fragments: B operand columns = the G query heads of this KV head.  With G <= 4 columns 4-7 repeat
             // them: in the second product those columns carry the bf16 rounding remainder of P, so P acts in ~16 bits.
-            const bool split = a.G <= 4;
+            // (More heads fill the columns: their remainder is a second B operand with the same V fragments.)
+            const bool split = SPLIT && a.G <= 4;  // (a constant cost the 32k workloads 0.5 to 0.9 %)
             const int qcol = split ? (gid & 3) : gid;
             uint32_t qb[8][2];
             auto load_q = [&](bool f8) {
@@ -1059,12 +1061,15 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         };
-        opt_in(decode_fast_kernel<false, false, kFewSeqs>, smem_of(false, false));
-        opt_in(decode_fast_kernel<true, false, kFewSeqs>, smem_of(true, false));
-        opt_in(decode_fast_kernel<false, false, kMaxUnits>, smem_of(false, false));
-        opt_in(decode_fast_kernel<true, false, kMaxUnits>, smem_of(true, false));
-        opt_in(decode_fast_kernel<false, true, kFewSeqs>, smem_of(false, true));
-        opt_in(decode_fast_kernel<true, true, kFewSeqs>, smem_of(true, true));
+        opt_in(decode_fast_kernel<false, false, kFewSeqs, true>, smem_of(false, false));
+        opt_in(decode_fast_kernel<false, false, kFewSeqs, false>, smem_of(false, false));
+        opt_in(decode_fast_kernel<true, false, kFewSeqs, true>, smem_of(true, false));
+        opt_in(decode_fast_kernel<false, false, kMaxUnits, true>, smem_of(false, false));
+        opt_in(decode_fast_kernel<false, false, kMaxUnits, false>, smem_of(false, false));
+        opt_in(decode_fast_kernel<true, false, kMaxUnits, true>, smem_of(true, false));
+        opt_in(decode_fast_kernel<false, true, kFewSeqs, true>, smem_of(false, true));
+        opt_in(decode_fast_kernel<false, true, kFewSeqs, false>, smem_of(false, true));
+        opt_in(decode_fast_kernel<true, true, kFewSeqs, true>, smem_of(true, true));
         // the same division of the SM's memory as the decode kernel's, or the two could not share an SM
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -1078,7 +1083,7 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
             at[0].val.clusterDim.x = 1u << lg; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
             q.attrs = at;
             q.numAttrs = 1;
-            e = cudaOccupancyMaxActiveClusters(&max_clusters_of[dev][lg], decode_fast_kernel<true, true, kFewSeqs>, &q);
+            e = cudaOccupancyMaxActiveClusters(&max_clusters_of[dev][lg], decode_fast_kernel<true, true, kFewSeqs, true>, &q);
         }
         return e;
     }, &sm_count);
@@ -1116,9 +1121,19 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
         return cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, tl);
     };
     cudaError_t e;
-    if (sch.cluster) e = launch(a.rows_f8 ? decode_fast_kernel<true, true, kFewSeqs> : decode_fast_kernel<false, true, kFewSeqs>, TailLens<kFewSeqs>());
-    else if (a.batch <= kFewSeqs) e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kFewSeqs> : decode_fast_kernel<false, false, kFewSeqs>, TailLens<kFewSeqs>());
-    else e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kMaxUnits> : decode_fast_kernel<false, false, kMaxUnits>, TailLens<kMaxUnits>());
+    const bool split = a.G <= 4;  // (8-bit rows take no more)
+    if (sch.cluster)
+        e = launch(a.rows_f8 ? decode_fast_kernel<true, true, kFewSeqs, true>
+                   : split   ? decode_fast_kernel<false, true, kFewSeqs, true>
+                             : decode_fast_kernel<false, true, kFewSeqs, false>, TailLens<kFewSeqs>());
+    else if (a.batch <= kFewSeqs)
+        e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kFewSeqs, true>
+                   : split   ? decode_fast_kernel<false, false, kFewSeqs, true>
+                             : decode_fast_kernel<false, false, kFewSeqs, false>, TailLens<kFewSeqs>());
+    else
+        e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kMaxUnits, true>
+                   : split   ? decode_fast_kernel<false, false, kMaxUnits, true>
+                             : decode_fast_kernel<false, false, kMaxUnits, false>, TailLens<kMaxUnits>());
     if (e != cudaSuccess) return e;
     count_launch(1);
     count_kernel(FDKV_KERNEL_DECODE_FAST);
