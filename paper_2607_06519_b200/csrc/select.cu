@@ -347,6 +347,9 @@ __global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a,
     };
     request_next(0);
     request_next(1);
+    // The warps' counts alternate between two sets with the items that are worked on, not with the stages: the barrier of the next such
+    // item is what separates a set's reads from its next writes, and in a second run other items lie between.
+    int cs = 0;
     for (int it = 0; left > 0; --left, it ^= 1, advance(now)) {
         const int ut = a.ut_base + now.blk * uts + now.u;
         const int64_t e0 = (int64_t)now.chunk * CE;
@@ -393,15 +396,16 @@ __global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a,
                 const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
                 if (lane >= o) incl += y;
             }
-            if (lane == 31) s_cnt[it][warp] = incl;
+            if (lane == 31) s_cnt[cs][warp] = incl;
             __syncthreads();
             uint32_t at = incl - mine, n = 0;
 #pragma unroll
             for (int w = 0; w < 8; ++w) {
-                const uint32_t y = s_cnt[it][w];
+                const uint32_t y = s_cnt[cs][w];
                 if (w < warp) at += y;
                 n += y;
             }
+            cs ^= 1;
             if (tid == 0) a.cand_n[(int64_t)ut * a.chunks_max + now.chunk] = (int32_t)n;
             uint16_t* const pos = a.cand_pos + (int64_t)ut * a.cand_stride + e0;
             T* const val = reinterpret_cast<T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0;

@@ -57,3 +57,37 @@ def test_chunk_edges(dtype, d, T):
     pf.compress(0)
     check_compression(pf.ctx, w, 0, 0, 0)
     assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("hkv", [4, 8])
+def test_a_sample_that_misleads_for_one_head(hkv):
+    """Only one head's K runs again with bound 0: a block then works on items that lie one, three, ... others apart."""
+    from paper_2607_06519_b200 import binding as B
+
+    T, d, L = 5003, 128, 8
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+    scale = torch.ones((T, 1, 1), device="cuda")
+    scale[torch.from_numpy(_sampled_tokens(T, d)).cuda()] = 100.0
+    k, v = [], []
+    for layer in range(L):
+        if layer % 2 == 0:
+            base = [torch.randn((T, hkv, d), generator=g, device="cuda") for _ in range(2)]
+            k.append(base[0].bfloat16())
+            v.append(base[1].bfloat16())
+        else:
+            dk, dv = (torch.randn((T, hkv, d), generator=g, device="cuda") for _ in range(2))
+            dk[:, 1:2] *= scale
+            k.append((base[0] + dk).bfloat16())
+            v.append((base[1] + dv).bfloat16())
+    ctx = B.Context(B.Config(L, hkv, hkv, d, 1, T, 1, B.BF16, 1, 16))
+    ctx.compress_prefill(0, 0, L // 2, T, k, v)
+    for p in range(L // 2):
+        for h in range(hkv):
+            for is_v, x in ((0, k), (1, v)):
+                _, z1 = R.depth_split(x[2 * p][:, h].float().cpu().numpy(), x[2 * p + 1][:, h].float().cpu().numpy(), True)
+                want = R.select_entries(z1, T * d // 16)
+                idx, val = ctx.get_residual(0, p, h, is_v)
+                assert np.array_equal(idx.cpu().numpy(), want), (p, h, is_v)
+                assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want]), (p, h, is_v)
+    assert ctx.device_status() == 0
