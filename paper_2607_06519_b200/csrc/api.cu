@@ -982,23 +982,28 @@ fdkv_status fdkv_fold_tail(fdkv_ctx* c, int32_t seq, int32_t n, void* stream) {
     }
     CopyJob* const table = reinterpret_cast<CopyJob*>(c->work + c->ws.jobs + quant_table_bytes(s) + gather_table_bytes(s));
     CU(copies.launch(table, reinterpret_cast<CopyJob*>(c->pin + c->pin_jobs), st));
-    // ---- the remaining tail rows move down: through the staging area, as many layers at a time as it holds, where the ranges
-    // overlap ----
+    // ---- the remaining tail rows move down: where the ranges overlap through the staging area, as many layers at a time as it
+    // holds, or a layer in pieces from the front (a piece ends before the rows that the next one reads) ----
     if (rest > 0) {
-        const size_t w = (size_t)rest * row_b, layer_b = 2 * (size_t)s.Hkv * w, room = (size_t)s.NU * s.NB * unit_stride_b;
-        const int group = rest <= n ? s.L : (int)std::max<size_t>(1, std::min<size_t>(s.L, room / layer_b));
-        for (int l0 = 0; l0 < s.L; l0 += group) {
-            CopyTable<2> moves;
-            char* tmp = c->work + c->ws.z1;
-            for (int l = l0; l < std::min(s.L, l0 + group); ++l)
-                for (char* base : {tail_base(tk, l), tail_base(tv, l)})
-                    for (int h = 0; h < s.Hkv; ++h, base += tail_head_b, tmp += w) {
-                        moves.plain(0, base + (size_t)n * row_b, rest <= n ? base : tmp, w);
-                        if (rest > n) moves.plain(1, tmp, base, w);
-                    }
-            if (l0 > 0) CU(cudaStreamSynchronize(st));  // (the page-locked table is written again)
-            CU(moves.launch(table, reinterpret_cast<CopyJob*>(c->pin + c->pin_jobs + align_up(max_copy_jobs(s) * sizeof(CopyJob))), st));
-        }
+        const bool overlap = rest > n;
+        const size_t room = (size_t)s.NU * s.NB * unit_stride_b / (2 * s.Hkv * row_b);  // tokens of a layer that fit: at least 8
+        const int piece = overlap ? (int)std::min<size_t>(rest, room) : rest;
+        const int group = overlap ? (int)std::min<size_t>(s.L, room / piece) : s.L;
+        for (int l0 = 0; l0 < s.L; l0 += group)
+            for (int r0 = 0; r0 < rest; r0 += piece) {
+                CopyTable<2> moves;
+                const size_t w = (size_t)std::min(piece, rest - r0) * row_b;
+                char* tmp = c->work + c->ws.z1;
+                for (int l = l0; l < std::min(s.L, l0 + group); ++l)
+                    for (char* base : {tail_base(tk, l), tail_base(tv, l)})
+                        for (int h = 0; h < s.Hkv; ++h, base += tail_head_b, tmp += w) {
+                            char* const to = base + (size_t)r0 * row_b;
+                            moves.plain(0, to + (size_t)n * row_b, overlap ? tmp : to, w);
+                            if (overlap) moves.plain(1, tmp, to, w);
+                        }
+                if (l0 > 0 || r0 > 0) CU(cudaStreamSynchronize(st));  // (the page-locked table is written again)
+                CU(moves.launch(table, reinterpret_cast<CopyJob*>(c->pin + c->pin_jobs + align_up(max_copy_jobs(s) * sizeof(CopyJob))), st));
+            }
     }
     CU(launch_set_tail_len(arp<int32_t>(c, c->ar.tail_len), s.L, s.max_batch, seq, rest, st));
     q.tail_len.assign(s.L, rest);

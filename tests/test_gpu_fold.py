@@ -181,3 +181,43 @@ def test_fold_of_a_short_chunk_moves_a_long_rest_down(dtype, d, keep):
             u.fold(16, *keep)
         assert _check_step(pf, w, modes, units, step, check=True) <= TOL[dtype]
     assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype,d,T,L,tail", [("bf16", 128, 16, 2, 2100), ("f32", 64, 48, 4, 1300), ("bf16", 128, 64, 2, 49)])
+def test_fold_of_a_tail_many_times_the_prompt(dtype, d, T, L, tail, monkeypatch):
+    """The rows that stay are longer than the staging area: they move in pieces and nothing behind the workspace changes.  Exact
+    units attend over the same rows before and after."""
+    arena_b, work_b = B.sizes(B.Config(L, 8, 2, d, 1, T, tail, B.BF16 if dtype == "bf16" else B.F32, 1, 16, max_fold=32))
+    guard = 8 << 20
+    monkeypatch.setattr(B, "sizes", lambda cfg: (arena_b, work_b + guard))
+    ctx = B.Context(B.Config(L, 8, 2, d, 1, T, tail, B.BF16 if dtype == "bf16" else B.F32, 1, 16, max_fold=32))
+    ctx.work[work_b:].fill_(0x5A)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+
+    def rand(*shape):
+        return torch.randn(shape, generator=g, device="cuda").to(tdt)
+
+    k, v = ([rand(T, 2, d) for _ in range(L)] for _ in range(2))
+    ctx.compress_prefill(0, 0, L // 2, T, k, v)
+    ctx.set_modes(0, np.full((L // 2, 2), 2, dtype=np.int32))
+    ctx.commit(0)
+    rows = rand(2, tail, L, 1, 2, d)
+    q = rand(L, 1, 8, d)
+    for j in range(tail):
+        for l in range(L):
+            ctx.decode_attn(l, q[l], rows[0, j, l], rows[1, j, l])
+    scale = d ** -0.5
+    for n in (0, 16, 16):
+        if n:
+            ctx.fold_tail(0, n)
+        for l in range(L):
+            got = f32(ctx.decode_attn(l, q[l], out_dtype=0))[0]
+            kk, vv = (torch.cat([x[l], rows[i, :, l, 0]]).double().repeat_interleave(4, dim=1) for i, x in ((0, k), (1, v)))
+            p = torch.softmax(torch.einsum("hd,thd->ht", q[l, 0].double(), kk) * scale, dim=1)
+            want = torch.einsum("ht,thd->hd", p, vv).cpu().numpy()
+            assert vector_errors(got, want).max() <= 3e-5, (n, l)
+    assert bool((ctx.work[work_b:] == 0x5A).all())
+    assert ctx.device_status() == 0
+    ctx.close()
