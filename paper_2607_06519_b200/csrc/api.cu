@@ -55,10 +55,10 @@ bool make_shape(const fdkv_config& c, Shape& s) {
     s.kcap = (int64_t)align_up((size_t)(s.kmax + kListPad), 64);
     s.ntiles_max = (s.Tmax + kResTile - 1) / kResTile;
     // per-unit partial-sum slots of the probe: one per 64-token tile (portable kernel) or one per work item of the
-    // tensor-core kernel (layers x 128-row blocks x key splits of at least 8 tiles) and the blocks of the second-moment
-    // kernel that share a unit, whichever is more
+    // tensor-core kernel (layers x 128-row blocks x key splits of at least 8 tiles; twice, where a unit is done again) and the
+    // blocks of the second-moment kernel that share a unit, whichever is more
     s.nptiles_max = std::max((s.Tmax + kProbeTile - 1) / kProbeTile,
-                             B * ((G * kMaxW + 127) / 128) * (((s.Tmax - 1) / kProbeBoxRows + 1 + 7) / 8) + kMaxGramCtas + 2 * 4);
+                             2 * B * ((G * kMaxW + 127) / 128) * (((s.Tmax - 1) / kProbeBoxRows + 1 + 7) / 8) + kMaxGramSlots);
     s.tail_rows = (s.max_tail + kRowPad - 1) / kRowPad * kRowPad;
     if (c.residual_rule != FDKV_RESIDUAL_ENTRIES && c.residual_rule != FDKV_RESIDUAL_TOKENS) return false;
     s.tok_rule = c.residual_rule == FDKV_RESIDUAL_TOKENS;
@@ -99,6 +99,8 @@ void make_layouts(const Shape& s, WsLayout& w, ArenaLayout& a) {
     w.tok_list = take(s.tok_rule ? (size_t)s.NU * s.ktok_cap * 4 : 0);
     w.tok_off = take(s.tok_rule ? (size_t)s.NU * (s.ntiles_max + 1) * 4 : 0);
     w.probe_part = take((size_t)s.NU * s.nptiles_max * 16);
+    w.probe_scale = take(s.dtype == FDKV_BF16 && s.d == 128 && !s.tok_rule ? (size_t)s.NU * kMaxGramSlots * 16 : 0);
+    w.probe_redo = take((size_t)s.NU * 4);
     w.probe_pos = take((size_t)kMaxW * 4 + (size_t)s.L * 8);
     w.scores = take((size_t)s.NU * 16);
     w.modes = take((size_t)s.NU * 4);
@@ -471,6 +473,8 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
     a.q_layers_dev = qptr_dev;
     a.pos = pos_dev;
     a.part = wsp<double>(c, c->ws.probe_part);
+    a.scale = wsp<double>(c, c->ws.probe_scale);
+    a.redo = wsp<int32_t>(c, c->ws.probe_redo);
     a.scores = wsp<double>(c, c->ws.scores);
     a.modes = wsp<int32_t>(c, c->ws.modes);
     a.lambda = lambda;

@@ -103,7 +103,8 @@ struct Shape {
 
 struct WsLayout {
     size_t tok_score, tok_err, tok_list, tok_off;
-    size_t status, z0, z1, z1drop, cand_pos, cand_val, cand_n, chunk_base, keep, sel, tile_off, idx, val, packed, probe_part, probe_pos, scores, modes,
+    size_t status, z0, z1, z1drop, cand_pos, cand_val, cand_n, chunk_base, keep, sel, tile_off, idx, val, packed, probe_part, probe_scale, probe_redo,
+        probe_pos, scores, modes,
         partials, io_q, io_k, io_v, io_out, jobs, total;  // io_*: host-I/O staging, [L] layers each
 };
 struct ArenaLayout {
@@ -236,6 +237,8 @@ struct ProbeArgs {
     const void* const* q_layers_dev;  // device array [L] of pointers
     const int32_t* pos;
     double* part;    // [NU][nptiles_max][2]
+    double* scale;   // [NU][kMaxGramSlots][2] what the second moments' sums are to be large against
+    int32_t* redo;   // [NU] the second moments' sums are not exact enough: the unit is done again by products
     double* scores;  // [NU][2]
     int32_t* modes;  // [NU]
     double lambda, omega[3];
@@ -250,7 +253,13 @@ struct ProbeArgs {
     int32_t* status;
 };
 cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st);
-constexpr int kMaxGramCtas = 160;  // blocks of the second-moment kernel, and so part slots a unit may need
+constexpr int kMaxGramCtas = 160;  // blocks of the second-moment kernel
+constexpr int kMaxGramSlots = kMaxGramCtas + 2 * 4;  // ... and so part slots a unit may need
+// Part slots of a unit: [0, gram) second moments, [gram, sure) products, [sure, all) products in the place of the second moments
+// for units that are done again.
+struct ProbeParts {
+    int gram, sure, all;
+};
 cudaError_t launch_probe_gram(const ProbeArgs& a, int t_full, cudaStream_t st, int* nparts);
 
 struct DecodeArgs {

@@ -132,12 +132,14 @@ __global__ void __launch_bounds__(kProbeThreads) probe_tile_kernel(ProbeArgs a) 
 }  // namespace
 
 // Sums the per-tile partials in a fixed order, applies the (c/sqrt d)^2 / (2 G W) factor and the mode rule.
-__global__ void __launch_bounds__(256) probe_finalize_kernel(ProbeArgs a, int nparts) {
+__global__ void __launch_bounds__(256) probe_finalize_kernel(ProbeArgs a, ProbeParts parts) {
     __shared__ double s0[256], s1[256];
     const int unit = a.unit_begin + blockIdx.x;
     const double* p = a.part + (int64_t)unit * a.nptiles_max * 2;
     double x0 = 0, x1 = 0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) { x0 += p[2 * i]; x1 += p[2 * i + 1]; }
+    const bool redo = parts.all > parts.sure && a.redo[unit];
+    const int first = redo ? parts.gram : 0, last = redo ? parts.all : parts.sure;
+    for (int i = first + threadIdx.x; i < last; i += blockDim.x) { x0 += p[2 * i]; x1 += p[2 * i + 1]; }
     s0[threadIdx.x] = x0;
     s1[threadIdx.x] = x1;
     __syncthreads();
@@ -167,14 +169,15 @@ __global__ void __launch_bounds__(256) probe_finalize_kernel(ProbeArgs a, int np
     }
 }
 
-cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool* handled, int* nparts);
+cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool* handled, ProbeParts* parts);
 
 cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st) {
     if (a.unit_count <= 0) return cudaSuccess;
-    int nparts = a.sums_ready ? 1 : (a.T + kProbeTile - 1) / kProbeTile;
+    const int nparts = a.sums_ready ? 1 : (a.T + kProbeTile - 1) / kProbeTile;
+    ProbeParts parts = {0, nparts, nparts};
     bool handled = a.sums_ready;
     cudaError_t e = cudaSuccess;
-    if (!handled && (e = launch_probe_tc(a, dtype, st, &handled, &nparts)) != cudaSuccess) return e;
+    if (!handled && (e = launch_probe_tc(a, dtype, st, &handled, &parts)) != cudaSuccess) return e;
     if (!handled) {
         const size_t smem = probe_tile_smem(a.d);
         static PerDevice once;
@@ -194,7 +197,7 @@ cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st) {
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    probe_finalize_kernel<<<a.unit_count, 256, 0, st>>>(a, nparts);
+    probe_finalize_kernel<<<a.unit_count, 256, 0, st>>>(a, parts);
     count_launch(1);
     return cudaGetLastError();
 }

@@ -15,11 +15,16 @@
 //     warps 6-13: write the tile with its kept entries zeroed next to it; warp 1: both products, tokens on K, so the
 //     operands are MN-major views of the row-major tiles, A and B the same tile (8 + 8 tcgen05.mma, M = N = 128, K = 16);
 //     warps 2-5: epilogue.
-//   * Q^T Q of the segment's rows comes first, through the same ring and tensor memory (three 128-column accumulators).
+//   * Q^T Q of the segment's rows comes first, through the same ring and accumulators, a tile of 128 rows at a time: the epilogue
+//     adds the tiles up in a third 128-column region of tensor memory.
 //   * The sums are drained every two tiles, one candidate's while the other's products run: <R^T R, Q^T Q> in float32 over 32
-//     columns of a row, added up in float64.  An accumulator then takes 16 steps, as precise as the product form's eight and the
-//     square (the errors of 32 layers of 32k tokens differ from the product form's by 1.1e-6; with eight tiles per drain by 2.9e-6, in
-//     312 instead of 360 us).
+//     columns of a row, added up in float64.
+//   * Precision.  The tensor core rounds its accumulators towards zero, so what counts is the number of steps that one takes: 16 for
+//     R^T R (eight tiles per drain were 15 % faster and ten times less exact) and eight for Q^T Q (all rows in one accumulator: 1.3e-6
+//     off float64 at 512 rows, 5.5e-6 at 2 048).
+//     The sum cancels where queries and coefficients are nearly orthogonal, which the products, sums of squares, do not.  So the
+//     traces are kept too: tr(R^T R) tr(Q^T Q) is the sum of |Q_r|^2 |R_j|^2, and a unit whose error is a small part of it (or not
+//     finite) is done again by products (probe_tc.cu).
 // Bound by shared memory: the products read 128 KiB of operands per tile, the masking 64 KiB, the copy 32 KiB (0.9 us at
 // 128 bytes per cycle); HBM's share of the tile is 0.7 us.
 #include <algorithm>
@@ -121,40 +126,36 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
     } else if (warp == 1) {
         if (lane == 0) {
             int it = 0;
-            uint32_t gen = 0;  // drains
+            uint32_t gen0 = 0, gen1 = 0;  // drains of either accumulator
             for (int64_t g = g_begin; g < g_end;) {
                 const int t0 = (int)(g % pl.nt), n = (int)min((int64_t)pl.nt - t0, g_end - g);
                 for (int i = -pl.qtiles; i < n; ++i, ++it) {
                     const int s = it % kGStages;
                     const uint32_t par = (uint32_t)(it / kGStages) & 1u;
-                    // Q^T Q is read with every group: it is replaced once both accumulators of the last one have been read
-                    if (i == -pl.qtiles)
-                        for (int c = 0; c < 2; ++c) mb_wait(sm0 + gAccEmpty + 8 * c, (gen & 1u) ^ 1u, abort_flag, a.status);
                     mb_wait(sm0 + gFull + 8 * s, par, abort_flag, a.status);
                     mb_wait(sm0 + gMasked + 8 * s, par, abort_flag, a.status);
                     if (*abort_flag) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t df = smem_desc_sw128(stage0 + s * kGStage, kGHalf, 1024);
                     const uint64_t dd = smem_desc_sw128(stage0 + s * kGStage + kGTile, kGHalf, 1024);
-                    if (i < 0) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            umma_ss<kGIdesc>(tmem + kGColA, dd + k * (2048 >> 4), dd + k * (2048 >> 4), k > 0 || i > -pl.qtiles);
-                    } else {
-                        // one candidate's accumulator is drained while the other's products run
-                        const bool opens = i % kGroup == 0, closes = i % kGroup == kGroup - 1 || i == n - 1;
-                        for (int c = 0; c < 2; ++c) {
-                            if (opens) {
-                                mb_wait(sm0 + gAccEmpty + 8 * c, (gen & 1u) ^ 1u, abort_flag, a.status);
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                            }
-                            const uint64_t desc = c ? dd : df;
-                            const uint32_t acc = tmem + (c ? kGColD : kGColF);
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) umma_ss<kGIdesc>(acc, desc + k * (2048 >> 4), desc + k * (2048 >> 4), k > 0 || !opens);
-                            if (closes) umma_commit(sm0 + gAccFull + 8 * c);
+                    for (int c = 0; c < 2; ++c) {
+                        // probe rows: a tile per drain, the accumulators in turn.  Tokens: one candidate's accumulator is drained while
+                        // the other's products run.
+                        if (i < 0 && ((i + pl.qtiles) & 1) != c) continue;
+                        const bool opens = i < 0 || i % kGroup == 0, closes = i < 0 || i % kGroup == kGroup - 1 || i == n - 1;
+                        if (opens) {
+                            mb_wait(sm0 + gAccEmpty + 8 * c, ((c ? gen1 : gen0) & 1u) ^ 1u, abort_flag, a.status);
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         }
-                        if (closes) ++gen;
+                        const uint64_t desc = c || i < 0 ? dd : df;
+                        const uint32_t acc = tmem + (c ? kGColD : kGColF);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) umma_ss<kGIdesc>(acc, desc + k * (2048 >> 4), desc + k * (2048 >> 4), k > 0 || !opens);
+                        if (closes) {
+                            umma_commit(sm0 + gAccFull + 8 * c);
+                            if (c) ++gen1; else ++gen0;
+                        }
                     }
                     umma_commit(sm0 + gEmpty + 8 * s);
                 }
@@ -165,23 +166,62 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
     } else if (warp < 6) {
         // ---- epilogue: thread = row of the 128 x 128 moments (tensor memory lane) ----
         const int lq = warp & 3;
-        uint32_t gen = 0;
+        const uint32_t tq = tmem + ((uint32_t)(lq * 32) << 16);
+        uint32_t gen0 = 0, gen1 = 0;  // drains of either accumulator
+        // block b of this row's moments; the diagonal element if it is there
+        auto diagonal = [&](int b, const uint32_t (&r)[32]) {
+            float x = 0.f;
+            if (b == lq)
+#pragma unroll
+                for (int j = 0; j < 32; ++j) x = j == lane ? __uint_as_float(r[j]) : x;
+            return x;
+        };
+        auto await = [&](int c) {
+            mb_wait(sm0 + gAccFull + 8 * c, (c ? gen1 : gen0) & 1u, abort_flag, a.status);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        };
+        auto drained = [&](int c) {
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mb_arrive(sm0 + gAccEmpty + 8 * c);
+            if (c) ++gen1; else ++gen0;
+        };
         for (int64_t g = g_begin; g < g_end;) {
             const int op = (int)(g / pl.nt), t0 = (int)(g % pl.nt), n = (int)min((int64_t)pl.nt - t0, g_end - g);
-            double tf = 0.0, td = 0.0;
-            for (int i0 = 0; i0 < n; i0 += kGroup, ++gen) {
+            double sum0 = 0.0, sum1 = 0.0, tr0 = 0.0, tr1 = 0.0;
+            float tr_q = 0.f;
+#pragma unroll 1
+            for (int q = 0; q < pl.qtiles; ++q) {
+                const int c = q & 1;
+                await(c);
+                if (!*abort_flag) {
+#pragma unroll 1
+                    for (int b = 0; b < 4; ++b) {
+                        uint32_t rr[32], ra[32];
+                        tmem_ld32(tq + (c ? kGColD : kGColF) + b * 32, rr);
+                        tmem_ld32(tq + kGColA + b * 32, ra);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) rr[j] = q > 0 ? __float_as_uint(__uint_as_float(rr[j]) + __uint_as_float(ra[j])) : rr[j];
+                        tmem_st32(tq + kGColA + b * 32, rr);
+                        if (q == pl.qtiles - 1) tr_q += diagonal(b, rr);
+                    }
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                }
+                drained(c);
+            }
+            for (int i0 = 0; i0 < n; i0 += kGroup) {
 #pragma unroll 1
                 for (int c = 0; c < 2; ++c) {
-                    mb_wait(sm0 + gAccFull + 8 * c, gen & 1u, abort_flag, a.status);
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    await(c);
                     if (!*abort_flag) {
-                        double sum = 0.0;
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
+                        double e = 0.0;
+                        float dg = 0.f;
+#pragma unroll 1
+                        for (int b = 0; b < 4; ++b) {  // (unrolled it takes more registers than a thread has)
                             uint32_t rr[32], ra[32];
-                            const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(b * 32);
-                            tmem_ld32(ta + (c ? kGColD : kGColF), rr);
-                            tmem_ld32(ta + kGColA, ra);
+                            tmem_ld32(tq + (c ? kGColD : kGColF) + b * 32, rr);
+                            tmem_ld32(tq + kGColA + b * 32, ra);
                             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                             float f0 = 0.f, f1 = 0.f;
 #pragma unroll
@@ -189,32 +229,39 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
                                 f0 = fmaf(__uint_as_float(rr[j]), __uint_as_float(ra[j]), f0);
                                 f1 = fmaf(__uint_as_float(rr[j + 1]), __uint_as_float(ra[j + 1]), f1);
                             }
-                            sum += (double)f0 + (double)f1;
+                            e += (double)f0 + (double)f1;
+                            dg += diagonal(b, rr);
                         }
-                        (c ? td : tf) += sum;
+                        (c ? sum1 : sum0) += e;
+                        (c ? tr1 : tr0) += (double)dg;
                     }
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mb_arrive(sm0 + gAccEmpty + 8 * c);
+                    drained(c);
                 }
             }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                tf += __shfl_xor_sync(0xFFFFFFFFu, tf, o);
-                td += __shfl_xor_sync(0xFFFFFFFFu, td, o);
-            }
+            // the four warps' five sums: both candidates' errors and traces, the queries' trace
+            double v[5] = {sum0, sum1, tr0, tr1, (double)tr_q};
             double* const red = reinterpret_cast<double*>(smem + gRed);
-            if (lane == 0) { red[2 * lq] = tf; red[2 * lq + 1] = td; }
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+#pragma unroll
+                for (int o = 16; o; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
+                if (lane == 0) red[4 * k + lq] = v[k];
+            }
             asm volatile("bar.sync 1, 128;" ::: "memory");
             if (warp == 2) {
                 // part slots of the operand: one per CTA that holds some of its tiles, in order; the last of them clears the rest
                 const int c0 = gram_cta_of((int64_t)op * pl.nt, n_tiles, pl.ncta);
                 const int unit = a.unit_begin + op / pl.n_ops;
-                double* const p = a.part + ((int64_t)unit * a.nptiles_max + (op % pl.n_ops) * pl.maxseg) * 2;
-                const int slot = (int)blockIdx.x - c0;
-                if (lane < 2) p[slot * 2 + lane] = (red[lane] + red[2 + lane]) + (red[4 + lane] + red[6 + lane]);
+                const int first = (op % pl.n_ops) * pl.maxseg, slot = (int)blockIdx.x - c0;
+                double* const p = a.part + ((int64_t)unit * a.nptiles_max + first) * 2;
+                double* const m = a.scale + ((int64_t)unit * kMaxGramSlots + first) * 2;
+                auto all = [&](int k) { return (red[4 * k] + red[4 * k + 1]) + (red[4 * k + 2] + red[4 * k + 3]); };
+                if (lane < 2) {
+                    p[slot * 2 + lane] = all(lane);
+                    m[slot * 2 + lane] = all(2 + lane) * all(4);
+                }
                 if (t0 + n == pl.nt)
-                    for (int i = (slot + 1) * 2 + lane; i < pl.maxseg * 2; i += 32) p[i] = 0.0;
+                    for (int i = (slot + 1) * 2 + lane; i < pl.maxseg * 2; i += 32) p[i] = m[i] = 0.0;
             }
             asm volatile("bar.sync 1, 128;" ::: "memory");
             if (*abort_flag) break;

@@ -54,6 +54,8 @@ struct TcPlan {
     int pos_min, pos_max;
     int tile_first;   // first 256-key tile (the keys before it are probe_gram_kernel's)
     int slot0;        // first part slot
+    // Units whose second moments are not exact enough: the keys before tile_first again, by the blocks behind the first sure_items
+    int sure_items, redo_per_unit, redo_nsplits, redo_tiles_per_split, redo_slot0;
 };
 
 // kBStages, kAccSets: three and two for items of many tiles; one and one for items of a tile or two, whose time is the chain from
@@ -74,18 +76,12 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
         if (threadIdx.x == 0) atomicMax(a.status, (int32_t)kFlagCountMismatch);
         return;
     }
-    // ---- decode the work item ----
-    int it = blockIdx.x;
-    const int unit = a.unit_begin + it / pl.items_per_unit;
-    it %= pl.items_per_unit;
-    const int split = it % pl.nsplits; it /= pl.nsplits;
-    const int cand = it & 1; it >>= 1;
-    const int mblock = it % pl.mblocks; it /= pl.mblocks;
-    const int layer = it;  // layer inside the depth block: 0 .. B-1
-    const int h = unit % a.Hkv, pair = unit / a.Hkv;
-    const int tile0 = pl.tile_first + split * pl.tiles_per_split;
-    const int tile1 = min(pl.ntiles, tile0 + pl.tiles_per_split);
-    const int ntile = max(0, tile1 - tile0);
+    const bool again = (int)blockIdx.x >= pl.sure_items;
+    if (again) {  // (almost always there is nothing to do again)
+        int any = 0;
+        for (int u = threadIdx.x; u < a.unit_count; u += kPThreads) any |= a.redo[a.unit_begin + u];
+        if (!__syncthreads_or(any)) return;
+    }
     const int rows_layer = a.G * a.W;
 
     if (threadIdx.x == 0) {
@@ -102,6 +98,23 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(smem + oSlot);
+    const int per_unit = again ? pl.redo_per_unit : pl.items_per_unit, nsplits = again ? pl.redo_nsplits : pl.nsplits;
+    const int per_split = again ? pl.redo_tiles_per_split : pl.tiles_per_split;
+    int done = 0;  // tiles of the items before: the stages and accumulators go on in turn
+    for (int item = again ? (int)blockIdx.x - pl.sure_items : (int)blockIdx.x; item < a.unit_count * per_unit; item += (int)gridDim.x - pl.sure_items) {
+    // ---- decode the work item ----
+    int it = item;
+    const int unit = a.unit_begin + it / per_unit;
+    if (again && !a.redo[unit]) continue;
+    it %= per_unit;
+    const int split = it % nsplits; it /= nsplits;
+    const int cand = it & 1; it >>= 1;
+    const int mblock = it % pl.mblocks; it /= pl.mblocks;
+    const int layer = it;  // layer inside the depth block: 0 .. B-1
+    const int h = unit % a.Hkv, pair = unit / a.Hkv;
+    const int tile0 = (again ? 0 : pl.tile_first) + split * per_split;
+    const int tile1 = min(again ? pl.tile_first : pl.ntiles, tile0 + per_split);
+    const int ntile = max(0, tile1 - tile0);
     // ---- A operand: row r = mblock*256 + mt*128 + rl of this layer's probe block, r = g*W + qi -> Q[layer][qi][h*G+g][:],
     //      row rl of M tile mt: 16 chunks of 16 bytes, chunk c of a 64-channel half stored at chunk c ^ (rl & 7) ----
     if (warp >= 2) {
@@ -128,8 +141,8 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
             // rows of this unit's K coefficients (a block of four stages one operand per layer)
             const int64_t row0 = a.B == 4 ? ((int64_t)unit * 4 + layer) * a.Tmax : (int64_t)unit * a.Tmax;
             for (int i = 0; i < ntile; ++i) {
-                const int s = i % kBStages;
-                const uint32_t ph = (uint32_t)(i / kBStages) & 1u;
+                const int s = (done + i) % kBStages;
+                const uint32_t ph = (uint32_t)((done + i) / kBStages) & 1u;
                 mb_wait(sm0 + oEmpty + 8 * s, ph ^ 1u, abort_flag, a.status);
                 if (*abort_flag) break;
                 const uint32_t full = sm0 + oFull + 8 * s, dst = b0 + s * kBStageBytes;
@@ -143,9 +156,9 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
         // ================= MMA issuer =================
         if (lane == 0) {
             for (int i = 0; i < ntile; ++i) {
-                const int s = i % kBStages, as = i % kAccSets;
-                mb_wait(sm0 + oTEmpty + 8 * as, ((uint32_t)(i / kAccSets) & 1u) ^ 1u, abort_flag, a.status);
-                mb_wait(sm0 + oFull + 8 * s, (uint32_t)(i / kBStages) & 1u, abort_flag, a.status);
+                const int s = (done + i) % kBStages, as = (done + i) % kAccSets;
+                mb_wait(sm0 + oTEmpty + 8 * as, ((uint32_t)((done + i) / kAccSets) & 1u) ^ 1u, abort_flag, a.status);
+                mb_wait(sm0 + oFull + 8 * s, (uint32_t)((done + i) / kBStages) & 1u, abort_flag, a.status);
                 if (*abort_flag) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // one descriptor per stage and for A; the k steps and the two M tiles only add compile-time constants
@@ -177,9 +190,9 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
         }
         double total = 0.0;
         for (int i = 0; i < ntile; ++i) {
-            const int as = i % kAccSets;
+            const int as = (done + i) % kAccSets;
             const int t0 = (tile0 + i) * kBN;
-            mb_wait(sm0 + oTFull + 8 * as, (uint32_t)(i / kAccSets) & 1u, abort_flag, a.status);
+            mb_wait(sm0 + oTFull + 8 * as, (uint32_t)((done + i) / kAccSets) & 1u, abort_flag, a.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             float acc = 0.f;
             if (!*abort_flag) {
@@ -229,23 +242,55 @@ probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_consta
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (threadIdx.x == 0) {
+        const double* red = reinterpret_cast<const double*>(smem + oRed);
+        // part slot of this item inside its unit: (layer, mblock, split); candidate selects the column
+        const int slot = (again ? pl.redo_slot0 : pl.slot0) + (layer * pl.mblocks + mblock) * nsplits + split;
+        a.part[((int64_t)unit * a.nptiles_max + slot) * 2 + cand] = red[0] + red[1] + red[2] + red[3];
+    }
+    if (!again || *abort_flag) break;
+    done += ntile;
+    }
     if (*abort_flag)
         for (int i = 0; i < 200; ++i) __nanosleep(1000);  // let copies and MMAs in flight finish before the memory goes away
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)kTmemCols) : "memory");
     }
-    if (threadIdx.x == 0) {
-        const double* red = reinterpret_cast<const double*>(smem + oRed);
-        // part slot of this item inside its unit: (layer, mblock, split); candidate selects the column
-        const int slot = pl.slot0 + (layer * pl.mblocks + mblock) * pl.nsplits + split;
-        a.part[((int64_t)unit * a.nptiles_max + slot) * 2 + cand] = red[0] + red[1] + red[2] + red[3];
-    }
 }
 
+// A second-moment sum has to be at least this part of the sum of |Q_r|^2 |R_j|^2: a quarter of what independent directions give
+// (1 / head_dim).  It is off by up to 3e-7 of that much, so an error that passes is off by about 1e-6.
+constexpr double kMomentShare = 1.0 / (4.0 * 128.0);
+
 // Rows [t0, t1) of every operand with the kept entries zeroed: the residual candidate's operand.  grid (blocks, units, operands
-// per unit), one 16-byte vector per thread and step.
-__global__ void __launch_bounds__(256) drop_rows_kernel(ProbeArgs a, int n_ops, int t0, int t1) {
+// per unit), one 16-byte vector per thread and step.  With second moments (gram part slots) it says which units are done again by
+// products, and forms all of their rows.
+__global__ void __launch_bounds__(256) drop_rows_kernel(ProbeArgs a, int n_ops, int t0, int t1, int gram) {
     const int unit = a.unit_begin + blockIdx.y;
+    if (gram > 0) {
+        __shared__ int s_redo;
+        if (threadIdx.x < 32) {
+            const double* p = a.part + (int64_t)unit * a.nptiles_max * 2;
+            const double* m = a.scale + (int64_t)unit * kMaxGramSlots * 2;
+            double v[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int i = threadIdx.x; i < gram; i += 32) {
+                v[0] += p[2 * i]; v[1] += p[2 * i + 1];
+                v[2] += m[2 * i]; v[3] += m[2 * i + 1];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int o = 16; o; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
+            // (written so that what is not a number counts as not exact enough)
+            const bool fine = v[0] >= kMomentShare * v[2] && v[1] >= kMomentShare * v[3] && isfinite(v[0]) && isfinite(v[1]);
+            if (threadIdx.x == 0) {
+                s_redo = !fine;
+                if (blockIdx.x == 0 && blockIdx.z == 0) a.redo[unit] = !fine;
+            }
+        }
+        __syncthreads();
+        if (s_redo) t0 = 0;
+    }
     const int64_t op = ((int64_t)unit * n_ops + blockIdx.z) * a.unit_stride;
     const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.z1) + op);
     uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.z1drop) + op);
@@ -257,7 +302,7 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(ProbeArgs a, int n_ops, 
 
 }  // namespace
 
-cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool* handled, int* nparts) {
+cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool* handled, ProbeParts* parts) {
     *handled = false;
     if (dtype != FDKV_BF16 || a.d != 128 || !a.tmap_z1 || !a.tmap_drop) return cudaSuccess;
     static PerDevice once;
@@ -292,21 +337,29 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     nsplits = ntiles > 0 ? (ntiles + pl.tiles_per_split - 1) / pl.tiles_per_split : 0;
     pl.nsplits = nsplits;
     pl.items_per_unit = a.B * pl.mblocks * 2 * nsplits;
-    const int slots = pl.slot0 + a.B * pl.mblocks * nsplits;
-    if (slots > a.nptiles_max) return cudaErrorInvalidValue;  // cannot happen: the part array is sized for max_probe_parts()
-    if (nsplits > 0) {
+    pl.sure_items = a.unit_count * pl.items_per_unit;
+    // units to do again: ranges of eight tiles as above, by as many blocks as run at one time
+    const bool shorts = pl.tiles_per_split <= kShortItem;
+    const int redo_blocks = pl.tile_first > 0 ? (shorts ? 2 : 1) * sm_count : 0;
+    pl.redo_nsplits = (pl.tile_first + 7) / 8;
+    pl.redo_tiles_per_split = 8;
+    pl.redo_per_unit = a.B * pl.mblocks * 2 * pl.redo_nsplits;
+    pl.redo_slot0 = pl.slot0 + a.B * pl.mblocks * nsplits;
+    const int slots = pl.redo_slot0 + a.B * pl.mblocks * pl.redo_nsplits;
+    if (slots > a.nptiles_max) return cudaErrorInvalidValue;  // cannot happen: the part array is sized for all of them
+    if (pl.sure_items + redo_blocks > 0) {
         const int t0 = pl.tile_first * kBN, t1 = std::min(a.T, pl.ntiles * kBN), n_ops = a.B == 4 ? 4 : 1;
-        const int blocks = (int)std::min<int64_t>(64, ((int64_t)(t1 - t0) * 16 + 255) / 256);
-        drop_rows_kernel<<<dim3(blocks, a.unit_count, n_ops), 256, 0, st>>>(a, n_ops, t0, t1);
+        const int blocks = (int)std::min<int64_t>(64, ((int64_t)std::max(t1 - t0, 1) * 16 + 255) / 256);
+        drop_rows_kernel<<<dim3(blocks, a.unit_count, n_ops), 256, 0, st>>>(a, n_ops, t0, t1, pl.slot0);
         const CUtensorMap &mz = *reinterpret_cast<const CUtensorMap*>(a.tmap_z1), &md = *reinterpret_cast<const CUtensorMap*>(a.tmap_drop);
-        if (pl.tiles_per_split <= kShortItem) probe_tc_kernel<1, 1><<<a.unit_count * pl.items_per_unit, kPThreads, probe_smem(1), st>>>(mz, md, a, pl);
-        else probe_tc_kernel<3, 2><<<a.unit_count * pl.items_per_unit, kPThreads, probe_smem(3), st>>>(mz, md, a, pl);
+        if (shorts) probe_tc_kernel<1, 1><<<pl.sure_items + redo_blocks, kPThreads, probe_smem(1), st>>>(mz, md, a, pl);
+        else probe_tc_kernel<3, 2><<<pl.sure_items + redo_blocks, kPThreads, probe_smem(3), st>>>(mz, md, a, pl);
         count_launch(2);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     count_kernel(FDKV_KERNEL_PROBE_TC);
-    *nparts = slots;
+    *parts = {pl.slot0, pl.redo_slot0, slots};
     *handled = true;
     return cudaSuccess;
 }

@@ -42,3 +42,39 @@ def test_probe_errors(block, hkv, group, T, pos):
 def test_products_of_short_prompts_and_items(hkv, T, pos):
     """The most keys that go to the products although every query sees them, and one tile more; items of eight tiles and of nine."""
     test_probe_errors(2, hkv, 1, T, pos)
+
+
+@pytest.mark.parametrize("block,group,W", [(2, 4, 64), (2, 8, 128), (4, 2, 16)])
+@pytest.mark.parametrize("eps", [1.0, 0.2, 0.03, 0.0])
+def test_queries_nearly_orthogonal_to_the_deviations(block, group, W, eps):
+    """Deviations in a random half of the directions, queries in the other half up to a share eps (and the rounding to bf16): the
+    second moments' sum cancels, the products do not.  A product is 8 steps of float32 rounded towards zero and its square, second
+    moments are 16 and 8: 2e-6 covers either and the float32 scores."""
+    from paper_2607_06519_b200 import binding as B
+
+    hkv, T, d = 2, 3100, 128
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+
+    def rand(*shape):
+        return torch.randn(shape, generator=g, device="cuda")
+
+    u, _ = torch.linalg.qr(rand(d, d))
+    x = [(rand(T, hkv, 64) @ u[:64]).bfloat16() for _ in range(block)]
+    q = [(rand(W, hkv * group, 64) @ u[64:] + eps * rand(W, hkv * group, 64) @ u[:64]).bfloat16() for _ in range(block)]
+    ctx = B.Context(B.Config(block, hkv * group, hkv, d, 1, T, 1, B.BF16, 1, 16, block_size=block))
+    ctx.compress_prefill(0, 0, 1, T, x, x)
+    pos = np.arange(T - W, T, dtype=np.int32)
+    _, scores = ctx.probe(0, 0, 1, q, pos, 0.0)
+    for h in range(hkv):
+        xs = [a[:, h].float().cpu().numpy() for a in x]
+        qs = [a.float().cpu().numpy() for a in q]
+        if block == 4:
+            u4 = R4.Unit4(xs, xs, True, 1, 16)
+            want = R4.probe_error4(u4.dev["k"], u4.kept["k"], qs, group, h, pos)
+        else:
+            u2 = R.Unit(*xs, *xs, True, 1, 16)
+            want = R.probe_error(u2.z1["k"], u2.kept["k"], qs[0], qs[1], group, h, pos)
+        np.testing.assert_allclose(scores[0, h].cpu().numpy(), want, rtol=2e-6)
+    assert ctx.device_status() == 0
+    ctx.close()
