@@ -158,6 +158,7 @@ fdkv_status fdkv_compress_prefill(fdkv_ctx* ctx, int32_t seq, int32_t pair_begin
  *   mode = argmin, ties to the lowest id.  The same mode applies to K and V.
  * q_layers: HOST array of n_layers DEVICE pointers to [W][n_q_heads][head_dim].
  * probe_pos: HOST int32[W], strictly ascending, each in [0, T).  1 <= W <= 128.
+ * A captured call carries the positions and the query pointers; its replays probe what the staging area holds then.
  * modes (may be NULL): DEVICE int32[pair_end-pair_begin][n_kv_heads].
  * scores (may be NULL): DEVICE float[pair_end-pair_begin][n_kv_heads][2] = {E(shared), E(residual)}.
  */

@@ -457,8 +457,7 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
     cudaStream_t st = S(stream);
     int32_t* pos_dev = wsp<int32_t>(c, c->ws.probe_pos);
     const void** qptr_dev = reinterpret_cast<const void**>(c->work + c->ws.probe_pos + kMaxW * 4);
-    CU(cudaMemcpyAsync(pos_dev, probe_pos, (size_t)W * 4, cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(qptr_dev + s.B * pb, q_layers + s.B * pb, (size_t)(pe - pb) * s.B * sizeof(void*), cudaMemcpyHostToDevice, st));
+    CU(launch_probe_inputs(pos_dev, probe_pos, W, qptr_dev, q_layers, s.B * pb, s.B * pe, st));
     ProbeArgs a;
     a.B = s.B;
     a.unit_begin = pb * s.Hkv; a.unit_count = (pe - pb) * s.Hkv;
@@ -504,12 +503,18 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
         for (int p = pb; p < pe; ++p) c->pair_scored[p] = 1;
     }
     CU(launch_probe(a, s.dtype, st));
-    const size_t su = (size_t)a.unit_begin * 16;
-    CU(cudaMemcpyAsync(c->pin + su, c->work + c->ws.scores + su, (size_t)a.unit_count * 16, cudaMemcpyDeviceToHost, st));
-    if (c->probe_recorded && c->probe_stream != st) CU(cudaStreamWaitEvent(st, c->probe_done, 0));
-    CU(cudaEventRecord(c->probe_done, st));
-    c->probe_stream = st;
-    c->probe_recorded = true;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CU(cudaStreamIsCapturing(st, &capture));
+    if (capture != cudaStreamCaptureStatusNone) {
+        c->probe_captured = true;  // (an event of a capture says nothing about its replays)
+    } else {
+        const size_t su = (size_t)a.unit_begin * 16;
+        CU(cudaMemcpyAsync(c->pin + su, c->work + c->ws.scores + su, (size_t)a.unit_count * 16, cudaMemcpyDeviceToHost, st));
+        if (c->probe_recorded && c->probe_stream != st) CU(cudaStreamWaitEvent(st, c->probe_done, 0));
+        CU(cudaEventRecord(c->probe_done, st));
+        c->probe_stream = st;
+        c->probe_recorded = true;
+    }
     for (int p = pb; p < pe; ++p) c->pair_probed[p] = 1;
     return FDKV_OK;
 }
@@ -522,7 +527,8 @@ fdkv_status fdkv_route_budget(fdkv_ctx* c, int32_t seq, size_t budget_bytes, dou
     for (int p = 0; p < s.P; ++p)
         if (!c->pair_probed[p]) return FDKV_ERR_STATE;
     CU(cudaStreamSynchronize(S(stream)));
-    CU(cudaEventSynchronize(c->probe_done));  // (probed on another stream)
+    if (c->probe_captured) CU(cudaMemcpy(c->pin, c->work + c->ws.scores, (size_t)s.NU * 16, cudaMemcpyDeviceToHost));
+    else CU(cudaEventSynchronize(c->probe_done));  // (probed on another stream)
     const double* const e = reinterpret_cast<const double*>(c->pin);
     // Omega of the staged sequence, as in fdkv_probe
     const int T = c->staged_T;

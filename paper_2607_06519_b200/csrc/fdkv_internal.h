@@ -163,6 +163,7 @@ struct fdkv_ctx {
     cudaEvent_t probe_done = nullptr;                   // the scores of every probe call so far have landed
     cudaStream_t probe_stream = nullptr;                // where it was recorded last
     bool probe_recorded = false;
+    bool probe_captured = false;                        // a probe call was captured: its replays leave the scores on the device only
     std::vector<uint8_t> pair_scored;            // token rule: the probe has chosen this pair's token sets
     bool packed_lists = false;              // decode runs the bf16 / head_dim 128 kernel on packed residual entries
     alignas(64) unsigned char tmap_u8[128]; // CUtensorMap of the arena as 128-byte rows (8-bit row streams)
@@ -253,6 +254,9 @@ struct ProbeArgs {
     int32_t* status;
 };
 cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st);
+// The probe positions and the query pointers of layers [layer_begin, layer_end) to the device, from HOST arrays.
+cudaError_t launch_probe_inputs(int32_t* pos_dev, const int32_t* pos, int W, const void** q_dev, const void* const* q_layers, int layer_begin, int layer_end,
+                                cudaStream_t st);
 constexpr int kMaxGramCtas = 160;  // blocks of the second-moment kernel
 constexpr int kMaxGramSlots = kMaxGramCtas + 2 * 4;  // ... and so part slots a unit may need
 // Part slots of a unit: [0, gram) second moments, [gram, sure) products, [sure, all) products in the place of the second moments

@@ -169,6 +169,32 @@ __global__ void __launch_bounds__(256) probe_finalize_kernel(ProbeArgs a, ProbeP
     }
 }
 
+// The positions and pointers travel in the launch parameters: a captured call carries them, and nothing is copied from pageable
+// memory.
+struct ProbeInputs {
+    int32_t pos[kMaxW];
+    const void* q[kSplitLayers];
+};
+__global__ void __launch_bounds__(kMaxW) probe_inputs_kernel(ProbeInputs in, int32_t* pos, int W, const void** q, int n) {
+    const int i = threadIdx.x;
+    if (i < W) pos[i] = in.pos[i];
+    if (i < n) q[i] = in.q[i];
+}
+static_assert(kSplitLayers <= kMaxW, "a thread per pointer");
+
+cudaError_t launch_probe_inputs(int32_t* pos_dev, const int32_t* pos, int W, const void** q_dev, const void* const* q_layers, int layer_begin, int layer_end,
+                                cudaStream_t st) {
+    ProbeInputs in = {};
+    for (int i = 0; i < W; ++i) in.pos[i] = pos[i];
+    for (int l = layer_begin; l < layer_end; l += kSplitLayers) {
+        const int n = layer_end - l < kSplitLayers ? layer_end - l : kSplitLayers;
+        for (int i = 0; i < n; ++i) in.q[i] = q_layers[l + i];
+        probe_inputs_kernel<<<1, kMaxW, 0, st>>>(in, pos_dev, W, q_dev + l, n);
+        count_launch(1);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool* handled, ProbeParts* parts);
 
 cudaError_t launch_probe(const ProbeArgs& a, int dtype, cudaStream_t st) {
