@@ -15,13 +15,13 @@
 //     warps 6-13: write the tile with its kept entries zeroed next to it; warp 1: both products, tokens on K, so the
 //     operands are MN-major views of the row-major tiles, A and B the same tile (8 + 8 tcgen05.mma, M = N = 128, K = 16);
 //     warps 2-5: epilogue.
-//   * Q^T Q of the segment's rows comes first, through the same ring and accumulators, a tile of 128 rows at a time: the epilogue
-//     adds the tiles up in a third 128-column region of tensor memory.
+//   * Q^T Q of the segment's rows comes first, through the same ring and accumulators, 32 rows at a time: the epilogue adds them up
+//     in a third 128-column region of tensor memory.
 //   * The sums are drained every two tiles, one candidate's while the other's products run: <R^T R, Q^T Q> in float32 over 32
 //     columns of a row, added up in float64.
 //   * Precision.  The tensor core rounds its accumulators towards zero, so what counts is the number of steps that one takes: 16 for
-//     R^T R (eight tiles per drain were 15 % faster and ten times less exact) and eight for Q^T Q (all rows in one accumulator: 1.3e-6
-//     off float64 at 512 rows, 5.5e-6 at 2 048).
+//     R^T R (the products: eight and a square) and two for Q^T Q (all rows in one accumulator: 1.3e-6 off float64 at 512 rows, 5.5e-6
+//     at 2 048; 128 rows: 6e-7).
 //     The sum cancels where queries and coefficients are nearly orthogonal, which the products, sums of squares, do not.  So the
 //     traces are kept too: tr(R^T R) tr(Q^T Q) is the sum of |Q_r|^2 |R_j|^2, and a unit whose error is a small part of it (or not
 //     finite) is done again by products (probe_tc.cu).
@@ -47,6 +47,7 @@ constexpr int kGSmem = kGHdr + kGStages * (kGStage + kGBits);  // 199 KiB
 constexpr int kGMaskWarps = 8;
 constexpr int kGThreads = (6 + kGMaskWarps) * 32;
 constexpr int kGroup = 2;                 // tiles per drain
+constexpr int kQSteps = 2;                // steps of 16 probe rows per drain
 constexpr int kGColF = 0, kGColD = 128, kGColA = 256;  // tensor memory: R^T R of both candidates, Q^T Q
 constexpr uint32_t kGIdesc = umma_idesc(128, 128, true);
 // (accumulator barriers: the shared candidate's at +0, the residual's at +8)
@@ -138,23 +139,33 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t df = smem_desc_sw128(stage0 + s * kGStage, kGHalf, 1024);
                     const uint64_t dd = smem_desc_sw128(stage0 + s * kGStage + kGTile, kGHalf, 1024);
+                    auto open = [&](int c) {
+                        mb_wait(sm0 + gAccEmpty + 8 * c, ((c ? gen1 : gen0) & 1u) ^ 1u, abort_flag, a.status);
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    };
+                    auto close = [&](int c) {
+                        umma_commit(sm0 + gAccFull + 8 * c);
+                        if (c) ++gen1; else ++gen0;
+                    };
+                    if (i < 0) {  // probe rows: kQSteps steps per drain, the accumulators in turn
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        // probe rows: a tile per drain, the accumulators in turn.  Tokens: one candidate's accumulator is drained while
-                        // the other's products run.
-                        if (i < 0 && ((i + pl.qtiles) & 1) != c) continue;
-                        const bool opens = i < 0 || i % kGroup == 0, closes = i < 0 || i % kGroup == kGroup - 1 || i == n - 1;
-                        if (opens) {
-                            mb_wait(sm0 + gAccEmpty + 8 * c, ((c ? gen1 : gen0) & 1u) ^ 1u, abort_flag, a.status);
-                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        for (int k = 0; k < 8; ++k) {
+                            const int c = k / kQSteps & 1;
+                            if (k % kQSteps == 0) open(c);
+                            umma_ss<kGIdesc>(tmem + (c ? kGColD : kGColF), dd + k * (2048 >> 4), dd + k * (2048 >> 4), k % kQSteps > 0);
+                            if (k % kQSteps == kQSteps - 1) close(c);
                         }
-                        const uint64_t desc = c || i < 0 ? dd : df;
-                        const uint32_t acc = tmem + (c ? kGColD : kGColF);
+                    } else {
+                        // one candidate's accumulator is drained while the other's products run
+                        const bool opens = i % kGroup == 0, closes = i % kGroup == kGroup - 1 || i == n - 1;
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) umma_ss<kGIdesc>(acc, desc + k * (2048 >> 4), desc + k * (2048 >> 4), k > 0 || !opens);
-                        if (closes) {
-                            umma_commit(sm0 + gAccFull + 8 * c);
-                            if (c) ++gen1; else ++gen0;
+                        for (int c = 0; c < 2; ++c) {
+                            if (opens) open(c);
+                            const uint64_t desc = c ? dd : df;
+#pragma unroll
+                            for (int k = 0; k < 8; ++k)
+                                umma_ss<kGIdesc>(tmem + (c ? kGColD : kGColF), desc + k * (2048 >> 4), desc + k * (2048 >> 4), k > 0 || !opens);
+                            if (closes) close(c);
                         }
                     }
                     umma_commit(sm0 + gEmpty + 8 * s);
@@ -168,13 +179,17 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
         const int lq = warp & 3;
         const uint32_t tq = tmem + ((uint32_t)(lq * 32) << 16);
         uint32_t gen0 = 0, gen1 = 0;  // drains of either accumulator
-        // block b of this row's moments; the diagonal element if it is there
+        // this row's diagonal element, if it is in these columns' block b (picked by the bits of the lane)
         auto diagonal = [&](int b, const uint32_t (&r)[32]) {
-            float x = 0.f;
-            if (b == lq)
+            if (b != lq) return 0.f;
+            uint32_t x[16];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) x = j == lane ? __uint_as_float(r[j]) : x;
-            return x;
+            for (int j = 0; j < 16; ++j) x[j] = lane & 16 ? r[j + 16] : r[j];
+#pragma unroll
+            for (int w = 8; w; w >>= 1)
+#pragma unroll
+                for (int j = 0; j < w; ++j) x[j] = lane & w ? x[j + w] : x[j];
+            return __uint_as_float(x[0]);
         };
         auto await = [&](int c) {
             mb_wait(sm0 + gAccFull + 8 * c, (c ? gen1 : gen0) & 1u, abort_flag, a.status);
@@ -188,10 +203,11 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
         };
         for (int64_t g = g_begin; g < g_end;) {
             const int op = (int)(g / pl.nt), t0 = (int)(g % pl.nt), n = (int)min((int64_t)pl.nt - t0, g_end - g);
-            double sum0 = 0.0, sum1 = 0.0, tr0 = 0.0, tr1 = 0.0;
-            float tr_q = 0.f;
+            double sum0 = 0.0, sum1 = 0.0;
+            float tr0 = 0.f, tr1 = 0.f, tr_q = 0.f;  // (only a measure: a few digits will do)
+            const int qdrains = pl.qtiles * (8 / kQSteps);
 #pragma unroll 1
-            for (int q = 0; q < pl.qtiles; ++q) {
+            for (int q = 0; q < qdrains; ++q) {
                 const int c = q & 1;
                 await(c);
                 if (!*abort_flag) {
@@ -204,7 +220,7 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
 #pragma unroll
                         for (int j = 0; j < 32; ++j) rr[j] = q > 0 ? __float_as_uint(__uint_as_float(rr[j]) + __uint_as_float(ra[j])) : rr[j];
                         tmem_st32(tq + kGColA + b * 32, rr);
-                        if (q == pl.qtiles - 1) tr_q += diagonal(b, rr);
+                        if (q == qdrains - 1) tr_q += diagonal(b, rr);
                     }
                     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 }
@@ -217,7 +233,7 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
                     if (!*abort_flag) {
                         double e = 0.0;
                         float dg = 0.f;
-#pragma unroll 1
+#pragma unroll 2
                         for (int b = 0; b < 4; ++b) {  // (unrolled it takes more registers than a thread has)
                             uint32_t rr[32], ra[32];
                             tmem_ld32(tq + (c ? kGColD : kGColF) + b * 32, rr);
@@ -233,13 +249,13 @@ probe_gram_kernel(const __grid_constant__ CUtensorMap tmap, ProbeArgs a, GramPla
                             dg += diagonal(b, rr);
                         }
                         (c ? sum1 : sum0) += e;
-                        (c ? tr1 : tr0) += (double)dg;
+                        (c ? tr1 : tr0) += dg;
                     }
                     drained(c);
                 }
             }
             // the four warps' five sums: both candidates' errors and traces, the queries' trace
-            double v[5] = {sum0, sum1, tr0, tr1, (double)tr_q};
+            double v[5] = {sum0, sum1, (double)tr0, (double)tr1, (double)tr_q};
             double* const red = reinterpret_cast<double*>(smem + gRed);
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
