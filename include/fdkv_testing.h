@@ -1,7 +1,7 @@
 /*
  * Test hooks of libfdkv.  Not part of the product API (include/fdkv.h): nothing here computes a step of the method.
  * They let the test-suite reach two pieces of failure handling that a healthy run never enters, without making a GPU
- * fault, trap or hang.  (The paper has no counterpart.)
+ * fault, trap or hang, and run either form of the probe at small sizes.  (The paper has no counterpart.)
  */
 #ifndef FDKV_TESTING_H
 #define FDKV_TESTING_H
@@ -21,6 +21,12 @@ extern "C" {
  */
 fdkv_status fdkv_test_wait_expiry(fdkv_ctx* ctx, int32_t poll_cap, void* stream);
 fdkv_status fdkv_test_clear_device_status(fdkv_ctx* ctx, void* stream);
+
+/*
+ * Which form the probe of a bf16 / head_dim 128 context with the entry rule takes for the keys that every query sees: 0 the
+ * library's rule, 1 second moments, 2 products.  Per context, until changed.
+ */
+fdkv_status fdkv_test_probe_moments(fdkv_ctx* ctx, int32_t form);
 
 /*
  * The per-device set-up table of the launchers (function attributes are per device, not per process), driven with a

@@ -474,6 +474,7 @@ fdkv_status fdkv_probe(fdkv_ctx* c, int32_t seq, int32_t pb, int32_t pe, const v
     a.part = wsp<double>(c, c->ws.probe_part);
     a.scale = wsp<double>(c, c->ws.probe_scale);
     a.redo = wsp<int32_t>(c, c->ws.probe_redo);
+    a.moments = c->probe_moments;
     a.scores = wsp<double>(c, c->ws.scores);
     a.modes = wsp<int32_t>(c, c->ws.modes);
     a.lambda = lambda;

@@ -163,6 +163,7 @@ struct fdkv_ctx {
     cudaEvent_t probe_done = nullptr;                   // the scores of every probe call so far have landed
     cudaStream_t probe_stream = nullptr;                // where it was recorded last
     bool probe_recorded = false;
+    int probe_moments = 0;                              // ProbeArgs::moments (set by tests)
     bool probe_captured = false;                        // a probe call was captured: its replays leave the scores on the device only
     std::vector<uint8_t> pair_scored;            // token rule: the probe has chosen this pair's token sets
     bool packed_lists = false;              // decode runs the bf16 / head_dim 128 kernel on packed residual entries
@@ -239,6 +240,7 @@ struct ProbeArgs {
     const int32_t* pos;
     double* part;    // [NU][nptiles_max][2]
     double* scale;   // [NU][kMaxGramSlots][2] what the second moments' sums are to be large against
+    int moments;     // second moments where they pay (0), for all keys that every query sees (1: tests), never (2: tests)
     int32_t* redo;   // [NU] the second moments' sums are not exact enough: the unit is done again by products
     double* scores;  // [NU][2]
     int32_t* modes;  // [NU]

@@ -22,6 +22,7 @@
 // Every mbarrier wait is bounded; on expiry the CTA flags the device status word, stops waiting and still frees
 // its tensor memory before it retires.
 #include <algorithm>
+#include <cmath>
 
 #include "fdkv_internal.h"
 #include "umma.cuh"
@@ -59,11 +60,10 @@ struct TcPlan {
 };
 
 // kBStages, kAccSets: three and two for items of many tiles; one and one for items of a tile or two, whose time is the chain from
-// the loads to the sum: two such blocks share an SM.  Us a probe of 32 layers, one block against two per SM: 300 tokens (one or
-// two tiles) 87 and 64, 1k (four) 110 and 89, 2k (eight) 143 and 128, 8k by products alone (nine or more) 338 and 363.
+// the loads to the sum: two such blocks share an SM where there are that many.  Us a probe of 32 layers, one block against two per
+// SM: 300 tokens (one or two tiles) 87 and 64, 1k (four) 110 and 89, 2k (eight) 143 and 128, 8k by products alone (nine or more) 338
+// and 363; 128 items of seven tiles 37 and 42.
 constexpr int kShortItem = 8;
-// 256-key tiles that every query sees up to which the product takes them too (see launch_probe_tc)
-constexpr int kGramTiles = 4;
 template <int kBStages, int kAccSets>
 __global__ void __launch_bounds__(kPThreads, kBStages == 1 ? 2 : 1)
 probe_tc_kernel(const __grid_constant__ CUtensorMap tmap_z1, const __grid_constant__ CUtensorMap tmap_drop, ProbeArgs a, TcPlan pl) {
@@ -302,6 +302,46 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(ProbeArgs a, int n_ops, 
 
 }  // namespace
 
+// How `base` items of `tiles` 256-key tiles are cut: so that the grid fills the machine several times over, but ranges of eight tiles
+// or more.
+struct Cut {
+    int nsplits, per_split;
+};
+static Cut cut_tiles(int base, int tiles, int sms) {
+    if (tiles <= 0) return {0, 0};
+    const int n = std::max(1, std::min((4 * sms + base - 1) / base, (tiles + 7) / 8)), per = (tiles + n - 1) / n;
+    return {(tiles + per - 1) / per, per};
+}
+static bool short_items(int items, int per_split, int sms) { return per_split <= kShortItem && items > sms; }
+
+// Whether second moments of the first `tiles` 256-key tiles take less time than their products; both estimated in us, from what the
+// parts took.  Products: turns of the device (3.5 us and 0.85 a tile; two blocks per SM 1.5), or the keys' bytes, and the
+// residual candidate's copy of the keys.  Moments: a thread block forms every operand's Q^T Q in each segment that it works on (4 us
+// per 128 rows, 6 where the queries of all units crowd L2) before its own tiles (1.6, both candidates).  Us a probe call, products of
+// all keys against moments:
+//   pairs, 512 rows an operand:    2 operands 8k keys 40 and 53; 16 operands 4k 47 and 73, 8k 73 and 77, 16k 130 and 87;
+//                                  128 operands 1k 88 and 105, 2k 132 and 123, 32k 1 214 and 428
+//   pairs, 2 048 rows an operand:  16 operands 8k 161 and 172, 16k 267 and 191; 128 operands 2k 323 and 366, 3k 419 and 382
+//   pairs, 8 rows an operand:      2 operands 8k 44 and 38; 16 operands 3k 43 and 48, 8k 56 and 52
+//   blocks of four, 256 rows:      32 operands 4k 51 and 61, 8k 89 and 73; 1 024 rows 8k 184 and 131
+static bool moments_pay(const ProbeArgs& a, int tiles, int sms) {
+    if (tiles <= 0) return false;
+    const int mblocks = (a.G * a.W + 127) / 128, base = a.unit_count * a.B * mblocks * 2;
+    const double ops = (double)a.unit_count * (a.B == 4 ? 4 : 1);
+    const Cut cut = cut_tiles(base, tiles, sms);
+    const bool shorts = short_items(base * cut.nsplits, cut.per_split, sms);
+    const double turns = std::ceil((double)base * cut.nsplits / (shorts ? 2 * sms : sms));
+    const double tile_bytes = kBN * 256.0, rate = 6e6;  // (bytes per us)
+    const double products = std::max(turns * (3.5 + cut.per_split * (shorts ? 1.5 : 0.85)), (double)a.unit_count * a.B * 2 * tiles * tile_bytes / rate) +
+                            ops * tiles * 2 * tile_bytes / rate;
+    const double qtiles = ((a.B == 4 ? 1 : a.B) * a.G * a.W + 127) / 128, per_op = 2.0 * tiles, all = ops * per_op;
+    const double per_block = std::ceil(all / std::min<double>(std::min(sms, kMaxGramCtas), all));
+    const double segments = per_block <= 1 ? 1 : 1 + std::ceil((per_block - 1) / per_op);
+    const double q_bytes = (double)a.unit_count * a.B * a.G * a.W * 256.0;
+    const double moments = 4.0 + segments * qtiles * (q_bytes > 32e6 ? 6.0 : 4.0) + per_block * 1.6;
+    return 1.1 * moments < products;
+}
+
 cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool* handled, ProbeParts* parts) {
     *handled = false;
     if (dtype != FDKV_BF16 || a.d != 128 || !a.tmap_z1 || !a.tmap_drop) return cudaSuccess;
@@ -320,9 +360,7 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     // copy of Z1 and 2 x 2 x rows x 128 flops here; 32 layers of 32k tokens, 512 rows per pair: 1 190 -> 320 us with this
     // kernel's share of the last keys)
     pl.tile_first = (pl.pos_min + 1) / kBN;
-    // ... from a range on that pays for the fixed part, every unit's queries times its moments (us, 32 layers, product of all
-    // keys against moments: 1k tokens 89 and 100, 2k 128 and 117, 4k 208 and 149; blocks of four 1k 105 and 110, 4k 256 and 175)
-    if (pl.tile_first <= kGramTiles) pl.tile_first = 0;
+    if (a.moments == 0 ? !moments_pay(a, pl.tile_first, sm_count) : a.moments == 2) pl.tile_first = 0;
     pl.slot0 = 0;
     if (pl.tile_first > 0) {
         cudaError_t e = launch_probe_gram(a, pl.tile_first * kBN, st, &pl.slot0);
@@ -330,16 +368,14 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     }
     const int ntiles = pl.ntiles - pl.tile_first;
     pl.mblocks = (a.G * a.W + 128 * kMT - 1) / (128 * kMT);
-    const int base_items = a.unit_count * a.B * pl.mblocks * 2;
-    // split the key range so that the grid fills the machine several times over, but keep >= 8 tiles per item
-    int nsplits = std::max(1, std::min((4 * sm_count + base_items - 1) / base_items, (ntiles + 7) / 8));
-    pl.tiles_per_split = (ntiles + nsplits - 1) / std::max(1, nsplits);
-    nsplits = ntiles > 0 ? (ntiles + pl.tiles_per_split - 1) / pl.tiles_per_split : 0;
+    const Cut cut = cut_tiles(a.unit_count * a.B * pl.mblocks * 2, ntiles, sm_count);
+    const int nsplits = cut.nsplits;
+    pl.tiles_per_split = cut.per_split;
     pl.nsplits = nsplits;
     pl.items_per_unit = a.B * pl.mblocks * 2 * nsplits;
     pl.sure_items = a.unit_count * pl.items_per_unit;
     // units to do again: ranges of eight tiles as above, by as many blocks as run at one time
-    const bool shorts = pl.tiles_per_split <= kShortItem;
+    const bool shorts = short_items(pl.sure_items, pl.tiles_per_split, sm_count);
     const int redo_blocks = pl.tile_first > 0 ? (shorts ? 2 : 1) * sm_count : 0;
     pl.redo_nsplits = (pl.tile_first + 7) / 8;
     pl.redo_tiles_per_split = 8;

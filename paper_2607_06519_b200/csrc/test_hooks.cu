@@ -47,6 +47,12 @@ fdkv_status fdkv_test_clear_device_status(fdkv_ctx* c, void* stream) {
     return e == cudaSuccess ? FDKV_OK : fdkv::record_cuda_error(e);
 }
 
+fdkv_status fdkv_test_probe_moments(fdkv_ctx* c, int32_t form) {
+    if (!c || form < 0 || form > 2) return FDKV_ERR_INVALID_ARG;
+    c->probe_moments = form;
+    return FDKV_OK;
+}
+
 int32_t fdkv_test_per_device_visits(const int32_t* devs, int32_t n) {
     if (!devs || n < 0) return -1;
     return fdkv::per_device_first_visits(reinterpret_cast<const int*>(devs), n);

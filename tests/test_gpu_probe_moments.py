@@ -78,3 +78,53 @@ def test_queries_nearly_orthogonal_to_the_deviations(block, group, W, eps):
         np.testing.assert_allclose(scores[0, h].cpu().numpy(), want, rtol=2e-6)
     assert ctx.device_status() == 0
     ctx.close()
+
+
+@pytest.fixture
+def moments(monkeypatch):
+    """Every probe call takes second moments for all keys that every query sees, however few."""
+    from paper_2607_06519_b200 import binding as B
+
+    probe = B.Context.probe
+
+    def always(self, *args, **kw):
+        assert B._lib.fdkv_test_probe_moments(self.h, 1) == 0
+        return probe(self, *args, **kw)
+
+    monkeypatch.setattr(B.Context, "probe", always)
+
+
+@pytest.mark.parametrize("block", [2, 4])
+@pytest.mark.parametrize("hkv,group,T,pos", [
+    (1, 1, 257, [254]), (1, 1, 257, [255]), (1, 2, 300, [256, 299]), (2, 4, 1000, range(990, 1000)), (1, 1, 20000, [19999]),
+    (3, 4, 700, range(600, 700)), (8, 4, 2049, range(1985, 2049)), (2, 8, 5000, range(4900, 5000)), (2, 1, 1100, [511, 512, 1023, 1024]),
+])
+def test_probe_errors_by_moments(block, hkv, group, T, pos, moments):
+    test_probe_errors(block, hkv, group, T, pos)
+
+
+@pytest.mark.parametrize("block,group,W", [(2, 4, 64), (2, 8, 128), (4, 2, 16)])
+@pytest.mark.parametrize("eps", [1.0, 0.2, 0.03, 0.0])
+def test_queries_nearly_orthogonal_by_moments(block, group, W, eps, moments):
+    test_queries_nearly_orthogonal_to_the_deviations(block, group, W, eps)
+
+
+@pytest.mark.parametrize("layers,hkv,group,W,T", [(32, 8, 4, 64, 1400), (32, 8, 4, 64, 2300), (8, 8, 1, 4, 2100), (8, 8, 1, 4, 4200)])
+def test_either_side_of_the_rule(layers, hkv, group, W, T):
+    """Where the rule turns from products to moments: both forms of the same call, and the rule's."""
+    from paper_2607_06519_b200 import binding as B
+
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    k = [torch.randn((T, hkv, 128), generator=g, device="cuda").bfloat16() for _ in range(layers)]
+    q = [torch.randn((W, hkv * group, 128), generator=g, device="cuda").bfloat16() for _ in range(layers)]
+    ctx = B.Context(B.Config(layers, hkv * group, hkv, 128, 1, T, 1, B.BF16, 1, 16))
+    ctx.compress_prefill(0, 0, layers // 2, T, k, k)
+    got = []
+    for form in (2, 1, 0):
+        assert B._lib.fdkv_test_probe_moments(ctx.h, form) == 0
+        got.append(ctx.probe(0, 0, layers // 2, q, np.arange(T - W, T, dtype=np.int32), 0.0)[1].double().cpu().numpy())
+    np.testing.assert_allclose(got[1], got[0], rtol=2e-6)
+    assert np.array_equal(got[2], got[0]) or np.array_equal(got[2], got[1])
+    assert ctx.device_status() == 0
+    ctx.close()
