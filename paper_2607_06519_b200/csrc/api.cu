@@ -247,6 +247,7 @@ CompressArgs entry_args(fdkv_ctx* c, int T) {
     a.chunk_base = wsp<int2>(c, c->ws.chunk_base);
     a.cand_stride = s.cand_stride; a.chunks_max = s.chunks_max;
     a.n_keep = (int64_t)T * s.d * s.keep_num / s.keep_den; a.kcap = s.kcap;
+    a.in_place = false;
     a.ntiles_max = s.ntiles_max;
     a.tile_off = wsp<int32_t>(c, c->ws.tile_off);
     a.idx = wsp<int32_t>(c, c->ws.idx);

@@ -317,7 +317,9 @@ extern "C" fdkv_status fdkv_compress_unit_noalloc(const void* x0, const void* x1
     a.cand_n = reinterpret_cast<int32_t*>(sc + kNaCount);
     a.chunk_base = reinterpret_cast<int2*>(sc + kNaBase);
     a.cand_stride = kNoAllocMaxElems; a.chunks_max = (int)kNoAllocChunks;
-    a.n_keep = k; a.kcap = 0; a.ntiles_max = (int)kNoAllocMaxTiles;
+    a.n_keep = k; a.kcap = 0;
+    a.in_place = false;
+    a.ntiles_max = (int)kNoAllocMaxTiles;
     a.tile_off = reinterpret_cast<int32_t*>(sc + kNaOff);
     a.idx = idx_out; a.val = val_out; a.packed = nullptr;
     a.keep = nullptr; a.keep_stride = 0;

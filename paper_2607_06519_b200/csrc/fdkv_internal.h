@@ -211,6 +211,7 @@ struct CompressArgs {
     int chunks_max;
     int chunks;           // set by launch_compress: chunks of T tokens
     int64_t n_keep, kcap; // entries per list and list capacity
+    bool in_place;        // z0 may be written where a layer's rows are
     int ntiles_max;
     int32_t* tile_off;    // [NT][ntiles_max + 1]
     int32_t* idx;         // [NT][kcap]

@@ -13,13 +13,14 @@
 //                        fixed jitter; all of them where there are no more) and sets a bound that about 1.2 k positions reach;
 //   2. split_kernel      reads every row once, writes Z0 (and, of K, the high-frequency rows the probe reads) and appends the
 //                        positions that reach the bound, in order, to the chunk's candidate list;
-//   3. threshold_kernel  one block per unit-tensor: the k-th largest key among the candidates (a radix select in shared
-//                        memory), then the keys above and equal to it before every chunk;
+//   3. threshold_kernel  one block per unit-tensor (a cluster of them for few and long ones): the k-th largest key among the
+//                        candidates (a radix select in shared memory), then the keys above and equal to it before every chunk;
 //   4. compact_kernel    one block per chunk: candidates -> the lists, the offsets of the 16-token tiles and, of K, a bit
 //                        map of the kept positions.
 // (Few short unit-tensors take small_kernel instead of all of these.)
 // The bound is only a guess: where fewer than k positions reach it, step 3 says so and steps 2 and 3 run again for that
-// unit-tensor with bound 0 (a chunk's list holds all of its positions), so the result never depends on the sample.
+// unit-tensor with bound 0 (a chunk's list holds all of its positions), so the result never depends on the sample.  Where most
+// positions are kept, or where Z0 overwrites the rows, every position is a candidate from the start.
 // Bound by HBM: K and V are read once and about k / N x 1.2 of them written again; a pass that writes all high-frequency
 // values and reads them back to select (what this replaces) moved 5 instead of 3.6 times a tensor's bytes, and its
 // histogram of every key took 128 KiB of shared memory, one block per SM.
@@ -37,6 +38,8 @@ constexpr int kSampleThreads = 512, kSampleBins = 4096;
 constexpr int64_t kSampleElems = 65536;
 constexpr int kThrThreads = 1024, kThrBins = 4096;
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;  // a bound or threshold above every key
+// Of the positions are kept: from there on every position is taken for a candidate (4 layers of 32k tokens, all kept, 2 940 -> 906 us).
+constexpr double kAllShare = 0.6;
 
 // two float32 operations at a time, each rounded to nearest
 typedef unsigned long long f32x2;
@@ -281,7 +284,8 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, 
 // block barrier per item (the warps' counts).  The issue slots are as busy as HBM here, hence the packed arithmetic, the
 // bit tricks and the running item coordinates (with scalar arithmetic, a binary search per list entry and divisions per item:
 // 1 550 us for 32 layers of 32k tokens).
-template <typename T, int B>
+// ALL: every position is a candidate, the values go to the list in their order and no positions are written (see kAllShare).
+template <typename T, int B, bool ALL>
 __global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a, int items, int redo) {
     constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
     constexpr int CE = compress_chunk(B, (int)sizeof(T)), NV = CE / kSplitThreads / 8;
@@ -353,12 +357,13 @@ __global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a,
     for (int it = 0; left > 0; --left, it ^= 1, advance(now)) {
         const int ut = a.ut_base + now.blk * uts + now.u;
         const int64_t e0 = (int64_t)now.chunk * CE;
-        const uint32_t lo = a.sel[ut].lo;
+        const uint32_t lo = ALL ? 0u : a.sel[ut].lo;
         uint8_t* const st = smem + it * STAGE;
         asm volatile("cp.async.wait_group 1;" ::: "memory");
-        if (!redo || a.sel[ut].redo) {  // (block-uniform)
+        if (ALL || !redo || a.sel[ut].redo) {  // (block-uniform)
             const int h = now.u / a.tensors;
             const bool is_k = now.u == h * a.tensors;
+            T* const val = reinterpret_cast<T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0;
             T* const z0 = reinterpret_cast<T*>(a.z0) + (int64_t)ut * a.z0_stride + e0 + p0;
             T* const z1 = a.z1 && is_k ? reinterpret_cast<T*>(a.z1) + (int64_t)(now.blk * a.Hkv + h + a.ut_base / a.tensors) * NB * a.unit_stride + e0 + p0 : nullptr;
 #pragma unroll
@@ -371,20 +376,26 @@ __global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a,
 #pragma unroll
                         for (int k = 0; k < Q; ++k) x[l][k] = reinterpret_cast<const uint4*>(st + l * ROW + (p0 + 256 * q) * sizeof(T))[k];
                     Eight<T, B>::split(x, z, hf);
-                    m8 = Eight<T, B>::reach(hf, lo);
+                    if constexpr (!ALL) m8 = Eight<T, B>::reach(hf, lo);
 #pragma unroll
                     for (int k = 0; k < Q; ++k) {
                         if (!redo) reinterpret_cast<uint4*>(z0 + 256 * q)[k] = z[k];
 #pragma unroll
                         for (int l = 0; l < NB; ++l) {
                             if (z1 && !redo) reinterpret_cast<uint4*>(z1 + (int64_t)l * a.unit_stride + 256 * q)[k] = hf[l][k];
-                            reinterpret_cast<uint4*>(st + l * ROW + (p0 + 256 * q) * sizeof(T))[k] = hf[l][k];
+                            if constexpr (ALL) reinterpret_cast<uint4*>(val + (int64_t)l * a.cand_stride + p0 + 256 * q)[k] = hf[l][k];
+                            else reinterpret_cast<uint4*>(st + l * ROW + (p0 + 256 * q) * sizeof(T))[k] = hf[l][k];
                         }
                     }
                 }
-                reinterpret_cast<uint8_t*>(s_map[warp])[32 * q + lane] = (uint8_t)m8;
+                if constexpr (!ALL) reinterpret_cast<uint8_t*>(s_map[warp])[32 * q + lane] = (uint8_t)m8;
             }
             __syncwarp();
+            if constexpr (ALL) {
+                if (tid == 0) a.cand_n[(int64_t)ut * a.chunks_max + now.chunk] = (int32_t)min((int64_t)CE, n_e - e0);
+                request_next(it);
+                continue;
+            }
             // the lane's BITS consecutive positions of the warp's part
             uint32_t bits = BITS == 32   ? s_map[warp][lane]
                             : BITS == 16 ? (uint32_t)reinterpret_cast<const uint16_t*>(s_map[warp])[lane]
@@ -408,13 +419,20 @@ __global__ void __launch_bounds__(kSplitThreads, 3) split_kernel(CompressArgs a,
             cs ^= 1;
             if (tid == 0) a.cand_n[(int64_t)ut * a.chunks_max + now.chunk] = (int32_t)n;
             uint16_t* const pos = a.cand_pos + (int64_t)ut * a.cand_stride + e0;
-            T* const val = reinterpret_cast<T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0;
             const uint32_t first = warp * (NV * 256) + lane * BITS;
-            for (; bits; bits &= bits - 1, ++at) {
-                const uint32_t p = first + __ffs((int)bits) - 1;
-                pos[at] = (uint16_t)p;
+            // positions into shared memory, then both lists in runs (two-byte stores at every lane's own place took most of the time
+            // where many positions are candidates: keep 1/2, 32k tokens, 1 080 of 1 740 us)
+            uint16_t* const s_pos = B == 2 ? reinterpret_cast<uint16_t*>(st + ROW + warp * (NV * 256) * sizeof(T))  // (a layer's rows that are done with)
+                                           : reinterpret_cast<uint16_t*>(smem + 2 * STAGE) + warp * (NV * 256);
+            for (uint32_t i = incl - mine; bits; bits &= bits - 1, ++i) s_pos[i] = (uint16_t)(first + __ffs((int)bits) - 1);
+            const uint32_t n_w = __shfl_sync(0xFFFFFFFFu, incl, 31);
+            at -= incl - mine;  // the warp's first
+            __syncwarp();
+            for (uint32_t i = lane; i < n_w; i += 32) {
+                const uint32_t p = s_pos[i];
+                pos[at + i] = (uint16_t)p;
 #pragma unroll
-                for (int l = 0; l < NB; ++l) val[(int64_t)l * a.cand_stride + at] = reinterpret_cast<const T*>(st + l * ROW)[p];
+                for (int l = 0; l < NB; ++l) val[(int64_t)l * a.cand_stride + at + i] = reinterpret_cast<const T*>(st + l * ROW)[p];
             }
             __syncwarp();  // (the warp's part of the stage is read)
         }
@@ -447,6 +465,53 @@ __device__ __forceinline__ void each_candidate(const CompressArgs& a, int ut, in
             if (m >= 8) Eight<T, B>::keys(v[s], [&](int, uint32_t key) { f(key); });
             else if (m > 0) Eight<T, B>::keys(v[s], [&](int j, uint32_t key) { if (j < m) f(key); });
         }
+    }
+}
+
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the sum over the cluster of two consecutive 32-bit words at a shared-memory address, all loads in flight together
+__device__ __forceinline__ uint2 cluster_sum2(uint32_t addr, int blocks) {
+    uint2 v[8], sum = make_uint2(0, 0);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        uint32_t at;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(r < blocks ? r : 0));
+        asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v[r].x), "=r"(v[r].y) : "r"(at));
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+        if (r < blocks) { sum.x += v[r].x; sum.y += v[r].y; }
+    return sum;
+}
+
+// counts of chunks [c_begin, c_end) (written by this block, a barrier ago) -> counts before each, the two given ones included
+__device__ __forceinline__ void scan_chunks(int2* base, int c_begin, int c_end, uint32_t run_gt, uint32_t run_eq, uint32_t (&s_sum)[2][32]) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int c0 = c_begin; c0 < c_end; c0 += kThrThreads) {
+        const int c = c0 + tid;
+        const int2 m = c < c_end ? base[c] : make_int2(0, 0);
+        uint32_t ig = (uint32_t)m.x, ie = (uint32_t)m.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t yg = __shfl_up_sync(0xFFFFFFFFu, ig, o), ye = __shfl_up_sync(0xFFFFFFFFu, ie, o);
+            if (lane >= o) { ig += yg; ie += ye; }
+        }
+        __syncthreads();
+        if (lane == 31) { s_sum[0][warp] = ig; s_sum[1][warp] = ie; }
+        __syncthreads();
+        uint32_t tg = 0, te = 0, bg = run_gt, be = run_eq;
+#pragma unroll
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) { bg += s_sum[0][w]; be += s_sum[1][w]; }
+            tg += s_sum[0][w];
+            te += s_sum[1][w];
+        }
+        if (c < c_end) base[c] = make_int2((int)(bg + ig) - m.x, (int)(be + ie) - m.y);
+        run_gt += tg;
+        run_eq += te;
     }
 }
 
@@ -541,30 +606,122 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
         }
     }
     __syncthreads();
-    uint32_t run_gt = 0, run_eq = 0;
-    for (int c0 = 0; c0 < chunks; c0 += kThrThreads) {
-        const int c = c0 + tid;
-        const int2 m = c < chunks ? base[c] : make_int2(0, 0);
-        uint32_t ig = (uint32_t)m.x, ie = (uint32_t)m.y;
+    scan_chunks(base, 0, chunks, 0, 0, s_sum);
+}
+
+// The same by a cluster of `blocks` blocks per unit-tensor, a range of its chunks each: few unit-tensors of many candidates leave most of
+// the device to others otherwise (64 of 32k x 128 positions at keep 1/8: 119 us by a block each), and where every position is a candidate.
+// Where all entries are kept there is nothing to look for.
+template <typename T, int B>
+__global__ void __launch_bounds__(kThrThreads) threshold_cluster_kernel(CompressArgs a, int ut_begin, int redo, int blocks) {
+    __shared__ __align__(16) uint32_t s_hist[kThrBins], s_all[kThrBins];
+    __shared__ uint32_t s_sum[2][32];
+    __shared__ __align__(8) uint32_t s_range[2];
+    constexpr bool F32KEY = !(sizeof(T) == 2 && B == 2);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x % blocks, ut = ut_begin + blockIdx.x / blocks, chunks = a.chunks;
+    const int c_begin = (int)((int64_t)chunks * rank / blocks), c_end = (int)((int64_t)chunks * (rank + 1) / blocks);
+    SelState* const sel = a.sel + ut;
+    chain_wait();
+    if (redo && !sel->redo) return;  // (the same for the whole cluster, as every branch below)
+    const int32_t* const cn = a.cand_n + (int64_t)ut * a.chunks_max;
+    // the threads' sums of two counts over the cluster's first `ranks` blocks
+    auto cluster_total = [&](uint32_t x, uint32_t y, int ranks) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t yg = __shfl_up_sync(0xFFFFFFFFu, ig, o), ye = __shfl_up_sync(0xFFFFFFFFu, ie, o);
-            if (lane >= o) { ig += yg; ie += ye; }
+        for (int o = 16; o; o >>= 1) {
+            x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+            y += __shfl_xor_sync(0xFFFFFFFFu, y, o);
         }
         __syncthreads();
-        if (lane == 31) { s_sum[0][warp] = ig; s_sum[1][warp] = ie; }
+        if (lane == 0) { s_sum[0][warp] = x; s_sum[1][warp] = y; }
         __syncthreads();
-        uint32_t tg = 0, te = 0, bg = run_gt, be = run_eq;
-#pragma unroll
-        for (int w = 0; w < 32; ++w) {
-            if (w < warp) { bg += s_sum[0][w]; be += s_sum[1][w]; }
-            tg += s_sum[0][w];
-            te += s_sum[1][w];
+        if (tid == 0) {
+            x = y = 0;
+            for (int w = 0; w < kThrThreads / 32; ++w) { x += s_sum[0][w]; y += s_sum[1][w]; }
+            s_range[0] = x;
+            s_range[1] = y;
         }
-        if (c < chunks) base[c] = make_int2((int)(bg + ig) - m.x, (int)(be + ie) - m.y);
-        run_gt += tg;
-        run_eq += te;
+        cluster_sync();
+        const uint2 t = cluster_sum2((uint32_t)__cvta_generic_to_shared(s_range), ranks);
+        cluster_sync();  // (before s_range is written again)
+        return t;
+    };
+    auto each = [&](auto&& f) {
+        int n = c_begin + warp < c_end ? cn[c_begin + warp] : 0;
+        for (int c = c_begin + warp; c < c_end; c += kThrThreads / 32) {
+            const int n_next = c + 32 < c_end ? cn[c + 32] : 0;
+            f(c, n);
+            n = n_next;
+        }
+    };
+    // counts of f's bins over the cluster, the one where their running sum from the top reaches `target` and the count above it
+    auto bin_of = [&](auto&& f, uint32_t target, uint32_t& bin, uint32_t& above) {
+        for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
+        __syncthreads();
+        each([&](int c, int n) { each_candidate<T, B>(a, ut, c, n, f); });
+        cluster_sync();
+        for (int i = 2 * tid; i < kThrBins; i += 2 * kThrThreads)
+            *reinterpret_cast<uint2*>(&s_all[i]) = cluster_sum2((uint32_t)__cvta_generic_to_shared(&s_hist[i]), blocks);
+        cluster_sync();  // (before anybody's counts start again)
+        return find_bin<kThrThreads, kThrBins>(s_all, target, bin, above);
+    };
+    uint32_t tau = a.n_keep > 0 ? 0u : kNoKey, need = (uint32_t)a.n_keep;  // (all of them: above 0 or equal to it)
+    if (a.n_keep > 0 && a.n_keep < (int64_t)a.T * a.d) {
+        uint32_t mine = 0;
+        each([&](int, int n) { mine += lane == 0 ? (uint32_t)n : 0u; });
+        const uint2 total = cluster_total(mine, 0, blocks);
+        if ((int64_t)total.x < a.n_keep) {
+            if (tid == 0 && rank == 0) { sel->redo = 1; sel->lo = 0; }
+            return;
+        }
+        uint32_t k_rem = (uint32_t)a.n_keep, prefix, above, bin;
+        for (uint32_t from = sel->lo >> 16;;) {
+            const bool found = bin_of([&](uint32_t key) {
+                const uint32_t k16 = key >> 16;
+                if (k16 >= from) atomicAdd(&s_hist[min(k16 - from, (uint32_t)kThrBins - 1)], 1u);
+            }, k_rem, bin, above);
+            if (!found) {  // (every position is a candidate and the sample misled: from the smallest key on)
+                from = 0;
+                continue;
+            }
+            prefix = from + bin;
+            if (bin < kThrBins - 1 || from + kThrBins - 1 >= 32767) break;
+            from += kThrBins - 1;
+        }
+        k_rem -= above;
+        if constexpr (F32KEY) {
+            const uint32_t top = prefix;
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                const int shift = pass == 0 ? 4 : 0, bits = pass == 0 ? 12 : 4;
+                const uint32_t want = pass == 0 ? top : prefix;
+                bin_of([&](uint32_t key) {
+                    if ((key >> (shift + bits)) == want) atomicAdd(&s_hist[(key >> shift) & ((1u << bits) - 1u)], 1u);
+                }, k_rem, bin, above);
+                prefix = (want << bits) | bin;
+                k_rem -= above;
+            }
+        }
+        tau = F32KEY ? prefix : prefix << 16;
+        need = k_rem;
     }
+    if (tid == 0 && rank == 0) { sel->tau = tau; sel->need = need; }
+    // ---- keys above and equal to the threshold before every chunk ----
+    int2* const base = a.chunk_base + (int64_t)ut * a.chunks_max;
+    uint32_t range_gt = 0, range_eq = 0;
+    each([&](int c, int n) {
+        uint32_t both = 0;  // (see threshold_kernel)
+        each_candidate<T, B>(a, ut, c, n, [&](uint32_t key) { both += key > tau ? 1u : key == tau ? 0x10000u : 0u; });
+#pragma unroll
+        for (int o = 16; o; o >>= 1) both += __shfl_xor_sync(0xFFFFFFFFu, both, o);
+        if (lane == 0) {
+            base[c] = make_int2((int)(both & 0xFFFFu), (int)(both >> 16));
+            range_gt += both & 0xFFFFu;
+            range_eq += both >> 16;
+        }
+    });
+    const uint2 before = cluster_total(range_gt, range_eq, rank);  // of the blocks before this one
+    scan_chunks(base, c_begin, c_end, before.x, before.y, s_sum);
 }
 
 // ---- 4: the lists -------------------------------------------------------------------------------------
@@ -578,7 +735,7 @@ __device__ __forceinline__ uint32_t packed_place(uint32_t p) {
 
 // grid (groups of eight chunks, unit-tensors), a chunk per warp: no block barriers, U rounds of candidates requested together
 // (one chunk per block with a block scan per round took 767 us for 32 layers of 32k tokens)
-template <typename T, int B>
+template <typename T, int B, bool ALL>
 __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_begin) {
     constexpr int NB = B == 4 ? 4 : 1, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
     constexpr int U = 4;
@@ -609,7 +766,7 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
         for (int q = 0; q < U; ++q) {
             const int i = i0 + 32 * q;
             if (i < n) {
-                p[q] = pos[i];
+                p[q] = ALL ? (uint32_t)i : pos[i];
 #pragma unroll
                 for (int l = 0; l < NB; ++l) raw[q][l] = val[(int64_t)l * a.cand_stride + i];
             }
@@ -672,27 +829,9 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 // shared memories (11, 10 and 10 bits of the key; a bf16 pair's has no more than 15), and a thread writes the entries of its 32
 // consecutive positions.  Bound by the chain of its steps (loads, five cluster barriers with reads across the cluster between, block
 // scans), not by bytes: one bf16 pair of 509 x 128 24.5 -> 11.7 us against the four kernels, 1000 x 128 32.8 -> 12.9, eight of
-// 900 x 128 47.9 -> 26.6.  Only while every cluster runs at once: 256 pairs of 1024 x 128, seven turns, 195 us against 133.
+// 900 x 128 47.9 -> 26.6.  While the clusters take two turns at most (two blocks fit an SM up to about 88 KiB of values each): 32 tensors
+// of blocks of four, 1000 x 128, two turns, 66 us against 64; 256 pairs of 1024 x 128, seven turns, 195 against 133.
 constexpr int kSmallThreads = 512, kSmallElems = 32 * kSmallThreads, kSmallSmem = 128 * 1024;
-
-__device__ __forceinline__ void cluster_sync() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// the sum over the cluster of two consecutive 32-bit words at a shared-memory address, all loads in flight together
-__device__ __forceinline__ uint2 cluster_sum2(uint32_t addr, int blocks) {
-    uint2 v[8], sum = make_uint2(0, 0);
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        uint32_t at;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(r < blocks ? r : 0));
-        asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v[r].x), "=r"(v[r].y) : "r"(at));
-    }
-#pragma unroll
-    for (int r = 0; r < 8; ++r)
-        if (r < blocks) { sum.x += v[r].x; sum.y += v[r].y; }
-    return sum;
-}
 
 template <typename T, int B>
 __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a, int blocks, int range) {
@@ -889,9 +1028,10 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     static PerDevice once;
     int sms = 0;
     constexpr int CE = compress_chunk(B, (int)sizeof(T));
-    const size_t smem = 2 * (size_t)B * CE * sizeof(T);
+    const size_t smem = 2 * (size_t)B * CE * sizeof(T) + (B == 4 ? CE * sizeof(uint16_t) : 0);  // (a block of four: room for positions)
     cudaError_t e = once.ensure([&]() {
-        const cudaError_t e1 = cudaFuncSetAttribute(split_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e1 = cudaFuncSetAttribute(split_kernel<T, B, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(split_kernel<T, B, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         return e1 != cudaSuccess ? e1 : cudaFuncSetAttribute(small_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
     }, &sms);
     if (e != cudaSuccess) return e;
@@ -905,7 +1045,9 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     const int64_t range = (tiles + cluster - 1) / cluster * tile_e;
     const size_t small_smem = (size_t)range * (B == 4 ? 4 : 1) * sizeof(T);
     const int uts = a.Hkv * a.tensors;
-    if (range <= kSmallElems && small_smem <= (size_t)kSmallSmem && (int64_t)cluster * uts * (block_end - block_begin) <= 2 * sms) {
+    // (blocks of four with nearly all entries: a thread writes too many of its own; 1000 x 128 293 and 108 us, 300 x 128 68 and 87)
+    const bool few = B == 2 || (double)a.n_keep <= kAllShare * (double)n || n <= 40 * 1024;
+    if (few && range <= kSmallElems && small_smem <= (size_t)kSmallSmem && (int64_t)cluster * uts * (block_end - block_begin) <= 2 * sms) {
         for (int b0 = block_begin; b0 < block_end; b0 += kSplitLayers / B) {
             const int nb = std::min(block_end - b0, kSplitLayers / B);
             for (int l = 0; l < nb * B; ++l) {
@@ -918,14 +1060,20 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
         return cudaSuccess;
     }
     const int ut_begin = block_begin * uts, ut_count = (block_end - block_begin) * uts;
-    // about 1.2 k candidates (and four standard deviations of a small sample on top); a sample of everything is exact
     const int n_rows = (int)std::min<int64_t>(a.T, std::max<int64_t>(1, kSampleElems / a.d));
     const bool exact = n_rows == a.T;
     const double expect = (double)a.n_keep * n_rows / a.T;
+    const bool all = a.in_place || (double)a.n_keep > kAllShare * (double)n;
+    // about 1.2 k candidates (and four standard deviations of a small sample on top); a sample of everything is exact
     const uint32_t target = exact ? (uint32_t)a.n_keep : (uint32_t)std::ceil(1.2 * expect + 4.0 * std::sqrt(expect) + 16.0);
+    // blocks per unit-tensor for the threshold: as many as run at one time, where each has a chunk per warp or the candidates are all.
+    // The joins cost about 5 us a digit: 64 lists of 98k entries 147 -> 136 us, of 65k 263 -> 278, one of 33k float32 entries 57 -> 67.
+    constexpr int kDigits = sizeof(T) == 2 && B == 2 ? 1 : 3;
+    int blocks = all || a.n_keep >= 96 * 1024 * (kDigits + 1) / 2 ? 8 : 1;
+    while (blocks > 1 && ((int64_t)blocks * ut_count > 2 * sms || a.chunks < (all ? 4 : 32) * blocks)) blocks /= 2;
     // (items are counted in 32 bits)
     const int per_launch = (int)std::max<int64_t>(1, std::min<int64_t>(kSplitLayers / B, 0x7FFFFFFF / ((int64_t)a.chunks * uts) / 4));
-    for (int redo = 0; redo < (exact || a.n_keep == 0 ? 1 : 2); ++redo) {
+    for (int redo = 0; redo < (all || exact || a.n_keep == 0 ? 1 : 2); ++redo) {
         for (int b0 = block_begin; b0 < block_end; b0 += per_launch) {
             const int nb = std::min(block_end - b0, per_launch);
             for (int l = 0; l < nb * B; ++l) {
@@ -935,11 +1083,20 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
             a.ut_base = b0 * uts;
             if (!redo && (e = launch_chain(0, sample_kernel<T, B>, dim3(uts, nb), kSampleThreads, 0, st, a, n_rows, target)) != cudaSuccess) return e;
             const int items = a.chunks * uts * nb;
-            if ((e = launch_chain(0, split_kernel<T, B>, dim3(std::min(items, 3 * sms)), kSplitThreads, smem, st, a, items, redo)) != cudaSuccess) return e;
+            if ((e = launch_chain(0, all ? split_kernel<T, B, true> : split_kernel<T, B, false>, dim3(std::min(items, 3 * sms)), kSplitThreads, smem, st, a, items,
+                                  redo)) != cudaSuccess)
+                return e;
         }
-        if ((e = launch_chain(0, threshold_kernel<T, B>, dim3(ut_count), kThrThreads, 0, st, a, ut_begin, redo)) != cudaSuccess) return e;
+        e = all || blocks > 1 ? launch_chain(blocks, threshold_cluster_kernel<T, B>, dim3(ut_count * blocks), kThrThreads, 0, st, a, ut_begin, redo, blocks)
+                              : launch_chain(0, threshold_kernel<T, B>, dim3(ut_count), kThrThreads, 0, st, a, ut_begin, redo);
+        if (e != cudaSuccess) return e;
     }
-    return launch_chain(0, compact_kernel<T, B>, dim3((a.chunks + 7) / 8, ut_count), 256, 0, st, a, ut_begin);
+    constexpr int kMostRows = 65535;  // of a grid
+    for (int u0 = 0; u0 < ut_count; u0 += kMostRows) {
+        const dim3 grid((a.chunks + 7) / 8, std::min(ut_count - u0, kMostRows));
+        if ((e = launch_chain(0, all ? compact_kernel<T, B, true> : compact_kernel<T, B, false>, grid, 256, 0, st, a, ut_begin + u0)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace

@@ -6,6 +6,7 @@ import torch
 
 from gpu_util import check_compression
 from oracle import fdkv_ref as R
+from oracle import fdkv_ref_b4 as R4
 from paper_2607_06519_b200 import synth
 
 pytestmark = pytest.mark.gpu
@@ -91,3 +92,39 @@ def test_a_sample_that_misleads_for_one_head(hkv):
                 assert np.array_equal(idx.cpu().numpy(), want), (p, h, is_v)
                 assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want]), (p, h, is_v)
     assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("bf16", 64), ("f32", 128), ("f32", 64)])
+@pytest.mark.parametrize("T,keep", [(4099, (3, 10)), (4099, (6, 10)), (4099, (61, 100)), (4099, (99, 100)), (4099, (1, 1)), (1030, (3, 4)), (9000, (2, 5))])
+@pytest.mark.parametrize("block", [2, 4])
+def test_lists_of_many_entries(dtype, d, T, keep, block):
+    """Either side of the shares from which every position is listed as a candidate, up to all of them."""
+    from paper_2607_06519_b200 import runner
+
+    if T == 9000 and (dtype, block, d) != ("bf16", 2, 128):
+        pytest.skip("one long case")
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=block, n_kv_heads=2, n_q_heads=2, head_dim=d, T=T, dtype=dtype, n_needles=2, W=1, keep_num=keep[0],
+                                            keep_den=keep[1], block_size=block, name="many")
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    for h in range(2):
+        if block == 2:
+            check_compression(pf.ctx, w, 0, 0, h)
+            continue
+        u = R4.Unit4(synth.block_tensor(w, 0, 0, h, False), synth.block_tensor(w, 0, 0, h, True), dtype == "bf16", *keep)
+        for is_v, name in ((0, "k"), (1, "v")):
+            idx, val = pf.ctx.get_residual(0, 0, h, is_v)
+            got = idx.cpu().numpy()
+            assert np.array_equal(got, u.kept[name])
+            want = np.stack([u.dev[name][l].ravel()[got] for l in range(4)])
+            assert np.array_equal(val.float().cpu().numpy().reshape(4, -1), want)
+    assert pf.ctx.device_status() == 0
+    pf.ctx.close()
+
+
+@pytest.mark.parametrize("keep", [(1, 3), (7, 10)])
+@pytest.mark.parametrize("factor", [100.0, 0.01])
+def test_a_sample_that_misleads_both_bounds(keep, factor):
+    """The k-th key below both bounds of the sample, or above them, where every position is a candidate and where not."""
+    test_a_sample_that_misleads("bf16", 128, factor, keep)
+    test_a_sample_that_misleads("f32", 64, factor, keep)
