@@ -318,7 +318,14 @@ extern "C" fdkv_status fdkv_compress_unit_noalloc(const void* x0, const void* x1
     a.chunk_base = reinterpret_cast<int2*>(sc + kNaBase);
     a.cand_stride = kNoAllocMaxElems; a.chunks_max = (int)kNoAllocChunks;
     a.n_keep = k; a.kcap = 0;
+    // (a layer's rows that z0 overwrites must not be read a second time)
+    const size_t esize = dtype == FDKV_BF16 ? 2 : 4;
+    const uintptr_t z0_at = reinterpret_cast<uintptr_t>(z0_out), z0_end = z0_at + (size_t)T * head_dim * esize;
     a.in_place = false;
+    for (const void* x : {x0, x1}) {
+        const uintptr_t at = reinterpret_cast<uintptr_t>(x), end = at + ((size_t)(T - 1) * stride_t + head_dim) * esize;
+        a.in_place = a.in_place || (z0_at < end && at < z0_end);
+    }
     a.ntiles_max = (int)kNoAllocMaxTiles;
     a.tile_off = reinterpret_cast<int32_t*>(sc + kNaOff);
     a.idx = idx_out; a.val = val_out; a.packed = nullptr;

@@ -128,3 +128,27 @@ def test_a_sample_that_misleads_both_bounds(keep, factor):
     """The k-th key below both bounds of the sample, or above them, where every position is a candidate and where not."""
     test_a_sample_that_misleads("bf16", 128, factor, keep)
     test_a_sample_that_misleads("f32", 64, factor, keep)
+
+
+
+@pytest.mark.parametrize("which", [0, 1])
+@pytest.mark.parametrize("dtype,T,keep", [("bf16", 5003, (1, 64)), ("f32", 5003, (1, 16)), ("bf16", 509, (1, 16)), ("bf16", 8192, (1, 2))])
+def test_shared_coefficients_in_a_layers_place(dtype, T, keep, which):
+    """One tensor pair whose shared coefficients replace a layer's rows, with a sample that misleads: no row is read twice."""
+    from paper_2607_06519_b200 import binding as B
+
+    d = 128
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    rng = np.random.default_rng(7)
+    scale = np.ones((T, 1), np.float32)
+    scale[_sampled_tokens(T, d)] = 100.0
+    base = rng.standard_normal((T, d)).astype(np.float32)
+    x = [torch.from_numpy(a).to(tdt).cuda() for a in (base, base + scale * rng.standard_normal((T, d)).astype(np.float32))]
+    want_z0, z1 = R.depth_split(x[0].float().cpu().numpy(), x[1].float().cpu().numpy(), dtype == "bf16")
+    k = T * d * keep[0] // keep[1]
+    want = R.select_entries(z1, k)
+    idx, val = torch.empty(k, dtype=torch.int32, device="cuda"), torch.empty(k, dtype=tdt, device="cuda")
+    assert B.compress_unit_noalloc(x[0], x[1], *keep, x[which], idx, val) == k
+    assert np.array_equal(x[which].float().cpu().numpy(), want_z0)
+    assert np.array_equal(idx.cpu().numpy(), want)
+    assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want])
