@@ -272,7 +272,10 @@ fdkv_status fdkv_footprint(fdkv_ctx* ctx, int32_t seq, size_t* bytes_by_mode_hos
  * lengths, modes[batch * n_kv_heads] of the layer's units.  Outputs (HOST): start_out[n_ctas + 1], block c handles the
  * range [start_out[c], start_out[c+1]) where an entry is unit << 20 | slice and the last one is units << 20;
  * *n_ctas_out <= n_ctas blocks are used; parts_out[batch * n_kv_heads] = split-K parts per unit (blocks whose range
- * holds at least one of its slices).  Errors: FDKV_ERR_INVALID_ARG for null pointers, sizes out of range or more units
+ * holds at least one of its slices).  Launches on short contexts are cut in another way where the device lets them: every unit
+ * gets the same number of blocks, which join their parts as a cluster in one kernel, each with whole tiles where that
+ * leaves the slowest less (it depends on how many clusters run at one time and on the tails, which this call does not
+ * know).  Errors: FDKV_ERR_INVALID_ARG for null pointers, sizes out of range or more units
  * than the kernel takes (1024).                                                                                      */
 fdkv_status fdkv_plan_decode(int32_t batch, int32_t n_kv_heads, const int32_t* T_host, const int32_t* modes_host,
                              int32_t keep_num, int32_t keep_den, int32_t residual_rule, int32_t row_format, int32_t n_ctas,

@@ -29,6 +29,16 @@ fdkv_status fdkv_test_clear_device_status(fdkv_ctx* ctx, void* stream);
 fdkv_status fdkv_test_probe_moments(fdkv_ctx* ctx, int32_t form);
 
 /*
+ * Host-only: the cut of a bf16 / head_dim 128 decode launch as the library makes it on a device of `n_ctas` SMs where
+ * max_clusters[i] (HOST, 4) clusters of 2^i thread blocks run at one time.  T, tails (HOST, [batch]): prefill lengths and
+ * generated tokens; modes (HOST, [batch * n_kv_heads]).  start_out / n_ctas_out as fdkv_plan_decode; *cluster_out: blocks per
+ * unit, one cluster each, or 0 (that call's cut).
+ */
+fdkv_status fdkv_test_plan_clusters(int32_t batch, int32_t n_kv_heads, int32_t group, const int32_t* T, const int32_t* modes,
+                                    const int32_t* tails, int32_t keep_num, int32_t keep_den, int32_t row_format, int32_t n_ctas,
+                                    const int32_t* max_clusters, uint32_t* start_out, int32_t* n_ctas_out, int32_t* cluster_out);
+
+/*
  * The per-device set-up table of the launchers (function attributes are per device, not per process), driven with a
  * list of device ids instead of the current device: returns how many of the n visits `devs` (HOST) would run the
  * set-up on a fresh table.  Host only; no GPU is touched.

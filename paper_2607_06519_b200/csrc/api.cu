@@ -1120,7 +1120,7 @@ fdkv_status fdkv_plan_decode(int32_t batch, int32_t n_kv_heads, const int32_t* T
     a.keep_num = keep_num; a.keep_den = keep_den;
     a.tok_rule = residual_rule == FDKV_RESIDUAL_TOKENS ? 1 : 0;
     a.rows_f8 = row_format != 0 ? 1 : 0;
-    return plan_decode_host(a, n_ctas, start_out, n_ctas_out, parts_out) == cudaSuccess ? FDKV_OK : FDKV_ERR_INVALID_ARG;
+    return plan_decode_host(a, n_ctas, nullptr, start_out, n_ctas_out, parts_out, nullptr) == cudaSuccess ? FDKV_OK : FDKV_ERR_INVALID_ARG;
 }
 
 fdkv_status fdkv_decode_bytes(fdkv_ctx* c, int32_t layer, int32_t batch, size_t* bytes_host) {

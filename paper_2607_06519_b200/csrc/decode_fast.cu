@@ -902,7 +902,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     // replayed (eight KV heads, clusters of eight), clusters against two kernels: 512 tokens 4.6 and 6.6, 1024 5.0 and 7.0, 2047 6.4
     // and 7.7, 4096 9.9 and 8.9; with a tail 1024 6.0 and 6.8, 2047 7.7 and 7.9, 3000 9.1 and 8.6.  8-bit rows, whose tails make the
     // last block later: 1024 6.5 and 8.8, 4096 10.5 and 10.7, 8192 15.2 and 11.5; with a tail 1024 8.5 and 9.1, 3000 9.1 and 9.9,
-    // 4096 13.0 and 11.5.
+    // 4096 13.0 and 11.5.  One block per unit, 144 units of 1 500 to 3 000 tokens: 43.0 and 36.3.
     if (max_clusters) {
         const double kClusterGain = a.rows_f8 ? 3.0 : 2.1;
         int least = ns[0];
@@ -933,7 +933,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
                     if (best < 0.0 || t < best) { best = t; per[u] = p; }
                 }
                 worst = std::max(worst, best);
-                all += (double)es[u] * wt[u] / (kTT / kResTile) / tile;
+                all += (double)ns[u] * wt[u] / (kTT / kResTile) / tile + tail;  // (not what a block that ends a unit is charged)
             }
             if (worst <= std::max(1.0, all / ctas) + kClusterGain) {
                 int c = 0;
@@ -1032,17 +1032,19 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     return cudaSuccess;
 }
 
-// The plan alone, for a given number of CTAs (fdkv_plan_decode: host only, no device is touched).
-cudaError_t plan_decode_host(const DecodeArgs& a, int n_ctas, uint32_t* start_out, int32_t* ncta_out, int32_t* parts_out) {
+// The plan alone, for a given number of CTAs (fdkv_plan_decode: host only, no device is touched).  max_clusters: as above.
+cudaError_t plan_decode_host(const DecodeArgs& a, int n_ctas, const int* max_clusters, uint32_t* start_out, int32_t* ncta_out, int32_t* parts_out,
+                             int32_t* cluster_out) {
     const int units = a.batch * a.Hkv;
     if (units < 1 || units > kMaxUnits || n_ctas < 1) return cudaErrorInvalidValue;
     FastSched sch;
     PartCount cs;
-    const cudaError_t e = plan_decode_schedule(a, units, n_ctas, nullptr, sch, cs);
+    const cudaError_t e = plan_decode_schedule(a, units, n_ctas, max_clusters, sch, cs);
     if (e != cudaSuccess) return e;
     for (int c = 0; c <= sch.ncta; ++c) start_out[c] = sch.start[c];
     for (int u = 0; u < units; ++u) parts_out[u] = cs.n[u];
     *ncta_out = sch.ncta;
+    if (cluster_out) *cluster_out = sch.cluster;
     return cudaSuccess;
 }
 

@@ -341,7 +341,8 @@ struct TokenGatherJob {
     int32_t twice, pad_;
 };
 cudaError_t launch_token_gather_jobs(const TokenGatherJob* jobs_dev, int njobs, int64_t k_tok, int d, int B, int dtype, cudaStream_t st);
-cudaError_t plan_decode_host(const DecodeArgs& a, int n_ctas, uint32_t* start_out, int32_t* ncta_out, int32_t* parts_out);
+cudaError_t plan_decode_host(const DecodeArgs& a, int n_ctas, const int* max_clusters, uint32_t* start_out, int32_t* ncta_out, int32_t* parts_out,
+                             int32_t* cluster_out);
 cudaError_t launch_copy_jobs(const CopyJob* jobs_dev, int njobs, int64_t bytes_max, cudaStream_t st);
 cudaError_t launch_quantise_jobs(const QuantJob* jobs_dev, int njobs, int T_max, cudaStream_t st);
 cudaError_t launch_repack_jobs(const RepackJob* jobs_dev, int njobs, int64_t n_max, cudaStream_t st);

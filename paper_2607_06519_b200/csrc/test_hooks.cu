@@ -1,4 +1,6 @@
 // Test hooks (include/fdkv_testing.h): reach the library's failure handling without a fault, a trap or a hang.
+#include <cstring>
+
 #include "../../include/fdkv_testing.h"
 #include "fdkv_internal.h"
 #include "mbar_wait.cuh"
@@ -51,6 +53,22 @@ fdkv_status fdkv_test_probe_moments(fdkv_ctx* c, int32_t form) {
     if (!c || form < 0 || form > 2) return FDKV_ERR_INVALID_ARG;
     c->probe_moments = form;
     return FDKV_OK;
+}
+
+fdkv_status fdkv_test_plan_clusters(int32_t batch, int32_t n_kv_heads, int32_t group, const int32_t* T, const int32_t* modes, const int32_t* tails,
+                                    int32_t keep_num, int32_t keep_den, int32_t row_format, int32_t n_ctas, const int32_t* max_clusters,
+                                    uint32_t* start_out, int32_t* n_ctas_out, int32_t* cluster_out) {
+    if (!T || !modes || !tails || !max_clusters || !start_out || !n_ctas_out || !cluster_out || batch < 1 || n_kv_heads < 1 || n_ctas < 1 ||
+        n_ctas > fdkv::kMaxSplits || (int64_t)batch * n_kv_heads > fdkv::kFastMaxUnits || keep_den < 1)
+        return FDKV_ERR_INVALID_ARG;
+    fdkv::DecodeArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.batch = batch; a.Hkv = n_kv_heads; a.G = group; a.d = 128;
+    a.host_T = T; a.host_modes = modes; a.host_tail = tails; a.max_tail = 1 << 20;
+    a.keep_num = keep_num; a.keep_den = keep_den; a.rows_f8 = row_format != 0;
+    std::vector<int32_t> parts((size_t)batch * n_kv_heads);
+    const cudaError_t e = fdkv::plan_decode_host(a, n_ctas, reinterpret_cast<const int*>(max_clusters), start_out, n_ctas_out, parts.data(), cluster_out);
+    return e == cudaSuccess ? FDKV_OK : FDKV_ERR_INVALID_ARG;
 }
 
 int32_t fdkv_test_per_device_visits(const int32_t* devs, int32_t n) {

@@ -129,3 +129,58 @@ def test_argument_checks():
         B.plan_decode([128] * 129, [[0] * 8] * 129, 8, 1, 16, 148)  # more units than the kernel takes (1024)
     with pytest.raises(B.FdkvError):
         B.plan_decode([128], [[0]], 1, 1, 16, 0)          # no blocks
+
+
+def _cluster_cut(T, modes, tails, hkv, group, row_format=0):
+    """(blocks per unit, starts) of the cut that a launch on 148 SMs takes; blocks per unit 0: not in clusters."""
+    import ctypes as C
+
+    from paper_2607_06519_b200 import binding as B
+
+    i32, batch, units = C.c_int32, len(T), len(T) * hkv
+    start, used, cluster = (C.c_uint32 * 161)(), i32(0), i32(0)
+    st = B._lib.fdkv_test_plan_clusters(batch, hkv, group, (i32 * batch)(*T), (i32 * units)(*modes), (i32 * batch)(*tails), 1, 16, row_format, 148,
+                                        (i32 * 4)(148, 74, 34, 16), start, C.byref(used), C.byref(cluster))
+    assert st == 0
+    return cluster.value, [int(v) for v in start[:used.value + 1]]
+
+
+@pytest.mark.parametrize("row_format", [0, 1])
+@pytest.mark.parametrize("seed", range(6))
+def test_cluster_cuts_cover_every_slice_once(row_format, seed):
+    """The cut for short contexts: the same number of blocks for every unit, ranges in order that tile its slices, none empty, and no
+    range much longer than an equal share with the tail counted."""
+    rng = np.random.default_rng(seed)
+    taken = 0
+    for _ in range(200):
+        batch, hkv, group = int(rng.integers(1, 5)), int(rng.choice([1, 2, 3, 8])), int(rng.choice([1, 4, 8]))
+        T = [int(x) for x in np.exp(rng.uniform(0, np.log(6000), batch))]
+        tails = [int(x) for x in rng.choice([0, 0, 1, 40, 129, 500], batch)]
+        modes = [int(m) for m in rng.integers(0, 3, batch * hkv)]
+        units = batch * hkv
+        n, start = _cluster_cut(T, modes, tails, hkv, group, row_format)
+        if n == 0:
+            continue
+        taken += 1
+        assert n in (1, 2, 4, 8) and len(start) == units * n + 1 and units <= {1: 148, 2: 74, 4: 34, 8: 16}[n]
+        assert start[-1] == units << 20
+        for u in range(units):
+            slices, tail = _slices(T[u // hkv]), -(-tails[u // hkv] // 128) * 8
+            at = start[u * n:(u + 1) * n]
+            assert all(a >> 20 == u for a in at) and at[0] & 0xFFFFF == 0
+            sizes = np.diff([a & 0xFFFFF for a in at] + [slices])
+            assert (sizes >= 1).all(), (T, tails, sizes)
+            tile = 16 if row_format else 8
+            share = -(-(slices + tail) // n)
+            assert sizes[:-1].max(initial=0) <= share + tile
+            assert sizes[-1] + tail <= max(share, tail + 1) + n * tile
+    assert taken > 20
+
+
+def test_uneven_units_are_not_one_block_each():
+    """Nine sequences of 1 500 to 3 000 tokens with sixteen KV heads are nearly as many units as there are SMs: one block per unit would
+    wait for the longest residual one."""
+    T = [3000 - b * 3000 // 18 for b in range(9)]
+    modes = [(0, 1, 0, 1, 2, 0, 1, 0)[u % 8] for u in range(9 * 16)]
+    assert _cluster_cut(T, modes, [0] * 9, 16, 2)[0] == 0
+    assert _cluster_cut([1024], modes[:8], [0], 8, 4)[0] == 8
