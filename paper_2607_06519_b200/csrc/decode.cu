@@ -379,8 +379,11 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, cudaStream_t st) {
     if (a.packed_lists) return cudaErrorNotSupported;  // packed residual lists are only read by the kernel above
 
     // one tile per warp while the blocks are resident at one time (two on an SM for bf16 up to two heads per group), then longer ranges
+    static PerDevice once;
+    int sms = 0;
+    if ((e = once.ensure([]() { return cudaSuccess; }, &sms)) != cudaSuccess) return e;
     const int ntiles = (a.Tmax_batch + kResTile - 1) / kResTile, units = a.Hkv * a.batch;
-    const int splits = std::max(1, std::min(std::min(((a.G <= 2 && dtype == FDKV_BF16 ? 2 : 1) * 148 + units - 1) / units, kMaxSplits), (ntiles + kWarps - 1) / kWarps));
+    const int splits = std::max(1, std::min(std::min(((a.G <= 2 && dtype == FDKV_BF16 ? 2 : 1) * sms + units - 1) / units, kMaxSplits), (ntiles + kWarps - 1) / kWarps));
     if (dtype == FDKV_BF16)
         e = a.d == 128 ? launch_generic<__nv_bfloat16, 128>(a, splits, st) : launch_generic<__nv_bfloat16, 64>(a, splits, st);
     else
