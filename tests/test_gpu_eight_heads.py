@@ -15,9 +15,9 @@ pytestmark = pytest.mark.gpu
 BOUND = 3e-5
 
 
-# clusters (the first three), a unit's blocks whole, ranges that straddle units, one block
+# clusters (the first three), a unit's blocks whole, ranges that straddle units, one block; more sequences than the short list of tails holds
 @pytest.mark.parametrize("group", [4, 8])
-@pytest.mark.parametrize("hkv,T,batch,tail", [(8, 1000, 1, 0), (2, 1024, 1, 130), (1, 37, 1, 1), (3, 4099, 1, 2), (8, 4096, 1, 0), (8, 1500, 6, 0), (2, 32768, 1, 0)])
+@pytest.mark.parametrize("hkv,T,batch,tail", [(8, 1000, 1, 0), (2, 1024, 1, 130), (1, 37, 1, 1), (3, 4099, 1, 2), (8, 4096, 1, 0), (8, 1500, 6, 0), (2, 32768, 1, 0), (2, 65, 70, 0)])
 def test_entries(hkv, group, T, batch, tail):
     w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=hkv, n_q_heads=hkv * group, T=T, batch=batch, n_needles=2, W=1, n_steps=max(tail, 1),
                                             name="eight")

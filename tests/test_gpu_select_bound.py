@@ -124,8 +124,8 @@ def test_lists_of_many_entries(dtype, d, T, keep, block):
 
 @pytest.mark.parametrize("keep", [(1, 3), (7, 10)])
 @pytest.mark.parametrize("factor", [100.0, 0.01])
-def test_a_sample_that_misleads_both_bounds(keep, factor):
-    """The k-th key below both bounds of the sample, or above them, where every position is a candidate and where not."""
+def test_a_sample_that_misleads_many(keep, factor):
+    """The same with many entries: a list of candidates, and every position one (whose threshold starts from the sample's bound too)."""
     test_a_sample_that_misleads("bf16", 128, factor, keep)
     test_a_sample_that_misleads("f32", 64, factor, keep)
 
