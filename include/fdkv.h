@@ -20,6 +20,8 @@
  *  - A "unit" is (sequence, layer pair p = layers 2p and 2p+1, KV head h).  Query head i reads KV head
  *    i / (n_q_heads / n_kv_heads).
  *  - A context is not thread-safe.
+ *  - A context holds a block of page-locked host memory (its commit tables and probe scores).  At most four such blocks of at
+ *    most 1 MiB of closed contexts stay with the process, for the next ones.
  *
  * Notation follows the paper's Method section: T context length, d head dimension, Z0 / Z1 the low /
  * high frequency depth coefficients of Eq. 1 with the 2x2 orthonormal DCT-II, c = 1/sqrt(2).

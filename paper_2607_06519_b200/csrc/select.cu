@@ -280,8 +280,8 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, 
 // neighbouring rows.  A warp owns NV * 256 consecutive positions of a chunk, a lane eight of them per step.  The rows of the
 // next item are copied to shared memory (cp.async, 16 bytes per lane and layer, every lane its own) while one is worked on; the
 // high-frequency values take the place of the rows they came from.  A byte per eight positions goes to a bit map; then
-// every lane writes the candidates of its NV * 8 consecutive positions behind those of the lanes and warps before it.  One
-// block barrier per item (the warps' counts).  The issue slots are as busy as HBM here, hence the packed arithmetic, the
+// the positions of every lane's NV * 8 go behind those of the lanes and warps before it, and the lists leave in runs.  One
+// block barrier per item (the warps' counts).  The issue slots are nearly as busy as HBM here (60 % and 69 %), hence the packed arithmetic, the
 // bit tricks and the running item coordinates (with scalar arithmetic, a binary search per list entry and divisions per item:
 // 1 550 us for 32 layers of 32k tokens).
 // ALL: every position is a candidate, the values go to the list in their order and no positions are written (see kAllShare).
