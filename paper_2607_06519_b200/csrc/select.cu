@@ -38,7 +38,7 @@ constexpr int kSampleThreads = 512, kSampleBins = 4096;
 constexpr int64_t kSampleElems = 65536;
 constexpr int kThrThreads = 1024, kThrBins = 4096;
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;  // a bound or threshold above every key
-// Of the positions are kept: from there on every position is taken for a candidate (4 layers of 32k tokens, all kept, 2 940 -> 906 us).
+// Of the positions are kept: from there on every position is taken for a candidate (4 layers of 32k tokens, all kept, 2 940 -> 872 us).
 constexpr double kAllShare = 0.6;
 
 // two float32 operations at a time, each rounded to nearest
@@ -1066,11 +1066,12 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     const bool all = a.in_place || (double)a.n_keep > kAllShare * (double)n;
     // about 1.2 k candidates (and four standard deviations of a small sample on top); a sample of everything is exact
     const uint32_t target = exact ? (uint32_t)a.n_keep : (uint32_t)std::ceil(1.2 * expect + 4.0 * std::sqrt(expect) + 16.0);
-    // blocks per unit-tensor for the threshold: as many as run at one time, where each has a chunk per warp or the candidates are all.
+    // blocks per unit-tensor for the threshold: one per SM, where each has a chunk per warp or the candidates are all.  (Two per SM leave
+    // clusters waiting: 32 tensors of 32k x 128, eight blocks each 316 us, four 277; keep 1/2 724 and 653.)
     // The joins cost about 5 us a digit: 64 lists of 98k entries 147 -> 136 us, of 65k 263 -> 278, one of 33k float32 entries 57 -> 67.
     constexpr int kDigits = sizeof(T) == 2 && B == 2 ? 1 : 3;
     int blocks = all || a.n_keep >= 96 * 1024 * (kDigits + 1) / 2 ? 8 : 1;
-    while (blocks > 1 && ((int64_t)blocks * ut_count > 2 * sms || a.chunks < (all ? 4 : 32) * blocks)) blocks /= 2;
+    while (blocks > 1 && ((int64_t)blocks * ut_count > sms || a.chunks < (all ? 4 : 32) * blocks)) blocks /= 2;
     // (items are counted in 32 bits)
     const int per_launch = (int)std::max<int64_t>(1, std::min<int64_t>(kSplitLayers / B, 0x7FFFFFFF / ((int64_t)a.chunks * uts) / 4));
     for (int redo = 0; redo < (all || exact || a.n_keep == 0 ? 1 : 2); ++redo) {
