@@ -902,7 +902,12 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     // replayed (eight KV heads, clusters of eight), clusters against two kernels: 512 tokens 4.6 and 6.6, 1024 5.0 and 7.0, 2047 6.4
     // and 7.7, 4096 9.9 and 8.9; with a tail 1024 6.0 and 6.8, 2047 7.7 and 7.9, 3000 9.1 and 8.6.  8-bit rows, whose tails make the
     // last block later: 1024 6.5 and 8.8, 4096 10.5 and 10.7, 8192 15.2 and 11.5; with a tail 1024 8.5 and 9.1, 3000 9.1 and 9.9,
-    // 4096 13.0 and 11.5.  One block per unit, 144 units of 1 500 to 3 000 tokens: 43.0 and 36.3.
+    // 4096 13.0 and 11.5.
+    // Up to five tiles per SM, the other cut also pays for rounding its shares to tiles, about what a block that ends a unit is
+    // charged: that counts then (units of bf16, ragged lengths up to the given one, a third to a half residual; clusters and two
+    // kernels: 128 of 459 tokens 11.9 and 14.8, 64 of 1181 9.4 and 10.8, 32 of 3267 10.7 and 11.7).  Longer ones don't (128 of 2174 36.1 and
+    // 31.7, 64 of 2972 26.1 and 20.4, 144 of 3000 43.0 and 36.3), nor 8-bit rows (48 of 537 10.1 and 8.8, 32 of 2270 13.2 and 11.3, though 128 of
+    // 949 20.5 and 22.4).
     if (max_clusters) {
         const double kClusterGain = a.rows_f8 ? 3.0 : 2.1;
         int least = ns[0];
@@ -933,7 +938,8 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
                     if (best < 0.0 || t < best) { best = t; per[u] = p; }
                 }
                 worst = std::max(worst, best);
-                all += (double)ns[u] * wt[u] / (kTT / kResTile) / tile + tail;  // (not what a block that ends a unit is charged)
+                all += (double)ns[u] * wt[u] / (kTT / kResTile) / tile + tail;
+                if (!a.rows_f8 && total_tiles <= 5 * ctas) all += (double)(5 * total_tiles / ctas) / 8.0;
             }
             if (worst <= std::max(1.0, all / ctas) + kClusterGain) {
                 int c = 0;

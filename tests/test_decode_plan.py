@@ -184,3 +184,13 @@ def test_uneven_units_are_not_one_block_each():
     modes = [(0, 1, 0, 1, 2, 0, 1, 0)[u % 8] for u in range(9 * 16)]
     assert _cluster_cut(T, modes, [0] * 9, 16, 2)[0] == 0
     assert _cluster_cut([1024], modes[:8], [0], 8, 4)[0] == 8
+
+
+def test_short_ragged_units_are_clusters():
+    """Many units of a few tiles: clusters, although the slowest block has up to twice the average (the other cut rounds its shares to
+    tiles too); the same batch at five times the length is cut by cost."""
+    for hkv, batch, T0, n in ((16, 8, 459, 1), (8, 8, 718, 2), (4, 8, 1477, 4)):
+        modes = [1 if u % hkv < hkv // 3 else 0 for u in range(hkv * batch)]
+        for scale, expect in ((1, n), (5, 0)):
+            T = [T0 * scale - b * T0 * scale // (2 * batch) - b for b in range(batch)]
+            assert _cluster_cut(T, modes, [0] * batch, hkv, 4)[0] == expect
