@@ -357,7 +357,7 @@ cudaError_t launch_probe_tc(const ProbeArgs& a, int dtype, cudaStream_t st, bool
     pl.pos_max = a.pos_host[a.W - 1];
     pl.ntiles = pl.pos_max / kBN + 1;  // keys after the last probe position never count
     // keys that every probe query sees: second moments (one read of Z1 and 2 x 2 x 128 x 128 flops per key, against a second
-    // copy of Z1 and 2 x 2 x rows x 128 flops here; 32 layers of 32k tokens, 512 rows per pair: 1 190 -> 320 us with this
+    // copy of Z1 and 2 x 2 x rows x 128 flops here; 32 layers of 32k tokens, 512 rows per pair: 1 190 -> 428 us with this
     // kernel's share of the last keys)
     pl.tile_first = (pl.pos_min + 1) / kBN;
     if (a.moments == 0 ? !moments_pay(a, pl.tile_first, sm_count) : a.moments == 2) pl.tile_first = 0;
