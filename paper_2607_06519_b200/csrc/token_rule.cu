@@ -30,25 +30,34 @@ namespace fdkv {
 namespace {
 
 constexpr int kTM = 128;                    // tokens per tile (M of the MMA)
-constexpr int kTN = 256;                    // probe rows per item (N of the MMA)
-constexpr int kTStages = 4;
+constexpr int kTN = 256;                    // probe rows per item (N of the MMA) at most
+constexpr int kTStages = 3;
 constexpr int kTAHalf = kTM * 128;          // one 64-channel half of a token tile: 16 KiB
 constexpr int kTAStage = 2 * kTAHalf;       // 32 KiB
-constexpr int kTBHalf = kTN * 128;          // one 64-channel half of the Q block: 32 KiB
-constexpr int kTBBytes = 2 * kTBHalf;       // 64 KiB
-constexpr int kTHdr = 2048;                 // barriers, TMEM slot, abort flag, probe position of every column
-constexpr int kTSmem = kTHdr + kTBBytes + kTStages * kTAStage;  // 194 KiB
-constexpr int kTThreads = 6 * 32;
-constexpr uint32_t kTIdesc = umma_idesc(kTM, kTN, false);
-constexpr int tFull = 0, tEmpty = 32, tTFull = 64, tTEmpty = 80, tSlot = 96, tAbort = 100, tPosCol = 1024;  // pos_col: 256 ints
+constexpr int kTHdr = 3072;                 // barriers, TMEM slot, abort flag, the epilogue's exchange
+constexpr int kTThreads = 12 * 32;          // copies, MMAs, probe rows, one idle, eight of the epilogue
+constexpr int tFull = 0, tEmpty = 32, tTFull = 64, tTEmpty = 80, tSlot = 96, tAbort = 100, tBFull = 112, tBEmpty = 128, tExch = 1024;
+constexpr int score_smem(int nt) { return kTHdr + 2 * nt * 256 + kTStages * kTAStage; }
+static_assert(score_smem(kTN) <= 227 * 1024, "shared memory budget");
 
-
+// The product of all items' tiles: item = (unit, layer, block of NT probe rows), ntiles tiles each; block b of the grid takes the
+// tiles [total b / blocks, total (b + 1) / blocks) of them.
 struct ScorePlan {
-    int items_per_unit, mblocks, nsplits, ntiles, tiles_per_split, pos_min;
+    int mblocks, ntiles, total, pos_min;
 };
 
+// NT: probe rows per item (64, 128 or 256: the smallest that holds a layer's rows, so that few probe rows do not pay for 256).
+// One persistent block per SM.  Warp 0 streams the token tiles, warp 2 the probe rows of the next item into the other of two
+// buffers, one thread of warp 1 issues the MMAs, eight warps take the results: two per quarter of the TMEM lanes, half of the columns
+// each, joined through shared memory.  Bound by the MMAs (1 024 cycles a tile of 128 x 256 x 128) with the epilogue close behind: four
+// warps took 1.6 us a tile, and a block per item and third of its tiles, each with its own probe rows, left the last of six waves a
+// fifth full (8 191 tokens, 8 blocks of four, 8 heads, 256 rows a layer: 214 -> SCORE_US us).
+template <int NT>
 __global__ void __launch_bounds__(kTThreads, 1)
 token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScorePlan pl) {
+    constexpr uint32_t kIdesc = umma_idesc(kTM, NT, false);
+    constexpr int kBHalf = NT * 128, kBBytes = 2 * kBHalf;  // one 64-channel half of the probe rows, both
+    constexpr uint32_t kCols = 2 * NT;                      // TMEM columns: two accumulators
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sm0 = s_u32(smem);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + tAbort);
@@ -57,144 +66,179 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
         if (threadIdx.x == 0) atomicMax(a.status, (int32_t)kFlagCountMismatch);
         return;
     }
-    int it = blockIdx.x;
-    const int unit = a.unit_begin + it / pl.items_per_unit;
-    it %= pl.items_per_unit;
-    const int split = it % pl.nsplits; it /= pl.nsplits;
-    const int mblock = it % pl.mblocks; it /= pl.mblocks;
-    const int layer = it;
-    const int h = unit % a.Hkv, pair = unit / a.Hkv;
-    const int tile0 = split * pl.tiles_per_split;
-    const int ntile = max(0, min(pl.ntiles, tile0 + pl.tiles_per_split) - tile0);
+    const int g_begin = (int)((int64_t)pl.total * blockIdx.x / gridDim.x), g_end = (int)((int64_t)pl.total * (blockIdx.x + 1) / gridDim.x);
     const int rows_layer = a.G * a.W;
-    int* const pos_col = reinterpret_cast<int*>(smem + tPosCol);
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < kTStages; ++s) { mb_init(sm0 + tFull + 8 * s, 1); mb_init(sm0 + tEmpty + 8 * s, 1); }
-        for (int s = 0; s < 2; ++s) { mb_init(sm0 + tTFull + 8 * s, 1); mb_init(sm0 + tTEmpty + 8 * s, 4); }
+        for (int s = 0; s < 2; ++s) {
+            mb_init(sm0 + tTFull + 8 * s, 1); mb_init(sm0 + tTEmpty + 8 * s, 8);
+            mb_init(sm0 + tBFull + 8 * s, 1); mb_init(sm0 + tBEmpty + 8 * s, 1);
+        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // ---- B: probe rows r = mblock*256 + i of this layer, r = g*W + qi -> Q[layer][qi][h*G+g][:]; padding rows zero ----
-    {
-        const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(a.q_layers_dev[a.B * pair + layer]);
-        for (int v = threadIdx.x; v < kTN * 16; v += kTThreads) {
-            const int i = v >> 4, chunk = v & 15;
-            const int r = mblock * kTN + i;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (r < rows_layer)
-                val = *reinterpret_cast<const uint4*>(q + ((int64_t)(r % a.W) * a.Hq + h * a.G + r / a.W) * 128 + chunk * 8);
-            *reinterpret_cast<uint4*>(smem + kTHdr + (chunk >> 3) * kTBHalf + i * 128 + (((chunk & 7) ^ (i & 7)) << 4)) = val;
-        }
-        for (int i = threadIdx.x; i < kTN; i += kTThreads) {
-            const int r = mblock * kTN + i;
-            pos_col[i] = r < rows_layer ? a.pos[r % a.W] : -1;
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm0 + tSlot), "r"(512u) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm0 + tSlot), "r"(kCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(smem + tSlot);
-    const uint32_t b_base = sm0 + kTHdr, a_base = b_base + kTBBytes;
+    const uint32_t b_base = sm0 + kTHdr, a_base = b_base + 2 * kBBytes;
+    // every role walks the block's items: f(its number here, unit, layer, row block, first tile, tiles, number of the first tile here)
+    auto items = [&](auto&& f) {
+        for (int g = g_begin, seg = 0; g < g_end; ++seg) {
+            const int item = g / pl.ntiles, t0 = g - item * pl.ntiles, n = min(pl.ntiles - t0, g_end - g);
+            const int mblock = item % pl.mblocks, ul = item / pl.mblocks;
+            f(seg, a.unit_begin + ul / a.B, ul % a.B, mblock, t0, n, g - g_begin);
+            g += n;
+        }
+    };
 
     if (warp == 0) {
-        if (lane == 0) {
-            // K high-frequency rows of the unit (a block of four stages one operand per layer)
-            const int64_t row0 = a.B == 4 ? ((int64_t)unit * 4 + layer) * a.Tmax : (int64_t)unit * a.Tmax;
-            for (int i = 0; i < ntile; ++i) {
-                const int s = i % kTStages;
-                mb_wait(sm0 + tEmpty + 8 * s, ((uint32_t)(i / kTStages) & 1u) ^ 1u, abort_flag, a.status);
-                if (*abort_flag) break;
-                const uint32_t full = sm0 + tFull + 8 * s, dst = a_base + s * kTAStage;
-                const int y = (int)(row0 + (int64_t)(tile0 + i) * kTM);
-                mb_expect_tx(full, kTAStage);
-                tma_2d(dst, &tmap, 0, y, full);
-                tma_2d(dst + kTAHalf, &tmap, 64, y, full);
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            const uint64_t db0 = smem_desc(b_base);
-            for (int i = 0; i < ntile; ++i) {
-                const int s = i % kTStages, as = i & 1;
-                mb_wait(sm0 + tTEmpty + 8 * as, (((uint32_t)i >> 1) & 1u) ^ 1u, abort_flag, a.status);
-                mb_wait(sm0 + tFull + 8 * s, (uint32_t)(i / kTStages) & 1u, abort_flag, a.status);
-                if (*abort_flag) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t da0 = smem_desc(a_base + s * kTAStage);
-                const uint32_t d_tmem = tmem_base + (uint32_t)(as * kTN);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const uint64_t da = da0 + (uint64_t)(((k >> 2) * kTAHalf + (k & 3) * 32) >> 4);
-                    const uint64_t db = db0 + (uint64_t)(((k >> 2) * kTBHalf + (k & 3) * 32) >> 4);
-                    umma_ss<kTIdesc>(d_tmem, da, db, k > 0);
+        if (lane == 0)
+            items([&](int, int unit, int layer, int, int t0, int n, int i0) {
+                // K high-frequency rows of the unit (a block of four stages one operand per layer)
+                const int64_t row0 = a.B == 4 ? ((int64_t)unit * 4 + layer) * a.Tmax : (int64_t)unit * a.Tmax;
+                for (int i = i0; i < i0 + n; ++i) {
+                    const int s = i % kTStages;
+                    mb_wait(sm0 + tEmpty + 8 * s, ((uint32_t)(i / kTStages) & 1u) ^ 1u, abort_flag, a.status);
+                    if (*abort_flag) break;
+                    const uint32_t full = sm0 + tFull + 8 * s, dst = a_base + s * kTAStage;
+                    const int y = (int)(row0 + (int64_t)(t0 + i - i0) * kTM);
+                    mb_expect_tx(full, kTAStage);
+                    tma_2d(dst, &tmap, 0, y, full);
+                    tma_2d(dst + kTAHalf, &tmap, 64, y, full);
                 }
-                umma_commit(sm0 + tEmpty + 8 * s);
-                umma_commit(sm0 + tTFull + 8 * as);
+            });
+    } else if (warp == 1) {
+        if (lane == 0)
+            items([&](int seg, int, int, int, int, int n, int i0) {
+                const int bs = seg & 1;
+                const uint64_t db0 = smem_desc(b_base + bs * kBBytes);
+                mb_wait(sm0 + tBFull + 8 * bs, ((uint32_t)seg >> 1) & 1u, abort_flag, a.status);
+                for (int i = i0; i < i0 + n; ++i) {
+                    const int s = i % kTStages, as = i & 1;
+                    mb_wait(sm0 + tTEmpty + 8 * as, (((uint32_t)i >> 1) & 1u) ^ 1u, abort_flag, a.status);
+                    mb_wait(sm0 + tFull + 8 * s, (uint32_t)(i / kTStages) & 1u, abort_flag, a.status);
+                    if (*abort_flag) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint64_t da0 = smem_desc(a_base + s * kTAStage);
+                    const uint32_t d_tmem = tmem_base + (uint32_t)(as * NT);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const uint64_t da = da0 + (uint64_t)(((k >> 2) * kTAHalf + (k & 3) * 32) >> 4);
+                        const uint64_t db = db0 + (uint64_t)(((k >> 2) * kBHalf + (k & 3) * 32) >> 4);
+                        umma_ss<kIdesc>(d_tmem, da, db, k > 0);
+                    }
+                    umma_commit(sm0 + tEmpty + 8 * s);
+                    umma_commit(sm0 + tTFull + 8 * as);
+                }
+                if (!*abort_flag) umma_commit(sm0 + tBEmpty + 8 * bs);
+            });
+    } else if (warp == 2) {
+        // probe rows r = mblock * NT + i of the layer, r = g*W + qi -> Q[layer][qi][h*G+g][:]; padding rows zero
+        items([&](int seg, int unit, int layer, int mblock, int, int, int) {
+            const int bs = seg & 1, h = unit % a.Hkv, pair = unit / a.Hkv;
+            mb_wait(sm0 + tBEmpty + 8 * bs, (((uint32_t)seg >> 1) & 1u) ^ 1u, abort_flag, a.status);
+            const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(a.q_layers_dev[a.B * pair + layer]);
+            const int chunk = lane & 15;
+#pragma unroll 4
+            for (int i = lane >> 4; i < NT; i += 2) {
+                const int r = mblock * NT + i;
+                const uint32_t dst = b_base + bs * kBBytes + (chunk >> 3) * kBHalf + i * 128 + (((chunk & 7) ^ (i & 7)) << 4);
+                if (r < rows_layer) {
+                    const int g = r / a.W;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(q + ((int64_t)(r - g * a.W) * a.Hq + h * a.G + g) * 128 + chunk * 8)
+                                 : "memory");
+                } else {
+                    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(dst), "r"(0u) : "memory");
+                }
             }
-        }
-    } else {
-        // ---- epilogue: thread = token (TMEM lane); maximum of |D| and sum of D^2 over the probe rows that see the token ----
-        const int lq = warp & 3;
-        float* const err = a.err + ((int64_t)unit * a.nslots + layer * pl.mblocks + mblock) * a.Tmax;
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mb_arrive(sm0 + tBFull + 8 * bs);
+        });
+    } else if (warp >= 4) {
+        // ---- epilogue: lane = token (TMEM lane); maximum of |D| and sum of D^2 over the probe rows that see the token ----
+        const int lq = warp & 3, half = (warp - 4) >> 2;
+        constexpr int kHalf = NT / 2, kLd = kHalf < 64 ? kHalf : 64;  // columns of a warp; of a round
+        float2* const exch = reinterpret_cast<float2*>(smem + tExch) + lq * 32 + lane;  // [2][128]
         const float c32 = a.B == 4 ? 1.f : __uint_as_float(0x3F3504F3u);  // a pair's rows are Z1: K - Khat^shared = +-c Z1
-        uint32_t* score = a.score + (int64_t)unit * a.Tmax;
-        for (int i = 0; i < ntile; ++i) {
-            const int as = i & 1;
-            const int t = (tile0 + i) * kTM + lq * 32 + lane;
-            mb_wait(sm0 + tTFull + 8 * as, ((uint32_t)i >> 1) & 1u, abort_flag, a.status);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float m = 0.f, e0 = 0.f, e1 = 0.f;
-            if (!*abort_flag) {
-                const bool all_visible = (tile0 + i) * kTM + kTM - 1 <= pl.pos_min;
+        items([&](int, int unit, int layer, int mblock, int t0, int n, int i0) {
+            float* const err = a.err + ((int64_t)unit * a.nslots + layer * pl.mblocks + mblock) * a.Tmax;
+            uint32_t* const score = a.score + (int64_t)unit * a.Tmax;
+            for (int i = i0; i < i0 + n; ++i) {
+                const int as = i & 1, tile_t0 = (t0 + i - i0) * kTM;
+                const int t = tile_t0 + lq * 32 + lane;
+                mb_wait(sm0 + tTFull + 8 * as, ((uint32_t)i >> 1) & 1u, abort_flag, a.status);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                float m0 = 0.f, m1 = 0.f, e0 = 0.f, e1 = 0.f;
+                if (!*abort_flag) {
+                    const bool all_visible = tile_t0 + kTM - 1 <= pl.pos_min;
 #pragma unroll
-                for (int cp = 0; cp < 4; ++cp) {
-                    uint32_t r0[32], r1[32];
-                    const uint32_t ta = tmem_base + ((uint32_t)(lq * 32) << 16) + (uint32_t)(as * kTN + cp * 64);
-                    tmem_ld32(ta, r0);
-                    tmem_ld32(ta + 32, r1);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (all_visible) {
+                    for (int c0 = 0; c0 < kHalf; c0 += kLd) {
+                        uint32_t r[kLd / 32][32];
+                        const uint32_t ta = tmem_base + ((uint32_t)(lq * 32) << 16) + (uint32_t)(as * NT + half * kHalf + c0);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float u = __uint_as_float(r0[j]), v = __uint_as_float(r1[j]);
-                            m = fmaxf(m, fmaxf(fabsf(u), fabsf(v)));
-                            e0 = fmaf(u, u, e0);
-                            e1 = fmaf(v, v, e1);
+                        for (int p = 0; p < kLd / 32; ++p) tmem_ld32(ta + 32 * p, r[p]);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        if (c0 + kLd == kHalf) {  // read: the next product may take the accumulator
+                            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                            __syncwarp();
+                            if (lane == 0) mb_arrive(sm0 + tTEmpty + 8 * as);
                         }
-                    } else {
+                        if (all_visible) {
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float u = __uint_as_float(r0[j]), v = __uint_as_float(r1[j]);
-                            if (pos_col[cp * 64 + j] >= t) { m = fmaxf(m, fabsf(u)); e0 = fmaf(u, u, e0); }
-                            if (pos_col[cp * 64 + 32 + j] >= t) { m = fmaxf(m, fabsf(v)); e1 = fmaf(v, v, e1); }
+                            for (int p = 0; p < kLd / 32; ++p)
+#pragma unroll
+                                for (int j = 0; j < 32; j += 4) {
+                                    const float u = __uint_as_float(r[p][j]), v = __uint_as_float(r[p][j + 1]);
+                                    const float w = __uint_as_float(r[p][j + 2]), x = __uint_as_float(r[p][j + 3]);
+                                    m0 = fmaxf(m0, fmaxf(fabsf(u), fabsf(v)));
+                                    m1 = fmaxf(m1, fmaxf(fabsf(w), fabsf(x)));
+                                    e0 = fmaf(u, u, e0);
+                                    e1 = fmaf(v, v, e1);
+                                    e0 = fmaf(w, w, e0);
+                                    e1 = fmaf(x, x, e1);
+                                }
+                        } else {
+#pragma unroll
+                            for (int p = 0; p < kLd / 32; ++p)
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) {
+                                    const int row = mblock * NT + half * kHalf + c0 + 32 * p + j;
+                                    const float u = __uint_as_float(r[p][j]);
+                                    if (row < rows_layer && a.pos[row % a.W] >= t) { m0 = fmaxf(m0, fabsf(u)); e0 = fmaf(u, u, e0); }
+                                }
                         }
                     }
                 }
+                // the two halves of the columns (one barrier a tile: the buffer of tile i is written again behind that of tile i + 1)
+                if (half) exch[128 * as] = make_float2(fmaxf(m0, m1), e0 + e1);
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + lq) : "memory");
+                if (!half && t < a.T && !*abort_flag) {
+                    const float2 o = exch[128 * as];
+                    const float m = fmaxf(fmaxf(m0, m1), o.x);
+                    if (m > 0.f) atomicMax(score + t, __float_as_uint(m * c32));
+                    err[t] = (e0 + e1) + o.y;
+                }
             }
-            if (t < a.T && !*abort_flag) {
-                if (m > 0.f) atomicMax(score + t, __float_as_uint(m * c32));
-                err[t] = e0 + e1;
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mb_arrive(sm0 + tTEmpty + 8 * as);
-        }
+        });
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (*abort_flag)
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
 }
 
-// ---- block-wide helpers for the select kernel (1024 threads) ----
+constexpr int kSelThreads = 1024, kSelBins = 4096;
+
+// exclusive sum over the block of a value per thread, and the total; s_warp: 32 words
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* s_warp, uint32_t* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t incl = v;
@@ -206,31 +250,28 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* s_warp
     __syncthreads();  // s_warp may still be read from the previous call
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-        uint32_t w = s_warp[lane];
-        uint32_t wi = w;
+    uint32_t w = s_warp[lane];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-            if (lane >= o) wi += x;
-        }
-        s_warp[lane] = wi - w;
-        if (lane == 31) s_warp[32] = wi;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, w, o);
+        if (lane >= o) w += x;
     }
-    __syncthreads();
-    *total = s_warp[32];
-    return s_warp[warp] + incl - v;
+    *total = __shfl_sync(0xFFFFFFFFu, w, 31);
+    const uint32_t before = __shfl_sync(0xFFFFFFFFu, w, (warp + 31) & 31);
+    return (warp ? before : 0u) + incl - v;
 }
 
 // One CTA per unit: threshold of the k-th largest score (32-bit patterns of non-negative floats order like the
-// floats), then the ascending list of kept tokens (score above the threshold, or equal and among the first `need`
-// such tokens), the number of kept tokens before every 16-token slice, and the unit's two error sums: all tokens'
-// (shared) and the unselected ones' (residual), float64 over the score kernel's per-token sums in a fixed order.
-__global__ void __launch_bounds__(1024) token_select_kernel(TokenArgs a) {
-    __shared__ uint32_t s_hist[256];
-    __shared__ uint32_t s_warp[33];
-    __shared__ uint32_t s_prefix, s_krem;
-    const int unit = a.unit_begin + blockIdx.x;
+// floats; three digits of 12, 12 and 7 bits: the first has 16 bins per octave, on which a warp's atomics seldom collide), then
+// the ascending list of kept tokens (score above the threshold, or equal and among the first `need` such tokens), the number of kept
+// tokens before every 16-token slice, and the unit's two error sums: all tokens' (shared) and the unselected ones' (residual),
+// float64 over the score kernel's per-token sums in a fixed order.  Bound by the chain of its steps: with digits of 8 bits, found by
+// one thread, and a scan of flags and one of ranks for every 1 024 tokens, 8 191 tokens took 46 us, now SELECT_US.
+__global__ void __launch_bounds__(kSelThreads) token_select_kernel(TokenArgs a) {
+    __shared__ __align__(16) uint32_t s_hist[kSelBins];
+    __shared__ uint32_t s_warp[32];
+    __shared__ uint32_t s_digit, s_above;
+    const int unit = a.unit_begin + blockIdx.x, tid = threadIdx.x;
     const uint32_t* key = a.score + (int64_t)unit * a.Tmax;
     const float* err = a.err + (int64_t)unit * a.nslots * a.Tmax;
     int32_t* list = a.list + (int64_t)unit * a.ktok_cap;
@@ -239,56 +280,73 @@ __global__ void __launch_bounds__(1024) token_select_kernel(TokenArgs a) {
     const int nslice = (T + kResTile - 1) / kResTile;
     uint32_t tau = 0xFFFFFFFFu, need = 0;
     if (a.k_tok > 0) {
-        if (threadIdx.x == 0) { s_prefix = 0; s_krem = (uint32_t)a.k_tok; }
-        for (int pass = 0; pass < 4; ++pass) {
-            const int shift = 24 - 8 * pass;
-            if (threadIdx.x < 256) s_hist[threadIdx.x] = 0;
+        uint32_t prefix = 0, left = (uint32_t)a.k_tok;
+#pragma unroll 1
+        for (int pass = 0; pass < 3; ++pass) {
+            const int shift = pass == 0 ? 19 : pass == 1 ? 7 : 0, bits = pass == 2 ? 7 : 12;
+            *reinterpret_cast<uint4*>(&s_hist[4 * tid]) = make_uint4(0u, 0u, 0u, 0u);
             __syncthreads();
-            const uint32_t prefix = s_prefix;
-            for (int t = threadIdx.x; t < T; t += blockDim.x) {
+#pragma unroll 4
+            for (int t = tid; t < T; t += kSelThreads) {
                 const uint32_t k = key[t];
-                if (pass == 0 || (k >> (shift + 8)) == prefix) atomicAdd(&s_hist[(k >> shift) & 0xFFu], 1u);
+                if (pass == 0 || (k >> (shift + bits)) == prefix) atomicAdd(&s_hist[(k >> shift) & ((1u << bits) - 1u)], 1u);
             }
             __syncthreads();
-            if (threadIdx.x == 0) {
-                uint32_t above = 0, krem = s_krem;
-                int b = 255;
-                for (; b > 0; --b) {
-                    if (above + s_hist[b] >= krem) break;
-                    above += s_hist[b];
-                }
-                s_prefix = (prefix << 8) | (uint32_t)b;
-                s_krem = krem - above;
+            // the bin, from the top, in which the running count reaches `left`: four bins per thread, the largest first
+            const uint4 v = *reinterpret_cast<const uint4*>(&s_hist[kSelBins - 4 - 4 * tid]);
+            const uint32_t c[4] = {v.w, v.z, v.y, v.x};
+            uint32_t total, before = block_excl_scan(c[0] + c[1] + c[2] + c[3], s_warp, &total);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (before < left && left <= before + c[i]) { s_digit = (uint32_t)(kSelBins - 1 - 4 * tid - i); s_above = before; }
+                before += c[i];
             }
             __syncthreads();
+            prefix = prefix << bits | s_digit;
+            left -= s_above;
         }
-        tau = s_prefix;
-        need = s_krem;
+        tau = prefix;
+        need = left;
     }
-    // ordered compaction, 1024 tokens per round
-    uint32_t base_keep = 0, base_eq = 0;
+    // ordered compaction: eight consecutive tokens per thread and round, counts of those above in the high half, equal in the low
+    uint32_t base_gt = 0, base_eq = 0;
     double sum_all = 0.0, sum_dropped = 0.0;
     const int seen = min(T, a.pos_last + 1);  // later tokens are seen by no probe query: no error, nothing was written
-    for (int t0 = 0; t0 < T; t0 += 1024) {
-        const int t = t0 + threadIdx.x;
-        const uint32_t k = t < T ? key[t] : 0u;
-        const uint32_t gt = t < T && a.k_tok > 0 && k > tau, eq = t < T && a.k_tok > 0 && k == tau;
-        uint32_t tot_eq, tot_keep;
-        const uint32_t rank_eq = base_eq + block_excl_scan(eq, s_warp, &tot_eq);
-        const uint32_t keep = gt || (eq && rank_eq < need);
-        const uint32_t posk = base_keep + block_excl_scan(keep, s_warp, &tot_keep);
-        if (t < seen) {
-            double e = 0.0;
-            for (int j = 0; j < a.nslots; ++j) e += (double)err[(int64_t)j * a.Tmax + t];
-            sum_all += e;
-            if (!keep) sum_dropped += e;
+    for (int t0 = 0; t0 < T; t0 += 8 * kSelThreads) {
+        const int t8 = t0 + 8 * tid;
+        uint32_t gt = 0, eq = 0;
+        if (a.k_tok > 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t k = t8 + i < T ? key[t8 + i] : 0u;
+                gt |= (uint32_t)(t8 + i < T && k > tau) << i;
+                eq |= (uint32_t)(t8 + i < T && k == tau) << i;
+            }
         }
-        if (t < T) {
-            if (keep) list[posk] = t;
-            if ((t & (kResTile - 1)) == 0) off[t / kResTile] = (int32_t)posk;
+        uint32_t total;
+        const uint32_t before = block_excl_scan((uint32_t)__popc(gt) << 16 | (uint32_t)__popc(eq), s_warp, &total);
+        const uint32_t eq_before = base_eq + (before & 0xFFFFu);
+        uint32_t at = base_gt + (before >> 16) + min(eq_before, need);
+        const int ties = (int)min((uint32_t)__popc(eq), need - min(eq_before, need));  // of the thread's, the first
+        uint32_t kept = gt, rest = eq;
+        for (int i = 0; i < ties; ++i) {
+            kept |= rest & (0u - rest);
+            rest &= rest - 1;
         }
-        base_eq += tot_eq;
-        base_keep += tot_keep;
+        if (t8 < T && (t8 & (kResTile - 1)) == 0) off[t8 / kResTile] = (int32_t)at;
+        for (uint32_t b = kept; b; b &= b - 1) list[at++] = t8 + __ffs((int)b) - 1;
+        double e[8] = {};
+        for (int j = 0; j < a.nslots; ++j)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (t8 + i < seen) e[i] += (double)err[(int64_t)j * a.Tmax + t8 + i];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            sum_all += e[i];
+            if (!(kept >> i & 1u)) sum_dropped += e[i];
+        }
+        base_gt += total >> 16;
+        base_eq += total & 0xFFFFu;
     }
     __shared__ double s_err[2][32];
 #pragma unroll
@@ -296,16 +354,17 @@ __global__ void __launch_bounds__(1024) token_select_kernel(TokenArgs a) {
         sum_all += __shfl_xor_sync(0xFFFFFFFFu, sum_all, o);
         sum_dropped += __shfl_xor_sync(0xFFFFFFFFu, sum_dropped, o);
     }
-    if ((threadIdx.x & 31) == 0) { s_err[0][threadIdx.x >> 5] = sum_all; s_err[1][threadIdx.x >> 5] = sum_dropped; }
+    if ((tid & 31) == 0) { s_err[0][tid >> 5] = sum_all; s_err[1][tid >> 5] = sum_dropped; }
     __syncthreads();
-    if (threadIdx.x < 2) {
+    if (tid < 2) {
         double e = 0.0;
-        for (int w = 0; w < 32; ++w) e += s_err[threadIdx.x][w];
-        a.part[(int64_t)unit * a.nptiles_max * 2 + threadIdx.x] = e;
+        for (int w = 0; w < 32; ++w) e += s_err[tid][w];
+        a.part[(int64_t)unit * a.nptiles_max * 2 + tid] = e;
     }
-    if (threadIdx.x == 0) {
-        off[nslice] = (int32_t)base_keep;
-        if ((int64_t)base_keep != a.k_tok) atomicMax(a.status, (int32_t)kFlagCountMismatch);
+    if (tid == 0) {
+        const uint32_t kept = base_gt + min(base_eq, need);
+        off[nslice] = (int32_t)kept;
+        if ((int64_t)kept != a.k_tok) atomicMax(a.status, (int32_t)kFlagCountMismatch);
     }
 }
 
@@ -391,7 +450,9 @@ cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tenso
     int sm_count = 0;
     const size_t tile_smem = (size_t)(kSTile * (d + 1) + kSRows * d) * sizeof(float);
     cudaError_t e0 = once.ensure([&]() {
-        cudaError_t e1 = cudaFuncSetAttribute(token_score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTSmem);
+        cudaError_t e1 = cudaFuncSetAttribute(token_score_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, score_smem(64));
+        if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(token_score_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, score_smem(128));
+        if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(token_score_kernel<kTN>, cudaFuncAttributeMaxDynamicSharedMemorySize, score_smem(kTN));
         if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(token_score_tile_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
         if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(token_score_tile_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
         return e1;
@@ -407,7 +468,7 @@ cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tenso
         else
             token_score_tile_kernel<float><<<dim3(ntiles, a.unit_count), 256, tile_smem, st>>>(a, d);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        token_select_kernel<<<a.unit_count, 1024, 0, st>>>(a);
+        token_select_kernel<<<a.unit_count, kSelThreads, 0, st>>>(a);
         count_launch(2);
         count_kernel(FDKV_KERNEL_PROBE_PORTABLE);
         return cudaGetLastError();
@@ -415,15 +476,18 @@ cudaError_t launch_token_select(const TokenArgs& a, int dtype, int d, bool tenso
     ScorePlan pl;
     pl.pos_min = a.pos_host[0];
     pl.ntiles = a.pos_host[a.W - 1] / kTM + 1;  // tokens after the last probe position are seen by nobody: score 0
-    pl.mblocks = (a.G * a.W + kTN - 1) / kTN;  // (a.nslots = B x mblocks)
-    const int base_items = a.unit_count * a.B * pl.mblocks;
-    int nsplits = std::max(1, std::min((4 * sm_count + base_items - 1) / base_items, (pl.ntiles + 7) / 8));
-    pl.tiles_per_split = (pl.ntiles + nsplits - 1) / nsplits;
-    pl.nsplits = (pl.ntiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
-    pl.items_per_unit = a.B * pl.mblocks * pl.nsplits;
-    token_score_kernel<<<a.unit_count * pl.items_per_unit, kTThreads, kTSmem, st>>>(*reinterpret_cast<const CUtensorMap*>(a.tmap_z1_128), a, pl);
+    pl.mblocks = (a.G * a.W + kTN - 1) / kTN;   // (a.nslots = B x mblocks)
+    const int64_t total = (int64_t)a.unit_count * a.B * pl.mblocks * pl.ntiles;
+    if (total > 0x7FFFFFFF) return cudaErrorInvalidValue;  // cannot happen: units x tokens are in memory
+    pl.total = (int)total;
+    auto score = [&](auto* kernel, int smem) {  // (blocks of fewer than four tiles would wait for their probe rows most of the time)
+        kernel<<<(int)std::min<int64_t>(sm_count, (total + 3) / 4), kTThreads, smem, st>>>(*reinterpret_cast<const CUtensorMap*>(a.tmap_z1_128), a, pl);
+    };
+    if (a.G * a.W <= 64) score(token_score_kernel<64>, score_smem(64));
+    else if (a.G * a.W <= 128) score(token_score_kernel<128>, score_smem(128));
+    else score(token_score_kernel<kTN>, score_smem(kTN));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    token_select_kernel<<<a.unit_count, 1024, 0, st>>>(a);
+    token_select_kernel<<<a.unit_count, kSelThreads, 0, st>>>(a);
     count_launch(2);
     count_kernel(FDKV_KERNEL_TOKEN_SCORE);
     count_kernel(FDKV_KERNEL_PROBE_TC);  // (it is the probe's product too)

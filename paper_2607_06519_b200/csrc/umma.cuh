@@ -46,7 +46,7 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lead
 }
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) { return smem_desc_sw128(addr, 1, 1024); }  // K-major
 // instruction descriptor: D = f32, A = B = bf16; mn_major: both operands MN-major instead of K-major
-constexpr uint32_t umma_idesc(int m, int n, bool mn_major) {
+__host__ __device__ constexpr uint32_t umma_idesc(int m, int n, bool mn_major) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (mn_major ? (1u << 15) | (1u << 16) : 0u) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 // D[tmem] (+)= A[smem] * B[smem]^T; acc = 0 overwrites D
