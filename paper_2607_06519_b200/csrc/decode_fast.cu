@@ -713,19 +713,23 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
 }
 
-// out = sum_s e^{m_s - M} acc_s / sum_s e^{m_s - M} l_s over a query head's split-K parts.  One warp per 32 VEC channels of a
+// out = sum_s e^{m_s - M} acc_s / sum_s e^{m_s - M} l_s over a query head's split-K parts.  One warp per 32 or 128 channels of a
 // head; it rides on programmatic dependent launch between two decode launches.  A block has 32 threads and few registers
 // so that it becomes resident beside a decode block (which leaves 2 048 registers and 1 KiB of shared memory of an SM) and
 // its start costs nothing.  Latency-bound: the maxima, sums and accumulators of 32 parts are requested in one round.
 // (Before, the last block of a unit combined behind an atomic ticket: a release, an atomic round trip and two rounds of
 // loads on the critical path of every layer call, and the SM it ran on started the next call late.)
+// VEC 4: a lane has four channels of every part, four parts in flight (many heads, few parts each).  VEC 2: a lane has two channels of
+// every other part, so that 20 parts are in flight at once (few heads, whose 18 or 19 parts took two rounds of 16 one after the other:
+// eight KV heads, us a call: 2 047 tokens 8.36 -> 8.26, 32k 26.2 -> 26.1, 32k of 8-bit rows 21.3 -> 21.2).
 template <int VEC>
 __global__ void __maxnreg__(48) decode_combine_kernel(const float* partials, int Hq, int Hkv, int G, PartCount pc, void* out, int out_dtype) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int lane = threadIdx.x, i = blockIdx.y, b = blockIdx.z, ch = (blockIdx.x * 32 + lane) * VEC;
+    constexpr int WAYS = VEC == 2 ? 2 : 1, BATCH = VEC == 2 ? 10 : 4;  // lanes that share a channel; parts a lane has in flight
+    const int lane = threadIdx.x, i = blockIdx.y, b = blockIdx.z;
+    const int way = WAYS == 2 ? lane >> 4 : 0, ch = (blockIdx.x * (32 / WAYS) + (lane & (32 / WAYS - 1))) * VEC;
     const int n = pc.n[b * Hkv + i / G];
     const float* const pp = partials + ((int64_t)b * Hq + i) * kMaxSplits * kPartStride;
-    constexpr int BATCH = VEC == 1 ? 16 : 4;  // accumulator loads in flight
     float M = -INFINITY, L = 0.f, A[VEC];
 #pragma unroll
     for (int k = 0; k < VEC; ++k) A[k] = 0.f;
@@ -733,23 +737,26 @@ __global__ void __maxnreg__(48) decode_combine_kernel(const float* partials, int
     for (int base = 0; base < n; base += 32) {
         float m = -INFINITY, l = 0.f;
         if (base + lane < n) {
-            m = __ldcg(pp + (base + lane) * kPartStride);
-            l = __ldcg(pp + (base + lane) * kPartStride + 1);
+            const float2 ml = __ldcg(reinterpret_cast<const float2*>(pp + (base + lane) * kPartStride));
+            m = ml.x;
+            l = ml.y;
         }
         float w = 0.f;
-        for (int j0 = 0; j0 < 32 && base + j0 < n; j0 += BATCH) {
+        for (int j0 = 0; j0 < 32 && base + j0 < n; j0 += BATCH * WAYS) {
             float v[BATCH][VEC];
 #pragma unroll
             for (int j = 0; j < BATCH; ++j) {
+                const int part = j0 + j * WAYS + way;
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) v[j][k] = 0.f;
-                if (base + j0 + j < n) {
-                    const float* p = pp + (base + j0 + j) * kPartStride + 4 + ch;
+                if (part < 32 && base + part < n) {
+                    const float* p = pp + (base + part) * kPartStride + 4 + ch;
                     if constexpr (VEC == 4) {
                         const float4 x = __ldcg(reinterpret_cast<const float4*>(p));
                         v[j][0] = x.x; v[j][1] = x.y; v[j][2] = x.z; v[j][3] = x.w;
                     } else {
-                        v[j][0] = __ldcg(p);
+                        const float2 x = __ldcg(reinterpret_cast<const float2*>(p));
+                        v[j][0] = x.x; v[j][1] = x.y;
                     }
                 }
             }
@@ -770,11 +777,17 @@ __global__ void __maxnreg__(48) decode_combine_kernel(const float* partials, int
             }
 #pragma unroll
             for (int j = 0; j < BATCH; ++j) {
-                const float wj = __shfl_sync(0xFFFFFFFFu, w, (j0 + j) & 31);  // (zero beyond the last part)
+                const int part = j0 + j * WAYS + way;
+                const float wj = __shfl_sync(0xFFFFFFFFu, w, part & 31);  // (a part that is not there has zeros)
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) A[k] = fmaf(v[j][k], wj, A[k]);
             }
         }
+    }
+    if constexpr (WAYS == 2) {
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) A[k] += __shfl_xor_sync(0xFFFFFFFFu, A[k], 16);
+        if (way) return;
     }
     const int64_t o = ((int64_t)b * Hq + i) * 128 + ch;
 #pragma unroll
@@ -1079,7 +1092,7 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
         opt_in(decode_fast_kernel<false, true, kFewSeqs, false>, smem_of(false, true));
         opt_in(decode_fast_kernel<true, true, kFewSeqs, true>, smem_of(true, true));
         // the same division of the SM's memory as the decode kernel's, or the two could not share an SM
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<2>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_combine_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         for (int lg = 0; lg < 4 && e == cudaSuccess; ++lg) {
             cudaLaunchConfig_t q = {};
@@ -1147,7 +1160,7 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     count_kernel(FDKV_KERNEL_DECODE_FAST);
     *handled = true;
     if (sch.cluster) return cudaSuccess;
-    // one channel per lane where a head has many parts (few heads: latency), four where the heads fill the machine
+    // two ways per channel where a head has many parts (few heads: latency), one where the heads fill the machine
     const bool wide = units * a.G > sm_count;
     cfg.gridDim = dim3(wide ? 1 : 4, a.Hq, a.batch);
     cfg.blockDim = dim3(32);
@@ -1155,7 +1168,7 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     cfg.numAttrs = 1;
     const float* parts = a.partials;
     e = wide ? cudaLaunchKernelEx(&cfg, decode_combine_kernel<4>, parts, a.Hq, a.Hkv, a.G, cs, a.out, a.out_dtype)
-             : cudaLaunchKernelEx(&cfg, decode_combine_kernel<1>, parts, a.Hq, a.Hkv, a.G, cs, a.out, a.out_dtype);
+             : cudaLaunchKernelEx(&cfg, decode_combine_kernel<2>, parts, a.Hq, a.Hkv, a.G, cs, a.out, a.out_dtype);
     if (e != cudaSuccess) return e;
     count_launch(1);
     return cudaGetLastError();

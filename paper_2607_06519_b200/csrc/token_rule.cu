@@ -51,7 +51,7 @@ struct ScorePlan {
 // buffers, one thread of warp 1 issues the MMAs, eight warps take the results: two per quarter of the TMEM lanes, half of the columns
 // each, joined through shared memory.  Bound by the MMAs (1 024 cycles a tile of 128 x 256 x 128) with the epilogue close behind: four
 // warps took 1.6 us a tile, and a block per item and third of its tiles, each with its own probe rows, left the last of six waves a
-// fifth full (8 191 tokens, 8 blocks of four, 8 heads, 256 rows a layer: 214 -> SCORE_US us).
+// fifth full (8 191 tokens, 8 blocks of four, 8 heads, 256 rows a layer: 214 -> 165 us).
 template <int NT>
 __global__ void __launch_bounds__(kTThreads, 1)
 token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScorePlan pl) {
@@ -266,7 +266,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* s_warp
 // the ascending list of kept tokens (score above the threshold, or equal and among the first `need` such tokens), the number of kept
 // tokens before every 16-token slice, and the unit's two error sums: all tokens' (shared) and the unselected ones' (residual),
 // float64 over the score kernel's per-token sums in a fixed order.  Bound by the chain of its steps: with digits of 8 bits, found by
-// one thread, and a scan of flags and one of ranks for every 1 024 tokens, 8 191 tokens took 46 us, now SELECT_US.
+// one thread, and a scan of flags and one of ranks for every 1 024 tokens, 8 191 tokens took 46 us, now 15.
 __global__ void __launch_bounds__(kSelThreads) token_select_kernel(TokenArgs a) {
     __shared__ __align__(16) uint32_t s_hist[kSelBins];
     __shared__ uint32_t s_warp[32];

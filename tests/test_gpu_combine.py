@@ -28,3 +28,20 @@ def test_parts_join(hkv, group, T, batch):
                 err = vector_errors(out[b], oracle_layer_out(units, modes[0], w, layer, f32(q)[b]))
                 assert err.max() <= TOL["bf16"], (layer, od, b, float(err.max()))
     assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("hkv,T", [(8, 5003), (7, 6007), (5, 4801)])
+def test_parts_beside_the_rounds(hkv, T):
+    """About 18, 21 and 29 parts per head: below, beside and above the 20 that are joined in one round."""
+    from paper_2607_06519_b200 import runner
+
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=hkv, n_q_heads=hkv, T=T, n_needles=4, W=8, name="combine_rounds")
+    pf = runner.Prefilled(w)
+    modes = np.array([[h % 3 for h in range(hkv)]])
+    pf.prefill(0, modes)
+    q = pf.decode_q(1, 0)
+    out = f32(pf.ctx.decode_attn(1, q))
+    for h in (0, hkv - 1):
+        ref = oracle_unit(w, 0, 0, h).attend(int(modes[0, h]), 1, f32(q)[0][h:h + 1])
+        assert vector_errors(out[0][h:h + 1], ref).max() <= TOL["bf16"], h
+    assert pf.ctx.device_status() == 0
