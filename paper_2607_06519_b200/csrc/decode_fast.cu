@@ -25,6 +25,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "fdkv_internal.h"
 #include "mbar_wait.cuh"
@@ -66,6 +67,17 @@ struct TailLens {
     int32_t n[NB];  // generated tokens in this layer's tail per sequence, this call's append included (host mirror)
 };
 static_assert(kMaxSplits < 256 && kMaxSplits % 32 == 0, "part counts are bytes; the combine holds one part per lane and round");
+
+// The descriptors of a launch of few units travel in its parameters (clusters only): the copies of a block then start with the block,
+// and its list ranges one round trip earlier.  A block that becomes resident only when one of the call before ends, as the last
+// cluster of eight does while seven fit beside those that run, was the one everybody waited for.  (With the other savings of a call of
+// one or two tiles, 1 024 tokens and a tail: 8.4 -> 7.7 us.)
+constexpr int kHeadUnits = 8;
+struct UnitHeads {
+    UnitDesc u[kHeadUnits];
+    int n;  // 0: read them from memory
+};
+struct NoHeads {};
 
 // header offsets
 constexpr int kOffFull = 0, kOffJoint = 64, kOffAbort = 128, kOffM = 256, kOffL = 512, kOffSeg = 1024, kOffSegInfo = 1920,
@@ -184,7 +196,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 template <bool F8, bool CL, int NB, bool SPLIT>
 __global__ void __maxnreg__(232)
 decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap8, DecodeArgs a, FastSched sch,
-                   TailLens<NB> tl) {
+                   TailLens<NB> tl, const __grid_constant__ std::conditional_t<CL, UnitHeads, NoHeads> heads) {
     constexpr int kStages = CL || F8 ? 2 : 3, kScratchBytes = F8 ? 2 * kScratchTile : kScratchTile;
     constexpr int TT = F8 ? kTT8 : kTT;   // tokens of a packed tile
     constexpr int SW = TT / 16 / kCW;     // 16-token slices of it per warp
@@ -275,6 +287,8 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         for (int u = u_first; u <= u_last && u < sch.units; ++u) {
             const int b = u / a.Hkv, h = u % a.Hkv;
             const UnitDesc* ud = a.desc + ((int64_t)b * a.L + a.layer) * a.Hkv + h;
+            if constexpr (CL)
+                if (heads.n) ud = heads.u + u;
             const int nsl = (ud->T + kResTile - 1) / kResTile;
             const int sb = u == u_first ? t_first : 0;
             const int se = u == u_last ? t_last : nsl;
@@ -335,7 +349,10 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         int it = 0;
         for (int u = u_first; u <= u_last && u < sch.units; ++u) {
             const int b = u / a.Hkv, h = u % a.Hkv;
-            const UnitDesc ud = a.desc[((int64_t)b * a.L + a.layer) * a.Hkv + h];
+            const UnitDesc* udp = a.desc + ((int64_t)b * a.L + a.layer) * a.Hkv + h;
+            if constexpr (CL)
+                if (heads.n) udp = heads.u + u;
+            const UnitDesc ud = *udp;
             const int T = ud.T;
             const int nres = (T + kResTile - 1) / kResTile;
             const int sb = u == u_first ? t_first : 0;
@@ -496,6 +513,9 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             }
 
             if (!waited) dependency_wait();
+            uint4 appended = make_uint4(0u, 0u, 0u, 0u);  // (clusters: requested with q, or the block with the tail is another round trip behind)
+            if constexpr (CL)
+                if (append) appended = reinterpret_cast<const uint4*>(lane < 16 ? a.k_new : a.v_new)[((int64_t)b * a.Hkv + h) * 16 + (lane & 15)];
             // q fragments: B operand columns = the G query heads of this KV head.  With G <= 4 columns 4-7 repeat
             // them: in the second product those columns carry the bf16 rounding remainder of P, so P acts in ~16 bits.
             // (More heads fill the columns: their remainder is a second B operand with the same V fragments.)
@@ -538,6 +558,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             const int unit_kr = (int)((reinterpret_cast<uint64_t>(ud.k_rows) - arena) >> (F8 ? 7 : 8));
             const int unit_vr = (int)((reinterpret_cast<uint64_t>(ud.v_rows) - arena) >> (F8 ? 7 : 8));
             auto release_here = [&](int s, int j) {
+                if (CL && it + j + kStages >= seg_info[1]) return;  // (nothing follows in this stage)
                 __syncwarp();
                 if (lane == 0) {
                     // (atomicInc wraps the counter back to zero at the eighth arrival; tile j + kStages reuses stage s)
@@ -1137,24 +1158,30 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     cfg.numAttrs = sch.cluster ? 2 : 1;
     const CUtensorMap& m16 = *reinterpret_cast<const CUtensorMap*>(a.tmap);
     const CUtensorMap& m8 = *reinterpret_cast<const CUtensorMap*>(a.rows_f8 ? a.tmap_u8 : a.tmap);
-    auto launch = [&](auto* kernel, auto tl) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;  // (a captured call reads the descriptors that are there when it is replayed)
+    if (sch.cluster && (e0 = cudaStreamIsCapturing(st, &capture)) != cudaSuccess) return e0;
+    auto launch = [&](auto* kernel, auto tl, auto heads) {
         for (int b = 0; b < a.batch; ++b) tl.n[b] = a.host_tail[b];
-        return cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, tl);
+        if constexpr (std::is_same_v<decltype(heads), UnitHeads>) {
+            heads.n = units <= kHeadUnits && capture == cudaStreamCaptureStatusNone ? units : 0;
+            for (int u = 0; u < heads.n; ++u) heads.u[u] = a.host_desc[((int64_t)(u / a.Hkv) * a.L + a.layer) * a.Hkv + u % a.Hkv];
+        }
+        return cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, tl, heads);
     };
     cudaError_t e;
     const bool split = a.G <= 4;  // (8-bit rows take no more)
     if (sch.cluster)
         e = launch(a.rows_f8 ? decode_fast_kernel<true, true, kFewSeqs, true>
                    : split   ? decode_fast_kernel<false, true, kFewSeqs, true>
-                             : decode_fast_kernel<false, true, kFewSeqs, false>, TailLens<kFewSeqs>());
+                             : decode_fast_kernel<false, true, kFewSeqs, false>, TailLens<kFewSeqs>(), UnitHeads());
     else if (a.batch <= kFewSeqs)
         e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kFewSeqs, true>
                    : split   ? decode_fast_kernel<false, false, kFewSeqs, true>
-                             : decode_fast_kernel<false, false, kFewSeqs, false>, TailLens<kFewSeqs>());
+                             : decode_fast_kernel<false, false, kFewSeqs, false>, TailLens<kFewSeqs>(), NoHeads());
     else
         e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kMaxUnits, true>
                    : split   ? decode_fast_kernel<false, false, kMaxUnits, true>
-                             : decode_fast_kernel<false, false, kMaxUnits, false>, TailLens<kMaxUnits>());
+                             : decode_fast_kernel<false, false, kMaxUnits, false>, TailLens<kMaxUnits>(), NoHeads());
     if (e != cudaSuccess) return e;
     count_launch(1);
     count_kernel(FDKV_KERNEL_DECODE_FAST);
