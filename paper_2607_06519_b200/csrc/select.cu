@@ -826,10 +826,12 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 // ---- all of it for a short unit-tensor ------------------------------------------------------------------
 // One cluster per unit-tensor, a range of whole 16-token tiles per block, at most kSmallElems positions: the high-frequency
 // values stay in shared memory, the threshold is a radix select over histograms that every block adds up from the cluster's
-// shared memories (11, 10 and 10 bits of the key; a bf16 pair's has no more than 15), and a thread writes the entries of its 32
-// consecutive positions.  Bound by the chain of its steps (loads, five cluster barriers with reads across the cluster between, block
-// scans), not by bytes: one bf16 pair of 509 x 128 24.5 -> 11.7 us against the four kernels, 1000 x 128 32.8 -> 12.9, eight of
-// 900 x 128 47.9 -> 26.6.  While the clusters take two turns at most (two blocks fit an SM up to about 88 KiB of values each): 32 tensors
+// shared memories (11, 10 and 10 bits of the key; a bf16 pair's has no more than 15: one histogram of 32 octaves, which also says how
+// many of the kept positions the blocks before have), and a thread writes the entries of its 32
+// consecutive positions.  Bound by the chain of its steps (loads, cluster barriers with reads across the cluster between, block
+// scans), not by bytes: one bf16 pair of 509 x 128 12.0 us with three exchanges, 9.4 with one (24.5 by the four kernels); 1000 x 128
+// 32.8 -> 12.9 and eight of 900 x 128 47.9 -> 26.6 against the four kernels, with three exchanges.
+// While the clusters take two turns at most (two blocks fit an SM up to about 88 KiB of values each): 32 tensors
 // of blocks of four, 1000 x 128, two turns, 66 us against 64; 256 pairs of 1024 x 128, seven turns, 195 against 133.
 constexpr int kSmallThreads = 512, kSmallElems = 32 * kSmallThreads, kSmallSmem = 128 * 1024;
 
@@ -839,8 +841,9 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
     constexpr bool TWO = sizeof(T) == 2 && B == 2;  // (the key's lower 16 bits are zero)
     constexpr int CH = 4 * Q;                       // 16-byte chunks of 32 positions
     extern __shared__ __align__(16) uint8_t smem[];  // [NB][range] values, the chunks of a word of 32 positions swizzled
-    __shared__ __align__(16) uint32_t s_h1[2048], s_h2[TWO ? 1024 : 2048], s_all[2048];
-    __shared__ uint32_t s_count, s_warp[kSmallThreads / 32];
+    // histograms: of the key's first digit (bf16 pairs: of the whole key in a window, two counts of 16 bits a word), the digits after it
+    __shared__ __align__(16) uint32_t s_h1[2048], s_h2[TWO ? 4 : 2048], s_all[TWO ? 4096 : 2048];
+    __shared__ uint32_t s_count, s_warp[kSmallThreads / 32], s_before[2][kSmallThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x % blocks, item = blockIdx.x / blocks, uts = a.Hkv * a.tensors;
     const int ut = a.ut_base + item, blk = item / uts, u = item % uts, h = u / a.tensors, is_v = u % a.tensors;
@@ -849,8 +852,16 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
     const int plane = range * (int)sizeof(T);
     for (int i = tid; i < 2048; i += kSmallThreads) {
         s_h1[i] = 0;
-        if (i < (TWO ? 1024 : 2048)) s_h2[i] = 0;
+        if (!TWO) s_h2[i] = 0;
     }
+    // (bf16 pairs) a key's bin: 4 095 keys from `from` up, 32 octaves, the last bin for what is larger.  At first 2^-24 to 2^8.
+    uint32_t from = (127u - 24u) << 7;
+    auto count_key = [&](uint32_t key) {
+        const uint32_t k16 = key >> 16;
+        if (k16 < from) return;
+        const uint32_t bin = min(k16 - from, 4095u);
+        atomicAdd(&s_h1[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has at most 2^14 positions)
+    };
     auto chunk_at = [&](int word, int j) { return (word * CH + (j ^ (Q == 1 ? (word >> 1) & 3 : word & 7))) * 16; };
     chain_wait();
     __syncthreads();
@@ -887,7 +898,10 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
                     *reinterpret_cast<uint4*>(smem + l * plane + chunk_at(p >> 5, ((p >> 3) & 3) * Q + k)) = hf[l][k];
                 }
             }
-            Eight<T, B>::keys(hf, [&](int, uint32_t key) { atomicAdd(&s_h1[key >> 20], 1u); });
+            Eight<T, B>::keys(hf, [&](int, uint32_t key) {
+                if constexpr (TWO) count_key(key);
+                else atomicAdd(&s_h1[key >> 20], 1u);
+            });
         }
     }
     // f(i, key) for the thread's 32 positions, which are all there or none of them
@@ -906,8 +920,55 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
     };
     // ---- the n_keep-th largest key of the cluster ----
     uint32_t tau = kNoKey, need = 0;
+    uint32_t gt_before = 0, eq_before = 0;  // (bf16 pairs) this thread's part of the counts of the blocks before this one
     cluster_sync();
-    if (a.n_keep > 0) {  // (the same for every block)
+    if (TWO && a.n_keep > 0) {
+        // The blocks' histograms give the threshold and, of the blocks before this one, how many keys are above it and equal to it: one
+        // exchange instead of three (a digit of 11 bits, one of 4, the counts).
+        uint32_t bin, above, of_before[8];
+        for (;;) {
+            const uint32_t at = (uint32_t)__cvta_generic_to_shared(s_h1) + 16 * tid;  // four words, eight bins
+            uint32_t all[8] = {};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) of_before[i] = 0;
+            uint4 v[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                uint32_t remote;
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(at), "r"(r < blocks ? r : 0));
+                asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[r].x), "=r"(v[r].y), "=r"(v[r].z), "=r"(v[r].w) : "r"(remote));
+            }
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                if (r >= blocks) continue;
+                const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t n_i = i & 1 ? w[i >> 1] >> 16 : w[i >> 1] & 0xFFFFu;
+                    all[i] += n_i;
+                    if (r < rank) of_before[i] += n_i;
+                }
+            }
+            *reinterpret_cast<uint4*>(&s_all[8 * tid]) = make_uint4(all[0], all[1], all[2], all[3]);
+            *reinterpret_cast<uint4*>(&s_all[8 * tid + 4]) = make_uint4(all[4], all[5], all[6], all[7]);
+            __syncthreads();
+            const bool found = find_bin<kSmallThreads, 4096>(s_all, (uint32_t)a.n_keep, bin, above);
+            if (found && (bin < 4095 || from + 4095 >= 32767)) break;
+            from = found ? from + 4095 : 0;  // another window (the same for the whole cluster): above, or from the smallest key on
+            cluster_sync();
+            for (int i = tid; i < 2048; i += kSmallThreads) s_h1[i] = 0;
+            __syncthreads();
+            each([&](int, uint32_t key) { count_key(key); });
+            cluster_sync();
+        }
+        tau = (from + bin) << 16;
+        need = (uint32_t)a.n_keep - above;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (8 * tid + i > (int)bin) gt_before += of_before[i];
+            if (8 * tid + i == (int)bin) eq_before += of_before[i];
+        }
+    } else if (a.n_keep > 0) {  // (the same for every block)
         uint32_t bin, above, left = (uint32_t)a.n_keep;
         {
             const uint32_t at = (uint32_t)__cvta_generic_to_shared(s_h1) + 8 * tid;
@@ -928,8 +989,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
             tau = tau << 10 | bin;
         };
         level(s_h2, 10);
-        if constexpr (TWO) tau <<= 10;
-        else level(s_h2 + 1024, 0);
+        level(s_h2 + (TWO ? 0 : 1024), 0);
         need = left;  // of the positions whose key is tau, the lowest
     }
     // ---- entries: those above in the blocks, warps and threads before, then those equal (counts in halves: at most 2^14) ----
@@ -946,6 +1006,11 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
         if (lane >= o) incl += y;
     }
     if (lane == 31) s_warp[warp] = incl;
+    if constexpr (TWO) {
+        gt_before = __reduce_add_sync(0xFFFFFFFFu, gt_before);
+        eq_before = __reduce_add_sync(0xFFFFFFFFu, eq_before);
+        if (lane == 0) { s_before[0][warp] = gt_before; s_before[1][warp] = eq_before; }
+    }
     __syncthreads();
     uint32_t before = incl - cnt, total = 0;
 #pragma unroll
@@ -953,10 +1018,13 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
         if (w < warp) before += s_warp[w];
         total += s_warp[w];
     }
-    if (tid == 0) s_count = total;
-    cluster_sync();
     uint32_t run_gt = before >> 16, run_eq = before & 0xFFFFu;
-    {
+    if constexpr (TWO) {
+#pragma unroll
+        for (int w = 0; w < kSmallThreads / 32; ++w) { run_gt += s_before[0][w]; run_eq += s_before[1][w]; }
+    } else {
+        if (tid == 0) s_count = total;
+        cluster_sync();
         uint32_t at, v;
         asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_count)), "r"(lane < rank ? lane : rank));
         asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");

@@ -63,3 +63,24 @@ def test_blocks_of_four(T):
             want = np.stack([u.dev[name][l].ravel()[u.kept[name]] for l in range(4)])
             assert np.array_equal(val.float().cpu().numpy(), want)
     assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("T", [30, 509, 1000])
+@pytest.mark.parametrize("scale", [0.0, 2.0**-40, 2.0**-24, 2.0**9, 2.0**60, 2.0**120])
+@pytest.mark.parametrize("den", [2, 16])
+def test_any_scale(scale, den, T):
+    """The k-th key below the first window of octaves, at its edges, above it, and with positions on both sides of it."""
+    d = 128
+    rng = np.random.default_rng(5)
+    x = rng.standard_normal((2, T, d)).astype(np.float32)
+    x[:, ::3] *= scale
+    if scale > 1:
+        x[:, 1::3] *= 2.0**-80
+    x0, x1 = (torch.from_numpy(a).cuda().bfloat16() for a in x)
+    k = T * d // den
+    z0, idx, val = torch.empty_like(x0), torch.empty(k, dtype=torch.int32, device="cuda"), torch.empty(k, dtype=torch.bfloat16, device="cuda")
+    assert B.compress_unit_noalloc(x0, x1, 1, den, z0, idx, val) == k
+    _, z1 = R.depth_split(x0.float().cpu().numpy(), x1.float().cpu().numpy(), True)
+    want = R.select_entries(z1, k)
+    assert np.array_equal(idx.cpu().numpy(), want)
+    assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want])
