@@ -492,7 +492,7 @@ __device__ __forceinline__ void scan_chunks(int2* base, int c_begin, int c_end, 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int c0 = c_begin; c0 < c_end; c0 += kThrThreads) {
         const int c = c0 + tid;
-        const int2 m = c < c_end ? base[c] : make_int2(0, 0);
+        const int2 m = c < c_end ? __ldcg(base + c) : make_int2(0, 0);  // (counted by atomics, which pass by the L1)
         uint32_t ig = (uint32_t)m.x, ie = (uint32_t)m.y;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -518,10 +518,17 @@ __device__ __forceinline__ void scan_chunks(int2* base, int c_begin, int c_end, 
 // One block per unit-tensor (grid ut_count).  First digit: the key's top 15 bits, in a window of 4 095 bins from the bound up
 // (32 octaves; the last bin counts what is larger, and in the unheard-of case that the k-th key is there the window moves
 // up): with 128 bins per octave the atomics hardly collide, and 16 KiB leave room for two blocks on an SM.  32-bit keys:
-// two more digits of 12 and 4 bits among the few keys that share the first.
+// two more digits of 12 and 4 bits among the few keys that share the first, which the second pass gathers while it counts the larger
+// ones of every chunk (a pass per digit and one for the counts: 12 289 tokens, 128 tensors of blocks of four: 112 -> 76 us).
+// bf16 magnitudes: the k-th is within half an octave of the bound, so a chunk's counts of the 63 keys from the bound up, kept in shared memory,
+// give both the threshold and the counts before every chunk in one pass (a second one for the counts: 512 tensors of 32k tokens, behind the split: 149 -> 88 us).
+// Where these don't hold the digits are counted one after the other.
+constexpr int kThrMini = 512;  // chunks whose counts fit beside another block's
 template <typename T, int B>
 __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, int ut_begin, int redo) {
-    __shared__ uint32_t s_hist[kThrBins], s_sum[2][32];
+    __shared__ __align__(16) uint32_t s_hist[kThrBins];
+    __shared__ uint32_t s_sum[2][32], s_found[2], s_near;
+    extern __shared__ __align__(16) uint32_t s_dyn[];  // bf16 pairs: [chunks][32] two counts a word; else [kThrBins] keys that share the first digit
     constexpr bool F32KEY = !(sizeof(T) == 2 && B == 2);  // a bf16 magnitude is 15 bits
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ut = ut_begin + blockIdx.x, chunks = a.chunks;
@@ -553,6 +560,69 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
             if (tid == 0) { sel->redo = 1; sel->lo = 0; }
             return;
         }
+        if constexpr (!F32KEY)
+            if (chunks <= kThrMini) {
+                uint32_t* const mini = s_hist + 64 * warp;
+                uint32_t* const total_of = s_hist + 64 * 32;
+                const uint32_t lo16 = sel->lo >> 16;
+                *reinterpret_cast<uint2*>(mini + 2 * lane) = make_uint2(0u, 0u);
+                if (tid < 64) total_of[tid] = 0;
+                __syncthreads();
+                uint2 sum = make_uint2(0u, 0u);
+                int n = warp < chunks ? cn[warp] : 0;
+                for (int c = warp; c < chunks; c += 32) {
+                    const int n_next = c + 32 < chunks ? cn[c + 32] : 0;
+                    each_candidate<T, B>(a, ut, c, n, [&](uint32_t key) {
+                        const uint32_t k = (key >> 16) - lo16;
+                        if (k < 63u) atomicAdd(&mini[k], 1u);
+                    });
+                    __syncwarp();
+                    uint2 v = *reinterpret_cast<const uint2*>(mini + 2 * lane);
+                    const uint32_t inside = __reduce_add_sync(0xFFFFFFFFu, v.x + v.y);
+                    if (lane == 31) v.y = (uint32_t)n - inside;  // the larger ones
+                    s_dyn[32 * c + lane] = v.x | v.y << 16;      // (a chunk has at most 2^13 positions)
+                    sum.x += v.x;
+                    sum.y += v.y;
+                    *reinterpret_cast<uint2*>(mini + 2 * lane) = make_uint2(0u, 0u);
+                    __syncwarp();
+                    n = n_next;
+                }
+                atomicAdd(&total_of[2 * lane], sum.x);
+                atomicAdd(&total_of[2 * lane + 1], sum.y);
+                __syncthreads();
+                if (warp == 0) {  // a lane's two bins, the largest first
+                    const uint32_t c0 = total_of[63 - 2 * lane], c1 = total_of[62 - 2 * lane], k = (uint32_t)a.n_keep;
+                    uint32_t before = c0 + c1;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, before, o);
+                        if (lane >= o) before += y;
+                    }
+                    before -= c0 + c1;
+                    if (before < k && k <= before + c0) { s_found[0] = 63 - 2 * lane; s_found[1] = before; }
+                    if (before + c0 < k && k <= before + c0 + c1) { s_found[0] = 62 - 2 * lane; s_found[1] = before + c0; }
+                }
+                __syncthreads();
+                const int bin = (int)s_found[0];
+                if (bin < 63) {
+                    if (tid == 0) { sel->tau = (lo16 + bin) << 16; sel->need = (uint32_t)a.n_keep - s_found[1]; }
+                    int2* const base = a.chunk_base + (int64_t)ut * a.chunks_max;
+                    for (int c = tid; c < chunks; c += kThrThreads) {
+                        uint32_t gt = 0, eq = 0;
+                        for (int i = 0; i < 32; ++i) {
+                            const int j = (i + c) & 31;  // (the threads of a warp in different banks)
+                            const uint32_t w = s_dyn[32 * c + j], x = w & 0xFFFFu, y = w >> 16;
+                            gt += (2 * j > bin ? x : 0u) + (2 * j + 1 > bin ? y : 0u);
+                            eq += (2 * j == bin ? x : 0u) + (2 * j + 1 == bin ? y : 0u);
+                        }
+                        base[c] = make_int2((int)gt, (int)eq);
+                    }
+                    __syncthreads();
+                    scan_chunks(base, 0, chunks, 0, 0, s_sum);
+                    return;
+                }
+                __syncthreads();
+            }
         uint32_t k_rem = (uint32_t)a.n_keep, prefix, above;
         for (uint32_t from = sel->lo >> 16;; from += kThrBins - 1) {
             for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
@@ -570,6 +640,57 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
         k_rem -= above;
         if constexpr (F32KEY) {
             const uint32_t top = prefix;
+            if (chunks <= 0x10000) {
+                // ---- larger keys of every chunk, and those that share the first digit: chunk and low half ----
+                int2* const base = a.chunk_base + (int64_t)ut * a.chunks_max;
+                if (tid == 0) s_near = 0;
+                __syncthreads();
+                int n = warp < chunks ? cn[warp] : 0;
+                for (int c = warp; c < chunks; c += 32) {
+                    const int n_next = c + 32 < chunks ? cn[c + 32] : 0;
+                    uint32_t gt = 0;
+                    each_candidate<T, B>(a, ut, c, n, [&](uint32_t key) {
+                        gt += key >> 16 > top ? 1u : 0u;
+                        if (key >> 16 == top) {
+                            const uint32_t i = atomicAdd(&s_near, 1u);
+                            if (i < (uint32_t)kThrBins) s_dyn[i] = (uint32_t)c << 16 | (key & 0xFFFFu);
+                        }
+                    });
+                    gt = __reduce_add_sync(0xFFFFFFFFu, gt);
+                    if (lane == 0) base[c] = make_int2((int)gt, 0);
+                    n = n_next;
+                }
+                __syncthreads();
+                const uint32_t near = s_near;
+                if (near <= (uint32_t)kThrBins) {
+                    uint32_t low = 0;
+#pragma unroll 1
+                    for (int pass = 0; pass < 2; ++pass) {
+                        const int shift = pass == 0 ? 4 : 0, bits = pass == 0 ? 12 : 4;
+                        for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
+                        __syncthreads();
+                        for (uint32_t i = tid; i < near; i += kThrThreads) {
+                            const uint32_t key = s_dyn[i] & 0xFFFFu;
+                            if (pass == 0 || key >> 4 == low) atomicAdd(&s_hist[(key >> shift) & ((1u << bits) - 1u)], 1u);
+                        }
+                        __syncthreads();
+                        uint32_t bin;
+                        find_bin<kThrThreads, kThrBins>(s_hist, k_rem, bin, above);
+                        low = low << bits | bin;
+                        k_rem -= above;
+                    }
+                    if (tid == 0) { sel->tau = top << 16 | low; sel->need = k_rem; }
+                    for (uint32_t i = tid; i < near; i += kThrThreads) {
+                        const uint32_t c = s_dyn[i] >> 16, key = s_dyn[i] & 0xFFFFu;
+                        if (key > low) atomicAdd(&base[c].x, 1);
+                        else if (key == low) atomicAdd(&base[c].y, 1);
+                    }
+                    __syncthreads();
+                    scan_chunks(base, 0, chunks, 0, 0, s_sum);
+                    return;
+                }
+                __syncthreads();
+            }
 #pragma unroll 1
             for (int pass = 0; pass < 2; ++pass) {
                 const int shift = pass == 0 ? 4 : 0, bits = pass == 0 ? 12 : 4;
@@ -1099,6 +1220,7 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     const size_t smem = 2 * (size_t)B * CE * sizeof(T) + (B == 4 ? CE * sizeof(uint16_t) : 0);  // (a block of four: room for positions)
     cudaError_t e = once.ensure([&]() {
         cudaError_t e1 = cudaFuncSetAttribute(split_kernel<T, B, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(threshold_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kThrMini * 128);
         if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(split_kernel<T, B, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         return e1 != cudaSuccess ? e1 : cudaFuncSetAttribute(small_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
     }, &sms);
@@ -1140,6 +1262,7 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     constexpr int kDigits = sizeof(T) == 2 && B == 2 ? 1 : 3;
     int blocks = all || a.n_keep >= 96 * 1024 * (kDigits + 1) / 2 ? 8 : 1;
     while (blocks > 1 && ((int64_t)blocks * ut_count > sms || a.chunks < (all ? 4 : 32) * blocks)) blocks /= 2;
+    const size_t thr_smem = kDigits == 1 ? (a.chunks <= kThrMini ? (size_t)a.chunks * 128 : 0) : (size_t)kThrBins * 4;
     // (items are counted in 32 bits)
     const int per_launch = (int)std::max<int64_t>(1, std::min<int64_t>(kSplitLayers / B, 0x7FFFFFFF / ((int64_t)a.chunks * uts) / 4));
     for (int redo = 0; redo < (all || exact || a.n_keep == 0 ? 1 : 2); ++redo) {
@@ -1157,7 +1280,7 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
                 return e;
         }
         e = all || blocks > 1 ? launch_chain(blocks, threshold_cluster_kernel<T, B>, dim3(ut_count * blocks), kThrThreads, 0, st, a, ut_begin, redo, blocks)
-                              : launch_chain(0, threshold_kernel<T, B>, dim3(ut_count), kThrThreads, 0, st, a, ut_begin, redo);
+                              : launch_chain(0, threshold_kernel<T, B>, dim3(ut_count), kThrThreads, thr_smem, st, a, ut_begin, redo);
         if (e != cudaSuccess) return e;
     }
     constexpr int kMostRows = 65535;  // of a grid
