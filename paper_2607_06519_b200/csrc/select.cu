@@ -25,6 +25,7 @@
 // values and reads them back to select (what this replaces) moved 5 instead of 3.6 times a tensor's bytes, and its
 // histogram of every key took 128 KiB of shared memory, one block per SM.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "fdkv_internal.h"
@@ -472,18 +473,24 @@ __device__ __forceinline__ void cluster_sync() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// the sum over the cluster of two consecutive 32-bit words at a shared-memory address, all loads in flight together
+// the sum over the cluster of two consecutive 32-bit words at a shared-memory address, eight loads in flight together
+template <int MOST = 8>  // blocks of a cluster at most
 __device__ __forceinline__ uint2 cluster_sum2(uint32_t addr, int blocks) {
-    uint2 v[8], sum = make_uint2(0, 0);
+    uint2 sum = make_uint2(0, 0);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        uint32_t at;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(r < blocks ? r : 0));
-        asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v[r].x), "=r"(v[r].y) : "r"(at));
+    for (int r0 = 0; r0 < MOST; r0 += 8) {
+        if (r0 > 0 && r0 >= blocks) break;
+        uint2 v[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            uint32_t at;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(r0 + r < blocks ? r0 + r : 0));
+            asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v[r].x), "=r"(v[r].y) : "r"(at));
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            if (r0 + r < blocks) { sum.x += v[r].x; sum.y += v[r].y; }
     }
-#pragma unroll
-    for (int r = 0; r < 8; ++r)
-        if (r < blocks) { sum.x += v[r].x; sum.y += v[r].y; }
     return sum;
 }
 
@@ -954,13 +961,15 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 // 32.8 -> 12.9 and eight of 900 x 128 47.9 -> 26.6 against the four kernels, with three exchanges.
 // While the clusters take two turns at most (two blocks fit an SM up to about 88 KiB of values each): 32 tensors
 // of blocks of four, 1000 x 128, two turns, 66 us against 64; 256 pairs of 1024 x 128, seven turns, 195 against 133.
+// W: words of 32 positions per thread.
 constexpr int kSmallThreads = 512, kSmallElems = 32 * kSmallThreads, kSmallSmem = 128 * 1024;
 
-template <typename T, int B>
-__global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a, int blocks, int range) {
+template <typename T, int B, int W>
+__global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(CompressArgs a, int blocks, int range) {
     constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
     constexpr bool TWO = sizeof(T) == 2 && B == 2;  // (the key's lower 16 bits are zero)
     constexpr int CH = 4 * Q;                       // 16-byte chunks of 32 positions
+    constexpr int MOST = W == 1 ? 8 : 16;           // blocks of a cluster
     extern __shared__ __align__(16) uint8_t smem[];  // [NB][range] values, the chunks of a word of 32 positions swizzled
     // histograms: of the key's first digit (bf16 pairs: of the whole key in a window, two counts of 16 bits a word), the digits after it
     __shared__ __align__(16) uint32_t s_h1[2048], s_h2[TWO ? 4 : 2048], s_all[TWO ? 4096 : 2048];
@@ -1025,18 +1034,21 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
             });
         }
     }
-    // f(i, key) for the thread's 32 positions, which are all there or none of them
-    const bool mine = 32 * tid < n;
+    // f(w, i, key) for position i of the thread's word w, whose 32 positions are all there or none of them
+    const int word0 = W * tid;
     auto each = [&](auto&& f) {
-        if (!mine) return;
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            uint4 hf[NB][Q];
+        for (int w = 0; w < W; ++w) {
+            if (32 * (word0 + w) >= n) return;
 #pragma unroll
-            for (int l = 0; l < NB; ++l)
+            for (int g = 0; g < 4; ++g) {
+                uint4 hf[NB][Q];
 #pragma unroll
-                for (int k = 0; k < Q; ++k) hf[l][k] = *reinterpret_cast<const uint4*>(smem + l * plane + chunk_at(tid, g * Q + k));
-            Eight<T, B>::keys(hf, [&](int i, uint32_t key) { f(8 * g + i, key); });
+                for (int l = 0; l < NB; ++l)
+#pragma unroll
+                    for (int k = 0; k < Q; ++k) hf[l][k] = *reinterpret_cast<const uint4*>(smem + l * plane + chunk_at(word0 + w, g * Q + k));
+                Eight<T, B>::keys(hf, [&](int i, uint32_t key) { f(w, 8 * g + i, key); });
+            }
         }
     };
     // ---- the n_keep-th largest key of the cluster ----
@@ -1052,22 +1064,26 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
             uint32_t all[8] = {};
 #pragma unroll
             for (int i = 0; i < 8; ++i) of_before[i] = 0;
-            uint4 v[8];
 #pragma unroll
-            for (int r = 0; r < 8; ++r) {
-                uint32_t remote;
-                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(at), "r"(r < blocks ? r : 0));
-                asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[r].x), "=r"(v[r].y), "=r"(v[r].z), "=r"(v[r].w) : "r"(remote));
-            }
+            for (int r0 = 0; r0 < MOST; r0 += 8) {
+                if (r0 > 0 && r0 >= blocks) break;
+                uint4 v[8];
 #pragma unroll
-            for (int r = 0; r < 8; ++r) {
-                if (r >= blocks) continue;
-                const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+                for (int r = 0; r < 8; ++r) {
+                    uint32_t remote;
+                    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(at), "r"(r0 + r < blocks ? r0 + r : 0));
+                    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[r].x), "=r"(v[r].y), "=r"(v[r].z), "=r"(v[r].w) : "r"(remote));
+                }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const uint32_t n_i = i & 1 ? w[i >> 1] >> 16 : w[i >> 1] & 0xFFFFu;
-                    all[i] += n_i;
-                    if (r < rank) of_before[i] += n_i;
+                for (int r = 0; r < 8; ++r) {
+                    if (r0 + r >= blocks) continue;
+                    const uint32_t x[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const uint32_t n_i = i & 1 ? x[i >> 1] >> 16 : x[i >> 1] & 0xFFFFu;
+                        all[i] += n_i;
+                        if (r0 + r < rank) of_before[i] += n_i;
+                    }
                 }
             }
             *reinterpret_cast<uint4*>(&s_all[8 * tid]) = make_uint4(all[0], all[1], all[2], all[3]);
@@ -1079,7 +1095,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
             cluster_sync();
             for (int i = tid; i < 2048; i += kSmallThreads) s_h1[i] = 0;
             __syncthreads();
-            each([&](int, uint32_t key) { count_key(key); });
+            each([&](int, int, uint32_t key) { count_key(key); });
             cluster_sync();
         }
         tau = (from + bin) << 16;
@@ -1094,16 +1110,16 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
         {
             const uint32_t at = (uint32_t)__cvta_generic_to_shared(s_h1) + 8 * tid;
 #pragma unroll
-            for (int i = 0; i < 2; ++i) *reinterpret_cast<uint2*>(&s_all[1024 * i + 2 * tid]) = cluster_sum2(at + 4096 * i, blocks);
+            for (int i = 0; i < 2; ++i) *reinterpret_cast<uint2*>(&s_all[1024 * i + 2 * tid]) = cluster_sum2<MOST>(at + 4096 * i, blocks);
         }
         __syncthreads();
         find_bin<kSmallThreads, 2048>(s_all, left, bin, above);
         left -= above;
         tau = bin;
         auto level = [&](uint32_t* hist, int shift) {
-            each([&](int, uint32_t key) { if (key >> (shift + 10) == tau) atomicAdd(&hist[key >> shift & 1023u], 1u); });
+            each([&](int, int, uint32_t key) { if (key >> (shift + 10) == tau) atomicAdd(&hist[key >> shift & 1023u], 1u); });
             cluster_sync();
-            *reinterpret_cast<uint2*>(&s_all[2 * tid]) = cluster_sum2((uint32_t)__cvta_generic_to_shared(hist) + 8 * tid, blocks);
+            *reinterpret_cast<uint2*>(&s_all[2 * tid]) = cluster_sum2<MOST>((uint32_t)__cvta_generic_to_shared(hist) + 8 * tid, blocks);
             __syncthreads();
             find_bin<kSmallThreads, 1024>(s_all, left, bin, above);
             left -= above;
@@ -1114,12 +1130,13 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
         need = left;  // of the positions whose key is tau, the lowest
     }
     // ---- entries: those above in the blocks, warps and threads before, then those equal (counts in halves: at most 2^14) ----
-    uint32_t gt = 0, eq = 0;
-    each([&](int i, uint32_t key) {
-        gt |= (uint32_t)(key > tau) << i;
-        eq |= (uint32_t)(key == tau) << i;
+    uint32_t gt[W] = {}, eq[W] = {}, cnt = 0;
+    each([&](int w, int i, uint32_t key) {
+        gt[w] |= (uint32_t)(key > tau) << i;
+        eq[w] |= (uint32_t)(key == tau) << i;
     });
-    const uint32_t cnt = (uint32_t)__popc(gt) << 16 | (uint32_t)__popc(eq);
+#pragma unroll
+    for (int w = 0; w < W; ++w) cnt += (uint32_t)__popc(gt[w]) << 16 | (uint32_t)__popc(eq[w]);
     uint32_t incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1159,23 +1176,28 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
     uint32_t* const packed = sizeof(T) == 2 && a.packed ? a.packed + (int64_t)ut * NB * a.kcap : nullptr;
     const int tile_words = kResTile * a.d / 32;
     int32_t* const off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1);
-    if (mine) {
-        if (tid % tile_words == 0) off[(e0 / 32 + tid) / tile_words] = (int32_t)(run_gt + min(run_eq, need));
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const int word = word0 + w;
+        if (32 * word >= n) break;
+        uint32_t at = run_gt + min(run_eq, need);
+        if (word % tile_words == 0) off[(e0 / 32 + word) / tile_words] = (int32_t)at;
         // the ties that are kept: while fewer than `need` precede them
-        const int ties = (int)min((uint32_t)__popc(eq), need - min(run_eq, need));
-        uint32_t kept = gt, rest = eq;
+        const int ties = (int)min((uint32_t)__popc(eq[w]), need - min(run_eq, need));
+        uint32_t kept = gt[w], rest = eq[w];
         for (int i = 0; i < ties; ++i) {
             kept |= rest & (0u - rest);
             rest &= rest - 1;
         }
-        uint32_t at = run_gt + min(run_eq, need);
-        if (a.keep && !is_v) a.keep[(int64_t)(ut / a.tensors) * a.keep_stride + e0 / 32 + tid] = kept;
+        run_gt += (uint32_t)__popc(gt[w]);
+        run_eq += (uint32_t)__popc(eq[w]);
+        if (a.keep && !is_v) a.keep[(int64_t)(ut / a.tensors) * a.keep_stride + e0 / 32 + word] = kept;
         for (uint32_t bits = kept; bits; bits &= bits - 1, ++at) {
-            const int i = __ffs((int)bits) - 1, p = 32 * tid + i;
+            const int i = __ffs((int)bits) - 1, p = 32 * word + i;
             idx[at] = e0 + p;
             const uint32_t place = sizeof(T) == 2 ? packed_place((uint32_t)p) : 0u;
             constexpr int PER = 16 / (int)sizeof(T);
-            const int from = chunk_at(tid, i / PER) + (i % PER) * (int)sizeof(T);
+            const int from = chunk_at(word, i / PER) + (i % PER) * (int)sizeof(T);
 #pragma unroll
             for (int l = 0; l < NB; ++l) {
                 const T raw = *reinterpret_cast<const T*>(smem + l * plane + from);
@@ -1185,7 +1207,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(CompressArgs a,
                     if (packed) packed[(int64_t)l * a.kcap + at] = (__float_as_uint(B == 4 ? 2.f * to_f32(raw) : to_f32(raw)) >> 16) | place;
             }
         }
-        if (e0 + 32 * (tid + 1) == n_e) {  // the last positions of all
+        if (e0 + 32 * (word + 1) == n_e) {  // the last positions of all
             off[(n_e / 32 + tile_words - 1) / tile_words] = (int32_t)at;
             if ((int64_t)at != a.n_keep) atomicMax(a.status, (int32_t)kFlagCountMismatch);
         }
@@ -1215,6 +1237,7 @@ cudaError_t launch_chain(int cluster, void (*kernel)(A...), dim3 grid, int threa
 template <typename T, int B>
 cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* const* v_layers, int block_begin, int block_end, cudaStream_t st) {
     static PerDevice once;
+    static std::atomic<int> long_clusters[PerDevice::kMaxDevices][2][kSmallSmem / 4096 + 1];  // [two or four words][4 KiB of shared memory]; 0: not known
     int sms = 0;
     constexpr int CE = compress_chunk(B, (int)sizeof(T));
     const size_t smem = 2 * (size_t)B * CE * sizeof(T) + (B == 4 ? CE * sizeof(uint16_t) : 0);  // (a block of four: room for positions)
@@ -1222,7 +1245,13 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
         cudaError_t e1 = cudaFuncSetAttribute(split_kernel<T, B, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(threshold_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kThrMini * 128);
         if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(split_kernel<T, B, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        return e1 != cudaSuccess ? e1 : cudaFuncSetAttribute(small_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+        if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(small_kernel<T, B, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+        for (int w = 0; w < 2 && e1 == cudaSuccess; ++w) {
+            auto* const kernel = w ? small_kernel<T, B, 4> : small_kernel<T, B, 2>;
+            e1 = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+            if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        }
+        return e1;
     }, &sms);
     if (e != cudaSuccess) return e;
     const int64_t n = (int64_t)a.T * a.d;
@@ -1230,14 +1259,48 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     // few short unit-tensors: a cluster each, of as many blocks as have a tile, two blocks per SM
     const int tile_e = kResTile * a.d;
     const int64_t tiles = (n + tile_e - 1) / tile_e;
-    int cluster = 8;
-    while (cluster > tiles) cluster /= 2;
-    const int64_t range = (tiles + cluster - 1) / cluster * tile_e;
-    const size_t small_smem = (size_t)range * (B == 4 ? 4 : 1) * sizeof(T);
-    const int uts = a.Hkv * a.tensors;
+    const int uts = a.Hkv * a.tensors, n_ut = uts * (block_end - block_begin);
     // (blocks of four with nearly all entries: a thread writes too many of its own; 1000 x 128 293 and 108 us, 300 x 128 68 and 87)
     const bool few = B == 2 || (double)a.n_keep <= kAllShare * (double)n || n <= 40 * 1024;
-    if (few && range <= kSmallElems && small_smem <= (size_t)kSmallSmem && (int64_t)cluster * uts * (block_end - block_begin) <= 2 * sms) {
+    int cluster = 8, words = 1;
+    while (cluster > tiles) cluster /= 2;
+    int64_t range = 0;
+    size_t small_smem = 0;
+    auto fits = [&]() {
+        range = (tiles + cluster - 1) / cluster * tile_e;
+        small_smem = (size_t)range * (B == 4 ? 4 : 1) * sizeof(T);
+        return range <= (int64_t)words * kSmallElems && range < 65536 && small_smem <= (size_t)kSmallSmem;  // (counts of 16 bits)
+    };
+    bool small = few && fits() && (int64_t)cluster * n_ut <= 2 * sms;
+    // Longer ones take clusters of sixteen blocks, two or four words of positions per thread, while all of the clusters run at one
+    // time (us, one tensor, keep 1/16, against the four kernels: bf16 192k positions 33.7 -> 16.1, 512k 39.9 -> 21.1; float32 256k 44.7 -> 31.5, 512k
+    // 55.9 -> 36.6).
+    if (few && !small && (int64_t)16 * n_ut <= 2 * sms && tiles >= 16) {
+        cluster = 16;
+        for (words = 2; words <= 4 && !small; words *= 2) {
+            if (!fits()) continue;
+            const int wi = words / 4, bucket = (int)((small_smem + 4095) / 4096);
+            int dev = 0, at_once = 0;
+            if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+            if ((at_once = long_clusters[dev][wi][bucket].load(std::memory_order_relaxed)) == 0) {  // (asked once per amount of shared memory)
+                cudaLaunchConfig_t q = {};
+                q.gridDim = dim3(16);
+                q.blockDim = dim3(kSmallThreads);
+                q.dynamicSmemBytes = (size_t)bucket * 4096;
+                cudaLaunchAttribute attr[1];
+                attr[0].id = cudaLaunchAttributeClusterDimension;
+                attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+                q.attrs = attr;
+                q.numAttrs = 1;
+                if ((e = cudaOccupancyMaxActiveClusters(&at_once, words == 2 ? small_kernel<T, B, 2> : small_kernel<T, B, 4>, &q)) != cudaSuccess) return e;
+                long_clusters[dev][wi][bucket].store(at_once > 0 ? at_once : -1, std::memory_order_relaxed);
+            }
+            small = n_ut <= at_once;
+            if (small) break;
+        }
+    }
+    if (small) {
+        auto* const kernel = words == 1 ? small_kernel<T, B, 1> : words == 2 ? small_kernel<T, B, 2> : small_kernel<T, B, 4>;
         for (int b0 = block_begin; b0 < block_end; b0 += kSplitLayers / B) {
             const int nb = std::min(block_end - b0, kSplitLayers / B);
             for (int l = 0; l < nb * B; ++l) {
@@ -1245,7 +1308,7 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
                 a.v[l] = v_layers[B * b0 + l];
             }
             a.ut_base = b0 * uts;
-            if ((e = launch_chain(cluster, small_kernel<T, B>, dim3(cluster * uts * nb), kSmallThreads, small_smem, st, a, cluster, (int)range)) != cudaSuccess) return e;
+            if ((e = launch_chain(cluster, kernel, dim3(cluster * uts * nb), kSmallThreads, small_smem, st, a, cluster, (int)range)) != cudaSuccess) return e;
         }
         return cudaSuccess;
     }

@@ -84,3 +84,45 @@ def test_any_scale(scale, den, T):
     want = R.select_entries(z1, k)
     assert np.array_equal(idx.cpu().numpy(), want)
     assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want])
+
+
+@pytest.mark.parametrize("dtype,d,T", [("bf16", 128, 2064), ("bf16", 64, 4111), ("bf16", 128, 4096), ("bf16", 128, 4097), ("bf16", 128, 8064), ("bf16", 128, 8065),
+                                       ("f32", 128, 4096), ("f32", 128, 4097), ("f32", 64, 4099), ("f32", 64, 8191)])
+@pytest.mark.parametrize("den", [3, 16])
+def test_clusters_of_sixteen(dtype, d, T, den):
+    """Two and four words of positions per thread, at and beside the most that each holds (counts of 16 bits, shared memory)."""
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=1, n_q_heads=1, head_dim=d, T=T, dtype=dtype, n_needles=2, W=1, keep_num=1, keep_den=den,
+                                            name="sixteen")
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    check_compression(pf.ctx, w, 0, 0, 0)
+    assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("T", [600, 1500, 1600])
+def test_blocks_of_four_in_clusters_of_sixteen(T):
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=4, n_kv_heads=1, n_q_heads=1, T=T, n_needles=2, W=1, keep_num=1, keep_den=9, block_size=4, name="sixteen4")
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    for is_v, name in ((0, "k"), (1, "v")):
+        u = R4.Unit4(synth.block_tensor(w, 0, 0, 0, False), synth.block_tensor(w, 0, 0, 0, True), True, 1, 9)
+        idx, val = pf.ctx.get_residual(0, 0, 0, is_v)
+        assert np.array_equal(idx.cpu().numpy(), u.kept[name])
+        assert np.array_equal(val.float().cpu().numpy(), np.stack([u.dev[name][l].ravel()[u.kept[name]] for l in range(4)]))
+    assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("keep", [(0, 1), (1, 1), (1, 3), (2, 3)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_ties_over_sixteen_blocks(dtype, keep):
+    T, d = 4099, 64
+    rng = np.random.default_rng(6)
+    diff, base = rng.integers(-1, 2, (T, d)).astype(np.float32), rng.integers(-4, 5, (T, d)).astype(np.float32)
+    x0, x1 = (torch.from_numpy(a).cuda().to(dtype) for a in (base + diff, base - diff))
+    k = T * d * keep[0] // keep[1]
+    z0, idx, val = torch.empty((T, d), dtype=dtype, device="cuda"), torch.full((max(k, 4),), -1, dtype=torch.int32, device="cuda"), torch.empty(max(k, 4), dtype=dtype, device="cuda")
+    assert B.compress_unit_noalloc(x0, x1, *keep, z0, idx[:k] if k else idx, val[:k] if k else val) == k
+    _, z1 = R.depth_split(x0.float().cpu().numpy(), x1.float().cpu().numpy(), dtype == torch.bfloat16)
+    want = R.select_entries(z1, k)
+    assert np.array_equal(idx[:k].cpu().numpy(), want)
+    assert np.array_equal(val[:k].float().cpu().numpy(), z1.ravel()[want])
