@@ -962,6 +962,7 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 // While the clusters take two turns at most (two blocks fit an SM up to about 88 KiB of values each): 32 tensors
 // of blocks of four, 1000 x 128, two turns, 66 us against 64; 256 pairs of 1024 x 128, seven turns, 195 against 133.
 // W: words of 32 positions per thread.
+constexpr int kSmallNear = 1024;  // keys that are gathered at most
 constexpr int kSmallThreads = 512, kSmallElems = 32 * kSmallThreads, kSmallSmem = 128 * 1024;
 
 template <typename T, int B, int W>
@@ -971,9 +972,11 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     constexpr int CH = 4 * Q;                       // 16-byte chunks of 32 positions
     constexpr int MOST = W == 1 ? 8 : 16;           // blocks of a cluster
     extern __shared__ __align__(16) uint8_t smem[];  // [NB][range] values, the chunks of a word of 32 positions swizzled
-    // histograms: of the key's first digit (bf16 pairs: of the whole key in a window, two counts of 16 bits a word), the digits after it
-    __shared__ __align__(16) uint32_t s_h1[2048], s_h2[TWO ? 4 : 2048], s_all[TWO ? 4096 : 2048];
-    __shared__ uint32_t s_count, s_warp[kSmallThreads / 32], s_before[2][kSmallThreads / 32];
+    // histograms: of the key's top 15 bits in a window (two counts of 16 bits a word), of two digits after it; the low halves of the keys that
+    // share the threshold's top half
+    __shared__ __align__(16) uint32_t s_h1[2048], s_h2[TWO ? 4 : 2048], s_all[4096];
+    __shared__ uint16_t s_near[TWO ? 4 : kSmallNear];
+    __shared__ uint32_t s_count, s_warp[kSmallThreads / 32], s_before[2][kSmallThreads / 32], s_n, s_off[17], s_low[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x % blocks, item = blockIdx.x / blocks, uts = a.Hkv * a.tensors;
     const int ut = a.ut_base + item, blk = item / uts, u = item % uts, h = u / a.tensors, is_v = u % a.tensors;
@@ -984,13 +987,15 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
         s_h1[i] = 0;
         if (!TWO) s_h2[i] = 0;
     }
-    // (bf16 pairs) a key's bin: 4 095 keys from `from` up, 32 octaves, the last bin for what is larger.  At first 2^-24 to 2^8.
-    uint32_t from = (127u - 24u) << 7;
+    if (tid == 0) s_n = 0;
+    // a key's bin: 4 095 values of its top 15 bits from `from` up, 32 octaves, the last bin for what is larger.  At first 2^-24 to 2^8, of
+    // energies 2^-16 to 2^16.
+    uint32_t from = (127u - (B == 4 ? 16u : 24u)) << 7;
     auto count_key = [&](uint32_t key) {
         const uint32_t k16 = key >> 16;
         if (k16 < from) return;
         const uint32_t bin = min(k16 - from, 4095u);
-        atomicAdd(&s_h1[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has at most 2^14 positions)
+        atomicAdd(&s_h1[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has fewer than 2^16 positions)
     };
     auto chunk_at = [&](int word, int j) { return (word * CH + (j ^ (Q == 1 ? (word >> 1) & 3 : word & 7))) * 16; };
     chain_wait();
@@ -1028,10 +1033,7 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
                     *reinterpret_cast<uint4*>(smem + l * plane + chunk_at(p >> 5, ((p >> 3) & 3) * Q + k)) = hf[l][k];
                 }
             }
-            Eight<T, B>::keys(hf, [&](int, uint32_t key) {
-                if constexpr (TWO) count_key(key);
-                else atomicAdd(&s_h1[key >> 20], 1u);
-            });
+            Eight<T, B>::keys(hf, [&](int, uint32_t key) { count_key(key); });
         }
     }
     // f(w, i, key) for position i of the thread's word w, whose 32 positions are all there or none of them
@@ -1053,11 +1055,12 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     };
     // ---- the n_keep-th largest key of the cluster ----
     uint32_t tau = kNoKey, need = 0;
-    uint32_t gt_before = 0, eq_before = 0;  // (bf16 pairs) this thread's part of the counts of the blocks before this one
+    uint32_t gt_before = 0, eq_before = 0;  // this thread's part of the counts of the blocks before this one
+    bool counted = true;                    // (the same for the whole cluster)
     cluster_sync();
-    if (TWO && a.n_keep > 0) {
-        // The blocks' histograms give the threshold and, of the blocks before this one, how many keys are above it and equal to it: one
-        // exchange instead of three (a digit of 11 bits, one of 4, the counts).
+    if (a.n_keep > 0) {  // (the same for every block)
+        // The blocks' histograms give the threshold's top half and, of the blocks before this one, how many keys are above it and equal to it:
+        // for bf16 magnitudes one exchange in all.
         uint32_t bin, above, of_before[8];
         for (;;) {
             const uint32_t at = (uint32_t)__cvta_generic_to_shared(s_h1) + 16 * tid;  // four words, eight bins
@@ -1105,29 +1108,89 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
             if (8 * tid + i > (int)bin) gt_before += of_before[i];
             if (8 * tid + i == (int)bin) eq_before += of_before[i];
         }
-    } else if (a.n_keep > 0) {  // (the same for every block)
-        uint32_t bin, above, left = (uint32_t)a.n_keep;
-        {
-            const uint32_t at = (uint32_t)__cvta_generic_to_shared(s_h1) + 8 * tid;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) *reinterpret_cast<uint2*>(&s_all[1024 * i + 2 * tid]) = cluster_sum2<MOST>(at + 4096 * i, blocks);
-        }
-        __syncthreads();
-        find_bin<kSmallThreads, 2048>(s_all, left, bin, above);
-        left -= above;
-        tau = bin;
-        auto level = [&](uint32_t* hist, int shift) {
-            each([&](int, int, uint32_t key) { if (key >> (shift + 10) == tau) atomicAdd(&hist[key >> shift & 1023u], 1u); });
+        if constexpr (!TWO) {
+            // The few keys with that top half (a 128th of an octave) are gathered, and every block ranks all of them: one more exchange instead of
+            // two digits and the counts.  float32 pairs, us: 509 x 128 15.7 -> 13.8, 2048 x 128 31.5 -> 26.5.
+            const uint32_t top = from + bin;
+            uint32_t left = need;
+            eq_before = 0;
+            each([&](int, int, uint32_t key) {
+                if (key >> 16 == top) {
+                    const uint32_t i = atomicAdd(&s_n, 1u);
+                    if (i < (uint32_t)kSmallNear) s_near[i] = (uint16_t)key;
+                }
+            });
             cluster_sync();
-            *reinterpret_cast<uint2*>(&s_all[2 * tid]) = cluster_sum2<MOST>((uint32_t)__cvta_generic_to_shared(hist) + 8 * tid, blocks);
-            __syncthreads();
-            find_bin<kSmallThreads, 1024>(s_all, left, bin, above);
-            left -= above;
-            tau = tau << 10 | bin;
-        };
-        level(s_h2, 10);
-        level(s_h2 + (TWO ? 0 : 1024), 0);
-        need = left;  // of the positions whose key is tau, the lowest
+            uint32_t mine_n = 0;
+            {
+                uint32_t at;
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_n)), "r"(lane < blocks ? lane : 0));
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(mine_n) : "r"(at) : "memory");
+                if (lane >= blocks) mine_n = 0;
+            }
+            uint32_t off_n = mine_n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, off_n, o);
+                if (lane >= o) off_n += y;
+            }
+            const uint32_t m = __shfl_sync(0xFFFFFFFFu, off_n, 31);
+            counted = m <= (uint32_t)kSmallNear;
+            if (counted) {
+                if (warp == 0 && lane < 17) s_off[lane] = off_n - mine_n;  // ([blocks, 16]: all of them)
+                __syncthreads();
+                for (uint32_t i = tid; i < m; i += kSmallThreads) {
+                    int r = 0;
+#pragma unroll
+                    for (int k = 1; k < MOST; ++k) r += k < blocks && s_off[k] <= i;
+                    uint32_t at;
+                    uint16_t low;
+                    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(s_near) + 2 * (i - s_off[r])), "r"(r));
+                    asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(low) : "r"(at) : "memory");
+                    s_all[i] = (uint32_t)low | (uint32_t)r << 16;
+                }
+                __syncthreads();
+                for (uint32_t i = tid; i < m; i += kSmallThreads) {
+                    const uint32_t low = s_all[i] & 0xFFFFu;
+                    uint32_t g = 0, e = 0;
+#pragma unroll 2
+                    for (uint32_t k = 0; k < m; k += 4) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(&s_all[k]);
+                        const uint32_t other[4] = {v.x & 0xFFFFu, v.y & 0xFFFFu, v.z & 0xFFFFu, v.w & 0xFFFFu};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            g += k + q < m && other[q] > low;
+                            e += k + q < m && other[q] == low;
+                        }
+                    }
+                    if (g < left && left <= g + e) { s_low[0] = low; s_low[1] = g; }
+                }
+                __syncthreads();
+                tau = top << 16 | s_low[0];
+                need = left - s_low[1];
+                for (uint32_t i = tid; i < m; i += kSmallThreads) {
+                    const uint32_t low = s_all[i] & 0xFFFFu;
+                    if ((int)(s_all[i] >> 16) < rank) {
+                        gt_before += low > s_low[0];
+                        eq_before += low == s_low[0];
+                    }
+                }
+            } else {  // many equal keys: digits of 10 and 6 bits
+                tau = top;
+                auto level = [&](uint32_t* hist, int shift, int bits) {
+                    each([&](int, int, uint32_t key) { if (key >> (shift + bits) == tau) atomicAdd(&hist[key >> shift & ((1u << bits) - 1u)], 1u); });
+                    cluster_sync();
+                    *reinterpret_cast<uint2*>(&s_all[2 * tid]) = cluster_sum2<MOST>((uint32_t)__cvta_generic_to_shared(hist) + 8 * tid, blocks);
+                    __syncthreads();
+                    find_bin<kSmallThreads, 1024>(s_all, left, bin, above);
+                    left -= above;
+                    tau = tau << bits | bin;
+                };
+                level(s_h2, 6, 10);
+                level(s_h2 + 1024, 0, 6);
+                need = left;  // of the positions whose key is tau, the lowest
+            }
+        }
     }
     // ---- entries: those above in the blocks, warps and threads before, then those equal (counts in halves: at most 2^14) ----
     uint32_t gt[W] = {}, eq[W] = {}, cnt = 0;
@@ -1144,11 +1207,9 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
         if (lane >= o) incl += y;
     }
     if (lane == 31) s_warp[warp] = incl;
-    if constexpr (TWO) {
-        gt_before = __reduce_add_sync(0xFFFFFFFFu, gt_before);
-        eq_before = __reduce_add_sync(0xFFFFFFFFu, eq_before);
-        if (lane == 0) { s_before[0][warp] = gt_before; s_before[1][warp] = eq_before; }
-    }
+    gt_before = __reduce_add_sync(0xFFFFFFFFu, gt_before);
+    eq_before = __reduce_add_sync(0xFFFFFFFFu, eq_before);
+    if (lane == 0) { s_before[0][warp] = gt_before; s_before[1][warp] = eq_before; }
     __syncthreads();
     uint32_t before = incl - cnt, total = 0;
 #pragma unroll
@@ -1157,7 +1218,7 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
         total += s_warp[w];
     }
     uint32_t run_gt = before >> 16, run_eq = before & 0xFFFFu;
-    if constexpr (TWO) {
+    if (counted) {
 #pragma unroll
         for (int w = 0; w < kSmallThreads / 32; ++w) { run_gt += s_before[0][w]; run_eq += s_before[1][w]; }
     } else {
