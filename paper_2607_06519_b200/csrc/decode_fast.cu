@@ -319,9 +319,11 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         seg_info[0] = n;
         seg_info[1] = it0;
         for (int s = 0; s < kStages; ++s) stage_cnt[s] = 0;
-        // fill the stages up to the first tile of a tail, whose rows may still be written by the kernels ahead
+        // fill the stages up to the first tile of a tail, whose rows may still be written by the kernels ahead; all but one of them (not in
+        // clusters): with all, the copies of 148 blocks keep the memory busy while the kernels ahead join their parts, whose few loads wait
+        // for them (us a call, 32k: all three stages 26.2, two 25.8, one 26.1; 8-bit rows, two stages: 21.3 and 20.7 with one)
         if (n > 0)
-            for (; prologue_issued < kStages && prologue_issued < segs[0].npre; ++prologue_issued)
+            for (; prologue_issued < (CL ? kStages : kStages - 1) && prologue_issued < segs[0].npre; ++prologue_issued)
                 issue_tile(prologue_issued);
     }
     // per-warp scratch starts zeroed
