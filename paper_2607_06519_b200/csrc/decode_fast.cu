@@ -955,18 +955,21 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     sch.units = units;
     sch.cluster = 0;
     // Clusters, as many blocks per unit as fit: one kernel instead of two, where that is worth more than the blocks that are
-    // left out.  The hand-over to the combine kernel and its launch cost as much as kClusterGain plain tiles of one block.  Us a layer
-    // replayed (eight KV heads, clusters of eight), clusters against two kernels: 512 tokens 4.6 and 6.6, 1024 5.0 and 7.0, 2047 6.4
-    // and 7.7, 4096 9.9 and 8.9; with a tail 1024 6.0 and 6.8, 2047 7.7 and 7.9, 3000 9.1 and 8.6.  8-bit rows, whose tails make the
-    // last block later: 1024 6.5 and 8.8, 4096 10.5 and 10.7, 8192 15.2 and 11.5; with a tail 1024 8.5 and 9.1, 3000 9.1 and 9.9,
-    // 4096 13.0 and 11.5.
+    // left out.  Measured on a stream, us a call of bf16 rows: clusters 3.55 + 1.03 for each plain tile of the slowest block (a tail tile counts 1.5),
+    // two kernels 5.7 + 1.1 for each of the average block and at least 7.75 (8.4 with tails), the two hand-overs.  Eight KV heads, clusters against
+    // two kernels: 1 024 tokens 5.4 and 7.7, 2 047 6.8 and 7.8, 3 000 8.1 and 7.8, 8 191 15.5 and 11.1; with a tail 1 024 6.3 and 8.4, 1 500
+    // 7.2 and 8.5, 2 047 8.4 and 8.4, 3 000 9.9 and 8.8; two KV heads 2 047 5.7 and 7.7, with a tail 7.2 and 8.4, 4 096 8.4 and 7.8.
+    // 8-bit rows (4.6 + 1.05 against 5.7 + 1.15 and 7.9): 1 024 7.1 and 7.9, 2 047 8.3 and 8.1, 3 000 9.7 and 8.5; their tails make the last block
+    // of the other cut later (at least 10.5): 1 024 9.3 and 10.5, 3 000 10.5 and 11.3, 4 096 12.3 and 11.1.
     // Up to five tiles per SM, the other cut also pays for rounding its shares to tiles, about what a block that ends a unit is
     // charged: that counts then (units of bf16, ragged lengths up to the given one, a third to a half residual; clusters and two
     // kernels: 128 of 459 tokens 11.9 and 14.8, 64 of 1181 9.4 and 10.8, 32 of 3267 10.7 and 11.7).  Longer ones don't (128 of 2174 36.1 and
     // 31.7, 64 of 2972 26.1 and 20.4, 144 of 3000 43.0 and 36.3), nor 8-bit rows (48 of 537 10.1 and 8.8, 32 of 2270 13.2 and 11.3, though 128 of
     // 949 20.5 and 22.4).
     if (max_clusters) {
-        const double kClusterGain = a.rows_f8 ? 3.0 : 2.1;
+        bool tails = false;
+        for (int b = 0; b < a.batch && a.host_tail; ++b) tails = tails || a.host_tail[b] > 0;
+        const double gain = tails ? 2.7 : a.rows_f8 ? 1.0 : 2.1, least_other = a.rows_f8 ? 2.1 : 1.9;
         int least = ns[0];
         for (int u = 1; u < units; ++u) least = std::min(least, ns[u]);
         int lg = 3;
@@ -998,7 +1001,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
                 all += (double)ns[u] * wt[u] / (kTT / kResTile) / tile + tail;
                 if (!a.rows_f8 && total_tiles <= 5 * ctas) all += (double)(5 * total_tiles / ctas) / 8.0;
             }
-            if (worst <= std::max(1.0, all / ctas) + kClusterGain) {
+            if (worst <= std::max(least_other, all / ctas) + gain) {
                 int c = 0;
                 for (int u = 0; u < units; ++u)
                     for (int j = 0; j < C; ++j, ++c) {

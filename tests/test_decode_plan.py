@@ -194,3 +194,12 @@ def test_short_ragged_units_are_clusters():
         for scale, expect in ((1, n), (5, 0)):
             T = [T0 * scale - b * T0 * scale // (2 * batch) - b for b in range(batch)]
             assert _cluster_cut(T, modes, [0] * batch, hkv, 4)[0] == expect
+
+
+@pytest.mark.parametrize("hkv,T,tail,row_format,expect", [(8, 1024, 0, 0, 8), (8, 2047, 0, 0, 8), (8, 2047, 41, 0, 8), (8, 3000, 0, 0, 0), (8, 3000, 41, 0, 0),
+                                                          (2, 2047, 41, 0, 8), (2, 4096, 0, 0, 0), (8, 8191, 0, 0, 0), (8, 3000, 0, 1, 0), (8, 3000, 41, 1, 8),
+                                                          (8, 4096, 41, 1, 0)])
+def test_clusters_of_middle_lengths(hkv, T, tail, row_format, expect):
+    """Either side of the length from which two kernels are faster, with tails (whose hand-over clusters save too) and without."""
+    modes = [0, 1, 2, 1, 0, 1, 0, 1][:hkv]
+    assert _cluster_cut([T], modes, [tail], hkv, 4, row_format)[0] == expect
