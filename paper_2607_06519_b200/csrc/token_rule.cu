@@ -34,9 +34,9 @@ constexpr int kTN = 256;                    // probe rows per item (N of the MMA
 constexpr int kTStages = 3;
 constexpr int kTAHalf = kTM * 128;          // one 64-channel half of a token tile: 16 KiB
 constexpr int kTAStage = 2 * kTAHalf;       // 32 KiB
-constexpr int kTHdr = 3072;                 // barriers, TMEM slot, abort flag, the epilogue's exchange
-constexpr int kTThreads = 12 * 32;          // copies, MMAs, probe rows, one idle, eight of the epilogue
-constexpr int tFull = 0, tEmpty = 32, tTFull = 64, tTEmpty = 80, tSlot = 96, tAbort = 100, tBFull = 112, tBEmpty = 128, tExch = 1024;
+constexpr int kTHdr = 2048;                 // barriers, TMEM slot, abort flag, the epilogue's exchange
+constexpr int kTThreads = 20 * 32;          // copies, MMAs, probe rows, one idle, sixteen of the epilogue
+constexpr int tFull = 0, tEmpty = 32, tTFull = 64, tTEmpty = 80, tSlot = 96, tAbort = 100, tBFull = 112, tBEmpty = 128, tExch = 256;
 constexpr int score_smem(int nt) { return kTHdr + 2 * nt * 256 + kTStages * kTAStage; }
 static_assert(score_smem(kTN) <= 227 * 1024, "shared memory budget");
 
@@ -48,16 +48,17 @@ struct ScorePlan {
 
 // NT: probe rows per item (64, 128 or 256: the smallest that holds a layer's rows, so that few probe rows do not pay for 256).
 // One persistent block per SM.  Warp 0 streams the token tiles, warp 2 the probe rows of the next item into the other of two
-// buffers, one thread of warp 1 issues the MMAs, eight warps take the results: two per quarter of the TMEM lanes, half of the columns
-// each, joined through shared memory.  Bound by the MMAs (1 024 cycles a tile of 128 x 256 x 128) with the epilogue close behind: four
-// warps took 1.6 us a tile, and a block per item and third of its tiles, each with its own probe rows, left the last of six waves a
-// fifth full (8 191 tokens, 8 blocks of four, 8 heads, 256 rows a layer: 214 -> 165 us).
+// buffers, one thread of warp 1 issues the MMAs, sixteen warps take the results: four per quarter of the TMEM lanes, a fourth of the columns
+// each (64 rows: two, a half).  Bound by the hand-overs between copies, MMAs (1 024 cycles a tile of 128 x 256 x 128) and epilogue: 8 191 tokens, 8
+// blocks of four, 8 heads, 256 rows a layer: four epilogue warps, and a block per item and third of its tiles, each with its own probe
+// rows, the last of six waves a fifth full, 214 us; eight warps 165; sixteen 159 (117 without an epilogue).
 template <int NT>
 __global__ void __launch_bounds__(kTThreads, 1)
 token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScorePlan pl) {
     constexpr uint32_t kIdesc = umma_idesc(kTM, NT, false);
     constexpr int kBHalf = NT * 128, kBBytes = 2 * kBHalf;  // one 64-channel half of the probe rows, both
     constexpr uint32_t kCols = 2 * NT;                      // TMEM columns: two accumulators
+    constexpr int kParts = NT >= 128 ? 4 : 2;               // epilogue warps that share a lane's columns
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sm0 = s_u32(smem);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + tAbort);
@@ -71,7 +72,7 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
     if (threadIdx.x == 0) {
         for (int s = 0; s < kTStages; ++s) { mb_init(sm0 + tFull + 8 * s, 1); mb_init(sm0 + tEmpty + 8 * s, 1); }
         for (int s = 0; s < 2; ++s) {
-            mb_init(sm0 + tTFull + 8 * s, 1); mb_init(sm0 + tTEmpty + 8 * s, 8);
+            mb_init(sm0 + tTFull + 8 * s, 1); mb_init(sm0 + tTEmpty + 8 * s, 4 * kParts);
             mb_init(sm0 + tBFull + 8 * s, 1); mb_init(sm0 + tBEmpty + 8 * s, 1);
         }
         *abort_flag = 0;
@@ -161,11 +162,11 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
             __syncwarp();
             if (lane == 0) mb_arrive(sm0 + tBFull + 8 * bs);
         });
-    } else if (warp >= 4) {
+    } else if (warp >= 4 && warp < 4 + 4 * kParts) {
         // ---- epilogue: lane = token (TMEM lane); maximum of |D| and sum of D^2 over the probe rows that see the token ----
-        const int lq = warp & 3, half = (warp - 4) >> 2;
-        constexpr int kHalf = NT / 2, kLd = kHalf < 64 ? kHalf : 64;  // columns of a warp; of a round
-        float2* const exch = reinterpret_cast<float2*>(smem + tExch) + lq * 32 + lane;  // [2][128]
+        const int lq = warp & 3, part = (warp - 4) >> 2;
+        constexpr int kPart = NT / kParts;  // columns of a warp: 32 or 64
+        float* const exch = reinterpret_cast<float*>(smem + tExch) + lq * 32 + lane;  // [kParts - 1][128] sums
         const float c32 = a.B == 4 ? 1.f : __uint_as_float(0x3F3504F3u);  // a pair's rows are Z1: K - Khat^shared = +-c Z1
         items([&](int, int unit, int layer, int mblock, int t0, int n, int i0) {
             float* const err = a.err + ((int64_t)unit * a.nslots + layer * pl.mblocks + mblock) * a.Tmax;
@@ -177,53 +178,56 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 float m0 = 0.f, m1 = 0.f, e0 = 0.f, e1 = 0.f;
                 if (!*abort_flag) {
-                    const bool all_visible = tile_t0 + kTM - 1 <= pl.pos_min;
+                    uint32_t r[kPart / 32][32];
+                    const uint32_t ta = tmem_base + ((uint32_t)(lq * 32) << 16) + (uint32_t)(as * NT + part * kPart);
 #pragma unroll
-                    for (int c0 = 0; c0 < kHalf; c0 += kLd) {
-                        uint32_t r[kLd / 32][32];
-                        const uint32_t ta = tmem_base + ((uint32_t)(lq * 32) << 16) + (uint32_t)(as * NT + half * kHalf + c0);
+                    for (int p = 0; p < kPart / 32; ++p) tmem_ld32(ta + 32 * p, r[p]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    // read: the next product may take the accumulator
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mb_arrive(sm0 + tTEmpty + 8 * as);
+                    if (tile_t0 + kTM - 1 <= pl.pos_min) {  // every row sees every token
 #pragma unroll
-                        for (int p = 0; p < kLd / 32; ++p) tmem_ld32(ta + 32 * p, r[p]);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        if (c0 + kLd == kHalf) {  // read: the next product may take the accumulator
-                            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                            __syncwarp();
-                            if (lane == 0) mb_arrive(sm0 + tTEmpty + 8 * as);
-                        }
-                        if (all_visible) {
+                        for (int p = 0; p < kPart / 32; ++p)
 #pragma unroll
-                            for (int p = 0; p < kLd / 32; ++p)
+                            for (int j = 0; j < 32; j += 4) {
+                                const float u = __uint_as_float(r[p][j]), v = __uint_as_float(r[p][j + 1]);
+                                const float w = __uint_as_float(r[p][j + 2]), x = __uint_as_float(r[p][j + 3]);
+                                m0 = fmaxf(m0, fmaxf(fabsf(u), fabsf(v)));
+                                m1 = fmaxf(m1, fmaxf(fabsf(w), fabsf(x)));
+                                e0 = fmaf(u, u, e0);
+                                e1 = fmaf(v, v, e1);
+                                e0 = fmaf(w, w, e0);
+                                e1 = fmaf(x, x, e1);
+                            }
+                    } else {
 #pragma unroll
-                                for (int j = 0; j < 32; j += 4) {
-                                    const float u = __uint_as_float(r[p][j]), v = __uint_as_float(r[p][j + 1]);
-                                    const float w = __uint_as_float(r[p][j + 2]), x = __uint_as_float(r[p][j + 3]);
-                                    m0 = fmaxf(m0, fmaxf(fabsf(u), fabsf(v)));
-                                    m1 = fmaxf(m1, fmaxf(fabsf(w), fabsf(x)));
-                                    e0 = fmaf(u, u, e0);
-                                    e1 = fmaf(v, v, e1);
-                                    e0 = fmaf(w, w, e0);
-                                    e1 = fmaf(x, x, e1);
-                                }
-                        } else {
+                        for (int p = 0; p < kPart / 32; ++p)
 #pragma unroll
-                            for (int p = 0; p < kLd / 32; ++p)
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) {
-                                    const int row = mblock * NT + half * kHalf + c0 + 32 * p + j;
-                                    const float u = __uint_as_float(r[p][j]);
-                                    if (row < rows_layer && a.pos[row % a.W] >= t) { m0 = fmaxf(m0, fabsf(u)); e0 = fmaf(u, u, e0); }
-                                }
-                        }
+                            for (int j = 0; j < 32; ++j) {
+                                const int row = mblock * NT + part * kPart + 32 * p + j;
+                                const float u = __uint_as_float(r[p][j]);
+                                if (row < rows_layer && a.pos[row % a.W] >= t) { m0 = fmaxf(m0, fabsf(u)); e0 = fmaf(u, u, e0); }
+                            }
                     }
+                    const float m = fmaxf(m0, m1);
+                    if (t < a.T && m > 0.f) atomicMax(score + t, __float_as_uint(m * c32));
                 }
-                // the two halves of the columns (one barrier a tile: the buffer of tile i is written again behind that of tile i + 1)
-                if (half) exch[128 * as] = make_float2(fmaxf(m0, m1), e0 + e1);
-                asm volatile("bar.sync %0, 64;" ::"r"(1 + lq) : "memory");
-                if (!half && t < a.T && !*abort_flag) {
-                    const float2 o = exch[128 * as];
-                    const float m = fmaxf(fmaxf(m0, m1), o.x);
-                    if (m > 0.f) atomicMax(score + t, __float_as_uint(m * c32));
-                    err[t] = (e0 + e1) + o.y;
+                // The parts' sums in their order: written behind the barrier that says that part 0 has read those of the tile before (not of
+                // the first), read behind the one that says that all are there.
+                const float e = e0 + e1;
+                if (part > 0) {
+                    if (i > 0) asm volatile("bar.sync %0, %1;" ::"r"(5 + lq), "n"(32 * kParts) : "memory");
+                    exch[128 * (part - 1)] = e;
+                }
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + lq), "n"(32 * kParts) : "memory");
+                if (part == 0) {
+                    float sum = e;
+#pragma unroll
+                    for (int p = 0; p < kParts - 1; ++p) sum += exch[128 * p];
+                    if (t < a.T && !*abort_flag) err[t] = sum;
+                    if (g_begin + i + 1 < g_end) asm volatile("bar.arrive %0, %1;" ::"r"(5 + lq), "n"(32 * kParts) : "memory");
                 }
             }
         });
