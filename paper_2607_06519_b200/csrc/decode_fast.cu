@@ -955,7 +955,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     sch.units = units;
     sch.cluster = 0;
     // Clusters, as many blocks per unit as fit: one kernel instead of two, where that is worth more than the blocks that are
-    // left out.  Measured on a stream, us a call of bf16 rows: clusters 3.55 + 1.03 for each plain tile of the slowest block (a tail tile counts 1.5),
+    // left out.  Measured on a stream, us a call of bf16 rows: clusters 3.55 + 1.03 for each plain tile of the slowest block (a tail tile counts 1.2),
     // two kernels 5.7 + 1.1 for each of the average block and at least 7.75 (8.4 with tails), the two hand-overs.  Eight KV heads, clusters against
     // two kernels: 1 024 tokens 5.4 and 7.7, 2 047 6.8 and 7.8, 3 000 8.1 and 7.8, 8 191 15.5 and 11.1; with a tail 1 024 6.3 and 8.4, 1 500
     // 7.2 and 8.5, 2 047 8.4 and 8.4, 3 000 9.9 and 8.8; two KV heads 2 047 5.7 and 7.7, with a tail 7.2 and 8.4, 4 096 8.4 and 7.8.
@@ -986,9 +986,10 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
                 const int tail = a.host_tail ? (std::min(a.host_tail[u / a.Hkv], a.max_tail) + kTT - 1) / kTT : 0;
                 const int even = (ns[u] + tail * (kTT / kResTile) + C - 1) / C;
                 // (Latencies of one block: a residual tile is less far above a plain one than in the throughput of a full device, and a
-                // tail tile, whose copy starts after the wait for the kernels ahead, takes half a tile more.  A 256-token tile of
-                // 8-bit rows counts as 1.7 plain ones.)
-                const double rl = std::sqrt(wt[u] / tile) * (a.rows_f8 ? 1.7 : 1.0), tl = 1.5 * tail;
+                // tail tile, whose copy starts after the wait for the kernels ahead, takes a fifth of a tile more, with 8-bit rows half of one.  With a
+                // half for all, 2 047 tokens and a tail were cut into blocks of 18 slices, three tiles, to spare the last block: 8.4 us a call against
+                // 8.0, of four heads 8.2 and 7.6.  A 256-token tile of 8-bit rows counts as 1.7 plain ones.)
+                const double rl = std::sqrt(wt[u] / tile) * (a.rows_f8 ? 1.7 : 1.0), tl = (a.rows_f8 ? 1.5 : 1.2) * tail;
                 double best = -1.0;
                 for (int p : {even / tsl * tsl, even, (even + tsl - 1) / tsl * tsl}) {
                     p = std::min(p, C > 1 ? (ns[u] - 1) / (C - 1) : 0);

@@ -156,3 +156,25 @@ def test_token_rule_on_blocks_of_four(T, keep, W, tail, dtype, d):
                 assert err.max() <= TOL[dtype], (step, layer, h, float(err.max()))
     assert pf.ctx.device_status() == 0
     pf.ctx.close()
+
+
+@pytest.mark.parametrize("group,W,T", [(1, 40, 700), (1, 64, 129), (2, 64, 1025), (1, 128, 128), (4, 64, 2048), (8, 64, 900), (8, 128, 300)])
+@pytest.mark.parametrize("hkv", [1, 8])
+def test_probe_rows_of_the_score_kernel(group, W, T, hkv):
+    """Products of 64, 128 and 256 columns and several of them per layer; tiles that end in the middle of a token tile, shares of the thread
+    blocks that end in the middle of an item; scores and the error sums that come from the same registers (float32 products, 2e-5 of
+    the largest for sums of squares of them)."""
+    from paper_2607_06519_b200 import runner
+
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=4, n_kv_heads=hkv, n_q_heads=hkv * group, T=T, n_needles=2, W=W, residual_rule=1, name="rows")
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    _, scores = pf.probe(0, 0.0)
+    for p, h in ((0, 0), (1, hkv - 1)):
+        u, pq = _unit(w, p, h), (synth.probe_q(w, 0, 2 * p), synth.probe_q(w, 0, 2 * p + 1))
+        tok, sc = pf.ctx.get_token_set(0, p, h, T)
+        s_ref = R.token_scores(u.z1["k"], pq[0], pq[1], group, h, synth.probe_positions(w))
+        np.testing.assert_allclose(f32(sc).astype(np.float64), s_ref, rtol=1e-5, atol=1e-6 * max(1.0, s_ref.max()))
+        u.use_tokens(tok.cpu().numpy())
+        np.testing.assert_allclose(scores[p, h], R.probe_error(u.z1["k"], u.kept["k"], pq[0], pq[1], group, h, synth.probe_positions(w)), rtol=2e-5, atol=1e-9)
+    assert pf.ctx.device_status() == 0
