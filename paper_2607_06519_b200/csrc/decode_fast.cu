@@ -958,7 +958,7 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     // left out.  Measured on a stream, us a call of bf16 rows: clusters 3.55 + 1.03 for each plain tile of the slowest block (a tail tile counts 1.2),
     // two kernels 5.7 + 1.1 for each of the average block and at least 7.75 (8.4 with tails), the two hand-overs.  Eight KV heads, clusters against
     // two kernels: 1 024 tokens 5.4 and 7.7, 2 047 6.8 and 7.8, 3 000 8.1 and 7.8, 8 191 15.5 and 11.1; with a tail 1 024 6.3 and 8.4, 1 500
-    // 7.2 and 8.5, 2 047 8.4 and 8.4, 3 000 9.9 and 8.8; two KV heads 2 047 5.7 and 7.7, with a tail 7.2 and 8.4, 4 096 8.4 and 7.8.
+    // 7.2 and 8.5, 2 047 8.0 and 8.4, 3 000 9.9 and 8.8; two KV heads 2 047 5.7 and 7.7, with a tail 6.7 and 8.4, 4 096 8.4 and 7.8.
     // 8-bit rows (4.6 + 1.05 against 5.7 + 1.15 and 7.9): 1 024 7.1 and 7.9, 2 047 8.3 and 8.1, 3 000 9.7 and 8.5; their tails make the last block
     // of the other cut later (at least 10.5): 1 024 9.3 and 10.5, 3 000 10.5 and 11.3, 4 096 12.3 and 11.1.
     // Up to five tiles per SM, the other cut also pays for rounding its shares to tiles, about what a block that ends a unit is

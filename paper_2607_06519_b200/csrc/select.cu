@@ -861,93 +861,132 @@ __device__ __forceinline__ uint32_t packed_place(uint32_t p) {
     return (half << 10 | row << 6 | chunk << 3 | (p & 7u)) << 16;
 }
 
-// grid (groups of eight chunks, unit-tensors), a chunk per warp: no block barriers, U rounds of candidates requested together
-// (one chunk per block with a block scan per round took 767 us for 32 layers of 32k tokens)
+// grid (groups of eight chunks, unit-tensors), a chunk per warp: no block barriers.  A round takes 256 candidates, eight per lane: one warp scan
+// of their counts, then positions and values of those that stay go through shared memory, so that the lists leave in runs.
+// Bound by the latency of a chunk's chain (loads, scan, both ways through shared memory) beside 2 GB of lists and candidates: 32 layers of 32k
+// tokens 300 -> 266 us, 8 blocks of four of 12 289 147 -> 130, against 32 candidates a round with two votes each.  (One chunk per block with
+// a block scan per round took 767; 6 or 8 blocks an SM by fewer registers 312 and 325.)
 template <typename T, int B, bool ALL>
 __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_begin) {
-    constexpr int NB = B == 4 ? 4 : 1, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
-    constexpr int U = 4;
+    constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
+    constexpr bool TWO = sizeof(T) == 2 && B == 2;
     __shared__ uint32_t s_map[8][WORDS];
+    __shared__ uint16_t s_pos[8][256];
+    __shared__ __align__(16) T s_val[8][NB][256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ut = ut_begin + blockIdx.y, c = blockIdx.x * 8 + warp;
     chain_wait();
     if (c >= a.chunks) return;
+    const bool map_k = a.keep && !(ut % a.tensors);  // K: a bit map of the kept positions
     uint32_t* const map = s_map[warp];
-    for (int w = lane; w < WORDS; w += 32) map[w] = 0;
+    if (map_k)
+        for (int w = lane; w < WORDS; w += 32) map[w] = 0;
     const uint32_t tau = a.sel[ut].tau, need = a.sel[ut].need;
     const int n = a.cand_n[(int64_t)ut * a.chunks_max + c];
     const int2 b0 = a.chunk_base[(int64_t)ut * a.chunks_max + c];
     const int64_t e0 = (int64_t)c * CE, n_e = (int64_t)a.T * a.d;
-    const uint16_t* const pos = a.cand_pos + (int64_t)ut * a.cand_stride + e0;
+    const uint4* const pos = reinterpret_cast<const uint4*>(a.cand_pos + (int64_t)ut * a.cand_stride + e0);
     const T* const val = reinterpret_cast<const T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0;
     uint32_t run_gt = (uint32_t)b0.x, run_eq = (uint32_t)b0.y;
-    const uint32_t first = run_gt + min(run_eq, need);  // list position of the chunk's first entry
-    const uint32_t below = (1u << lane) - 1u;
     int32_t* const idx = a.idx + (int64_t)ut * a.kcap;
     T* const out = reinterpret_cast<T*>(a.val) + (int64_t)ut * NB * a.kcap;
     uint32_t* const packed = sizeof(T) == 2 && a.packed ? a.packed + (int64_t)ut * NB * a.kcap : nullptr;
+    const int tile_shift = a.d == 128 ? 11 : 10;  // positions of a 16-token tile
+    int32_t* const off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1) + (int)(e0 >> tile_shift);
+    int tile = -1;  // of the entry before
     __syncwarp();
-    for (int i0 = lane; i0 < n + lane; i0 += 32 * U) {
-        uint32_t p[U];
-        T raw[U][NB];
+    uint4 p_next = make_uint4(0, 0, 0, 0), v_next[NB][Q];
+    auto load = [&](int i) {
+        if (i >= n) return;
+        if constexpr (!ALL) p_next = pos[i >> 3];
 #pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const int i = i0 + 32 * q;
-            if (i < n) {
-                p[q] = ALL ? (uint32_t)i : pos[i];
+        for (int l = 0; l < NB; ++l)
 #pragma unroll
-                for (int l = 0; l < NB; ++l) raw[q][l] = val[(int64_t)l * a.cand_stride + i];
+            for (int k = 0; k < Q; ++k) v_next[l][k] = reinterpret_cast<const uint4*>(val + (int64_t)l * a.cand_stride + i)[k];
+    };
+    load(8 * lane);
+    for (int base = 0; base < n; base += 256) {
+        const int i = base + 8 * lane;
+        const uint4 p8 = p_next;
+        uint4 v8[NB][Q];
+#pragma unroll
+        for (int l = 0; l < NB; ++l)
+#pragma unroll
+            for (int k = 0; k < Q; ++k) v8[l][k] = v_next[l][k];
+        load(i + 256);
+        const uint32_t valid = i >= n || tau == kNoKey ? 0u : n - i >= 8 ? 0xFFu : (1u << (n - i)) - 1u;
+        uint32_t gt = 0, eq = 0;
+        if constexpr (TWO) {
+            gt = Eight<T, B>::reach(v8, tau + 0x10000u);
+            eq = Eight<T, B>::reach(v8, tau) & ~gt;
+        } else {
+            Eight<T, B>::keys(v8, [&](int k, uint32_t key) {
+                gt |= (uint32_t)(key > tau) << k;
+                eq |= (uint32_t)(key == tau) << k;
+            });
+        }
+        gt &= valid;
+        eq &= valid;
+        const uint32_t cnt = (uint32_t)__popc(gt) << 16 | (uint32_t)__popc(eq);
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31), before = incl - cnt;
+        // ties in index order while fewer than `need` precede them
+        const uint32_t eq_before = run_eq + (before & 0xFFFFu);
+        const uint32_t first = run_gt + min(run_eq, need);  // list position of the round's first entry
+        uint32_t kept = gt, ties = min((uint32_t)__popc(eq), need - min(eq_before, need));
+        if (ties == (uint32_t)__popc(eq)) kept |= eq;
+        else
+            for (uint32_t rest = eq; ties; --ties, rest &= rest - 1) kept |= rest & (0u - rest);
+        uint32_t at = run_gt + (before >> 16) + min(eq_before, need) - first;
+        run_gt += total >> 16;
+        run_eq += total & 0xFFFFu;
+        const uint32_t n_out = run_gt + min(run_eq, need) - first;
+        const uint32_t pw[4] = {p8.x, p8.y, p8.z, p8.w};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (!(kept >> k & 1u)) continue;
+            s_pos[warp][at] = ALL ? (uint16_t)(i + k) : (uint16_t)(pw[k >> 1] >> (16 * (k & 1)));
+#pragma unroll
+            for (int l = 0; l < NB; ++l) s_val[warp][l][at] = reinterpret_cast<const T*>(&v8[l][0])[k];
+            ++at;
+        }
+        __syncwarp();
+        for (uint32_t j = lane; j < n_out; j += 32) {
+            const uint32_t p = s_pos[warp][j];
+            const int t = (int)(p >> tile_shift), t_before = j ? (int)(s_pos[warp][j - 1] >> tile_shift) : tile;
+            for (int x = t_before + 1; x <= t; ++x) off[x] = (int32_t)(first + j);
+            if (map_k) atomicOr(&map[p >> 5], 1u << (p & 31));
+            idx[first + j] = (int)e0 + (int)p;
+            const uint32_t place = sizeof(T) == 2 ? packed_place(p) : 0u;
+#pragma unroll
+            for (int l = 0; l < NB; ++l) {
+                const T raw = s_val[warp][l][j];
+                out[(int64_t)l * a.kcap + first + j] = raw;
+                // (a block of four scales its rows by 1/2 at decode time and its deviations by 1: twice the deviation is stored)
+                if constexpr (sizeof(T) == 2)
+                    if (packed) packed[(int64_t)l * a.kcap + first + j] = (__float_as_uint(B == 4 ? 2.f * to_f32(raw) : to_f32(raw)) >> 16) | place;
             }
         }
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const bool on = i0 + 32 * q < n;
-            float v[NB];
-#pragma unroll
-            for (int l = 0; l < NB; ++l) v[l] = to_f32(raw[q][l]);
-            const uint32_t key = key_of<B>(v);
-            const bool gt = on && key > tau, eq = on && key == tau;
-            const uint32_t mg = __ballot_sync(0xFFFFFFFFu, gt), me = __ballot_sync(0xFFFFFFFFu, eq);
-            const uint32_t be = run_eq + __popc(me & below);
-            if (gt || (eq && be < need)) {  // ties in index order while fewer than `need` precede them
-                const uint32_t at = run_gt + __popc(mg & below) + min(be, need);
-                idx[at] = (int)e0 + (int)p[q];
-                const uint32_t place = sizeof(T) == 2 ? packed_place(p[q]) : 0u;
-#pragma unroll
-                for (int l = 0; l < NB; ++l) {
-                    out[(int64_t)l * a.kcap + at] = raw[q][l];
-                    // (a block of four scales its rows by 1/2 at decode time and its deviations by 1: twice the deviation is stored)
-                    if constexpr (sizeof(T) == 2)
-                        if (packed) packed[(int64_t)l * a.kcap + at] = (__float_as_uint(B == 4 ? 2.f * v[l] : v[l]) >> 16) | place;
-                }
-                atomicOr(&map[p[q] >> 5], 1u << (p[q] & 31));
-            }
-            run_gt += __popc(mg);
-            run_eq += __popc(me);
-        }
+        if (n_out) tile = (int)(s_pos[warp][n_out - 1] >> tile_shift);
+        __syncwarp();
     }
-    __syncwarp();
-    // K: the bit map of the kept positions (whole chunks: the map is padded like the candidate lists)
-    if (a.keep && !(ut % a.tensors)) {
+    // K: whole chunks (the map is padded like the candidate lists)
+    if (map_k) {
         uint32_t* const keep = a.keep + (int64_t)(ut / a.tensors) * a.keep_stride + e0 / 32;
         for (int w = lane; w < WORDS; w += 32) keep[w] = map[w];
     }
-    // tile offsets
-    const int tile_e = kResTile * a.d, tile_words = tile_e / 32;
-    const int tiles = (int)((min((int64_t)CE, n_e - e0) + tile_e - 1) / tile_e);
-    int32_t* const off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1) + (int)(e0 / tile_e);
-    uint32_t at = first;
-    for (int j = 0; j < tiles; ++j) {
-        uint32_t s = 0;
-        for (int w = lane; w < tile_words; w += 32) s += __popc(map[j * tile_words + w]);
-#pragma unroll
-        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        if (lane == 0) off[j] = (int32_t)at;
-        at += s;
-    }
+    // tiles behind the last entry
+    const int tiles = (int)((min((int64_t)CE, n_e - e0) + (1 << tile_shift) - 1) >> tile_shift);
+    const uint32_t end = run_gt + min(run_eq, need);
+    for (int x = tile + 1 + lane; x < tiles; x += 32) off[x] = (int32_t)end;
     if (lane == 0 && c == a.chunks - 1) {
-        off[tiles] = (int32_t)at;
-        if ((int64_t)at != a.n_keep) atomicMax(a.status, (int32_t)kFlagCountMismatch);
+        off[tiles] = (int32_t)end;
+        if ((int64_t)end != a.n_keep) atomicMax(a.status, (int32_t)kFlagCountMismatch);
     }
 }
 
