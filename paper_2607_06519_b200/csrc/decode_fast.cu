@@ -73,7 +73,7 @@ static_assert(kMaxSplits < 256 && kMaxSplits % 32 == 0, "part counts are bytes; 
 // and its list ranges one round trip earlier.  A block that becomes resident only when one of the call before ends, as the last
 // cluster of eight does while seven fit beside those that run, was the one everybody waited for.  (With the other savings of a call of
 // one or two tiles, 1 024 tokens and a tail: 8.4 -> 7.7 us.)
-constexpr int kHeadUnits = 8;
+constexpr int kHeadUnits = 8;  // (0.8 KiB; a KiB of parameters takes 0.14 us to issue)
 struct UnitHeads {
     UnitDesc u[kHeadUnits];
     int n;  // 0: read them from memory

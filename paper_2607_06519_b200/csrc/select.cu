@@ -865,7 +865,7 @@ __device__ __forceinline__ uint32_t packed_place(uint32_t p) {
 // of their counts, then positions and values of those that stay go through shared memory, so that the lists leave in runs.
 // Bound by the latency of a chunk's chain (loads, scan, both ways through shared memory) beside 2 GB of lists and candidates: 32 layers of 32k
 // tokens 300 -> 266 us, 8 blocks of four of 12 289 147 -> 130, against 32 candidates a round with two votes each.  (One chunk per block with
-// a block scan per round took 767; 6 or 8 blocks an SM by fewer registers 312 and 325.)
+// a block scan per round took 767.)
 template <typename T, int B, bool ALL>
 __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_begin) {
     constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
