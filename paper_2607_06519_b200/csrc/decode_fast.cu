@@ -581,8 +581,8 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             const int unit_kr = (int)((reinterpret_cast<uint64_t>(ud.k_rows) - arena) >> (F8 ? 7 : 8));
             const int unit_vr = (int)((reinterpret_cast<uint64_t>(ud.v_rows) - arena) >> (F8 ? 7 : 8));
             auto release_here = [&](int s, int j) {
+                __syncwarp();  // (also between what a lane has cleared in the scratch and what the others write there next)
                 if (CL && it + j + kStages >= seg_info[1]) return;  // (nothing follows in this stage)
-                __syncwarp();
                 if (lane == 0) {
                     // (atomicInc wraps the counter back to zero at the eighth arrival; tile j + kStages reuses stage s)
                     const unsigned old = atomicInc(reinterpret_cast<unsigned*>(stage_cnt) + s, kCW - 1);

@@ -6,6 +6,7 @@ import torch
 
 from gpu_util import TOL, f32, oracle_unit, vector_errors
 from oracle import fdkv_ref_fp8 as R8
+from paper_2607_06519_b200 import binding as B
 from paper_2607_06519_b200 import runner, synth
 
 pytestmark = pytest.mark.gpu
@@ -62,5 +63,40 @@ def test_whole_tiles(hkv, T, tail, rows):
                 u.append(layer, f32(kn)[0, h], f32(vn)[0, h])
             ref = u.attend(int(modes[0, h]), layer, f32(q)[0][h * 2:(h + 1) * 2])
             assert vector_errors(f32(out)[0][h * 2:(h + 1) * 2], ref).max() <= TOL["bf16"], (layer, h)
+    assert pf.ctx.device_status() == 0
+    pf.ctx.close()
+
+
+@pytest.mark.parametrize("rows", [0, 1])
+@pytest.mark.parametrize("rule", [0, 1])
+@pytest.mark.parametrize("hkv,T,tail", [(2, 256, 0), (2, 2048, 0), (2, 2048, 2), (32, 2000, 0), (32, 2000, 2), (30, 2800, 0)])
+def test_full_scratch_behind_the_last_tiles(hkv, T, tail, rule, rows):
+    """Every position kept, one to three tiles a block: the last ones fill all of the scratch that the next tile's entries, the state put
+    aside before a tail and the merge are written over.  The same bits from every call, within the tolerance of the oracle's."""
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=hkv, n_q_heads=hkv, T=T, n_needles=1, W=1, n_steps=max(tail, 1), row_format=rows,
+                                            residual_rule=rule, keep_num=1, keep_den=1, name="full_scratch")
+    pf = runner.Prefilled(w, max_tail=max(tail, 1))
+    pf.prefill(0, np.ones((1, hkv), np.int64))
+    for layer in range(2):
+        for step in range(tail):
+            pf.ctx.decode_attn(layer, pf.decode_q(layer, step), *pf.new_rows(layer, step))
+        q = pf.decode_q(layer, 0)
+        launches = B.launch_count()
+        first = pf.ctx.decode_attn(layer, q).clone()
+        assert B.launch_count() == launches + 1  # (clusters: no kernel that joins)
+        for _ in range(10):
+            assert torch.equal(pf.ctx.decode_attn(layer, q), first)
+        for h in (0, hkv - 1):
+            if rows:
+                u = R8.UnitFp8(*synth.unit_tensor(w, 0, 0, h, False), *synth.unit_tensor(w, 0, 0, h, True), True, 1, 1)
+            else:
+                u = oracle_unit(w, 0, 0, h)
+            if rule:
+                u.use_tokens(np.arange(T))
+            for step in range(tail):
+                kn, vn = pf.new_rows(layer, step)
+                u.append(layer, f32(kn)[0, h], f32(vn)[0, h])
+            ref = u.attend(1, layer, f32(q)[0][h:h + 1])
+            assert vector_errors(f32(first)[0][h:h + 1], ref).max() <= TOL["bf16"], (layer, h)
     assert pf.ctx.device_status() == 0
     pf.ctx.close()
