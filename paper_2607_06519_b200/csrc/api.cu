@@ -839,7 +839,6 @@ static fdkv_status decode_impl(fdkv_ctx* c, int32_t layer, int32_t batch, const 
     a.packed_lists = c->packed_lists ? 1 : 0;
     a.tok_rule = s.tok_rule;
     a.desc = arp<UnitDesc>(c, c->ar.desc);
-    a.host_desc = c->desc_host.data();
     a.L = s.L; a.layer = layer; a.batch = batch; a.Hq = s.Hq; a.Hkv = s.Hkv; a.G = s.G; a.d = s.d;
     a.max_tail = s.max_tail; a.max_batch = s.max_batch; a.Tmax_batch = Tmax;
     a.q = q; a.k_new = k_new; a.v_new = v_new; a.out = out; a.out_dtype = out_dtype;

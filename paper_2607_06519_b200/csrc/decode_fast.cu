@@ -25,7 +25,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <type_traits>
 
 #include "fdkv_internal.h"
 #include "mbar_wait.cuh"
@@ -68,17 +67,6 @@ struct TailLens {
     int32_t n[NB];  // generated tokens in this layer's tail per sequence, this call's append included (host mirror)
 };
 static_assert(kMaxSplits < 256 && kMaxSplits % 32 == 0, "part counts are bytes; the combine holds one part per lane and round");
-
-// The descriptors of a launch of few units travel in its parameters (clusters only): the copies of a block then start with the block,
-// and its list ranges one round trip earlier.  A block that becomes resident only when one of the call before ends, as the last
-// cluster of eight does while seven fit beside those that run, was the one everybody waited for.  (With the other savings of a call of
-// one or two tiles, 1 024 tokens and a tail: 8.4 -> 7.7 us.)
-constexpr int kHeadUnits = 8;  // (0.8 KiB; a KiB of parameters takes 0.14 us to issue)
-struct UnitHeads {
-    UnitDesc u[kHeadUnits];
-    int n;  // 0: read them from memory
-};
-struct NoHeads {};
 
 // header offsets
 constexpr int kOffFull = 0, kOffJoint = 64, kOffAbort = 128, kOffM = 256, kOffL = 512, kOffSeg = 1024, kOffSegInfo = 1920,
@@ -197,7 +185,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 template <bool F8, bool CL, int NB, bool SPLIT>
 __global__ void __maxnreg__(232)
 decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap8, DecodeArgs a, FastSched sch,
-                   TailLens<NB> tl, const __grid_constant__ std::conditional_t<CL, UnitHeads, NoHeads> heads) {
+                   TailLens<NB> tl) {
     constexpr int kStages = CL || F8 ? 2 : 3, kScratchBytes = scratch_of(F8, CL);
     // Clusters: the entries of K and of V have a tile each, filled before the tile is worked on (of the first one before the dependency
     // wait), so that neither their stores nor the clearing between lie in the chain from q to the outputs (1 024 tokens and a tail 7.3 -> 6.9 us).
@@ -291,8 +279,6 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         for (int u = u_first; u <= u_last && u < sch.units; ++u) {
             const int b = u / a.Hkv, h = u % a.Hkv;
             const UnitDesc* ud = a.desc + ((int64_t)b * a.L + a.layer) * a.Hkv + h;
-            if constexpr (CL)
-                if (heads.n) ud = heads.u + u;
             const int nsl = (ud->T + kResTile - 1) / kResTile;
             const int sb = u == u_first ? t_first : 0;
             const int se = u == u_last ? t_last : nsl;
@@ -355,10 +341,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         int it = 0;
         for (int u = u_first; u <= u_last && u < sch.units; ++u) {
             const int b = u / a.Hkv, h = u % a.Hkv;
-            const UnitDesc* udp = a.desc + ((int64_t)b * a.L + a.layer) * a.Hkv + h;
-            if constexpr (CL)
-                if (heads.n) udp = heads.u + u;
-            const UnitDesc ud = *udp;
+            const UnitDesc ud = a.desc[((int64_t)b * a.L + a.layer) * a.Hkv + h];
             const int T = ud.T;
             const int nres = (T + kResTile - 1) / kResTile;
             const int sb = u == u_first ? t_first : 0;
@@ -1185,30 +1168,24 @@ cudaError_t launch_decode_fast(const DecodeArgs& a, cudaStream_t st, bool* handl
     cfg.numAttrs = sch.cluster ? 2 : 1;
     const CUtensorMap& m16 = *reinterpret_cast<const CUtensorMap*>(a.tmap);
     const CUtensorMap& m8 = *reinterpret_cast<const CUtensorMap*>(a.rows_f8 ? a.tmap_u8 : a.tmap);
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;  // (a captured call reads the descriptors that are there when it is replayed)
-    if (sch.cluster && (e0 = cudaStreamIsCapturing(st, &capture)) != cudaSuccess) return e0;
-    auto launch = [&](auto* kernel, auto tl, auto heads) {
+    auto launch = [&](auto* kernel, auto tl) {
         for (int b = 0; b < a.batch; ++b) tl.n[b] = a.host_tail[b];
-        if constexpr (std::is_same_v<decltype(heads), UnitHeads>) {
-            heads.n = units <= kHeadUnits && capture == cudaStreamCaptureStatusNone ? units : 0;
-            for (int u = 0; u < heads.n; ++u) heads.u[u] = a.host_desc[((int64_t)(u / a.Hkv) * a.L + a.layer) * a.Hkv + u % a.Hkv];
-        }
-        return cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, tl, heads);
+        return cudaLaunchKernelEx(&cfg, kernel, m16, m8, a, sch, tl);
     };
     cudaError_t e;
     const bool split = a.G <= 4;  // (8-bit rows take no more)
     if (sch.cluster)
         e = launch(a.rows_f8 ? decode_fast_kernel<true, true, kFewSeqs, true>
                    : split   ? decode_fast_kernel<false, true, kFewSeqs, true>
-                             : decode_fast_kernel<false, true, kFewSeqs, false>, TailLens<kFewSeqs>(), UnitHeads());
+                             : decode_fast_kernel<false, true, kFewSeqs, false>, TailLens<kFewSeqs>());
     else if (a.batch <= kFewSeqs)
         e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kFewSeqs, true>
                    : split   ? decode_fast_kernel<false, false, kFewSeqs, true>
-                             : decode_fast_kernel<false, false, kFewSeqs, false>, TailLens<kFewSeqs>(), NoHeads());
+                             : decode_fast_kernel<false, false, kFewSeqs, false>, TailLens<kFewSeqs>());
     else
         e = launch(a.rows_f8 ? decode_fast_kernel<true, false, kMaxUnits, true>
                    : split   ? decode_fast_kernel<false, false, kMaxUnits, true>
-                             : decode_fast_kernel<false, false, kMaxUnits, false>, TailLens<kMaxUnits>(), NoHeads());
+                             : decode_fast_kernel<false, false, kMaxUnits, false>, TailLens<kMaxUnits>());
     if (e != cudaSuccess) return e;
     count_launch(1);
     count_kernel(FDKV_KERNEL_DECODE_FAST);

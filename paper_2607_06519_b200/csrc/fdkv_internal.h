@@ -282,7 +282,6 @@ struct DecodeArgs {
     const int32_t* host_T;      // [batch]
     const int32_t* host_modes;  // [batch][Hkv] modes of this layer's pair
     const int32_t* host_tail;   // [batch] generated tokens in this layer's tail per sequence (after this call's append), or null
-    const UnitDesc* host_desc;  // the host's copy of desc, or null (planning without a context)
     FastPlan* plan;             // the layer's kept schedule, or null (planning without a context)
     uint64_t plan_epoch;
     int any_tail;               // some sequence of the batch has generated tokens in this layer's tail (after this call's append)

@@ -1,5 +1,5 @@
 """Captured decode calls of short contexts: a replay reads the descriptors that the device holds then, so it serves a later prompt of the
-same length with other modes too; few units, whose descriptors travel in the parameters of a call on a stream, and more."""
+same length with other modes too; few units and more."""
 import pytest
 import torch
 
