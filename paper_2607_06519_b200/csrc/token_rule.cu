@@ -52,6 +52,9 @@ struct ScorePlan {
 // each (64 rows: two, a half).  Bound by the hand-overs between copies, MMAs (1 024 cycles a tile of 128 x 256 x 128) and epilogue: 8 191 tokens, 8
 // blocks of four, 8 heads, 256 rows a layer: four epilogue warps, and a block per item and third of its tiles, each with its own probe
 // rows, the last of six waves a fifth full, 214 us; eight warps 165; sixteen 159 (117 without an epilogue).
+// Tiles that some query does not see take a comparison per column, with the query that the column is for and the token's first one (probe call of
+// 8 191 tokens, 8 layers in blocks of four, 64 positions all over the prompt: 135 us; with a division and a load per column 363; the last 64
+// positions 98).
 template <int NT>
 __global__ void __launch_bounds__(kTThreads, 1)
 token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScorePlan pl) {
@@ -171,9 +174,23 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
         items([&](int, int unit, int layer, int mblock, int t0, int n, int i0) {
             float* const err = a.err + ((int64_t)unit * a.nslots + layer * pl.mblocks + mblock) * a.Tmax;
             uint32_t* const score = a.score + (int64_t)unit * a.Tmax;
+            const int row0 = mblock * NT + part * kPart;  // probe row of the warp's first column
             for (int i = i0; i < i0 + n; ++i) {
                 const int as = i & 1, tile_t0 = (t0 + i - i0) * kTM;
                 const int t = tile_t0 + lq * 32 + lane;
+                // First query that sees the token: the positions ascend, so it is the number of those before it.  All of them are looked at,
+                // four a lane: those before the warp's 32 tokens are counted, those among them set a bit.
+                int q_seen = 0;
+                if (tile_t0 + kTM - 1 > pl.pos_min) {
+                    uint32_t inside = 0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int rel = 32 * k + lane < a.W ? a.pos[32 * k + lane] - (t - lane) : 32;
+                        q_seen += __popc(__ballot_sync(0xFFFFFFFFu, rel < 0));
+                        if (rel >= 0 && rel < 32) inside |= 1u << rel;
+                    }
+                    q_seen += __popc(__reduce_or_sync(0xFFFFFFFFu, inside) & ((1u << lane) - 1u));
+                }
                 mb_wait(sm0 + tTFull + 8 * as, ((uint32_t)i >> 1) & 1u, abort_flag, a.status);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 float m0 = 0.f, m1 = 0.f, e0 = 0.f, e1 = 0.f;
@@ -202,13 +219,17 @@ token_score_kernel(const __grid_constant__ CUtensorMap tmap, TokenArgs a, ScoreP
                                 e1 = fmaf(x, x, e1);
                             }
                     } else {
+                        int q = row0 % a.W;  // (the columns go through the queries, head after head)
 #pragma unroll
                         for (int p = 0; p < kPart / 32; ++p)
 #pragma unroll
                             for (int j = 0; j < 32; ++j) {
-                                const int row = mblock * NT + part * kPart + 32 * p + j;
                                 const float u = __uint_as_float(r[p][j]);
-                                if (row < rows_layer && a.pos[row % a.W] >= t) { m0 = fmaxf(m0, fabsf(u)); e0 = fmaf(u, u, e0); }
+                                if (q >= q_seen && row0 + 32 * p + j < rows_layer) {
+                                    if (j & 2) m1 = fmaxf(m1, fabsf(u)); else m0 = fmaxf(m0, fabsf(u));
+                                    if (j & 1) e1 = fmaf(u, u, e1); else e0 = fmaf(u, u, e0);
+                                }
+                                q = q + 1 == a.W ? 0 : q + 1;
                             }
                     }
                     const float m = fmaxf(m0, m1);

@@ -178,3 +178,41 @@ def test_probe_rows_of_the_score_kernel(group, W, T, hkv):
         u.use_tokens(tok.cpu().numpy())
         np.testing.assert_allclose(scores[p, h], R.probe_error(u.z1["k"], u.kept["k"], pq[0], pq[1], group, h, synth.probe_positions(w)), rtol=2e-5, atol=1e-9)
     assert pf.ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("block", [2, 4])
+@pytest.mark.parametrize("group,W,T", [(1, 40, 700), (2, 33, 1025), (4, 64, 2048), (4, 128, 1000), (8, 64, 900), (1, 1, 300)])
+@pytest.mark.parametrize("where", ["ends", "spread", "random"])
+def test_positions_with_gaps(where, group, W, T, block):
+    """Probe queries all over the prompt: tokens of nearly every tile that some queries see and others do not, positions at both ends of a
+    warp's 32 tokens, heads whose columns start in the middle of a warp's (tolerances as above)."""
+    from oracle import fdkv_ref_b4 as R4
+    from paper_2607_06519_b200 import runner
+
+    w = synth.WORKLOADS["decode32k"].scaled(n_layers=2 * block, n_kv_heads=2, n_q_heads=2 * group, T=T, n_needles=2, W=W, residual_rule=1, block_size=block,
+                                            name="gaps")
+    pos = {"ends": np.concatenate([np.arange((W + 1) // 2), np.arange(T - W // 2, T)]),
+           "spread": np.linspace(T - 1 if W == 1 else 0, T - 1, W).astype(np.int64),
+           "random": np.sort(np.random.default_rng(W).choice(T, W, replace=False))}[where].astype(np.int32)
+    pf = runner.Prefilled(w)
+    pf.compress(0)
+    _, scores = pf.ctx.probe(0, 0, 2, pf.upload_probe_q(0), pos, 0.0)
+    scores = scores.cpu().numpy().astype(np.float64)
+    for p, h in ((0, 0), (1, 1)):
+        pq = [synth.probe_q(w, 0, block * p + l) for l in range(block)]
+        tok, sc = pf.ctx.get_token_set(0, p, h, T)
+        tok = tok.cpu().numpy()
+        if block == 4:
+            u = R4.Unit4(synth.block_tensor(w, 0, p, h, False), synth.block_tensor(w, 0, p, h, True), True, w.keep_num, w.keep_den, select=False)
+            s_ref = R4.token_scores4(u.dev["k"], pq, group, h, pos)
+            u.use_tokens(tok)
+            e = R4.probe_error4(u.dev["k"], u.kept["k"], pq, group, h, pos)
+        else:
+            u = _unit(w, p, h)
+            s_ref = R.token_scores(u.z1["k"], pq[0], pq[1], group, h, pos)
+            u.use_tokens(tok)
+            e = R.probe_error(u.z1["k"], u.kept["k"], pq[0], pq[1], group, h, pos)
+        np.testing.assert_allclose(f32(sc).astype(np.float64), s_ref, rtol=1e-5, atol=1e-6 * max(1.0, s_ref.max()))
+        np.testing.assert_allclose(scores[p, h], e, rtol=2e-5, atol=1e-9)
+    assert pf.ctx.device_status() == 0
+    pf.ctx.close()
