@@ -1011,10 +1011,12 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     constexpr int CH = 4 * Q;                       // 16-byte chunks of 32 positions
     constexpr int MOST = W == 1 ? 8 : 16;           // blocks of a cluster
     extern __shared__ __align__(16) uint8_t smem[];  // [NB][range] values, the chunks of a word of 32 positions swizzled
-    // histograms: of the key's top 15 bits in a window (two counts of 16 bits a word), of two digits after it; the low halves of the keys that
-    // share the threshold's top half
-    __shared__ __align__(16) uint32_t s_h1[2048], s_h2[TWO ? 4 : 2048], s_all[4096];
-    __shared__ uint16_t s_near[TWO ? 4 : kSmallNear];
+    // Histogram of the key's top 15 bits in a window (two counts of 16 bits a word), its sums over the cluster.  When the threshold's top half is
+    // known the sums are done with: their place holds this block's keys with that top half, and then the cluster's, or the digits'
+    // histograms.  (With arrays of their own blocks of four at 513 to 640 tokens had one block on an SM instead of two: 16 heads 36.9 -> 48.9 us.)
+    __shared__ __align__(16) uint32_t s_h1[2048], s_all[4096];
+    uint16_t* const s_near = reinterpret_cast<uint16_t*>(s_all + 3072);  // [kSmallNear]
+    static_assert(sizeof(s_h1) + sizeof(s_all) + 1024 + 88 * 1024 + 1024 <= 228 * 1024 / 2, "two blocks fit an SM with 88 KiB of values each");
     __shared__ uint32_t s_count, s_warp[kSmallThreads / 32], s_before[2][kSmallThreads / 32], s_n, s_off[17], s_low[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x % blocks, item = blockIdx.x / blocks, uts = a.Hkv * a.tensors;
@@ -1022,10 +1024,7 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     const int n_e = a.T * a.d, e0 = rank * range, n = max(0, min(range, n_e - e0));
     const int dshift = a.d == 128 ? 7 : 6;
     const int plane = range * (int)sizeof(T);
-    for (int i = tid; i < 2048; i += kSmallThreads) {
-        s_h1[i] = 0;
-        if (!TWO) s_h2[i] = 0;
-    }
+    for (int i = tid; i < 2048; i += kSmallThreads) s_h1[i] = 0;
     if (tid == 0) s_n = 0;
     // a key's bin: 4 095 values of its top 15 bits from `from` up, 32 octaves, the last bin for what is larger.  At first 2^-24 to 2^8, of
     // energies 2^-16 to 2^16.
@@ -1216,17 +1215,19 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
                 }
             } else {  // many equal keys: digits of 10 and 6 bits
                 tau = top;
+                for (int i = tid; i < 2048; i += kSmallThreads) s_all[i] = 0;
+                __syncthreads();
                 auto level = [&](uint32_t* hist, int shift, int bits) {
                     each([&](int, int, uint32_t key) { if (key >> (shift + bits) == tau) atomicAdd(&hist[key >> shift & ((1u << bits) - 1u)], 1u); });
                     cluster_sync();
-                    *reinterpret_cast<uint2*>(&s_all[2 * tid]) = cluster_sum2<MOST>((uint32_t)__cvta_generic_to_shared(hist) + 8 * tid, blocks);
+                    *reinterpret_cast<uint2*>(&s_all[2048 + 2 * tid]) = cluster_sum2<MOST>((uint32_t)__cvta_generic_to_shared(hist) + 8 * tid, blocks);
                     __syncthreads();
-                    find_bin<kSmallThreads, 1024>(s_all, left, bin, above);
+                    find_bin<kSmallThreads, 1024>(s_all + 2048, left, bin, above);
                     left -= above;
                     tau = tau << bits | bin;
                 };
-                level(s_h2, 6, 10);
-                level(s_h2 + 1024, 0, 6);
+                level(s_all, 6, 10);
+                level(s_all + 1024, 0, 6);
                 need = left;  // of the positions whose key is tau, the lowest
             }
         }
