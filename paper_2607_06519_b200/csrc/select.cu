@@ -1013,7 +1013,8 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     extern __shared__ __align__(16) uint8_t smem[];  // [NB][range] values, the chunks of a word of 32 positions swizzled
     // Histogram of the key's top 15 bits in a window (two counts of 16 bits a word), its sums over the cluster.  When the threshold's top half is
     // known the sums are done with: their place holds this block's keys with that top half, and then the cluster's, or the digits'
-    // histograms.  (With arrays of their own blocks of four at 513 to 640 tokens had one block on an SM instead of two: 16 heads 36.9 -> 48.9 us.)
+    // histograms.  (With arrays of their own blocks of four at 513 to 640 tokens had one block on an SM instead of two: 4 layers of 640
+    // tokens, 16 heads 49.0 us against 29.8, 8 heads 33.8 against 25.5.)
     __shared__ __align__(16) uint32_t s_h1[2048], s_all[4096];
     uint16_t* const s_near = reinterpret_cast<uint16_t*>(s_all + 3072);  // [kSmallNear]
     static_assert(sizeof(s_h1) + sizeof(s_all) + 1024 + 88 * 1024 + 1024 <= 228 * 1024 / 2, "two blocks fit an SM with 88 KiB of values each");
