@@ -1002,6 +1002,9 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 // of blocks of four, 1000 x 128, two turns, 66 us against 64; 256 pairs of 1024 x 128, seven turns, 195 against 133.
 // W: words of 32 positions per thread.
 constexpr int kSmallNear = 1024;  // keys that are gathered at most
+// Of them are compared each with all others; digits among more.  (All compared, up to 1 024: 4096 x 128 float32 at keep 1/2 109.9 us, now 48.7;
+// 1000 x 128 at keep 1/4, some 160 keys, 23.3 and 19.9.)
+constexpr int kSmallRank = 128;
 constexpr int kSmallThreads = 512, kSmallElems = 32 * kSmallThreads, kSmallSmem = 128 * 1024;
 
 template <typename T, int B, int W>
@@ -1148,34 +1151,32 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
             if (8 * tid + i == (int)bin) eq_before += of_before[i];
         }
         if constexpr (!TWO) {
-            // The few keys with that top half (a 128th of an octave) are gathered, and every block ranks all of them: one more exchange instead of
-            // two digits and the counts.  float32 pairs, us: 509 x 128 15.7 -> 13.8, 2048 x 128 31.5 -> 26.5.
-            const uint32_t top = from + bin;
+            // The few keys with that top half (a 128th of an octave) are gathered, and every block looks through all of them: one more exchange
+            // instead of two digits and the counts.  float32 pairs, us: 509 x 128 15.7 -> 13.8, 2048 x 128 31.5 -> 26.5.  Where many share it
+            // (equal keys) the digits are counted by the cluster at once.
+            const uint32_t top = from + bin, m = s_all[bin];
             uint32_t left = need;
             eq_before = 0;
-            each([&](int, int, uint32_t key) {
-                if (key >> 16 == top) {
-                    const uint32_t i = atomicAdd(&s_n, 1u);
-                    if (i < (uint32_t)kSmallNear) s_near[i] = (uint16_t)key;
-                }
-            });
-            cluster_sync();
-            uint32_t mine_n = 0;
-            {
-                uint32_t at;
-                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_n)), "r"(lane < blocks ? lane : 0));
-                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(mine_n) : "r"(at) : "memory");
-                if (lane >= blocks) mine_n = 0;
-            }
-            uint32_t off_n = mine_n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, off_n, o);
-                if (lane >= o) off_n += y;
-            }
-            const uint32_t m = __shfl_sync(0xFFFFFFFFu, off_n, 31);
-            counted = m <= (uint32_t)kSmallNear;
+            counted = m <= (uint32_t)kSmallNear;  // (the cluster's count: the same for all of its blocks)
+            __syncthreads();                      // (the sums are read)
             if (counted) {
+                each([&](int, int, uint32_t key) {
+                    if (key >> 16 == top) s_near[atomicAdd(&s_n, 1u)] = (uint16_t)key;
+                });
+                cluster_sync();
+                uint32_t mine_n = 0;
+                {
+                    uint32_t at;
+                    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_n)), "r"(lane < blocks ? lane : 0));
+                    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(mine_n) : "r"(at) : "memory");
+                    if (lane >= blocks) mine_n = 0;
+                }
+                uint32_t off_n = mine_n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, off_n, o);
+                    if (lane >= o) off_n += y;
+                }
                 if (warp == 0 && lane < 17) s_off[lane] = off_n - mine_n;  // ([blocks, 16]: all of them)
                 __syncthreads();
                 for (uint32_t i = tid; i < m; i += kSmallThreads) {
@@ -1189,32 +1190,51 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
                     s_all[i] = (uint32_t)low | (uint32_t)r << 16;
                 }
                 __syncthreads();
-                for (uint32_t i = tid; i < m; i += kSmallThreads) {
-                    const uint32_t low = s_all[i] & 0xFFFFu;
-                    uint32_t g = 0, e = 0;
+                uint32_t low = 0;
+                if (m <= (uint32_t)kSmallRank) {  // each against all others
+                    for (uint32_t i = tid; i < m; i += kSmallThreads) {
+                        const uint32_t one = s_all[i] & 0xFFFFu;
+                        uint32_t g = 0, e = 0;
 #pragma unroll 2
-                    for (uint32_t k = 0; k < m; k += 4) {
-                        const uint4 v = *reinterpret_cast<const uint4*>(&s_all[k]);
-                        const uint32_t other[4] = {v.x & 0xFFFFu, v.y & 0xFFFFu, v.z & 0xFFFFu, v.w & 0xFFFFu};
+                        for (uint32_t k = 0; k < m; k += 4) {
+                            const uint4 v = *reinterpret_cast<const uint4*>(&s_all[k]);
+                            const uint32_t other[4] = {v.x & 0xFFFFu, v.y & 0xFFFFu, v.z & 0xFFFFu, v.w & 0xFFFFu};
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            g += k + q < m && other[q] > low;
-                            e += k + q < m && other[q] == low;
+                            for (int q = 0; q < 4; ++q) {
+                                g += k + q < m && other[q] > one;
+                                e += k + q < m && other[q] == one;
+                            }
                         }
+                        if (g < left && left <= g + e) { s_low[0] = one; s_low[1] = g; }
                     }
-                    if (g < left && left <= g + e) { s_low[0] = low; s_low[1] = g; }
+                    __syncthreads();
+                    low = s_low[0];
+                    left -= s_low[1];
+                } else {  // digits of 10 and 6 bits among them
+#pragma unroll 1
+                    for (int shift = 6; shift >= 0; shift -= 6) {
+                        for (int i = tid; i < 1024; i += kSmallThreads) s_all[2048 + i] = 0;
+                        __syncthreads();
+                        for (uint32_t i = tid; i < m; i += kSmallThreads) {
+                            const uint32_t one = s_all[i] & 0xFFFFu;
+                            if (shift || one >> 6 == low) atomicAdd(&s_all[2048 + (shift ? one >> 6 : one & 63u)], 1u);
+                        }
+                        __syncthreads();
+                        find_bin<kSmallThreads, 1024>(s_all + 2048, left, bin, above);
+                        low = low << 6 | bin;
+                        left -= above;
+                    }
                 }
-                __syncthreads();
-                tau = top << 16 | s_low[0];
-                need = left - s_low[1];
+                tau = top << 16 | low;
+                need = left;
                 for (uint32_t i = tid; i < m; i += kSmallThreads) {
-                    const uint32_t low = s_all[i] & 0xFFFFu;
+                    const uint32_t one = s_all[i] & 0xFFFFu;
                     if ((int)(s_all[i] >> 16) < rank) {
-                        gt_before += low > s_low[0];
-                        eq_before += low == s_low[0];
+                        gt_before += one > low;
+                        eq_before += one == low;
                     }
                 }
-            } else {  // many equal keys: digits of 10 and 6 bits
+            } else {  // digits of 10 and 6 bits
                 tau = top;
                 for (int i = tid; i < 2048; i += kSmallThreads) s_all[i] = 0;
                 __syncthreads();

@@ -126,3 +126,29 @@ def test_ties_over_sixteen_blocks(dtype, keep):
     want = R.select_entries(z1, k)
     assert np.array_equal(idx[:k].cpu().numpy(), want)
     assert np.array_equal(val[:k].float().cpu().numpy(), z1.ravel()[want])
+
+
+@pytest.mark.parametrize("T", [40, 500, 2100])
+@pytest.mark.parametrize("near", [1, 127, 128, 129, 1023, 1024, 1025, 4000])
+@pytest.mark.parametrize("copies", [1, 3])
+def test_keys_that_share_the_top_half(copies, near, T):
+    """float32 keys of which exactly `near` share the threshold's upper 16 bits, each value `copies` times: ranked one by one, by digits
+    among those gathered, or by digits over the cluster; the threshold at the first, in the middle and at the last of them."""
+    d = 128
+    rng = np.random.default_rng(near)
+    x = (1 + rng.random(200_000) * 2.0**-7).astype(np.float32)
+    key = R.depth_split(x, np.zeros_like(x), False)[1].view(np.uint32)
+    x = np.unique(x[key >> 16 == key[0] >> 16])
+    band = np.tile(x[:-(-near // copies)], copies)[:near] * rng.choice([-1, 1], near).astype(np.float32)
+    x0 = np.where(rng.random(T * d) < 0.5, rng.uniform(2, 3, T * d), rng.uniform(0.1, 0.5, T * d)).astype(np.float32)
+    x0[rng.choice(T * d, near, replace=False)] = band
+    x0 = x0.reshape(T, d)
+    _, z1 = R.depth_split(x0, np.zeros_like(x0), False)
+    above = int((np.abs(x0) > 1.5).sum())
+    dev = torch.from_numpy(x0).cuda()
+    for k in sorted({above + 1, above + (near + 1) // 2, above + near}):
+        z0, idx, val = torch.empty_like(dev), torch.empty(k, dtype=torch.int32, device="cuda"), torch.empty(k, device="cuda")
+        assert B.compress_unit_noalloc(dev, torch.zeros_like(dev), k, T * d, z0, idx, val) == k
+        want = R.select_entries(z1, k)
+        assert np.array_equal(idx.cpu().numpy(), want)
+        assert np.array_equal(val.cpu().numpy(), z1.ravel()[want])
