@@ -152,3 +152,27 @@ def test_keys_that_share_the_top_half(copies, near, T):
         want = R.select_entries(z1, k)
         assert np.array_equal(idx.cpu().numpy(), want)
         assert np.array_equal(val.cpu().numpy(), z1.ravel()[want])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("T", [300, 2100])
+@pytest.mark.parametrize("tiny", [0.0, 2.0**-70, 2.0**-30])
+@pytest.mark.parametrize("keep", [(3, 10), (13, 20), (17, 20), (19, 20), (1, 1)])
+def test_threshold_at_zero(keep, tiny, T, dtype):
+    """A third of the keys normal, a third zero and a third zero or tiny, below the first window: the k-th among each of them, and zero
+    with keys between it and the window and without."""
+    d = 128
+    rng = np.random.default_rng(9)
+    diff = rng.standard_normal((T, d)).astype(np.float32)
+    part = rng.integers(0, 3, (T, d))
+    diff[part == 1] = 0
+    diff[part == 2] *= tiny
+    x0 = torch.from_numpy(diff).cuda().to(dtype)
+    x1 = torch.zeros_like(x0)
+    k = T * d * keep[0] // keep[1]
+    z0, idx, val = torch.empty_like(x0), torch.empty(k, dtype=torch.int32, device="cuda"), torch.empty(k, dtype=dtype, device="cuda")
+    assert B.compress_unit_noalloc(x0, x1, *keep, z0, idx, val) == k
+    _, z1 = R.depth_split(x0.float().cpu().numpy(), x1.float().cpu().numpy(), dtype == torch.bfloat16)
+    want = R.select_entries(z1, k)
+    assert np.array_equal(idx.cpu().numpy(), want)
+    assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want])
