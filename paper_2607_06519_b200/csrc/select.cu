@@ -526,7 +526,8 @@ __device__ __forceinline__ void scan_chunks(int2* base, int c_begin, int c_end, 
 // (32 octaves; the last bin counts what is larger, and in the unheard-of case that the k-th key is there the window moves
 // up): with 128 bins per octave the atomics hardly collide, and 16 KiB leave room for two blocks on an SM.  32-bit keys:
 // two more digits of 12 and 4 bits among the few keys that share the first, which the second pass gathers while it counts the larger
-// ones of every chunk (a pass per digit and one for the counts: 12 289 tokens, 128 tensors of blocks of four: 112 -> 76 us).
+// ones of every chunk (a pass per digit and one for the counts: 12 289 tokens, 128 tensors of blocks of four: 112 -> 76 us), where the first
+// one's histogram says that they fit.
 // bf16 magnitudes: the k-th is within half an octave of the bound, so a chunk's counts of the 63 keys from the bound up, kept in shared memory,
 // give both the threshold and the counts before every chunk in one pass (a second one for the counts: 512 tensors of 32k tokens, behind the split: 149 -> 88 us).
 // Where these don't hold the digits are counted one after the other.
@@ -630,7 +631,7 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
                 }
                 __syncthreads();
             }
-        uint32_t k_rem = (uint32_t)a.n_keep, prefix, above;
+        uint32_t k_rem = (uint32_t)a.n_keep, prefix, above, in_bin;
         for (uint32_t from = sel->lo >> 16;; from += kThrBins - 1) {
             for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
             __syncthreads();
@@ -642,12 +643,14 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
             uint32_t bin;
             find_bin<kThrThreads, kThrBins>(s_hist, k_rem, bin, above);
             prefix = from + bin;
+            in_bin = s_hist[bin];
+            __syncthreads();
             if (bin < kThrBins - 1 || from + kThrBins - 1 >= 32767) break;
         }
         k_rem -= above;
         if constexpr (F32KEY) {
-            const uint32_t top = prefix;
-            if (chunks <= 0x10000) {
+            const uint32_t top = prefix, near = in_bin;
+            if (chunks <= 0x10000 && near <= (uint32_t)kThrBins) {
                 // ---- larger keys of every chunk, and those that share the first digit: chunk and low half ----
                 int2* const base = a.chunk_base + (int64_t)ut * a.chunks_max;
                 if (tid == 0) s_near = 0;
@@ -658,45 +661,38 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
                     uint32_t gt = 0;
                     each_candidate<T, B>(a, ut, c, n, [&](uint32_t key) {
                         gt += key >> 16 > top ? 1u : 0u;
-                        if (key >> 16 == top) {
-                            const uint32_t i = atomicAdd(&s_near, 1u);
-                            if (i < (uint32_t)kThrBins) s_dyn[i] = (uint32_t)c << 16 | (key & 0xFFFFu);
-                        }
+                        if (key >> 16 == top) s_dyn[atomicAdd(&s_near, 1u)] = (uint32_t)c << 16 | (key & 0xFFFFu);
                     });
                     gt = __reduce_add_sync(0xFFFFFFFFu, gt);
                     if (lane == 0) base[c] = make_int2((int)gt, 0);
                     n = n_next;
                 }
                 __syncthreads();
-                const uint32_t near = s_near;
-                if (near <= (uint32_t)kThrBins) {
-                    uint32_t low = 0;
+                uint32_t low = 0;
 #pragma unroll 1
-                    for (int pass = 0; pass < 2; ++pass) {
-                        const int shift = pass == 0 ? 4 : 0, bits = pass == 0 ? 12 : 4;
-                        for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
-                        __syncthreads();
-                        for (uint32_t i = tid; i < near; i += kThrThreads) {
-                            const uint32_t key = s_dyn[i] & 0xFFFFu;
-                            if (pass == 0 || key >> 4 == low) atomicAdd(&s_hist[(key >> shift) & ((1u << bits) - 1u)], 1u);
-                        }
-                        __syncthreads();
-                        uint32_t bin;
-                        find_bin<kThrThreads, kThrBins>(s_hist, k_rem, bin, above);
-                        low = low << bits | bin;
-                        k_rem -= above;
-                    }
-                    if (tid == 0) { sel->tau = top << 16 | low; sel->need = k_rem; }
+                for (int pass = 0; pass < 2; ++pass) {
+                    const int shift = pass == 0 ? 4 : 0, bits = pass == 0 ? 12 : 4;
+                    for (int i = tid; i < kThrBins; i += kThrThreads) s_hist[i] = 0;
+                    __syncthreads();
                     for (uint32_t i = tid; i < near; i += kThrThreads) {
-                        const uint32_t c = s_dyn[i] >> 16, key = s_dyn[i] & 0xFFFFu;
-                        if (key > low) atomicAdd(&base[c].x, 1);
-                        else if (key == low) atomicAdd(&base[c].y, 1);
+                        const uint32_t key = s_dyn[i] & 0xFFFFu;
+                        if (pass == 0 || key >> 4 == low) atomicAdd(&s_hist[(key >> shift) & ((1u << bits) - 1u)], 1u);
                     }
                     __syncthreads();
-                    scan_chunks(base, 0, chunks, 0, 0, s_sum);
-                    return;
+                    uint32_t bin;
+                    find_bin<kThrThreads, kThrBins>(s_hist, k_rem, bin, above);
+                    low = low << bits | bin;
+                    k_rem -= above;
+                }
+                if (tid == 0) { sel->tau = top << 16 | low; sel->need = k_rem; }
+                for (uint32_t i = tid; i < near; i += kThrThreads) {
+                    const uint32_t c = s_dyn[i] >> 16, key = s_dyn[i] & 0xFFFFu;
+                    if (key > low) atomicAdd(&base[c].x, 1);
+                    else if (key == low) atomicAdd(&base[c].y, 1);
                 }
                 __syncthreads();
+                scan_chunks(base, 0, chunks, 0, 0, s_sum);
+                return;
             }
 #pragma unroll 1
             for (int pass = 0; pass < 2; ++pass) {

@@ -128,12 +128,13 @@ def test_ties_over_sixteen_blocks(dtype, keep):
     assert np.array_equal(val[:k].float().cpu().numpy(), z1.ravel()[want])
 
 
-@pytest.mark.parametrize("T", [40, 500, 2100])
-@pytest.mark.parametrize("near", [1, 127, 128, 129, 1023, 1024, 1025, 4000])
+@pytest.mark.parametrize("T,near", [(T, near) for T in (40, 500, 2100) for near in (1, 127, 128, 129, 1023, 1024, 1025, 4000)] +
+                         [(8000, near) for near in (1, 4095, 4096, 4097, 20000)])
 @pytest.mark.parametrize("copies", [1, 3])
-def test_keys_that_share_the_top_half(copies, near, T):
+def test_keys_that_share_the_top_half(copies, T, near):
     """float32 keys of which exactly `near` share the threshold's upper 16 bits, each value `copies` times: ranked one by one, by digits
-    among those gathered, or by digits over the cluster; the threshold at the first, in the middle and at the last of them."""
+    among those gathered, or by digits over the cluster, and (8000 tokens) gathered or counted over the chunks; the threshold at the
+    first, in the middle and at the last of them."""
     d = 128
     rng = np.random.default_rng(near)
     x = (1 + rng.random(200_000) * 2.0**-7).astype(np.float32)
