@@ -74,7 +74,7 @@ struct FastPlan {
 
 struct SelState {
     uint32_t lo;      // bound the candidates reach (31-bit key pattern; bf16 magnitudes are shifted left by 16)
-    uint32_t tau;     // threshold key: that of the k-th largest
+    uint32_t tau;     // threshold key: that of the k-th largest (until it is known: whether the sample puts it near the bound)
     uint32_t need;    // entries with key == tau to keep (lowest flat indices first)
     uint32_t redo;    // fewer than k positions reached the bound: split and threshold run again with bound 0
 };

@@ -228,7 +228,7 @@ __device__ __forceinline__ bool find_bin(const uint32_t* bins, uint32_t target, 
 // ---- 1: the bound -------------------------------------------------------------------------------------
 // grid (heads x tensors, blocks of the launch)
 template <typename T, int B>
-__global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, int n_rows, uint32_t target) {
+__global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, int n_rows, uint32_t target, uint32_t among) {
     __shared__ uint32_t s_hist[kSampleBins];
     constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q;
     const int tid = threadIdx.x;
@@ -273,6 +273,9 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(CompressArgs a, 
     if (tid == 0) {
         a.sel[ut].redo = 0;
         a.sel[ut].lo = a.n_keep == 0 ? kNoKey : enough ? bin << 19 : 0u;
+        // is the k-th among the 63 bf16 keys from the bound up: seven bins and seven eighths of one?
+        for (uint32_t i = 1; i < 7 && bin + i < (uint32_t)kSampleBins; ++i) above -= s_hist[bin + i];
+        a.sel[ut].tau = enough && 8 * above < 8 * among + (bin + 7 < (uint32_t)kSampleBins ? 7 * s_hist[bin + 7] : 0u);
     }
 }
 
@@ -528,10 +531,12 @@ __device__ __forceinline__ void scan_chunks(int2* base, int c_begin, int c_end, 
 // two more digits of 12 and 4 bits among the few keys that share the first, which the second pass gathers while it counts the larger
 // ones of every chunk (a pass per digit and one for the counts: 12 289 tokens, 128 tensors of blocks of four: 112 -> 76 us), where the first
 // one's histogram says that they fit.
-// bf16 magnitudes: the k-th is within half an octave of the bound, so a chunk's counts of the 63 keys from the bound up, kept in shared memory,
-// give both the threshold and the counts before every chunk in one pass (a second one for the counts: 512 tensors of 32k tokens, behind the split: 149 -> 88 us).
+// bf16 magnitudes: where the k-th is within half an octave of the bound, a chunk's counts of the 63 keys from the bound up, kept in shared memory,
+// give both the threshold and the counts before every chunk in one pass (a second one for the counts: 256 tensors of 32k tokens, behind the split:
+// 149 -> 88 us).  The sample says whether it is: with keep 1/3 and more of log-normal channel scales it is not, and a pass for nothing made 128
+// tensors of 8 192 tokens at keep 1/2 673 us instead of 622.
 // Where these don't hold the digits are counted one after the other.
-constexpr int kThrMini = 512;  // chunks whose counts fit beside another block's
+constexpr int kThrMini = 512;  // chunks whose counts are kept
 template <typename T, int B>
 __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, int ut_begin, int redo) {
     __shared__ __align__(16) uint32_t s_hist[kThrBins];
@@ -569,7 +574,7 @@ __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, 
             return;
         }
         if constexpr (!F32KEY)
-            if (chunks <= kThrMini) {
+            if (chunks <= kThrMini && !redo && sel->tau) {
                 uint32_t* const mini = s_hist + 64 * warp;
                 uint32_t* const total_of = s_hist + 64 * 32;
                 const uint32_t lo16 = sel->lo >> 16;
@@ -1448,6 +1453,7 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     const bool all = a.in_place || (double)a.n_keep > kAllShare * (double)n;
     // about 1.2 k candidates (and four standard deviations of a small sample on top); a sample of everything is exact
     const uint32_t target = exact ? (uint32_t)a.n_keep : (uint32_t)std::ceil(1.2 * expect + 4.0 * std::sqrt(expect) + 16.0);
+    const uint32_t among = (uint32_t)std::ceil(std::max(0.0, expect - 2.0 * std::sqrt(expect)));  // of the sample, at least, of the k largest
     // blocks per unit-tensor for the threshold: one per SM, where each has a chunk per warp or the candidates are all.  (Two per SM leave
     // clusters waiting: 32 tensors of 32k x 128, eight blocks each 316 us, four 277; keep 1/2 724 and 653.)
     // The joins cost about 5 us a digit: 64 lists of 98k entries 147 -> 136 us, of 65k 263 -> 278, one of 33k float32 entries 57 -> 67.
@@ -1465,7 +1471,7 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
                 a.v[l] = v_layers[B * b0 + l];
             }
             a.ut_base = b0 * uts;
-            if (!redo && (e = launch_chain(0, sample_kernel<T, B>, dim3(uts, nb), kSampleThreads, 0, st, a, n_rows, target)) != cudaSuccess) return e;
+            if (!redo && (e = launch_chain(0, sample_kernel<T, B>, dim3(uts, nb), kSampleThreads, 0, st, a, n_rows, target, among)) != cudaSuccess) return e;
             const int items = a.chunks * uts * nb;
             if ((e = launch_chain(0, all ? split_kernel<T, B, true> : split_kernel<T, B, false>, dim3(std::min(items, 3 * sms)), kSplitThreads, smem, st, a, items,
                                   redo)) != cudaSuccess)

@@ -157,9 +157,10 @@ def test_shared_coefficients_in_a_layers_place(dtype, T, keep, which):
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("values", ["normal", "few", "wide"])
 @pytest.mark.parametrize("hkv,T", [(12, 1501), (10, 4099)])
-def test_threshold_of_many_tensors(hkv, T, values, dtype):
+@pytest.mark.parametrize("den", [9, 2])
+def test_threshold_of_many_tensors(den, hkv, T, values, dtype):
     """A block per tensor: the k-th key among the 63 above the bound and far from it (values over forty octaves), and more keys that share
-    the first digit than are gathered (integers)."""
+    the first digit than are gathered (integers); with half of them kept the sample expects it far away more often."""
     from paper_2607_06519_b200 import binding as B
 
     d, tdt = 128, torch.bfloat16 if dtype == "bf16" else torch.float32
@@ -171,11 +172,11 @@ def test_threshold_of_many_tensors(hkv, T, values, dtype):
     elif values == "wide":
         base, diff = 0 * base, np.ldexp(diff, rng.integers(-20, 20, diff.shape)).astype(np.float32)
     x = [torch.from_numpy(a).to(tdt).cuda() for a in (base, base + diff)]
-    ctx = B.Context(B.Config(2, hkv, hkv, d, 1, T, 1, B.BF16 if dtype == "bf16" else B.F32, 1, 9))
+    ctx = B.Context(B.Config(2, hkv, hkv, d, 1, T, 1, B.BF16 if dtype == "bf16" else B.F32, 1, den))
     ctx.compress_prefill(0, 0, 1, T, x, x)
     for h in (0, hkv - 1):
         _, z1 = R.depth_split(x[0][:, h].float().cpu().numpy(), x[1][:, h].float().cpu().numpy(), dtype == "bf16")
-        want = R.select_entries(z1, T * d // 9)
+        want = R.select_entries(z1, T * d // den)
         idx, val = ctx.get_residual(0, 0, h, 1)
         assert np.array_equal(idx.cpu().numpy(), want)
         assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want])
