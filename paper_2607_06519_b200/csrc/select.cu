@@ -1037,6 +1037,7 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     const int n_e = a.T * a.d, e0 = rank * range, n = max(0, min(range, n_e - e0));
     const int dshift = a.d == 128 ? 7 : 6;
     const int plane = range * (int)sizeof(T);
+    const bool every = a.n_keep == n_e;  // all of them are kept: above zero or equal to it
     for (int i = tid; i < 2048; i += kSmallThreads) s_h1[i] = 0;
     if (tid == 0) s_n = 0;
     // a key's bin: 4 094 values of its top 15 bits above `from`, 32 octaves, the last bin for what is larger, the first for zero (rows that are
@@ -1083,7 +1084,7 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
                     *reinterpret_cast<uint4*>(smem + l * plane + chunk_at(p >> 5, ((p >> 3) & 3) * Q + k)) = hf[l][k];
                 }
             }
-            Eight<T, B>::keys(hf, [&](int, uint32_t key) { count_key(key); });
+            if (!every) Eight<T, B>::keys(hf, [&](int, uint32_t key) { count_key(key); });
         }
     }
     // f(w, i, key) for position i of the thread's word w, whose 32 positions are all there or none of them
@@ -1104,11 +1105,11 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
         }
     };
     // ---- the n_keep-th largest key of the cluster ----
-    uint32_t tau = kNoKey, need = 0;
-    uint32_t gt_before = 0, eq_before = 0;  // this thread's part of the counts of the blocks before this one
-    bool counted = true;                    // (the same for the whole cluster)
+    uint32_t tau = every ? 0u : kNoKey, need = every ? (uint32_t)n_e : 0u;
+    uint32_t gt_before = every && tid == 0 ? (uint32_t)e0 : 0u, eq_before = 0;  // this thread's part of the counts of the blocks before this one
+    bool counted = true;                                                        // (the same for the whole cluster)
     cluster_sync();
-    if (a.n_keep > 0) {  // (the same for every block)
+    if (a.n_keep > 0 && !every) {  // (the same for every block)
         // The blocks' histograms give the threshold's top half and, of the blocks before this one, how many keys are above it and equal to it:
         // for bf16 magnitudes one exchange in all.
         uint32_t bin, above, of_before[8];
@@ -1408,8 +1409,9 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     bool small = few && fits() && (int64_t)cluster * n_ut <= 2 * sms;
     // Longer ones take clusters of sixteen blocks, two or four words of positions per thread, while all of the clusters run at one
     // time (us, one tensor, keep 1/16, against the four kernels: bf16 192k positions 33.7 -> 16.1, 512k 39.9 -> 21.1; float32 256k 44.7 -> 31.5, 512k
-    // 55.9 -> 36.6).
-    if (few && !small && (int64_t)16 * n_ut <= 2 * sms && tiles >= 16) {
+    // 55.9 -> 36.6).  Where everything is kept a thread's entries are many and there is nothing to select: up to 384 Ki positions in all (one
+    // bf16 tensor of 384k 54.6 us, four kernels 66.6, 512k 84.6 and 66.8; float32 39.6 and 53.1, 66.0 and 63.1; eight bf16 tensors of 256k 103.9 and 91.5).
+    if (few && !small && (int64_t)16 * n_ut <= 2 * sms && tiles >= 16 && (a.n_keep < n || n * n_ut <= 384 * 1024)) {
         cluster = 16;
         for (words = 2; words <= 4 && !small; words *= 2) {
             if (!fits()) continue;

@@ -177,3 +177,19 @@ def test_threshold_at_zero(keep, tiny, T, dtype):
     want = R.select_entries(z1, k)
     assert np.array_equal(idx.cpu().numpy(), want)
     assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("T,kernels", [(17, 1), (500, 1), (1100, 1), (3072, 1), (3073, 4), (7936, 4)])
+def test_everything_kept(T, kernels, dtype):
+    """Zero keys among them; either side of the length up to which one kernel writes all of them."""
+    d = 128
+    x0, x1 = (torch.randint(-3, 4, (T, d), device="cuda", generator=torch.Generator("cuda").manual_seed(s)).to(dtype) for s in (1, 2))
+    z0, idx, val = torch.empty_like(x0), torch.empty(T * d, dtype=torch.int32, device="cuda"), torch.empty(T * d, dtype=dtype, device="cuda")
+    before = B.launch_count()
+    assert B.compress_unit_noalloc(x0, x1, 1, 1, z0, idx, val) == T * d
+    assert B.launch_count() - before == kernels
+    want_z0, z1 = R.depth_split(x0.float().cpu().numpy(), x1.float().cpu().numpy(), dtype == torch.bfloat16)
+    assert np.array_equal(z0.float().cpu().numpy(), want_z0)
+    assert np.array_equal(idx.cpu().numpy(), np.arange(T * d))
+    assert np.array_equal(val.float().cpu().numpy(), z1.ravel())
