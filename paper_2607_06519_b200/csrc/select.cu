@@ -1369,9 +1369,21 @@ cudaError_t launch_chain(int cluster, void (*kernel)(A...), dim3 grid, int threa
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Words of 32 positions per thread of a cluster of sixteen at most: with four bytes a position or more two words fill the shared memory.
+template <typename T, int B>
+constexpr int most_words() { return sizeof(T) == 2 && B == 2 ? 4 : 2; }
+typedef void (*SmallKernel)(CompressArgs, int, int);
+template <typename T, int B>
+SmallKernel small_of(int words) {
+    if constexpr (most_words<T, B>() == 4)
+        if (words == 4) return small_kernel<T, B, 4>;
+    return words == 2 ? small_kernel<T, B, 2> : small_kernel<T, B, 1>;
+}
+
 template <typename T, int B>
 cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* const* v_layers, int block_begin, int block_end, cudaStream_t st) {
     static PerDevice once;
+    constexpr int kMostWords = most_words<T, B>();
     static std::atomic<int> long_clusters[PerDevice::kMaxDevices][2][kSmallSmem / 4096 + 1];  // [two or four words][4 KiB of shared memory]; 0: not known
     int sms = 0;
     constexpr int CE = compress_chunk(B, (int)sizeof(T));
@@ -1380,11 +1392,9 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
         cudaError_t e1 = cudaFuncSetAttribute(split_kernel<T, B, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(threshold_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kThrMini * 128);
         if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(split_kernel<T, B, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(small_kernel<T, B, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
-        for (int w = 0; w < 2 && e1 == cudaSuccess; ++w) {
-            auto* const kernel = w ? small_kernel<T, B, 4> : small_kernel<T, B, 2>;
-            e1 = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
-            if (e1 == cudaSuccess) e1 = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (int w = 1; w <= kMostWords && e1 == cudaSuccess; w *= 2) {
+            e1 = cudaFuncSetAttribute(small_of<T, B>(w), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+            if (e1 == cudaSuccess && w > 1) e1 = cudaFuncSetAttribute(small_of<T, B>(w), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         }
         return e1;
     }, &sms);
@@ -1413,8 +1423,8 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
     // bf16 tensor of 384k 54.6 us, four kernels 66.6, 512k 84.6 and 66.8; float32 39.6 and 53.1, 66.0 and 63.1; eight bf16 tensors of 256k 103.9 and 91.5).
     if (few && !small && (int64_t)16 * n_ut <= 2 * sms && tiles >= 16 && (a.n_keep < n || n * n_ut <= 384 * 1024)) {
         cluster = 16;
-        for (words = 2; words <= 4 && !small; words *= 2) {
-            if (!fits()) continue;
+        for (words = 2; words < kMostWords && !fits();) words *= 2;
+        if (fits()) {
             const int wi = words / 4, bucket = (int)((small_smem + 4095) / 4096);
             int dev = 0, at_once = 0;
             if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1428,15 +1438,14 @@ cudaError_t compress(CompressArgs& a, const void* const* k_layers, const void* c
                 attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
                 q.attrs = attr;
                 q.numAttrs = 1;
-                if ((e = cudaOccupancyMaxActiveClusters(&at_once, words == 2 ? small_kernel<T, B, 2> : small_kernel<T, B, 4>, &q)) != cudaSuccess) return e;
+                if ((e = cudaOccupancyMaxActiveClusters(&at_once, small_of<T, B>(words), &q)) != cudaSuccess) return e;
                 long_clusters[dev][wi][bucket].store(at_once > 0 ? at_once : -1, std::memory_order_relaxed);
             }
             small = n_ut <= at_once;
-            if (small) break;
         }
     }
     if (small) {
-        auto* const kernel = words == 1 ? small_kernel<T, B, 1> : words == 2 ? small_kernel<T, B, 2> : small_kernel<T, B, 4>;
+        const SmallKernel kernel = small_of<T, B>(words);
         for (int b0 = block_begin; b0 < block_end; b0 += kSplitLayers / B) {
             const int nb = std::min(block_end - b0, kSplitLayers / B);
             for (int l = 0; l < nb * B; ++l) {
