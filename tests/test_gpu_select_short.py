@@ -90,7 +90,7 @@ def test_any_scale(scale, den, T):
                                        ("f32", 128, 4096), ("f32", 128, 4097), ("f32", 64, 4099), ("f32", 64, 8191)])
 @pytest.mark.parametrize("den", [3, 16])
 def test_clusters_of_sixteen(dtype, d, T, den):
-    """Two and four words of positions per thread, at and beside the most that each holds (counts of 16 bits, shared memory)."""
+    """Two and four words of positions per thread, at and beside the most that two of them hold, and lengths that four no longer hold."""
     w = synth.WORKLOADS["decode32k"].scaled(n_layers=2, n_kv_heads=1, n_q_heads=1, head_dim=d, T=T, dtype=dtype, n_needles=2, W=1, keep_num=1, keep_den=den,
                                             name="sixteen")
     pf = runner.Prefilled(w)
@@ -193,3 +193,23 @@ def test_everything_kept(T, kernels, dtype):
     assert np.array_equal(z0.float().cpu().numpy(), want_z0)
     assert np.array_equal(idx.cpu().numpy(), np.arange(T * d))
     assert np.array_equal(val.float().cpu().numpy(), z1.ravel())
+
+
+@pytest.mark.parametrize("d,T,kernels", [(128, 4096, 1), (128, 4097, 1), (128, 7936, 1), (128, 7937, 6), (64, 16128, 1), (64, 16129, 6)])
+@pytest.mark.parametrize("values,keep", [("normal", (1, 16)), ("normal", (3, 5)), ("three", (1, 3)), ("three", (3, 5)), ("equal", (1, 3)), ("equal", (3, 5))])
+def test_four_words_per_thread(values, keep, d, T, kernels):
+    """bf16 pairs in clusters of sixteen up to the most that a block's counts of 16 bits hold (31 tiles of 2 048, 63 of 1 024 positions), among them keys that
+    are all equal or of three values; one tile more a block takes the separate kernels."""
+    rng = np.random.default_rng(8)
+    diff = {"normal": rng.standard_normal((T, d)), "three": rng.integers(-1, 2, (T, d)), "equal": np.ones((T, d))}[values].astype(np.float32)
+    x0 = torch.from_numpy(diff).cuda().bfloat16()
+    x1 = torch.zeros_like(x0)
+    k = T * d * keep[0] // keep[1]
+    z0, idx, val = torch.empty_like(x0), torch.empty(k, dtype=torch.int32, device="cuda"), torch.empty(k, dtype=torch.bfloat16, device="cuda")
+    before = B.launch_count()
+    assert B.compress_unit_noalloc(x0, x1, *keep, z0, idx, val) == k
+    assert B.launch_count() - before == kernels
+    _, z1 = R.depth_split(x0.float().cpu().numpy(), x1.float().cpu().numpy(), True)
+    want = R.select_entries(z1, k)
+    assert np.array_equal(idx.cpu().numpy(), want)
+    assert np.array_equal(val.float().cpu().numpy(), z1.ravel()[want])
