@@ -877,11 +877,13 @@ __device__ __forceinline__ uint32_t packed_place(uint32_t p) {
 // a block scan per round took 767.)
 template <typename T, int B, bool ALL>
 __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_begin) {
-    constexpr int NB = B == 4 ? 4 : 1, Q = Eight<T, B>::Q, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
+    constexpr int NB = B == 4 ? 4 : 1, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
+    constexpr int PER = NB * sizeof(T) > 8 ? 4 : 8, Q = PER * (int)sizeof(T) / 16;  // candidates per lane and round; 16-byte vectors of theirs per layer
+    constexpr uint32_t FULL = (1u << PER) - 1u;
     constexpr bool TWO = sizeof(T) == 2 && B == 2;
     __shared__ uint32_t s_map[8][WORDS];
-    __shared__ uint16_t s_pos[8][256];
-    __shared__ __align__(16) T s_val[8][NB][256];
+    __shared__ __align__(16) uint16_t s_pos[8][32 * PER];
+    __shared__ __align__(16) T s_val[8][NB][32 * PER];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ut = ut_begin + blockIdx.y, c = blockIdx.x * 8 + warp;
     chain_wait();
@@ -894,7 +896,7 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
     const int n = a.cand_n[(int64_t)ut * a.chunks_max + c];
     const int2 b0 = a.chunk_base[(int64_t)ut * a.chunks_max + c];
     const int64_t e0 = (int64_t)c * CE, n_e = (int64_t)a.T * a.d;
-    const uint4* const pos = reinterpret_cast<const uint4*>(a.cand_pos + (int64_t)ut * a.cand_stride + e0);
+    const uint2* const pos = reinterpret_cast<const uint2*>(a.cand_pos + (int64_t)ut * a.cand_stride + e0);
     const T* const val = reinterpret_cast<const T*>(a.cand_val) + (int64_t)ut * NB * a.cand_stride + e0;
     uint32_t run_gt = (uint32_t)b0.x, run_eq = (uint32_t)b0.y;
     int32_t* const idx = a.idx + (int64_t)ut * a.kcap;
@@ -904,30 +906,51 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
     int32_t* const off = a.tile_off + (int64_t)ut * (a.ntiles_max + 1) + (int)(e0 >> tile_shift);
     int tile = -1;  // of the entry before
     __syncwarp();
-    uint4 p_next = make_uint4(0, 0, 0, 0), v_next[NB][Q];
+    uint2 p_next[PER / 4] = {};
+    uint4 v_next[NB][Q];
     auto load = [&](int i) {
         if (i >= n) return;
-        if constexpr (!ALL) p_next = pos[i >> 3];
+        if constexpr (!ALL) {
+            if constexpr (PER == 8) {
+                const uint4 x = reinterpret_cast<const uint4*>(pos)[i >> 3];
+                p_next[0] = make_uint2(x.x, x.y);
+                p_next[PER / 4 - 1] = make_uint2(x.z, x.w);
+            } else {
+                p_next[0] = pos[i >> 2];
+            }
+        }
 #pragma unroll
         for (int l = 0; l < NB; ++l)
 #pragma unroll
             for (int k = 0; k < Q; ++k) v_next[l][k] = reinterpret_cast<const uint4*>(val + (int64_t)l * a.cand_stride + i)[k];
     };
-    load(8 * lane);
-    for (int base = 0; base < n; base += 256) {
-        const int i = base + 8 * lane;
-        const uint4 p8 = p_next;
+    load(PER * lane);
+    for (int base = 0; base < n; base += 32 * PER) {
+        const int i = base + PER * lane;
+        uint32_t pw[PER / 2];
+#pragma unroll
+        for (int k = 0; k < PER / 4; ++k) { pw[2 * k] = p_next[k].x; pw[2 * k + 1] = p_next[k].y; }
         uint4 v8[NB][Q];
 #pragma unroll
         for (int l = 0; l < NB; ++l)
 #pragma unroll
             for (int k = 0; k < Q; ++k) v8[l][k] = v_next[l][k];
-        load(i + 256);
-        const uint32_t valid = i >= n || tau == kNoKey ? 0u : n - i >= 8 ? 0xFFu : (1u << (n - i)) - 1u;
+        load(i + 32 * PER);
+        const uint32_t valid = i >= n || tau == kNoKey ? 0u : n - i >= PER ? FULL : (1u << (n - i)) - 1u;
         uint32_t gt = 0, eq = 0;
         if constexpr (TWO) {
             gt = Eight<T, B>::reach(v8, tau + 0x10000u);
             eq = Eight<T, B>::reach(v8, tau) & ~gt;
+        } else if constexpr (PER == 4) {
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                float h[NB];
+#pragma unroll
+                for (int l = 0; l < NB; ++l) h[l] = to_f32(reinterpret_cast<const T*>(&v8[l][0])[k]);
+                const uint32_t key = key_of<B>(h);
+                gt |= (uint32_t)(key > tau) << k;
+                eq |= (uint32_t)(key == tau) << k;
+            }
         } else {
             Eight<T, B>::keys(v8, [&](int k, uint32_t key) {
                 gt |= (uint32_t)(key > tau) << k;
@@ -955,21 +978,30 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
         run_gt += total >> 16;
         run_eq += total & 0xFFFFu;
         const uint32_t n_out = run_gt + min(run_eq, need) - first;
-        const uint32_t pw[4] = {p8.x, p8.y, p8.z, p8.w};
+        if (ALL && map_k && kept) atomicOr(&map[i >> 5], kept << (i & 31));  // (the lane's positions follow one another)
+        if (ALL && kept == FULL && at % PER == 0) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (!(kept >> k & 1u)) continue;
-            s_pos[warp][at] = ALL ? (uint16_t)(i + k) : (uint16_t)(pw[k >> 1] >> (16 * (k & 1)));
+            for (int k = 0; k < PER; k += 2) reinterpret_cast<uint32_t*>(s_pos[warp])[(at + k) / 2] = (uint32_t)(i + k) | (uint32_t)(i + k + 1) << 16;
 #pragma unroll
-            for (int l = 0; l < NB; ++l) s_val[warp][l][at] = reinterpret_cast<const T*>(&v8[l][0])[k];
-            ++at;
+            for (int l = 0; l < NB; ++l)
+#pragma unroll
+                for (int k = 0; k < Q; ++k) reinterpret_cast<uint4*>(s_val[warp][l])[at * Q / PER + k] = v8[l][k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                if (!(kept >> k & 1u)) continue;
+                s_pos[warp][at] = ALL ? (uint16_t)(i + k) : (uint16_t)(pw[k >> 1] >> (16 * (k & 1)));
+#pragma unroll
+                for (int l = 0; l < NB; ++l) s_val[warp][l][at] = reinterpret_cast<const T*>(&v8[l][0])[k];
+                ++at;
+            }
         }
         __syncwarp();
         for (uint32_t j = lane; j < n_out; j += 32) {
             const uint32_t p = s_pos[warp][j];
             const int t = (int)(p >> tile_shift), t_before = j ? (int)(s_pos[warp][j - 1] >> tile_shift) : tile;
             for (int x = t_before + 1; x <= t; ++x) off[x] = (int32_t)(first + j);
-            if (map_k) atomicOr(&map[p >> 5], 1u << (p & 31));
+            if (!ALL && map_k) atomicOr(&map[p >> 5], 1u << (p & 31));
             idx[first + j] = (int)e0 + (int)p;
             const uint32_t place = sizeof(T) == 2 ? packed_place(p) : 0u;
 #pragma unroll
