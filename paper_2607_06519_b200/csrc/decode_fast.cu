@@ -743,7 +743,7 @@ decode_fast_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
 // out = sum_s e^{m_s - M} acc_s / sum_s e^{m_s - M} l_s over a query head's split-K parts.  One warp per 32 or 128 channels of a
 // head; it rides on programmatic dependent launch between two decode launches.  A block has 32 threads and few registers
 // so that it becomes resident beside a decode block (which leaves 2 048 registers and 1 KiB of shared memory of an SM) and
-// its start costs nothing.  Latency-bound: the maxima, sums and accumulators of 32 parts are requested in one round.
+// its start costs nothing.  Latency-bound: the maxima and sums of 32 parts are requested together, then accumulators by 20 (VEC 2) or 4.
 // (Before, the last block of a unit combined behind an atomic ticket: a release, an atomic round trip and two rounds of
 // loads on the critical path of every layer call, and the SM it ran on started the next call late.)
 // VEC 4: a lane has four channels of every part, four parts in flight (many heads, few parts each).  VEC 2: a lane has two channels of
@@ -938,7 +938,8 @@ static cudaError_t plan_decode_schedule(const DecodeArgs& a, int units, int sm_c
     sch.units = units;
     sch.cluster = 0;
     // Clusters, as many blocks per unit as fit: one kernel instead of two, where that is worth more than the blocks that are
-    // left out.  Measured on a stream, us a call of bf16 rows: clusters 3.55 + 1.03 for each plain tile of the slowest block (a tail tile counts 1.2),
+    // left out.  Measured on a stream, us a call of bf16 rows (clusters with 0.8 KiB more of parameters, which took 0.15, 8-bit rows 0.25): clusters
+    // 3.55 + 1.03 for each plain tile of the slowest block (a tail tile counts 1.2),
     // two kernels 5.7 + 1.1 for each of the average block and at least 7.75 (8.4 with tails), the two hand-overs.  Eight KV heads, clusters against
     // two kernels: 1 024 tokens 5.4 and 7.7, 2 047 6.8 and 7.8, 3 000 8.1 and 7.8, 8 191 15.5 and 11.1; with a tail 1 024 6.3 and 8.4, 1 500
     // 7.2 and 8.5, 2 047 8.0 and 8.4, 3 000 9.9 and 8.8; two KV heads 2 047 5.7 and 7.7, with a tail 6.7 and 8.4, 4 096 8.4 and 7.8.

@@ -15,7 +15,7 @@
 //                        positions that reach the bound, in order, to the chunk's candidate list;
 //   3. threshold_kernel  one block per unit-tensor (a cluster of them for few and long ones): the k-th largest key among the
 //                        candidates (a radix select in shared memory), then the keys above and equal to it before every chunk;
-//   4. compact_kernel    one block per chunk: candidates -> the lists, the offsets of the 16-token tiles and, of K, a bit
+//   4. compact_kernel    one warp per chunk: candidates -> the lists, the offsets of the 16-token tiles and, of K, a bit
 //                        map of the kept positions.
 // (Few short unit-tensors take small_kernel instead of all of these.)
 // The bound is only a guess: where fewer than k positions reach it, step 3 says so and steps 2 and 3 run again for that
@@ -536,7 +536,7 @@ __device__ __forceinline__ void scan_chunks(int2* base, int c_begin, int c_end, 
 // 149 -> 88 us).  The sample says whether it is: with keep 1/3 and more of log-normal channel scales it is not, and a pass for nothing made 128
 // tensors of 8 192 tokens at keep 1/2 673 us instead of 622.
 // Where these don't hold the digits are counted one after the other.
-constexpr int kThrMini = 512;  // chunks whose counts are kept
+constexpr int kThrMini = 512;  // chunks whose counts are kept: 64 KiB, 32k x 128 positions.  (Longer tensors take the passes; more chunks were not measured.)
 template <typename T, int B>
 __global__ void __launch_bounds__(kThrThreads) threshold_kernel(CompressArgs a, int ut_begin, int redo) {
     __shared__ __align__(16) uint32_t s_hist[kThrBins];
@@ -870,11 +870,12 @@ __device__ __forceinline__ uint32_t packed_place(uint32_t p) {
     return (half << 10 | row << 6 | chunk << 3 | (p & 7u)) << 16;
 }
 
-// grid (groups of eight chunks, unit-tensors), a chunk per warp: no block barriers.  A round takes 256 candidates, eight per lane: one warp scan
-// of their counts, then positions and values of those that stay go through shared memory, so that the lists leave in runs.
-// Bound by the latency of a chunk's chain (loads, scan, both ways through shared memory) beside 2 GB of lists and candidates: 32 layers of 32k
-// tokens 300 -> 266 us, 8 blocks of four of 12 289 147 -> 130, against 32 candidates a round with two votes each.  (One chunk per block with
-// a block scan per round took 767.)
+// grid (groups of eight chunks, unit-tensors), a chunk per warp: no block barriers.  A round takes 256 candidates, eight per lane (of float32
+// blocks of four 128, four per lane): one warp scan of their counts, then positions and values of those that stay go through shared memory, so that the lists leave in runs.
+// Bound by instructions: issue slots 80 % busy, HBM 24 % (counters on 4 layers of 32k tokens).  32 layers of 32k tokens (0.32 GB of candidates read,
+// 0.67 GB of lists written) 300 -> 266 us, 8 blocks of four of 12 289 147 -> 130, against 32 candidates a round with two votes each.  (One chunk
+// per block with a block scan per round took 767.)  Four candidates per lane where eight are 32 registers of values and as many of the next ones':
+// with eight, float32 blocks of four had 119 registers and two blocks on an SM, 8 layers of 65 536 tokens 2 389 us in all, now 2 338.
 template <typename T, int B, bool ALL>
 __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_begin) {
     constexpr int NB = B == 4 ? 4 : 1, CE = compress_chunk(B, (int)sizeof(T)), WORDS = CE / 32;
@@ -1032,16 +1033,17 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 }
 
 // ---- all of it for a short unit-tensor ------------------------------------------------------------------
-// One cluster per unit-tensor, a range of whole 16-token tiles per block, at most kSmallElems positions: the high-frequency
-// values stay in shared memory, the threshold is a radix select over histograms that every block adds up from the cluster's
-// shared memories (11, 10 and 10 bits of the key; a bf16 pair's has no more than 15: one histogram of 32 octaves, which also says how
-// many of the kept positions the blocks before have), and a thread writes the entries of its 32
-// consecutive positions.  Bound by the chain of its steps (loads, cluster barriers with reads across the cluster between, block
+// One cluster per unit-tensor, a range of whole 16-token tiles per block, at most W x kSmallElems positions and fewer than 2^16: the
+// high-frequency values stay in shared memory.  Every block adds up the cluster's histograms of the key's top 15 bits, a window of 32 octaves, from
+// their shared memories; for bf16 pairs that is the threshold and says how many of the kept positions the blocks before have.  Wider
+// keys: those that share the threshold's top half are gathered and looked through by every block, or counted in two more digits (10 and 6
+// bits) where they are many.  A thread writes the entries of its W x 32 consecutive positions.  Bound by the chain of its steps (loads, cluster barriers with reads across the cluster between, block
 // scans), not by bytes: one bf16 pair of 509 x 128 12.0 us with three exchanges, 9.4 with one (24.5 by the four kernels); 1000 x 128
 // 32.8 -> 12.9 and eight of 900 x 128 47.9 -> 26.6 against the four kernels, with three exchanges.
-// While the clusters take two turns at most (two blocks fit an SM up to about 88 KiB of values each): 32 tensors
+// Taken while the clusters need two turns at most (two blocks fit an SM up to 88 KiB of values each): 32 tensors
 // of blocks of four, 1000 x 128, two turns, 66 us against 64; 256 pairs of 1024 x 128, seven turns, 195 against 133.
-// W: words of 32 positions per thread.
+// W: words of 32 positions per thread.  (Keys of few different values meet in the histogram's bins: two tensors of 1000 x 128, bf16 all equal 32.6 us,
+// five values 16.6; float32 38.1 and 26.2; where a thread adds eight equal ones at once all equal take 26, and normal ones 4 % more.)
 constexpr int kSmallNear = 1024;  // keys that are gathered at most
 // Of them are compared each with all others; digits among more.  (All compared, up to 1 024: 4096 x 128 float32 at keep 1/2 109.9 us, now 48.7;
 // 1000 x 128 at keep 1/4, some 160 keys, 23.3 and 19.9.)
@@ -1298,7 +1300,7 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
             }
         }
     }
-    // ---- entries: those above in the blocks, warps and threads before, then those equal (counts in halves: at most 2^14) ----
+    // ---- entries: those above in the blocks, warps and threads before, then those equal (counts in halves: a block has fewer than 2^16) ----
     uint32_t gt[W] = {}, eq[W] = {}, cnt = 0;
     each([&](int w, int i, uint32_t key) {
         gt[w] |= (uint32_t)(key > tau) << i;

@@ -9,14 +9,14 @@
 //
 // 1. token_score_kernel (tcgen05): the transposed probe product D[token][probe row] = Z1K . Q^T, so that a thread
 //    of the epilogue owns one token (TMEM lane) and takes the maximum over its row's columns in registers.  A = 128
-//    tokens of Z1K per tile (TMA ring, shared memory), B = the item's 256 Q rows (shared memory, resident),
-//    M = 128, N = 256, K = 16, two accumulator sets of 256 TMEM columns.  Items of the two layers / row blocks of a
+//    tokens of Z1K per tile (TMA ring, shared memory), B = the item's Q rows (64, 128 or 256 of them; shared memory, the next
+//    item's in a second buffer), M = 128, N = 64, 128 or 256, K = 16, two accumulator sets of N TMEM columns.  Items of the two layers / row blocks of a
 //    unit merge with atomicMax on the (non-negative) float bit patterns, which is order-independent.
 //    The same registers give Eq. 2's errors: the token's sum of D^2 over the rows that see it, one float per item.  Shared
 //    drops every token's high-frequency row, residual every unselected one's, so both errors are sums of these numbers
 //    and the probe needs no second product (it was two more passes over T x rows x 128, and a copy of Z1K with the
 //    selected rows zeroed to run one of them on: 8 191 tokens, 8 blocks of four: the probe 627 -> 250 us).
-// 2. token_select_kernel: per unit an MSB-first radix select (4 x 8 bits) of the k_tok-th largest score and an
+// 2. token_select_kernel: per unit an MSB-first radix select (12, 12 and 7 bits) of the k_tok-th largest score and an
 //    index-ordered compaction: ascending token list, per-16-token-slice counts, and the two error sums in float64.
 // (The commit step forms the selected rows from the caller's K and V: token_gather_kernel in compress.cu.)
 #include <algorithm>
