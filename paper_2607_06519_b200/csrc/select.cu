@@ -1064,7 +1064,7 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     __shared__ __align__(16) uint32_t s_h1[2048], s_all[4096];
     uint16_t* const s_near = reinterpret_cast<uint16_t*>(s_all + 3072);  // [kSmallNear]
     static_assert(sizeof(s_h1) + sizeof(s_all) + 1024 + 88 * 1024 + 1024 <= 228 * 1024 / 2, "two blocks fit an SM with 88 KiB of values each");
-    __shared__ uint32_t s_count, s_warp[kSmallThreads / 32], s_before[2][kSmallThreads / 32], s_n, s_off[17], s_low[2];
+    __shared__ uint32_t s_count, s_warp[kSmallThreads / 32], s_before[2][kSmallThreads / 32], s_n, s_off[17], s_low[2], s_below;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x % blocks, item = blockIdx.x / blocks, uts = a.Hkv * a.tensors;
     const int ut = a.ut_base + item, blk = item / uts, u = item % uts, h = u / a.tensors, is_v = u % a.tensors;
@@ -1074,13 +1074,12 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
     const bool every = a.n_keep == n_e;  // all of them are kept: above zero or equal to it
     for (int i = tid; i < 2048; i += kSmallThreads) s_h1[i] = 0;
     if (tid == 0) s_n = 0;
-    // a key's bin: 4 094 values of its top 15 bits above `from`, 32 octaves, the last bin for what is larger, the first for zero (rows that are
-    // the same in both layers, or padding: bf16 pairs of 300 x 128, all kept, 24.5 us by further windows, 16.7 with the bin).  At first 2^-24 to 2^8, of energies
-    // 2^-16 to 2^16.
+    // a key's bin: 4 094 values of its top 15 bits above `from`, 32 octaves, the last bin for what is larger, the first for all others: zero (rows
+    // that are the same in both layers, or padding) and what is below the window.  At first 2^-24 to 2^8, of energies 2^-16 to 2^16.
     uint32_t from = (127u - (B == 4 ? 16u : 24u)) << 7;
     auto count_key = [&](uint32_t key) {
-        const uint32_t k16 = key >> 16, bin = k16 > from ? min(k16 - from, 4095u) : 0u;
-        if (bin || !k16) atomicAdd(&s_h1[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has fewer than 2^16 positions)
+        const uint32_t bin = min(max(key >> 16, from) - from, 4095u);
+        atomicAdd(&s_h1[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has fewer than 2^16 positions)
     };
     auto chunk_at = [&](int word, int j) { return (word * CH + (j ^ (Q == 1 ? (word >> 1) & 3 : word & 7))) * 16; };
     chain_wait();
@@ -1177,13 +1176,24 @@ __global__ void __launch_bounds__(kSmallThreads, W > 2 ? 1 : 2) small_kernel(Com
             *reinterpret_cast<uint4*>(&s_all[8 * tid]) = make_uint4(all[0], all[1], all[2], all[3]);
             *reinterpret_cast<uint4*>(&s_all[8 * tid + 4]) = make_uint4(all[4], all[5], all[6], all[7]);
             __syncthreads();
-            const bool found = find_bin<kSmallThreads, 4096>(s_all, (uint32_t)a.n_keep, bin, above);
-            if (found && bin > 0 && (bin < 4095 || from + 4095 >= 32767)) break;
-            if (found && bin == 0 && above + s_all[0] == (uint32_t)n_e) {  // zero, and nothing lies between it and the window
+            find_bin<kSmallThreads, 4096>(s_all, (uint32_t)a.n_keep, bin, above);
+            if ((bin > 0 || from == 0) && (bin < 4095 || from + 4095 >= 32767)) break;
+            if (bin == 0) {
+                // the k-th is zero unless a key lies between zero and the window: a look at the keys instead of another window
+                bool below = false;
+                each([&](int, int, uint32_t key) { below |= key != 0 && key >> 16 <= from; });
+                const int any = __syncthreads_or(below);
+                if (tid == 0) s_below = any;
+                cluster_sync();
+                uint32_t at, v;
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_below)), "r"(lane < blocks ? lane : 0));
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
                 from = 0;
-                break;
+                if (!__any_sync(0xFFFFFFFFu, v != 0)) break;
+            } else {
+                from += 4094;
             }
-            from = found && bin > 0 ? from + 4094 : 0;  // another window (the same for the whole cluster): above, or from the smallest key on
+            // another window (the same for the whole cluster): from the smallest key on, or above
             cluster_sync();
             for (int i = tid; i < 2048; i += kSmallThreads) s_h1[i] = 0;
             __syncthreads();
