@@ -1039,13 +1039,13 @@ __global__ void __launch_bounds__(256) compact_kernel(CompressArgs a, int ut_beg
 // high-frequency values stay in shared memory.  Every block adds up the cluster's histograms of the key's top 15 bits, a window of 32 octaves, from
 // their shared memories; for bf16 pairs that is the threshold and says how many of the kept positions the blocks before have.  Wider
 // keys: those that share the threshold's top half are gathered and looked through by every block, or counted in two more digits (10 and 6
-// bits) where they are many.  A thread writes the entries of its W x 32 consecutive positions.  Bound by the chain of its steps (loads, cluster barriers with reads across the cluster between, block
-// scans), not by bytes: one bf16 pair of 509 x 128 12.0 us with three exchanges, 9.4 with one (24.5 by the four kernels); 1000 x 128
+// bits) where they are many.  A thread writes the entries of its W x 32 consecutive positions.  Bound by the chain of its steps (loads,
+// cluster barriers with reads across the cluster between, block scans), not by bytes: one bf16 pair of 509 x 128 12.0 us with three exchanges, 9.4 with one (24.5 by the four kernels); 1000 x 128
 // 32.8 -> 12.9 and eight of 900 x 128 47.9 -> 26.6 against the four kernels, with three exchanges.
 // Taken while the clusters need two turns at most (two blocks fit an SM up to 88 KiB of values each): 32 tensors
 // of blocks of four, 1000 x 128, two turns, 66 us against 64; 256 pairs of 1024 x 128, seven turns, 195 against 133.
-// W: words of 32 positions per thread.  (Keys of few different values meet in the histogram's bins: two tensors of 1000 x 128, bf16 all equal 32.6 us,
-// five values 16.6; float32 38.1 and 26.2; adding a thread's eight equal ones at once made the float32 32.5, and normal bf16 11.3 -> 11.8.)
+// W: words of 32 positions per thread.  (Keys of few different values meet in the histogram's bins: two tensors of 1000 x 128, bf16 all equal 32.9 us,
+// five values 16.5; float32 36.2 and 25.9; adding a thread's eight equal ones at once made the float32 32.5, and normal bf16 11.3 -> 11.8.)
 constexpr int kSmallNear = 1024;  // keys that are gathered at most
 // Of them are compared each with all others; digits among more.  (All compared, up to 1 024: 4096 x 128 float32 at keep 1/2 109.9 us, now 48.7;
 // 1000 x 128 at keep 1/4, some 160 keys, 23.3 and 19.9.)
